@@ -83,8 +83,10 @@ def draw(rng):
     per_row = tokens // seqs
     if rng.random() < 0.4 and per_row >= 64:                               # whole chunks as often as odd lengths
         per_row -= per_row % 64
-    return _case("drawn", entry, gates, dtype, seqs, per_row * seqs if packed else per_row, heads, d_k, d_v, packed=packed,
+    case = _case(None, entry, gates, dtype, seqs, per_row * seqs if packed else per_row, heads, d_k, d_v, packed=packed,
                  states=rng.random() < 0.5, delta=delta, decay=rng.choice(decays))
+    del case["name"]
+    return case
 
 
 def _sizes(case):
