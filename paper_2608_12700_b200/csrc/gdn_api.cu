@@ -81,8 +81,7 @@ WsLayout layout_for(const gdn_desc& d) {
         L.fwd_end = L.total;
         return L;
     }
-    // The SIMT kernels keep every factor in fp32, whatever the I/O dtype.
-    return make_layout(d, sizeof(float), sizeof(float), simt_scratch_per_chunkhead(d));
+    return make_layout_ffma(d);   // the FFMA kernels keep everything in fp32, whatever the I/O dtype
 }
 
 // Channel-wise calls: the layout the kernels see (of the widened problem when a head dimension of 64 is zero-padded onto

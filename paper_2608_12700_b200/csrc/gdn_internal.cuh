@@ -45,6 +45,7 @@ struct WsLayout {
                                          // U~^T, the scaled keys Kb (16 KB per chunk-head each) and E (32 KB); else unused
     size_t img_QKp, img_Km, img_Vt, img_dO;   // ... of [Q~; K+] (32 KB), K-, V~ and scale dO (16 KB each)
     int tc_scans;                        // ... and T, P, hc, dhn are bf16 tile images as well (8, 8, 32, 32 KB)
+    size_t Kb, U, dU;      // FFMA families (fp32): keys scaled to the chunk end [CH, 64, d_k]; U = U~ - W h and dU [CH, 64, d_v]
     size_t scratch;        // kernel-private staging, per chunk-head
     size_t scratch_per_ch; // bytes of scratch per chunk-head
     size_t total;
@@ -80,6 +81,34 @@ inline WsLayout make_layout(const gdn_desc& d, size_t elem, size_t elem_add, siz
     L.scratch_per_ch = scratch_per_ch;
     L.scratch = take(scratch_per_ch * CH);
     L.total = o;
+    return L;
+}
+
+// Layout of the scalar-gate FFMA family: everything fp32, carries in low-rank form.
+inline WsLayout make_layout_ffma(const gdn_desc& d) {
+    WsLayout L{};
+    const size_t Ttot = (size_t)d.B * (size_t)d.T;
+    L.max_chunks = (int)((Ttot + kC - 1) / kC + (size_t)d.N);
+    const size_t CH = (size_t)L.max_chunks * d.H;
+    size_t o = sizeof(WsHeader);
+    auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
+    L.seq_first = take(4 * ((size_t)d.N + 1));
+    L.chunk_seq = take(4 * (size_t)L.max_chunks);
+    L.chunk_tok0 = take(4 * (size_t)L.max_chunks);
+    L.chunk_len = take(4 * (size_t)L.max_chunks);
+    L.gamma = take(4 * CH * kC);
+    L.Tm = take(4 * CH * kC * kC);
+    L.W = take(4 * CH * kC * d.d_k);
+    L.Ut = take(4 * CH * kC * d.d_v);
+    L.Pm = take(4 * CH * kC * kC);
+    L.Kb = take(4 * CH * kC * d.d_k);
+    L.U = take(4 * CH * kC * d.d_v);
+    L.hc = take(4 * CH * d.d_k * d.d_v);
+    L.Nm = L.Bf = L.fwd_end = o;
+    L.E = take(4 * CH * d.d_k * d.d_v);
+    L.dhn = take(4 * CH * d.d_k * d.d_v);
+    L.dU = take(4 * CH * kC * d.d_v);
+    L.scratch = L.total = o;
     return L;
 }
 
@@ -180,7 +209,6 @@ gdn_status check_bwd_args(const gdn_desc* desc, const void* q, const void* k, co
 cudaError_t launch_table(const Problem& p, cudaStream_t st);
 cudaError_t simt_launch_fwd(const Problem& p, cudaStream_t st);
 cudaError_t simt_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st);
-size_t simt_scratch_per_chunkhead(const gdn_desc& d);
 
 // FFMA family for per-channel gates (Eq. 1 with gate vectors).
 cudaError_t vec_launch_fwd(const Problem& p, cudaStream_t st);

@@ -2,19 +2,27 @@
 // out tf32/bf16 operands) and a plain-CUDA-core statement of every stage of the chunked method.
 //
 // Stage map (Section 4.2 of the paper; names follow the library header):
-//   table  : chunk table from cu_seqlens
-//   prep   : gamma = cumsum(g); A = stril(Diag(b)(K K^T . D)); T = (I + A)^-1 by forward substitution;
-//            W = T Diag(b Gam) K; Ut = T Diag(w) V; Nm = Kb^T W; Bf = Kb^T Ut
-//   fscan  : h' = Gam_e h - Nm h + Bf           (forward carry; stores the state entering each chunk)
-//   eprep  : P = tril(Q K^T . D); E = scale (Diag(Gam) Q - P W)^T dO
-//   rscan  : dh = Gam_e dh' - Nm^T dh' + E       (reverse carry, the paper's K#1; stores dh' per chunk)
+//   table  : chunk table from cu_seqlens (packed sequences only)
+//   prep   : gamma = cumsum(g); A = stril(Diag(b)(K K^T . D)); P = tril(Q K^T . D); T = (I + A)^-1; W = T Diag(b Gam) K;
+//            Ut = T Diag(w) V; Kb = Diag(exp(gam_e - gam)) K; and for the backward
+//            dU0 = scale P^T dO, E = scale (Diag(Gam) Q - P W)^T dO (alone on a workspace fresh from the forward)
+//   scan   : h' = Gam_e h + Kb^T U with U = Ut - W h, and dh = Gam_e dh' + E - W^T (Kb dh') (the paper's K#1), both
+//            directions in one launch when both are wanted (ffma_scan.cuh)
 //   intra  : all token gradients of a chunk, including the VJP of the triangular solve (the paper's K#2)
-// One CTA handles one (chunk, head) in the parallel stages and one (sequence, head) chain in the scans.
-// Every reduction has a fixed order: results are bit-identical from run to run.
-#include "simt_common.cuh"
+//   out    : forward output
+// One CTA handles one (chunk, head) in the parallel stages.  Operands are staged in shared memory, products are register
+// tiles (ffma_tile.cuh).  Every reduction has a fixed order: results are bit-identical from run to run.
+// The FMAs bound these kernels: at d = 128 the gradient stage of a chunk-head is 6.8 M of them, 28 us at the rate of one SM;
+// measured 55 us (forward preparation 22 us, the backward's share of it 21 us).  With the operands of every FMA read from
+// global memory, and the solve and the sums over a chunk done by single threads, the same stages took 907, 165 and 102 us
+// (2 x 4 heads of 1000 tokens); the smallest call, 2 heads of 128 tokens at d = 64, went from 370 to 53 us.
+#include "ffma_scan.cuh"
+#include "tc_inverse.cuh"
 
 namespace gdn {
 namespace {
+
+using namespace ffma;
 
 // ------------------------------------------------------------------------------------------------
 // Chunk table.  One block.  Validates cu_seqlens; on failure records the status and leaves no work.
@@ -70,475 +78,554 @@ __global__ void table_kernel(Problem p) {
     }
 }
 
-// Loads the gate rows of a chunk: g (0 when padded), erase gate b, write gate w.
-__device__ __forceinline__ void load_gates(const Problem& p, const ChunkCtx& x, int i, float& g, float& b, float& w) {
-    g = 0.f; b = 0.f; w = 0.f;
-    if (i < x.len) {
-        const size_t idx = (size_t)(x.tok0 + i) * p.d.H + x.hd;
-        g = p.g[idx];
-        if (p.d.delta_rule) { b = p.beta[idx]; w = b; } else { b = 0.f; w = 1.f; }
+// One (chunk, head) of the grid; false when there is none or an earlier stage has failed.
+__device__ __forceinline__ bool chunk_head(const Problem& p, ChunkInfo& x) {
+    return reinterpret_cast<const WsHeader*>(p.ws)->status == GDN_OK && chunk_info(p, x);
+}
+
+// Gate arrays of a chunk in shared memory, made by warp 0: lane l owns tokens l and l + 32.
+struct Gates {
+    float gam[kC], Gam[kC], ee[kC];   // cumulative log decay, its exponential, exp(gam_e - gam)
+    float bb[kC], ww[kC];             // erase and write gate (0 beyond the sequence)
+};
+__device__ __forceinline__ void finish_gates(Gates& s, int lane, float a, float b, float gend) {
+    s.gam[lane] = a; s.gam[lane + 32] = b;
+    s.Gam[lane] = expf(a); s.Gam[lane + 32] = expf(b);
+    s.ee[lane] = expf(gend - a); s.ee[lane + 32] = expf(gend - b);
+}
+__device__ __forceinline__ void load_erase_write(const Problem& p, const ChunkInfo& x, Gates& s, int lane) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int i = lane + 32 * h;
+        const bool live = i < x.len;
+        const float beta = live && p.d.delta_rule ? p.beta[(size_t)(x.tok0 + i) * p.d.H + x.hd] : 0.f;
+        s.bb[i] = beta;
+        s.ww[i] = p.d.delta_rule ? beta : (live ? 1.f : 0.f);
     }
+}
+// ... from the log decays: inclusive sums over the chunk; gam goes to the workspace for the other stages.
+__device__ __forceinline__ void make_gates(const Problem& p, const ChunkInfo& x, Gates& s, float* wsG) {
+    const int lane = threadIdx.x;
+    auto g = [&](int i) { return i < x.len ? p.g[(size_t)(x.tok0 + i) * p.d.H + x.hd] : 0.f; };
+    float a = g(lane), b = g(lane + 32);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float ua = __shfl_up_sync(0xffffffffu, a, o), ub = __shfl_up_sync(0xffffffffu, b, o);
+        if (lane >= o) { a += ua; b += ub; }
+    }
+    b += __shfl_sync(0xffffffffu, a, 31);
+    const float gend = __shfl_sync(0xffffffffu, b, 31);
+    wsG[lane] = a; wsG[lane + 32] = b;
+    finish_gates(s, lane, a, b, gend);
+    load_erase_write(p, x, s, lane);
+}
+// ... from the stored gam.
+__device__ __forceinline__ void load_gates(const Problem& p, const ChunkInfo& x, Gates& s, const float* wsG) {
+    finish_gates(s, threadIdx.x, wsG[threadIdx.x], wsG[threadIdx.x + 32], wsG[kC - 1]);
+    load_erase_write(p, x, s, threadIdx.x);
+}
+
+template <typename IO>
+__device__ __forceinline__ const IO* rows_of(const void* base, const ChunkInfo& x, int H, int d) {
+    return reinterpret_cast<const IO*>(base) + ((size_t)x.tok0 * H + x.hd) * d;
+}
+template <typename IO>
+__device__ __forceinline__ IO* rows_of(void* base, const ChunkInfo& x, int H, int d) {
+    return reinterpret_cast<IO*>(base) + ((size_t)x.tok0 * H + x.hd) * d;
+}
+__device__ __forceinline__ float* block_of(const Problem& p, size_t region, int ch, int floats) {
+    return reinterpret_cast<float*>(p.ws + region) + (size_t)ch * floats;
 }
 
 // ------------------------------------------------------------------------------------------------
 // prep
 // ------------------------------------------------------------------------------------------------
-template <typename IO, int DK, int DV>
-__global__ void __launch_bounds__(kThreads) prep_kernel(Problem p) {
-    ChunkCtx x;
-    if (!chunk_ctx(p, x)) return;
-    __shared__ float gam[kC], Gam[kC], ee[kC], bb[kC], ww[kC];
-    __shared__ float A[kC][kC + 1], Ti[kC][kC + 1];
-    const int H = p.d.H;
-    const IO* kp = reinterpret_cast<const IO*>(p.k) + ((size_t)x.tok0 * H + x.hd) * DK;
-    const IO* vp = reinterpret_cast<const IO*>(p.v) + ((size_t)x.tok0 * H + x.hd) * DV;
-    const size_t rk = (size_t)H * DK, rv = (size_t)H * DV;
-    auto Kf = [&](int i, int m) -> float { return i < x.len ? ldf(kp + i * rk + m) : 0.f; };
-    auto Vf = [&](int i, int m) -> float { return i < x.len ? ldf(vp + i * rv + m) : 0.f; };
-    float* wsG = reinterpret_cast<float*>(p.ws + p.L.gamma) + (size_t)x.ch * kC;
-    float* wsT = reinterpret_cast<float*>(p.ws + p.L.Tm) + (size_t)x.ch * kC * kC;
-    float* wsW = reinterpret_cast<float*>(p.ws + p.L.W) + (size_t)x.ch * kC * DK;
-    float* wsU = reinterpret_cast<float*>(p.ws + p.L.Ut) + (size_t)x.ch * kC * DV;
-    float* wsN = reinterpret_cast<float*>(p.ws + p.L.Nm) + (size_t)x.ch * DK * DK;
-    float* wsB = reinterpret_cast<float*>(p.ws + p.L.Bf) + (size_t)x.ch * DK * DV;
+enum PrepMode { PREP_FWD = 0, PREP_FWD_BWD = 1, PREP_BWD = 2 };
+template <int DK, int DV>
+constexpr size_t prep_smem() {
+    return sizeof(float) * (kC * (2 * pitch(DK) + pitch(DK > DV ? DK : DV) + pitch(DV)) + 4 * kC * kPc);
+}
 
-    if (threadIdx.x < kC) {
-        float g, b, w;
-        load_gates(p, x, threadIdx.x, g, b, w);
-        gam[threadIdx.x] = g; bb[threadIdx.x] = b; ww[threadIdx.x] = w;
+template <typename IO, int DK, int DV>
+__global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) {
+    const bool fwd = mode != PREP_BWD, bwd = mode != PREP_FWD;
+    init_header_if_untabled(p);
+    ChunkInfo x;
+    if (!chunk_info(p, x)) return;   // (no chunk at all when the table was refused)
+    constexpr int PK = pitch(DK), PV = pitch(DV);
+    extern __shared__ __align__(16) float sm[];
+    float* sK = sm;                                   // K
+    float* sQ = sK + kC * PK;                         // Q, then X = Diag(Gam) Q - P W
+    float* sV = sQ + kC * PK;                         // V, then W
+    float* sO = sV + kC * pitch(DK > DV ? DK : DV);   // dO
+    float* A = sO + kC * PV;                          // A, then T Diag(w)
+    float* T = A + kC * kPc;
+    float* S = T + kC * kPc;                          // scratch of the inversion, then T Diag(b Gam)
+    float* Pm = S + kC * kPc;
+    __shared__ Gates gs;
+    const int H = p.d.H, tid = threadIdx.x;
+    const Thread t;
+    const Out<DK> ok(t);
+    const Out<DV> ov(t);
+    const size_t rk = (size_t)H * DK, rv = (size_t)H * DV;
+    float* wsG = block_of(p, p.L.gamma, x.ch, kC);
+    float* wsW = block_of(p, p.L.W, x.ch, kC * DK);
+    float* wsP = block_of(p, p.L.Pm, x.ch, kC * kC);
+    const float sc = p.d.scale;
+
+    load_rows<DK>(sQ, rows_of<IO>(p.q, x, H, DK), rk, x.len);
+    if (fwd) load_rows<DK>(sK, rows_of<IO>(p.k, x, H, DK), rk, x.len);
+    cp_commit();
+    if (fwd) {
+        load_rows<DV>(sV, rows_of<IO>(p.v, x, H, DV), rv, x.len);
+    } else {
+        load_block<kC, DK>(sV, wsW);
+        load_block<kC, kC>(Pm, wsP);
+    }
+    if (bwd) load_rows<DV>(sO, rows_of<IO>(p.dO, x, H, DV), rv, x.len);
+    cp_commit();
+    if (tid < 32) { if (fwd) make_gates(p, x, gs, wsG); else load_gates(p, x, gs, wsG); }
+    if (fwd) {
+        cp_wait<1>();
+        __syncthreads();
+        // P = tril(Q K^T . D) and A = stril(Diag(b)(K K^T . D)) in one pass over K; the decay exponent is only evaluated where
+        // j <= i (non-positive)
+        {
+            float acc[8][4];
+            zero(acc);
+            mac<2, A_ROW, B_ROW>(acc, sQ, sK, PK, t.rn, sK, PK, t.cn, 0, DK);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                    const int i = t.rn + r, j = t.cn + 8 * y;
+                    const float D = j <= i ? expf(gs.gam[i] - gs.gam[j]) : 0.f;
+                    const float P_ = j <= i ? acc[r][y] * D : 0.f;
+                    Pm[i * kPc + j] = P_;
+                    wsP[i * kC + j] = P_;
+                    A[i * kPc + j] = j < i ? gs.bb[i] * acc[4 + r][y] * D : 0.f;
+                }
+        }
+        // Kb = Diag(exp(gam_e - gam)) K, for the carries
+        float* wsKb = block_of(p, p.L.Kb, x.ch, kC * DK);
+        for (int e = tid; e < kC * DK / 4; e += kThreads) {
+            const int i = e / (DK / 4), c = (e % (DK / 4)) * 4;
+            float4 k = ld4(sK + i * PK + c);
+            const float w = gs.ee[i];
+            *reinterpret_cast<float4*>(wsKb + (size_t)e * 4) = make_float4(w * k.x, w * k.y, w * k.z, w * k.w);
+        }
+        __syncthreads();
+        // T = (I + A)^-1, blocked (the blocks above the block diagonal are not written: zero them)
+        for (int e = tid; e < kC * kC; e += kThreads)
+            if ((e % kC) / 16 > e / kC / 16) T[(e / kC) * kPc + e % kC] = 0.f;
+        static_assert(kPc == kLdi, "the inversion works on the tiles of this family");
+        inv_diag8(A, T);
+        __syncthreads();
+        inv_diag16(A, T, S);
+        __syncthreads();
+        inv_premul<2>(A, T, S);
+        __syncthreads();
+        inv_level<1, 1, 2>(S, T);
+        __syncthreads();
+        inv_level<2, 2, 2>(S, T);
+        __syncthreads();
+        inv_level<3, 4, 2>(S, T);
+        cp_wait<0>();
+        __syncthreads();
+        float* wsT = block_of(p, p.L.Tm, x.ch, kC * kC);
+        for (int e = tid; e < kC * kC; e += kThreads) {
+            const int i = e / kC, j = e % kC;
+            const float v = T[i * kPc + j];
+            wsT[e] = v;
+            S[i * kPc + j] = v * gs.bb[j] * gs.Gam[j];
+            A[i * kPc + j] = v * gs.ww[j];
+        }
+        __syncthreads();
+        // Ut = T Diag(w) V, then W = T Diag(b Gam) K (over V)
+        float* wsU = block_of(p, p.L.Ut, x.ch, kC * DV);
+        {
+            float acc[Out<DV>::R][4];
+            tri_product<DV, A_ROW, A_LOWER>(t, A, sV, PV, acc);
+#pragma unroll
+            for (int r = 0; r < Out<DV>::R; ++r)
+#pragma unroll
+                for (int y = 0; y < 4; ++y) wsU[ov.row(r) * DV + ov.c + 8 * y] = acc[r][y];
+        }
+        __syncthreads();
+        {
+            float acc[Out<DK>::R][4];
+            tri_product<DK, A_ROW, A_LOWER>(t, S, sK, PK, acc);
+#pragma unroll
+            for (int r = 0; r < Out<DK>::R; ++r)
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                    wsW[ok.row(r) * DK + ok.c + 8 * y] = acc[r][y];
+                    sV[ok.row(r) * PK + ok.c + 8 * y] = acc[r][y];
+                }
+        }
+        if (!bwd) return;
+    } else {
+        cp_wait<0>();
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float s = 0.f;
-        for (int i = 0; i < kC; ++i) { s += gam[i]; gam[i] = s; }
+    // dU0 = scale P^T dO
+    float* wsD = block_of(p, p.L.dU, x.ch, kC * DV);
+    {
+        float acc[Out<DV>::R][4];
+        tri_product<DV, A_COL, A_UPPER>(t, Pm, sO, PV, acc);
+#pragma unroll
+        for (int r = 0; r < Out<DV>::R; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) wsD[ov.row(r) * DV + ov.c + 8 * y] = sc * acc[r][y];
     }
-    __syncthreads();
-    if (threadIdx.x < kC) {
-        const int i = threadIdx.x;
-        Gam[i] = expf(gam[i]);
-        ee[i] = expf(gam[kC - 1] - gam[i]);
-        wsG[i] = gam[i];
-    }
-    // A = stril(Diag(b) (K K^T . D)); the decay exponent is only evaluated where j < i (non-positive).
-    tiles(kC, kC, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        if (j0 < i0 + 4) mac(acc, i0, j0, DK, Kf, [&](int m, int j) { return Kf(j, m); });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-                const int i = i0 + a, j = j0 + b;
-                A[i][j] = (j < i) ? bb[i] * acc[a][b] * expf(gam[i] - gam[j]) : 0.f;
-            }
-    });
-    __syncthreads();
-    // T = (I + A)^-1: column j of T solves (I + A) x = e_j by forward substitution (one thread per column).
-    if (threadIdx.x < kC) {
-        const int j = threadIdx.x;
-        for (int i = 0; i < kC; ++i) {
-            float s = (i == j) ? 1.f : 0.f;
-            for (int m = j; m < i; ++m) s = fmaf(-A[i][m], Ti[m][j], s);
-            Ti[i][j] = (i >= j) ? s : 0.f;
+    {   // X = Diag(Gam) Q - P W, in place over Q
+        float acc[Out<DK>::R][4];
+        tri_product<DK, A_ROW, A_LOWER>(t, Pm, sV, PK, acc);
+#pragma unroll
+        for (int r = 0; r < Out<DK>::R; ++r) {
+            float* q = sQ + ok.row(r) * PK + ok.c;
+            const float G = gs.Gam[ok.row(r)];
+#pragma unroll
+            for (int y = 0; y < 4; ++y) q[8 * y] = G * q[8 * y] - acc[r][y];
         }
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < kC * kC; t += blockDim.x) wsT[t] = Ti[t / kC][t % kC];
-    // W = T Diag(b Gam) K,  Ut = T Diag(w) V
-    tiles(kC, DK, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, kC, [&](int i, int m) { return Ti[i][m]; }, [&](int m, int j) { return bb[m] * Gam[m] * Kf(m, j); });
-        for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) wsW[(i0 + a) * DK + j0 + b] = acc[a][b];
-    });
-    tiles(kC, DV, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, kC, [&](int i, int m) { return Ti[i][m]; }, [&](int m, int j) { return ww[m] * Vf(m, j); });
-        for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) wsU[(i0 + a) * DV + j0 + b] = acc[a][b];
-    });
-    __syncthreads();
-    // Nm = Kb^T W,  Bf = Kb^T Ut,  Kb = Diag(exp(gam_e - gam)) K
-    tiles(DK, DK, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, kC, [&](int i, int m) { return ee[m] * Kf(m, i); }, [&](int m, int j) { return wsW[m * DK + j]; });
-        for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) wsN[(i0 + a) * DK + j0 + b] = acc[a][b];
-    });
-    tiles(DK, DV, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, kC, [&](int i, int m) { return ee[m] * Kf(m, i); }, [&](int m, int j) { return wsU[m * DV + j]; });
-        for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) wsB[(i0 + a) * DV + j0 + b] = acc[a][b];
-    });
-}
-
-// ------------------------------------------------------------------------------------------------
-// eprep: E = scale (Diag(Gam) Q - P W)^T dO
-// ------------------------------------------------------------------------------------------------
-template <typename IO, int DK, int DV>
-__global__ void __launch_bounds__(kThreads) eprep_kernel(Problem p) {
-    ChunkCtx x;
-    if (!chunk_ctx(p, x)) return;
-    __shared__ float gam[kC];
-    __shared__ float P[kC][kC + 1];
-    const int H = p.d.H;
-    const IO* qp = reinterpret_cast<const IO*>(p.q) + ((size_t)x.tok0 * H + x.hd) * DK;
-    const IO* kp = reinterpret_cast<const IO*>(p.k) + ((size_t)x.tok0 * H + x.hd) * DK;
-    const IO* gp = reinterpret_cast<const IO*>(p.dO) + ((size_t)x.tok0 * H + x.hd) * DV;
-    const size_t rk = (size_t)H * DK, rv = (size_t)H * DV;
-    auto Qf = [&](int i, int m) -> float { return i < x.len ? ldf(qp + i * rk + m) : 0.f; };
-    auto Kf = [&](int i, int m) -> float { return i < x.len ? ldf(kp + i * rk + m) : 0.f; };
-    auto Gf = [&](int i, int m) -> float { return i < x.len ? ldf(gp + i * rv + m) : 0.f; };
-    const float* wsG = reinterpret_cast<const float*>(p.ws + p.L.gamma) + (size_t)x.ch * kC;
-    const float* wsW = reinterpret_cast<const float*>(p.ws + p.L.W) + (size_t)x.ch * kC * DK;
-    float* wsE = reinterpret_cast<float*>(p.ws + p.L.E) + (size_t)x.ch * DK * DV;
-    float* X = reinterpret_cast<float*>(p.ws + p.L.scratch + p.L.scratch_per_ch * x.ch);  // [64, DK]
-    if (threadIdx.x < kC) gam[threadIdx.x] = wsG[threadIdx.x];
-    __syncthreads();
-    tiles(kC, kC, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        if (j0 <= i0 + 3) mac(acc, i0, j0, DK, Qf, [&](int m, int j) { return Kf(j, m); });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-                const int i = i0 + a, j = j0 + b;
-                P[i][j] = (j <= i) ? acc[a][b] * expf(gam[i] - gam[j]) : 0.f;
-            }
-    });
-    __syncthreads();
-    tiles(kC, DK, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, kC, [&](int i, int m) { return P[i][m]; }, [&](int m, int j) { return wsW[m * DK + j]; });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) X[(i0 + a) * DK + j0 + b] = expf(gam[i0 + a]) * Qf(i0 + a, j0 + b) - acc[a][b];
-    });
-    __syncthreads();
-    const float sc = p.d.scale;
-    tiles(DK, DV, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, kC, [&](int i, int m) { return X[m * DK + i]; }, Gf);
-        for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) wsE[(i0 + a) * DV + j0 + b] = sc * acc[a][b];
-    });
-}
-
-// ------------------------------------------------------------------------------------------------
-// Forward and reverse carries.  One CTA per (sequence, head); the fp32 state lives in shared memory.
-// REVERSE = false:  h' = Gam_e h - Nm h + Bf, stores h entering each chunk, optional final state.
-// REVERSE = true :  dh = Gam_e dh' - Nm^T dh' + E, stores dh' per chunk, optional dh0.
-// ------------------------------------------------------------------------------------------------
-template <int DK, int DV, bool REVERSE>
-__global__ void __launch_bounds__(kThreads) scan_kernel(Problem p) {
-    extern __shared__ float sm[];
-    float* cur = sm;
-    float* nxt = sm + DK * DV;
-    const int n = blockIdx.x / p.d.H, hd = blockIdx.x % p.d.H;
-    const int32_t* seq_first = reinterpret_cast<const int32_t*>(p.ws + p.L.seq_first);
-    const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
-    if (hdr->status != GDN_OK) return;
-    const int c0 = seq_first[n], c1 = seq_first[n + 1];
-    const size_t soff = ((size_t)n * p.d.H + hd) * DK * DV;
-    const float* init = REVERSE ? p.dhT : p.h0;
-    for (int t = threadIdx.x; t < DK * DV; t += blockDim.x) cur[t] = init ? init[soff + t] : 0.f;
-    __syncthreads();
-    for (int s = 0; s < c1 - c0; ++s) {
-        const int c = REVERSE ? (c1 - 1 - s) : (c0 + s);
-        const size_t ch = (size_t)c * p.d.H + hd;
-        const float* wsN = reinterpret_cast<const float*>(p.ws + p.L.Nm) + ch * DK * DK;
-        const float* add = reinterpret_cast<const float*>(p.ws + (REVERSE ? p.L.E : p.L.Bf)) + ch * DK * DV;
-        float* keep = reinterpret_cast<float*>(p.ws + (REVERSE ? p.L.dhn : p.L.hc)) + ch * DK * DV;
-        const float Ge = expf(reinterpret_cast<const float*>(p.ws + p.L.gamma)[ch * kC + kC - 1]);
-        for (int t = threadIdx.x; t < DK * DV; t += blockDim.x) keep[t] = cur[t];
-        tiles(DK, DV, [&](int i0, int j0) {
-            float acc[4][4] = {};
-            mac(acc, i0, j0, DK, [&](int i, int m) { return REVERSE ? wsN[m * DK + i] : wsN[i * DK + m]; },
-                [&](int m, int j) { return cur[m * DV + j]; });
-            for (int a = 0; a < 4; ++a)
-                for (int b = 0; b < 4; ++b) {
-                    const int t = (i0 + a) * DV + j0 + b;
-                    nxt[t] = Ge * cur[t] - acc[a][b] + add[t];
-                }
-        });
-        __syncthreads();
-        float* tmp = cur; cur = nxt; nxt = tmp;
+    // E = scale X^T dO, 64 rows at a time
+    float* wsE = block_of(p, p.L.E, x.ch, DK * DV);
+#pragma unroll 1
+    for (int r0 = 0; r0 < DK; r0 += 64) {
+        float acc[Out<DV>::R][4];
+        zero(acc);
+        mac<Out<DV>::R / 4, A_COL, B_COL>(acc, sQ + r0, sQ + r0 + 32, PK, ov.r0, sO, PV, ov.c, 0, kC);
+#pragma unroll
+        for (int r = 0; r < Out<DV>::R; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) wsE[(r0 + ov.row(r)) * DV + ov.c + 8 * y] = sc * acc[r][y];
     }
-    float* fin = REVERSE ? p.dh0 : p.hT;
-    if (fin) for (int t = threadIdx.x; t < DK * DV; t += blockDim.x) fin[soff + t] = cur[t];
 }
 
 // ------------------------------------------------------------------------------------------------
-// Forward output (optional): o = scale (Diag(Gam) Q h + P (Ut - W h))
+// Forward and reverse carries (ffma_scan.cuh).
 // ------------------------------------------------------------------------------------------------
+template <int DK, int DV>
+__global__ void __launch_bounds__(kThreads) scan_kernel(Problem p, int dirs) {
+    extern __shared__ __align__(16) float sm[];
+    if (reinterpret_cast<const WsHeader*>(p.ws)->status != GDN_OK) return;
+    scan_block<DK, DV, false>(p, dirs, sm);
+}
+
+// ------------------------------------------------------------------------------------------------
+// Forward output (optional): o = scale (Diag(Gam) Q h + P U)
+// ------------------------------------------------------------------------------------------------
+template <int DK, int DV>
+constexpr size_t out_smem() { return sizeof(float) * (kC * pitch(DK) + DK * pitch(DV) + kC * pitch(DV) + kC * kPc); }
+
 template <typename IO, int DK, int DV>
-__global__ void __launch_bounds__(kThreads) out_kernel(Problem p) {
-    ChunkCtx x;
-    if (!chunk_ctx(p, x)) return;
-    __shared__ float gam[kC];
-    __shared__ float P[kC][kC + 1];
+__global__ void __launch_bounds__(kThreads, 1) out_kernel(Problem p) {
+    ChunkInfo x;
+    if (!chunk_head(p, x)) return;
+    constexpr int PK = pitch(DK), PV = pitch(DV);
+    extern __shared__ __align__(16) float sm[];
+    float* sQ = sm;
+    float* sH = sQ + kC * PK;
+    float* sU = sH + DK * PV;
+    float* Pm = sU + kC * PV;
     const int H = p.d.H;
-    const IO* qp = reinterpret_cast<const IO*>(p.q) + ((size_t)x.tok0 * H + x.hd) * DK;
-    const IO* kp = reinterpret_cast<const IO*>(p.k) + ((size_t)x.tok0 * H + x.hd) * DK;
-    IO* op = reinterpret_cast<IO*>(p.o) + ((size_t)x.tok0 * H + x.hd) * DV;
-    const size_t rk = (size_t)H * DK, rv = (size_t)H * DV;
-    auto Qf = [&](int i, int m) -> float { return i < x.len ? ldf(qp + i * rk + m) : 0.f; };
-    auto Kf = [&](int i, int m) -> float { return i < x.len ? ldf(kp + i * rk + m) : 0.f; };
-    const float* wsG = reinterpret_cast<const float*>(p.ws + p.L.gamma) + (size_t)x.ch * kC;
-    const float* wsW = reinterpret_cast<const float*>(p.ws + p.L.W) + (size_t)x.ch * kC * DK;
-    const float* wsU = reinterpret_cast<const float*>(p.ws + p.L.Ut) + (size_t)x.ch * kC * DV;
-    const float* h = reinterpret_cast<const float*>(p.ws + p.L.hc) + (size_t)x.ch * DK * DV;
-    float* U = reinterpret_cast<float*>(p.ws + p.L.scratch + p.L.scratch_per_ch * x.ch);  // [64, DV]
-    if (threadIdx.x < kC) gam[threadIdx.x] = wsG[threadIdx.x];
-    __syncthreads();
-    tiles(kC, kC, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        if (j0 <= i0 + 3) mac(acc, i0, j0, DK, Qf, [&](int m, int j) { return Kf(j, m); });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-                const int i = i0 + a, j = j0 + b;
-                P[i][j] = (j <= i) ? acc[a][b] * expf(gam[i] - gam[j]) : 0.f;
-            }
-    });
-    tiles(kC, DV, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, DK, [&](int i, int m) { return wsW[i * DK + m]; }, [&](int m, int j) { return h[m * DV + j]; });
-        for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) U[(i0 + a) * DV + j0 + b] = wsU[(i0 + a) * DV + j0 + b] - acc[a][b];
-    });
-    __syncthreads();
+    const Thread t;
+    load_rows<DK>(sQ, rows_of<IO>(p.q, x, H, DK), (size_t)H * DK, x.len);
+    load_block<DK, DV>(sH, block_of(p, p.L.hc, x.ch, DK * DV));
+    cp_commit();
+    load_block<kC, DV>(sU, block_of(p, p.L.U, x.ch, kC * DV));
+    load_block<kC, kC>(Pm, block_of(p, p.L.Pm, x.ch, kC * kC));
+    cp_commit();
+    const float* wsG = block_of(p, p.L.gamma, x.ch, kC);
+    IO* op = rows_of<IO>(p.o, x, H, DV);
+    const size_t rv = (size_t)H * DV;
     const float sc = p.d.scale;
-    tiles(kC, DV, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, DK, [&](int i, int m) { return expf(gam[i]) * Qf(i, m); }, [&](int m, int j) { return h[m * DV + j]; });
-        mac(acc, i0, j0, kC, [&](int i, int m) { return P[i][m]; }, [&](int m, int j) { return U[m * DV + j]; });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b)
-                if (i0 + a < x.len) stf(op + (i0 + a) * rv + j0 + b, sc * acc[a][b]);
-    });
+    cp_wait<1>();
+    __syncthreads();
+    const Out<DV> o(t);
+    constexpr int R = Out<DV>::R;
+    float acc[R][4];
+    zero(acc);
+    mac<R / 4, A_ROW, B_COL>(acc, sQ, sQ + 32 * PK, PK, o.r0, sH, PV, o.c, 0, DK);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const float G = expf(wsG[o.row(r)]);
+#pragma unroll
+        for (int y = 0; y < 4; ++y) acc[r][y] *= G;
+    }
+    cp_wait<0>();
+    __syncthreads();
+    mac<R / 4, A_ROW, B_COL>(acc, Pm, Pm + 32 * kPc, kPc, o.r0, sU, PV, o.c, 0, kC);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (o.row(r) < x.len)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) stf(op + o.row(r) * rv + o.c + 8 * y, sc * acc[r][y]);
 }
 
 // ------------------------------------------------------------------------------------------------
 // intra: token gradients of one (chunk, head).
+//
+// The solve's VJP (K#2) in its short form: dXv = T^T dU, dXk = -dXv h^T, dA = -stril(dXv U^T).  With dPD = scale
+// tril(dO U^T) . D and G = dA . D:
+//     dq = scale Gam (dO h^T) + dPD K        dk^row = G K + Gam dXk       dv = w dXv
+//     dk = b dk^row + dk^col                 dk^col = e (U dh'^T) + dPD^T Q + (b G)^T K
+//     dgam_i = <q, dq> + b <k, dk^row> - <k, dk^col>, and the last row adds sum_j e_j <k_j, (U dh'^T)_j> + Gam_e <dh', h>
+// Tiles: dO, U, dU (then dXv) and h first; K and Q over dO and dXv, dh' over h, once the products with h are done (their
+// results wait in registers: at d = 128 the seven tiles do not fit beside each other).
 // ------------------------------------------------------------------------------------------------
-struct IntraSmem {
-    float gam[kC], Gam[kC], ee[kC], bb[kC], ww[kC];
-    float r[kC], rq[kC], xk[kC], xv[kC], dgam[kC];
-    float red[kThreads / 32];
-    float P[kC][kC + 1];    // tril(Q K^T . D)
-    float KK[kC][kC + 1];   // K K^T, later Z = G . KK
-    float dP[kC][kC + 1];   // scale tril(dO U^T)
-    float G[kC][kC + 1];    // dA . D
-};
+template <int DK, int DV>
+constexpr size_t intra_smem() {
+    constexpr int PM = pitch(DK > DV ? DK : DV);
+    return sizeof(float) * (2 * kC * PM + kC * pitch(DV) + DK * pitch(DV) + 3 * kC * kPc);
+}
 
 template <typename IO, int DK, int DV>
-__global__ void __launch_bounds__(kThreads) intra_kernel(Problem p) {
-    ChunkCtx x;
-    if (!chunk_ctx(p, x)) return;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    IntraSmem& S = *reinterpret_cast<IntraSmem*>(smraw);
-    const int H = p.d.H;
-    const size_t base_k = ((size_t)x.tok0 * H + x.hd) * DK, base_v = ((size_t)x.tok0 * H + x.hd) * DV;
+__global__ void __launch_bounds__(kThreads, DK + DV == 128 ? 2 : 1) intra_kernel(Problem p) {
+    ChunkInfo x;
+    if (!chunk_head(p, x)) return;
+    constexpr int PK = pitch(DK), PV = pitch(DV), PM = pitch(DK > DV ? DK : DV), NH = DK / 64;
+    extern __shared__ __align__(16) float sm[];
+    float* s0 = sm;                  // dO, then K
+    float* s1 = s0 + kC * PM;        // dU, then dXv, then Q
+    float* sU = s1 + kC * PM;        // U
+    float* sH = sU + kC * PV;        // h, then dh'
+    float* sT = sH + DK * PV;        // T, then G
+    float* sB = sT + kC * kPc;       // Diag(b) G
+    float* sP = sB + kC * kPc;       // dPD
+    __shared__ Gates gs;
+    __shared__ float red[4][4][kC];  // row dots <q, dq>, <k, dk^row>, <k, dk^col>, <v, dXv>: [which][column block][row]
+    __shared__ float dgam[kC], part[2][kThreads / 32];
+    const int H = p.d.H, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const Thread t;
     const size_t rk = (size_t)H * DK, rv = (size_t)H * DV;
-    const IO* qp = reinterpret_cast<const IO*>(p.q) + base_k;
-    const IO* kp = reinterpret_cast<const IO*>(p.k) + base_k;
-    const IO* vp = reinterpret_cast<const IO*>(p.v) + base_v;
-    const IO* gp = reinterpret_cast<const IO*>(p.dO) + base_v;
-    IO* dqp = reinterpret_cast<IO*>(p.dq) + base_k;
-    IO* dkp = reinterpret_cast<IO*>(p.dk) + base_k;
-    IO* dvp = reinterpret_cast<IO*>(p.dv) + base_v;
-    auto Qf = [&](int i, int m) -> float { return i < x.len ? ldf(qp + i * rk + m) : 0.f; };
-    auto Kf = [&](int i, int m) -> float { return i < x.len ? ldf(kp + i * rk + m) : 0.f; };
-    auto Vf = [&](int i, int m) -> float { return i < x.len ? ldf(vp + i * rv + m) : 0.f; };
-    auto Of = [&](int i, int m) -> float { return i < x.len ? ldf(gp + i * rv + m) : 0.f; };
-    const float* wsG = reinterpret_cast<const float*>(p.ws + p.L.gamma) + (size_t)x.ch * kC;
-    const float* Tm = reinterpret_cast<const float*>(p.ws + p.L.Tm) + (size_t)x.ch * kC * kC;
-    const float* W = reinterpret_cast<const float*>(p.ws + p.L.W) + (size_t)x.ch * kC * DK;
-    const float* Ut = reinterpret_cast<const float*>(p.ws + p.L.Ut) + (size_t)x.ch * kC * DV;
-    const float* h = reinterpret_cast<const float*>(p.ws + p.L.hc) + (size_t)x.ch * DK * DV;
-    const float* dhn = reinterpret_cast<const float*>(p.ws + p.L.dhn) + (size_t)x.ch * DK * DV;
-    float* scr = reinterpret_cast<float*>(p.ws + p.L.scratch + p.L.scratch_per_ch * x.ch);
-    float* U = scr;                    // [64, DV]
-    float* dU = U + kC * DV;           // [64, DV]
-    float* dXv = dU + kC * DV;         // [64, DV]  (first holds Kb dh')
-    float* dOh = dXv + kC * DV;        // [64, DK]  dO h^T
-    float* dW = dOh + kC * DK;         // [64, DK]
-    float* dXk = dW + kC * DK;         // [64, DK]
     const float sc = p.d.scale;
+    const float* wsH = block_of(p, p.L.hc, x.ch, DK * DV);
 
-    if (threadIdx.x < kC) {
-        const int i = threadIdx.x;
-        float g, b, w;
-        load_gates(p, x, i, g, b, w);
-        (void)g;
-        S.bb[i] = b; S.ww[i] = w;
-        S.gam[i] = wsG[i];
+    load_rows<DV>(s0, rows_of<IO>(p.dO, x, H, DV), rv, x.len);
+    load_block<kC, DV>(sU, block_of(p, p.L.U, x.ch, kC * DV));
+    cp_commit();
+    load_block<kC, DV>(s1, block_of(p, p.L.dU, x.ch, kC * DV));
+    load_block<kC, kC>(sT, block_of(p, p.L.Tm, x.ch, kC * kC));
+    cp_commit();
+    load_block<DK, DV>(sH, wsH);
+    cp_commit();
+    if (tid < 32) load_gates(p, x, gs, block_of(p, p.L.gamma, x.ch, kC));
+    cp_wait<2>();
+    __syncthreads();
+    // 64 x 64 matrices: warps whose 16 x 32 block lies above the diagonal have nothing to add up
+    const bool below = (warp >> 2) * 32 <= (t.rn >> 4) * 16 + 15;
+    {   // dPD = scale tril(dO U^T) . D; the decay exponent is only evaluated where it is non-positive
+        float acc[4][4];
+        zero(acc);
+        if (below) mac<1, A_ROW, B_ROW>(acc, s0, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int i = t.rn + r, j = t.cn + 8 * y;
+                sP[i * kPc + j] = j <= i ? sc * acc[r][y] * expf(gs.gam[i] - gs.gam[j]) : 0.f;
+            }
+    }
+    cp_wait<1>();
+    __syncthreads();
+    {   // dXv = T^T dU, in place; dv = w dXv; <v, dXv>
+        const Out<DV> o(t);
+        constexpr int R = Out<DV>::R;
+        float acc[R][4], vv[R][4];
+        const IO* vp = rows_of<IO>(p.v, x, H, DV);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) vv[r][y] = o.row(r) < x.len ? ldf(vp + o.row(r) * rv + o.c + 8 * y) : 0.f;
+        tri_product<DV, A_COL, A_UPPER>(t, sT, s1, PV, acc);
+        __syncthreads();
+        IO* dvp = rows_of<IO>(p.dv, x, H, DV);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int i = o.row(r);
+            const float w = gs.ww[i];
+            float dot = 0.f;
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                s1[i * PV + o.c + 8 * y] = acc[r][y];
+                dot = fmaf(vv[r][y], acc[r][y], dot);
+                if (i < x.len) stf(dvp + i * rv + o.c + 8 * y, w * acc[r][y]);
+            }
+            dot = row_sum8(dot);
+            if ((lane & 7) == 0) red[3][DV == 128 ? warp >> 1 : warp >> 2][i] = dot;
+        }
+    }
+    cp_wait<0>();
+    __syncthreads();
+    {   // G = -stril(dXv U^T) . D and Diag(b) G (over T)
+        float acc[4][4];
+        zero(acc);
+        if (below) mac<1, A_ROW, B_ROW>(acc, s1, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int i = t.rn + r, j = t.cn + 8 * y;
+                const float g = j < i ? -acc[r][y] * expf(gs.gam[i] - gs.gam[j]) : 0.f;
+                sT[i * kPc + j] = g;
+                sB[i * kPc + j] = gs.bb[i] * g;
+            }
+    }
+    // [dO; dXv] h^T: rows 0..3 become dq, rows 4..7 dk^row
+    float acc[NH][8][4];
+#pragma unroll
+    for (int n = 0; n < NH; ++n) {
+        zero(acc[n]);
+        mac<2, A_ROW, B_ROW>(acc[n], s0, s1, PV, t.rn, sH + n * 64 * PV, PV, t.cn, 0, DV);
     }
     __syncthreads();
-    if (threadIdx.x < kC) {
-        const int i = threadIdx.x;
-        S.Gam[i] = expf(S.gam[i]);
-        S.ee[i] = expf(S.gam[kC - 1] - S.gam[i]);
+    load_rows<DK>(s0, rows_of<IO>(p.k, x, H, DK), rk, x.len);
+    cp_commit();
+    load_rows<DK>(s1, rows_of<IO>(p.q, x, H, DK), rk, x.len);
+    load_block<DK, DV>(sH, block_of(p, p.L.dhn, x.ch, DK * DV));
+    cp_commit();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const float a = sc * gs.Gam[t.rn + r], b = -gs.Gam[t.rn + r];
+#pragma unroll
+        for (int n = 0; n < NH; ++n)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) { acc[n][r][y] *= a; acc[n][4 + r][y] *= b; }
     }
-    // D_ij, only ever evaluated for j <= i so that the exponent is non-positive
-    auto D = [&](int i, int j) -> float { return expf(S.gam[i] - S.gam[j]); };
-
-    // (1) U = Ut - W h ;  K K^T ;  P
-    tiles(kC, DV, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, DK, [&](int i, int m) { return W[i * DK + m]; }, [&](int m, int j) { return h[m * DV + j]; });
-        for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) U[(i0 + a) * DV + j0 + b] = Ut[(i0 + a) * DV + j0 + b] - acc[a][b];
-    });
-    tiles(kC, kC, [&](int i0, int j0) {
-        float kk[4][4] = {}, qk[4][4] = {};
-        if (j0 <= i0 + 3) {
-            mac(kk, i0, j0, DK, Kf, [&](int m, int j) { return Kf(j, m); });
-            mac(qk, i0, j0, DK, Qf, [&](int m, int j) { return Kf(j, m); });
+    cp_wait<1>();
+    __syncthreads();
+    // += [dPD; G] K
+    const int w16 = (t.rn >> 4) * 16;
+#pragma unroll
+    for (int n = 0; n < NH; ++n) mac<2, A_ROW, B_COL>(acc[n], sP, sT, kPc, t.rn, s0 + n * 64, PK, t.cn, 0, w16 + 16);
+    cp_wait<0>();
+    __syncthreads();
+    // dk^col = e (U dh'^T) + dPD^T Q + (b G)^T K, then everything is written
+    IO* dqp = rows_of<IO>(p.dq, x, H, DK);
+    IO* dkp = rows_of<IO>(p.dk, x, H, DK);
+    float rsum = 0.f, dqq[4] = {}, drow[4] = {}, dcol[4] = {};
+#pragma unroll
+    for (int n = 0; n < NH; ++n) {
+        float col[4][4];
+        zero(col);
+        mac<1, A_ROW, B_ROW>(col, sU, nullptr, PV, t.rn, sH + n * 64 * PV, PV, t.cn, 0, DV);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const float e = gs.ee[t.rn + r];
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                col[r][y] *= e;
+                rsum = fmaf(s0[(t.rn + r) * PK + n * 64 + t.cn + 8 * y], col[r][y], rsum);
+            }
         }
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-                const int i = i0 + a, j = j0 + b;
-                S.KK[i][j] = (j < i) ? kk[a][b] : 0.f;
-                S.P[i][j] = (j <= i) ? qk[a][b] * D(i, j) : 0.f;
+        mac<1, A_COL, B_COL>(col, sP, nullptr, kPc, t.rn, s1 + n * 64, PK, t.cn, w16, kC);
+        mac<1, A_COL, B_COL>(col, sB, nullptr, kPc, t.rn, s0 + n * 64, PK, t.cn, w16, kC);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int i = t.rn + r;
+            const float b = gs.bb[i];
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int c = n * 64 + t.cn + 8 * y;
+                const float q = s1[i * PK + c], k = s0[i * PK + c];
+                dqq[r] = fmaf(q, acc[n][r][y], dqq[r]);
+                drow[r] = fmaf(k, acc[n][4 + r][y], drow[r]);
+                dcol[r] = fmaf(k, col[r][y], dcol[r]);
+                if (i < x.len) {
+                    stf(dqp + i * rk + c, acc[n][r][y]);
+                    stf(dkp + i * rk + c, fmaf(b, acc[n][4 + r][y], col[r][y]));
+                }
             }
-    });
-    __syncthreads();
-    // (2) Kb dh' -> dXv (temporarily) ;  dU = scale P^T dO + Kb dh'
-    tiles(kC, DV, [&](int i0, int j0) {
-        float a1[4][4] = {}, a2[4][4] = {};
-        mac(a1, i0, j0, DK, [&](int i, int m) { return S.ee[i] * Kf(i, m); }, [&](int m, int j) { return dhn[m * DV + j]; });
-        mac(a2, i0, j0, kC, [&](int i, int m) { return S.P[m][i]; }, Of);
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-                dXv[(i0 + a) * DV + j0 + b] = a1[a][b];
-                dU[(i0 + a) * DV + j0 + b] = sc * a2[a][b] + a1[a][b];
-            }
-    });
-    __syncthreads();
-    // (3) dP = scale tril(dO U^T) ;  dO h^T ;  dW = -dU h^T ;  r_i = <(Kb dh')_i, U_i>
-    tiles(kC, kC, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        if (j0 <= i0 + 3) mac(acc, i0, j0, DV, Of, [&](int m, int j) { return U[j * DV + m]; });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) S.dP[i0 + a][j0 + b] = (j0 + b <= i0 + a) ? sc * acc[a][b] : 0.f;
-    });
-    tiles(kC, DK, [&](int i0, int j0) {
-        float a1[4][4] = {}, a2[4][4] = {};
-        mac(a1, i0, j0, DV, Of, [&](int m, int j) { return h[j * DV + m]; });
-        mac(a2, i0, j0, DV, [&](int i, int m) { return dU[i * DV + m]; }, [&](int m, int j) { return h[j * DV + m]; });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-                dOh[(i0 + a) * DK + j0 + b] = a1[a][b];
-                dW[(i0 + a) * DK + j0 + b] = -a2[a][b];
-            }
-    });
-    row_reduce(S.r, DV, [&](int i, int j) { return dXv[i * DV + j] * U[i * DV + j]; });
-    __syncthreads();
-    // (4) dQ ;  dXk = T^T dW ;  dXv = T^T dU ;  rq_i = <Q_i, (dO h^T)_i>
-    tiles(kC, DK, [&](int i0, int j0) {
-        float acc[4][4] = {}, ax[4][4] = {};
-        mac(acc, i0, j0, kC, [&](int i, int m) { return m <= i ? S.dP[i][m] * D(i, m) : 0.f; }, Kf);
-        mac(ax, i0, j0, kC, [&](int i, int m) { return Tm[m * kC + i]; }, [&](int m, int j) { return dW[m * DK + j]; });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-                const int i = i0 + a, j = j0 + b;
-                if (i < x.len) stf(dqp + i * rk + j, sc * S.Gam[i] * dOh[i * DK + j] + acc[a][b]);
-                dXk[i * DK + j] = ax[a][b];
-            }
-    });
-    tiles(kC, DV, [&](int i0, int j0) {
-        float ax[4][4] = {};
-        mac(ax, i0, j0, kC, [&](int i, int m) { return Tm[m * kC + i]; }, [&](int m, int j) { return dU[m * DV + j]; });
-        for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) dXv[(i0 + a) * DV + j0 + b] = ax[a][b];
-    });
-    row_reduce(S.rq, DK, [&](int i, int j) { return Qf(i, j) * dOh[i * DK + j]; });
-    __syncthreads();
-    // (5) dA = -stril(dXk W^T + dXv Ut^T) ;  G = dA . D ;  Z = G . KK ;  row dots of dXk.K and dXv.V
-    tiles(kC, kC, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        if (j0 < i0 + 3) {
-            mac(acc, i0, j0, DK, [&](int i, int m) { return dXk[i * DK + m]; }, [&](int m, int j) { return W[j * DK + m]; });
-            mac(acc, i0, j0, DV, [&](int i, int m) { return dXv[i * DV + m]; }, [&](int m, int j) { return Ut[j * DV + m]; });
         }
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-                const int i = i0 + a, j = j0 + b;
-                const float g_ = (j < i) ? -acc[a][b] * D(i, j) : 0.f;
-                S.G[i][j] = g_;
-                S.KK[i][j] = g_ * S.KK[i][j];
-            }
-    });
-    row_reduce(S.xk, DK, [&](int i, int j) { return dXk[i * DK + j] * Kf(i, j); });
-    row_reduce(S.xv, DV, [&](int i, int j) { return dXv[i * DV + j] * Vf(i, j); });
-    __syncthreads();
-    // (6) dK, dV, gate gradients
-    tiles(kC, DK, [&](int i0, int j0) {
-        float acc[4][4] = {}, a2[4][4] = {};
-        mac(acc, i0, j0, kC, [&](int i, int m) { return m >= i ? S.dP[m][i] * D(m, i) : 0.f; }, Qf);
-        mac(acc, i0, j0, kC, [&](int i, int m) { return S.bb[i] * S.G[i][m] + S.bb[m] * S.G[m][i]; }, Kf);
-        mac(a2, i0, j0, DV, [&](int i, int m) { return U[i * DV + m]; }, [&](int m, int j) { return dhn[j * DV + m]; });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-                const int i = i0 + a, j = j0 + b;
-                if (i < x.len) stf(dkp + i * rk + j, acc[a][b] + S.ee[i] * a2[a][b] + S.bb[i] * S.Gam[i] * dXk[i * DK + j]);
-            }
-    });
-    for (int t = threadIdx.x; t < kC * DV; t += blockDim.x) {
-        const int i = t / DV, j = t % DV;
-        if (i < x.len) stf(dvp + i * rv + j, S.ww[i] * dXv[t]);
     }
-    // <dh', h> over the whole state, fixed order
-    float part = 0.f;
-    for (int t = threadIdx.x; t < DK * DV; t += blockDim.x) part = fmaf(dhn[t], h[t], part);
-    part = warp_sum(part);
-    if ((threadIdx.x & 31) == 0) S.red[threadIdx.x >> 5] = part;
-    if (threadIdx.x < kC) {
-        const int i = threadIdx.x;
-        float rowZ = 0.f, colZ = 0.f, rowPP = 0.f, colPP = 0.f;
-        for (int j = 0; j < kC; ++j) {
-            rowZ += S.KK[i][j];
-            colZ += S.bb[j] * S.KK[j][i];
-            rowPP += S.dP[i][j] * S.P[i][j];
-            colPP += S.dP[j][i] * S.P[j][i];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        dqq[r] = row_sum8(dqq[r]); drow[r] = row_sum8(drow[r]); dcol[r] = row_sum8(dcol[r]);
+        if ((lane & 7) == 0) {
+            const int cb = warp >> 2, i = t.rn + r;
+            red[0][cb][i] = dqq[r]; red[1][cb][i] = drow[r]; red[2][cb][i] = dcol[r];
         }
-        const float db = rowZ + S.Gam[i] * S.xk[i];
-        const float dw = S.xv[i];
+    }
+    // <dh', h> over the whole state (h from the workspace: its tile has been overwritten)
+    float hh = 0.f;
+#pragma unroll 4
+    for (int e = tid; e < DK * DV / 4; e += kThreads) {
+        const float4 a = ld4(wsH + (size_t)e * 4), b = ld4(sH + (e / (DV / 4)) * PV + (e % (DV / 4)) * 4);
+        hh = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, hh))));
+    }
+    rsum = warp_total(rsum);
+    hh = warp_total(hh);
+    if (lane == 0) { part[0][warp] = rsum; part[1][warp] = hh; }
+    __syncthreads();
+    if (tid < kC) {
+        const int i = tid;
+        const float db = red[1][0][i] + red[1][1][i];
+        float dw = red[3][0][i] + red[3][1][i];
+        if (DV == 128) dw += red[3][2][i] + red[3][3][i];
         if (p.d.delta_rule && i < x.len) p.dbeta[(size_t)(x.tok0 + i) * H + x.hd] = db + dw;
-        S.dgam[i] = S.bb[i] * rowZ - colZ + rowPP - colPP + S.bb[i] * S.Gam[i] * S.xk[i] + sc * S.Gam[i] * S.rq[i] - S.r[i];
+        dgam[i] = (red[0][0][i] + red[0][1][i]) + gs.bb[i] * db - (red[2][0][i] + red[2][1][i]);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float hh = 0.f, rs = 0.f;
-        for (int w_ = 0; w_ < kThreads / 32; ++w_) hh += S.red[w_];
-        for (int i = 0; i < kC; ++i) rs += S.r[i];
-        S.dgam[kC - 1] += rs + S.Gam[kC - 1] * hh;
-        // gam_i = sum_{j<=i} g_j  =>  dg_j = sum_{i>=j} dgam_i
-        float run = 0.f;
-        for (int i = kC - 1; i >= 0; --i) {
-            run += S.dgam[i];
-            if (i < x.len) p.dg[(size_t)(x.tok0 + i) * H + x.hd] = run;
+    if (warp == 0) {   // dg_j = sum_{i >= j} dgam_i: lane l owns tokens l and l + 32
+        float rs = 0.f, hs = 0.f;
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w) { rs += part[0][w]; hs += part[1][w]; }
+        float a = dgam[lane], b = dgam[lane + 32] + (lane == 31 ? rs + gs.Gam[kC - 1] * hs : 0.f);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float ta = __shfl_down_sync(0xffffffffu, a, o), tb = __shfl_down_sync(0xffffffffu, b, o);
+            if (lane + o < 32) { a += ta; b += tb; }
         }
+        a += __shfl_sync(0xffffffffu, b, 0);
+        float* dg = p.dg + (size_t)x.tok0 * H + x.hd;
+        if (lane < x.len) dg[(size_t)lane * H] = a;
+        if (lane + 32 < x.len) dg[(size_t)(lane + 32) * H] = b;
     }
+}
+
+template <int DK, int DV>
+cudaError_t launch_scan_t(const Problem& p, int dirs, cudaStream_t st) {
+    static SmemLimitOnce once;
+    const cudaError_t e = once.ensure(scan_kernel<DK, DV>, (uint32_t)scan_smem<DK>());
+    if (e != cudaSuccess) return e;
+    const int ctas = p.d.N * p.d.H * (dirs == 2 ? 2 : 1) * (DV / kScanCols);
+    { StageScope t(dirs == 2 ? ST_SCANS : dirs == 1 ? ST_RSCAN : ST_FSCAN, st); scan_kernel<DK, DV><<<ctas, kThreads, scan_smem<DK>(), st>>>(p, dirs); }
+    return cudaGetLastError();
+}
+
+template <typename IO, int DK, int DV>
+cudaError_t launch_prep_t(const Problem& p, PrepMode mode, cudaStream_t st) {
+    static SmemLimitOnce once;
+    const cudaError_t e = once.ensure(prep_kernel<IO, DK, DV>, (uint32_t)prep_smem<DK, DV>());
+    if (e != cudaSuccess) return e;
+    { StageScope t(mode == PREP_BWD ? ST_EPREP : ST_PREP, st); prep_kernel<IO, DK, DV><<<p.L.max_chunks * p.d.H, kThreads, prep_smem<DK, DV>(), st>>>(p, mode); }
+    return cudaGetLastError();
 }
 
 template <typename IO, int DK, int DV>
 cudaError_t launch_fwd_t(const Problem& p, cudaStream_t st) {
-    const int CH = p.L.max_chunks * p.d.H, chains = p.d.N * p.d.H;
-    launch_table(p, st);
-    if (CH > 0) { StageScope t(ST_PREP, st); prep_kernel<IO, DK, DV><<<CH, kThreads, 0, st>>>(p); }
-    const size_t sm = 2 * sizeof(float) * DK * DV;
-    cudaError_t e = cudaFuncSetAttribute(scan_kernel<DK, DV, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    if (chains > 0) { StageScope t(ST_FSCAN, st); scan_kernel<DK, DV, false><<<chains, kThreads, sm, st>>>(p); }
-    if (p.o && CH > 0) { StageScope t(ST_OUT, st); out_kernel<IO, DK, DV><<<CH, kThreads, 0, st>>>(p); }
+    cudaError_t e;
+    if (p.cu && (e = launch_table(p, st)) != cudaSuccess) return e;
+    if ((e = launch_prep_t<IO, DK, DV>(p, PREP_FWD, st)) != cudaSuccess) return e;
+    if ((e = launch_scan_t<DK, DV>(p, 0, st)) != cudaSuccess || !p.o) return e;
+    static SmemLimitOnce once;
+    if ((e = once.ensure(out_kernel<IO, DK, DV>, (uint32_t)out_smem<DK, DV>())) != cudaSuccess) return e;
+    { StageScope t(ST_OUT, st); out_kernel<IO, DK, DV><<<p.L.max_chunks * p.d.H, kThreads, out_smem<DK, DV>(), st>>>(p); }
     return cudaGetLastError();
 }
 
 template <typename IO, int DK, int DV>
 cudaError_t launch_bwd_t(const Problem& p, bool skip_recompute, cudaStream_t st) {
     cudaError_t e;
-    if (!skip_recompute) {
-        e = launch_fwd_t<IO, DK, DV>(p, st);
-        if (e != cudaSuccess) return e;
-    }
-    const int CH = p.L.max_chunks * p.d.H, chains = p.d.N * p.d.H;
-    if (CH > 0) { StageScope t(ST_EPREP, st); eprep_kernel<IO, DK, DV><<<CH, kThreads, 0, st>>>(p); }
-    const size_t sm = 2 * sizeof(float) * DK * DV;
-    e = cudaFuncSetAttribute(scan_kernel<DK, DV, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    if (chains > 0) { StageScope t(ST_RSCAN, st); scan_kernel<DK, DV, true><<<chains, kThreads, sm, st>>>(p); }
-    e = cudaFuncSetAttribute(intra_kernel<IO, DK, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(IntraSmem));
-    if (e != cudaSuccess) return e;
-    if (CH > 0) { StageScope t(ST_INTRA, st); intra_kernel<IO, DK, DV><<<CH, kThreads, sizeof(IntraSmem), st>>>(p); }
+    if (p.cu && !skip_recompute && (e = launch_table(p, st)) != cudaSuccess) return e;
+    if ((e = launch_prep_t<IO, DK, DV>(p, skip_recompute ? PREP_BWD : PREP_FWD_BWD, st)) != cudaSuccess) return e;
+    if ((e = launch_scan_t<DK, DV>(p, skip_recompute ? 1 : 2, st)) != cudaSuccess) return e;
+    static SmemLimitOnce once;
+    if ((e = once.ensure(intra_kernel<IO, DK, DV>, (uint32_t)intra_smem<DK, DV>())) != cudaSuccess) return e;
+    { StageScope t(ST_INTRA, st); intra_kernel<IO, DK, DV><<<p.L.max_chunks * p.d.H, kThreads, intra_smem<DK, DV>(), st>>>(p); }
     return cudaGetLastError();
 }
 
@@ -549,8 +636,6 @@ cudaError_t launch_table(const Problem& p, cudaStream_t st) {
     table_kernel<<<1, 256, 0, st>>>(p);
     return cudaGetLastError();
 }
-
-size_t simt_scratch_per_chunkhead(const gdn_desc& d) { return sizeof(float) * kC * 3 * ((size_t)d.d_k + d.d_v); }
 
 #define GDN_DISPATCH(FN, ...)                                                                       \
     do {                                                                                            \

@@ -1,8 +1,8 @@
 // fp32 blocked inversion of a unit lower triangular 64 x 64 matrix in shared memory (T = (I + A)^-1 of the chunk-local
-// solve, Section 4.2), shared by the tcgen05 kernel families.  Thread indices are those of the calling CTA; every step
+// solve, Section 4.2), shared by every kernel family.  Thread indices are those of the calling CTA; every step
 // uses at most its first 256 threads, and the caller separates the steps by CTA-wide barriers.
 #pragma once
-#include "tc_common.cuh"
+#include "gdn_internal.cuh"
 
 namespace gdn {
 namespace {

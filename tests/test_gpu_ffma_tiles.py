@@ -1,0 +1,34 @@
+"""The register-tiled fp32 kernels at the edges of their tiles, for every pair of head dimensions: sequences that end at,
+before and after the 4-row, 16-row and 32-row blocks of a chunk, one chunk and several (the carries' double buffer), closed
+and on a workspace fresh from the forward.
+
+Tolerance: every output is a chain of at most six products with contractions of up to 128 terms, each summed in fp32; rounding
+adds up like sqrt(6 * 128) * 2^-24 = 1.7e-6 of the summands, and the decay gradient is a difference of such sums.  3e-6 for
+whole tensors, three times that for one 64-token block."""
+import numpy as np
+import pytest
+
+from paper_2608_12700_b200 import runner, synth
+from helpers import check_against_oracle, oracle_grads, rel
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dk,dv", [(64, 64), (128, 128), (128, 64), (64, 128)])
+@pytest.mark.parametrize("lengths", [[1, 3, 5, 15, 16, 17], [31, 32, 33, 63, 64, 65], [127, 0, 193, 256, 321]])
+@pytest.mark.parametrize("delta_rule", [1, 0])
+def test_tile_edges(dk, dv, lengths, delta_rule):
+    wl = synth.make_workload("tiles", dtype="f32", lengths=lengths, H=3, d_k=dk, d_v=dv, seed=310, states=True, scale=0.7,
+                             delta_rule=delta_rule)
+    ref = oracle_grads(wl)
+    buf = runner.to_device(wl, want_o=True)
+    runner.run_bwd(buf)
+    got = runner.fetch(buf)
+    check_against_oracle(wl, got, tol=3e-6, ref=ref, block_tol=9e-6)
+    runner.run_fwd(buf)
+    f = runner.fetch(buf)
+    assert rel(f["o"], ref["o"]) < 3e-6 and rel(f["hT"], ref["hT"]) < 3e-6
+    runner.run_bwd(buf, fresh=1)
+    fresh = runner.fetch(buf)
+    for n in ("dq", "dk", "dv", "dg", "dh0"):
+        assert np.array_equal(fresh[n], got[n]), n
