@@ -17,6 +17,7 @@
 // give conflict-free loads: tile pitches are 64 + 4 or 128 + 4 floats.
 #pragma once
 #include "chunk_geom.cuh"
+#include "tc_inverse.cuh"
 
 namespace gdn {
 namespace {
@@ -52,7 +53,8 @@ enum BForm { B_ROW, B_COL };   // B(k, j) = B[j * pb + k] / B[k * pb + j]
 
 // acc[R0 + 4 h + x][y] += sum over k in [k0, k1) of A_h(i + x, k) B(k, j + 8 y);  i, j: first row and column of this thread;
 // (k0, k1 multiples of 4; pointers at row / column 0)
-template <int HALVES, AForm AF, BForm BF, int R0 = 0, int R>
+// (CS: distance of a thread's columns)
+template <int HALVES, AForm AF, BForm BF, int R0 = 0, int CS = 8, int R>
 __device__ __forceinline__ void mac(float (&acc)[R][4], const float* A0, const float* A1, int pa, int i, const float* B,
                                     int pb, int j, int k0, int k1) {
     static_assert(R0 + 4 * HALVES <= R, "rows of the accumulator");
@@ -78,11 +80,11 @@ __device__ __forceinline__ void mac(float (&acc)[R][4], const float* A0, const f
 #pragma unroll
         for (int y = 0; y < 4; ++y) {
             if (BF == B_ROW) {
-                const float4 v = *reinterpret_cast<const float4*>(b0 + 8 * y * pb + k);
+                const float4 v = *reinterpret_cast<const float4*>(b0 + CS * y * pb + k);
                 b[0][y] = v.x; b[1][y] = v.y; b[2][y] = v.z; b[3][y] = v.w;
             } else {
 #pragma unroll
-                for (int z = 0; z < 4; ++z) b[z][y] = b0[(k + z) * pb + 8 * y];
+                for (int z = 0; z < 4; ++z) b[z][y] = b0[(k + z) * pb + CS * y];
             }
         }
 #pragma unroll
@@ -162,6 +164,39 @@ __device__ __forceinline__ void load_block(float* tile, const float* src) {
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+template <typename IO>
+__device__ __forceinline__ const IO* rows_of(const void* base, const ChunkInfo& x, int H, int d) {
+    return reinterpret_cast<const IO*>(base) + ((size_t)x.tok0 * H + x.hd) * d;
+}
+template <typename IO>
+__device__ __forceinline__ IO* rows_of(void* base, const ChunkInfo& x, int H, int d) {
+    return reinterpret_cast<IO*>(base) + ((size_t)x.tok0 * H + x.hd) * d;
+}
+__device__ __forceinline__ float* block_of(const Problem& p, size_t region, int ch, int floats) {
+    return reinterpret_cast<float*>(p.ws + region) + (size_t)ch * floats;
+}
+
+// T = (I + A)^-1, blocked; S is scratch.  Everybody takes part; the caller synchronises afterwards.
+__device__ __forceinline__ void invert(const float* A, float* T, float* S) {
+    static_assert(kPc == kLdi, "the inversion works on the tiles of this family");
+    for (int e = threadIdx.x; e < kC * kC; e += kThreads)   // the blocks above the block diagonal are not written by the steps below
+        if ((e % kC) / 16 > e / kC / 16) T[(e / kC) * kPc + e % kC] = 0.f;
+    inv_diag8(A, T);
+    __syncthreads();
+    inv_diag16(A, T, S);
+    __syncthreads();
+    inv_premul<2>(A, T, S);
+    __syncthreads();
+    inv_level<1, 1, 2>(S, T);
+    __syncthreads();
+    inv_level<2, 2, 2>(S, T);
+    __syncthreads();
+    inv_level<3, 4, 2>(S, T);
+}
+
+// Which part of the preparation a launch makes: the forward's, that and the backward's, the backward's alone.
+enum PrepMode { PREP_FWD = 0, PREP_FWD_BWD = 1, PREP_BWD = 2 };
 
 // Sum over the eight lanes that share a row (fixed order).
 __device__ __forceinline__ float row_sum8(float v) {

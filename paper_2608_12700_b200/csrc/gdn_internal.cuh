@@ -138,14 +138,17 @@ inline WsLayout make_layout_vec(const gdn_desc& d, size_t scratch_per_ch) {
     L.img_QKp = take(L.tc_scans ? CH * 32768 : 0);
     L.img_Km = take(L.tc_scans ? CH * 16384 : 0);
     L.img_Vt = take(L.tc_scans ? CH * 16384 : 0);
+    L.Kb = take(4 * CH * kC * d.d_k);
+    L.U = take(4 * CH * kC * d.d_v);
     L.hc = take(4 * CH * d.d_k * d.d_v);   // (fp32, or a bf16 tile image in the first half of each slot)
     L.fwd_end = o;
     L.E = take(4 * CH * d.d_k * d.d_v);
     L.img_E = take(L.tc_scans ? CH * 32768 : 0);
     L.img_dO = take(L.tc_scans ? CH * 16384 : 0);
     L.dhn = take(4 * CH * d.d_k * d.d_v);
-    L.scratch_per_ch = scratch_per_ch;
-    L.scratch = take(scratch_per_ch * CH);
+    L.dU = take(4 * CH * kC * d.d_v);
+    L.scratch_per_ch = L.tc_scans ? scratch_per_ch : 0;   // (of the tensor-core kernels)
+    L.scratch = take(L.scratch_per_ch * CH);
     L.total = o;
     return L;
 }
@@ -213,7 +216,6 @@ cudaError_t simt_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t 
 // FFMA family for per-channel gates (Eq. 1 with gate vectors).
 cudaError_t vec_launch_fwd(const Problem& p, cudaStream_t st);
 cudaError_t vec_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st);
-size_t vec_scratch_per_chunkhead(const gdn_desc& d);
 // ... and its tensor-core route (bf16 I/O, d_k = d_v = 128; gdn_tc_cw.cu): forward (bwd = false) or backward.
 cudaError_t cw_tc_launch(const Problem& p, bool bwd, bool skip_recompute, cudaStream_t st);
 size_t cw_tc_scratch_per_chunkhead();

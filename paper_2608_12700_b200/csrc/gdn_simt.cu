@@ -17,7 +17,6 @@
 // global memory, and the solve and the sums over a chunk done by single threads, the same stages took 907, 165 and 102 us
 // (2 x 4 heads of 1000 tokens); the smallest call, 2 heads of 128 tokens at d = 64, went from 370 to 53 us.
 #include "ffma_scan.cuh"
-#include "tc_inverse.cuh"
 
 namespace gdn {
 namespace {
@@ -125,22 +124,9 @@ __device__ __forceinline__ void load_gates(const Problem& p, const ChunkInfo& x,
     load_erase_write(p, x, s, threadIdx.x);
 }
 
-template <typename IO>
-__device__ __forceinline__ const IO* rows_of(const void* base, const ChunkInfo& x, int H, int d) {
-    return reinterpret_cast<const IO*>(base) + ((size_t)x.tok0 * H + x.hd) * d;
-}
-template <typename IO>
-__device__ __forceinline__ IO* rows_of(void* base, const ChunkInfo& x, int H, int d) {
-    return reinterpret_cast<IO*>(base) + ((size_t)x.tok0 * H + x.hd) * d;
-}
-__device__ __forceinline__ float* block_of(const Problem& p, size_t region, int ch, int floats) {
-    return reinterpret_cast<float*>(p.ws + region) + (size_t)ch * floats;
-}
-
 // ------------------------------------------------------------------------------------------------
 // prep
 // ------------------------------------------------------------------------------------------------
-enum PrepMode { PREP_FWD = 0, PREP_FWD_BWD = 1, PREP_BWD = 2 };
 template <int DK, int DV>
 constexpr size_t prep_smem() {
     return sizeof(float) * (kC * (2 * pitch(DK) + pitch(DK > DV ? DK : DV) + pitch(DV)) + 4 * kC * kPc);
@@ -215,21 +201,7 @@ __global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) 
             *reinterpret_cast<float4*>(wsKb + (size_t)e * 4) = make_float4(w * k.x, w * k.y, w * k.z, w * k.w);
         }
         __syncthreads();
-        // T = (I + A)^-1, blocked (the blocks above the block diagonal are not written: zero them)
-        for (int e = tid; e < kC * kC; e += kThreads)
-            if ((e % kC) / 16 > e / kC / 16) T[(e / kC) * kPc + e % kC] = 0.f;
-        static_assert(kPc == kLdi, "the inversion works on the tiles of this family");
-        inv_diag8(A, T);
-        __syncthreads();
-        inv_diag16(A, T, S);
-        __syncthreads();
-        inv_premul<2>(A, T, S);
-        __syncthreads();
-        inv_level<1, 1, 2>(S, T);
-        __syncthreads();
-        inv_level<2, 2, 2>(S, T);
-        __syncthreads();
-        inv_level<3, 4, 2>(S, T);
+        invert(A, T, S);
         cp_wait<0>();
         __syncthreads();
         float* wsT = block_of(p, p.L.Tm, x.ch, kC * kC);

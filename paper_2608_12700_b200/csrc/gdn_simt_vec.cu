@@ -3,45 +3,33 @@
 //
 // The channel-wise decay does not factor out of the chunk-local contractions as a token-token matrix; it folds inside
 // them (Appendix A, last paragraph): every token-token quantity is a sum over the channel r that carries the factor
-// exp(gam_i[r] - gam_j[r]), evaluated for j <= i only, so that no exponent is ever positive.  This family is the
-// plain CUDA-core statement of that formulation (arithmetic in fp32 whatever the I/O dtype), stage by stage:
+// exp(gam_i[r] - gam_j[r]), j <= i, so that no exponent is ever positive.  The chunk is cut into four blocks of 16 tokens.
+// Between two blocks J < I the factor splits at the start of the later one, ref_I = gam at the last token before block I:
+//     exp(gam_i - gam_j) = exp(gam_i - ref_I) exp(ref_I - gam_j)      (both exponents non-positive)
+// so rows are scaled once (q, b k by exp(gam_i - ref)), the columns once per later block (k by exp(ref_I - gam_j)), and the
+// off-diagonal blocks are plain products; only the pairs inside a block, a quarter of all, are summed with the exponential
+// in place.  Stages (arithmetic in fp32 whatever the I/O dtype):
 //   table  : chunk table from cu_seqlens (shared with the scalar-gate family)
-//   vprep  : gam = cumsum(g) per channel;  A_ij = sum_r b_i k_i k_j e^{gam_i - gam_j} (j < i);  T = (I + A)^-1;
-//            P_ij = sum_r q_i k_j e^{gam_i - gam_j} (j <= i);  W = T (Gam . b . K);  Ut = T (w . V)
-//   vscan  : forward   h'  = Diag(Gam_e) h   + Kb^T (Ut - W h),   Kb_j = e^{gam_e - gam_j} . k_j   (stores h per chunk)
-//            reverse   dh  = Diag(Gam_e) dh' + E - W^T (Kb dh')                                     (stores dh'; K#1)
-//   veprep : E = scale (Gam . Q - P W)^T dO
+//   vprep  : gam = cumsum(g) per channel;  A_ij = sum_r b_i k_i k_j e^{gam_i - gam_j} (j < i);  P_ij = sum_r q_i k_j
+//            e^{gam_i - gam_j} (j <= i);  T = (I + A)^-1;  W = T (Gam . b . K);  Ut = T (w . V);  Kb_j = e^{gam_e - gam_j} . k_j;
+//            and for the backward dU0 = scale P^T dO, E = scale (Gam . Q - P W)^T dO
+//   vscan  : the carries (ffma_scan.cuh; the state decays by one factor per row)
 //   vintra : every token gradient, including the VJP of the triangular solve from the stored T (K#2), the gate
 //            gradients per channel, and dg by a reverse cumulative sum inside the chunk
-// One CTA handles one (chunk, head) in the parallel stages and one (sequence, head) chain in the scans.  Every
-// reduction has a fixed order: results are bit-identical from run to run.
-// With bf16 I/O at d_k = d_v = 128 the whole path runs on the tensor cores instead (gdn_tc_cw.cu and tc_scan_cw in
-// gdn_tc.cu); only the optional forward output is formed here, from the bf16 tile images those kernels leave.
-#include "simt_common.cuh"
-#include "tc_ptx.cuh"
+//   vout   : forward output
+// One CTA handles one (chunk, head) in the parallel stages.  Every reduction has a fixed order: results are bit-identical
+// from run to run.  Measured against the plain statement (decay evaluated for every pair and channel, operands read from global
+// memory, one CTA per chain in the carries): 8 heads of 1024 tokens at d = 128, bf16 I/O, decay beyond the tensor-core route:
+// 4.4 ms -> 0.30 ms; a step of 2 x 4 heads of 500 tokens at d = 64, fp32: 1.01 -> 0.14 ms.  With bf16 I/O at d_k = d_v = 128 the path runs on the tensor cores instead (gdn_tc_cw.cu), with these
+// kernels enqueued behind it for gates that leave its range.
+#include "ffma_scan.cuh"
 
 namespace gdn {
 namespace {
 
-// acc[a][b] += sum_m fa(i0 + a, m) fb(j0 + b, m) exp(gam[i][m] - gam[j][m])  for j <= i - strict (else 0 is added)
-template <int DK, class FA, class FB>
-__device__ __forceinline__ void mac_decay(float (&acc)[4][4], int i0, int j0, int strict, const float* gam, FA fa, FB fb) {
-    if (j0 > i0 + 3 - strict) return;
-#pragma unroll 2
-    for (int m = 0; m < DK; ++m) {
-        float a[4], b[4], gi[4], gj[4];
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            a[x] = fa(i0 + x, m); b[x] = fb(j0 + x, m);
-            gi[x] = gam[(i0 + x) * (DK + 1) + m]; gj[x] = gam[(j0 + x) * (DK + 1) + m];
-        }
-#pragma unroll
-        for (int x = 0; x < 4; ++x)
-#pragma unroll
-            for (int y = 0; y < 4; ++y)
-                if (j0 + y <= i0 + x - strict) acc[x][y] = fmaf(a[x] * b[y], expf(gi[x] - gj[y]), acc[x][y]);
-    }
-}
+using namespace ffma;
+
+constexpr int kB = 16, kNB = kC / kB;   // tokens of a block, blocks of a chunk
 
 // Whether this launch has work: normally when no earlier stage has reported an error; a launch of the fall-back sequence
 // only when the tensor-core route has refused the gates of this call (decided on the device, no host round trip).
@@ -56,421 +44,612 @@ __global__ void vec_clear_refusal_kernel(Problem p) {
     if (refused) { hdr->status = GDN_OK; hdr->detail = 0; }
 }
 
-// Chunk-local cumulative log decay per channel into shared memory (pitch DK + 1); rows beyond the sequence repeat the
-// last valid row (identity padding: g = 0 there).
+// References of the four blocks and their exponentials: ref_0 = 0 (the chunk start), ref_I = gam of token 16 I - 1.
 template <int DK>
-__device__ __forceinline__ void cumulate_gates(const Problem& p, const ChunkCtx& x, float* gam) {
-    for (int r = threadIdx.x; r < DK; r += blockDim.x) {
-        float s = 0.f;
-        for (int i = 0; i < kC; ++i) {
-            if (i < x.len) s += p.gv[((size_t)(x.tok0 + i) * p.d.H + x.hd) * DK + r];
-            gam[i * (DK + 1) + r] = s;
-        }
+struct Refs { float ref[kNB][DK], eref[kNB][DK]; };
+template <int DK>
+__device__ __forceinline__ void make_refs(Refs<DK>& s, const float* G) {
+    for (int t = threadIdx.x; t < kNB * DK; t += kThreads) {
+        const int I = t / DK, r = t % DK;
+        const float v = I ? G[(I * kB - 1) * pitch(DK) + r] : 0.f;
+        s.ref[I][r] = v;
+        s.eref[I][r] = expf(v);
     }
 }
+// Rows of a tile times exp(gam - ref of their block), in place.
 template <int DK>
-__device__ __forceinline__ void load_gamma(const float* wsG, float* gam) {
-    for (int t = threadIdx.x; t < kC * DK; t += blockDim.x) gam[(t / DK) * (DK + 1) + t % DK] = wsG[t];
+__device__ __forceinline__ void scale_rows(float* X, const float* G, const Refs<DK>& s) {
+    for (int t = threadIdx.x; t < kC * DK; t += kThreads) {
+        const int i = t / DK, r = t % DK;
+        X[i * pitch(DK) + r] *= expf(G[i * pitch(DK) + r] - s.ref[i / kB][r]);
+    }
+}
+// The scaled copies of the keys, k_j exp(ref_I - gam_j) for j < 16 I, I = 1 .. 3, one behind the other (96 rows).
+__host__ __device__ constexpr int copy_row(int I) { return kB * (I * (I - 1) / 2); }   // first row of copy I
+template <int DK, class KF>
+__device__ __forceinline__ void make_copies(float* C, const float* G, const Refs<DK>& s, KF key) {
+    for (int t = threadIdx.x; t < (kC - kB) * DK; t += kThreads) {
+        const int j = t / DK, r = t % DK;
+        const float k = key(j, r), g = G[j * pitch(DK) + r];
+#pragma unroll
+        for (int I = 1; I < kNB; ++I)
+            if (j < I * kB) C[(copy_row(I) + j) * pitch(DK) + r] = k * expf(s.ref[I][r] - g);
+    }
 }
 
 // ------------------------------------------------------------------------------------------------
 // vprep
 // ------------------------------------------------------------------------------------------------
-template <typename IO, int DK, int DV>
-__global__ void __launch_bounds__(kThreads) vprep_kernel(Problem p) {
-    ChunkCtx x;
-    if (!vec_go(p) || !chunk_ctx(p, x)) return;
-    extern __shared__ __align__(16) float smf[];
-    float* gam = smf;                                   // [64][DK + 1]
-    float (*A)[kC + 1] = reinterpret_cast<float (*)[kC + 1]>(smf + kC * (DK + 1));
-    float (*Ti)[kC + 1] = A + kC;
-    const int H = p.d.H;
-    const size_t base_k = ((size_t)x.tok0 * H + x.hd) * DK, base_v = ((size_t)x.tok0 * H + x.hd) * DV;
-    const size_t rk = (size_t)H * DK, rv = (size_t)H * DV;
-    const IO* qp = reinterpret_cast<const IO*>(p.q) + base_k;
-    const IO* kp = reinterpret_cast<const IO*>(p.k) + base_k;
-    const IO* vp = reinterpret_cast<const IO*>(p.v) + base_v;
-    auto Qf = [&](int i, int m) -> float { return i < x.len ? ldf(qp + i * rk + m) : 0.f; };
-    auto Kf = [&](int i, int m) -> float { return i < x.len ? ldf(kp + i * rk + m) : 0.f; };
-    auto Vf = [&](int i, int m) -> float { return i < x.len ? ldf(vp + i * rv + m) : 0.f; };
-    auto Bf = [&](int i, int m) -> float { return i < x.len ? p.bv[base_k + i * rk + m] : 0.f; };
-    auto Wf = [&](int i, int m) -> float { return i < x.len ? p.wv[base_v + i * rv + m] : 0.f; };
-    float* wsG = reinterpret_cast<float*>(p.ws + p.L.gamma) + (size_t)x.ch * kC * DK;
-    float* wsT = reinterpret_cast<float*>(p.ws + p.L.Tm) + (size_t)x.ch * kC * kC;
-    float* wsP = reinterpret_cast<float*>(p.ws + p.L.Pm) + (size_t)x.ch * kC * kC;
-    float* wsW = reinterpret_cast<float*>(p.ws + p.L.W) + (size_t)x.ch * kC * DK;
-    float* wsU = reinterpret_cast<float*>(p.ws + p.L.Ut) + (size_t)x.ch * kC * DV;
+template <int DK, int DV>
+struct PrepTiles {
+    static constexpr int PM = pitch(DK > DV ? DK : DV), COPY = 96 * pitch(DK) > 2 * kC * kPc ? 96 * pitch(DK) : 2 * kC * kPc;
+    static constexpr int G = 0;                       // gam, then dO
+    static constexpr int Q = G + kC * PM;             // q, scaled, then X = Gam . Q - P W
+    static constexpr int K = Q + kC * pitch(DK);      // k, then Gam . b . K
+    static constexpr int R = K + kC * pitch(DK);      // b . k, scaled, then w . V, then W
+    static constexpr int C = R + kC * PM;             // scaled copies of the keys, then T and scratch
+    static constexpr int A = C + COPY;
+    static constexpr int P = A + kC * kPc;
+    static constexpr size_t BYTES = sizeof(float) * (P + kC * kPc);
+    static_assert(BYTES + sizeof(Refs<DK>) <= 227 * 1024, "shared memory budget");
+};
 
-    cumulate_gates<DK>(p, x, gam);
-    __syncthreads();
-    for (int t = threadIdx.x; t < kC * DK; t += blockDim.x) wsG[t] = gam[(t / DK) * (DK + 1) + t % DK];
-    // A (strictly lower) and P (lower, diagonal included): the decay sits inside the contraction over the channel
-    tiles(kC, kC, [&](int i0, int j0) {
-        float aa[4][4] = {}, pp[4][4] = {};
-        mac_decay<DK>(aa, i0, j0, 1, gam, [&](int i, int m) { return Bf(i, m) * Kf(i, m); }, Kf);
-        mac_decay<DK>(pp, i0, j0, 0, gam, Qf, Kf);
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-                A[i0 + a][j0 + b] = aa[a][b];
-                wsP[(i0 + a) * kC + j0 + b] = pp[a][b];
+template <typename IO, int DK, int DV>
+__global__ void __launch_bounds__(kThreads, 1) vprep_kernel(Problem p, int mode) {
+    if (!p.fallback) init_header_if_untabled(p);
+    ChunkInfo x;
+    if ((p.fallback && !vec_go(p)) || !chunk_info(p, x)) return;
+    using L = PrepTiles<DK, DV>;
+    constexpr int PK = pitch(DK), PV = pitch(DV);
+    extern __shared__ __align__(16) float sm[];
+    float *G = sm + L::G, *Q = sm + L::Q, *K = sm + L::K, *R = sm + L::R, *C = sm + L::C, *A = sm + L::A, *Pm = sm + L::P;
+    float *T = C, *S = C + kC * kPc, *O = G;
+    __shared__ Refs<DK> refs;
+    const bool fwd = mode != PREP_BWD, bwd = mode != PREP_FWD;
+    const int H = p.d.H, tid = threadIdx.x;
+    const Thread t;
+    const Out<DK> ok(t);
+    const Out<DV> ov(t);
+    const size_t rk = (size_t)H * DK, rv = (size_t)H * DV, base_k = ((size_t)x.tok0 * H + x.hd) * DK, base_v = ((size_t)x.tok0 * H + x.hd) * DV;
+    float* wsG = block_of(p, p.L.gamma, x.ch, kC * DK);
+    float* wsW = block_of(p, p.L.W, x.ch, kC * DK);
+    float* wsP = block_of(p, p.L.Pm, x.ch, kC * kC);
+    const float sc = p.d.scale;
+
+    load_rows<DK>(Q, rows_of<IO>(p.q, x, H, DK), rk, x.len);
+    if (fwd) {
+        load_rows<DK>(K, rows_of<IO>(p.k, x, H, DK), rk, x.len);
+        cp_commit();
+        // chunk-local cumulative log decay per channel; rows beyond the sequence repeat the last valid one
+        if (tid < DK) {
+            float s = 0.f;
+#pragma unroll 1
+            for (int i0 = 0; i0 < kC; i0 += 16) {   // sixteen loads in flight, then their running sum in token order
+                float g[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) g[k] = i0 + k < x.len ? p.gv[base_k + (size_t)(i0 + k) * rk + tid] : 0.f;
+#pragma unroll
+                for (int k = 0; k < 16; ++k) { s += g[k]; G[(i0 + k) * PK + tid] = s; }
             }
-    });
+        }
+        for (int e = tid; e < 2 * kC * kPc; e += kThreads) A[e] = 0.f;   // (A and P lie behind each other)
+        cp_wait<0>();
+        __syncthreads();
+        make_refs(refs, G);
+        for (int e = tid; e < kC * DK; e += kThreads) {
+            const int i = e / DK, r = e % DK;
+            const float k = K[i * PK + r];
+            R[i * PK + r] = i < x.len ? p.bv[base_k + i * rk + r] * k : 0.f;
+            wsG[e] = G[i * PK + r];
+            block_of(p, p.L.Kb, x.ch, kC * DK)[e] = k * expf(G[(kC - 1) * PK + r] - G[i * PK + r]);
+        }
+        __syncthreads();
+        // pairs inside a block: 2 x 2 of them per thread, the 36 pieces of a block that reach the diagonal
+        if (tid < kNB * 36) {
+            const int I = tid / 36;
+            int n = tid % 36, a = 0;
+            while (n > a) { n -= a + 1; ++a; }   // piece (a, n), n <= a
+            const int i = I * kB + 2 * a, j = I * kB + 2 * n;
+            float aa[2][2] = {}, pp[2][2] = {};
+#pragma unroll 1
+            for (int r = 0; r < DK; r += 4) {
+                float gi[2][4], gj[2][4], q[2][4], b[2][4], k[2][4];
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    *reinterpret_cast<float4*>(gi[y]) = ld4(G + (i + y) * PK + r);
+                    *reinterpret_cast<float4*>(gj[y]) = ld4(G + (j + y) * PK + r);
+                    *reinterpret_cast<float4*>(q[y]) = ld4(Q + (i + y) * PK + r);
+                    *reinterpret_cast<float4*>(b[y]) = ld4(R + (i + y) * PK + r);
+                    *reinterpret_cast<float4*>(k[y]) = ld4(K + (j + y) * PK + r);
+                }
+#pragma unroll
+                for (int z = 0; z < 4; ++z)
+#pragma unroll
+                    for (int y = 0; y < 2; ++y)
+#pragma unroll
+                        for (int w = 0; w < 2; ++w) {
+                            const float ke = k[w][z] * expf(i + y >= j + w ? gi[y][z] - gj[w][z] : 0.f);   // (above the diagonal: not used)
+                            aa[y][w] = fmaf(b[y][z], ke, aa[y][w]);
+                            pp[y][w] = fmaf(q[y][z], ke, pp[y][w]);
+                        }
+            }
+#pragma unroll
+            for (int y = 0; y < 2; ++y)
+#pragma unroll
+                for (int w = 0; w < 2; ++w) {
+                    if (j + w < i + y) A[(i + y) * kPc + j + w] = aa[y][w];
+                    if (j + w <= i + y) Pm[(i + y) * kPc + j + w] = pp[y][w];
+                }
+        }
+        __syncthreads();
+        make_copies<DK>(C, G, refs, [&](int j, int r) { return K[j * PK + r]; });
+        scale_rows<DK>(Q, G, refs);
+        scale_rows<DK>(R, G, refs);
+        __syncthreads();
+        // pairs of blocks J < I: A and P, 16 threads a 16 x 16 block, 4 x 4 each
+        if (tid < 192) {
+            const int which = tid / 96, o = tid % 96, blk = o / 16, ti = ((o % 16) >> 2) * 4, tj = o & 3;
+            const int I = blk == 0 ? 1 : blk < 3 ? 2 : 3, J = blk == 0 ? 0 : blk < 3 ? blk - 1 : blk - 3;
+            float acc[4][4];
+            zero(acc);
+            mac<1, A_ROW, B_ROW, 0, 4>(acc, which ? Q : R, nullptr, PK, I * kB + ti, C + (copy_row(I) + J * kB) * PK, PK, tj, 0, DK);
+            float* dst = (which ? Pm : A) + (I * kB + ti) * kPc + J * kB + tj;
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int y = 0; y < 4; ++y) dst[r * kPc + 4 * y] = acc[r][y];
+        }
+        for (int e = tid; e < kC * DK; e += kThreads) {   // Gam . b . K, the right-hand side of W
+            const int i = e / DK, r = e % DK;
+            K[i * PK + r] = R[i * PK + r] * refs.eref[i / kB][r];
+        }
+        __syncthreads();
+        load_rows<DV>(R, rows_of<IO>(p.v, x, H, DV), rv, x.len);
+        cp_commit();
+        if (bwd) load_rows<DV>(O, rows_of<IO>(p.dO, x, H, DV), rv, x.len);
+        cp_commit();
+        for (int e = tid; e < kC * kC; e += kThreads) wsP[e] = Pm[(e / kC) * kPc + e % kC];
+        invert(A, T, S);
+        cp_wait<1>();
+        __syncthreads();
+        float* wsT = block_of(p, p.L.Tm, x.ch, kC * kC);
+        for (int e = tid; e < kC * kC; e += kThreads) wsT[e] = T[(e / kC) * kPc + e % kC];
+        for (int e = tid; e < kC * DV; e += kThreads) {
+            const int i = e / DV, r = e % DV;
+            if (i < x.len) R[i * PV + r] *= p.wv[base_v + i * rv + r];
+        }
+        __syncthreads();
+        float* wsU = block_of(p, p.L.Ut, x.ch, kC * DV);
+        {
+            float acc[Out<DV>::R][4];
+            tri_product<DV, A_ROW, A_LOWER>(t, T, R, PV, acc);
+#pragma unroll
+            for (int r = 0; r < Out<DV>::R; ++r)
+#pragma unroll
+                for (int y = 0; y < 4; ++y) wsU[ov.row(r) * DV + ov.c + 8 * y] = acc[r][y];
+        }
+        __syncthreads();
+        {
+            float acc[Out<DK>::R][4];
+            tri_product<DK, A_ROW, A_LOWER>(t, T, K, PK, acc);
+#pragma unroll
+            for (int r = 0; r < Out<DK>::R; ++r)
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                    wsW[ok.row(r) * DK + ok.c + 8 * y] = acc[r][y];
+                    R[ok.row(r) * PK + ok.c + 8 * y] = acc[r][y];
+                }
+        }
+        if (!bwd) return;
+    } else {
+        load_block<kC, DK>(G, wsG);
+        load_block<kC, DK>(R, wsW);
+        load_block<kC, kC>(Pm, wsP);
+        cp_commit();
+        cp_wait<0>();
+        __syncthreads();
+        make_refs(refs, G);
+        __syncthreads();
+        scale_rows<DK>(Q, G, refs);
+        __syncthreads();
+        load_rows<DV>(O, rows_of<IO>(p.dO, x, H, DV), rv, x.len);
+        cp_commit();
+    }
+    cp_wait<0>();
     __syncthreads();
-    // T = (I + A)^-1: column j of T solves (I + A) x = e_j by forward substitution (one thread per column).
-    if (threadIdx.x < kC) {
-        const int j = threadIdx.x;
-        for (int i = 0; i < kC; ++i) {
-            float s = (i == j) ? 1.f : 0.f;
-            for (int m = j; m < i; ++m) s = fmaf(-A[i][m], Ti[m][j], s);
-            Ti[i][j] = (i >= j) ? s : 0.f;
+    // dU0 = scale P^T dO
+    float* wsD = block_of(p, p.L.dU, x.ch, kC * DV);
+    {
+        float acc[Out<DV>::R][4];
+        tri_product<DV, A_COL, A_UPPER>(t, Pm, O, PV, acc);
+#pragma unroll
+        for (int r = 0; r < Out<DV>::R; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) wsD[ov.row(r) * DV + ov.c + 8 * y] = sc * acc[r][y];
+    }
+    {   // X = Gam . Q - P W, in place over Q
+        float acc[Out<DK>::R][4];
+        tri_product<DK, A_ROW, A_LOWER>(t, Pm, R, PK, acc);
+#pragma unroll
+        for (int r = 0; r < Out<DK>::R; ++r) {
+            float* q = Q + ok.row(r) * PK + ok.c;
+#pragma unroll
+            for (int y = 0; y < 4; ++y) q[8 * y] = fmaf(q[8 * y], refs.eref[ok.row(r) / kB][ok.c + 8 * y], -acc[r][y]);
         }
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < kC * kC; t += blockDim.x) wsT[t] = Ti[t / kC][t % kC];
-    // W = T (Gam . b . K),  Ut = T (w . V)
-    tiles(kC, DK, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, kC, [&](int i, int m) { return Ti[i][m]; },
-            [&](int m, int j) { return expf(gam[m * (DK + 1) + j]) * Bf(m, j) * Kf(m, j); });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) wsW[(i0 + a) * DK + j0 + b] = acc[a][b];
-    });
-    tiles(kC, DV, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, kC, [&](int i, int m) { return Ti[i][m]; }, [&](int m, int j) { return Wf(m, j) * Vf(m, j); });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) wsU[(i0 + a) * DV + j0 + b] = acc[a][b];
-    });
-}
-
-// ------------------------------------------------------------------------------------------------
-// veprep: E = scale (Gam . Q - P W)^T dO
-// ------------------------------------------------------------------------------------------------
-template <typename IO, int DK, int DV>
-__global__ void __launch_bounds__(kThreads) veprep_kernel(Problem p) {
-    ChunkCtx x;
-    if (!vec_go(p) || !chunk_ctx(p, x)) return;
-    const int H = p.d.H;
-    const IO* qp = reinterpret_cast<const IO*>(p.q) + ((size_t)x.tok0 * H + x.hd) * DK;
-    const IO* gp = reinterpret_cast<const IO*>(p.dO) + ((size_t)x.tok0 * H + x.hd) * DV;
-    const size_t rk = (size_t)H * DK, rv = (size_t)H * DV;
-    auto Qf = [&](int i, int m) -> float { return i < x.len ? ldf(qp + i * rk + m) : 0.f; };
-    auto Of = [&](int i, int m) -> float { return i < x.len ? ldf(gp + i * rv + m) : 0.f; };
-    const float* wsG = reinterpret_cast<const float*>(p.ws + p.L.gamma) + (size_t)x.ch * kC * DK;
-    const float* wsP = reinterpret_cast<const float*>(p.ws + p.L.Pm) + (size_t)x.ch * kC * kC;
-    const float* wsW = reinterpret_cast<const float*>(p.ws + p.L.W) + (size_t)x.ch * kC * DK;
-    float* wsE = reinterpret_cast<float*>(p.ws + p.L.E) + (size_t)x.ch * DK * DV;
-    float* X = reinterpret_cast<float*>(p.ws + p.L.scratch + p.L.scratch_per_ch * x.ch);  // [64, DK]
-    tiles(kC, DK, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, kC, [&](int i, int m) { return wsP[i * kC + m]; }, [&](int m, int j) { return wsW[m * DK + j]; });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b)
-                X[(i0 + a) * DK + j0 + b] = expf(wsG[(i0 + a) * DK + j0 + b]) * Qf(i0 + a, j0 + b) - acc[a][b];
-    });
-    __syncthreads();
-    const float sc = p.d.scale;
-    tiles(DK, DV, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, kC, [&](int i, int m) { return X[m * DK + i]; }, Of);
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) wsE[(i0 + a) * DV + j0 + b] = sc * acc[a][b];
-    });
-}
-
-// ------------------------------------------------------------------------------------------------
-// Forward and reverse carries in low-rank form.  One CTA per (sequence, head); the fp32 state lives in shared memory.
-// ------------------------------------------------------------------------------------------------
-template <typename IO, int DK, int DV, bool REVERSE>
-__global__ void __launch_bounds__(kThreads) vscan_kernel(Problem p) {
-    extern __shared__ __align__(16) float sm[];
-    float* cur = sm;                  // [DK][DV]
-    float* nxt = sm + DK * DV;
-    float* Y = nxt + DK * DV;         // [64][DV]: U = Ut - W h (forward) or Kb dh' (reverse)
-    const int H = p.d.H, n = blockIdx.x / H, hd = blockIdx.x % H;
-    const int32_t* seq_first = reinterpret_cast<const int32_t*>(p.ws + p.L.seq_first);
-    if (!vec_go(p)) return;
-    const int c0 = seq_first[n], c1 = seq_first[n + 1];
-    const size_t soff = ((size_t)n * H + hd) * DK * DV;
-    const float* init = REVERSE ? p.dhT : p.h0;
-    for (int t = threadIdx.x; t < DK * DV; t += blockDim.x) cur[t] = init ? init[soff + t] : 0.f;
-    __syncthreads();
-    const size_t rk = (size_t)H * DK;
-    for (int s = 0; s < c1 - c0; ++s) {
-        const int c = REVERSE ? (c1 - 1 - s) : (c0 + s);
-        const size_t ch = (size_t)c * H + hd;
-        const int tok0 = reinterpret_cast<const int32_t*>(p.ws + p.L.chunk_tok0)[c];
-        const int len = reinterpret_cast<const int32_t*>(p.ws + p.L.chunk_len)[c];
-        const IO* kp = reinterpret_cast<const IO*>(p.k) + ((size_t)tok0 * H + hd) * DK;
-        const float* wsG = reinterpret_cast<const float*>(p.ws + p.L.gamma) + ch * kC * DK;
-        const float* wsW = reinterpret_cast<const float*>(p.ws + p.L.W) + ch * kC * DK;
-        const float* wsU = reinterpret_cast<const float*>(p.ws + p.L.Ut) + ch * kC * DV;
-        const float* wsE = reinterpret_cast<const float*>(p.ws + p.L.E) + ch * DK * DV;
-        float* keep = reinterpret_cast<float*>(p.ws + (REVERSE ? p.L.dhn : p.L.hc)) + ch * DK * DV;
-        // Kb_j[r] = exp(gam_e[r] - gam_j[r]) k_j[r]
-        auto Kb = [&](int j, int r) -> float {
-            return j < len ? expf(wsG[(kC - 1) * DK + r] - wsG[j * DK + r]) * ldf(kp + j * rk + r) : 0.f;
-        };
-        for (int t = threadIdx.x; t < DK * DV; t += blockDim.x) keep[t] = cur[t];
-        tiles(kC, DV, [&](int i0, int j0) {
-            float acc[4][4] = {};
-            if (REVERSE) mac(acc, i0, j0, DK, Kb, [&](int m, int j) { return cur[m * DV + j]; });
-            else mac(acc, i0, j0, DK, [&](int i, int m) { return wsW[i * DK + m]; }, [&](int m, int j) { return cur[m * DV + j]; });
-            for (int a = 0; a < 4; ++a)
-                for (int b = 0; b < 4; ++b) {
-                    const int t = (i0 + a) * DV + j0 + b;
-                    Y[t] = REVERSE ? acc[a][b] : wsU[t] - acc[a][b];
-                }
-        });
-        __syncthreads();
-        tiles(DK, DV, [&](int i0, int j0) {
-            float acc[4][4] = {};
-            if (REVERSE) mac(acc, i0, j0, kC, [&](int i, int m) { return wsW[m * DK + i]; }, [&](int m, int j) { return Y[m * DV + j]; });
-            else mac(acc, i0, j0, kC, [&](int i, int m) { return Kb(m, i); }, [&](int m, int j) { return Y[m * DV + j]; });
-            for (int a = 0; a < 4; ++a)
-                for (int b = 0; b < 4; ++b) {
-                    const int t = (i0 + a) * DV + j0 + b;
-                    const float Ge = expf(wsG[(kC - 1) * DK + i0 + a]);
-                    nxt[t] = REVERSE ? Ge * cur[t] + wsE[t] - acc[a][b] : Ge * cur[t] + acc[a][b];
-                }
-        });
-        __syncthreads();
-        float* tmp = cur; cur = nxt; nxt = tmp;
+    // E = scale X^T dO, 64 rows at a time
+    float* wsE = block_of(p, p.L.E, x.ch, DK * DV);
+#pragma unroll 1
+    for (int r0 = 0; r0 < DK; r0 += 64) {
+        float acc[Out<DV>::R][4];
+        zero(acc);
+        mac<Out<DV>::R / 4, A_COL, B_COL>(acc, Q + r0, Q + r0 + 32, PK, ov.r0, O, PV, ov.c, 0, kC);
+#pragma unroll
+        for (int r = 0; r < Out<DV>::R; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) wsE[(r0 + ov.row(r)) * DV + ov.c + 8 * y] = sc * acc[r][y];
     }
-    float* fin = REVERSE ? p.dh0 : p.hT;
-    if (fin) for (int t = threadIdx.x; t < DK * DV; t += blockDim.x) fin[soff + t] = cur[t];
 }
 
 // ------------------------------------------------------------------------------------------------
-// Forward output (optional): o = scale ((Gam . Q) h + P (Ut - W h))
+// vscan: forward and reverse carries (ffma_scan.cuh).
 // ------------------------------------------------------------------------------------------------
+template <int DK, int DV>
+__global__ void __launch_bounds__(kThreads) vscan_kernel(Problem p, int dirs) {
+    extern __shared__ __align__(16) float sm[];
+    if (!vec_go(p)) return;
+    scan_block<DK, DV, true>(p, dirs, sm);
+}
+
+// ------------------------------------------------------------------------------------------------
+// vout, forward output (optional): o = scale ((Gam . Q) h + P U)
+// ------------------------------------------------------------------------------------------------
+template <int DK, int DV>
+constexpr size_t vout_smem() { return sizeof(float) * (kC * pitch(DK) + DK * pitch(DV) + kC * pitch(DV) + kC * kPc); }
+
 template <typename IO, int DK, int DV>
-__global__ void __launch_bounds__(kThreads) vout_kernel(Problem p) {
-    ChunkCtx x;
-    if (!vec_go(p) || !chunk_ctx(p, x)) return;
+__global__ void __launch_bounds__(kThreads, 1) vout_kernel(Problem p) {
+    ChunkInfo x;
+    if (!vec_go(p) || !chunk_info(p, x)) return;
+    constexpr int PK = pitch(DK), PV = pitch(DV), R = Out<DV>::R;
+    extern __shared__ __align__(16) float sm[];
+    float* sQ = sm;
+    float* sH = sQ + kC * PK;
+    float* sU = sH + DK * PV;
+    float* Pm = sU + kC * PV;
     const int H = p.d.H;
-    const IO* qp = reinterpret_cast<const IO*>(p.q) + ((size_t)x.tok0 * H + x.hd) * DK;
-    IO* op = reinterpret_cast<IO*>(p.o) + ((size_t)x.tok0 * H + x.hd) * DV;
-    const size_t rk = (size_t)H * DK, rv = (size_t)H * DV;
-    auto Qf = [&](int i, int m) -> float { return i < x.len ? ldf(qp + i * rk + m) : 0.f; };
-    const float* wsG = reinterpret_cast<const float*>(p.ws + p.L.gamma) + (size_t)x.ch * kC * DK;
-    const float* wsP = reinterpret_cast<const float*>(p.ws + p.L.Pm) + (size_t)x.ch * kC * kC;
-    const float* wsW = reinterpret_cast<const float*>(p.ws + p.L.W) + (size_t)x.ch * kC * DK;
-    const float* wsU = reinterpret_cast<const float*>(p.ws + p.L.Ut) + (size_t)x.ch * kC * DV;
-    const float* wsH = reinterpret_cast<const float*>(p.ws + p.L.hc) + (size_t)x.ch * DK * DV;
-    auto Pf = [&](int i, int m) -> float { return wsP[i * kC + m]; };
-    auto Wm = [&](int i, int m) -> float { return wsW[i * DK + m]; };
-    auto Um = [&](int i, int j) -> float { return wsU[i * DV + j]; };
-    auto Hf = [&](int m, int j) -> float { return wsH[m * DV + j]; };
-    float* U = reinterpret_cast<float*>(p.ws + p.L.scratch + p.L.scratch_per_ch * x.ch);  // [64, DV]
-    tiles(kC, DV, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, DK, Wm, Hf);
-        for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) U[(i0 + a) * DV + j0 + b] = Um(i0 + a, j0 + b) - acc[a][b];
-    });
+    const Thread t;
+    const Out<DV> o(t);
+    load_rows<DK>(sQ, rows_of<IO>(p.q, x, H, DK), (size_t)H * DK, x.len);
+    load_block<DK, DV>(sH, block_of(p, p.L.hc, x.ch, DK * DV));
+    load_block<kC, DV>(sU, block_of(p, p.L.U, x.ch, kC * DV));
+    load_block<kC, kC>(Pm, block_of(p, p.L.Pm, x.ch, kC * kC));
+    cp_commit();
+    cp_wait<0>();
     __syncthreads();
+    const float* wsG = block_of(p, p.L.gamma, x.ch, kC * DK);
+    for (int e = threadIdx.x; e < kC * DK; e += kThreads) sQ[(e / DK) * PK + e % DK] *= expf(wsG[e]);
+    __syncthreads();
+    float acc[R][4];
+    zero(acc);
+    mac<R / 4, A_ROW, B_COL>(acc, sQ, sQ + 32 * PK, PK, o.r0, sH, PV, o.c, 0, DK);
+    mac<R / 4, A_ROW, B_COL>(acc, Pm, Pm + 32 * kPc, kPc, o.r0, sU, PV, o.c, 0, kC);
+    IO* op = rows_of<IO>(p.o, x, H, DV);
+    const size_t rv = (size_t)H * DV;
     const float sc = p.d.scale;
-    tiles(kC, DV, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        mac(acc, i0, j0, DK, [&](int i, int m) { return expf(wsG[i * DK + m]) * Qf(i, m); }, Hf);
-        mac(acc, i0, j0, kC, Pf, [&](int m, int j) { return U[m * DV + j]; });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b)
-                if (i0 + a < x.len) stf(op + (i0 + a) * rv + j0 + b, sc * acc[a][b]);
-    });
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (o.row(r) < x.len)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) stf(op + o.row(r) * rv + o.c + 8 * y, sc * acc[r][y]);
 }
 
 // ------------------------------------------------------------------------------------------------
-// vintra: token gradients of one (chunk, head).
+// vintra: token gradients of one (chunk, head).  K#2 in its short form: dXv = T^T dU, dXk = -dXv h^T, dA = -stril(dXv U^T).
+//     dq_i = scale Gam_i (dO h^T)_i + sum_{j <= i} dP_ij e^{gam_i - gam_j} k_j
+//     row_i = -Gam_i (dXv h^T)_i + sum_{j < i} dA_ij e^{gam_i - gam_j} k_j
+//     col_j = e_j (U dh'^T)_j + sum_{i >= j} e^{gam_i - gam_j} (dP_ij q_i + dA_ij b_i k_i)
+//     dk = b row + col,  db = k row,  dgam = q dq + b k row - k col,  and the last row adds
+//     sum_j k_j e_j (U dh'^T)_j + Gam_e rowdot(dh', h)
+// First the products with the states (results in registers), then, with their tiles gone, the pairs of blocks from the scaled
+// tiles; a last pass in which a thread owns a channel of a block adds the pairs inside the block and writes everything.
 // ------------------------------------------------------------------------------------------------
+template <int DK, int DV>
+struct IntraTiles {
+    static constexpr int PM = pitch(DK > DV ? DK : DV), PK = pitch(DK), PV = pitch(DV);
+    static constexpr int S0 = 0;                  // dO
+    static constexpr int S1 = S0 + kC * PM;       // dU, then dXv
+    static constexpr int U = S1 + kC * PM;
+    static constexpr int H = U + kC * PV;         // h, then dh'
+    static constexpr int END1 = H + DK * PV;
+    static constexpr int G = 0;                   // gam                        (over dO)
+    static constexpr int Q = G + kC * PK;         // q, scaled; then row        (over dXv)
+    static constexpr int R = Q + kC * PK;         // b . k, scaled; then col
+    static constexpr int C = R + kC * PK;         // scaled copies of the keys; then dq, then dgam
+    static constexpr int END2 = C + 96 * PK;
+    static constexpr int T = END1 > END2 ? END1 : END2;   // T, then dA
+    static constexpr int P = T + kC * kPc;        // scale tril(dO U^T)
+    static constexpr size_t BYTES = sizeof(float) * (P + kC * kPc);
+    static_assert(Q + kC * PK <= U, "gam and q arrive while U and dh' are in use");
+    static_assert(BYTES + sizeof(Refs<DK>) + 4 * (kNB + 1) * DK <= 227 * 1024, "shared memory budget");
+};
+
 template <typename IO, int DK, int DV>
-__global__ void __launch_bounds__(kThreads) vintra_kernel(Problem p) {
-    ChunkCtx x;
-    if (!vec_go(p) || !chunk_ctx(p, x)) return;
-    extern __shared__ __align__(16) float smf[];
-    float* gam = smf;                                                                       // [64][DK + 1]
-    float (*dP)[kC + 1] = reinterpret_cast<float (*)[kC + 1]>(smf + kC * (DK + 1));         // scale tril(dO U^T)
-    float (*dA)[kC + 1] = dP + kC;                                                          // -stril(dXk W^T + dXv Ut^T)
-    const int H = p.d.H;
-    const size_t base_k = ((size_t)x.tok0 * H + x.hd) * DK, base_v = ((size_t)x.tok0 * H + x.hd) * DV;
+__global__ void __launch_bounds__(kThreads, 1) vintra_kernel(Problem p) {
+    ChunkInfo x;
+    if (!vec_go(p) || !chunk_info(p, x)) return;
+    using L = IntraTiles<DK, DV>;
+    constexpr int PK = pitch(DK), PV = pitch(DV), NH = DK / 64;
+    extern __shared__ __align__(16) float sm[];
+    float *s0 = sm + L::S0, *s1 = sm + L::S1, *sU = sm + L::U, *sH = sm + L::H, *sT = sm + L::T, *sP = sm + L::P;
+    float *G = sm + L::G, *Q = sm + L::Q, *R = sm + L::R, *C = sm + L::C;
+    __shared__ Refs<DK> refs;
+    __shared__ float ends[DK], blk[kNB][DK];   // chunk-end term of dg; first: its parts by row blocks; later: block sums of dgam
+    const int H = p.d.H, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const Thread t;
     const size_t rk = (size_t)H * DK, rv = (size_t)H * DV;
+    const size_t base_k = ((size_t)x.tok0 * H + x.hd) * DK, base_v = ((size_t)x.tok0 * H + x.hd) * DV;
     const IO* qp = reinterpret_cast<const IO*>(p.q) + base_k;
     const IO* kp = reinterpret_cast<const IO*>(p.k) + base_k;
-    const IO* vp = reinterpret_cast<const IO*>(p.v) + base_v;
-    const IO* gp = reinterpret_cast<const IO*>(p.dO) + base_v;
+    const float* wsH = block_of(p, p.L.hc, x.ch, DK * DV);
+    const float* wsG = block_of(p, p.L.gamma, x.ch, kC * DK);
+    const float sc = p.d.scale;
+
+    load_rows<DV>(s0, rows_of<IO>(p.dO, x, H, DV), rv, x.len);
+    load_block<kC, DV>(sU, block_of(p, p.L.U, x.ch, kC * DV));
+    cp_commit();
+    load_block<kC, DV>(s1, block_of(p, p.L.dU, x.ch, kC * DV));
+    load_block<kC, kC>(sT, block_of(p, p.L.Tm, x.ch, kC * kC));
+    cp_commit();
+    load_block<DK, DV>(sH, wsH);
+    cp_commit();
+    cp_wait<2>();
+    __syncthreads();
+    const int I = t.rn / kB;                      // the rows of a warp are one block of tokens
+    const bool below = (warp >> 2) * 32 <= I * kB + kB - 1;
+    {   // dP = scale tril(dO U^T)
+        float acc[4][4];
+        zero(acc);
+        if (below) mac<1, A_ROW, B_ROW>(acc, s0, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) sP[(t.rn + r) * kPc + t.cn + 8 * y] = t.cn + 8 * y <= t.rn + r ? sc * acc[r][y] : 0.f;
+    }
+    cp_wait<1>();
+    __syncthreads();
+    {   // dXv = T^T dU, in place; dv = w . dXv, dw = v . dXv
+        const Out<DV> o(t);
+        float acc[Out<DV>::R][4];
+        tri_product<DV, A_COL, A_UPPER>(t, sT, s1, PV, acc);
+        __syncthreads();
+        const IO* vp = reinterpret_cast<const IO*>(p.v) + base_v;
+        IO* dvp = reinterpret_cast<IO*>(p.dv) + base_v;
+#pragma unroll
+        for (int r = 0; r < Out<DV>::R; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int i = o.row(r), c = o.c + 8 * y;
+                s1[i * PV + c] = acc[r][y];
+                if (i < x.len) {
+                    stf(dvp + i * rv + c, p.wv[base_v + i * rv + c] * acc[r][y]);
+                    p.dwv[base_v + i * rv + c] = ldf(vp + i * rv + c) * acc[r][y];
+                }
+            }
+    }
+    cp_wait<0>();
+    __syncthreads();
+    {   // dA = -stril(dXv U^T), over T
+        float acc[4][4];
+        zero(acc);
+        if (below) mac<1, A_ROW, B_ROW>(acc, s1, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) sT[(t.rn + r) * kPc + t.cn + 8 * y] = t.cn + 8 * y < t.rn + r ? -acc[r][y] : 0.f;
+    }
+    // [dO; dXv] h^T: rows 0..3 become dq, rows 4..7 the row role of k
+    float acc[NH][8][4];
+#pragma unroll
+    for (int n = 0; n < NH; ++n) {
+        zero(acc[n]);
+        mac<2, A_ROW, B_ROW>(acc[n], s0, s1, PV, t.rn, sH + n * 64 * PV, PV, t.cn, 0, DV);
+    }
+    __syncthreads();
+    load_block<DK, DV>(sH, block_of(p, p.L.dhn, x.ch, DK * DV));
+    load_block<kC, DK>(G, wsG);
+    load_rows<DK>(Q, qp, rk, x.len);
+    cp_commit();
+    cp_wait<0>();
+    __syncthreads();
+    make_refs(refs, G);
+    // col = e . (U dh'^T); its dot with k over the tokens, per channel, goes to the chunk end
+    float col[NH][4][4];
+#pragma unroll
+    for (int n = 0; n < NH; ++n) {
+        zero(col[n]);
+        mac<1, A_ROW, B_ROW>(col[n], sU, nullptr, PV, t.rn, sH + n * 64 * PV, PV, t.cn, 0, DV);
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+            const int c = n * 64 + t.cn + 8 * y;
+            float s = 0.f;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int i = t.rn + r;
+                const float g = G[i * PK + c], Gi = expf(g);
+                col[n][r][y] *= expf(G[(kC - 1) * PK + c] - g);
+                acc[n][r][y] *= sc * Gi;
+                acc[n][4 + r][y] *= -Gi;
+                if (i < x.len) s = fmaf(ldf(kp + i * rk + c), col[n][r][y], s);
+            }
+            s += __shfl_xor_sync(0xffffffffu, s, 8);
+            s += __shfl_xor_sync(0xffffffffu, s, 16);
+            if (lane < 8) blk[I][c] = s;
+        }
+    }
+    // Gam_e rowdot(dh', h): one warp per state row (h from the workspace: its tile has been overwritten)
+    for (int r = warp; r < DK; r += kThreads / 32) {
+        float s = 0.f;
+        if (lane * 4 < DV) {
+            const float4 a = ld4(wsH + (size_t)r * DV + lane * 4), b = ld4(sH + r * PV + lane * 4);
+            s = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w)));
+        }
+        s = warp_total(s);
+        if (lane == 0) ends[r] = expf(G[(kC - 1) * PK + r]) * s;
+    }
+    __syncthreads();
+    if (tid < DK) ends[tid] += (blk[0][tid] + blk[1][tid]) + (blk[2][tid] + blk[3][tid]);
+    for (int e = tid; e < kC * DK; e += kThreads) {
+        const int i = e / DK, r = e % DK;
+        R[i * PK + r] = i < x.len ? p.bv[base_k + i * rk + r] * ldf(kp + i * rk + r) * expf(G[i * PK + r] - refs.ref[i / kB][r]) : 0.f;
+    }
+    scale_rows<DK>(Q, G, refs);
+    make_copies<DK>(C, G, refs, [&](int j, int r) { return j < x.len ? ldf(kp + j * rk + r) : 0.f; });
+    __syncthreads();
+    // pairs of blocks J < I
+#pragma unroll
+    for (int n = 0; n < NH; ++n) {
+        float tmp[8][4];
+        zero(tmp);
+        mac<2, A_ROW, B_COL>(tmp, sP, sT, kPc, t.rn, C + copy_row(I) * PK + n * 64, PK, t.cn, 0, I * kB);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int c = n * 64 + t.cn + 8 * y;
+                const float e = expf(G[(t.rn + r) * PK + c] - refs.ref[I][c]);
+                acc[n][r][y] = fmaf(e, tmp[r][y], acc[n][r][y]);
+                acc[n][4 + r][y] = fmaf(e, tmp[4 + r][y], acc[n][4 + r][y]);
+            }
+#pragma unroll 1
+        for (int I2 = I + 1; I2 < kNB; ++I2) {
+            float tc[4][4];
+            zero(tc);
+            mac<1, A_COL, B_COL>(tc, sP, nullptr, kPc, t.rn, Q + n * 64, PK, t.cn, I2 * kB, I2 * kB + kB);
+            mac<1, A_COL, B_COL>(tc, sT, nullptr, kPc, t.rn, R + n * 64, PK, t.cn, I2 * kB, I2 * kB + kB);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                    const int c = n * 64 + t.cn + 8 * y;
+                    col[n][r][y] = fmaf(expf(refs.ref[I2][c] - G[(t.rn + r) * PK + c]), tc[r][y], col[n][r][y]);
+                }
+        }
+    }
+    __syncthreads();
+    // hand the sums so far to the owners of the channels: row over Q, col over R, dq over the copies
+#pragma unroll
+    for (int n = 0; n < NH; ++n)
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int o = (t.rn + r) * PK + n * 64 + t.cn + 8 * y;
+                C[o] = acc[n][r][y];
+                Q[o] = acc[n][4 + r][y];
+                R[o] = col[n][r][y];
+            }
+    __syncthreads();
     IO* dqp = reinterpret_cast<IO*>(p.dq) + base_k;
     IO* dkp = reinterpret_cast<IO*>(p.dk) + base_k;
-    IO* dvp = reinterpret_cast<IO*>(p.dv) + base_v;
-    auto Qf = [&](int i, int m) -> float { return i < x.len ? ldf(qp + i * rk + m) : 0.f; };
-    auto Kf = [&](int i, int m) -> float { return i < x.len ? ldf(kp + i * rk + m) : 0.f; };
-    auto Vf = [&](int i, int m) -> float { return i < x.len ? ldf(vp + i * rv + m) : 0.f; };
-    auto Of = [&](int i, int m) -> float { return i < x.len ? ldf(gp + i * rv + m) : 0.f; };
-    auto Bf = [&](int i, int m) -> float { return i < x.len ? p.bv[base_k + i * rk + m] : 0.f; };
-    auto Wf = [&](int i, int m) -> float { return i < x.len ? p.wv[base_v + i * rv + m] : 0.f; };
-    const float* wsG = reinterpret_cast<const float*>(p.ws + p.L.gamma) + (size_t)x.ch * kC * DK;
-    const float* Tm = reinterpret_cast<const float*>(p.ws + p.L.Tm) + (size_t)x.ch * kC * kC;
-    const float* Pm = reinterpret_cast<const float*>(p.ws + p.L.Pm) + (size_t)x.ch * kC * kC;
-    const float* W = reinterpret_cast<const float*>(p.ws + p.L.W) + (size_t)x.ch * kC * DK;
-    const float* Ut = reinterpret_cast<const float*>(p.ws + p.L.Ut) + (size_t)x.ch * kC * DV;
-    const float* hs = reinterpret_cast<const float*>(p.ws + p.L.hc) + (size_t)x.ch * DK * DV;     // per-chunk states, fp32
-    const float* dhs = reinterpret_cast<const float*>(p.ws + p.L.dhn) + (size_t)x.ch * DK * DV;
-    auto Hs = [&](int m, int j) -> float { return hs[m * DV + j]; };     // h[m][j]
-    auto DHs = [&](int m, int j) -> float { return dhs[m * DV + j]; };   // dh'[m][j]
-    float* scr = reinterpret_cast<float*>(p.ws + p.L.scratch + p.L.scratch_per_ch * x.ch);
-    float* U = scr;                    // [64, DV]
-    float* dU = U + kC * DV;           // [64, DV]
-    float* dXv = dU + kC * DV;         // [64, DV]
-    float* dOh = dXv + kC * DV;        // [64, DK]  dO h^T
-    float* dW = dOh + kC * DK;         // [64, DK]  later dgam
-    float* dXk = dW + kC * DK;         // [64, DK]
-    float* UdH = dXk + kC * DK;        // [64, DK]  U dh'^T
-    const float sc = p.d.scale;
-    auto G = [&](int i, int r) -> float { return gam[i * (DK + 1) + r]; };
+#pragma unroll 1
+    for (int task = tid; task < kNB * DK; task += kThreads) {   // one channel of one block of tokens
+        const int B = task / DK, r = task % DK, i0 = B * kB;
+        float q[kB], k[kB], b[kB], g[kB], dc[kB];
+#pragma unroll
+        for (int i = 0; i < kB; ++i) {
+            const bool live = i0 + i < x.len;
+            q[i] = live ? ldf(qp + (i0 + i) * rk + r) : 0.f;
+            k[i] = live ? ldf(kp + (i0 + i) * rk + r) : 0.f;
+            b[i] = live ? p.bv[base_k + (i0 + i) * rk + r] : 0.f;
+            g[i] = G[(i0 + i) * PK + r];
+            dc[i] = R[(i0 + i) * PK + r];
+        }
+        // a row at a time: its dq and row role are complete at once, the column roles collect
+#pragma unroll
+        for (int i = 0; i < kB; ++i) {
+            float dq = C[(i0 + i) * PK + r], row = Q[(i0 + i) * PK + r];
+            const float bk = b[i] * k[i];
+            const float* P_ = sP + (i0 + i) * kPc + i0;
+            const float* A_ = sT + (i0 + i) * kPc + i0;
+#pragma unroll
+            for (int j = 0; j <= i; ++j) {
+                const float e = j < i ? expf(g[i] - g[j]) : 1.f, pe = P_[j] * e, ae = A_[j] * e;   // (dA_ii = 0)
+                dq = fmaf(pe, k[j], dq);
+                row = fmaf(ae, k[j], row);
+                dc[j] = fmaf(pe, q[i], fmaf(ae, bk, dc[j]));
+            }
+            if (i0 + i < x.len) {
+                stf(dqp + (i0 + i) * rk + r, dq);
+                p.dbv[base_k + (i0 + i) * rk + r] = k[i] * row;
+            }
+            Q[(i0 + i) * PK + r] = row;
+            C[(i0 + i) * PK + r] = fmaf(q[i], dq, bk * row);
+        }
+        float run = 0.f;   // dgam, summed from the end of the block
+#pragma unroll
+        for (int i = kB - 1; i >= 0; --i) {
+            if (i0 + i < x.len) stf(dkp + (i0 + i) * rk + r, fmaf(b[i], Q[(i0 + i) * PK + r], dc[i]));
+            run += fmaf(-k[i], dc[i], C[(i0 + i) * PK + r]);
+            C[(i0 + i) * PK + r] = run;
+        }
+        blk[B][r] = run;
+    }
+    __syncthreads();
+    // dg_j = sum_{i >= j} dgam_i: the sum inside the block, the blocks behind it and the chunk end
+    for (int e = tid; e < kC * DK; e += kThreads) {
+        const int i = e / DK, r = e % DK;
+        if (i >= x.len) continue;
+        float s = ends[r];
+        for (int B = kNB - 1; B > i / kB; --B) s += blk[B][r];
+        p.dgv[base_k + i * rk + r] = s + C[i * PK + r];
+    }
+}
 
-    load_gamma<DK>(wsG, gam);
-    // (1) U = Ut - W h ;  dU = scale P^T dO + Kb dh'
-    tiles(kC, DV, [&](int i0, int j0) {
-        float a0[4][4] = {}, a1[4][4] = {}, a2[4][4] = {};
-        mac(a0, i0, j0, DK, [&](int i, int m) { return W[i * DK + m]; }, Hs);
-        mac(a1, i0, j0, DK, [&](int i, int m) { return expf(wsG[(kC - 1) * DK + m] - wsG[i * DK + m]) * Kf(i, m); },
-            DHs);
-        mac(a2, i0, j0, kC, [&](int i, int m) { return Pm[m * kC + i]; }, Of);
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-                const int t = (i0 + a) * DV + j0 + b;
-                U[t] = Ut[t] - a0[a][b];
-                dU[t] = sc * a2[a][b] + a1[a][b];
-            }
-    });
-    __syncthreads();
-    // (2) dP = scale tril(dO U^T) ;  dO h^T ;  dW = -dU h^T ;  U dh'^T
-    tiles(kC, kC, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        if (j0 <= i0 + 3) mac(acc, i0, j0, DV, Of, [&](int m, int j) { return U[j * DV + m]; });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) dP[i0 + a][j0 + b] = (j0 + b <= i0 + a) ? sc * acc[a][b] : 0.f;
-    });
-    tiles(kC, DK, [&](int i0, int j0) {
-        float a1[4][4] = {}, a2[4][4] = {}, a3[4][4] = {};
-        mac(a1, i0, j0, DV, Of, [&](int m, int j) { return Hs(j, m); });
-        mac(a2, i0, j0, DV, [&](int i, int m) { return dU[i * DV + m]; }, [&](int m, int j) { return Hs(j, m); });
-        mac(a3, i0, j0, DV, [&](int i, int m) { return U[i * DV + m]; }, [&](int m, int j) { return DHs(j, m); });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-                const int t = (i0 + a) * DK + j0 + b;
-                dOh[t] = a1[a][b];
-                dW[t] = -a2[a][b];
-                UdH[t] = a3[a][b];
-            }
-    });
-    __syncthreads();
-    // (3) dXk = T^T dW ;  dXv = T^T dU ;  dv = w . dXv ;  dw = v . dXv
-    tiles(kC, DK, [&](int i0, int j0) {
-        float ax[4][4] = {};
-        mac(ax, i0, j0, kC, [&](int i, int m) { return Tm[m * kC + i]; }, [&](int m, int j) { return dW[m * DK + j]; });
-        for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) dXk[(i0 + a) * DK + j0 + b] = ax[a][b];
-    });
-    tiles(kC, DV, [&](int i0, int j0) {
-        float ax[4][4] = {};
-        mac(ax, i0, j0, kC, [&](int i, int m) { return Tm[m * kC + i]; }, [&](int m, int j) { return dU[m * DV + j]; });
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-                const int i = i0 + a, j = j0 + b;
-                dXv[i * DV + j] = ax[a][b];
-                if (i < x.len) {
-                    stf(dvp + i * rv + j, Wf(i, j) * ax[a][b]);
-                    p.dwv[base_v + i * rv + j] = Vf(i, j) * ax[a][b];
-                }
-            }
-    });
-    __syncthreads();
-    // (4) dA = -stril(dXk W^T + dXv Ut^T)
-    tiles(kC, kC, [&](int i0, int j0) {
-        float acc[4][4] = {};
-        if (j0 < i0 + 3) {
-            mac(acc, i0, j0, DK, [&](int i, int m) { return dXk[i * DK + m]; }, [&](int m, int j) { return W[j * DK + m]; });
-            mac(acc, i0, j0, DV, [&](int i, int m) { return dXv[i * DV + m]; }, [&](int m, int j) { return Ut[j * DV + m]; });
-        }
-        for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) dA[i0 + a][j0 + b] = (j0 + b < i0 + a) ? -acc[a][b] : 0.f;
-    });
-    __syncthreads();
-    // (5) per (token i, channel r): the sums over the other token carry the decay of that channel
-    float* dgam = dW;   // dW is dead
-    for (int t = threadIdx.x; t < kC * DK; t += blockDim.x) {
-        const int i = t / DK, r = t % DK;
-        const float gi = G(i, r);
-        float sq = 0.f, srow = 0.f, scol = 0.f;
-        for (int j = 0; j <= i; ++j) {           // row role: e^{gam_i - gam_j}, j <= i
-            const float e = expf(gi - G(j, r)), kj = Kf(j, r);
-            sq = fmaf(dP[i][j] * e, kj, sq);
-            srow = fmaf(dA[i][j] * e, kj, srow);                       // (dA_ii = 0)
-        }
-        for (int j = i; j < kC; ++j) {           // column role: e^{gam_j - gam_i}, j >= i
-            const float e = expf(G(j, r) - gi);
-            scol = fmaf(dP[j][i] * e, Qf(j, r), scol);
-            scol = fmaf(dA[j][i] * e, Bf(j, r) * Kf(j, r), scol);      // (dA_ii = 0)
-        }
-        const float Gi = expf(gi), ei = expf(G(kC - 1, r) - gi);
-        const float ki = Kf(i, r), qi = Qf(i, r), bi = Bf(i, r);
-        const float dq = sc * Gi * dOh[t] + sq;
-        const float row = srow + Gi * dXk[t];
-        const float col = scol + ei * UdH[t];
-        if (i < x.len) {
-            stf(dqp + i * rk + r, dq);
-            stf(dkp + i * rk + r, bi * row + col);
-            p.dbv[base_k + i * rk + r] = ki * row;
-        }
-        dgam[t] = qi * dq + ki * bi * row - ki * col;
-    }
-    __syncthreads();
-    // the last row collects what enters through Gam_e: sum_j k_j . e_j . (U dh'^T)_j and Gam_e . rowdot(dh', h);
-    // then dg_j = sum_{i >= j} dgam_i, channel by channel
-    for (int r = threadIdx.x; r < DK; r += blockDim.x) {
-        float extra = 0.f, hh = 0.f;
-        const float ge = G(kC - 1, r);
-        for (int j = 0; j < kC; ++j) extra = fmaf(Kf(j, r) * expf(ge - G(j, r)), UdH[j * DK + r], extra);
-        for (int c = 0; c < DV; ++c) hh = fmaf(DHs(r, c), Hs(r, c), hh);
-        float run = extra + expf(ge) * hh;
-        for (int i = kC - 1; i >= 0; --i) {
-            run += dgam[i * DK + r];
-            if (i < x.len) p.dgv[base_k + i * rk + r] = run;
-        }
-    }
+template <int DK, int DV>
+cudaError_t launch_vscan(const Problem& p, int dirs, cudaStream_t st) {
+    static SmemLimitOnce once;
+    const cudaError_t e = once.ensure(vscan_kernel<DK, DV>, (uint32_t)scan_smem<DK>());
+    if (e != cudaSuccess) return e;
+    const int ctas = p.d.N * p.d.H * (dirs == 2 ? 2 : 1) * (DV / kScanCols);
+    { StageScope t(p.fallback ? ST_FALLBACK : dirs == 2 ? ST_SCANS : dirs == 1 ? ST_RSCAN : ST_FSCAN, st); vscan_kernel<DK, DV><<<ctas, kThreads, scan_smem<DK>(), st>>>(p, dirs); }
+    return cudaGetLastError();
+}
+template <typename IO, int DK, int DV>
+cudaError_t launch_vprep(const Problem& p, PrepMode mode, cudaStream_t st) {
+    static SmemLimitOnce once;
+    constexpr size_t sm = PrepTiles<DK, DV>::BYTES;
+    const cudaError_t e = once.ensure(vprep_kernel<IO, DK, DV>, (uint32_t)sm);
+    if (e != cudaSuccess) return e;
+    { StageScope t(p.fallback ? ST_FALLBACK : mode == PREP_BWD ? ST_EPREP : ST_PREP, st); vprep_kernel<IO, DK, DV><<<p.L.max_chunks * p.d.H, kThreads, sm, st>>>(p, mode); }
+    return cudaGetLastError();
 }
 
 // The FFMA sequences.  `q` is the problem as these kernels see it (fp32 factors and states); with q.fallback set the chunk
 // table is not rebuilt (the tensor-core route has built it, and rebuilding would reset the status word the launches look at).
 template <typename IO, int DK, int DV>
 cudaError_t ffma_fwd(const Problem& q, cudaStream_t st) {
-    const int CH = q.L.max_chunks * q.d.H, chains = q.d.N * q.d.H;
-    if (!q.fallback) launch_table(q, st);
-    const size_t smp = sizeof(float) * (kC * (DK + 1) + 2 * kC * (kC + 1));
-    cudaError_t e = cudaFuncSetAttribute(vprep_kernel<IO, DK, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smp);
-    if (e != cudaSuccess) return e;
-    if (CH > 0) { StageScope t(q.fallback ? ST_FALLBACK : ST_PREP, st); vprep_kernel<IO, DK, DV><<<CH, kThreads, smp, st>>>(q); }
-    const size_t sm = sizeof(float) * (2 * DK * DV + kC * DV);
-    e = cudaFuncSetAttribute(vscan_kernel<IO, DK, DV, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    if (chains > 0) { StageScope t(q.fallback ? ST_FALLBACK : ST_FSCAN, st); vscan_kernel<IO, DK, DV, false><<<chains, kThreads, sm, st>>>(q); }
-    if (q.o && CH > 0) { StageScope t(q.fallback ? ST_FALLBACK : ST_OUT, st); vout_kernel<IO, DK, DV><<<CH, kThreads, 0, st>>>(q); }
+    cudaError_t e;
+    if (q.cu && !q.fallback && (e = launch_table(q, st)) != cudaSuccess) return e;
+    if ((e = launch_vprep<IO, DK, DV>(q, PREP_FWD, st)) != cudaSuccess) return e;
+    if ((e = launch_vscan<DK, DV>(q, 0, st)) != cudaSuccess || !q.o) return e;
+    static SmemLimitOnce once;
+    if ((e = once.ensure(vout_kernel<IO, DK, DV>, (uint32_t)vout_smem<DK, DV>())) != cudaSuccess) return e;
+    { StageScope t(q.fallback ? ST_FALLBACK : ST_OUT, st); vout_kernel<IO, DK, DV><<<q.L.max_chunks * q.d.H, kThreads, vout_smem<DK, DV>(), st>>>(q); }
     return cudaGetLastError();
 }
 
 template <typename IO, int DK, int DV>
 cudaError_t ffma_bwd(const Problem& q, bool skip_recompute, cudaStream_t st) {
     cudaError_t e;
-    if (!skip_recompute && (e = ffma_fwd<IO, DK, DV>(q, st)) != cudaSuccess) return e;
-    const int CH = q.L.max_chunks * q.d.H, chains = q.d.N * q.d.H;
-    if (CH > 0) { StageScope t(q.fallback ? ST_FALLBACK : ST_EPREP, st); veprep_kernel<IO, DK, DV><<<CH, kThreads, 0, st>>>(q); }
-    const size_t sm = sizeof(float) * (2 * DK * DV + kC * DV);
-    e = cudaFuncSetAttribute(vscan_kernel<IO, DK, DV, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    if (chains > 0) { StageScope t(q.fallback ? ST_FALLBACK : ST_RSCAN, st); vscan_kernel<IO, DK, DV, true><<<chains, kThreads, sm, st>>>(q); }
-    const size_t smi = sizeof(float) * (kC * (DK + 1) + 2 * kC * (kC + 1));
-    e = cudaFuncSetAttribute(vintra_kernel<IO, DK, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smi);
-    if (e != cudaSuccess) return e;
-    if (CH > 0) { StageScope t(q.fallback ? ST_FALLBACK : ST_INTRA, st); vintra_kernel<IO, DK, DV><<<CH, kThreads, smi, st>>>(q); }
+    if (q.cu && !q.fallback && !skip_recompute && (e = launch_table(q, st)) != cudaSuccess) return e;
+    if ((e = launch_vprep<IO, DK, DV>(q, skip_recompute ? PREP_BWD : PREP_FWD_BWD, st)) != cudaSuccess) return e;
+    if ((e = launch_vscan<DK, DV>(q, skip_recompute ? 1 : 2, st)) != cudaSuccess) return e;
+    static SmemLimitOnce once;
+    constexpr size_t sm = IntraTiles<DK, DV>::BYTES;
+    if ((e = once.ensure(vintra_kernel<IO, DK, DV>, (uint32_t)sm)) != cudaSuccess) return e;
+    { StageScope t(q.fallback ? ST_FALLBACK : ST_INTRA, st); vintra_kernel<IO, DK, DV><<<q.L.max_chunks * q.d.H, kThreads, sm, st>>>(q); }
     return cudaGetLastError();
 }
 
@@ -507,8 +686,6 @@ cudaError_t vlaunch_bwd_t(const Problem& p, bool skip_recompute, cudaStream_t st
 }
 
 }  // namespace
-
-size_t vec_scratch_per_chunkhead(const gdn_desc& d) { return sizeof(float) * kC * (4 * (size_t)d.d_k + 3 * (size_t)d.d_v); }
 
 #define GDN_VDISPATCH(FN, ...)                                                                      \
     do {                                                                                            \

@@ -8,8 +8,10 @@ whole tensors, three times that for one 64-token block."""
 import numpy as np
 import pytest
 
+import oracle
+
 from paper_2608_12700_b200 import runner, synth
-from helpers import check_against_oracle, oracle_grads, rel
+from helpers import block_errors, check_against_oracle, oracle_grads, rel
 
 pytestmark = pytest.mark.gpu
 
@@ -31,4 +33,31 @@ def test_tile_edges(dk, dv, lengths, delta_rule):
     runner.run_bwd(buf, fresh=1)
     fresh = runner.fetch(buf)
     for n in ("dq", "dk", "dv", "dg", "dh0"):
+        assert np.array_equal(fresh[n], got[n]), n
+
+
+@pytest.mark.parametrize("dk,dv", [(64, 64), (128, 128), (128, 64), (64, 128)])
+@pytest.mark.parametrize("lengths,decay", [([1, 15, 16, 17, 31], 0.1), ([32, 33, 47, 48, 49, 63, 64, 65], 0.1), ([127, 0, 193], 0.1),
+                                           ([100, 64, 17], 4.0)])
+def test_channelwise_tile_edges(dk, dv, lengths, decay):
+    """Per-channel gates: lengths around the 16-token blocks in which the decay is split, and a decay (about -3.2 per token)
+    whose factor underflows inside a chunk.  There the decay gradient is what is left of sums e^3.2 = 25 times its size:
+    25 times the tolerance, for it alone."""
+    wl = synth.make_channelwise("cw_tiles", member="gdn", dtype="f32", lengths=lengths, H=2, d_k=dk, d_v=dv, seed=311, states=True,
+                                scale=0.7, g_scale=decay)
+    ref = oracle.vec_bwd_workload(wl)
+    buf = runner.to_device_channelwise(wl, want_o=True)
+    runner.run_bwd_channelwise(buf)
+    got = runner.fetch(buf)
+    for n in ("dq", "dk", "dv", "dg", "db", "dw", "dh0"):
+        tol = 3e-6 * (25 if decay > 1 and n == "dg" else 1)
+        assert rel(got[n], ref[n]) < tol, (n, rel(got[n], ref[n]))
+        e, _ = block_errors(wl, n, got[n], ref[n])
+        assert e.max() < 3 * tol, (n, e.max())
+    runner.run_fwd_channelwise(buf)
+    f = runner.fetch(buf)
+    assert rel(f["o"], ref["o"]) < 3e-6 and rel(f["hT"], ref["hT"]) < 3e-6
+    runner.run_bwd_channelwise(buf, fresh=1)
+    fresh = runner.fetch(buf)
+    for n in ("dq", "dk", "dv", "dg", "db", "dw", "dh0"):
         assert np.array_equal(fresh[n], got[n]), n
