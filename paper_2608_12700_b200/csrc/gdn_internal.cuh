@@ -5,6 +5,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "gdn.h"
 
 namespace gdn {
@@ -196,6 +198,29 @@ struct SmemLimitOnce {
         return e;
     }
 };
+
+// Programmatic dependent launch.  Every launch allows its kernel to be set up while the one before it in the stream runs, and
+// every kernel of the library begins with wait_prerequisites(), which returns when that one is complete and its writes are
+// visible: what a launch costs between two dependent kernels shrinks by about two microseconds.  (A training step of 4 heads
+// of 333 tokens, six launches: 63.5 -> 51.8 us; a backward of 4 x 16 heads of 2048 tokens, three: 307 -> 301 us.)  All threads
+// of all blocks wait, those without work too: a grid that ended without waiting would let the kernel after it run beside the
+// one before it.  No kernel triggers its dependents early (griddepcontrol.launch_dependents): their blocks then take up
+// room while others still work; the same two calls took 54.4 and 326 us that way.
+__device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... Params, class... Args>
+cudaError_t launch_kernel(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
 
 gdn_status check_desc(const gdn_desc* d);                       // shape / dtype envelope
 gdn_status check_seq(const gdn_desc& d, const int32_t* cu);     // B, N against cu_seqlens

@@ -9,7 +9,8 @@ namespace gdn {
 namespace {
 
 // rows of 64 bf16 -> rows of 128 bf16 (upper half zero), 16 bytes per thread and step
-__global__ void widen_rows_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, size_t rows) {
+__global__ void widen_rows_kernel(const uint4* src, uint4* dst, size_t rows) {
+    wait_prerequisites();
     for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < rows * 16; t += (size_t)gridDim.x * blockDim.x) {
         const size_t r = t >> 4;
         const int c = (int)(t & 15);
@@ -17,19 +18,22 @@ __global__ void widen_rows_kernel(const uint4* __restrict__ src, uint4* __restri
     }
 }
 // rows of 128 bf16 -> their first 64
-__global__ void narrow_rows_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, size_t rows) {
+__global__ void narrow_rows_kernel(const uint4* src, uint4* dst, size_t rows) {
+    wait_prerequisites();
     for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < rows * 8; t += (size_t)gridDim.x * blockDim.x)
         dst[t] = src[(t >> 3) * 16 + (t & 7)];
 }
 // fp32 states [n, dk, dv] <-> [n, 128, 128]
-__global__ void widen_state_kernel(const float* __restrict__ src, float* __restrict__ dst, size_t n, int dk, int dv) {
+__global__ void widen_state_kernel(const float* src, float* dst, size_t n, int dk, int dv) {
+    wait_prerequisites();
     for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * 128 * 128; t += (size_t)gridDim.x * blockDim.x) {
         const size_t s = t >> 14;
         const int r = (int)((t >> 7) & 127), c = (int)(t & 127);
         dst[t] = (r < dk && c < dv) ? src[(s * dk + r) * dv + c] : 0.f;
     }
 }
-__global__ void narrow_state_kernel(const float* __restrict__ src, float* __restrict__ dst, size_t n, int dk, int dv) {
+__global__ void narrow_state_kernel(const float* src, float* dst, size_t n, int dk, int dv) {
+    wait_prerequisites();
     for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * dk * dv; t += (size_t)gridDim.x * blockDim.x) {
         const size_t s = t / ((size_t)dk * dv);
         const int r = (int)((t / dv) % dk), c = (int)(t % dv);
@@ -38,14 +42,16 @@ __global__ void narrow_state_kernel(const float* __restrict__ src, float* __rest
 }
 
 // gate vectors: rows of 64 fp32 <-> rows of 128 fp32 (upper half zero: log decay 0, erase gate 0, write gate 0)
-__global__ void widen_rows_f32_kernel(const float4* __restrict__ src, float4* __restrict__ dst, size_t rows) {
+__global__ void widen_rows_f32_kernel(const float4* src, float4* dst, size_t rows) {
+    wait_prerequisites();
     for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < rows * 32; t += (size_t)gridDim.x * blockDim.x) {
         const size_t r = t >> 5;
         const int c = (int)(t & 31);
         dst[t] = c < 16 ? src[r * 16 + c] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
-__global__ void narrow_rows_f32_kernel(const float4* __restrict__ src, float4* __restrict__ dst, size_t rows) {
+__global__ void narrow_rows_f32_kernel(const float4* src, float4* dst, size_t rows) {
+    wait_prerequisites();
     for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < rows * 16; t += (size_t)gridDim.x * blockDim.x)
         dst[t] = src[(t >> 4) * 32 + (t & 15)];
 }
@@ -103,19 +109,19 @@ cudaError_t tc_padded_launch(const Problem& p, const WsLayout& inner, bool bwd, 
     auto widen = [&](const void* src, size_t off) -> const void* {
         if (!src || rows == 0) return src;
         StageScope t(ST_TABLE, st);
-        widen_rows_kernel<<<grid_for(rows * 16), 256, 0, st>>>(static_cast<const uint4*>(src), reinterpret_cast<uint4*>(pad + off), rows);
+        launch_kernel(widen_rows_kernel, grid_for(rows * 16), 256, 0, st, static_cast<const uint4*>(src), reinterpret_cast<uint4*>(pad + off), rows);
         return pad + off;
     };
     auto widen_state = [&](const float* src, size_t off) -> const float* {
         if (!src) return nullptr;
         StageScope t(ST_TABLE, st);
-        widen_state_kernel<<<grid_for(chains * 16384), 256, 0, st>>>(src, reinterpret_cast<float*>(pad + off), chains, d.d_k, d.d_v);
+        launch_kernel(widen_state_kernel, grid_for(chains * 16384), 256, 0, st, src, reinterpret_cast<float*>(pad + off), chains, d.d_k, d.d_v);
         return reinterpret_cast<const float*>(pad + off);
     };
     auto widen_gate = [&](const float* src, size_t off) -> const float* {
         if (!src || rows == 0) return src;
         StageScope t(ST_TABLE, st);
-        widen_rows_f32_kernel<<<grid_for(rows * 32), 256, 0, st>>>(reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(pad + off), rows);
+        launch_kernel(widen_rows_f32_kernel, grid_for(rows * 32), 256, 0, st, reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(pad + off), rows);
         return reinterpret_cast<const float*>(pad + off);
     };
     const bool fresh = bwd && skip_recompute;   // the widened forward inputs are still in the workspace
@@ -151,17 +157,17 @@ cudaError_t tc_padded_launch(const Problem& p, const WsLayout& inner, bool bwd, 
     auto narrow = [&](const void* src, void* dst) {
         if (!dst || rows == 0) return;
         StageScope t(ST_TABLE, st);
-        narrow_rows_kernel<<<grid_for(rows * 8), 256, 0, st>>>(static_cast<const uint4*>(src), static_cast<uint4*>(dst), rows);
+        launch_kernel(narrow_rows_kernel, grid_for(rows * 8), 256, 0, st, static_cast<const uint4*>(src), static_cast<uint4*>(dst), rows);
     };
     auto narrow_state = [&](const float* src, float* dst) {
         if (!dst) return;
         StageScope t(ST_TABLE, st);
-        narrow_state_kernel<<<grid_for(chains * d.d_k * d.d_v), 256, 0, st>>>(src, dst, chains, d.d_k, d.d_v);
+        launch_kernel(narrow_state_kernel, grid_for(chains * d.d_k * d.d_v), 256, 0, st, src, dst, chains, d.d_k, d.d_v);
     };
     auto narrow_gate = [&](const float* src, float* dst) {
         if (!dst || rows == 0) return;
         StageScope t(ST_TABLE, st);
-        narrow_rows_f32_kernel<<<grid_for(rows * 16), 256, 0, st>>>(reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(dst), rows);
+        launch_kernel(narrow_rows_f32_kernel, grid_for(rows * 16), 256, 0, st, reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(dst), rows);
     };
     if (bwd) {
         if (d.d_k == 64) { narrow(w.dq, p.dq); narrow(w.dk, p.dk); }

@@ -27,6 +27,7 @@ using namespace ffma;
 // Chunk table.  One block.  Validates cu_seqlens; on failure records the status and leaves no work.
 // ------------------------------------------------------------------------------------------------
 __global__ void table_kernel(Problem p) {
+    wait_prerequisites();
     WsHeader* hdr = reinterpret_cast<WsHeader*>(p.ws);
     int32_t* seq_first = reinterpret_cast<int32_t*>(p.ws + p.L.seq_first);
     int32_t* chunk_seq = reinterpret_cast<int32_t*>(p.ws + p.L.chunk_seq);
@@ -134,6 +135,7 @@ constexpr size_t prep_smem() {
 
 template <typename IO, int DK, int DV>
 __global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) {
+    wait_prerequisites();
     const bool fwd = mode != PREP_BWD, bwd = mode != PREP_FWD;
     init_header_if_untabled(p);
     ChunkInfo x;
@@ -281,6 +283,7 @@ __global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) 
 // ------------------------------------------------------------------------------------------------
 template <int DK, int DV>
 __global__ void __launch_bounds__(kThreads) scan_kernel(Problem p, int dirs) {
+    wait_prerequisites();
     extern __shared__ __align__(16) float sm[];
     if (reinterpret_cast<const WsHeader*>(p.ws)->status != GDN_OK) return;
     scan_block<DK, DV, false>(p, dirs, sm);
@@ -294,6 +297,7 @@ constexpr size_t out_smem() { return sizeof(float) * (kC * pitch(DK) + DK * pitc
 
 template <typename IO, int DK, int DV>
 __global__ void __launch_bounds__(kThreads, 1) out_kernel(Problem p) {
+    wait_prerequisites();
     ChunkInfo x;
     if (!chunk_head(p, x)) return;
     constexpr int PK = pitch(DK), PV = pitch(DV);
@@ -356,6 +360,7 @@ constexpr size_t intra_smem() {
 
 template <typename IO, int DK, int DV>
 __global__ void __launch_bounds__(kThreads, DK + DV == 128 ? 2 : 1) intra_kernel(Problem p) {
+    wait_prerequisites();
     ChunkInfo x;
     if (!chunk_head(p, x)) return;
     constexpr int PK = pitch(DK), PV = pitch(DV), PM = pitch(DK > DV ? DK : DV), NH = DK / 64;
@@ -564,7 +569,7 @@ cudaError_t launch_scan_t(const Problem& p, int dirs, cudaStream_t st) {
     const cudaError_t e = once.ensure(scan_kernel<DK, DV>, (uint32_t)scan_smem<DK>());
     if (e != cudaSuccess) return e;
     const int ctas = p.d.N * p.d.H * (dirs == 2 ? 2 : 1) * (DV / kScanCols);
-    { StageScope t(dirs == 2 ? ST_SCANS : dirs == 1 ? ST_RSCAN : ST_FSCAN, st); scan_kernel<DK, DV><<<ctas, kThreads, scan_smem<DK>(), st>>>(p, dirs); }
+    { StageScope t(dirs == 2 ? ST_SCANS : dirs == 1 ? ST_RSCAN : ST_FSCAN, st); launch_kernel(scan_kernel<DK, DV>, ctas, kThreads, scan_smem<DK>(), st, p, dirs); }
     return cudaGetLastError();
 }
 
@@ -573,7 +578,7 @@ cudaError_t launch_prep_t(const Problem& p, PrepMode mode, cudaStream_t st) {
     static SmemLimitOnce once;
     const cudaError_t e = once.ensure(prep_kernel<IO, DK, DV>, (uint32_t)prep_smem<DK, DV>());
     if (e != cudaSuccess) return e;
-    { StageScope t(mode == PREP_BWD ? ST_EPREP : ST_PREP, st); prep_kernel<IO, DK, DV><<<p.L.max_chunks * p.d.H, kThreads, prep_smem<DK, DV>(), st>>>(p, mode); }
+    { StageScope t(mode == PREP_BWD ? ST_EPREP : ST_PREP, st); launch_kernel(prep_kernel<IO, DK, DV>, p.L.max_chunks * p.d.H, kThreads, prep_smem<DK, DV>(), st, p, mode); }
     return cudaGetLastError();
 }
 
@@ -585,7 +590,7 @@ cudaError_t launch_fwd_t(const Problem& p, cudaStream_t st) {
     if ((e = launch_scan_t<DK, DV>(p, 0, st)) != cudaSuccess || !p.o) return e;
     static SmemLimitOnce once;
     if ((e = once.ensure(out_kernel<IO, DK, DV>, (uint32_t)out_smem<DK, DV>())) != cudaSuccess) return e;
-    { StageScope t(ST_OUT, st); out_kernel<IO, DK, DV><<<p.L.max_chunks * p.d.H, kThreads, out_smem<DK, DV>(), st>>>(p); }
+    { StageScope t(ST_OUT, st); launch_kernel(out_kernel<IO, DK, DV>, p.L.max_chunks * p.d.H, kThreads, out_smem<DK, DV>(), st, p); }
     return cudaGetLastError();
 }
 
@@ -597,7 +602,7 @@ cudaError_t launch_bwd_t(const Problem& p, bool skip_recompute, cudaStream_t st)
     if ((e = launch_scan_t<DK, DV>(p, skip_recompute ? 1 : 2, st)) != cudaSuccess) return e;
     static SmemLimitOnce once;
     if ((e = once.ensure(intra_kernel<IO, DK, DV>, (uint32_t)intra_smem<DK, DV>())) != cudaSuccess) return e;
-    { StageScope t(ST_INTRA, st); intra_kernel<IO, DK, DV><<<p.L.max_chunks * p.d.H, kThreads, intra_smem<DK, DV>(), st>>>(p); }
+    { StageScope t(ST_INTRA, st); launch_kernel(intra_kernel<IO, DK, DV>, p.L.max_chunks * p.d.H, kThreads, intra_smem<DK, DV>(), st, p); }
     return cudaGetLastError();
 }
 
@@ -605,7 +610,7 @@ cudaError_t launch_bwd_t(const Problem& p, bool skip_recompute, cudaStream_t st)
 
 cudaError_t launch_table(const Problem& p, cudaStream_t st) {
     StageScope t(ST_TABLE, st);
-    table_kernel<<<1, 256, 0, st>>>(p);
+    launch_kernel(table_kernel, 1, 256, 0, st, p);
     return cudaGetLastError();
 }
 

@@ -38,6 +38,7 @@ __device__ __forceinline__ bool vec_go(const Problem& p) {
     return p.fallback ? st == GDN_ERR_DECAY_RANGE : st == GDN_OK;
 }
 __global__ void vec_clear_refusal_kernel(Problem p) {
+    wait_prerequisites();
     WsHeader* hdr = reinterpret_cast<WsHeader*>(p.ws);
     const bool refused = hdr->status == GDN_ERR_DECAY_RANGE;
     hdr->cw_fallback = refused ? 1 : 0;   // a backward on this workspace "fresh from the forward" must know whose data it holds
@@ -96,6 +97,7 @@ struct PrepTiles {
 
 template <typename IO, int DK, int DV>
 __global__ void __launch_bounds__(kThreads, 1) vprep_kernel(Problem p, int mode) {
+    wait_prerequisites();
     if (!p.fallback) init_header_if_untabled(p);
     ChunkInfo x;
     if ((p.fallback && !vec_go(p)) || !chunk_info(p, x)) return;
@@ -297,6 +299,7 @@ __global__ void __launch_bounds__(kThreads, 1) vprep_kernel(Problem p, int mode)
 // ------------------------------------------------------------------------------------------------
 template <int DK, int DV>
 __global__ void __launch_bounds__(kThreads) vscan_kernel(Problem p, int dirs) {
+    wait_prerequisites();
     extern __shared__ __align__(16) float sm[];
     if (!vec_go(p)) return;
     scan_block<DK, DV, true>(p, dirs, sm);
@@ -310,6 +313,7 @@ constexpr size_t vout_smem() { return sizeof(float) * (kC * pitch(DK) + DK * pit
 
 template <typename IO, int DK, int DV>
 __global__ void __launch_bounds__(kThreads, 1) vout_kernel(Problem p) {
+    wait_prerequisites();
     ChunkInfo x;
     if (!vec_go(p) || !chunk_info(p, x)) return;
     constexpr int PK = pitch(DK), PV = pitch(DV), R = Out<DV>::R;
@@ -377,6 +381,7 @@ struct IntraTiles {
 
 template <typename IO, int DK, int DV>
 __global__ void __launch_bounds__(kThreads, 1) vintra_kernel(Problem p) {
+    wait_prerequisites();
     ChunkInfo x;
     if (!vec_go(p) || !chunk_info(p, x)) return;
     using L = IntraTiles<DK, DV>;
@@ -613,7 +618,7 @@ cudaError_t launch_vscan(const Problem& p, int dirs, cudaStream_t st) {
     const cudaError_t e = once.ensure(vscan_kernel<DK, DV>, (uint32_t)scan_smem<DK>());
     if (e != cudaSuccess) return e;
     const int ctas = p.d.N * p.d.H * (dirs == 2 ? 2 : 1) * (DV / kScanCols);
-    { StageScope t(p.fallback ? ST_FALLBACK : dirs == 2 ? ST_SCANS : dirs == 1 ? ST_RSCAN : ST_FSCAN, st); vscan_kernel<DK, DV><<<ctas, kThreads, scan_smem<DK>(), st>>>(p, dirs); }
+    { StageScope t(p.fallback ? ST_FALLBACK : dirs == 2 ? ST_SCANS : dirs == 1 ? ST_RSCAN : ST_FSCAN, st); launch_kernel(vscan_kernel<DK, DV>, ctas, kThreads, scan_smem<DK>(), st, p, dirs); }
     return cudaGetLastError();
 }
 template <typename IO, int DK, int DV>
@@ -622,7 +627,7 @@ cudaError_t launch_vprep(const Problem& p, PrepMode mode, cudaStream_t st) {
     constexpr size_t sm = PrepTiles<DK, DV>::BYTES;
     const cudaError_t e = once.ensure(vprep_kernel<IO, DK, DV>, (uint32_t)sm);
     if (e != cudaSuccess) return e;
-    { StageScope t(p.fallback ? ST_FALLBACK : mode == PREP_BWD ? ST_EPREP : ST_PREP, st); vprep_kernel<IO, DK, DV><<<p.L.max_chunks * p.d.H, kThreads, sm, st>>>(p, mode); }
+    { StageScope t(p.fallback ? ST_FALLBACK : mode == PREP_BWD ? ST_EPREP : ST_PREP, st); launch_kernel(vprep_kernel<IO, DK, DV>, p.L.max_chunks * p.d.H, kThreads, sm, st, p, mode); }
     return cudaGetLastError();
 }
 
@@ -636,7 +641,7 @@ cudaError_t ffma_fwd(const Problem& q, cudaStream_t st) {
     if ((e = launch_vscan<DK, DV>(q, 0, st)) != cudaSuccess || !q.o) return e;
     static SmemLimitOnce once;
     if ((e = once.ensure(vout_kernel<IO, DK, DV>, (uint32_t)vout_smem<DK, DV>())) != cudaSuccess) return e;
-    { StageScope t(q.fallback ? ST_FALLBACK : ST_OUT, st); vout_kernel<IO, DK, DV><<<q.L.max_chunks * q.d.H, kThreads, vout_smem<DK, DV>(), st>>>(q); }
+    { StageScope t(q.fallback ? ST_FALLBACK : ST_OUT, st); launch_kernel(vout_kernel<IO, DK, DV>, q.L.max_chunks * q.d.H, kThreads, vout_smem<DK, DV>(), st, q); }
     return cudaGetLastError();
 }
 
@@ -649,7 +654,7 @@ cudaError_t ffma_bwd(const Problem& q, bool skip_recompute, cudaStream_t st) {
     static SmemLimitOnce once;
     constexpr size_t sm = IntraTiles<DK, DV>::BYTES;
     if ((e = once.ensure(vintra_kernel<IO, DK, DV>, (uint32_t)sm)) != cudaSuccess) return e;
-    { StageScope t(q.fallback ? ST_FALLBACK : ST_INTRA, st); vintra_kernel<IO, DK, DV><<<q.L.max_chunks * q.d.H, kThreads, sm, st>>>(q); }
+    { StageScope t(q.fallback ? ST_FALLBACK : ST_INTRA, st); launch_kernel(vintra_kernel<IO, DK, DV>, q.L.max_chunks * q.d.H, kThreads, sm, st, q); }
     return cudaGetLastError();
 }
 
@@ -664,7 +669,7 @@ cudaError_t ffma_fallback(const Problem& p, bool bwd, bool skip_recompute, cudaS
     q.L.tc_scans = 0;
     cudaError_t e = bwd ? ffma_bwd<IO, DK, DV>(q, skip_recompute, st) : ffma_fwd<IO, DK, DV>(q, st);
     if (e != cudaSuccess) return e;
-    { StageScope t(ST_FALLBACK, st); vec_clear_refusal_kernel<<<1, 1, 0, st>>>(q); }
+    { StageScope t(ST_FALLBACK, st); launch_kernel(vec_clear_refusal_kernel, 1, 1, 0, st, q); }
     return cudaGetLastError();
 }
 

@@ -77,6 +77,7 @@ constexpr uint32_t C_E_LR = 256;   // low-rank mode (no Nm, Bf): E is started ea
 }  // namespace prep
 
 __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __grid_constant__ TcParams P) {
+    wait_prerequisites();
     using namespace prep;
     const Problem& p = P.p;
     // Persistent: a CTA walks over chunk-heads blockIdx.x, blockIdx.x + gridDim.x, ...; the inputs of its next one
@@ -539,6 +540,7 @@ template <int S> struct Cfg {
 
 template <int S>
 __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_constant__ TcParams P) {
+    wait_prerequisites();
     using namespace scan;
     using C = Cfg<S>;
     constexpr int NS = C::NS, NSH = NS / 2, STAGES = C::STAGES, PREFETCH_AHEAD = C::PREFETCH_AHEAD;
@@ -915,6 +917,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
 // (S = 1 only); with S = 2 (one direction per launch) the low bit is the column block.
 template <int S>
 __global__ void __launch_bounds__(kThreads, 1) tc_scan_lr_kernel(const __grid_constant__ TcParams P) {
+    wait_prerequisites();
     using namespace scanlr;
     __shared__ float ge[GE_CAP];
     __shared__ __align__(16) float ee2[2][kC];   // e_j of a step, made during the step before it
@@ -932,6 +935,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_lr_kernel(const __grid_co
 // The carries of the channel-wise path (per-channel gates, d_k = d_v = 128, bf16 I/O) on the same machinery.
 template <int S>
 __global__ void __launch_bounds__(kThreads, 1) tc_scan_cw_kernel(const __grid_constant__ TcParams P) {
+    wait_prerequisites();
     using namespace scanlr;
     __shared__ __align__(16) float ee2[2][kC];   // (unused: the key tile arrives scaled)
     __shared__ uint64_t bar_full[Cfg<S>::STAGES], bar_mma;
@@ -991,6 +995,7 @@ __host__ __device__ constexpr uint32_t slot(int k) { return 64u * k; }   // eigh
 }  // namespace intra
 
 __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_intra_kernel(const __grid_constant__ TcParams P) {
+    wait_prerequisites();
     using namespace intra;
     const Problem& p = P.p;
     // Persistent: a CTA walks over chunk-heads blockIdx.x, blockIdx.x + gridDim.x, ...  While it works on one, the
@@ -1541,6 +1546,7 @@ static_assert(2 * (SMEM_BYTES + 4096) <= 228 * 1024, "two CTAs per SM");
 
 template <bool CW>
 __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_constant__ TcParams P) {
+    wait_prerequisites();
     using namespace outk;
     const Problem& p = P.p;
     const int H = p.d.H;
@@ -1756,7 +1762,7 @@ static cudaError_t launch_chunk_kernel(Kernel kernel, SmemLimitOnce& once, uint3
     if (e != cudaSuccess) return e;
     if (grid > 0) {
         StageScope t(stage, st);
-        kernel<<<grid, threads, smem, st>>>(P);
+        launch_kernel(kernel, grid, threads, smem, st, P);
     }
     return cudaGetLastError();
 }

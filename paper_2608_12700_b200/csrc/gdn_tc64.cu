@@ -32,6 +32,7 @@ struct Tc64Params {
 // read token by token (128 contiguous bytes each), then each warp scans the tokens of four heads (lane l owns
 // tokens l and l + 32).  First kernel of a call.
 __global__ void __launch_bounds__(256) tc64_gamma_kernel(Problem p) {
+    wait_prerequisites();
     init_header_if_untabled(p);
     __shared__ float gs[kC][33];
     const int c = blockIdx.x, h0 = blockIdx.y * 32, H = p.d.H;
@@ -74,6 +75,7 @@ constexpr uint32_t SMEM_BYTES = PT + 8192 + 1024;
 }  // namespace f64
 
 __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_constant__ Tc64Params P) {
+    wait_prerequisites();
     using namespace f64;
     const Problem& p = P.p;
     const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
@@ -266,6 +268,7 @@ constexpr uint32_t C0 = 0, C1 = 64, C2 = 128, C3 = 192, LB = 16u << 16;
 }  // namespace b64
 
 __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __grid_constant__ Tc64Params P) {
+    wait_prerequisites();
     using namespace b64;
     const Problem& p = P.p;
     const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
@@ -567,7 +570,7 @@ static cudaError_t tc64_prologue(const Problem& p, cudaStream_t st) {
     }
     if (p.L.max_chunks > 0 && p.Ttot > 0) {
         StageScope t(ST_PREP, st);
-        tc64_gamma_kernel<<<dim3(p.L.max_chunks, (p.d.H + 31) / 32), 256, 0, st>>>(p);
+        launch_kernel(tc64_gamma_kernel, dim3(p.L.max_chunks, (p.d.H + 31) / 32), 256, 0, st, p);
     }
     return cudaGetLastError();
 }
@@ -579,7 +582,7 @@ static cudaError_t tc64_fwd_pass(const Tc64Params& P, cudaStream_t st) {
     const int chains = P.p.d.N * P.p.d.H;
     if (chains > 0) {
         StageScope t(ST_FSCAN, st);
-        tc64_fwd_kernel<<<chains, kThreads64, f64::SMEM_BYTES, st>>>(P);
+        launch_kernel(tc64_fwd_kernel, chains, kThreads64, f64::SMEM_BYTES, st, P);
     }
     return cudaGetLastError();
 }
@@ -618,7 +621,7 @@ cudaError_t tc64_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t 
     const int chains = p.d.N * p.d.H;
     if (chains > 0) {
         StageScope t(ST_RSCAN, st);
-        tc64_bwd_kernel<<<chains, kThreads64 + 32, b64::SMEM_BYTES, st>>>(P);
+        launch_kernel(tc64_bwd_kernel, chains, kThreads64 + 32, b64::SMEM_BYTES, st, P);
     }
     return cudaGetLastError();
 }

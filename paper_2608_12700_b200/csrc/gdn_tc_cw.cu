@@ -60,6 +60,7 @@ constexpr size_t S_DQ = 0, S_DKP = 32768, S_DKM = 65536, S_DXV = 98304, S_HH = 1
 // fall-back kernels (its gates were refused; the header remembers), the workspace holds their fp32 data instead: the
 // refusal is raised again and the fall-back sequence computes this call too.
 __global__ void __launch_bounds__(kT) cw_scale_kernel(Problem p, int mode) {
+    wait_prerequisites();
     ChunkCtx x;
     if (!chunk_ctx(p, x)) return;
     extern __shared__ __align__(16) float gam[];   // [64][D + 1]
@@ -192,6 +193,7 @@ static_assert(TT % 1024 == 0 && SMEM_BYTES <= 225 * 1024, "tile alignment and sh
 // mode 0: the forward's share (P, A, T, W, U~); 1: that and E (closed backward); 2: E alone from the stored P and W^T
 // (backward on a workspace fresh from the forward: no product, inversion or store of the forward is repeated).
 __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
+    wait_prerequisites();
     using namespace prepcw;
     const int H = p.d.H;
     const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
@@ -454,6 +456,7 @@ static_assert(SMEM_BYTES <= 220 * 1024, "shared memory budget");
 }  // namespace intracw
 
 __global__ void __launch_bounds__(kT, 1) cw_intra_kernel(Problem p) {
+    wait_prerequisites();
     using namespace intracw;
     const int H = p.d.H;
     const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
@@ -721,6 +724,7 @@ __global__ void __launch_bounds__(kT, 1) cw_intra_kernel(Problem p) {
 // cw_post
 // ------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kT) cw_post_kernel(Problem p) {
+    wait_prerequisites();
     ChunkCtx x;
     if (!chunk_ctx(p, x)) return;
     if (reinterpret_cast<const WsHeader*>(p.ws)->status != GDN_OK) return;
@@ -815,8 +819,8 @@ cudaError_t cw_tc_launch(const Problem& p, bool bwd, bool skip_recompute, cudaSt
         if ((e = once_scale.ensure(cw_scale_kernel, sm_scale)) != cudaSuccess) return e;
         if ((e = once_prep.ensure(cw_prep_kernel, prepcw::SMEM_BYTES)) != cudaSuccess) return e;
         const int mode = bwd ? (skip_recompute ? 2 : 1) : 0;
-        { StageScope t(ST_SCALE, st); cw_scale_kernel<<<CH, kT, sm_scale, st>>>(p, mode); }
-        { StageScope t(ST_PREP, st); cw_prep_kernel<<<grid, kT, prepcw::SMEM_BYTES, st>>>(p, mode); }
+        { StageScope t(ST_SCALE, st); launch_kernel(cw_scale_kernel, CH, kT, sm_scale, st, p, mode); }
+        { StageScope t(ST_PREP, st); launch_kernel(cw_prep_kernel, grid, kT, prepcw::SMEM_BYTES, st, p, mode); }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (chains > 0 && (e = tc_launch_scan_channelwise(p, bwd ? (skip_recompute ? 1 : 2) : 0, st)) != cudaSuccess) return e;
@@ -827,8 +831,8 @@ cudaError_t cw_tc_launch(const Problem& p, bool bwd, bool skip_recompute, cudaSt
         const uint32_t sm_post = sizeof(float) * kC * D;
         if ((e = once_intra.ensure(cw_intra_kernel, intracw::SMEM_BYTES)) != cudaSuccess) return e;
         if ((e = once_post.ensure(cw_post_kernel, sm_post)) != cudaSuccess) return e;
-        { StageScope t(ST_INTRA, st); cw_intra_kernel<<<grid, kT, intracw::SMEM_BYTES, st>>>(p); }
-        { StageScope t(ST_POST, st); cw_post_kernel<<<CH, kT, sm_post, st>>>(p); }
+        { StageScope t(ST_INTRA, st); launch_kernel(cw_intra_kernel, grid, kT, intracw::SMEM_BYTES, st, p); }
+        { StageScope t(ST_POST, st); launch_kernel(cw_post_kernel, CH, kT, sm_post, st, p); }
     }
     return cudaGetLastError();
 }

@@ -33,6 +33,7 @@ static_assert(2 * (SMEM_BYTES + 4096) <= 228 * 1024, "two CTAs per SM");
 }  // namespace factors
 
 __global__ void __launch_bounds__(split::kT, 2) tc_factors_kernel(const __grid_constant__ TcParams P) {
+    wait_prerequisites();
     using namespace factors;
     const Problem& p = P.p;
     const int H = p.d.H;
@@ -257,6 +258,7 @@ static_assert(2 * (SMEM_BYTES + 4096) <= 228 * 1024, "two CTAs per SM");
 }  // namespace eprep
 
 __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_constant__ TcParams P) {
+    wait_prerequisites();
     using namespace eprep;
     const Problem& p = P.p;
     const int H = p.d.H;
