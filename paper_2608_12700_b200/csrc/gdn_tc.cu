@@ -952,14 +952,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_cw_kernel(const __grid_co
 // ------------------------------------------------------------------------------------------------
 // tc_intra: token gradients of one (chunk, head).
 //
-// Products (all on tcgen05, outputs transposed: features on TMEM lanes, tokens on columns, except the 64 x 64
-// token-token matrices which use M = 64):
-//   phase 1  (W h)^T ; (K dh')^T          (P = tril(Q K^T . D) comes from tc_prep, which forms it anyway)
-//   phase 2  (P^T dO)^T ; then, under the readout, dO h^T          -> U = U~ - W h ; dU = scale P^T dO + Diag(e) K dh'
-//   phase 3  dO U^T ; T^T dU                                       -> dPD = scale tril(dO U^T) . D ; dXv ; dv ; dw
-//   phase 4  dXv U^T ; dPD K ; -dXv h^T ; under the readout dPD^T Q ; U dh'^T
-//                                                                  -> G = -stril(dXv U^T) . D ; Diag(b) G ; dq ; (dXk)
-//   phase 5  G K ; += (Diag(b) G)^T K                               -> dk ; db ; dgamma -> dg
+// Products (all on tcgen05), in four dependent phases:
+//   phase 1  (W h)^T ; (K dh')^T ; (P^T dO)^T              -> U = U~ - W h ; dU = scale P^T dO + Diag(e) K dh'
+//   phase 2  dO U^T ; T^T dU ; under the readout U dh'^T   -> dPD = scale tril(dO U^T) . D ; dXv ; dv ; dw
+//   phase 3  dXv U^T ; under the readout [dO; dXv] h^T ; dPD^T Q   -> G = -stril(dXv U^T) . D ; Diag(b) G
+//   phase 4  [dPD; G] K ; += (Diag(b) G)^T K               -> dq ; dk ; db ; dgamma -> dg
+// (P = tril(Q K^T . D) comes from tc_prep, which forms it anyway.)
 // The vector-Jacobian product of the triangular solve (K#2) is taken in a shorter form than its definition
 // dW = -dU h^T, dXk = T^T dW, dXv = T^T dU, dA = -stril(dXk W^T + dXv U~^T):  T^T dW = -(T^T dU) h^T, so dXk = -dXv h^T,
 // and with it dXk W^T + dXv U~^T = dXv (U~ - W h)^T = dXv U^T.  dW is never formed, dXv follows dU directly (beside dP,
@@ -967,34 +965,56 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_cw_kernel(const __grid_co
 // The decay gradient uses the identities  rowsum(dP.P) + scale Gam <q, dO h^T> = <q, dq>  and its analogues for
 // k:  dgamma_i = <q_i, dq_i> + <k_i, dk_i^row> - <k_i, dk_i^col>, where dk^row = Diag(b)(G K + Diag(Gam) dXk)
 // collects the terms in which k_i enters with exp(+gamma_i) and dk^col those with exp(-gamma_i); the last row
-// of the chunk adds sum_j r_j + Gam_e <dh', h> (r_j = <(Kb dh')_j, U_j>).  Phases 1-2 produce transposed
-// accumulators (features on TMEM lanes) because their results feed later products; from phase 3 on every
-// accumulator that becomes a gradient is token-major.
+// of the chunk adds sum_j r_j + Gam_e <dh', h> (r_j = <(Kb dh')_j, U_j>).
+//
+// What bounds it: the chain of phases (issue and completion of the products, readout, barrier) and, within a readout, the
+// instruction issue; HBM needs 10 k of the cycles.  The forms of the products follow from that:
+// * Phase 1 is transposed (features on TMEM lanes) because its results feed later products.
+// * The two pairs of products with a common second operand, dO h^T with dXv h^T and dPD K with G K, are stacked along M: one
+//   instruction of M = 128 costs little more than one of M = 64 (97 against 86 cycles at N = 128), and the last readout finds a
+//   token of dq on each of lanes 0..63 and one of dk on each of lanes 64..127, where 64-row accumulators would leave half of
+//   the lanes of every warp idle.  The two products of dk^col are issued with M = 128 as well, their A operand shifted by one
+//   64-column block so that the 64 rows that count land on lanes 64..127, beside the other half of dk (the rows on lanes
+//   0..63 are made from whatever lies there and are never read).
+// * T^T dU is issued as two 64-column halves, one on lanes 0..15 and one on lanes 16..31 of each quadrant.
+// Measured on 4 x 16 heads of 2048 tokens (2048 chunk-heads): 108 us, 13.5 k cycles per chunk-head; with separate M = 64
+// products, gate gradients finished by two of the readout warps and dq assembled in a readout of its own it was 142 us (17.7 k).
+// 8 packed sequences, 32768 tokens, 32 heads: 971 -> 757 us.
 // ------------------------------------------------------------------------------------------------
 namespace intra {
-constexpr uint32_t QK = 0;                 // [Q ; K] x 128                     32 KB
-constexpr uint32_t VT = 32768;             // V  [64][128]                      16 KB   later staged dv
-constexpr uint32_t DO = VT + 16384;        // dO [64][128]                      16 KB   later dXv [64][128], then G and Diag(b) G [64][64] each
-constexpr uint32_t WT = DO + 16384;        // W^T  [128][64]                    16 KB
-constexpr uint32_t UTT = WT + 16384;       // U~^T [128][64]                    16 KB
-constexpr uint32_t TT = UTT + 16384;       // T [64][64]                         8 KB
-constexpr uint32_t HH = TT + 8192;         // h [128][128]                      32 KB
-constexpr uint32_t DH = HH + 32768;        // dh' [128][128]                    32 KB
-constexpr uint32_t PT = DH + 32768;        // P [64][64]                         8 KB   later dPD
-constexpr uint32_t UT = PT + 8192;         // U^T [128][64]                     16 KB   later staged dk
-constexpr uint32_t DUT = UT + 16384;       // dU^T [128][64]                    16 KB   later staged dq
+constexpr uint32_t OX = 0;                 // rows 0..63 dO, rows 64..127 dXv  x 128            32 KB
+constexpr uint32_t QT = OX + 32768;        // Q  [64][128]                                      16 KB
+constexpr uint32_t KT = QT + 16384;        // K  [64][128]                                      16 KB
+constexpr uint32_t VT = KT + 16384;        // V  [64][128], later staged dv                     16 KB
+constexpr uint32_t PG = VT + 16384;        // dPD [64][64]                                       8 KB  (these two: the stacked
+constexpr uint32_t TT = PG + 8192;         // T [64][64], later G                                8 KB   operand [dPD; G])
+constexpr uint32_t PT = TT + 8192;         // P [64][64], later Diag(b) G                        8 KB
+constexpr uint32_t HH = PT + 8192;         // h [128][128]                                      32 KB
+constexpr uint32_t DH = HH + 32768;        // dh' [128][128]                                    32 KB
+constexpr uint32_t UTT = DH + 32768;       // U~^T [128][64]                                    16 KB
+constexpr uint32_t UT = UTT + 16384;       // U^T [128][64], later staged dk                    16 KB
+constexpr uint32_t DUT = UT + 16384;       // dU^T [128][64], later staged dq                   16 KB
 constexpr uint32_t SMEM_BYTES = DUT + 16384 + 1024;
-constexpr uint32_t DXV = DO, DPD = PT, GT = DO, BGT = DO + 8192;
-// token-major staging of dq (over dU^T, last read by phase 3), of dv (in place over V: a thread overwrites exactly the
-// chunk it has just read) and of dk (over U^T, last read by the products of phase 4).  None of these is read by a later
-// product or rewritten within the trip, and of the loads that run ahead only V targets one of them (after its store
-// has read it), so the asynchronous stores need no wait on the critical path.
-constexpr uint32_t STG_A = DUT, STG_B = VT, STG_K = UT;
-static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
-__host__ __device__ constexpr uint32_t slot(int k) { return 64u * k; }   // eight accumulators of 64 columns
+// W^T lies where dXv will be written (rows 64..127 of the two column blocks of OX: two pieces of 64 rows)
+constexpr uint32_t W0 = OX + 8192, W1 = OX + 16384 + 8192;
+constexpr uint32_t BGT = PT;
+// Staging of dq, dv (in place: a thread overwrites exactly the piece it has just read) and dk: over tiles that no later
+// product reads.
+constexpr uint32_t STG_Q = DUT, STG_V = VT, STG_K = UT;
+static_assert(SMEM_BYTES + 8192 <= 227 * 1024, "shared memory budget");
+static_assert(TT == PG + 8192, "[dPD; G] is one operand tile");
+// TMEM columns (512 allocated).  The four accumulators of the last readout fill all of them; what earlier phases read out
+// lies where their products have not started yet.
+constexpr uint32_t C_UH = 0, C_A1 = 128, C_A2 = 256, C_C2 = 384;    // U dh'^T | [dO; dXv] h^T | [dPD; G] K | rest of dk^col
+constexpr uint32_t C_WH = 128, C_KD = 192, C_PD = 256;              // phase 1
+constexpr uint32_t C_DP = 320, C_DX = 384;                          // phase 2
+constexpr uint32_t C_DA = 256;                                      // phase 3
+constexpr int kGateWarp = 18;                       // the warp of the gate arrays and gradients
+constexpr int kThreadsAll = kIntraThreads + 64;     // 16 readout warps, issuer, loader, gates
+constexpr int kBarThreads = kIntraThreads + 32;     // ... all but the loader meet at the named barrier
 }  // namespace intra
 
-__global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_intra_kernel(const __grid_constant__ TcParams P) {
+__global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const __grid_constant__ TcParams P) {
     wait_prerequisites();
     using namespace intra;
     const Problem& p = P.p;
@@ -1010,8 +1030,8 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_intra_kernel(const _
     unsigned char* sm = align1024(smem_raw);
     __shared__ __align__(16) float gate_sets[2][5][kC];   // two sets: a trip's gate arrays are written during the trip before
     __shared__ float red[4][kGroups][kC];       // four token-wise partial sums: [which][column group][token]
-    __shared__ float dgam[kC], scal[2][kIntraThreads / 32];
-    __shared__ uint64_t bar_k, bar_g1, bar_g2, bar_do, bar_ld0, bar_ldw, bar_ldh, bar_ld1, bar_ld2, bar_st1, bar_st2, bar_kfree, bar_free, bar_mma;
+    __shared__ float scal[2][kWideThreads / 32];
+    __shared__ uint64_t bar_a, bar_u, bar_b, bar_ld0, bar_e0, bar_e1, bar_e2, bar_e3, bar_st1, bar_st2, bar_v, bar_kq, bar_free, bar_mma;
     __shared__ uint32_t tmem_slot;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int q4 = warp & 3, grp = warp >> 2;
@@ -1026,11 +1046,13 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_intra_kernel(const _
     // soon as the region it goes to has been read for the last time in this trip.  It shares no block-wide barrier
     // with the other warps inside the loop (they use a named barrier); it follows them through mbarriers.
     const bool loader = warp == 17;
+    // Warp 18 makes the next trip's gate arrays and finishes the previous trip's gate gradients beside the readouts.
+    const bool gates = warp == kGateWarp;
 
     if (threadIdx.x == 0) {
-        mbar_init(&bar_k, 1); mbar_init(&bar_g1, 1); mbar_init(&bar_g2, 1); mbar_init(&bar_do, 1);
-        mbar_init(&bar_ld0, 1); mbar_init(&bar_ldw, 1); mbar_init(&bar_ldh, 1); mbar_init(&bar_ld1, 1); mbar_init(&bar_ld2, 1);
-        mbar_init(&bar_st1, 1); mbar_init(&bar_st2, 1); mbar_init(&bar_kfree, 16); mbar_init(&bar_free, 1);
+        mbar_init(&bar_a, 1); mbar_init(&bar_u, 1); mbar_init(&bar_b, 1);
+        mbar_init(&bar_ld0, 1); mbar_init(&bar_e0, 1); mbar_init(&bar_e1, 1); mbar_init(&bar_e2, 1); mbar_init(&bar_e3, 1);
+        mbar_init(&bar_st1, 1); mbar_init(&bar_st2, 1); mbar_init(&bar_v, 1); mbar_init(&bar_kq, 16); mbar_init(&bar_free, 1);
         mbar_init(&bar_mma, 1);
         fence_mbar_init();
     }
@@ -1041,27 +1063,28 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_intra_kernel(const _
     const uint32_t tmem = tmem_slot;
     bool ok = true;
 
-    // The tiles of a trip arrive in groups, one mbarrier each, loaded during the previous trip as their regions fall free:
-    //   g1  W, U~^T              once the second readout is done             needed by phase 1
-    //       h, dh', P            once the products of phase 4 are done
-    //       Q                    once the readout of phase 4 is done
-    //   do  dO;  g2  T, V        once the products of the last phase are done  needed from phase 2 / 3 on
-    //                            (V goes where dv is staged: its store, or the flush of a ragged tail, must have read it)
-    //   k   K                    once the last readout holds its K values    needed by phase 1
-    constexpr uint32_t K_BYTES = 16384, G1_BYTES = 16384 + 16384 + 32768 + 32768 + 16384 + 8192, G2_BYTES = 8192 + 16384, DO_BYTES = 16384;
+    // The tiles of a trip arrive in three groups, one mbarrier each, loaded during the previous trip as their regions fall free:
+    //   u  U~^T             once the first readout is done (e0)
+    //   a  dh'              once U dh'^T is done (e1)
+    //      h, dO, W^T       once [dO; dXv] h^T is done (e2)
+    //      P, K             once the products of phase 4 are done (e3); K also read by the last readout
+    //   b  V                once the staged dv has left (needed by the second readout)
+    //      T, Q             once the products of phase 4 are done; Q also read by the last readout
+    constexpr uint32_t A_BYTES = 16384 + 32768 + 32768 + 16384 + 16384 + 8192, B_BYTES = 8192 + 16384 + 16384, U_BYTES = 16384;
     auto load_piece = [&](int piece, const ChunkInfo& c) {
         const int cb = piece & 1, xq = c.hd * D + cb * 64;
         switch (piece) {
-            case 0: case 1: tma_load_2d(sm + QK + cb * 16384 + 8192, &P.tm_k, xq, c.tok0, &bar_k); break;
-            case 2: case 3: tma_load_2d(sm + QK + cb * 16384, &P.tm_q, xq, c.tok0, &bar_g1); break;
-            case 4: bulk_load(sm + UTT, p.ws + p.L.Ut + (size_t)c.ch * 16384, 16384, &bar_g1); break;
-            case 5: bulk_load(sm + DH, p.ws + p.L.dhn + (size_t)c.ch * 32768, 32768, &bar_g1); break;
-            case 6: bulk_load(sm + HH, p.ws + p.L.hc + (size_t)c.ch * 32768, 32768, &bar_g1); break;
-            case 7: bulk_load(sm + WT, p.ws + p.L.W + (size_t)c.ch * 16384, 16384, &bar_g1); break;
-            case 8: case 9: tma_load_2d(sm + DO + cb * 8192, &P.tm_do, xq, c.tok0, &bar_do); break;
-            case 10: case 11: tma_load_2d(sm + VT + cb * 8192, &P.tm_v, xq, c.tok0, &bar_g2); break;
-            case 12: bulk_load(sm + TT, p.ws + p.L.Tm + (size_t)c.ch * 8192, 8192, &bar_g2); break;
-            case 13: bulk_load(sm + PT, p.ws + p.L.Pm + (size_t)c.ch * 8192, 8192, &bar_g1); break;
+            case 0: case 1: tma_load_2d(sm + KT + cb * 8192, &P.tm_k, xq, c.tok0, &bar_a); break;
+            case 2: case 3: tma_load_2d(sm + OX + cb * 16384, &P.tm_do, xq, c.tok0, &bar_a); break;
+            case 4: bulk_load(sm + DH, p.ws + p.L.dhn + (size_t)c.ch * 32768, 32768, &bar_a); break;
+            case 5: bulk_load(sm + HH, p.ws + p.L.hc + (size_t)c.ch * 32768, 32768, &bar_a); break;
+            case 6: bulk_load(sm + W0, p.ws + p.L.W + (size_t)c.ch * 16384, 8192, &bar_a); break;
+            case 7: bulk_load(sm + W1, p.ws + p.L.W + (size_t)c.ch * 16384 + 8192, 8192, &bar_a); break;
+            case 8: bulk_load(sm + PT, p.ws + p.L.Pm + (size_t)c.ch * 8192, 8192, &bar_a); break;
+            case 9: bulk_load(sm + UTT, p.ws + p.L.Ut + (size_t)c.ch * 16384, 16384, &bar_u); break;
+            case 10: case 11: tma_load_2d(sm + QT + cb * 8192, &P.tm_q, xq, c.tok0, &bar_b); break;
+            case 12: case 13: tma_load_2d(sm + VT + cb * 8192, &P.tm_v, xq, c.tok0, &bar_b); break;
+            case 14: bulk_load(sm + TT, p.ws + p.L.Tm + (size_t)c.ch * 8192, 8192, &bar_b); break;
             default: break;
         }
     };
@@ -1069,7 +1092,7 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_intra_kernel(const _
     if (loader) {
         if (lane == 0) {
             uint32_t ph = 0;
-            bool lok = true, pend_k = false, pend1 = false, pend2 = false, pend_do = false;
+            bool lok = true, pend_a = false, pend_b = false, pend_u = false;
 #pragma unroll 1
             for (int item = blockIdx.x; item < n_items && lok; item += gridDim.x, ph ^= 1) {
                 ChunkInfo x, nx;
@@ -1077,137 +1100,140 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_intra_kernel(const _
                 const bool has_next = item + (int)gridDim.x < n_items;
                 if (has_next) chunk_entry(p, nx, item + gridDim.x);
                 const bool full = x.len == kC;
-                pend_k = pend1 = pend2 = pend_do = false;
-                // the trip is under way (all its tiles have arrived): K of the next one, the only late load, -> L2
-                if (!(lok = mbar_wait(&bar_ld0, ph))) break;
-                if (has_next) {
-                    prefetch_l2_tma_2d(&P.tm_k, nx.hd * D, nx.tok0);
-                    prefetch_l2_tma_2d(&P.tm_k, nx.hd * D + 64, nx.tok0);
-                }
+                pend_a = pend_b = pend_u = false;
                 // (Early loads not in a CTA's first trip: there every CTA of the grid reaches these points at the same moment,
                 // the loads come as one burst of 25 MB, and the instruction fetches of the last phases, which run for the
                 // first time, queue behind it for microseconds.  The first trip loads at its end instead.)
-                const bool early = item != (int)blockIdx.x;
-                // the second readout is done: W^T and U~^T have been read for the last time
-                if (!(lok = mbar_wait(&bar_ldw, ph))) break;
-                if (has_next && early) {
-                    mbar_expect_tx(&bar_g1, G1_BYTES);   // the first piece of the group announces all of it
-                    pend1 = true;
-                    load_piece(7, nx);
-                    load_piece(4, nx);
+                const bool early = has_next && item != (int)blockIdx.x;
+                if (!(lok = mbar_wait(&bar_ld0, ph))) break;   // the trip is under way: the late loads of the next one -> L2
+                if (early) {
+                    for (int cb = 0; cb < 2; ++cb) prefetch_l2_tma_2d(&P.tm_k, nx.hd * D + cb * 64, nx.tok0);
+                    prefetch_l2_bulk(p.ws + p.L.Pm + (size_t)nx.ch * 8192, 8192);
+                    prefetch_l2_bulk(p.ws + p.L.Tm + (size_t)nx.ch * 8192, 8192);
+                    for (int cb = 0; cb < 2; ++cb) prefetch_l2_tma_2d(&P.tm_do, nx.hd * D + cb * 64, nx.tok0);
                 }
-                // the products of phase 4 are done: h, dh' and dPD (over P) have been read for the last time
-                if (!(lok = mbar_wait(&bar_ldh, ph))) break;
-                if (has_next && early) {
-                    load_piece(6, nx);
-                    load_piece(5, nx);
-                    load_piece(13, nx);
-                }
-                // dq, dv are staged
-                if (!(lok = mbar_wait(&bar_st1, ph))) break;
+                if (!(lok = mbar_wait(&bar_e0, ph))) break;    // U~^T has been read by the first readout
+                if (early) { mbar_expect_tx(&bar_u, U_BYTES); pend_u = true; load_piece(9, nx); }
+                if (!(lok = mbar_wait(&bar_e1, ph))) break;    // dh'
+                if (early) { mbar_expect_tx(&bar_a, A_BYTES); pend_a = true; load_piece(4, nx); }   // (the first piece announces the group)
+                if (!(lok = mbar_wait(&bar_st1, ph))) break;   // dv is staged
                 if (full) {
-                    for (int cb = 0; cb < 2; ++cb) {
-                        tma_store_2d(&P.tm_dq, x.hd * D + cb * 64, x.tok0, sm + STG_A + cb * 8192);
-                        tma_store_2d(&P.tm_dv, x.hd * D + cb * 64, x.tok0, sm + STG_B + cb * 8192);
-                    }
+                    for (int cb = 0; cb < 2; ++cb) tma_store_2d(&P.tm_dv, x.hd * D + cb * 64, x.tok0, sm + STG_V + cb * 8192);
                     bulk_commit();
                 }
-                // the readout of phase 4 is done too: Q has been read for the last time
-                if (!(lok = mbar_wait(&bar_ld1, ph))) break;
-                if (has_next && early) {
+                if (!(lok = mbar_wait(&bar_e2, ph))) break;    // dO, h and dXv (over W^T)
+                if (early) {
+                    load_piece(5, nx);
+                    load_piece(6, nx);
+                    load_piece(7, nx);
                     load_piece(2, nx);
                     load_piece(3, nx);
                 }
-                // the last phase is done and its readout holds its K values in registers: K first, the next trip starts with
-                // it; dO, T, V are not needed before its second phase (V goes where dv is staged, so that store must have
-                // read its source)
-                if (!(lok = mbar_wait(&bar_ld2, ph))) break;
-                if (!(lok = mbar_wait(&bar_kfree, ph))) break;
-                if (has_next && early) {
-                    mbar_expect_tx(&bar_k, K_BYTES);
-                    pend_k = true;
+                if (!(lok = mbar_wait(&bar_v, ph))) break;     // (a ragged tail's dv has been flushed)
+                bulk_wait_read<0>();
+                if (early) {
+                    mbar_expect_tx(&bar_b, B_BYTES);
+                    pend_b = true;
+                    load_piece(12, nx);
+                    load_piece(13, nx);
+                }
+                if (!(lok = mbar_wait(&bar_e3, ph))) break;    // the products of phase 4 are done: Diag(b) G (over P), G (over T)
+                if (early) { load_piece(8, nx); }
+                if (!(lok = mbar_wait(&bar_kq, ph))) break;    // ... and the readout holds its rows of K and Q
+                if (early) {
                     load_piece(0, nx);
                     load_piece(1, nx);
-                    mbar_expect_tx(&bar_do, DO_BYTES);   // dO next: the second phase starts with it
-                    pend_do = true;
-                    load_piece(8, nx);
-                    load_piece(9, nx);
-                    bulk_wait_read<0>();
-                    mbar_expect_tx(&bar_g2, G2_BYTES);
-                    pend2 = true;
-#pragma unroll 1
-                    for (int piece = 10; piece <= 12; ++piece) load_piece(piece, nx);
+                    load_piece(14, nx);
+                    load_piece(10, nx);
+                    load_piece(11, nx);
                 }
-                // dk is staged
-                if (!(lok = mbar_wait(&bar_st2, ph))) break;
+                if (!(lok = mbar_wait(&bar_st2, ph))) break;   // dq, dk are staged
                 if (full) {
-                    for (int cb = 0; cb < 2; ++cb) tma_store_2d(&P.tm_dk, x.hd * D + cb * 64, x.tok0, sm + STG_K + cb * 8192);
+                    for (int cb = 0; cb < 2; ++cb) {
+                        tma_store_2d(&P.tm_dq, x.hd * D + cb * 64, x.tok0, sm + STG_Q + cb * 8192);
+                        tma_store_2d(&P.tm_dk, x.hd * D + cb * 64, x.tok0, sm + STG_K + cb * 8192);
+                    }
                     bulk_commit();
+                }
+                if (has_next && !early) {
+                    mbar_expect_tx(&bar_a, A_BYTES);
+                    mbar_expect_tx(&bar_b, B_BYTES);
+                    mbar_expect_tx(&bar_u, U_BYTES);
+                    pend_a = pend_b = pend_u = true;
+#pragma unroll 1
+                    for (int piece = 0; piece <= 14; ++piece) load_piece(piece, nx);
                 }
                 bulk_wait_read<0>();
                 mbar_arrive(&bar_free);   // the staging regions may be rewritten
-                if (has_next && !early) {
-                    mbar_expect_tx(&bar_k, K_BYTES);
-                    mbar_expect_tx(&bar_g1, G1_BYTES);
-                    mbar_expect_tx(&bar_g2, G2_BYTES);
-                    mbar_expect_tx(&bar_do, DO_BYTES);
-                    pend_k = pend1 = pend2 = pend_do = true;
-#pragma unroll 1
-                    for (int piece = 0; piece <= 13; ++piece) load_piece(piece, nx);
-                }
             }
             bulk_wait_read<0>();
             if (!lok) {   // after a timeout a copy may still be in flight: wait for it before the CTA may retire
-                if (pend_k) (void)mbar_wait(&bar_k, ph ^ 1);
-                if (pend1) (void)mbar_wait(&bar_g1, ph ^ 1);
-                if (pend2) (void)mbar_wait(&bar_g2, ph ^ 1);
-                if (pend_do) (void)mbar_wait(&bar_do, ph ^ 1);
+                if (pend_a) (void)mbar_wait(&bar_a, ph ^ 1);
+                if (pend_b) (void)mbar_wait(&bar_b, ph ^ 1);
+                if (pend_u) (void)mbar_wait(&bar_u, ph ^ 1);
             }
         }
         return;
     }
 
-    auto cta_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kIntraThreads) : "memory"); };   // all warps but the loader
+    auto cta_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kBarThreads) : "memory"); };   // all warps but the loader
     uint32_t mma_phase = 0, in_phase = 0;
-    // chunk table entry and gates of a trip are fetched one trip ahead into registers (their latency would be exposed)
     ChunkInfo xn;
     chunk_entry(p, xn, blockIdx.x);
-    float ng = 0.f, ngend = 0.f, nb = 0.f;
-    auto fetch_gates = [&](const ChunkInfo& c) {   // cumulative log decay of this thread's token and of the chunk end, gate b
+    // The gate warp: lane l owns tokens l and l + 32.  Values are fetched one phase before they are turned into arrays.
+    float ng[2] = {0.f, 0.f}, nb[2] = {0.f, 0.f}, ngend = 0.f, bb_prev[2] = {0.f, 0.f}, Gam_last_prev = 0.f;
+    auto fetch_gates = [&](const ChunkInfo& c) {   // cumulative log decays and the one of the chunk end, erase gates
         const float* gsrc = reinterpret_cast<const float*>(p.ws + p.L.gamma) + (size_t)c.ch * kC;
-        ng = gsrc[threadIdx.x];
         ngend = gsrc[kC - 1];
-        nb = ((int)threadIdx.x < c.len && p.d.delta_rule) ? p.beta[(size_t)(c.tok0 + (int)threadIdx.x) * H + c.hd] : 0.f;
-    };
-    auto make_gates = [&](int set) {   // threads 0..63: the fetched values -> gate arrays of set `set`
-        const int i = threadIdx.x;
-        gate_sets[set][0][i] = ng * kLog2e;
-        gate_sets[set][1][i] = expf(ng);
-        gate_sets[set][2][i] = expf(ngend - ng);
-        gate_sets[set][3][i] = nb;                                                    // erase gate
-        gate_sets[set][4][i] = p.d.delta_rule ? nb : (i < xn.len ? 1.f : 0.f);        // write gate (delta rule off: 0 and 1)
-    };
-    // dbeta and dg of the previous trip's chunk, from its token-wise partial sums (warps 0 and 1; see the trip's end)
-    ChunkInfo xp = xn;
-    bool have_prev = false;
-    float bb_prev = 0.f, Gam_last_prev = 0.f;
-    auto finish_gates = [&]() {
-        const int i = threadIdx.x;
-        auto tot = [&](int w) { return (red[w][0][i] + red[w][1][i]) + (red[w][2][i] + red[w][3][i]); };
-        const float qdq = tot(0), dw = tot(1), db = tot(2), kcol = tot(3);
-        if (i < xp.len && p.dbeta) p.dbeta[(size_t)(xp.tok0 + i) * H + xp.hd] = db + dw;
-        dgam[i] = fmaf(bb_prev, db, qdq - kcol);
-        asm volatile("bar.sync 2, 64;" ::: "memory");
-        if (warp == 0) {
-            constexpr int nw = kIntraThreads / 32;   // per-warp partial sums, one per lane
-            const float rsum = warp_sum(lane < nw ? scal[0][lane] : 0.f), hsum = warp_sum(lane < nw ? scal[1][lane] : 0.f);
-            write_dg_suffix(dgam, nullptr, rsum + Gam_last_prev * hsum, p.dg + (size_t)xp.tok0 * H + xp.hd, (size_t)H, xp.len, lane);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = lane + 32 * h;
+            ng[h] = gsrc[i];
+            nb[h] = (i < c.len && p.d.delta_rule) ? p.beta[(size_t)(c.tok0 + i) * H + c.hd] : 0.f;
         }
     };
+    auto make_gates = [&](int set) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = lane + 32 * h;
+            gate_sets[set][0][i] = ng[h] * kLog2e;
+            gate_sets[set][1][i] = expf(ng[h]);
+            gate_sets[set][2][i] = expf(ngend - ng[h]);
+            gate_sets[set][3][i] = nb[h];                                                 // erase gate
+            gate_sets[set][4][i] = p.d.delta_rule ? nb[h] : (i < xn.len ? 1.f : 0.f);     // write gate (delta rule off: 0 and 1)
+        }
+    };
+    // dbeta and dg of the previous trip's chunk, from its token-wise partial sums
+    ChunkInfo xp = xn;
+    bool have_prev = false;
+    auto finish_gates = [&]() {
+        float v[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = lane + 32 * h;
+            auto tot = [&](int w) { return (red[w][0][i] + red[w][1][i]) + (red[w][2][i] + red[w][3][i]); };
+            const float qdq = tot(0), dw = tot(1), db = tot(2), kcol = tot(3);
+            if (i < xp.len && p.dbeta) p.dbeta[(size_t)(xp.tok0 + i) * H + xp.hd] = db + dw;
+            v[h] = fmaf(bb_prev[h], db, qdq - kcol);
+        }
+        constexpr int nw = kWideThreads / 32;   // per-warp partial sums, one per lane
+        const float rsum = warp_sum(lane < nw ? scal[0][lane] : 0.f), hsum = warp_sum(lane < nw ? scal[1][lane] : 0.f);
+        // dg_j = sum_{i >= j} dgam_i inside the chunk
+        float a = v[0], b = v[1] + (lane == 31 ? rsum + Gam_last_prev * hsum : 0.f);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float ta = __shfl_down_sync(0xffffffffu, a, o), tb = __shfl_down_sync(0xffffffffu, b, o);
+            if (lane + o < 32) { a += ta; b += tb; }
+        }
+        a += __shfl_sync(0xffffffffu, b, 0);
+        float* dg = p.dg + (size_t)xp.tok0 * H + xp.hd;
+        if (lane < xp.len) dg[(size_t)lane * H] = a;
+        if (lane + 32 < xp.len) dg[(size_t)(lane + 32) * H] = b;
+    };
     // first trip: every group is loaded at once, one instruction per warp
-    if (issuer) { mbar_expect_tx(&bar_k, K_BYTES); mbar_expect_tx(&bar_g1, G1_BYTES); mbar_expect_tx(&bar_g2, G2_BYTES); mbar_expect_tx(&bar_do, DO_BYTES); }
-    if (lane == 0 && warp < 14) load_piece(warp, xn);
-    if (threadIdx.x < kC) { fetch_gates(xn); make_gates(0); }
+    if (issuer) { mbar_expect_tx(&bar_a, A_BYTES); mbar_expect_tx(&bar_b, B_BYTES); mbar_expect_tx(&bar_u, U_BYTES); }
+    if (lane == 0 && warp < 15) load_piece(warp, xn);
+    if (gates) { fetch_gates(xn); make_gates(0); }
 #pragma unroll 1
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, in_phase ^= 1) {
     const ChunkInfo x = xn;
@@ -1217,64 +1243,51 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_intra_kernel(const _
     const float* ee = gate_sets[in_phase][2];
     const float* bb = gate_sets[in_phase][3];
     const bool has_next = item + (int)gridDim.x < n_items;
-    const bool first = item == (int)blockIdx.x;
+    const bool first = item == (int)blockIdx.x, full = x.len == kC;
     if (has_next) chunk_entry(p, xn, item + gridDim.x);
 
     if (ok) {
-        ok = mbar_wait(&bar_g1, in_phase);
-        ok = ok && mbar_wait(&bar_k, in_phase);
+        ok = mbar_wait(&bar_a, in_phase);
         if (!ok && threadIdx.x == 0) report_timeout(p.ws, 20);
     }
-    if (ok && x.len < kC) {
-        zero_tail_rows(sm + QK, 128, 0, x.len, kIntraThreads);
-        zero_tail_rows(sm + QK, 128, 64, x.len, kIntraThreads);
+    if (ok && !full) {
+        zero_tail_rows(sm + KT, 64, 0, x.len, kWideThreads);
+        zero_tail_rows(sm + OX, 128, 0, x.len, kWideThreads);
         fence_async_smem();
     }
     cta_sync();
 
-    // ---- phase 1: (W h)^T and (K dh')^T.  P = tril(Q K^T . D) is not formed here: tc_prep made it and it arrived
-    // with the first group of tiles.
+    // ---- phase 1: (W h)^T, (K dh')^T, (P^T dO)^T
     if (ok && issuer) {
         tc_fence_after();
-        mma_tile<128, 64, 128>(tmem + slot(1), op_mn_major(sm + HH, 128), op_mn_major(sm + WT, 128), false);
-        mma_tile<128, 64, 128>(tmem + slot(2), op_mn_major(sm + DH, 128), op_k_major(sm + QK, 128, 64), false);
+        Operand w = op_mn_major(sm + W0, 64);   // W^T in two pieces of 64 rows
+        w.jump = (W1 - W0 - 8192) / 16;
+        mma_tile<128, 64, 128>(tmem + C_WH, op_mn_major(sm + HH, 128), w, false);
+        mma_tile<128, 64, 128>(tmem + C_KD, op_mn_major(sm + DH, 128), op_k_major(sm + KT, 64), false);
+        mma_tile<128, 64, 64>(tmem + C_PD, op_mn_major(sm + OX, 128), op_mn_major(sm + PT, 64), false);
+        mma_commit(&bar_mma);
     }
+    if (threadIdx.x == 32) mbar_arrive(&bar_ld0);
+    if (gates && have_prev && ok) finish_gates();   // the previous chunk's gate gradients
     if (ok) {
-        ok = mbar_wait(&bar_do, in_phase);
+        ok = mbar_wait(&bar_u, in_phase);
         if (!ok && threadIdx.x == 0) report_timeout(p.ws, 27);
     }
-    if (ok && x.len < kC) {
-        zero_tail_rows(sm + DO, 64, 0, x.len, kIntraThreads);
-        fence_async_smem();
-    }
-    cta_sync();
-
-    // ---- phase 2
-    if (ok && issuer) {
-        tc_fence_after();
-        mma_tile<128, 64, 64>(tmem + slot(3), op_mn_major(sm + DO, 64), op_mn_major(sm + PT, 64), false);
-        mma_commit(&bar_mma);
-        // dO h^T (token-major, group A of columns 384..511) is first read after phase 4: it runs under the readout
-        mma_tile<64, 128, 128>(tmem + 384, op_k_major(sm + DO, 64), op_k_major(sm + HH, 128), false);
-    }
-    if (threadIdx.x == 32) mbar_arrive(&bar_ld0);   // every tile of this trip has arrived
-    if (has_next && threadIdx.x < kC) fetch_gates(xn);
-    if (ok && have_prev && warp < 2) finish_gates();   // warps 0 and 1: the previous chunk's gate gradients
     GDN_WAIT_MMA(22)
     if (ok && !first) {   // U^T and dU^T held the previous trip's staged dk and dq: their stores must have read them
         ok = mbar_wait(&bar_free, in_phase ^ 1);
         if (!ok && threadIdx.x == 0) report_timeout(p.ws, 28);
     }
-    const int f = q4 * 32 + lane;      // feature (lane of the transposed accumulators)
-    const int i0 = grp * kTG;          // first of this thread's 32 tokens
+    const int i0 = grp * kTG;          // first of this thread's 16 tokens (or columns of a 64-column accumulator)
     float rs = 0.f;
     if (ok && worker) {
+        const int f = q4 * 32 + lane;      // feature (lane of the transposed accumulators)
         float t2[2][8], kb2[2][8], pd2[2][8];
 #pragma unroll
         for (int part = 0; part < 2; ++part) {
-            tmem_ld8(tmem + lane_base + slot(1) + i0 + part * 8, t2[part]);
-            tmem_ld8(tmem + lane_base + slot(2) + i0 + part * 8, kb2[part]);
-            tmem_ld8(tmem + lane_base + slot(3) + i0 + part * 8, pd2[part]);
+            tmem_ld8(tmem + lane_base + C_WH + i0 + part * 8, t2[part]);
+            tmem_ld8(tmem + lane_base + C_KD + i0 + part * 8, kb2[part]);
+            tmem_ld8(tmem + lane_base + C_PD + i0 + part * 8, pd2[part]);
         }
         tmem_wait_ld();
 #pragma unroll
@@ -1295,149 +1308,123 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_intra_kernel(const _
             chunk_store(sm + DUT, 128, f, ib >> 3, pd);
         }
     }
-    if (ok) {   // T and V, the last tiles of this trip, are needed from phase 3 on
-        ok = mbar_wait(&bar_g2, in_phase);
+    if (ok) {   // T and V are needed from phase 2 on, Q from phase 3 on
+        ok = mbar_wait(&bar_b, in_phase);
         if (!ok && threadIdx.x == 0) report_timeout(p.ws, 31);
     }
-    if (ok && x.len < kC) zero_tail_rows(sm + VT, 64, 0, x.len, kIntraThreads);
+    if (ok && !full) zero_tail_rows(sm + QT, 64, 0, x.len, kWideThreads);
     tc_fence_before();
     fence_async_smem();
     cta_sync();
-    if (threadIdx.x == 32) mbar_arrive(&bar_ldw);   // W^T (read by phase 1) and U~^T (read by the readout) are free
+    if (threadIdx.x == 32) mbar_arrive(&bar_e0);   // U~^T has been read
 
-    // From here on the accumulators that become gradients are produced token-major (64 token rows x 128 features,
-    // M = 64): a thread owns a token row, so row dots are thread-local and rows leave with 16-byte stores.  A 64-row
-    // accumulator occupies lanes 0..15 of each quadrant ("group A"); a second one sits in lanes 16..31 of the same
-    // columns ("group B", address + 16 lanes), and one tcgen05.ld serves both groups.
-    //   columns   group A                               group B
-    //   0..127    U dh'^T (ph 4)                        dP (ph 3, 64 cols)
-    //   128..255  (dP.D) K (ph 4)                       dXv (ph 3)
-    //   256..383  dk^col: (dP.D)^T Q (ph 4) += (bG)^T K  dXk = -dXv h^T (ph 4; read with dk^col, handed over by shuffle)
-    //   384..511  dO h^T (ph 2) -> G K (ph 5)           dXv U^T (ph 4, 64 cols)
+    // Token-major accumulators with 64 rows (M = 64) occupy lanes 0..15 of each quadrant, or lanes 16..31 (address + 16 lanes).
     constexpr uint32_t LB = 16u << 16;
     const bool ga = lane < 16;
-    const int tr = q4 * 16 + (lane & 15);   // token row of this lane in token-major accumulators
-    const int cb0 = grp * 32;               // first of this thread's 32 feature columns
-    const int j0b = grp * kTG;              // first of its 16 columns in 64-column accumulators
+    const int tr = q4 * 16 + (lane & 15);   // token row of this lane there
 
-    // ---- phase 3: dO U^T and dXv = T^T dU
+    // ---- phase 2: dO U^T and dXv = T^T dU (features 0..63 on lanes 0..15, 64..127 on lanes 16..31)
     if (ok && issuer) {
         tc_fence_after();
-        mma_tile<64, 64, 128>(tmem + 0 + LB, op_k_major(sm + DO, 64), op_mn_major(sm + UT, 128), false);           // dO U^T
-        mma_tile<64, 128, 64>(tmem + 128 + LB, op_mn_major(sm + TT, 64), op_k_major(sm + DUT, 128), false);         // T^T dU
+        mma_tile<64, 64, 128>(tmem + C_DP, op_k_major(sm + OX, 128), op_mn_major(sm + UT, 128), false);
+        mma_tile<64, 64, 64>(tmem + C_DX, op_mn_major(sm + TT, 64), op_k_major(sm + DUT, 128, 0), false);
+        mma_tile<64, 64, 64>(tmem + C_DX + LB, op_mn_major(sm + TT, 64), op_k_major(sm + DUT, 128, 64), false);
         mma_commit(&bar_mma);
+        // U dh'^T, rows on lanes 64..127, is first read after phase 4: it runs under the readout
+        mma_tile<128, 128, 128>(tmem + C_UH, op_mn_major(sm + UT - 16384, 128), op_k_major(sm + DH, 128), false);
     }
-    if (has_next && threadIdx.x < kC) make_gates(in_phase ^ 1);   // the next trip's gate arrays, while the products run
     // <dh', h> over the whole state, while the products run (both tiles share one format, so offsets pair up)
     float hh = 0.f;
-#pragma unroll 1
-    for (int t = (int)threadIdx.x - 64; t >= 0 && t < 2048; t += kIntraThreads - 64) {
-        float a[8], b[8];
-        unpack8(*reinterpret_cast<const uint4*>(sm + HH + t * 16), a);
-        unpack8(*reinterpret_cast<const uint4*>(sm + DH + t * 16), b);
+    if (worker) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) hh = fmaf(a[k], b[k], hh);
+        for (int t = 0; t < 4; ++t) {
+            float a[8], b[8];
+            unpack8(*reinterpret_cast<const uint4*>(sm + HH + (threadIdx.x + t * kWideThreads) * 16), a);
+            unpack8(*reinterpret_cast<const uint4*>(sm + DH + (threadIdx.x + t * kWideThreads) * 16), b);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) hh = fmaf(a[k], b[k], hh);
+        }
     }
+    if (gates && has_next) fetch_gates(xn);
     GDN_WAIT_MMA(23)
-    const bool full = x.len == kC;
     // (addresses of the ragged-tail flushes are formed where they are used: nothing of them lives across the phases)
     auto grad_rows = [&](void* base) { return reinterpret_cast<__nv_bfloat16*>(base) + ((size_t)x.tok0 * H + x.hd) * D; };
-    if (ok && worker) {   // group B holds both accumulators (the loads are warp-wide instructions)
+    if (ok && worker) {
         float v2[2][8];
-        tmem_ld8(tmem + lane_base + 0 + j0b, v2[0]);
-        tmem_ld8(tmem + lane_base + 0 + j0b + 8, v2[1]);
+        tmem_ld8(tmem + lane_base + C_DP + i0, v2[0]);
+        tmem_ld8(tmem + lane_base + C_DP + i0 + 8, v2[1]);
         tmem_wait_ld();
-        if (!ga) {   // dPD = scale tril(dO U^T) . D
+        if (ga) {   // dPD = scale tril(dO U^T) . D
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
-                const int jb = j0b + part * 8;
+                const int jb = i0 + part * 8;
                 float (&v)[8] = v2[part];
                 float g8[8];
                 ld8s(gl + jb, g8);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) v[j] = (jb + j <= tr) ? sc * v[j] * ex2(gl[tr] - g8[j]) : 0.f;
-                chunk_store(sm + DPD, 64, tr, jb >> 3, v);
+                chunk_store(sm + PG, 128, tr, jb >> 3, v);
             }
         }
-        // dXv -> operand tile (over dO, which every product has read) ; <v, dXv> (dw partial) ; dv = w dXv, staged over V
+        // dXv -> operand tile beside dO (over W^T) ; <v, dXv> (dw partial) ; dv = w dXv, staged over V
+        tmem_ld8(tmem + lane_base + C_DX + i0, v2[0]);
+        tmem_ld8(tmem + lane_base + C_DX + i0 + 8, v2[1]);
+        tmem_wait_ld();
         float acc = 0.f;
         const float wg = gate_sets[in_phase][4][tr];
 #pragma unroll
-        for (int part = 0; part < 4; ++part) {
-            const int cb = cb0 + part * 8;
-            float b[8], t8[8];
-            tmem_ld8(tmem + lane_base + 128 + cb, b);
-            tmem_wait_ld();
-            if (!ga) {
-                unpack8(*reinterpret_cast<const uint4*>(sm + VT + tile_chunk_off(64, tr, cb >> 3)), t8);
-                chunk_store(sm + DXV, 64, tr, cb >> 3, b);
+        for (int part = 0; part < 2; ++part) {
+            const int chk = (ga ? 0 : 8) + (i0 >> 3) + part;   // 8-feature piece
+            float (&b)[8] = v2[part];
+            float t8[8];
+            chunk_load(sm + VT, 64, tr, chk, t8);
+            chunk_store(sm + OX, 128, 64 + tr, chk, b);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    acc = fmaf(t8[j], b[j], acc);
-                    b[j] *= wg;
-                }
-                chunk_store(sm + STG_B, 64, tr, cb >> 3, b);
+            for (int j = 0; j < 8; ++j) {
+                acc = fmaf(t8[j], b[j], acc);
+                b[j] *= wg;
             }
+            chunk_store(sm + STG_V, 64, tr, chk, b);
         }
-        if (!ga) red[1][grp][tr] = acc;
+        acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+        if (ga) red[1][grp][tr] = acc;
     }
     tc_fence_before();
     fence_async_smem();
     cta_sync();
+    if (threadIdx.x == 32) mbar_arrive(&bar_st1);   // dv is staged: the loader stores it (async proxy)
+    if (ok && !full) flush_rows(sm + STG_V, grad_rows(p.dv), (size_t)H * D, x.len, kWideThreads);   // rows beyond the sequence must not be written
 
-    // ---- phase 4: dA = -stril(dXv U^T) (= -stril(dXk W^T + dXv U~^T), since dXk = T^T dW = -dXv h^T and U = U~ - W h),
-    // (dP.D) K, dXk = -dXv h^T; under the readout (dP.D)^T Q and U dh'^T
+    // ---- phase 3: dA = -stril(dXv U^T) ; under its readout [dO; dXv] h^T and dPD^T Q (rows on lanes 64..127)
     if (ok && issuer) {
         tc_fence_after();
-        mma_tile<64, 64, 128>(tmem + 384 + LB, op_k_major(sm + DXV, 64), op_mn_major(sm + UT, 128), false);         // dXv U^T
-        mma_tile<64, 128, 64>(tmem + 128, op_k_major(sm + DPD, 64), op_mn_major(sm + QK, 128, 64), false);          // (dP.D) K
-        mma_tile<64, 128, 128>(tmem + 256 + LB, op_k_major(sm + DXV, 64), op_k_major(sm + HH, 128), false, /*neg_a=*/true);   // dXk
-        mma_commit(&bar_mma);   // the two dk^col products are first read after the last phase
-        mma_tile<64, 128, 64>(tmem + 256, op_mn_major(sm + DPD, 64), op_mn_major(sm + QK, 128, 0), false);           // (dP.D)^T Q
-        mma_tile<64, 128, 128>(tmem + 0, op_mn_major(sm + UT, 128), op_k_major(sm + DH, 128), false);                // U dh'^T
-        mma_commit(&bar_ldh);   // h, dh' and dPD (over P) have been read for the last time
+        mma_commit(&bar_e1);   // U dh'^T is done: dh' has been read for the last time
+        mma_tile<64, 64, 128>(tmem + C_DA, op_k_major(sm + OX, 128, 64), op_mn_major(sm + UT, 128), false);
+        mma_commit(&bar_mma);
+        mma_tile<128, 128, 128>(tmem + C_A1, op_k_major(sm + OX, 128), op_k_major(sm + HH, 128), false);
+        mma_commit(&bar_e2);   // dO, dXv and h have been read for the last time
+        mma_tile<128, 128, 64>(tmem + C_C2, op_mn_major(sm + PG - 8192, 64), op_mn_major(sm + QT, 64), false);
     }
+    if (gates && has_next) make_gates(in_phase ^ 1);   // the next trip's gate arrays
     GDN_WAIT_MMA(24)
-    if (ok && worker) {
-        // group A: dq = scale Gam (dO h^T) + (dP.D) K, staged ; acc = <q, dq>
-        float acc = 0.f;
-        const float coef = sc * Gam[tr];
-#pragma unroll
-        for (int part = 0; part < 4; ++part) {
-            const int cb = cb0 + part * 8;
-            float a[8], b[8], t8[8];
-            tmem_ld8(tmem + lane_base + 384 + cb, a);     // A: dO h^T
-            tmem_ld8(tmem + lane_base + 128 + cb, b);     // A: (dP.D) K
-            tmem_wait_ld();
-            if (ga) {
-                unpack8(*reinterpret_cast<const uint4*>(sm + QK + tile_chunk_off(128, tr, cb >> 3)), t8);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    b[j] = fmaf(coef, a[j], b[j]);
-                    acc = fmaf(t8[j], b[j], acc);
-                }
-                chunk_store(sm + STG_A, 64, tr, cb >> 3, b);
-            }
-        }
-        if (ga) red[0][grp][tr] = acc;
-        // group B: G = dA . D and Diag(b) G (over dXv, which the products above have read)
+    if (ok && worker) {   // G = dA . D and Diag(b) G (over T and P, which no product reads any more)
         float v2[2][8];
-        tmem_ld8(tmem + lane_base + 384 + j0b, v2[0]);
-        tmem_ld8(tmem + lane_base + 384 + j0b + 8, v2[1]);
+        tmem_ld8(tmem + lane_base + C_DA + i0, v2[0]);
+        tmem_ld8(tmem + lane_base + C_DA + i0 + 8, v2[1]);
         tmem_wait_ld();
-        if (!ga) {
+        if (ga) {
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float (&v)[8] = v2[part];
                 float w[8], g8[8];
-                const int jb = j0b + part * 8;
+                const int jb = i0 + part * 8;
                 ld8s(gl + jb, g8);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     v[j] = (jb + j < tr) ? -v[j] * ex2(gl[tr] - g8[j]) : 0.f;
                     w[j] = bb[tr] * v[j];
                 }
-                chunk_store(sm + GT, 64, tr, jb >> 3, v);
+                chunk_store(sm + PG, 128, 64 + tr, jb >> 3, v);
                 chunk_store(sm + BGT, 64, tr, jb >> 3, w);
             }
         }
@@ -1445,78 +1432,98 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_intra_kernel(const _
     tc_fence_before();
     fence_async_smem();
     cta_sync();
-    if (threadIdx.x == 32) mbar_arrive(&bar_st1);   // dq, dv are staged: the loader stores them (async proxy)
-    if (ok && !full) {   // ragged tail: rows beyond the sequence must not be written
-        flush_rows(sm + STG_A, grad_rows(p.dq), (size_t)H * D, x.len, kIntraThreads);
-        flush_rows(sm + STG_B, grad_rows(p.dv), (size_t)H * D, x.len, kIntraThreads);
-    }
+    if (threadIdx.x == 32) mbar_arrive(&bar_v);     // the flush of a ragged dv is done
 
-    // ---- phase 5: G K ; += (Diag(b) G)^T K
+    // ---- phase 4: [dPD; G] K ; += (Diag(b) G)^T K
     if (ok && issuer) {
         tc_fence_after();
-        mma_commit(&bar_ld1);   // Q has been read for the last time (by (dP.D)^T Q and by the readout before this phase)
-        mma_tile<64, 128, 64>(tmem + 384, op_k_major(sm + GT, 64), op_mn_major(sm + QK, 128, 64), false);            // G K
-        mma_tile<64, 128, 64>(tmem + 256, op_mn_major(sm + BGT, 64), op_mn_major(sm + QK, 128, 64), true);           // += (bG)^T K
+        mma_tile<128, 128, 64>(tmem + C_A2, op_k_major(sm + PG, 128), op_mn_major(sm + KT, 64), false);
+        mma_tile<128, 128, 64>(tmem + C_C2, op_mn_major(sm + BGT - 8192, 64), op_mn_major(sm + KT, 64), true);
         mma_commit(&bar_mma);
-        mma_commit(&bar_ld2);   // G (over dXv, over dO) and T have been read for the last time
+        mma_commit(&bar_e3);   // every product of this trip is done
     }
     GDN_WAIT_MMA(26)
-    if (worker) {   // this thread's K values leave shared memory now, so that the next trip's K can be loaded over them
-        uint4 kraw[4];
+    if (worker) {
+        // Warps of quadrants 0, 1 (lanes 0..63) assemble dq = scale Gam (dO h^T) + dPD K, those of quadrants 2, 3
+        // dk = Diag(b)(G K - Gam dXv h^T) + e U dh'^T + dPD^T Q + (Diag(b) G)^T K, and the row dots.
+        const bool is_k = q4 >= 2;
+        const int i = (q4 & 1) * 32 + lane, c0 = grp * 32;
+        uint4 raw[4];   // this thread's part of its row of K or Q leaves shared memory now: the next trip's is loaded over it
 #pragma unroll
         for (int part = 0; part < 4; ++part)
-            kraw[part] = *reinterpret_cast<const uint4*>(sm + QK + tile_chunk_off(128, 64 + tr, (cb0 >> 3) + part));
+            raw[part] = *reinterpret_cast<const uint4*>(sm + (is_k ? KT : QT) + tile_chunk_off(64, i, (c0 >> 3) + part));
         __syncwarp();
-        if (lane == 0) mbar_arrive(&bar_kfree);
-        // Group A assembles dk = Diag(b)(G K + Gam dXk) + dk^col and both row dots with k; the lanes of group B hold
-        // nothing of this phase (Diag(b) G K is a row scaling of G K, so one product serves dk and db).
-        float acc_col = 0.f, acc_db = 0.f;   // <k, dk^col> ; db = <k, G K + Gam dXk>
-        const float e6 = ee[tr], G6 = Gam[tr], b6 = bb[tr];
-        if (ok) {
+        if (lane == 0) mbar_arrive(&bar_kq);
+        const float G = Gam[i];
+        if (ok && !is_k) {
+            float acc = 0.f;
+            const float coef = sc * G;
 #pragma unroll
-        for (int part = 0; part < 4; ++part) {
-            const int cb = cb0 + part * 8;
-            float a[8], b[8], c8[8], d8[8], kk[8];
-            tmem_ld8(tmem + lane_base + 384 + cb, a);     // A: G K
-            tmem_ld8(tmem + lane_base + 256 + cb, c8);    // A: (dP.D)^T Q + (bG)^T K      B: dXk
-            tmem_ld8(tmem + lane_base + 0 + cb, d8);      // A: U dh'^T
-            tmem_wait_ld();
+            for (int part = 0; part < 4; ++part) {
+                const int cb = c0 + part * 8;
+                float a[8], b[8], t8[8];
+                tmem_ld8(tmem + lane_base + C_A1 + cb, a);     // dO h^T
+                tmem_ld8(tmem + lane_base + C_A2 + cb, b);     // dPD K
+                tmem_wait_ld();
+                unpack8(raw[part], t8);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) b[j] = __shfl_down_sync(0xffffffffu, c8[j], 16);   // dXk of this token row comes over from group B
-            if (ga) {
-                unpack8(kraw[part], kk);
+                for (int j = 0; j < 8; ++j) {
+                    b[j] = fmaf(coef, a[j], b[j]);
+                    acc = fmaf(t8[j], b[j], acc);
+                }
+                chunk_store(sm + STG_Q, 64, i, cb >> 3, b);
+            }
+            red[0][grp][i] = acc;     // <q, dq>
+        } else if (ok) {
+            float acc_col = 0.f, acc_db = 0.f;   // <k, dk^col> ; db = <k, G K + Gam dXk>
+            const float e6 = ee[i], b6 = bb[i];
+#pragma unroll
+            for (int part = 0; part < 4; ++part) {
+                const int cb = c0 + part * 8;
+                float a[8], b[8], c8[8], d8[8], kk[8];
+                tmem_ld8(tmem + lane_base + C_A2 + cb, a);     // G K
+                tmem_ld8(tmem + lane_base + C_A1 + cb, b);     // dXv h^T = -dXk
+                tmem_ld8(tmem + lane_base + C_C2 + cb, c8);    // dPD^T Q + (bG)^T K
+                tmem_ld8(tmem + lane_base + C_UH + cb, d8);    // U dh'^T
+                tmem_wait_ld();
+                unpack8(raw[part], kk);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const float kcol = fmaf(e6, d8[j], c8[j]);       // dk^col
-                    const float t = fmaf(G6, b[j], a[j]);            // G K + Gam dXk
+                    const float t = fmaf(-G, b[j], a[j]);            // G K + Gam dXk
                     acc_col = fmaf(kk[j], kcol, acc_col);
                     acc_db = fmaf(kk[j], t, acc_db);
                     a[j] = fmaf(b6, t, kcol);
                 }
-                chunk_store(sm + STG_K, 64, tr, cb >> 3, a);
+                chunk_store(sm + STG_K, 64, i, cb >> 3, a);
             }
+            red[2][grp][i] = acc_db;
+            red[3][grp][i] = acc_col;
         }
-        }
-        if (ga) { red[2][grp][tr] = acc_db; red[3][grp][tr] = acc_col; }
+        // block totals of sum_j r_j and <dh', h>
+        rs = warp_sum(rs);
+        hh = warp_sum(hh);
+        if (lane == 0) { scal[0][warp] = rs; scal[1][warp] = hh; }
     }
-    // block totals of sum_j r_j and <dh', h>
-    rs = warp_sum(rs);
-    hh = warp_sum(hh);
-    if (lane == 0) { scal[0][warp] = rs; scal[1][warp] = hh; }
-    fence_async_smem();
-    cta_sync();
-    if (threadIdx.x == 32) mbar_arrive(&bar_st2);   // dk is staged: the loader stores it
-    if (ok && !full) flush_rows(sm + STG_K, grad_rows(p.dk), (size_t)H * D, x.len, kIntraThreads);
-    // The token-wise sums are complete; turning them into dbeta and dg is left to warps 0 and 1 during the next trip's
-    // first products (finish_gates).  They keep what the next trip overwrites: this chunk's gates and place.
-    if (threadIdx.x < kC) { bb_prev = bb[threadIdx.x]; Gam_last_prev = Gam[kC - 1]; }
+    // The token-wise sums are turned into dbeta and dg by the gate warp during the next trip's first products.  It keeps what
+    // the next trip overwrites: this chunk's gates and place.
+    if (gates) {
+        bb_prev[0] = bb[lane]; bb_prev[1] = bb[lane + 32];
+        Gam_last_prev = Gam[kC - 1];
+    }
     xp = x;
     have_prev = true;
     tc_fence_before();
+    fence_async_smem();
     cta_sync();   // every reader of this trip's tiles and scratch is done
+    if (threadIdx.x == 32) mbar_arrive(&bar_st2);   // dq, dk are staged: the loader stores them
+    if (ok && !full) {
+        flush_rows(sm + STG_Q, grad_rows(p.dq), (size_t)H * D, x.len, kWideThreads);
+        flush_rows(sm + STG_K, grad_rows(p.dk), (size_t)H * D, x.len, kWideThreads);
+    }
     if (!ok) break;
     }
-    if (ok && have_prev && warp < 2) finish_gates();
+    if (ok && have_prev && gates) finish_gates();
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
@@ -1818,7 +1825,7 @@ static cudaError_t launch_scan(const TcParams& P, cudaStream_t st) {
 static cudaError_t launch_intra(const TcParams& P, cudaStream_t st) {
     static SmemLimitOnce done;
     const int items = P.p.L.max_chunks * P.p.d.H, sms = sm_count();
-    return launch_chunk_kernel(tc_intra_kernel, done, intra::SMEM_BYTES, ST_INTRA, items < sms ? items : sms, kIntraThreads + 32, P, st);
+    return launch_chunk_kernel(tc_intra_kernel, done, intra::SMEM_BYTES, ST_INTRA, items < sms ? items : sms, intra::kThreadsAll, P, st);
 }
 static cudaError_t launch_out(const TcParams& P, cudaStream_t st) {
     static SmemLimitOnce done;
