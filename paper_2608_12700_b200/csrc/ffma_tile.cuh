@@ -177,22 +177,11 @@ __device__ __forceinline__ float* block_of(const Problem& p, size_t region, int 
     return reinterpret_cast<float*>(p.ws + region) + (size_t)ch * floats;
 }
 
-// T = (I + A)^-1, blocked; S is scratch.  Everybody takes part; the caller synchronises afterwards.
-__device__ __forceinline__ void invert(const float* A, float* T, float* S) {
+// T = (I + A)^-1 with a clean upper right quadrant.  Everybody takes part; the caller synchronises afterwards.
+__device__ __forceinline__ void invert(const float* A, float* T) {
     static_assert(kPc == kLdi, "the inversion works on the tiles of this family");
-    for (int e = threadIdx.x; e < kC * kC; e += kThreads)   // the blocks above the block diagonal are not written by the steps below
-        if ((e % kC) / 16 > e / kC / 16) T[(e / kC) * kPc + e % kC] = 0.f;
-    inv_diag8(A, T);
-    __syncthreads();
-    inv_diag16(A, T, S);
-    __syncthreads();
-    inv_premul<2>(A, T, S);
-    __syncthreads();
-    inv_level<1, 1, 2>(S, T);
-    __syncthreads();
-    inv_level<2, 2, 2>(S, T);
-    __syncthreads();
-    inv_level<3, 4, 2>(S, T);
+    invert64(A, T, [] { __syncthreads(); });
+    for (int e = threadIdx.x; e < 32 * 32; e += kThreads) T[(e >> 5) * kPc + 32 + (e & 31)] = 0.f;
 }
 
 // Which part of the preparation a launch makes: the forward's, that and the backward's, the backward's alone.

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) 
     float* sO = sV + kC * pitch(DK > DV ? DK : DV);   // dO
     float* A = sO + kC * PV;                          // A, then T Diag(w)
     float* T = A + kC * kPc;
-    float* S = T + kC * kPc;                          // scratch of the inversion, then T Diag(b Gam)
+    float* S = T + kC * kPc;                          // T Diag(b Gam)
     float* Pm = S + kC * kPc;
     __shared__ Gates gs;
     const int H = p.d.H, tid = threadIdx.x;
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) 
             *reinterpret_cast<float4*>(wsKb + (size_t)e * 4) = make_float4(w * k.x, w * k.y, w * k.z, w * k.w);
         }
         __syncthreads();
-        invert(A, T, S);
+        invert(A, T);
         cp_wait<0>();
         __syncthreads();
         float* wsT = block_of(p, p.L.Tm, x.ch, kC * kC);

@@ -83,12 +83,12 @@ __device__ __forceinline__ void make_copies(float* C, const float* G, const Refs
 // ------------------------------------------------------------------------------------------------
 template <int DK, int DV>
 struct PrepTiles {
-    static constexpr int PM = pitch(DK > DV ? DK : DV), COPY = 96 * pitch(DK) > 2 * kC * kPc ? 96 * pitch(DK) : 2 * kC * kPc;
+    static constexpr int PM = pitch(DK > DV ? DK : DV), COPY = 96 * pitch(DK);
     static constexpr int G = 0;                       // gam, then dO
     static constexpr int Q = G + kC * PM;             // q, scaled, then X = Gam . Q - P W
     static constexpr int K = Q + kC * pitch(DK);      // k, then Gam . b . K
     static constexpr int R = K + kC * pitch(DK);      // b . k, scaled, then w . V, then W
-    static constexpr int C = R + kC * PM;             // scaled copies of the keys, then T and scratch
+    static constexpr int C = R + kC * PM;             // scaled copies of the keys, then T
     static constexpr int A = C + COPY;
     static constexpr int P = A + kC * kPc;
     static constexpr size_t BYTES = sizeof(float) * (P + kC * kPc);
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kThreads, 1) vprep_kernel(Problem p, int mode)
     constexpr int PK = pitch(DK), PV = pitch(DV);
     extern __shared__ __align__(16) float sm[];
     float *G = sm + L::G, *Q = sm + L::Q, *K = sm + L::K, *R = sm + L::R, *C = sm + L::C, *A = sm + L::A, *Pm = sm + L::P;
-    float *T = C, *S = C + kC * kPc, *O = G;
+    float *T = C, *O = G;
     __shared__ Refs<DK> refs;
     const bool fwd = mode != PREP_BWD, bwd = mode != PREP_FWD;
     const int H = p.d.H, tid = threadIdx.x;
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kThreads, 1) vprep_kernel(Problem p, int mode)
         if (bwd) load_rows<DV>(O, rows_of<IO>(p.dO, x, H, DV), rv, x.len);
         cp_commit();
         for (int e = tid; e < kC * kC; e += kThreads) wsP[e] = Pm[(e / kC) * kPc + e % kC];
-        invert(A, T, S);
+        invert(A, T);
         cp_wait<1>();
         __syncthreads();
         float* wsT = block_of(p, p.L.Tm, x.ch, kC * kC);

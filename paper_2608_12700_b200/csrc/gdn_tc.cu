@@ -60,7 +60,7 @@ constexpr uint32_t TT = 65536;                // T                      [64][64]
 constexpr uint32_t TP = TT + 8192;            // T Diag(b Gam)                                    the Nm image)
 constexpr uint32_t TPP = TP + 8192;           // T Diag(w)
 constexpr uint32_t PT = TPP + 8192;           // P = tril(Q K^T . D)
-constexpr uint32_t WT = PT + 8192;            // W^T   [128 dk][64 tokens]                16 KB (before: fp32 scratch S)
+constexpr uint32_t WT = PT + 8192;            // W^T   [128 dk][64 tokens]                16 KB
 constexpr uint32_t UTT = WT + 16384;          // U~^T  [128 dv][64]
 constexpr uint32_t WET = UTT + 16384;         // (Diag(e) W)^T                                    (these two: finally
 constexpr uint32_t UET = WET + 16384;         // (Diag(e) U~)^T                                   the Bf image)
@@ -308,7 +308,6 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     if (threadIdx.x == 32) mbar_arrive(&bar_ld0);   // this trip's inputs have arrived
     float* Af = reinterpret_cast<float*>(sm + XA);   // [64][kLdi]  strictly lower part of I + A
     float* Tf = reinterpret_cast<float*>(sm + XT);   // [64][kLdi]  T
-    float* Sf = reinterpret_cast<float*>(sm + WT);   // [64][kLdi]  scratch of the blocked inversion
     if (has_next && warp == 0) fetch_gates(xn);   // next trip's gates -> registers while the product runs
     // R = Diag(Gam) dO (token-major tile) while the product runs.  In low-rank mode the tiles of Diag(e) W and
     // Diag(e) U~ are never written, so R has a tile of its own from here on and Q^T R can run under the inversion.
@@ -367,23 +366,12 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
         // low-rank mode: so does the first half of E = Q^T R - W^T (P^T dO), into columns no other product uses
         if (!opform) mma_tile<128, 128, 64>(tmem + C_E_LR, op_mn_major(sm + QK, 128, 0), op_mn_major(sm + WET, 64), false);
     }
-    // ---- T = (I + A)^-1, blocked (see inv_diag8 ... inv_level).  All fp32.
+    // ---- T = (I + A)^-1, blocked, fp32 (invert64)
     if (ok && !first) {   // ... and what lies under the fp32 T block
         ok = mbar_wait(&bar_free2, in_phase ^ 1);
         if (!ok && threadIdx.x == 0) report_timeout(p.ws, 8);
     }
-    inv_diag8(Af, Tf);
-    cta_sync();
-    inv_diag16(Af, Tf, Sf);
-    cta_sync();
-    inv_premul<2>(Af, Tf, Sf);   // Sf <- T_rr A_rk for every block below the diagonal
-    cta_sync();
-    inv_level<1, 1, 2>(Sf, Tf);
-    cta_sync();
-    inv_level<2, 2, 2>(Sf, Tf);
-    cta_sync();
-    inv_level<3, 4, 2>(Sf, Tf);
-    cta_sync();
+    invert64(Af, Tf, cta_sync);
     if (ok && !first) {   // every store of the previous trip has read its tile (the T tiles and the second readout are next)
         ok = mbar_wait(&bar_free, in_phase ^ 1);
         if (!ok && threadIdx.x == 0) report_timeout(p.ws, 5);

@@ -177,8 +177,7 @@ constexpr uint32_t VT = KM + 16384;         // V~ [64][128]                     
 constexpr uint32_t DOT = VT + 16384;        // dO' [64][128]                                    16 KB
 constexpr uint32_t XA = DOT + 16384;        // fp32 A [64][kLdi]
 constexpr uint32_t XT = XA + 17408;         // fp32 T
-constexpr uint32_t SF = XT + 17408;         // fp32 scratch of the inversion
-constexpr uint32_t TT = SF + 17408;         // T  bf16 [64][64]                                  8 KB
+constexpr uint32_t TT = XT + 17408;         // T  bf16 [64][64]                                  8 KB
 constexpr uint32_t PT = TT + 8192;          // P  bf16 [64][64]                                  8 KB
 constexpr uint32_t WT = PT + 8192;          // W^T  [128][64]                                   16 KB
 constexpr uint32_t UTT = WT + 16384;        // U~^T [128][64]                                   16 KB
@@ -186,7 +185,7 @@ constexpr uint32_t PDOT = UTT + 16384;      // (P^T dO')^T [128][64]            
 constexpr uint32_t EST = XA;                // staged E image [128][128] over the fp32 A and T blocks                       32 KB
 constexpr uint32_t SMEM_BYTES = PDOT + 16384 + 1024;
 constexpr uint32_t C_S1 = 0, C_W = 64, C_U = 128, C_PDO = 192, C_E = 256;   // TMEM columns (512 allocated)
-static_assert(EST % 1024 == 0 && EST + 32768 <= SF + 17408, "the E image fits over the inversion's scratch");
+static_assert(EST % 1024 == 0 && EST + 32768 <= TT, "the E image fits over the fp32 A and T blocks");
 static_assert(TT % 1024 == 0 && SMEM_BYTES <= 225 * 1024, "tile alignment and shared memory budget");
 }  // namespace prepcw
 
@@ -215,12 +214,11 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
     const uint32_t tmem = tmem_slot;
     float* Af = reinterpret_cast<float*>(sm + XA);
     float* Tf = reinterpret_cast<float*>(sm + XT);
-    float* Sf = reinterpret_cast<float*>(sm + SF);
     const bool bwd = mode != 0, fresh = mode == 2;
     bool ok = true, pending = false;
     uint32_t mma_phase = 0, in_phase = 0, pending_phase = 0;   // (pending_phase: the phase of bar_in the loads in flight belong to)
     // The tiles of a trip arrive in two pieces on one mbarrier phase, each issued during the trip before as soon as the
-    // last product that reads its region is done (E is staged over the inversion's scratch, never over an input tile):
+    // last product that reads its region is done (E is staged over the fp32 A and T blocks, never over an input tile):
     //   closed / forward:  a = K-                     after step 1      b = [Q~; K+], V~, dO'     after step 2
     //   fresh workspace:   a = Q~, dO', stored P      after its first products      b = stored W^T   after step 3
     auto load_a = [&](size_t c, uint32_t phase) {   // thread 0; the first piece announces the whole trip's bytes
@@ -320,18 +318,7 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
             mma_tile<128, 128, 64>(tmem + C_E, op_mn_major(sm + QKP, 128, 0), op_mn_major(sm + DOT, 64), false);
         }
         // ---- T = (I + A)^-1, blocked, fp32
-        inv_diag8(Af, Tf);
-        __syncthreads();
-        inv_diag16(Af, Tf, Sf);
-        __syncthreads();
-        inv_premul<2>(Af, Tf, Sf);
-        __syncthreads();
-        inv_level<1, 1, 2>(Sf, Tf);
-        __syncthreads();
-        inv_level<2, 2, 2>(Sf, Tf);
-        __syncthreads();
-        inv_level<3, 4, 2>(Sf, Tf);
-        __syncthreads();
+        invert64(Af, Tf, [] { __syncthreads(); });
         {   // T -> bf16 tile: a thread converts two rows of one 8-column piece
             const int cch = threadIdx.x & 7;
 #pragma unroll
@@ -390,7 +377,7 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
             }
             GDN_WAIT_MMA(43)
             if (ok && fresh && has_next && threadIdx.x == 0) load_b(chn);   // W^T has been read for the last time
-            if (ok) {   // E -> bf16 tile image, staged over the scratch of the inversion (dead since T was converted)
+            if (ok) {   // E -> bf16 tile image, staged over the fp32 A and T blocks (dead since T was converted)
                 const int r = q4 * 32 + lane, c0 = grp * 64;
 #pragma unroll 1
                 for (int part = 0; part < 8; ++part) {

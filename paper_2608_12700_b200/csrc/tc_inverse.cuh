@@ -1,112 +1,113 @@
 // fp32 blocked inversion of a unit lower triangular 64 x 64 matrix in shared memory (T = (I + A)^-1 of the chunk-local
-// solve, Section 4.2), shared by every kernel family.  Thread indices are those of the calling CTA; every step
-// uses at most its first 256 threads, and the caller separates the steps by CTA-wide barriers.
+// solve, Section 4.2), shared by every kernel family.  The first 256 threads of the calling CTA work; all of them have to
+// call, because the steps are separated by the caller's CTA-wide barrier.
 #pragma once
 #include "gdn_internal.cuh"
 
 namespace gdn {
 namespace {
 
-constexpr int kInvMaxThreads = 512;   // bound used by the static checks of the level passes
+// Rows of kLdi floats: 16-byte aligned, eight consecutive rows on distinct banks.
+constexpr int kLdi = 68;
 
-// Blocked inverse of I + A (unit lower triangular), fp32 in shared memory, rows of kLdi floats:
-//   diagonal 8 x 8 blocks by forward substitution; the 8 x 8 block below the diagonal of every 16 x 16 diagonal block
-//   from T10 = -T11 (A10 T00); then with 16 x 16 blocks  At_rk = T_rr A_rk (r > k)  and
-//   T_rc = -sum_{k=c}^{r-1} At_rk T_kc, one block diagonal at a time.
-// These steps are chains of dependent FMAs fed by shared-memory loads, so a thread produces four adjacent outputs of a
-// row (one broadcast scalar and one 16-byte load feed four FMAs) and the longer sums are split over SPLIT adjacent
-// lanes and combined by shuffles.
-constexpr int kLdi = 68;   // row pitch: 16-byte aligned rows, conflict-free for the access patterns below
-__device__ __forceinline__ void inv_diag8(const float* Af, float* Tf) {   // threads 0..63: column j of block b0
-    if (threadIdx.x < kC) {   // t_i = [i == j] - sum_{m<i} A_im t_m
-        const int b0 = (threadIdx.x >> 3) * 8, j = threadIdx.x & 7;
-        float t[8];
+// A chain of dependent steps on one small matrix: what bounds it is latency (barriers, shared-memory loads, FMA chains) and the
+// shared-memory pipe, hence few steps and register tiles.  The inverse doubles its block size twice:
+//   1  the four 16 x 16 diagonal blocks, one per warp, a column per lane, forward substitution in registers
+//   2  X = A10 T00, 3  T10 = -T11 X                 for the two pairs of 16 x 16 blocks
+//   4  Y = A10 T00, 5  T10 = -T11 Y                 for the pair of 32 x 32 blocks
+// X and Y lie in the upper right 32 x 32 quadrant of T and Y is left there (consumers take that quadrant as zero); the other
+// blocks above the block diagonal are zeroed.
+// In steps 2 to 5 a thread multiplies a 4 x 4 tile over a quarter of the contraction; the four partial tiles are added by two
+// exchanges that also leave every lane with one row of four results.
+// (Against 8 x 8 diagonal blocks, six barriers and rows of four outputs per thread, whole calls: backward of 16 heads of 16384
+// tokens 643 -> 626 us, of 4 x 16 heads of 2048 tokens 281 -> 277 us, forward and backward of 6 x 16 x 1500 380 -> 374 us.)
+__device__ __forceinline__ void inv_diag16(const float* A, float* T) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp < 4 && lane < 16) {   // t_i = [i == j] - sum_{m<i} A_im t_m
+        const float* a = A + (warp * 16) * kLdi + warp * 16;
+        float t[16];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            float s = (i == j) ? 1.f : 0.f;
+        for (int i = 0; i < 16; ++i) {
+            float s0 = (i == lane) ? 1.f : 0.f, s1 = 0.f;
 #pragma unroll
-            for (int m = 0; m < i; ++m) s = fmaf(-Af[(b0 + i) * kLdi + b0 + m], t[m], s);
-            t[i] = s;
-            Tf[(b0 + i) * kLdi + b0 + j] = s;
+            for (int m = 0; m < i; m += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(a + i * kLdi + m);
+                s0 = fmaf(-v.x, t[m], s0);
+                if (m + 1 < i) s1 = fmaf(-v.y, t[m + 1], s1);
+                if (m + 2 < i) s0 = fmaf(-v.z, t[m + 2], s0);
+                if (m + 3 < i) s1 = fmaf(-v.w, t[m + 3], s1);
+            }
+            t[i] = s0 + s1;
+            T[(warp * 16 + i) * kLdi + warp * 16 + lane] = t[i];
         }
+    } else if (warp == 0 || warp == 2) {   // lanes 16..31: the block right of the diagonal block
+#pragma unroll
+        for (int i = 0; i < 16; ++i) T[(warp * 16 + i) * kLdi + warp * 16 + lane] = 0.f;
     }
 }
-__device__ __forceinline__ void inv_diag16(const float* Af, float* Tf, float* Xf) {   // threads 0..255: one entry each
-    if (threadIdx.x < 256) {
-        const int r0 = (threadIdx.x >> 6) * 16, i = (threadIdx.x >> 3) & 7, j = threadIdx.x & 7;
-        float x = 0.f;   // X = A10 T00
+// D = (NEG ? -1 : 1) * A B, [4 rows of this lane's group x 4 columns] over 4 * STEPS indices from this lane's k0 on, summed
+// over the four lanes that differ in the bits KS and 2 KS of the lane index (q: this lane's two bits); lane q stores row q.
+template <int STEPS, int KS, bool NEG>
+__device__ __forceinline__ void inv_tile(const float* A, const float* B, float* D, int k0, int q) {
+    float acc[4][4] = {};
 #pragma unroll
-        for (int m = 0; m < 8; ++m) x = fmaf(Af[(r0 + 8 + i) * kLdi + r0 + m], Tf[(r0 + m) * kLdi + r0 + j], x);
-        Xf[(r0 + 8 + i) * kLdi + r0 + j] = x;
-        asm volatile("bar.sync 4, 256;" ::: "memory");
-        float s = 0.f;   // T10 = -T11 X
+    for (int s = 0; s < STEPS; ++s) {
+        const int k = k0 + 4 * s;
+        float4 a[4], b[4];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) s = fmaf(Tf[(r0 + 8 + i) * kLdi + r0 + 8 + k], Xf[(r0 + 8 + k) * kLdi + r0 + j], s);
-        Tf[(r0 + 8 + i) * kLdi + r0 + j] = -s;     // (disjoint from T00 and T11, which other threads still read)
-        Tf[(r0 + i) * kLdi + r0 + 8 + j] = 0.f;    // the block above the diagonal
-    }
-}
-// R rows of a block per thread: the 16-byte load of a row of A feeds R x 4 FMAs (these steps are bound by the number of
-// shared-memory wavefronts, and a 16-byte load costs a warp four of them however many lanes share an address).
-template <int R>
-__device__ __forceinline__ void inv_premul(const float* Af, const float* Tf, float* Sf) {
-    // six blocks below the diagonal: (1,0) (2,0) (2,1) (3,0) (3,1) (3,2); per block 16 / R row groups x 4 column groups
-    constexpr int per_blk = (16 / R) * 4;
-    if (threadIdx.x < 6 * per_blk) {
-        const int o = threadIdx.x, blk = o / per_blk, ig = (o % per_blk) >> 2, j4 = (o & 3) * 4;
-        const int rb = (blk == 0 ? 1 : blk < 3 ? 2 : 3) * 16, cb = (blk == 0 ? 0 : blk < 3 ? blk - 1 : blk - 3) * 16;
-        float4 s[R];
+        for (int z = 0; z < 4; ++z) {
+            a[z] = *reinterpret_cast<const float4*>(A + z * kLdi + k);
+            b[z] = *reinterpret_cast<const float4*>(B + (k + z) * kLdi);
+        }
 #pragma unroll
-        for (int q = 0; q < R; ++q) s[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int r = 0; r < 4; ++r) {
+            const float w[4] = {a[r].x, a[r].y, a[r].z, a[r].w};
 #pragma unroll
-        for (int m = 0; m < 16; ++m) {   // T_rr is lower triangular: zeros above the diagonal
-            const float4 v = *reinterpret_cast<const float4*>(Af + (rb + m) * kLdi + cb + j4);
-#pragma unroll
-            for (int q = 0; q < R; ++q) {   // rows ig, ig + 16 / R, ...: a warp's scalar loads fall into distinct banks
-                const float a = Tf[(rb + ig + q * (16 / R)) * kLdi + rb + m];
-                s[q].x = fmaf(a, v.x, s[q].x); s[q].y = fmaf(a, v.y, s[q].y); s[q].z = fmaf(a, v.z, s[q].z); s[q].w = fmaf(a, v.w, s[q].w);
+            for (int z = 0; z < 4; ++z) {
+                acc[r][0] = fmaf(w[z], b[z].x, acc[r][0]);
+                acc[r][1] = fmaf(w[z], b[z].y, acc[r][1]);
+                acc[r][2] = fmaf(w[z], b[z].z, acc[r][2]);
+                acc[r][3] = fmaf(w[z], b[z].w, acc[r][3]);
             }
         }
-#pragma unroll
-        for (int q = 0; q < R; ++q) *reinterpret_cast<float4*>(Sf + (rb + ig + q * (16 / R)) * kLdi + cb + j4) = s[q];
     }
-}
-template <int DIST, int SPLIT, int R>
-__device__ __forceinline__ void inv_level(const float* At, float* Tf) {
-    constexpr int items = (4 - DIST) * (16 / R) * 4, len = 16 * DIST / SPLIT;
-    static_assert(items * SPLIT <= kInvMaxThreads && (items * SPLIT) % 32 == 0, "one pass, whole warps");
-    if (threadIdx.x < items * SPLIT) {
-        // a warp serves 32 / SPLIT items; the lanes of a quarter-warp share `part`, so their 16-byte loads fall into one
-        // row of T (no bank conflicts), and the partial sums of an item sit 32 / SPLIT lanes apart
-        constexpr int G = 32 / SPLIT, per_blk = (16 / R) * 4;
-        const int wl = threadIdx.x & 31, o = (threadIdx.x >> 5) * G + (wl % G), part = wl / G;
-        const int cb = (o / per_blk) * 16, rb = cb + DIST * 16, ig = (o % per_blk) >> 2, j4 = (o & 3) * 4;
-        float4 s[R];
+    // rows 0, 1 go to the lanes with bit 2 KS clear, rows 2, 3 to the others; then one row each
+    const bool hi = (q & 2) != 0, odd = (q & 1) != 0;
+    float h[2][4], r4[4];
 #pragma unroll
-        for (int q = 0; q < R; ++q) s[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int r = 0; r < 2; ++r)
 #pragma unroll
-        for (int mm = 0; mm < len; ++mm) {
-            const int m = part * len + mm;
-            const float4 v = *reinterpret_cast<const float4*>(Tf + (cb + m) * kLdi + cb + j4);
-#pragma unroll
-            for (int q = 0; q < R; ++q) {
-                const float a = At[(rb + ig + q * (16 / R)) * kLdi + cb + m];
-                s[q].x = fmaf(a, v.x, s[q].x); s[q].y = fmaf(a, v.y, s[q].y); s[q].z = fmaf(a, v.z, s[q].z); s[q].w = fmaf(a, v.w, s[q].w);
-            }
+        for (int y = 0; y < 4; ++y) {
+            const float send = hi ? acc[r][y] : acc[r + 2][y], keep = hi ? acc[r + 2][y] : acc[r][y];
+            h[r][y] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * KS);
         }
 #pragma unroll
-        for (int q = 0; q < R; ++q) {
-#pragma unroll
-            for (int d = G; d < 32; d <<= 1) {
-                s[q].x += __shfl_xor_sync(0xffffffffu, s[q].x, d); s[q].y += __shfl_xor_sync(0xffffffffu, s[q].y, d);
-                s[q].z += __shfl_xor_sync(0xffffffffu, s[q].z, d); s[q].w += __shfl_xor_sync(0xffffffffu, s[q].w, d);
-            }
-            if (part == 0)
-                *reinterpret_cast<float4*>(Tf + (rb + ig + q * (16 / R)) * kLdi + cb + j4) = make_float4(-s[q].x, -s[q].y, -s[q].z, -s[q].w);
-        }
+    for (int y = 0; y < 4; ++y) {
+        const float send = odd ? h[0][y] : h[1][y], keep = odd ? h[1][y] : h[0][y];
+        r4[y] = keep + __shfl_xor_sync(0xffffffffu, send, KS);
+        if (NEG) r4[y] = -r4[y];
     }
+    *reinterpret_cast<float4*>(D + q * kLdi) = make_float4(r4[0], r4[1], r4[2], r4[3]);
 }
-
+template <class Sync>
+__device__ __forceinline__ void invert64(const float* A, float* T, Sync sync) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    inv_diag16(A, T);
+    sync();
+    // pairs of 16 x 16 blocks: warps 0, 1 the first, warps 2, 3 the second; eight rows a warp, lane = (row group, quarter, columns)
+    const int pr = warp >> 1, p0 = pr * 32, r16 = (warp & 1) * 8 + (lane >> 4) * 4, q16 = (lane >> 2) & 3, c16 = (lane & 3) * 4;
+    float* X = T + (pr * 16) * kLdi + 32 + pr * 16;
+    if (warp < 4) inv_tile<1, 4, false>(A + (p0 + 16 + r16) * kLdi + p0, T + p0 * kLdi + p0 + c16, X + r16 * kLdi + c16, q16 * 4, q16);
+    sync();
+    if (warp < 4) inv_tile<1, 4, true>(T + (p0 + 16 + r16) * kLdi + p0 + 16, X + c16, T + (p0 + 16 + r16) * kLdi + p0 + c16, q16 * 4, q16);
+    sync();
+    // the pair of 32 x 32 blocks: four rows a warp, lane = (quarter, columns)
+    const int r32 = warp * 4, q32 = lane >> 3, c32 = (lane & 7) * 4;
+    if (warp < 8) inv_tile<2, 8, false>(A + (32 + r32) * kLdi, T + c32, T + r32 * kLdi + 32 + c32, q32 * 8, q32);
+    sync();
+    if (warp < 8) inv_tile<2, 8, true>(T + (32 + r32) * kLdi + 32, T + 32 + c32, T + (32 + r32) * kLdi + c32, q32 * 8, q32);
+    sync();
+}
 
 }  // namespace
 }  // namespace gdn

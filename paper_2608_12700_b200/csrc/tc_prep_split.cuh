@@ -23,7 +23,7 @@ namespace factors {
 constexpr uint32_t KV = 0;                  // [K rows 0..63 ; V rows 64..127] x 128          32 KB
 constexpr uint32_t XA = 32768;              // fp32 A [64][kLdi]; after the inversion the bf16 tiles T and T Diag(b Gam)
 constexpr uint32_t XT = XA + 17408;         // fp32 T [64][kLdi]
-constexpr uint32_t WU = XT + 17408;         // fp32 scratch of the inversion; later the staged images W^T | U~^T   32 KB
+constexpr uint32_t WU = XT + 17408;         // staged images W^T | U~^T                                      32 KB
 constexpr uint32_t TPP = WU + 32768;        // T Diag(w)                                       8 KB
 constexpr uint32_t TT = XA, TP = XA + 8192;
 constexpr uint32_t SMEM_BYTES = TPP + 8192 + 1024 /* alignment slack */;
@@ -61,7 +61,6 @@ __global__ void __launch_bounds__(split::kT, 2) tc_factors_kernel(const __grid_c
     const float* bgam = gates[5];
     float* Af = reinterpret_cast<float*>(sm + XA);
     float* Tf = reinterpret_cast<float*>(sm + XT);
-    float* Sf = reinterpret_cast<float*>(sm + WU);
     bool ok = true, pending = false;
     uint32_t mma_phase = 0, in_phase = 0;
     // K and V of a trip are dead once its last product is done, so the next trip's are loaded right then, under the last
@@ -158,18 +157,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_factors_kernel(const __grid_c
         tc_fence_before();
         __syncthreads();
         // ---- T = (I + A)^-1, blocked, fp32
-        inv_diag8(Af, Tf);
-        __syncthreads();
-        inv_diag16(Af, Tf, Sf);
-        __syncthreads();
-        inv_premul<2>(Af, Tf, Sf);
-        __syncthreads();
-        inv_level<1, 1, 2>(Sf, Tf);
-        __syncthreads();
-        inv_level<2, 2, 2>(Sf, Tf);
-        __syncthreads();
-        inv_level<3, 4, 2>(Sf, Tf);
-        __syncthreads();
+        invert64(Af, Tf, [] { __syncthreads(); });
         {   // T -> bf16 tiles T, T Diag(b Gam), T Diag(w): a thread scales two rows of one 8-column piece
             const int cch = threadIdx.x & 7;
             float gb8[8], gw8[8];
