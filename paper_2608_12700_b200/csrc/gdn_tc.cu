@@ -43,7 +43,7 @@ struct TcParams {
     CUtensorMap tm_o;                      // same geometry, for the forward output (forward calls that want it)
     int with_bwd;                          // prep: also produce E
     int scan_dirs;                         // scan: 0 = forward carry only, 1 = reverse only, 2 = both
-    int lowrank;                           // carries in low-rank form (tc_scan_lr): tc_prep makes no Nm, Bf
+    int lowrank;                           // carries in low-rank form (tc_scan_lr): prepared by tc_prep_lr / tc_factors without Nm, Bf
     int withhold;                          // debugging hook: tc_prep leaves out one of its first loads, so that the wait
                                            // for it runs out (exercises the time-out path without any fault)
 };
@@ -73,7 +73,6 @@ constexpr uint32_t SMEM_BYTES = TILES_END + 1024 /* alignment slack */;
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
 // TMEM columns (512 allocated): accumulators at fixed offsets, allocated once, released once.
 constexpr uint32_t C_S1 = 0, C_W = 64, C_U = 128, C_PDO = 192, C_NM = 256, C_BF = 384, C_E = 0;
-constexpr uint32_t C_E_LR = 256;   // low-rank mode (no Nm, Bf): E is started early, in columns of its own
 }  // namespace prep
 
 __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __grid_constant__ TcParams P) {
@@ -87,7 +86,6 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     const int n_items = n_chunks_of(p) * H;
     if ((int)blockIdx.x >= n_items) return;
     const bool bwd = P.with_bwd != 0;
-    const bool opform = P.lowrank == 0;   // the carries want the chunk operator Nm and the additive term Bf
 
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sm = align1024(smem_raw);
@@ -157,15 +155,6 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
                 bulk_store(p.ws + p.L.Tm + (size_t)x.ch * 8192, sm + TT, 8192);
                 if (bwd) bulk_store(p.ws + p.L.Pm + (size_t)x.ch * 8192, sm + PT, 8192);   // the gradient stage reads P from here
                 bulk_commit();
-                if (!opform) {   // low-rank mode: Q, K are dead after phase 2, before W^T, U~^T are staged
-                    if (!(lok = mbar_wait(&bar_ld1, ph))) break;
-                    if (has_next) {
-                        mbar_expect_tx(&bar_qk, 32768);
-                        pend_qk = true;
-#pragma unroll 1
-                        for (int piece = 0; piece < 4; ++piece) load_piece(piece, nx);
-                    }
-                }
                 // W^T, U~^T are staged and V, dO have been read for the last time
                 if (!(lok = mbar_wait(&bar_vofree, ph))) break;
                 bulk_wait_read<0>();
@@ -180,8 +169,8 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
                 bulk_store(p.ws + p.L.Ut + (size_t)x.ch * 16384, sm + UTT, 16384);
                 bulk_commit();
                 // phase 3 is done: Q, K have been read for the last time
-                if (opform && !(lok = mbar_wait(&bar_ld1, ph))) break;
-                if (opform && has_next) {
+                if (!(lok = mbar_wait(&bar_ld1, ph))) break;
+                if (has_next) {
                     mbar_expect_tx(&bar_qk, 32768);
                     pend_qk = true;
 #pragma unroll 1
@@ -196,16 +185,14 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
                 if (!(lok = mbar_wait(&bar_st, ph))) break;
                 constexpr uint32_t A_BYTES = XT - XA;
                 if (bwd) bulk_store(p.ws + p.L.E + (size_t)x.ch * 32768, sm + ES, A_BYTES);
-                if (opform) bulk_store(p.ws + p.L.Nm + (size_t)x.ch * 32768 + (PT - TT), sm + NMS + (PT - TT), 8192);
+                bulk_store(p.ws + p.L.Nm + (size_t)x.ch * 32768 + (PT - TT), sm + NMS + (PT - TT), 8192);
                 bulk_commit();
                 if (bwd) bulk_store(p.ws + p.L.E + (size_t)x.ch * 32768 + A_BYTES, sm + ES + A_BYTES, 32768 - A_BYTES);
                 bulk_commit();
                 bulk_wait_read<1>();       // (issuing a store takes hundreds of cycles: the first group has drained by now)
                 mbar_arrive(&bar_free1);   // the fp32 A block and P may be written (and the scratch over W^T: its store is older)
-                if (opform) {
-                    bulk_store(p.ws + p.L.Nm + (size_t)x.ch * 32768, sm + NMS, PT - TT);
-                    bulk_store(p.ws + p.L.Bf + (size_t)x.ch * 32768, sm + BFS, 32768);
-                }
+                bulk_store(p.ws + p.L.Nm + (size_t)x.ch * 32768, sm + NMS, PT - TT);
+                bulk_store(p.ws + p.L.Bf + (size_t)x.ch * 32768, sm + BFS, 32768);
                 bulk_commit();
                 bulk_wait_read<1>();
                 mbar_arrive(&bar_free2);   // the fp32 T block may be written
@@ -309,8 +296,7 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     float* Af = reinterpret_cast<float*>(sm + XA);   // [64][kLdi]  strictly lower part of I + A
     float* Tf = reinterpret_cast<float*>(sm + XT);   // [64][kLdi]  T
     if (has_next && warp == 0) fetch_gates(xn);   // next trip's gates -> registers while the product runs
-    // R = Diag(Gam) dO (token-major tile) while the product runs.  In low-rank mode the tiles of Diag(e) W and
-    // Diag(e) U~ are never written, so R has a tile of its own from here on and Q^T R can run under the inversion.
+    // R = Diag(Gam) dO (token-major tile)
     auto form_R = [&](unsigned char* dst) {   // the 512 worker threads, two 16-byte pieces each (both loads in flight)
         if (worker) {
             float v[2][8];
@@ -326,7 +312,6 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
             }
         }
     };
-    if (bwd && !opform) form_R(sm + WET);
     GDN_WAIT_MMA(2)
     if (ok && !first) {   // the previous trip's stores have read what lies under the fp32 A block and under P
         ok = mbar_wait(&bar_free1, in_phase ^ 1);
@@ -363,8 +348,6 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     if (ok && issuer && bwd) {
         tc_fence_after();
         mma_tile<128, 64, 64>(tmem + C_PDO, op_mn_major(sm + VO, 128, 64), op_mn_major(sm + PT, 64), false);
-        // low-rank mode: so does the first half of E = Q^T R - W^T (P^T dO), into columns no other product uses
-        if (!opform) mma_tile<128, 128, 64>(tmem + C_E_LR, op_mn_major(sm + QK, 128, 0), op_mn_major(sm + WET, 64), false);
     }
     // ---- T = (I + A)^-1, blocked, fp32 (invert64)
     if (ok && !first) {   // ... and what lies under the fp32 T block
@@ -410,11 +393,10 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
         mma_tile<128, 64, 64>(tmem + C_W, op_mn_major(sm + QK, 128, 64), op_k_major(sm + TP, 64), false);
         mma_tile<128, 64, 64>(tmem + C_U, op_mn_major(sm + VO, 128, 0), op_k_major(sm + TPP, 64), false);
         mma_commit(&bar_mma);
-        if (!opform) mma_commit(&bar_ld1);   // low-rank mode: Q, K have been read for the last time
     }
     if (threadIdx.x == 32) mbar_arrive(&bar_t);   // the loader stores the T tile
-    // operator mode: R while the MMAs run, over the fp32 A / T scratch, which is dead by now
-    if (bwd && opform) form_R(sm + XR);
+    // R while the MMAs run, over the fp32 A / T scratch, which is dead by now
+    if (bwd) form_R(sm + XR);
     GDN_WAIT_MMA(3)
     if (ok && worker) {
         const int f = q4 * 32 + lane, i0 = grp * kTG;
@@ -429,13 +411,13 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
 #pragma unroll
             for (int i = 0; i < 8; ++i) ve[i] = v[i] * e8[i];
             chunk_store(sm + WT, 128, f, ib >> 3, v);
-            if (opform) chunk_store(sm + WET, 128, f, ib >> 3, ve);
+            chunk_store(sm + WET, 128, f, ib >> 3, ve);
             tmem_ld8(tmem + lane_base + C_U + ib, v);
             tmem_wait_ld();
 #pragma unroll
             for (int i = 0; i < 8; ++i) ve[i] = v[i] * e8[i];
             chunk_store(sm + UTT, 128, f, ib >> 3, v);
-            if (opform) chunk_store(sm + UET, 128, f, ib >> 3, ve);
+            chunk_store(sm + UET, 128, f, ib >> 3, ve);
             if (bwd) {
                 tmem_ld8(tmem + lane_base + C_PDO + ib, v);
                 tmem_wait_ld();
@@ -452,11 +434,11 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
         tc_fence_after();
         // Nm and Bf share the operand K^T; their other operands and their accumulators are neighbours: one N = 256 product
         static_assert(UET == WET + 16384 && C_BF == C_NM + 128, "Nm | Bf as one product");
-        if (opform) mma_tile<128, 256, 64>(tmem + C_NM, op_mn_major(sm + QK, 128, 64), op_k_major(sm + WET, 128), false);
-        if (bwd && opform) mma_tile<128, 128, 64>(tmem + C_E, op_mn_major(sm + QK, 128, 0), op_mn_major(sm + XR, 64), false);
-        if (bwd) mma_tile<128, 128, 64>(tmem + (opform ? C_E : C_E_LR), op_k_major(sm + WT, 128), op_k_major(sm + XPDO, 128), true, /*neg_a=*/true);
+        mma_tile<128, 256, 64>(tmem + C_NM, op_mn_major(sm + QK, 128, 64), op_k_major(sm + WET, 128), false);
+        if (bwd) mma_tile<128, 128, 64>(tmem + C_E, op_mn_major(sm + QK, 128, 0), op_mn_major(sm + XR, 64), false);
+        if (bwd) mma_tile<128, 128, 64>(tmem + C_E, op_k_major(sm + WT, 128), op_k_major(sm + XPDO, 128), true, /*neg_a=*/true);
         mma_commit(&bar_mma);
-        if (opform) mma_commit(&bar_ld1);   // Q, K have been read for the last time
+        mma_commit(&bar_ld1);   // Q, K have been read for the last time
     } else if (threadIdx.x == 32) {
         mbar_arrive(&bar_vofree);   // W^T, U~^T are staged; V, dO were last read by phase 2 and the pass that formed R
     }
@@ -473,16 +455,14 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
         for (int part = 0; part < D / kGroups / 8; ++part) {
             const int cb = c0 + part * 8;
             float v[8];
-            if (opform) {
-                tmem_ld8(tmem + lane_base + C_NM + cb, v);
-                tmem_wait_ld();
-                chunk_store(sm + NMS, 128, r, cb >> 3, v);
-                tmem_ld8(tmem + lane_base + C_BF + cb, v);
-                tmem_wait_ld();
-                chunk_store(sm + BFS, 128, r, cb >> 3, v);
-            }
+            tmem_ld8(tmem + lane_base + C_NM + cb, v);
+            tmem_wait_ld();
+            chunk_store(sm + NMS, 128, r, cb >> 3, v);
+            tmem_ld8(tmem + lane_base + C_BF + cb, v);
+            tmem_wait_ld();
+            chunk_store(sm + BFS, 128, r, cb >> 3, v);
             if (bwd) {
-                tmem_ld8(tmem + lane_base + (opform ? C_E : C_E_LR) + cb, v);
+                tmem_ld8(tmem + lane_base + C_E + cb, v);
                 tmem_wait_ld();
 #pragma unroll
                 for (int k = 0; k < 8; ++k) v[k] *= sc;
@@ -1792,6 +1772,12 @@ static cudaError_t launch_eprep(const TcParams& P, cudaStream_t st) {
     return launch_chunk_kernel(tc_eprep_kernel, done, eprep::SMEM_BYTES, ST_EPREP, items < ctas ? items : ctas, split::kT, P, st);
 }
 
+static cudaError_t launch_prep_lr(const TcParams& P, cudaStream_t st) {
+    static SmemLimitOnce done;
+    const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count();
+    return launch_chunk_kernel(tc_prep_lr_kernel, done, both::SMEM_BYTES, ST_PREP, items < ctas ? items : ctas, split::kT, P, st);
+}
+
 static cudaError_t launch_scan(const TcParams& P, cudaStream_t st) {
     static SmemLimitOnce done;
     static SmemLimitOnce done2;
@@ -1890,9 +1876,9 @@ cudaError_t tc_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st
         P.withhold = 1;
         if ((e = cudaMemcpyToSymbolAsync(g_wait_limit_ns, &ns, sizeof(ns), 0, cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
     }
-    // (the closed arm keeps the fused kernel: it reads k once and never moves W through HBM on its way to E; measured on
-    // B = 4, T = 2048, H = 16: fused 99 us, tc_factors + tc_eprep 62 + 45 us)
-    if ((e = skip_recompute ? launch_eprep(P, st) : launch_prep(P, st)) != cudaSuccess) return e;
+    // (the closed arm keeps fused kernels: they read k once and never move W through HBM on its way to E; measured on
+    // B = 4, T = 2048, H = 16: tc_prep_lr 77 us, tc_factors + tc_eprep 62 + 45 us)
+    if ((e = skip_recompute ? launch_eprep(P, st) : P.lowrank ? launch_prep_lr(P, st) : launch_prep(P, st)) != cudaSuccess) return e;
     if ((e = launch_scan(P, st)) != cudaSuccess) return e;
     e = launch_intra(P, st);
     if (inject) {
