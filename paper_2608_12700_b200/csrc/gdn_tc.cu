@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     __shared__ __align__(16) float gate_sets[2][6][kC];
     __shared__ uint64_t bar_qk, bar_vo, bar_ld0, bar_t, bar_vofree, bar_ld1, bar_st, bar_tfree, bar_free1, bar_free2, bar_free, bar_mma;
     __shared__ uint32_t tmem_slot;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, grp = warp >> 2;
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
     const bool worker = warp < 16;                       // warps 0..15 read accumulators and do the fp32 work
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     cta_sync();
 
     // ---- phase 1: S1 = [Q; K] K^T  (rows 0..63: Q K^T, rows 64..127: K K^T)
-    if (ok && issuer) {
+    if (warp == 16 && elect_one() && ok) {
         tc_fence_after();
         mma_tile<128, 64, 128>(tmem + C_S1, op_k_major(sm + QK, 128, 0), op_k_major(sm + QK, 128, 64), false);
         mma_commit(&bar_mma);
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     fence_async_smem();
     cta_sync();
     // (P^T dO)^T = dO^T P needs nothing of the inversion: it runs under it and is covered by phase 2's commit
-    if (ok && issuer && bwd) {
+    if (warp == 16 && elect_one() && ok && bwd) {
         tc_fence_after();
         mma_tile<128, 64, 64>(tmem + C_PDO, op_mn_major(sm + VO, 128, 64), op_mn_major(sm + PT, 64), false);
     }
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     cta_sync();
 
     // ---- phase 2: W^T = K^T (T Diag(b Gam))^T ; U~^T = V^T (T Diag(w))^T
-    if (ok && issuer) {
+    if (warp == 16 && elect_one() && ok) {
         tc_fence_after();
         mma_tile<128, 64, 64>(tmem + C_W, op_mn_major(sm + QK, 128, 64), op_k_major(sm + TP, 64), false);
         mma_tile<128, 64, 64>(tmem + C_U, op_mn_major(sm + VO, 128, 0), op_k_major(sm + TPP, 64), false);
@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     cta_sync();
 
     // ---- phase 3: Nm = K^T (Diag(e) W) ; Bf = K^T (Diag(e) U~) ; E = Q^T R - W^T (P^T dO)
-    if (ok && issuer) {
+    if (warp == 16 && elect_one() && ok) {
         tc_fence_after();
         // Nm and Bf share the operand K^T; their other operands and their accumulators are neighbours: one N = 256 product
         static_assert(UET == WET + 16384 && C_BF == C_NM + 128, "Nm | Bf as one product");
@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
     __shared__ float ge[GE_CAP];
     __shared__ uint64_t bar_full[STAGES], bar_mma;
     __shared__ uint32_t tmem_slot;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, hf = warp >> 2;
     const int r = q4 * 32 + lane;              // state row owned by this thread
     const int lc0 = hf * NSH;                  // first of its NSH columns inside the CTA's block
@@ -599,7 +599,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
         for (int k = 0; k < NSH / 8; ++k) *reinterpret_cast<uint4*>(Ht + tile_chunk_off(128, r, (lc0 >> 3) + k)) = pack8(st + 8 * k);
         fence_async_smem();
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (warp == 0 && elect_one()) {
             ok = mbar_wait(&bar_full[stage], (s / STAGES) & 1);
             if (ok) {
                 tc_fence_after();
@@ -642,7 +642,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
 #pragma unroll
         for (int k = 0; k < NSH / 4; ++k) *reinterpret_cast<float4*>(fin + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
     }
-    if (threadIdx.x == 0) bulk_wait_read<0>();
+    if (warp == 0) bulk_wait_read<0>();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, NS);
@@ -700,7 +700,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
 
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sm = align1024(smem_raw);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, hf = warp >> 2;
     const int r = q4 * 32 + lane;              // TMEM lane of this thread: state row (d_k) or feature of the first product (d_v)
     const int lc0 = hf * NSH;                  // first of its NSH state columns inside the CTA's block
@@ -803,7 +803,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         }
         fence_async_smem();
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (warp == 0 && elect_one()) {
             ok = mbar_wait_inline(&bar_full[stage], (s / STAGES) & 1);
             if (ok) {
                 tc_fence_after();
@@ -844,7 +844,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         tc_fence_before();
         fence_async_smem();
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (warp == 0 && elect_one()) {
             tc_fence_after();
             if (reverse) mma_tile<128, NS, 64>(tmem + C_D2, op_k_major(ring + WT, 128), op_k_major(sm + GT, NS), false, /*neg_a=*/true);
             else mma_tile<128, NS, 64>(tmem + C_D2, op_mn_major(ring + KT, 64), op_k_major(sm + GT, NS), false);
@@ -875,7 +875,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
 #pragma unroll
         for (int k = 0; k < NSH / 4; ++k) *reinterpret_cast<float4*>(fin + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
     }
-    if (threadIdx.x == 0) bulk_wait_read<0>();
+    if (warp == 0) bulk_wait_read<0>();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, C::TMEM_COLS);
@@ -1533,7 +1533,7 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
     __shared__ __align__(16) float gl[kC], Gam[kC];
     __shared__ uint64_t bar_in, bar_mma;
     __shared__ uint32_t tmem_slot;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, half = warp >> 2;
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
     if (threadIdx.x == 0) { mbar_init(&bar_in, 1); mbar_init(&bar_mma, 1); fence_mbar_init(); }
@@ -1596,7 +1596,7 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
         }
         __syncthreads();
         // ---- step 1: Q K^T ; (W h)^T ; Q h
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             if (!CW) mma_tile<64, 64, 128>(tmem + C_P, op_k_major(sm + QK, 128, 0), op_k_major(sm + QK, 128, 64), false);
             mma_tile<128, 64, 128>(tmem + C_WH, op_mn_major(sm + HH, 128), op_mn_major(sm + WT, 128), false);
@@ -1634,7 +1634,7 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
         fence_async_smem();
         __syncthreads();
         // ---- step 2: P U (token-major, over the columns of the first two accumulators)
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             if (CW) mma_tile<64, 128, 64>(tmem + C_QH, op_k_major(sm + PT_CW, 64), op_k_major(sm + UTT, 128), true);
             else mma_tile<64, 128, 64>(tmem + C_PU, op_k_major(sm + PT, 64), op_k_major(sm + UTT, 128), false);

@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(256) tc64_gamma_kernel(Problem p) {
     if (c >= n_chunks_of(p)) return;
     const ChunkGeom cg = chunk_geom(p);
     const int tok0 = cg.chunk_tok0(c), len = cg.chunk_len(c);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     for (int i = warp; i < kC; i += 8)
         gs[i][lane] = (i < len && h0 + lane < H) ? p.g[(size_t)(tok0 + i) * H + h0 + lane] : 0.f;
     __syncthreads();
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
     __shared__ __align__(16) float gl[kC], Gam[kC], ee[kC];
     __shared__ uint64_t bar_full[STAGES], bar_mma;
     __shared__ uint32_t tmem_slot;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, half = warp >> 2;
     const int r = q4 * 16 + (lane & 15);      // row of the 64 x 64 accumulators / of the state held by this lane
     const bool act = lane < 16;
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
             bulk_store(p.ws + p.L.hc + ch * 8192, sm + HT, 8192);
             bulk_commit();
         }
-        if (threadIdx.x == 0) {
+        if (warp == 0 && elect_one()) {
             tc_fence_after();
             mma_tile<64, 64, 64>(tmem + 0, op_mn_major(tiles + KT, 64), op_mn_major(sm + VE, 64), false);              // Kb^T V
             if (want_o) {
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
             tc_fence_before();
             fence_async_smem();
             __syncthreads();
-            if (threadIdx.x == 0) {
+            if (warp == 0 && elect_one()) {
                 tc_fence_after();
                 mma_tile<64, 64, 64>(tmem + 192, op_k_major(sm + PT, 64), op_mn_major(tiles + VT, 64), false);          // P V
                 mma_commit(&bar_mma);
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
     __shared__ __align__(16) float gl2[2][kC], Gam2[2][kC], ee2[2][kC], dgp[2][kC], scal[2][kThreads64 / 32];
     __shared__ uint64_t bar_full[STAGES], bar_st, bar_mma;
     __shared__ uint32_t tmem_slot;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, half = warp >> 2;
     const int r = q4 * 16 + (lane & 15);      // accumulator / state row of this lane
     const bool ga = lane < 16;                // group A: lanes 0..15, group B: lanes 16..31
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
         cta_sync();
         const float Ge = Gam[kC - 1];
         // ---- phase 1: S = Q K^T ; dO V^T ; K dh' (group A) | dO h^T ; V dh'^T (group B)
-        if (threadIdx.x == 0) {
+        if (warp == 0 && elect_one()) {
             tc_fence_after();
             mma_tile<64, 64, 64>(tmem + C0, op_k_major(tiles + QT, 64), op_k_major(tiles + KT, 64), false);
             mma_tile<64, 64, 64>(tmem + C1, op_k_major(tiles + OT, 64), op_k_major(tiles + VT, 64), false);
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
         fence_async_smem();
         cta_sync();
         // ---- phase 2: P^T dO ; (Diag(Gam) Q)^T dO (group A) | (dP.D) K ; (dP.D)^T Q (group B)
-        if (threadIdx.x == 0) {
+        if (warp == 0 && elect_one()) {
             tc_fence_after();
             mma_tile<64, 64, 64>(tmem + C3, op_mn_major(sm + PX, 64), op_mn_major(tiles + OT, 64), false);
             mma_tile<64, 64, 64>(tmem + C0, op_mn_major(tiles + QT, 64), op_mn_major(sm + DH, 64), false);

@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
     unsigned char* sm = align1024(smem_raw);
     __shared__ uint64_t bar_in, bar_mma;
     __shared__ uint32_t tmem_slot;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, grp = warp >> 2;
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
     if (threadIdx.x == 0) { mbar_init(&bar_in, 1); mbar_init(&bar_mma, 1); fence_mbar_init(); }
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, in_phase ^= 1) {
         const size_t ch = (size_t)item, chn = ch + gridDim.x;
         const bool has_next = item + (int)gridDim.x < n_items;
-        if (threadIdx.x == 0) bulk_wait_read<0>();   // the previous trip's stores have read their tiles (rewritten from here on)
+        if (warp == 0) bulk_wait_read<0>();   // the previous trip's stores have read their tiles (rewritten from here on)
         if (ok) {
             ok = mbar_wait(&bar_in, in_phase);
             if (!ok && threadIdx.x == 0) report_timeout(p.ws, 40);
@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
         __syncthreads();
         if (fresh) {
             // (P^T dO')^T and Q~^T dO' from the loaded tiles; then E = Q~^T dO' - W^T (P^T dO') as in the closed arm
-            if (ok && threadIdx.x == 0) {
+            if (warp == 0 && elect_one() && ok) {
                 tc_fence_after();
                 mma_tile<128, 64, 64>(tmem + C_PDO, op_mn_major(sm + DOT, 64), op_mn_major(sm + PT, 64), false);
                 mma_tile<128, 128, 64>(tmem + C_E, op_mn_major(sm + QKP, 128, 0), op_mn_major(sm + DOT, 64), false);
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
             __syncthreads();
         } else {
         // ---- step 1: S1 = [Q~; K+] K-^T  (rows 0..63: P before masking, rows 64..127: A)
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 128>(tmem + C_S1, op_k_major(sm + QKP, 128, 0), op_k_major(sm + KM, 64), false);
             mma_commit(&bar_mma);
@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
         fence_async_smem();
         __syncthreads();
         // (P^T dO')^T and Q~^T dO' need nothing of the inversion: they run under it, covered by the next commit
-        if (ok && bwd && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok && bwd) {
             tc_fence_after();
             mma_tile<128, 64, 64>(tmem + C_PDO, op_mn_major(sm + DOT, 64), op_mn_major(sm + PT, 64), false);
             mma_tile<128, 128, 64>(tmem + C_E, op_mn_major(sm + QKP, 128, 0), op_mn_major(sm + DOT, 64), false);
@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
         fence_async_smem();
         __syncthreads();
         // ---- step 2: W^T = K+^T T^T ; U~^T = V~^T T^T
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 64>(tmem + C_W, op_mn_major(sm + QKP, 128, 64), op_k_major(sm + TT, 64), false);
             mma_tile<128, 64, 64>(tmem + C_U, op_mn_major(sm + VT, 64), op_k_major(sm + TT, 64), false);
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
         }   // (!fresh)
         // ---- step 3: E = Q~^T dO' - W^T (P^T dO')
         if (bwd) {
-            if (ok && threadIdx.x == 0) {
+            if (warp == 0 && elect_one() && ok) {
                 tc_fence_after();
                 mma_tile<128, 128, 64>(tmem + C_E, op_k_major(sm + WT, 128), op_k_major(sm + PDOT, 128), true, /*neg_a=*/true);
                 mma_commit(&bar_mma);
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
             fence_async_smem();
             __syncthreads();
         }
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             if (!fresh) {
                 bulk_store(p.ws + p.L.Tm + ch * 8192, sm + TT, 8192);
                 bulk_store(p.ws + p.L.Pm + ch * 8192, sm + PT, 8192);
@@ -404,10 +404,8 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
         }
         if (!ok) break;
     }
-    if (threadIdx.x == 0) {
-        bulk_wait_read<0>();
-        if (pending) (void)mbar_wait(&bar_in, pending_phase);   // after a timeout a load may still be in flight
-    }
+    if (warp == 0) bulk_wait_read<0>();
+    if (threadIdx.x == 0 && pending) (void)mbar_wait(&bar_in, pending_phase);   // after a timeout a load may still be in flight
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, 512);
@@ -455,7 +453,7 @@ __global__ void __launch_bounds__(kT, 1) cw_intra_kernel(Problem p) {
     __shared__ uint64_t bar_s, bar_a, bar_b, bar_k, bar_q, bar_mma;
     __shared__ uint32_t tmem_slot;
     __shared__ float end_sum[3][D];   // per key channel: rowdot(dh'', h) and the two halves of rowdot(dh'', K-^T U)
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, grp = warp >> 2;
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
     if (threadIdx.x == 0) {
@@ -525,7 +523,7 @@ __global__ void __launch_bounds__(kT, 1) cw_intra_kernel(Problem p) {
         }
         __syncthreads();
         // ---- step 1: (W h)^T ; (K- dh'')^T ; (P^T dO')^T
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 128>(tmem + C_A, op_mn_major(sm + HH, 128), op_mn_major(sm + WT, 128), false);
             mma_tile<128, 64, 128>(tmem + C_B, op_mn_major(sm + DH, 128), op_k_major(sm + QKM, 128, 64), false);
@@ -574,7 +572,7 @@ __global__ void __launch_bounds__(kT, 1) cw_intra_kernel(Problem p) {
             if (!ok && threadIdx.x == 0) report_timeout(p.ws, 51);
             if (ok && threadIdx.x == 0) pend_q = false;
         }
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<64, 64, 128>(tmem + C_PP, op_k_major(sm + DOT, 64), op_mn_major(sm + UT, 128), false);
             mma_tile<128, 64, 64>(tmem + C_A, op_k_major(sm + DUT, 128), op_mn_major(sm + TT, 64), false);
@@ -630,7 +628,7 @@ __global__ void __launch_bounds__(kT, 1) cw_intra_kernel(Problem p) {
         if (ok && threadIdx.x < D) scr[S_HH / 4 + threadIdx.x] = end_sum[0][threadIdx.x] + end_sum[1][threadIdx.x] + end_sum[2][threadIdx.x];
         // ---- step 3 (K#2): dA = -stril(dXv U^T) (= -stril(dXk W^T + dXv U~^T): dXk = T^T dW = -dXv h^T, U = U~ - W h) ;
         // dK+ = dXk = -dXv h^T ; dQ~ += dP K- ; dK- += dP^T Q~
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<64, 64, 128>(tmem + C_PP, op_mn_major(sm + DXVT, 128), op_mn_major(sm + UT, 128), false);
             mma_tile<64, 128, 128>(tmem + C_KP, op_mn_major(sm + DXVT, 128), op_k_major(sm + HH, 128), false, /*neg_a=*/true);
@@ -662,7 +660,7 @@ __global__ void __launch_bounds__(kT, 1) cw_intra_kernel(Problem p) {
         fence_async_smem();
         __syncthreads();
         // ---- step 4: dK+ += dA K- ; dK- += dA^T K+
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<64, 128, 64>(tmem + C_KP, op_k_major(sm + DA, 64), op_mn_major(sm + QKM, 128, 64), true);
             mma_tile<64, 128, 64>(tmem + C_KM, op_mn_major(sm + DA, 64), op_mn_major(sm + KP, 64), true);

@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_factors_kernel(const __grid_c
     __shared__ __align__(16) float gates[6][kC];   // gam log2e, Gam, e, b, w, b Gam
     __shared__ uint64_t bar_in, bar_mma;
     __shared__ uint32_t tmem_slot;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, grp = warp >> 2;
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
     if (threadIdx.x == 0) { mbar_init(&bar_in, 1); mbar_init(&bar_mma, 1); fence_mbar_init(); }
@@ -132,12 +132,12 @@ __global__ void __launch_bounds__(split::kT, 2) tc_factors_kernel(const __grid_c
         }
         __syncthreads();
         // ---- phase 1: S1 = [K; V] K^T (rows 0..63: K K^T; the V rows ride along unused)
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 128>(tmem + C_S1, op_k_major(sm + KV, 128, 0), op_k_major(sm + KV, 128, 0), false);
             mma_commit(&bar_mma);
         }
-        if (threadIdx.x == 0) bulk_wait_read<0>();   // the previous trip's stores have read their tiles (rewritten from here on)
+        if (warp == 0) bulk_wait_read<0>();   // the previous trip's stores have read their tiles (rewritten from here on)
         GDN_WAIT_MMA(22)
         __syncthreads();
         if (ok && q4 < 2) {   // A_ij = b_i (k_i . k_j) exp(gam_i - gam_j), j < i (mask before exponentiating)
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_factors_kernel(const __grid_c
         fence_async_smem();
         __syncthreads();
         // ---- phase 2: W^T = K^T (T Diag(b Gam))^T ; U~^T = V^T (T Diag(w))^T
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 64>(tmem + C_W, op_mn_major(sm + KV, 128, 0), op_k_major(sm + TP, 64), false);
             mma_tile<128, 64, 64>(tmem + C_U, op_mn_major(sm + KV, 128, 64), op_k_major(sm + TPP, 64), false);
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_factors_kernel(const __grid_c
         tc_fence_before();
         fence_async_smem();
         __syncthreads();
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             bulk_store(p.ws + p.L.Tm + (size_t)x.ch * 8192, sm + TT, 8192);
             bulk_store(p.ws + p.L.W + (size_t)x.ch * 16384, sm + WU, 16384);
             bulk_store(p.ws + p.L.Ut + (size_t)x.ch * 16384, sm + WU + 16384, 16384);
@@ -221,10 +221,8 @@ __global__ void __launch_bounds__(split::kT, 2) tc_factors_kernel(const __grid_c
         if (!ok) break;
         x = xn;
     }
-    if (threadIdx.x == 0) {
-        bulk_wait_read<0>();
-        if (pending) (void)mbar_wait(&bar_in, in_phase);   // after a timeout a load may still be in flight
-    }
+    if (warp == 0) bulk_wait_read<0>();
+    if (threadIdx.x == 0 && pending) (void)mbar_wait(&bar_in, in_phase);   // after a timeout a load may still be in flight
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, 256);
@@ -260,7 +258,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
     __shared__ __align__(16) float gl[kC], Gam[kC];
     __shared__ uint64_t bar_in, bar_mma;
     __shared__ uint32_t tmem_slot;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, grp = warp >> 2;
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
     if (threadIdx.x == 0) { mbar_init(&bar_in, 1); mbar_init(&bar_mma, 1); fence_mbar_init(); }
@@ -314,12 +312,12 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
         }
         __syncthreads();
         // ---- phase 1: S1 = [Q; K] K^T (rows 0..63: Q K^T)
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 128>(tmem + C_S1, op_k_major(sm + QK, 128, 0), op_k_major(sm + QK, 128, 64), false);
             mma_commit(&bar_mma);
         }
-        if (threadIdx.x == 0) bulk_wait_read<0>();   // the previous trip's stores have read P and the staged E image
+        if (warp == 0) bulk_wait_read<0>();   // the previous trip's stores have read P and the staged E image
         GDN_WAIT_MMA(25)
         __syncthreads();
         // R = Diag(Gam) dO: four 16-byte pieces per thread
@@ -351,7 +349,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
         fence_async_smem();
         __syncthreads();
         // ---- phase 2: (P^T dO)^T = dO^T P ; first half of E: Q^T R
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 64>(tmem + C_PDO, op_mn_major(sm + DOT, 64), op_mn_major(sm + PT, 64), false);
             mma_tile<128, 128, 64>(tmem + C_E, op_mn_major(sm + QK, 128, 0), op_mn_major(sm + RT, 64), false);
@@ -373,7 +371,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
         fence_async_smem();
         __syncthreads();
         // ---- phase 3: E -= W^T (P^T dO)
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 128, 64>(tmem + C_E, op_k_major(sm + WT, 128), op_k_major(sm + PDOT, 128), true, /*neg_a=*/true);
             mma_commit(&bar_mma);
@@ -399,7 +397,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
         tc_fence_before();
         fence_async_smem();
         __syncthreads();
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             bulk_store(p.ws + p.L.Pm + (size_t)x.ch * 8192, sm + PT, 8192);
             bulk_store(p.ws + p.L.E + (size_t)x.ch * 32768, sm + RT, 32768);
             bulk_commit();
@@ -407,10 +405,8 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
         if (!ok) break;
         x = xn;
     }
-    if (threadIdx.x == 0) {
-        bulk_wait_read<0>();
-        if (pending) (void)mbar_wait(&bar_in, in_phase);   // after a timeout a load may still be in flight
-    }
+    if (warp == 0) bulk_wait_read<0>();
+    if (threadIdx.x == 0 && pending) (void)mbar_wait(&bar_in, in_phase);   // after a timeout a load may still be in flight
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, 256);
@@ -452,7 +448,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
     __shared__ __align__(16) float gates[5][kC];   // gam log2e, Gam, b, w, b Gam
     __shared__ uint64_t bar_in, bar_mma;
     __shared__ uint32_t tmem_slot;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, grp = warp >> 2;
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
     if (threadIdx.x == 0) { mbar_init(&bar_in, 1); mbar_init(&bar_mma, 1); fence_mbar_init(); }
@@ -538,7 +534,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
         }
         __syncthreads();
         // ---- phase 1: S1 = [Q; K] K^T  (rows 0..63: Q K^T, rows 64..127: K K^T)
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 128>(tmem + C_S1, op_k_major(sm + QK, 128, 0), op_k_major(sm + QK, 128, 64), false);
             bulk_wait_read<0>();   // (the previous trip's stores have read P and the E image: rewritten from here on)
@@ -570,7 +566,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
         fence_async_smem();
         __syncthreads();
         // (P^T dO)^T = dO^T P runs under the inversion and is covered by phase 2's commit
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 64>(tmem + C_PDO, op_mn_major(sm + VO, 128, 64), op_mn_major(sm + PT, 64), false);
             bulk_store(p.ws + p.L.Pm + (size_t)x.ch * 8192, sm + PT, 8192);   // the gradient stage reads P from here
@@ -608,7 +604,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
         fence_async_smem();
         __syncthreads();
         // ---- phase 2: W^T = K^T (T Diag(b Gam))^T ; U~^T = V^T (T Diag(w))^T
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 64>(tmem + C_W, op_mn_major(sm + QK, 128, 64), op_k_major(sm + TP, 64), false);
             mma_tile<128, 64, 64>(tmem + C_U, op_mn_major(sm + VO, 128, 0), op_k_major(sm + TPP, 64), false);
@@ -648,7 +644,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
         fence_async_smem();
         __syncthreads();
         // ---- phase 3: E = Q^T R - W^T (P^T dO)   (the second operand of the second product in two pieces: 64 columns each)
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 128, 64>(tmem + C_E, op_mn_major(sm + QK, 128, 0), op_mn_major(sm + VO, 128, 64), false);
             mma_tile<128, 64, 64>(tmem + C_E, op_k_major(sm + WT, 128), op_k_major(sm + PDOT, 64), true, /*neg_a=*/true);
@@ -681,17 +677,15 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
         tc_fence_before();
         fence_async_smem();
         __syncthreads();
-        if (ok && threadIdx.x == 0) {
+        if (warp == 0 && elect_one() && ok) {
             bulk_store(p.ws + p.L.E + (size_t)x.ch * 32768, sm + ES, 32768);
             bulk_commit();
         }
         if (!ok) break;
         x = xn;
     }
-    if (threadIdx.x == 0) {
-        bulk_wait_read<0>();
-        if (pending) (void)mbar_wait(&bar_in, in_phase);   // after a timeout a load may still be in flight
-    }
+    if (warp == 0) bulk_wait_read<0>();
+    if (threadIdx.x == 0 && pending) (void)mbar_wait(&bar_in, in_phase);   // after a timeout a load may still be in flight
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, 256);

@@ -228,6 +228,19 @@ __device__ __forceinline__ void mma_issue(uint32_t tmem_d, uint64_t adesc, uint6
         ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// Products are issued by one elected lane of a warp, under a condition that the compiler can see is uniform for the warp:
+// if (warp_id() == w && elect_one()).  Descriptors then live in uniform registers, where the instruction wants them, and an
+// M64 x N64 instruction costs 34 cycles instead of 47 (issued behind threadIdx.x == 0 each of them moves its descriptors there
+// first; larger shapes are bound by the pipe either way, but the issuer needs fewer of the slots that the readout warps want).
+// All 32 lanes have to reach elect_one() together; it always elects the same one.  Whole calls: 8 x 32 heads of 4096 tokens of
+// the scalar-gate recurrence 481 -> 462 us, 4 heads of 640 tokens of it 64 -> 58 us, 6 x 16 x 1500 forward and backward
+// 372 -> 370 us.  (tc_intra keeps threadIdx.x: the uniform warp index cost it registers it does not have, 64 bytes of spills.)
+__device__ __forceinline__ int warp_id() { return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0); }
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 // D[M x N] (+)= A[M x Kt] * B[Kt x N]: one thread issues Kt / 16 instructions, fully unrolled so that each costs two
 // integer adds besides the tcgen05.mma itself (the tensor pipe accepts one such instruction every ~50-60 cycles).
 template <int M, int N, int Kt>
