@@ -12,6 +12,10 @@
 //             dgamma_i = <q_i,dq_i> - <k_i,dk_i>,  dgamma_63 += sum_j r_j + Gam_e <dh',h>,  dg = reverse cumsum.
 // Accumulators are 64 x 64 (M = 64: row i on TMEM lane i % 16 + 32 (i / 16)), token rows on lanes, so a thread owns
 // a token row: row dots are thread-local and gradient rows leave with 16-byte stores.  Two CTAs share an SM.
+// A 64-row accumulator occupies lanes 0..15 of each quadrant ("group A"), a second one lanes 16..31 of the same columns
+// ("group B", address + 16 lanes).  What bounds a step is the issue of the readouts, so both groups run one instruction
+// stream: either they hold two accumulators that are treated alike (Q K^T and dO V^T; K dh' and V dh'^T; P^T dO and
+// (dP.D)^T Q), or the two column halves of one, which is then issued as two N = 32 products.
 #define GDN_INLINE_WAIT   // small kernels: the polling loops sit at the wait sites (see tc_ptx.cuh)
 #include "tc_common.cuh"
 
@@ -94,8 +98,10 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
     const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, half = warp >> 2;
     const int r = q4 * 16 + (lane & 15);      // row of the 64 x 64 accumulators / of the state held by this lane
-    const bool act = lane < 16;
-    const int cb0 = half * 32;                // first of its 32 columns
+    const bool act = lane < 16;               // (output path: its accumulators are on lanes 0..15)
+    const int cb0 = half * 32;                // first of its 32 columns there
+    const int sc0 = (act ? 0 : 32) + half * 16;   // first of its 16 state columns (lanes 16..31 hold columns 32..63)
+    constexpr uint32_t LB = 16u << 16;
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
 
     if (threadIdx.x == 0) {
@@ -120,11 +126,11 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
     if (threadIdx.x == 0)
         for (int s = 0; s < STAGES && s < nsteps; ++s) fill(s);
 
-    float st[32];
-    const size_t soff = ((size_t)n * H + hd) * D6 * D6 + (size_t)r * D6 + cb0;
+    float st[16];
+    const size_t soff = ((size_t)n * H + hd) * D6 * D6 + (size_t)r * D6 + sc0;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        float4 v = (p.h0 && act) ? *reinterpret_cast<const float4*>(p.h0 + soff + 4 * k) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < 4; ++k) {
+        float4 v = p.h0 ? *reinterpret_cast<const float4*>(p.h0 + soff + 4 * k) : make_float4(0.f, 0.f, 0.f, 0.f);
         st[4 * k] = v.x; st[4 * k + 1] = v.y; st[4 * k + 2] = v.z; st[4 * k + 3] = v.w;
     }
     const float* gamma = reinterpret_cast<const float*>(p.ws + p.L.gamma);
@@ -163,11 +169,10 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
             for (int k = 0; k < 8; ++k) v[k] *= ee[i];
             chunk_store(sm + VE, 64, i, cch, v);
         }
-        if (act) {   // state entering the chunk -> bf16 tile: the workspace copy (and, for o, the MMA operand)
+        // state entering the chunk -> bf16 tile: the workspace copy (and, for o, the MMA operand)
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                *reinterpret_cast<uint4*>(sm + HT + tile_chunk_off(64, r, (cb0 >> 3) + k)) = pack8(st + 8 * k);
-        }
+        for (int k = 0; k < 2; ++k)
+            *reinterpret_cast<uint4*>(sm + HT + tile_chunk_off(64, r, (sc0 >> 3) + k)) = pack8(st + 8 * k);
         fence_async_smem();
         __syncthreads();
         if (threadIdx.x == 32) {   // the tile leaves through the async proxy (generic global stores would stall the next proxy fence)
@@ -176,7 +181,8 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
         }
         if (warp == 0 && elect_one()) {
             tc_fence_after();
-            mma_tile<64, 64, 64>(tmem + 0, op_mn_major(tiles + KT, 64), op_mn_major(sm + VE, 64), false);              // Kb^T V
+            mma_tile<64, 32, 64>(tmem + 0, op_mn_major(tiles + KT, 64), op_mn_major(sm + VE, 64), false);              // Kb^T V
+            mma_tile<64, 32, 64>(tmem + 0 + LB, op_mn_major(tiles + KT, 64), op_mn_major(sm + VE + 64, 64), false);    // (columns 32..63)
             if (want_o) {
                 mma_tile<64, 64, 64>(tmem + 64, op_k_major(tiles + QT, 64), op_k_major(tiles + KT, 64), false);         // Q K^T
                 mma_tile<64, 64, 64>(tmem + 128, op_k_major(tiles + QT, 64), op_mn_major(sm + HT, 64), false);          // Q h
@@ -226,9 +232,9 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
             }
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {   // h' = Gam_e h + Kb^T V
+        for (int k = 0; k < 2; ++k) {   // h' = Gam_e h + Kb^T V
             float bf[8];
-            tmem_ld8(tmem + lane_base + 0 + cb0 + 8 * k, bf);
+            tmem_ld8(tmem + lane_base + 0 + half * 16 + 8 * k, bf);
             tmem_wait_ld();
 #pragma unroll
             for (int j = 0; j < 8; ++j) st[8 * k + j] = fmaf(Ge, st[8 * k + j], bf[j]);
@@ -240,9 +246,9 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
         }
     }
     if (threadIdx.x == 32) bulk_wait_read<0>();
-    if (p.hT && ok && act) {
+    if (p.hT && ok) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) *reinterpret_cast<float4*>(p.hT + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
+        for (int k = 0; k < 4; ++k) *reinterpret_cast<float4*>(p.hT + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
     }
     tc_fence_before();
     __syncthreads();
@@ -260,11 +266,14 @@ constexpr uint32_t PX = DH + 8192;              // P
 constexpr uint32_t DPD = PX + 8192;             // scale tril(dO V^T) . D
 constexpr uint32_t SMEM_BYTES = DPD + 8192 + 1024;
 static_assert(2 * (SMEM_BYTES + 4096) <= 227 * 1024, "two CTAs per SM");
-// Tensor memory: 256 columns per CTA so that two CTAs share an SM.  A 64-row accumulator occupies lanes 0..15 of
-// each 32-lane quadrant; a second one lives in lanes 16..31 of the same columns (address + 16 lanes).  Lanes 0..15
-// of every warp ("group A") therefore read S, dO V^T, K dh', P^T dO and the state increment, lanes 16..31 ("group
-// B") read dO h^T, (dP.D) K, V dh'^T and (dP.D)^T Q with the same load instructions.
-constexpr uint32_t C0 = 0, C1 = 64, C2 = 128, C3 = 192, LB = 16u << 16;
+// Tensor memory: 256 columns per CTA so that two CTAs share an SM.
+//   columns       lanes 0..15 (A)                      lanes 16..31 (B)
+//   C0  64        Q K^T;  (Diag(Gam) Q)^T dO, columns 0..31 (32 wide)      dO V^T;  ... columns 32..63
+//   C1  64        K dh'                                V dh'^T
+//   C2  64        P^T dO                               (dP.D)^T Q
+//   C3  32        dO h^T, columns 0..31                dO h^T, columns 32..63
+//   C4  32        (dP.D) K, columns 0..31              (dP.D) K, columns 32..63
+constexpr uint32_t C0 = 0, C1 = 64, C2 = 128, C3 = 192, C4 = 224, LB = 16u << 16;
 }  // namespace b64
 
 __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __grid_constant__ Tc64Params P) {
@@ -282,13 +291,14 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sm = align1024(smem_raw);
     __shared__ __align__(16) float gl2[2][kC], Gam2[2][kC], ee2[2][kC], dgp[2][kC], scal[2][kThreads64 / 32];
-    __shared__ uint64_t bar_full[STAGES], bar_st, bar_mma;
+    __shared__ uint64_t bar_full[STAGES], bar_st, bar_mma, bar_mma2;
     __shared__ uint32_t tmem_slot;
     const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, half = warp >> 2;
     const int r = q4 * 16 + (lane & 15);      // accumulator / state row of this lane
     const bool ga = lane < 16;                // group A: lanes 0..15, group B: lanes 16..31
-    const int cb0 = half * 32;                // first of this thread's 32 columns
+    const int cb0 = half * 32;                // first of this thread's 32 columns of a whole accumulator
+    const int sc0 = (ga ? 0 : 32) + half * 16;   // first of its 16 columns of one issued in halves, and of the state
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
 
     // Warp 8 only moves data: its first lane stores a step's staged gradients and then loads the tiles of the step
@@ -299,6 +309,7 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
         for (int s = 0; s < STAGES; ++s) mbar_init(&bar_full[s], 1);
         mbar_init(&bar_st, 1);
         mbar_init(&bar_mma, 1);
+        mbar_init(&bar_mma2, 1);
         fence_mbar_init();
     }
     if (warp == 0) { tmem_alloc(&tmem_slot, 256); tmem_relinquish(); }
@@ -341,11 +352,11 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
     }
     auto cta_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kThreads64) : "memory"); };   // all warps but the loader
 
-    float st[32];   // group A: dh' row r, columns cb0 .. cb0 + 31 (gradient w.r.t. the state leaving the current chunk)
-    const size_t soff = ((size_t)n * H + hd) * D6 * D6 + (size_t)r * D6 + cb0;
+    float st[16];   // dh' row r, columns sc0 .. sc0 + 15 (gradient w.r.t. the state leaving the current chunk)
+    const size_t soff = ((size_t)n * H + hd) * D6 * D6 + (size_t)r * D6 + sc0;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        float4 v = (p.dhT && ga) ? *reinterpret_cast<const float4*>(p.dhT + soff + 4 * k) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < 4; ++k) {
+        float4 v = p.dhT ? *reinterpret_cast<const float4*>(p.dhT + soff + 4 * k) : make_float4(0.f, 0.f, 0.f, 0.f);
         st[4 * k] = v.x; st[4 * k + 1] = v.y; st[4 * k + 2] = v.z; st[4 * k + 3] = v.w;
     }
     // Gate arrays of a step (log2-scaled cumulative decay, Gam = exp(gam), e = exp(gam_end - gam)) are prepared one
@@ -380,28 +391,28 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
             zero_tail_rows64(tiles + OT, len);
         }
         float hh = 0.f;   // <dh', h> restricted to this thread's part of the state
-        if (ga) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                float hv[8];
-                chunk_load(tiles + HT, 64, r, (cb0 >> 3) + k, hv);
+        for (int k = 0; k < 2; ++k) {
+            float hv[8];
+            chunk_load(tiles + HT, 64, r, (sc0 >> 3) + k, hv);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) hh = fmaf(st[8 * k + j], hv[j], hh);
-                chunk_store(sm + DH, 64, r, (cb0 >> 3) + k, st + 8 * k);
-            }
+            for (int j = 0; j < 8; ++j) hh = fmaf(st[8 * k + j], hv[j], hh);
+            chunk_store(sm + DH, 64, r, (sc0 >> 3) + k, st + 8 * k);
         }
         fence_async_smem();
         cta_sync();
         const float Ge = Gam[kC - 1];
-        // ---- phase 1: S = Q K^T ; dO V^T ; K dh' (group A) | dO h^T ; V dh'^T (group B)
+        // ---- phase 1: Q K^T, dO V^T; under their readout K dh', V dh'^T, dO h^T
         if (warp == 0 && elect_one()) {
             tc_fence_after();
             mma_tile<64, 64, 64>(tmem + C0, op_k_major(tiles + QT, 64), op_k_major(tiles + KT, 64), false);
-            mma_tile<64, 64, 64>(tmem + C1, op_k_major(tiles + OT, 64), op_k_major(tiles + VT, 64), false);
-            mma_tile<64, 64, 64>(tmem + C2, op_k_major(tiles + KT, 64), op_mn_major(sm + DH, 64), false);
-            mma_tile<64, 64, 64>(tmem + C0 + LB, op_k_major(tiles + OT, 64), op_k_major(tiles + HT, 64), false);
-            mma_tile<64, 64, 64>(tmem + C2 + LB, op_k_major(tiles + VT, 64), op_k_major(sm + DH, 64), false);
+            mma_tile<64, 64, 64>(tmem + C0 + LB, op_k_major(tiles + OT, 64), op_k_major(tiles + VT, 64), false);
             mma_commit(&bar_mma);
+            mma_tile<64, 64, 64>(tmem + C1, op_k_major(tiles + KT, 64), op_mn_major(sm + DH, 64), false);
+            mma_tile<64, 64, 64>(tmem + C1 + LB, op_k_major(tiles + VT, 64), op_k_major(sm + DH, 64), false);
+            mma_tile<64, 32, 64>(tmem + C3, op_k_major(tiles + OT, 64), op_k_major(tiles + HT, 64, 0), false);
+            mma_tile<64, 32, 64>(tmem + C3 + LB, op_k_major(tiles + OT, 64), op_k_major(tiles + HT, 64, 32), false);
+            mma_commit(&bar_mma2);
         }
         if (threadIdx.x < kC && s + 1 < nsteps) {
             make_gates((s + 1) & 1, gnext, gend_next);
@@ -409,102 +420,104 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
         }
         GDN_WAIT_MMA(51)
         if (!ok) break;
-        for (int t = threadIdx.x; t < kC * 8; t += kThreads64) {   // Diag(Gam) dO over the dh' tile, which no MMA reads any more
-            const int i = t >> 3, cch = t & 7;
-            float v[8];
-            chunk_load(tiles + OT, 64, i, cch, v);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] *= Gam[i];
-            chunk_store(sm + DH, 64, i, cch, v);
-        }
-        float rs = 0.f;   // sum_j r_j, r_j = e_j <(K dh')_j, V_j>
-#pragma unroll 1
-        for (int part = 0; part < 4; ++part) {
-            float s8[8], p8[8], kd[8], vv[8];
-            const int jb = cb0 + part * 8;
-            tmem_ld8(tmem + lane_base + C0 + jb, s8);
-            tmem_ld8(tmem + lane_base + C1 + jb, p8);
-            tmem_ld8(tmem + lane_base + C2 + jb, kd);
-            tmem_wait_ld();
-            if (ga) {
-                chunk_load(tiles + VT, 64, r, jb >> 3, vv);
-                float g8[8];
+        {   // A: P = tril(Q K^T . D)   B: dP . D = scale tril(dO V^T) . D
+            const float glr = gl[r], f = ga ? 1.f : sc;
+            unsigned char* dst = sm + (ga ? PX : DPD);
+#pragma unroll 2
+            for (int part = 0; part < 4; ++part) {
+                float s8[8], g8[8];
+                const int jb = cb0 + part * 8;
+                tmem_ld8(tmem + lane_base + C0 + jb, s8);
                 ld8s(gl + jb, g8);
+                tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float dcy = (jb + j <= r) ? ex2(gl[r] - g8[j]) : 0.f;   // masked first: the exponent is never positive
-                    s8[j] *= dcy;                   // P
-                    p8[j] *= sc * dcy;              // dP . D
-                    rs = fmaf(kd[j], vv[j], rs);
-                }
-                chunk_store(sm + PX, 64, r, jb >> 3, s8);
-                chunk_store(sm + DPD, 64, r, jb >> 3, p8);
+                for (int j = 0; j < 8; ++j) s8[j] *= (jb + j <= r) ? f * ex2(glr - g8[j]) : 0.f;   // masked first: the exponent is never positive
+                chunk_store(dst, 64, r, jb >> 3, s8);
             }
         }
-        rs *= ee[r];
+        ok = mbar_wait(&bar_mma2, 0);
+        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 53); break; }
+        tc_fence_after();
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {   // Diag(Gam) dO over the dh' tile, which no MMA reads any more
+            const int i = (threadIdx.x >> 3) + 32 * t, cch = threadIdx.x & 7;
+            float v[8];
+            chunk_load(tiles + OT, 64, i, cch, v);
+            const float G = Gam[i];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] *= G;
+            chunk_store(sm + DH, 64, i, cch, v);
+        }
         tc_fence_before();
         fence_async_smem();
         cta_sync();
-        // ---- phase 2: P^T dO ; (Diag(Gam) Q)^T dO (group A) | (dP.D) K ; (dP.D)^T Q (group B)
+        // ---- phase 2: P^T dO, (dP.D)^T Q, (dP.D) K; under their readout (Diag(Gam) Q)^T dO
         if (warp == 0 && elect_one()) {
             tc_fence_after();
-            mma_tile<64, 64, 64>(tmem + C3, op_mn_major(sm + PX, 64), op_mn_major(tiles + OT, 64), false);
-            mma_tile<64, 64, 64>(tmem + C0, op_mn_major(tiles + QT, 64), op_mn_major(sm + DH, 64), false);
-            mma_tile<64, 64, 64>(tmem + C1 + LB, op_k_major(sm + DPD, 64), op_mn_major(tiles + KT, 64), false);
-            mma_tile<64, 64, 64>(tmem + C3 + LB, op_mn_major(sm + DPD, 64), op_mn_major(tiles + QT, 64), false);
+            mma_tile<64, 64, 64>(tmem + C2, op_mn_major(sm + PX, 64), op_mn_major(tiles + OT, 64), false);
+            mma_tile<64, 64, 64>(tmem + C2 + LB, op_mn_major(sm + DPD, 64), op_mn_major(tiles + QT, 64), false);
+            mma_tile<64, 32, 64>(tmem + C4, op_k_major(sm + DPD, 64), op_mn_major(tiles + KT, 64), false);
+            mma_tile<64, 32, 64>(tmem + C4 + LB, op_k_major(sm + DPD, 64), op_mn_major(tiles + KT + 64, 64), false);
             mma_commit(&bar_mma);
+            mma_tile<64, 32, 64>(tmem + C0, op_mn_major(tiles + QT, 64), op_mn_major(sm + DH, 64), false);
+            mma_tile<64, 32, 64>(tmem + C0 + LB, op_mn_major(tiles + QT, 64), op_mn_major(sm + DH + 64, 64), false);
+            mma_commit(&bar_mma2);
         }
         GDN_WAIT_MMA(52)
         if (!ok) break;
-        float dot = 0.f;   // group B: <q_r, dq_r> - <k_r, dk_r> over this thread's columns
-        // Gradient rows are staged token-major in place over this step's input tiles (dv over V, which was last read in
-        // phase 1; dk over K and dq over Q, where a thread overwrites exactly the piece it has just read) and leave by TMA
+        // Gradient rows are staged token-major in place over this step's input tiles (dv over V, dk over K and dq over Q, where
+        // a thread overwrites exactly the piece it has just read; every product that reads the tile is done) and leave by TMA
         // stores; generic global stores here would be one 16-byte piece per row.
-#pragma unroll 1
-        for (int part = 0; part < 4; ++part) {
-            float a[8], b[8], x[8];
-            const int jb = cb0 + part * 8;
-            tmem_ld8(tmem + lane_base + C3 + jb, a);     // A: P^T dO        B: (dP.D)^T Q
-            tmem_ld8(tmem + lane_base + C2 + jb, b);     // A: K dh'         B: V dh'^T
-            tmem_wait_ld();
-            if (ga) {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) a[j] = fmaf(sc, a[j], ee[r] * b[j]);      // dv = scale P^T dO + Diag(e) K dh'
-                chunk_store(tiles + VT, 64, r, jb >> 3, a);
-            } else {
-                chunk_load(tiles + KT, 64, r, jb >> 3, x);
+        float rs = 0.f;    // A: sum_j r_j, r_j = e_j <(K dh')_j, V_j>
+        float dot = 0.f;   // B: -<k_r, dk_r>;  both: <q_r, dq_r> over this thread's columns
+        {   // A: dv = scale P^T dO + Diag(e) K dh'     B: dk = (dP.D)^T Q + Diag(e) V dh'^T
+            const float e = ee[r], f = ga ? sc : 1.f;
+            unsigned char* tile = tiles + (ga ? VT : KT);
+#pragma unroll 2
+            for (int part = 0; part < 4; ++part) {
+                float a[8], b[8], x[8];
+                const int jb = cb0 + part * 8;
+                tmem_ld8(tmem + lane_base + C2 + jb, a);
+                tmem_ld8(tmem + lane_base + C1 + jb, b);
+                chunk_load(tile, 64, r, jb >> 3, x);
+                tmem_wait_ld();
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    a[j] = fmaf(ee[r], b[j], a[j]);                                    // dk = (dP.D)^T Q + Diag(e) V dh'^T
+                    rs = fmaf(b[j], x[j], rs);
+                    a[j] = fmaf(f, a[j], e * b[j]);
                     dot = fmaf(-x[j], a[j], dot);
                 }
-                chunk_store(tiles + KT, 64, r, jb >> 3, a);
+                chunk_store(tile, 64, r, jb >> 3, a);
             }
-            tmem_ld8(tmem + lane_base + C0 + jb, a);     //                  B: dO h^T
-            tmem_ld8(tmem + lane_base + C1 + jb, b);     //                  B: (dP.D) K
-            tmem_wait_ld();
-            if (!ga) {
-                chunk_load(tiles + QT, 64, r, jb >> 3, x);
+            rs *= e;
+            if (ga) dot = 0.f;
+        }
+        ok = mbar_wait(&bar_mma2, 1);
+        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 54); break; }
+        tc_fence_after();
+        {   // dq = scale Gam dO h^T + (dP.D) K ;  dh = Gam_e dh' + scale (Diag(Gam) Q)^T dO
+            const float G = sc * Gam[r];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                float a[8], b[8], x[8], e8[8];
+                tmem_ld8(tmem + lane_base + C3 + half * 16 + 8 * k, a);
+                tmem_ld8(tmem + lane_base + C4 + half * 16 + 8 * k, b);
+                tmem_ld8(tmem + lane_base + C0 + half * 16 + 8 * k, e8);
+                chunk_load(tiles + QT, 64, r, (sc0 >> 3) + k, x);
+                tmem_wait_ld();
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    a[j] = fmaf(sc * Gam[r], a[j], b[j]);                              // dq = scale Gam dO h^T + (dP.D) K
+                    a[j] = fmaf(G, a[j], b[j]);
                     dot = fmaf(x[j], a[j], dot);
+                    st[8 * k + j] = fmaf(Ge, st[8 * k + j], sc * e8[j]);
                 }
-                chunk_store(tiles + QT, 64, r, jb >> 3, a);
+                chunk_store(tiles + QT, 64, r, (sc0 >> 3) + k, a);
             }
         }
-        if (!ga) dgp[half][r] = dot;
-        // group A: dh = Gam_e dh' + scale (Diag(Gam) Q)^T dO
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            float e8[8];
-            tmem_ld8(tmem + lane_base + C0 + cb0 + 8 * k, e8);
-            tmem_wait_ld();
-#pragma unroll
-            for (int j = 0; j < 8; ++j) st[8 * k + j] = fmaf(Ge, st[8 * k + j], sc * e8[j]);
-        }
+        dot += __shfl_xor_sync(0xffffffffu, dot, 16);
+        if (ga) dgp[half][r] = dot;
         rs = warp_sum(ga ? rs : 0.f);
-        hh = warp_sum(ga ? hh : 0.f);
+        hh = warp_sum(hh);
         if (lane == 0) { scal[0][warp] = rs; scal[1][warp] = hh; }
         tc_fence_before();
         fence_async_smem();
@@ -529,9 +542,9 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
             write_dg_suffix(dgp[0], dgp[1], rsum + Ge * hsum, p.dg + (size_t)tok0 * H + hd, (size_t)H, len, lane);
         }
     }
-    if (p.dh0 && ok && ga) {
+    if (p.dh0 && ok) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) *reinterpret_cast<float4*>(p.dh0 + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
+        for (int k = 0; k < 4; ++k) *reinterpret_cast<float4*>(p.dh0 + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
     }
     tc_fence_before();
     cta_sync();
