@@ -70,17 +70,26 @@ __device__ __forceinline__ void zero_tail_rows64(unsigned char* tile, int len) {
 // forward pass
 // ------------------------------------------------------------------------------------------------
 namespace f64 {
-constexpr int STAGES = 2;
-constexpr uint32_t KT = 0, VT = 8192, QT = 16384, STAGE_BYTES = 24576;   // per stage: K, V (and Q when o is wanted)
-constexpr uint32_t VE = STAGES * STAGE_BYTES;   // Diag(e) V
-constexpr uint32_t HT = VE + 8192;              // bf16 state tile: leaves for the workspace by a bulk store; operand of Q h
-constexpr uint32_t PT = HT + 8192;              // P (only when o is wanted)
-constexpr uint32_t SMEM_BYTES = PT + 8192 + 1024;
+// The ring is what feeds a chain (a step is shorter than the latency of HBM), so it takes the shared memory that two CTAs per
+// SM leave: with two slots a step waited for its tiles (256 chains of 64 chunks: 97 us with two slots, three barriers a step and the
+// state on half of the lanes; 75 us now, 5.3 TB/s).
+template <bool O> struct Cfg {   // O: the forward output is wanted
+    static constexpr int STAGES = O ? 3 : 5;
+    static constexpr uint32_t KT = 0, VT = 8192, QT = 16384, STAGE_BYTES = O ? 24576 : 16384;   // per slot: K, V (and Q)
+    static constexpr uint32_t VE = STAGES * STAGE_BYTES;   // Diag(e) V
+    static constexpr uint32_t HT = VE + 8192;              // two bf16 state tiles: leave for the workspace by bulk stores; operand of Q h
+    static constexpr uint32_t PT = HT + 16384;             // P (only when o is wanted)
+    static constexpr uint32_t SMEM_BYTES = PT + (O ? 8192 : 0) + 1024;
+    static_assert(2 * (SMEM_BYTES + 4096) <= 228 * 1024, "two CTAs per SM");
+};
 }  // namespace f64
 
+template <bool O>
 __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_constant__ Tc64Params P) {
     wait_prerequisites();
-    using namespace f64;
+    using C = f64::Cfg<O>;
+    constexpr int STAGES = C::STAGES;
+    constexpr uint32_t KT = C::KT, VT = C::VT, QT = C::QT, STAGE_BYTES = C::STAGE_BYTES, VE = C::VE, PT = C::PT;
     const Problem& p = P.p;
     const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
     if (hdr->status != GDN_OK) return;
@@ -88,11 +97,10 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
     const int n = blockIdx.x / H, hd = blockIdx.x % H;
     const SeqGeom cg = seq_geom(p, n);
     const int c0 = cg.c0, nsteps = cg.n_chunks;
-    const bool want_o = p.o != nullptr;
 
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sm = align1024(smem_raw);
-    __shared__ __align__(16) float gl[kC], Gam[kC], ee[kC];
+    __shared__ __align__(16) float gl2[2][kC], Gam2[2][kC], ee2[2][kC];   // two sets: a step's gate arrays are made during the step before
     __shared__ uint64_t bar_full[STAGES], bar_mma;
     __shared__ uint32_t tmem_slot;
     const int warp = warp_id(), lane = threadIdx.x & 31;
@@ -118,10 +126,10 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
     auto fill = [&](int s) {
         const int stage = s % STAGES, tok0 = cg.chunk_tok0(c0 + s);
         unsigned char* st = sm + stage * STAGE_BYTES;
-        mbar_expect_tx(&bar_full[stage], want_o ? 24576 : 16384);
+        mbar_expect_tx(&bar_full[stage], STAGE_BYTES);
         tma_load_2d(st + KT, &P.tm_k, hd * D6, tok0, &bar_full[stage]);
         tma_load_2d(st + VT, &P.tm_v, hd * D6, tok0, &bar_full[stage]);
-        if (want_o) tma_load_2d(st + QT, &P.tm_q, hd * D6, tok0, &bar_full[stage]);
+        if (O) tma_load_2d(st + QT, &P.tm_q, hd * D6, tok0, &bar_full[stage]);
     };
     if (threadIdx.x == 0)
         for (int s = 0; s < STAGES && s < nsteps; ++s) fill(s);
@@ -134,66 +142,76 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
         st[4 * k] = v.x; st[4 * k + 1] = v.y; st[4 * k + 2] = v.z; st[4 * k + 3] = v.w;
     }
     const float* gamma = reinterpret_cast<const float*>(p.ws + p.L.gamma);
-    float gnext = (threadIdx.x < kC && nsteps > 0) ? gamma[((size_t)c0 * H + hd) * kC + threadIdx.x] : 0.f;
+    auto gate_row = [&](int step) { return gamma + ((size_t)(c0 + step) * H + hd) * kC; };
+    auto make_gates = [&](int set, float g, float gend) {
+        gl2[set][threadIdx.x] = g * kLog2e;
+        Gam2[set][threadIdx.x] = expf(g);
+        ee2[set][threadIdx.x] = ex2((gend - g) * kLog2e);
+    };
+    float gnext = 0.f, gend_next = 0.f;   // of the step after next
+    if (threadIdx.x < kC && nsteps > 0) {
+        make_gates(0, gate_row(0)[threadIdx.x], gate_row(0)[kC - 1]);
+        if (nsteps > 1) { gnext = gate_row(1)[threadIdx.x]; gend_next = gate_row(1)[kC - 1]; }
+    }
+    __syncthreads();
     bool ok = true;
     uint32_t mma_phase = 0;
-    int len_n = nsteps > 0 ? cg.chunk_len(c0) : 0;   // fetched a step ahead
 #pragma unroll 1
     for (int s = 0; s < nsteps; ++s) {
-        const int c = c0 + s, stage = s % STAGES, len = len_n;
-        if (s + 1 < nsteps) len_n = cg.chunk_len(c + 1);
+        const int c = c0 + s, stage = s % STAGES, len = cg.chunk_len(c);
         const size_t ch = (size_t)c * H + hd;
         unsigned char* tiles = sm + stage * STAGE_BYTES;
-        if (threadIdx.x == 32) bulk_wait_read<0>();   // the previous step's state tile has left shared memory
-        if (threadIdx.x < kC) {
-            gl[threadIdx.x] = gnext * kLog2e;
-            Gam[threadIdx.x] = expf(gnext);
-            if (s + 1 < nsteps) gnext = gamma[(ch + H) * kC + threadIdx.x];
-        }
-        __syncthreads();
-        if (threadIdx.x < kC) ee[threadIdx.x] = ex2(gl[kC - 1] - gl[threadIdx.x]);
+        unsigned char* HT = sm + C::HT + (s & 1) * 8192;
+        const float *gl = gl2[s & 1], *Gam = Gam2[s & 1], *ee = ee2[s & 1];
         ok = mbar_wait(&bar_full[stage], (s / STAGES) & 1);
         if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 40); break; }
         if (len < kC) {
             zero_tail_rows64(tiles + KT, len);
             zero_tail_rows64(tiles + VT, len);
-            if (want_o) zero_tail_rows64(tiles + QT, len);
+            if (O) zero_tail_rows64(tiles + QT, len);
+            __syncthreads();
         }
-        __syncthreads();
         const float Ge = Gam[kC - 1];
-        for (int t = threadIdx.x; t < kC * 8; t += blockDim.x) {   // Diag(e) V
-            const int i = t >> 3, cch = t & 7;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {   // Diag(e) V
+            const int i = (threadIdx.x >> 3) + 32 * t, cch = threadIdx.x & 7;
             float v[8];
             chunk_load(tiles + VT, 64, i, cch, v);
+            const float e = ee[i];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] *= ee[i];
+            for (int k = 0; k < 8; ++k) v[k] *= e;
             chunk_store(sm + VE, 64, i, cch, v);
         }
         // state entering the chunk -> bf16 tile: the workspace copy (and, for o, the MMA operand)
 #pragma unroll
         for (int k = 0; k < 2; ++k)
-            *reinterpret_cast<uint4*>(sm + HT + tile_chunk_off(64, r, (sc0 >> 3) + k)) = pack8(st + 8 * k);
+            *reinterpret_cast<uint4*>(HT + tile_chunk_off(64, r, (sc0 >> 3) + k)) = pack8(st + 8 * k);
         fence_async_smem();
         __syncthreads();
-        if (threadIdx.x == 32) {   // the tile leaves through the async proxy (generic global stores would stall the next proxy fence)
-            bulk_store(p.ws + p.L.hc + ch * 8192, sm + HT, 8192);
-            bulk_commit();
-        }
         if (warp == 0 && elect_one()) {
             tc_fence_after();
             mma_tile<64, 32, 64>(tmem + 0, op_mn_major(tiles + KT, 64), op_mn_major(sm + VE, 64), false);              // Kb^T V
             mma_tile<64, 32, 64>(tmem + 0 + LB, op_mn_major(tiles + KT, 64), op_mn_major(sm + VE + 64, 64), false);    // (columns 32..63)
-            if (want_o) {
+            if (O) {
                 mma_tile<64, 64, 64>(tmem + 64, op_k_major(tiles + QT, 64), op_k_major(tiles + KT, 64), false);         // Q K^T
-                mma_tile<64, 64, 64>(tmem + 128, op_k_major(tiles + QT, 64), op_mn_major(sm + HT, 64), false);          // Q h
+                mma_tile<64, 64, 64>(tmem + 128, op_k_major(tiles + QT, 64), op_mn_major(HT, 64), false);               // Q h
             }
+            // the tile leaves through the async proxy (generic global stores would stall the next proxy fence); waiting for the
+            // store of the step before to have read its tile, ahead of the commit, orders that read before the overwrite in the next step
+            bulk_store(p.ws + p.L.hc + ch * 8192, HT, 8192);
+            bulk_commit();
+            bulk_wait_read<1>();
             mma_commit(&bar_mma);
+        }
+        if (threadIdx.x < kC && s + 1 < nsteps) {
+            make_gates((s + 1) & 1, gnext, gend_next);
+            if (s + 2 < nsteps) { gnext = gate_row(s + 2)[threadIdx.x]; gend_next = gate_row(s + 2)[kC - 1]; }
         }
         GDN_WAIT_MMA(41)
         if (!ok) break;
-        // without o the stage's K and V have now been read for the last time: refill it while the state is updated
-        if (!want_o && threadIdx.x == 32 && s + STAGES < nsteps) fill(s + STAGES);
-        if (want_o) {   // o = scale (Gam_i (Q h)_i + (P V)_i)
+        // without o the slot's K and V have now been read for the last time: refill it while the state is updated
+        if (!O && threadIdx.x == 96 && s + STAGES < nsteps) fill(s + STAGES);
+        if (O) {   // o = scale (Gam_i (Q h)_i + (P V)_i)
 #pragma unroll 1
             for (int part = 0; part < 4; ++part) {
                 float v[8];
@@ -240,12 +258,12 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
             for (int j = 0; j < 8; ++j) st[8 * k + j] = fmaf(Ge, st[8 * k + j], bf[j]);
         }
         tc_fence_before();
-        if (want_o) {
+        if (O) {
             __syncthreads();   // every reader of this stage's tiles is done
             if (threadIdx.x == 0 && s + STAGES < nsteps) fill(s + STAGES);
         }
     }
-    if (threadIdx.x == 32) bulk_wait_read<0>();
+    if (warp == 0) bulk_wait_read<0>();
     if (p.hT && ok) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) *reinterpret_cast<float4*>(p.hT + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
@@ -589,13 +607,15 @@ static cudaError_t tc64_prologue(const Problem& p, cudaStream_t st) {
 }
 
 static cudaError_t tc64_fwd_pass(const Tc64Params& P, cudaStream_t st) {
-    static SmemLimitOnce once;
-    const cudaError_t e0 = once.ensure(tc64_fwd_kernel, f64::SMEM_BYTES);
+    static SmemLimitOnce once, once_o;
+    const bool o = P.p.o != nullptr;
+    const uint32_t smem = o ? f64::Cfg<true>::SMEM_BYTES : f64::Cfg<false>::SMEM_BYTES;
+    const cudaError_t e0 = o ? once_o.ensure(tc64_fwd_kernel<true>, smem) : once.ensure(tc64_fwd_kernel<false>, smem);
     if (e0 != cudaSuccess) return e0;
     const int chains = P.p.d.N * P.p.d.H;
     if (chains > 0) {
         StageScope t(ST_FSCAN, st);
-        launch_kernel(tc64_fwd_kernel, chains, kThreads64, f64::SMEM_BYTES, st, P);
+        launch_kernel(o ? tc64_fwd_kernel<true> : tc64_fwd_kernel<false>, chains, kThreads64, smem, st, P);
     }
     return cudaGetLastError();
 }
