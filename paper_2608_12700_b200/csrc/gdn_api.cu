@@ -95,7 +95,7 @@ VecPlan vec_plan(const gdn_desc& d) {
     VecPlan v{};
     v.padded = tc_padded_supported(d) && g_force_family != 1;
     const gdn_desc w = v.padded ? tc_padded_desc(d) : d;
-    v.inner = make_layout_vec(w, cw_tc_scratch_per_chunkhead());
+    v.inner = make_layout_vec(w);
     if (g_force_family == 1) v.inner.tc_scans = 0;   // (debug override: the FFMA kernels; the image regions stay unused)
     v.total = v.padded ? align_up(v.inner.total, 256) + tc_padded_extra_bytes(d, true) : v.inner.total;
     v.fwd_bytes = v.padded ? v.total : v.inner.fwd_end;

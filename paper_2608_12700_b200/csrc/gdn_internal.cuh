@@ -116,7 +116,7 @@ inline WsLayout make_layout_ffma(const gdn_desc& d) {
 
 // Layout of the channel-wise FFMA family: everything fp32; gamma is per channel ([CH, 64, d_k]), no chunk operator.
 inline bool vec_tc_scans(const gdn_desc& d) { return d.dtype == GDN_BF16 && d.d_k == 128 && d.d_v == 128; }
-inline WsLayout make_layout_vec(const gdn_desc& d, size_t scratch_per_ch) {
+inline WsLayout make_layout_vec(const gdn_desc& d) {
     WsLayout L{};
     const size_t Ttot = (size_t)d.B * (size_t)d.T;
     L.max_chunks = (int)((Ttot + kC - 1) / kC + (size_t)d.N);
@@ -149,9 +149,7 @@ inline WsLayout make_layout_vec(const gdn_desc& d, size_t scratch_per_ch) {
     L.img_dO = take(L.tc_scans ? CH * 16384 : 0);
     L.dhn = take(4 * CH * d.d_k * d.d_v);
     L.dU = take(4 * CH * kC * d.d_v);
-    L.scratch_per_ch = L.tc_scans ? scratch_per_ch : 0;   // (of the tensor-core kernels)
-    L.scratch = take(L.scratch_per_ch * CH);
-    L.total = o;
+    L.scratch = L.total = o;
     return L;
 }
 
@@ -243,7 +241,6 @@ cudaError_t vec_launch_fwd(const Problem& p, cudaStream_t st);
 cudaError_t vec_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st);
 // ... and its tensor-core route (bf16 I/O, d_k = d_v = 128; gdn_tc_cw.cu): forward (bwd = false) or backward.
 cudaError_t cw_tc_launch(const Problem& p, bool bwd, bool skip_recompute, cudaStream_t st);
-size_t cw_tc_scratch_per_chunkhead();
 
 // tcgen05 family (bf16 I/O, d_k = d_v = 128, delta rule on).
 extern thread_local int g_force_carries;   // form of the inter-chunk carries: 0 = chosen by shape, 1 = operator form, 2 = low-rank

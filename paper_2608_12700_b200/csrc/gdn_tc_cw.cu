@@ -12,14 +12,14 @@
 //     U = U~ - W h   dU = P^T dO' + K- dh''   (dh'' = Diag(Gam_e) dh')
 //     dP = tril(dO' U^T)   dW = -dU h^T   dXk = T^T dW   dXv = T^T dU   dA = -stril(dXk W^T + dXv U~^T)
 //     dQ~ = dO' h^T + dP K-     dK+ = dXk + dA K-     dK- = U dh''^T + dP^T Q~ + dA^T K+
-// and the gradients of the caller's tensors follow element by element (cw_post).  Four kernels beside the carries
+// and the gradients of the caller's tensors follow element by element.  Three kernels beside the carries
 // (tc_scan_cw in gdn_tc.cu):
 //   cw_scale  scaled operand tiles as bf16 tile images, gam; checks that |gam| stays below 80 (beyond that the split
 //             would need reference points inside the chunk): otherwise it records GDN_ERR_DECAY_RANGE, the kernels below
 //             stand down, and the FFMA sequence enqueued behind them computes the call (gdn_simt_vec.cu)
 //   cw_prep   [Q~;K+] K-^T, fp32 blocked inversion, W^T, U~^T, (P^T dO')^T, E               (tcgen05)
-//   cw_intra  the sixteen products of the gradient stage in five dependent steps (K#2 reuses T)   (tcgen05)
-//   cw_post   dq, dk, dv, db, dw, and dg by a reverse cumulative sum per channel
+//   cw_intra  the thirteen products of the gradient stage in four dependent steps (K#2 reuses T), and from them dq, dk, dv,
+//             db, dw, and dg by a reverse cumulative sum per channel                                  (tcgen05)
 // The tensor-core kernels are written straight-line (one CTA per SM walks over chunk-heads; one thread issues every
 // product and copy; CTA-wide barriers between the steps): the plain statement of the channel-wise path on tcgen05,
 // not a tuned one.  Accumulators live in one TMEM reservation at fixed column offsets; every wait is bounded.
@@ -47,10 +47,6 @@ __device__ __forceinline__ bool chunk_ctx(const Problem& p, ChunkCtx& x) {
     x.len = reinterpret_cast<const int32_t*>(p.ws + p.L.chunk_len)[c];
     return true;
 }
-
-// Per chunk-head scratch between cw_intra and cw_post (fp32): dQ~, dK+, dK-, dXv [64][128] each, and per key channel
-// rowdot(dh'', h + K-^T U) [128], the chunk-end part of the decay gradient.
-constexpr size_t S_DQ = 0, S_DKP = 32768, S_DKM = 65536, S_DXV = 98304, S_HH = 131072, S_BYTES = 131584;
 
 // ------------------------------------------------------------------------------------------------
 // cw_scale
@@ -412,7 +408,19 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// cw_intra
+// cw_intra: every gradient of one (chunk, head).
+//
+// Four dependent steps (products; [readout] what the threads make of them):
+//   1  (W h)^T ; (K- dh'')^T ; (P^T dO')^T            [U = U~ - W h ; dU = P^T dO' + K- dh'']
+//   2  dP = dO' U^T ; dXv^T = dU^T T ; under the readout dQ~^T = h dO'^T ; dK-^T = dh'' U^T        [tril ; dv, dw]
+//   3  dA = dXv U^T (K#2) ; under the readout dK+^T = -h dXv^T ; dQ~^T += K-^T dP^T ; Q~^T dP      [-stril]
+//   4  dK+^T += K-^T dA^T ; (Q~^T dP) += K+^T dA                                                   [dq, dk, db, dg]
+// What bounds it is HBM: 176 KB of operand images, 144 KB of gates, inputs and gammas, 144 KB of gradients per chunk-head.  The
+// gradients are made with features on the TMEM lanes and tokens on the columns: a warp's accesses to the gate vectors and
+// gradients are then whole 128-byte lines, all lanes work (a 64-row accumulator fills half of them), and the sums of dg
+// over the tokens of a chunk run along a thread's own columns.  So nothing passes through HBM between the products and the
+// elementwise part: with fp32 scratch and a kernel of its own (256 KB more traffic per chunk-head) the two took 300 us on
+// 4 x 16 heads of 2048 tokens, this kernel 262 us.
 // ------------------------------------------------------------------------------------------------
 namespace intracw {
 constexpr uint32_t QKM = 0;                 // [Q~ rows 0..63 ; K- rows 64..127] x 128         32 KB
@@ -428,19 +436,17 @@ constexpr uint32_t UT = DH + 32768;         // U^T  [128][64]                   
 constexpr uint32_t DUT = UT + 16384;        // dU^T [128][64]; later dXv^T [128][64]            16 KB
 constexpr uint32_t SMEM_BYTES = DUT + 16384 + 1024;
 constexpr uint32_t DA = TT, DP = PT, DXVT = DUT;   // (dA over T, dP over P, dXv^T over dU^T, each after its last reader)
-// TMEM columns (512 allocated, fixed offsets).  Accumulators with features on the lanes use all 128 lanes (M = 128);
-// token-major ones (M = 64) occupy lanes 0..15 of each lane quadrant.
-//   0..63     (W h)^T  -> dXv^T                    (M = 128)
-//   64..191   (K- dh'')^T | (P^T dO')^T (M = 128) -> K-^T U (M = 128) -> dK+ = dXk + dA K-   (M = 64, 128 columns)
-//   192..255  dP -> dA                              (M = 64)
-//   256..383  dQ~ = dO' h^T + dP K-                 (M = 64)
-//   384..511  dK- = U dh''^T + dP^T Q~ + dA^T K+    (M = 64)
-constexpr uint32_t C_A = 0, C_B = 64, C_PDO = 128, C_KP = 64, C_PP = 192, C_DQ = 256, C_KM = 384;
-constexpr uint32_t C_X = 64;   // K-^T U [128][128] over C_B | C_PDO (read by then), gone before dXk lands on C_KP
+// TMEM columns (512 allocated, fixed offsets): eight accumulators of 64 columns, features on the lanes except dP and dA
+// (token rows on lanes 0..15 of each quadrant).
+constexpr uint32_t C_A = 0, C_B = 64, C_PDO = 128, C_PP = 192, C_DQ = 256, C_KM = 320, C_KP = 384, C_KM2 = 448;
+constexpr int kWorkers = 512;               // 16 readout warps: lane quadrant = warp % 4, tokens 16 (warp / 4) ..
+                                            // (a seventeenth warp would cost every thread 32 of its 128 registers; warp 0 issues
+                                            // the products, warp 1 the loads)
+constexpr int kTok = 16;                    // tokens of a thread
 static_assert(SMEM_BYTES <= 220 * 1024, "shared memory budget");
 }  // namespace intracw
 
-__global__ void __launch_bounds__(kT, 1) cw_intra_kernel(Problem p) {
+__global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem p) {
     wait_prerequisites();
     using namespace intracw;
     const int H = p.d.H;
@@ -450,15 +456,14 @@ __global__ void __launch_bounds__(kT, 1) cw_intra_kernel(Problem p) {
     if ((int)blockIdx.x >= n_items) return;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sm = align1024(smem_raw);
-    __shared__ uint64_t bar_s, bar_a, bar_b, bar_k, bar_q, bar_mma;
+    __shared__ uint64_t bar_s, bar_a, bar_b, bar_k, bar_mma;
     __shared__ uint32_t tmem_slot;
-    __shared__ float end_sum[3][D];   // per key channel: rowdot(dh'', h) and the two halves of rowdot(dh'', K-^T U)
+    __shared__ float tot[4][D], end_part[4][D];   // per token group and channel: sum of dgam, part of the chunk-end term
     const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, grp = warp >> 2;
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
     if (threadIdx.x == 0) {
-        mbar_init(&bar_s, 1); mbar_init(&bar_a, 1); mbar_init(&bar_b, 1); mbar_init(&bar_k, 1); mbar_init(&bar_q, 1);
-        mbar_init(&bar_mma, 1);
+        mbar_init(&bar_s, 1); mbar_init(&bar_a, 1); mbar_init(&bar_b, 1); mbar_init(&bar_k, 1); mbar_init(&bar_mma, 1);
         fence_mbar_init();
     }
     if (warp == 0) { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
@@ -468,94 +473,97 @@ __global__ void __launch_bounds__(kT, 1) cw_intra_kernel(Problem p) {
     const uint32_t tmem = tmem_slot;
     const int f = q4 * 32 + lane;             // feature row of the M = 128 accumulators
     const int tr = q4 * 16 + (lane & 15);     // token row of the M = 64 accumulators (lanes 0..15 of the quadrant)
+    const int i0 = grp * kTok;                // first of this thread's 16 tokens
     const bool ga = lane < 16;
     bool ok = true;
     uint32_t mma_phase = 0, in_phase = 0;
-    // The tiles of a trip arrive in five groups, each loaded during the previous trip as soon as the last product that
-    // reads its region is done (look-ahead without a second buffer):
-    //   b  W^T, U~^T       after the first readout       s  h, dh''          after step 3
-    //   a  dO'             after step 2                  k  K-               after step 4
-    //      P               after step 3                  q  Q~, K+, T        after step 4 (needed from step 2 on)
-    bool pend_s = false, pend_a = false, pend_b = false, pend_k = false, pend_q = false;   // thread 0
-    auto load_s = [&](size_t c) {
+    // The tiles of a trip arrive in groups, each loaded during the previous trip as soon as the last product that reads its
+    // region is done (look-ahead without a second buffer):
+    //   b  W^T, U~^T     after the first readout          a  dO' after step 2, P after step 4
+    //   s  dh'' after step 2, h after step 4              k  Q~, K-, K+, T after step 4
+    bool pend_s = false, pend_a = false, pend_b = false, pend_k = false;   // the elected lane of warp 1
+    auto load_s1 = [&](size_t c) {
         mbar_expect_tx(&bar_s, 65536);
-        bulk_load(sm + HH, p.ws + p.L.hc + c * 32768, 32768, &bar_s);
         bulk_load(sm + DH, p.ws + p.L.dhn + c * 32768, 32768, &bar_s);
         pend_s = true;
     };
-    auto load_a = [&](size_t c) {
+    auto load_s2 = [&](size_t c) { bulk_load(sm + HH, p.ws + p.L.hc + c * 32768, 32768, &bar_s); };
+    auto load_a1 = [&](size_t c) {
         mbar_expect_tx(&bar_a, 24576);
         bulk_load(sm + DOT, p.ws + p.L.img_dO + c * 16384, 16384, &bar_a);
-        bulk_load(sm + PT, p.ws + p.L.Pm + c * 8192, 8192, &bar_a);
         pend_a = true;
     };
+    auto load_a2 = [&](size_t c) { bulk_load(sm + PT, p.ws + p.L.Pm + c * 8192, 8192, &bar_a); };
     auto load_b = [&](size_t c) {
         mbar_expect_tx(&bar_b, 32768);
         bulk_load(sm + WT, p.ws + p.L.img_W + c * 16384, 16384, &bar_b);
         bulk_load(sm + UTT, p.ws + p.L.img_U + c * 16384, 16384, &bar_b);
         pend_b = true;
     };
-    auto load_kq = [&](size_t c) {
+    auto load_k = [&](size_t c) {
         const char* iQKp = p.ws + p.L.img_QKp + c * 32768;
         const char* iKm = p.ws + p.L.img_Km + c * 16384;
-        mbar_expect_tx(&bar_k, 16384);
-        for (int cb = 0; cb < 2; ++cb) bulk_load(sm + QKM + cb * 16384 + 8192, iKm + cb * 8192, 8192, &bar_k);      // K-
-        pend_k = true;
-        mbar_expect_tx(&bar_q, 40960);
+        mbar_expect_tx(&bar_k, 57344);
         for (int cb = 0; cb < 2; ++cb) {
-            bulk_load(sm + QKM + cb * 16384, iQKp + cb * 16384, 8192, &bar_q);                                        // Q~
-            bulk_load(sm + KP + cb * 8192, iQKp + cb * 16384 + 8192, 8192, &bar_q);                                   // K+
+            bulk_load(sm + QKM + cb * 16384 + 8192, iKm + cb * 8192, 8192, &bar_k);             // K-
+            bulk_load(sm + QKM + cb * 16384, iQKp + cb * 16384, 8192, &bar_k);                  // Q~
+            bulk_load(sm + KP + cb * 8192, iQKp + cb * 16384 + 8192, 8192, &bar_k);             // K+
         }
-        bulk_load(sm + TT, p.ws + p.L.Tm + c * 8192, 8192, &bar_q);
-        pend_q = true;
+        bulk_load(sm + TT, p.ws + p.L.Tm + c * 8192, 8192, &bar_k);
+        pend_k = true;
     };
-    if (threadIdx.x == 0) { load_s(blockIdx.x); load_kq(blockIdx.x); load_b(blockIdx.x); load_a(blockIdx.x); }
+    if (warp == 1 && elect_one()) {
+        const size_t c = blockIdx.x;
+        load_s1(c); load_s2(c); load_k(c); load_b(c); load_a1(c); load_a2(c);
+    }
 #pragma unroll 1
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, in_phase ^= 1) {
         const size_t ch = (size_t)item;
         const bool has_next = item + (int)gridDim.x < n_items;
         const size_t chn = ch + gridDim.x;
-        float* scr = reinterpret_cast<float*>(p.ws + p.L.scratch + p.L.scratch_per_ch * ch);
+        ChunkInfo x;
+        x.c = item / H; x.hd = item % H;
+        x.tok0 = reinterpret_cast<const int32_t*>(p.ws + p.L.chunk_tok0)[x.c];
+        x.len = reinterpret_cast<const int32_t*>(p.ws + p.L.chunk_len)[x.c];
+        const size_t rs = (size_t)H * D, base = ((size_t)x.tok0 * H + x.hd) * D + (size_t)i0 * rs + f;   // this thread's channel of its first token
+        const int live = x.len - i0;          // tokens of this thread inside the sequence (may be negative)
         if (ok) {   // everything step 1 reads (the reverse carry left dh'' = Diag(Gam_e) dh', the form used here)
             ok = mbar_wait(&bar_s, in_phase) && mbar_wait(&bar_k, in_phase) && mbar_wait(&bar_b, in_phase) && mbar_wait(&bar_a, in_phase);
             if (!ok && threadIdx.x == 0) report_timeout(p.ws, 44);
-            if (ok && threadIdx.x == 0) pend_s = pend_k = pend_a = pend_b = false;
+            if (ok) pend_s = pend_k = pend_a = pend_b = false;
         }
         __syncthreads();
-        // ---- step 1: (W h)^T ; (K- dh'')^T ; (P^T dO')^T
+        // ---- step 1
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 128>(tmem + C_A, op_mn_major(sm + HH, 128), op_mn_major(sm + WT, 128), false);
             mma_tile<128, 64, 128>(tmem + C_B, op_mn_major(sm + DH, 128), op_k_major(sm + QKM, 128, 64), false);
             mma_tile<128, 64, 64>(tmem + C_PDO, op_mn_major(sm + DOT, 64), op_mn_major(sm + PT, 64), false);
             mma_commit(&bar_mma);
+            prefetch_l2_bulk(p.ws + p.L.gamma + ch * (kC * D * 4), kC * D * 4);   // for the last readout
         }
-        {   // rowdot(dh'', h) for the decay gradient of the chunk end, while the products run: two threads per state row
-            const int r = threadIdx.x >> 1, half = threadIdx.x & 1;
-            float hh = 0.f;
+        float end = 0.f;   // chunk-end term of the decay gradient: rowdot(dh'', h), and below sum_j k-_j (U dh''^T)_j
+        {
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
+            for (int k = 0; k < 4; ++k) {
                 float a[8], b[8];
-                chunk_load(sm + DH, 128, r, half * 8 + k, a);
-                chunk_load(sm + HH, 128, r, half * 8 + k, b);
+                chunk_load(sm + DH, 128, f, grp * 4 + k, a);
+                chunk_load(sm + HH, 128, f, grp * 4 + k, b);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) hh = fmaf(a[j], b[j], hh);
+                for (int j = 0; j < 8; ++j) end = fmaf(a[j], b[j], end);
             }
-            hh += __shfl_xor_sync(0xffffffffu, hh, 1);
-            if (half == 0) end_sum[0][r] = hh;
         }
         GDN_WAIT_MMA(45)
         if (ok) {   // U^T = U~^T - (W h)^T ; dU^T = (P^T dO')^T + (K- dh'')^T
-            const int i0 = grp * 32;
-#pragma unroll 1
-            for (int part = 0; part < 4; ++part) {
+#pragma unroll
+            for (int part = 0; part < 2; ++part) {
                 const int ib = i0 + part * 8;
                 float t[8], kb[8], pd[8], u[8];
                 tmem_ld8(tmem + lane_base + C_A + ib, t);
                 tmem_ld8(tmem + lane_base + C_B + ib, kb);
                 tmem_ld8(tmem + lane_base + C_PDO + ib, pd);
-                tmem_wait_ld();
                 chunk_load(sm + UTT, 128, f, ib >> 3, u);
+                tmem_wait_ld();
 #pragma unroll
                 for (int j = 0; j < 8; ++j) { u[j] -= t[j]; pd[j] += kb[j]; }
                 chunk_store(sm + UT, 128, f, ib >> 3, u);
@@ -565,88 +573,78 @@ __global__ void __launch_bounds__(kT, 1) cw_intra_kernel(Problem p) {
         tc_fence_before();
         fence_async_smem();
         __syncthreads();
-        if (ok && has_next && threadIdx.x == 0) load_b(chn);   // W^T (step 1) and U~^T (the readout) have been read for the last time
-        // ---- step 2: dP = dO' U^T ; dXv^T = dU^T T ; dO' h^T ; K-^T U ; under the readout U dh''^T
-        if (ok) {
-            ok = mbar_wait(&bar_q, in_phase);   // T (and Q~, K+, needed from step 3 on)
-            if (!ok && threadIdx.x == 0) report_timeout(p.ws, 51);
-            if (ok && threadIdx.x == 0) pend_q = false;
-        }
+        // ---- step 2
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<64, 64, 128>(tmem + C_PP, op_k_major(sm + DOT, 64), op_mn_major(sm + UT, 128), false);
             mma_tile<128, 64, 64>(tmem + C_A, op_k_major(sm + DUT, 128), op_mn_major(sm + TT, 64), false);
-            mma_tile<64, 128, 128>(tmem + C_DQ, op_k_major(sm + DOT, 64), op_k_major(sm + HH, 128), false);
-            // K-^T U: its row dots with dh'' are the part sum_j k-_j . (U dh''^T)_j of the decay gradient of the chunk end
-            mma_tile<128, 128, 64>(tmem + C_X, op_mn_major(sm + QKM, 128, 64), op_k_major(sm + UT, 128), false);
             mma_commit(&bar_mma);
-            // U dh''^T is only accumulated upon: it runs under the readout (its operands stay untouched until step 3's
-            // products, whose commit covers it, are done)
-            mma_tile<64, 128, 128>(tmem + C_KM, op_mn_major(sm + UT, 128), op_k_major(sm + DH, 128), false);
+            mma_tile<128, 64, 128>(tmem + C_DQ, op_k_major(sm + HH, 128), op_k_major(sm + DOT, 64), false);
+            mma_tile<128, 64, 128>(tmem + C_KM, op_k_major(sm + DH, 128), op_mn_major(sm + UT, 128), false);
+        }
+        if (warp == 1 && elect_one() && ok && has_next) load_b(chn);   // W^T (step 1) and U~^T (the readout) have been read for the last time
+        float wv[kTok];
+        uint32_t vraw[kTok];
+        {   // v and w of this thread's channel, while the products run
+            const uint16_t* vp = reinterpret_cast<const uint16_t*>(p.v) + base;
+            const float* wp = p.wv + base;
+#pragma unroll
+            for (int i = 0; i < kTok; ++i) {
+                wv[i] = i < live ? wp[i * rs] : 0.f;
+                vraw[i] = i < live ? vp[i * rs] : 0u;
+            }
         }
         GDN_WAIT_MMA(46)
-        if (ok && has_next && threadIdx.x == 0) {   // dO' has been read for the last time; P (by then dP) follows after step 3
-            mbar_expect_tx(&bar_a, 24576);
-            bulk_load(sm + DOT, p.ws + p.L.img_dO + chn * 16384, 16384, &bar_a);
-            pend_a = true;
-        }
         if (ok) {
-            const int j0 = grp * 32, i0 = grp * 32, c0 = grp * 64;
-#pragma unroll 1
-            for (int part = 0; part < 4; ++part) {
-                float v[8], x8[8];
-                const int ib = i0 + part * 8;
-                tmem_ld8(tmem + lane_base + C_PP + j0 + part * 8, v);     // dP rows on lanes 0..15
-                tmem_ld8(tmem + lane_base + C_A + ib, x8);                // dXv^T, all lanes
+            float x8[2][8], v[8];
+#pragma unroll
+            for (int part = 0; part < 2; ++part) tmem_ld8(tmem + lane_base + C_A + i0 + part * 8, x8[part]);   // dXv^T, all lanes
+            tmem_wait_ld();
+            __nv_bfloat16* dvp = reinterpret_cast<__nv_bfloat16*>(p.dv) + base;
+            float* dwp = p.dwv + base;
+#pragma unroll
+            for (int part = 0; part < 2; ++part) {   // dXv^T: operand tile (over dU^T, which its product has read); dv = w . dXv, dw = v . dXv
+                chunk_store(sm + DXVT, 128, f, (i0 >> 3) + part, x8[part]);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int i = part * 8 + j;
+                    if (i < live) {
+                        dvp[i * rs] = __float2bfloat16_rn(wv[i] * x8[part][j]);
+                        dwp[i * rs] = __uint_as_float(vraw[i] << 16) * x8[part][j];
+                    }
+                }
+            }
+#pragma unroll
+            for (int part = 0; part < 2; ++part) {   // dP = tril(dO' U^T), rows on lanes 0..15
+                const int jb = i0 + part * 8;
+                tmem_ld8(tmem + lane_base + C_PP + jb, v);
                 tmem_wait_ld();
-                if (ga) {   // dP = tril(dO' U^T)
-                    const int jb = j0 + part * 8;
+                if (ga) {
 #pragma unroll
                     for (int j = 0; j < 8; ++j) v[j] = (jb + j <= tr) ? v[j] : 0.f;
                     chunk_store(sm + DP, 64, tr, jb >> 3, v);
                 }
-                // dXv^T: operand tile (over dU^T, which its product has read) and, in fp32, the input of dv and dw
-                chunk_store(sm + DXVT, 128, f, ib >> 3, x8);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) scr[S_DXV / 4 + (ib + j) * D + f] = x8[j];   // token-major: a warp writes 128 contiguous bytes
             }
-            float xs = 0.f;   // rowdot(dh'', K-^T U): this thread's state row f, its half of the columns
-#pragma unroll 1
-            for (int part = 0; part < 8; ++part) {
-                float v[8], d8[8];
-                tmem_ld8(tmem + lane_base + C_X + c0 + part * 8, v);
-                chunk_load(sm + DH, 128, f, (c0 >> 3) + part, d8);
-                tmem_wait_ld();
-#pragma unroll
-                for (int j = 0; j < 8; ++j) xs = fmaf(v[j], d8[j], xs);
-            }
-            end_sum[1 + grp][f] = xs;
         }
         tc_fence_before();
         fence_async_smem();
         __syncthreads();
-        if (ok && threadIdx.x < D) scr[S_HH / 4 + threadIdx.x] = end_sum[0][threadIdx.x] + end_sum[1][threadIdx.x] + end_sum[2][threadIdx.x];
-        // ---- step 3 (K#2): dA = -stril(dXv U^T) (= -stril(dXk W^T + dXv U~^T): dXk = T^T dW = -dXv h^T, U = U~ - W h) ;
-        // dK+ = dXk = -dXv h^T ; dQ~ += dP K- ; dK- += dP^T Q~
+        // ---- step 3 (K#2): dA = -stril(dXv U^T) (= -stril(dXk W^T + dXv U~^T): dXk = T^T dW = -dXv h^T, U = U~ - W h)
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<64, 64, 128>(tmem + C_PP, op_mn_major(sm + DXVT, 128), op_mn_major(sm + UT, 128), false);
-            mma_tile<64, 128, 128>(tmem + C_KP, op_mn_major(sm + DXVT, 128), op_k_major(sm + HH, 128), false, /*neg_a=*/true);
-            mma_tile<64, 128, 64>(tmem + C_DQ, op_k_major(sm + DP, 64), op_mn_major(sm + QKM, 128, 64), true);
-            mma_tile<64, 128, 64>(tmem + C_KM, op_mn_major(sm + DP, 64), op_mn_major(sm + QKM, 128, 0), true);
             mma_commit(&bar_mma);
+            mma_tile<128, 64, 128>(tmem + C_KP, op_k_major(sm + HH, 128), op_mn_major(sm + DXVT, 128), false, /*neg_a=*/true);
+            mma_tile<128, 64, 64>(tmem + C_DQ, op_mn_major(sm + QKM, 128, 64), op_k_major(sm + DP, 64), true);
+            mma_tile<128, 64, 64>(tmem + C_KM2, op_mn_major(sm + QKM, 128, 0), op_mn_major(sm + DP, 64), false);
         }
         GDN_WAIT_MMA(47)
-        if (ok && has_next && threadIdx.x == 0) {   // h, dh'' (U dh''^T is done too) and dP (over P) have been read for the last time
-            load_s(chn);
-            bulk_load(sm + PT, p.ws + p.L.Pm + chn * 8192, 8192, &bar_a);   // (the second piece of group a)
-        }
+        if (warp == 1 && elect_one() && ok && has_next) { load_a1(chn); load_s1(chn); }   // dO' and dh'' have been read for the last time
         if (ok) {   // dA = -stril(.)  (over T, which step 2 has read)
-            const int j0 = grp * 32;
-#pragma unroll 1
-            for (int part = 0; part < 4; ++part) {
+#pragma unroll
+            for (int part = 0; part < 2; ++part) {
                 float v[8];
-                const int jb = j0 + part * 8;
+                const int jb = i0 + part * 8;
                 tmem_ld8(tmem + lane_base + C_PP + jb, v);
                 tmem_wait_ld();
                 if (ga) {
@@ -659,45 +657,95 @@ __global__ void __launch_bounds__(kT, 1) cw_intra_kernel(Problem p) {
         tc_fence_before();
         fence_async_smem();
         __syncthreads();
-        // ---- step 4: dK+ += dA K- ; dK- += dA^T K+
+        // ---- step 4
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
-            mma_tile<64, 128, 64>(tmem + C_KP, op_k_major(sm + DA, 64), op_mn_major(sm + QKM, 128, 64), true);
-            mma_tile<64, 128, 64>(tmem + C_KM, op_mn_major(sm + DA, 64), op_mn_major(sm + KP, 64), true);
+            mma_tile<128, 64, 64>(tmem + C_KP, op_mn_major(sm + QKM, 128, 64), op_k_major(sm + DA, 64), true);
+            mma_tile<128, 64, 64>(tmem + C_KM2, op_mn_major(sm + KP, 64), op_mn_major(sm + DA, 64), true);
             mma_commit(&bar_mma);
         }
+        const float* gp = reinterpret_cast<const float*>(p.ws + p.L.gamma) + ch * (kC * D) + i0 * D + f;
+        const uint16_t* qp = reinterpret_cast<const uint16_t*>(p.q) + base;
+        const uint16_t* kp = reinterpret_cast<const uint16_t*>(p.k) + base;
+        const float* bp = p.bv + base;
+        float g8[8], b8[8];
+        uint32_t q8[8], k8[8];
+        auto fetch = [&](int i1) {   // eight tokens' gates and inputs of this channel
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int i = i1 + j;
+                g8[j] = gp[i * D];
+                b8[j] = i < live ? bp[i * rs] : 0.f;
+                q8[j] = i < live ? qp[i * rs] : 0u;
+                k8[j] = i < live ? kp[i * rs] : 0u;
+            }
+        };
+        fetch(0);   // while the products run
         GDN_WAIT_MMA(49)
-        if (ok && has_next && threadIdx.x == 0) load_kq(chn);   // every tile of this trip has been read for the last time
+        if (warp == 1 && elect_one() && ok && has_next) { load_k(chn); load_s2(chn); load_a2(chn); }   // every tile has been read for the last time
+        float dgm[kTok];
         if (ok) {
-            const int c0 = grp * 64;
-#pragma unroll 1
-            for (int part = 0; part < 8; ++part) {
-                float a[8], b[8], c[8];
-                tmem_ld8(tmem + lane_base + C_DQ + c0 + part * 8, a);
-                tmem_ld8(tmem + lane_base + C_KP + c0 + part * 8, b);
-                tmem_ld8(tmem + lane_base + C_KM + c0 + part * 8, c);
+            __nv_bfloat16* dqp = reinterpret_cast<__nv_bfloat16*>(p.dq) + base;
+            __nv_bfloat16* dkp = reinterpret_cast<__nv_bfloat16*>(p.dk) + base;
+            float* dbp = p.dbv + base;
+#pragma unroll
+            for (int part = 0; part < 2; ++part) {
+                float dq[8], kr[8], km[8], km2[8];
+                tmem_ld8(tmem + lane_base + C_DQ + i0 + part * 8, dq);
+                tmem_ld8(tmem + lane_base + C_KP + i0 + part * 8, kr);
+                tmem_ld8(tmem + lane_base + C_KM + i0 + part * 8, km);
+                tmem_ld8(tmem + lane_base + C_KM2 + i0 + part * 8, km2);
                 tmem_wait_ld();
-                if (ga) {
-                    const int o = tr * D + c0 + part * 8;
-                    *reinterpret_cast<float4*>(scr + S_DQ / 4 + o) = make_float4(a[0], a[1], a[2], a[3]);
-                    *reinterpret_cast<float4*>(scr + S_DQ / 4 + o + 4) = make_float4(a[4], a[5], a[6], a[7]);
-                    *reinterpret_cast<float4*>(scr + S_DKP / 4 + o) = make_float4(b[0], b[1], b[2], b[3]);
-                    *reinterpret_cast<float4*>(scr + S_DKP / 4 + o + 4) = make_float4(b[4], b[5], b[6], b[7]);
-                    *reinterpret_cast<float4*>(scr + S_DKM / 4 + o) = make_float4(c[0], c[1], c[2], c[3]);
-                    *reinterpret_cast<float4*>(scr + S_DKM / 4 + o + 4) = make_float4(c[4], c[5], c[6], c[7]);
+                float dk[8], db[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float G = expf(g8[j]), iG = expf(-g8[j]);
+                    const float q = __uint_as_float(q8[j] << 16), k = __uint_as_float(k8[j] << 16);
+                    dq[j] *= G;                                      // dq = Gam . dQ~
+                    const float row = G * kr[j];                     // what multiplies b . k in the row role
+                    const float ucol = iG * km[j];
+                    const float col = fmaf(iG, km2[j], ucol);        // column role
+                    end = fmaf(k, ucol, end);
+                    dk[j] = fmaf(b8[j], row, col);
+                    db[j] = k * row;
+                    dgm[part * 8 + j] = q * dq[j] + k * b8[j] * row - k * col;
+                }
+                if (part == 0) fetch(8);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int i = part * 8 + j;
+                    if (i < live) {
+                        dqp[i * rs] = __float2bfloat16_rn(dq[j]);
+                        dkp[i * rs] = __float2bfloat16_rn(dk[j]);
+                        dbp[i * rs] = db[j];
+                    }
                 }
             }
+#pragma unroll
+            for (int i = kTok - 2; i >= 0; --i) dgm[i] += dgm[i + 1];   // sums from the end of this thread's tokens
+            tot[grp][f] = dgm[0];
+            end_part[grp][f] = end;
         }
         tc_fence_before();
-        __syncthreads();   // every reader of this trip's tiles and accumulators is done
+        __syncthreads();   // every reader of this trip's tiles and accumulators is done; the sums are visible
+        if (ok) {   // dg_j = sum_{i >= j} dgam_i + the chunk end
+            float run = (end_part[0][f] + end_part[1][f]) + (end_part[2][f] + end_part[3][f]);
+#pragma unroll
+            for (int k = 3; k > 0; --k)
+                if (k > grp) run += tot[k][f];
+            float* dgp = p.dgv + base;
+#pragma unroll
+            for (int i = 0; i < kTok; ++i)
+                if (i < live) dgp[i * rs] = run + dgm[i];
+        }
         if (!ok) break;
     }
-    if (threadIdx.x == 0 && !ok) {   // after a timeout a load may still be in flight: wait for it (bounded) before the CTA retires
+    if (warp == 1 && elect_one() && !ok) {   // after a timeout a load may still be in flight: wait for it (bounded) before the CTA retires
         // a group issued during the trip that gave up belongs to the next phase of its barrier; one pending since the top of
         // that trip to the current one.  Both parities are tried; the wrong one returns at once or after the bound.
-        uint64_t* bars[5] = {&bar_s, &bar_a, &bar_b, &bar_k, &bar_q};
-        const bool pend[5] = {pend_s, pend_a, pend_b, pend_k, pend_q};
-        for (int i = 0; i < 5; ++i)
+        uint64_t* bars[4] = {&bar_s, &bar_a, &bar_b, &bar_k};
+        const bool pend[4] = {pend_s, pend_a, pend_b, pend_k};
+        for (int i = 0; i < 4; ++i)
             if (pend[i]) { (void)mbar_wait(bars[i], in_phase); (void)mbar_wait(bars[i], in_phase ^ 1); }
     }
     tc_fence_before();
@@ -705,94 +753,13 @@ __global__ void __launch_bounds__(kT, 1) cw_intra_kernel(Problem p) {
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-// ------------------------------------------------------------------------------------------------
-// cw_post
-// ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kT) cw_post_kernel(Problem p) {
-    wait_prerequisites();
-    ChunkCtx x;
-    if (!chunk_ctx(p, x)) return;
-    if (reinterpret_cast<const WsHeader*>(p.ws)->status != GDN_OK) return;
-    extern __shared__ __align__(16) float dgam[];   // [64][D]
-    const int H = p.d.H;
-    const size_t base = ((size_t)x.tok0 * H + x.hd) * D, rs = (size_t)H * D;
-    const __nv_bfloat16* qp = reinterpret_cast<const __nv_bfloat16*>(p.q) + base;
-    const __nv_bfloat16* kp = reinterpret_cast<const __nv_bfloat16*>(p.k) + base;
-    const __nv_bfloat16* vp = reinterpret_cast<const __nv_bfloat16*>(p.v) + base;
-    __nv_bfloat16* dqp = reinterpret_cast<__nv_bfloat16*>(p.dq) + base;
-    __nv_bfloat16* dkp = reinterpret_cast<__nv_bfloat16*>(p.dk) + base;
-    __nv_bfloat16* dvp = reinterpret_cast<__nv_bfloat16*>(p.dv) + base;
-    const float* wsG = reinterpret_cast<const float*>(p.ws + p.L.gamma) + (size_t)x.ch * kC * D;
-    const float* scr = reinterpret_cast<const float*>(p.ws + p.L.scratch + p.L.scratch_per_ch * x.ch);
-    const float *dQ = scr + S_DQ / 4, *dKp = scr + S_DKP / 4, *dKm = scr + S_DKM / 4;
-    const float *dXv = scr + S_DXV / 4, *hh = scr + S_HH / 4;
-    // a thread owns four adjacent channels and every eighth token: 16-byte accesses, coalesced rows
-    const int r4 = (threadIdx.x & 31) * 4;
-#pragma unroll 2
-    for (int i = threadIdx.x >> 5; i < kC; i += kT / 32) {
-        const int t = i * D + r4;
-        const bool live = i < x.len;
-        const float4 g4 = *reinterpret_cast<const float4*>(wsG + t), a4 = *reinterpret_cast<const float4*>(dQ + t);
-        const float4 p4 = *reinterpret_cast<const float4*>(dKp + t), m4 = *reinterpret_cast<const float4*>(dKm + t);
-        const float4 x4 = *reinterpret_cast<const float4*>(dXv + t);
-        float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f), w4 = b4;
-        uint2 qr = make_uint2(0, 0), kr = qr, vr = qr;
-        if (live) {
-            b4 = *reinterpret_cast<const float4*>(p.bv + base + i * rs + r4);
-            w4 = *reinterpret_cast<const float4*>(p.wv + base + i * rs + r4);
-            qr = *reinterpret_cast<const uint2*>(qp + i * rs + r4);
-            kr = *reinterpret_cast<const uint2*>(kp + i * rs + r4);
-            vr = *reinterpret_cast<const uint2*>(vp + i * rs + r4);
-        }
-        const float g[4] = {g4.x, g4.y, g4.z, g4.w}, dqt[4] = {a4.x, a4.y, a4.z, a4.w}, dkp4[4] = {p4.x, p4.y, p4.z, p4.w};
-        const float dkm4[4] = {m4.x, m4.y, m4.z, m4.w}, xv[4] = {x4.x, x4.y, x4.z, x4.w};
-        const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, ww[4] = {w4.x, w4.y, w4.z, w4.w};
-        const float q[4] = {bf16_lo(qr.x), bf16_hi(qr.x), bf16_lo(qr.y), bf16_hi(qr.y)};
-        const float k[4] = {bf16_lo(kr.x), bf16_hi(kr.x), bf16_lo(kr.y), bf16_hi(kr.y)};
-        const float v[4] = {bf16_lo(vr.x), bf16_hi(vr.x), bf16_lo(vr.y), bf16_hi(vr.y)};
-        float dq[4], dk[4], db[4], dv[4], dw[4], dgm[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float G = expf(g[j]), iG = expf(-g[j]);
-            dq[j] = G * dqt[j];                       // dq = Gam . dQ~
-            const float row = G * dkp4[j];            // what multiplies b . k in the row role
-            const float col = iG * dkm4[j];           // column role
-            dk[j] = fmaf(bb[j], row, col);
-            db[j] = k[j] * row;
-            dgm[j] = q[j] * dq[j] + k[j] * bb[j] * row - k[j] * col;
-            dv[j] = ww[j] * xv[j];                    // dv = w . dXv
-            dw[j] = v[j] * xv[j];                     // dw = v . dXv
-        }
-        *reinterpret_cast<float4*>(dgam + t) = make_float4(dgm[0], dgm[1], dgm[2], dgm[3]);
-        if (live) {
-            *reinterpret_cast<uint2*>(dqp + i * rs + r4) = make_uint2(pack_bf16(dq[0], dq[1]), pack_bf16(dq[2], dq[3]));
-            *reinterpret_cast<uint2*>(dkp + i * rs + r4) = make_uint2(pack_bf16(dk[0], dk[1]), pack_bf16(dk[2], dk[3]));
-            *reinterpret_cast<uint2*>(dvp + i * rs + r4) = make_uint2(pack_bf16(dv[0], dv[1]), pack_bf16(dv[2], dv[3]));
-            *reinterpret_cast<float4*>(p.dbv + base + i * rs + r4) = make_float4(db[0], db[1], db[2], db[3]);
-            *reinterpret_cast<float4*>(p.dwv + base + i * rs + r4) = make_float4(dw[0], dw[1], dw[2], dw[3]);
-        }
-    }
-    __syncthreads();
-    // the chunk end collects rowdot(dh'', h + K-^T U) (from cw_intra); then dg_j = sum_{i >= j} dgam_i per channel
-    if (threadIdx.x < D) {
-        const int r = threadIdx.x;
-        float run = hh[r];
-        for (int i = kC - 1; i >= 0; --i) {
-            run += dgam[i * D + r];
-            if (i < x.len) p.dgv[base + i * rs + r] = run;
-        }
-    }
-}
-
 }  // namespace
 
 #undef GDN_WAIT_MMA
 
 // Host side: the channel-wise calls on this route (bf16 I/O, d_k = d_v = 128).
-size_t cw_tc_scratch_per_chunkhead() { return S_BYTES; }
-
 cudaError_t cw_tc_launch(const Problem& p, bool bwd, bool skip_recompute, cudaStream_t st) {
-    static SmemLimitOnce once_scale, once_prep, once_intra, once_post;
+    static SmemLimitOnce once_scale, once_prep, once_intra;
     const int CH = p.L.max_chunks * p.d.H, chains = p.d.N * p.d.H;
     cudaError_t e = launch_table(p, st);
     if (e != cudaSuccess) return e;
@@ -813,11 +780,8 @@ cudaError_t cw_tc_launch(const Problem& p, bool bwd, bool skip_recompute, cudaSt
         int dev = 0, sms = 148;
         if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const int grid = CH < sms ? CH : sms;
-        const uint32_t sm_post = sizeof(float) * kC * D;
         if ((e = once_intra.ensure(cw_intra_kernel, intracw::SMEM_BYTES)) != cudaSuccess) return e;
-        if ((e = once_post.ensure(cw_post_kernel, sm_post)) != cudaSuccess) return e;
-        { StageScope t(ST_INTRA, st); launch_kernel(cw_intra_kernel, grid, kT, intracw::SMEM_BYTES, st, p); }
-        { StageScope t(ST_POST, st); launch_kernel(cw_post_kernel, CH, kT, sm_post, st, p); }
+        { StageScope t(ST_INTRA, st); launch_kernel(cw_intra_kernel, grid, intracw::kWorkers, intracw::SMEM_BYTES, st, p); }
     }
     return cudaGetLastError();
 }
