@@ -420,7 +420,8 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
 // gradients are then whole 128-byte lines, all lanes work (a 64-row accumulator fills half of them), and the sums of dg
 // over the tokens of a chunk run along a thread's own columns.  So nothing passes through HBM between the products and the
 // elementwise part: with fp32 scratch and a kernel of its own (256 KB more traffic per chunk-head) the two took 300 us on
-// 4 x 16 heads of 2048 tokens, this kernel 262 us.
+// 4 x 16 heads of 2048 tokens, this kernel 208 us.
+// (L2 prefetches of what the elementwise part reads, a trip ahead, made it slower: 481 -> 495 us for the call.)
 // ------------------------------------------------------------------------------------------------
 namespace intracw {
 constexpr uint32_t QKM = 0;                 // [Q~ rows 0..63 ; K- rows 64..127] x 128         32 KB
@@ -512,6 +513,13 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
         bulk_load(sm + TT, p.ws + p.L.Tm + c * 8192, 8192, &bar_k);
         pend_k = true;
     };
+    auto chunk_of = [&](int it) {
+        ChunkInfo x;
+        x.c = it / H; x.hd = it % H; x.ch = it;
+        x.tok0 = reinterpret_cast<const int32_t*>(p.ws + p.L.chunk_tok0)[x.c];
+        x.len = reinterpret_cast<const int32_t*>(p.ws + p.L.chunk_len)[x.c];
+        return x;
+    };
     if (warp == 1 && elect_one()) {
         const size_t c = blockIdx.x;
         load_s1(c); load_s2(c); load_k(c); load_b(c); load_a1(c); load_a2(c);
@@ -521,12 +529,10 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
         const size_t ch = (size_t)item;
         const bool has_next = item + (int)gridDim.x < n_items;
         const size_t chn = ch + gridDim.x;
-        ChunkInfo x;
-        x.c = item / H; x.hd = item % H;
-        x.tok0 = reinterpret_cast<const int32_t*>(p.ws + p.L.chunk_tok0)[x.c];
-        x.len = reinterpret_cast<const int32_t*>(p.ws + p.L.chunk_len)[x.c];
+        const ChunkInfo x = chunk_of(item);
         const size_t rs = (size_t)H * D, base = ((size_t)x.tok0 * H + x.hd) * D + (size_t)i0 * rs + f;   // this thread's channel of its first token
         const int live = x.len - i0;          // tokens of this thread inside the sequence (may be negative)
+        const bool whole = live >= kTok;      // (two copies of the accesses: a condition at each of them costs more than it skips)
         if (ok) {   // everything step 1 reads (the reverse carry left dh'' = Diag(Gam_e) dh', the form used here)
             ok = mbar_wait(&bar_s, in_phase) && mbar_wait(&bar_k, in_phase) && mbar_wait(&bar_b, in_phase) && mbar_wait(&bar_a, in_phase);
             if (!ok && threadIdx.x == 0) report_timeout(p.ws, 44);
@@ -540,7 +546,6 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
             mma_tile<128, 64, 128>(tmem + C_B, op_mn_major(sm + DH, 128), op_k_major(sm + QKM, 128, 64), false);
             mma_tile<128, 64, 64>(tmem + C_PDO, op_mn_major(sm + DOT, 64), op_mn_major(sm + PT, 64), false);
             mma_commit(&bar_mma);
-            prefetch_l2_bulk(p.ws + p.L.gamma + ch * (kC * D * 4), kC * D * 4);   // for the last readout
         }
         float end = 0.f;   // chunk-end term of the decay gradient: rowdot(dh'', h), and below sum_j k-_j (U dh''^T)_j
         {
@@ -588,10 +593,12 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
         {   // v and w of this thread's channel, while the products run
             const uint16_t* vp = reinterpret_cast<const uint16_t*>(p.v) + base;
             const float* wp = p.wv + base;
+            if (whole) {
 #pragma unroll
-            for (int i = 0; i < kTok; ++i) {
-                wv[i] = i < live ? wp[i * rs] : 0.f;
-                vraw[i] = i < live ? vp[i * rs] : 0u;
+                for (int i = 0; i < kTok; ++i) { wv[i] = wp[i * rs]; vraw[i] = vp[i * rs]; }
+            } else {
+#pragma unroll
+                for (int i = 0; i < kTok; ++i) { wv[i] = i < live ? wp[i * rs] : 0.f; vraw[i] = i < live ? vp[i * rs] : 0u; }
             }
         }
         GDN_WAIT_MMA(46)
@@ -608,7 +615,7 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int i = part * 8 + j;
-                    if (i < live) {
+                    if (whole || i < live) {
                         dvp[i * rs] = __float2bfloat16_rn(wv[i] * x8[part][j]);
                         dwp[i * rs] = __uint_as_float(vraw[i] << 16) * x8[part][j];
                     }
@@ -671,13 +678,21 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
         float g8[8], b8[8];
         uint32_t q8[8], k8[8];
         auto fetch = [&](int i1) {   // eight tokens' gates and inputs of this channel
+            if (whole) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int i = i1 + j;
-                g8[j] = gp[i * D];
-                b8[j] = i < live ? bp[i * rs] : 0.f;
-                q8[j] = i < live ? qp[i * rs] : 0u;
-                k8[j] = i < live ? kp[i * rs] : 0u;
+                for (int j = 0; j < 8; ++j) {
+                    const int i = i1 + j;
+                    g8[j] = gp[i * D]; b8[j] = bp[i * rs]; q8[j] = qp[i * rs]; k8[j] = kp[i * rs];
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int i = i1 + j;
+                    g8[j] = gp[i * D];
+                    b8[j] = i < live ? bp[i * rs] : 0.f;
+                    q8[j] = i < live ? qp[i * rs] : 0u;
+                    k8[j] = i < live ? kp[i * rs] : 0u;
+                }
             }
         };
         fetch(0);   // while the products run
@@ -714,7 +729,7 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int i = part * 8 + j;
-                    if (i < live) {
+                    if (whole || i < live) {
                         dqp[i * rs] = __float2bfloat16_rn(dq[j]);
                         dkp[i * rs] = __float2bfloat16_rn(dk[j]);
                         dbp[i * rs] = db[j];
@@ -736,7 +751,7 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
             float* dgp = p.dgv + base;
 #pragma unroll
             for (int i = 0; i < kTok; ++i)
-                if (i < live) dgp[i * rs] = run + dgm[i];
+                if (whole || i < live) dgp[i * rs] = run + dgm[i];
         }
         if (!ok) break;
     }
