@@ -186,6 +186,11 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
 #pragma unroll
         for (int k = 0; k < 2; ++k)
             *reinterpret_cast<uint4*>(HT + tile_chunk_off(64, r, (sc0 >> 3) + k)) = pack8(st + 8 * k);
+        // the next step's gate arrays (read from the top of that step on: this step's barrier publishes them)
+        if (threadIdx.x < kC && s + 1 < nsteps) {
+            make_gates((s + 1) & 1, gnext, gend_next);
+            if (s + 2 < nsteps) { gnext = gate_row(s + 2)[threadIdx.x]; gend_next = gate_row(s + 2)[kC - 1]; }
+        }
         fence_async_smem();
         __syncthreads();
         if (warp == 0 && elect_one()) {
@@ -202,10 +207,6 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
             bulk_commit();
             bulk_wait_read<1>();
             mma_commit(&bar_mma);
-        }
-        if (threadIdx.x < kC && s + 1 < nsteps) {
-            make_gates((s + 1) & 1, gnext, gend_next);
-            if (s + 2 < nsteps) { gnext = gate_row(s + 2)[threadIdx.x]; gend_next = gate_row(s + 2)[kC - 1]; }
         }
         GDN_WAIT_MMA(41)
         if (!ok) break;
