@@ -60,9 +60,8 @@ Path pick_path(const gdn_desc& d) {
     if (d.dtype == GDN_F32) return Path::SimtF32;
     if (d.dtype == GDN_BF16) {
         if (g_force_family == 1) return Path::SimtBf16;
-        if (tc_supported(d)) return Path::TcBf16;
         if (tc64_supported(d)) return Path::Tc64Bf16;
-        if (tc_padded_supported(d)) return Path::TcBf16Padded;
+        if (tc_supported(d)) return d.d_k == 128 && d.d_v == 128 ? Path::TcBf16 : Path::TcBf16Padded;
         return Path::SimtBf16;
     }
     return Path::None;
@@ -71,16 +70,9 @@ Path pick_path(const gdn_desc& d) {
 WsLayout layout_for(const gdn_desc& d) {
     // tcgen05 path: every factor, state and additive term of the carries is a bf16 tile image.
     // The d = 128 family keeps the chunk operator Nm and the additive term Bf only when its carries use them.
-    if (pick_path(d) == Path::TcBf16) return make_layout(d, 2, 2, 0, !tc_carries_lowrank(d));
+    // A head dimension of 64 takes the workspace of 128: its tiles are half zero.
+    if (pick_path(d) == Path::TcBf16 || pick_path(d) == Path::TcBf16Padded) return make_layout(tc_padded_desc(d), 2, 2, 0, !tc_carries_lowrank(d));
     if (pick_path(d) == Path::Tc64Bf16) return make_layout(d, 2, 2, 0);
-    if (pick_path(d) == Path::TcBf16Padded) {   // the widened problem's layout, then the padded copies; one size for both calls
-        const gdn_desc w = tc_padded_desc(d);
-        WsLayout L = make_layout(w, 2, 2, 0, !tc_carries_lowrank(w));
-        L.scratch = align_up(L.total, 256);
-        L.total = L.scratch + tc_padded_extra_bytes(d, false);
-        L.fwd_end = L.total;
-        return L;
-    }
     return make_layout_ffma(d);   // the FFMA kernels keep everything in fp32, whatever the I/O dtype
 }
 
@@ -97,7 +89,7 @@ VecPlan vec_plan(const gdn_desc& d) {
     const gdn_desc w = v.padded ? tc_padded_desc(d) : d;
     v.inner = make_layout_vec(w);
     if (g_force_family == 1) v.inner.tc_scans = 0;   // (debug override: the FFMA kernels; the image regions stay unused)
-    v.total = v.padded ? align_up(v.inner.total, 256) + tc_padded_extra_bytes(d, true) : v.inner.total;
+    v.total = v.padded ? align_up(v.inner.total, 256) + tc_padded_extra_bytes(d) : v.inner.total;
     v.fwd_bytes = v.padded ? v.total : v.inner.fwd_end;
     return v;
 }
@@ -176,13 +168,8 @@ gdn_status gdn_fwd_recompute(const gdn_desc* desc, const void* q, const void* k,
     p.ws = static_cast<char*>(workspace);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const Path path = pick_path(*desc);
-    cudaError_t e;
-    if (path == Path::TcBf16Padded) {
-        const gdn_desc w = tc_padded_desc(*desc);
-        e = tc_padded_launch(p, make_layout(w, 2, 2, 0, !tc_carries_lowrank(w)), false, false, false, st);
-    } else {
-        e = path == Path::TcBf16 ? tc_launch_fwd(p, st) : path == Path::Tc64Bf16 ? tc64_launch_fwd(p, st) : simt_launch_fwd(p, st);
-    }
+    const cudaError_t e = path == Path::TcBf16 || path == Path::TcBf16Padded ? tc_launch_fwd(p, st)
+                          : path == Path::Tc64Bf16 ? tc64_launch_fwd(p, st) : simt_launch_fwd(p, st);
     return e == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }
 
@@ -203,14 +190,8 @@ gdn_status gdn_bwd(const gdn_desc* desc, const void* q, const void* k, const voi
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const bool fresh = workspace_is_fresh_from_fwd != 0;
     const Path path = pick_path(*desc);
-    cudaError_t e;
-    if (path == Path::TcBf16Padded) {
-        const gdn_desc w = tc_padded_desc(*desc);
-        e = tc_padded_launch(p, make_layout(w, 2, 2, 0, !tc_carries_lowrank(w)), true, fresh, false, st);
-    } else {
-        e = path == Path::TcBf16 ? tc_launch_bwd(p, fresh, st)
-            : path == Path::Tc64Bf16 ? tc64_launch_bwd(p, fresh, st) : simt_launch_bwd(p, fresh, st);
-    }
+    const cudaError_t e = path == Path::TcBf16 || path == Path::TcBf16Padded ? tc_launch_bwd(p, fresh, st)
+                          : path == Path::Tc64Bf16 ? tc64_launch_bwd(p, fresh, st) : simt_launch_bwd(p, fresh, st);
     return e == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }
 
@@ -245,7 +226,7 @@ gdn_status gdn_fwd_recompute_channelwise(const gdn_desc* desc, const void* q, co
     p.q = q; p.k = k; p.v = v; p.gv = g; p.bv = b; p.wv = w; p.h0 = h0; p.cu = cu; p.o = o; p.hT = hT;
     p.ws = static_cast<char*>(workspace);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    const cudaError_t e = plan.padded ? tc_padded_launch(p, plan.inner, false, false, true, st) : vec_launch_fwd(p, st);
+    const cudaError_t e = plan.padded ? tc_padded_launch(p, plan.inner, false, false, st) : vec_launch_fwd(p, st);
     return e == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }
 
@@ -273,7 +254,7 @@ gdn_status gdn_bwd_channelwise(const gdn_desc* desc, const void* q, const void* 
     p.ws = static_cast<char*>(workspace);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const bool fresh = workspace_is_fresh_from_fwd != 0;
-    const cudaError_t e = plan.padded ? tc_padded_launch(p, plan.inner, true, fresh, true, st) : vec_launch_bwd(p, fresh, st);
+    const cudaError_t e = plan.padded ? tc_padded_launch(p, plan.inner, true, fresh, st) : vec_launch_bwd(p, fresh, st);
     return e == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }
 

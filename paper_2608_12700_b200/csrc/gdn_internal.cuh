@@ -242,7 +242,7 @@ cudaError_t vec_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t s
 // ... and its tensor-core route (bf16 I/O, d_k = d_v = 128; gdn_tc_cw.cu): forward (bwd = false) or backward.
 cudaError_t cw_tc_launch(const Problem& p, bool bwd, bool skip_recompute, cudaStream_t st);
 
-// tcgen05 family (bf16 I/O, d_k = d_v = 128, delta rule on).
+// tcgen05 family (bf16 I/O; tiles of 128 features, a head dimension of 64 fills half of them).
 extern thread_local int g_force_carries;   // form of the inter-chunk carries: 0 = chosen by shape, 1 = operator form, 2 = low-rank
 extern thread_local int g_inject_timeout;   // debugging hook: the next gdn_bwd of this family provokes a device-side time-out
 bool tc_supported(const gdn_desc& d);
@@ -255,12 +255,11 @@ cudaError_t tc_launch_fwd(const Problem& p, cudaStream_t st);
 cudaError_t tc_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st);
 
 
-// bf16 shapes with a head dimension of 64, zero-padded onto the d = 128 kernels (gdn_pad.cu); `channelwise`: the call has
-// gate vectors, which are padded too, and the widened problem runs through vec_launch_fwd / vec_launch_bwd.
+// Channel-wise calls with bf16 I/O and a head dimension of 64, zero-padded onto the d = 128 kernels (gdn_pad.cu).
 bool tc_padded_supported(const gdn_desc& d);
 gdn_desc tc_padded_desc(const gdn_desc& d);          // the widened descriptor (d_k = d_v = 128)
-size_t tc_padded_extra_bytes(const gdn_desc& d, bool channelwise);   // bytes of padded copies behind the widened problem's own workspace
-cudaError_t tc_padded_launch(const Problem& p, const WsLayout& inner, bool bwd, bool skip_recompute, bool channelwise, cudaStream_t st);
+size_t tc_padded_extra_bytes(const gdn_desc& d);     // bytes of padded copies behind the widened problem's own workspace
+cudaError_t tc_padded_launch(const Problem& p, const WsLayout& inner, bool bwd, bool skip_recompute, cudaStream_t st);
 
 // tcgen05 family for the scalar-gate recurrence (bf16 I/O, d_k = d_v = 64, delta rule off).
 bool tc64_supported(const gdn_desc& d);

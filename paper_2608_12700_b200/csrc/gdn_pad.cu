@@ -1,5 +1,5 @@
-// bf16 shapes with a head dimension of 64 on the tcgen05 d = 128 kernels (scalar gates and channel-wise calls alike): the narrow dimension is padded
-// with zeros to 128.  The recurrence is exact under this padding: a zero key/query column adds nothing to any dot
+// Channel-wise calls with bf16 I/O and a head dimension of 64 on the tcgen05 d = 128 kernels: the narrow dimension is padded
+// with zeros to 128 (calls with scalar gates need no copies: their kernels read a narrow tensor as if it were padded).  The recurrence is exact under this padding: a zero key/query column adds nothing to any dot
 // product and leaves its state row at zero; a zero value / dO column evolves independently of the others (state
 // columns never mix) and yields zero gradients.  The padded copies live in the caller's workspace behind the
 // kernels' own regions; small copy kernels widen the inputs before and narrow the outputs after the three main kernels.
@@ -63,13 +63,13 @@ int grid_for(size_t items) {
 
 struct PadPlan {
     size_t q, k, v, dO, dq, dk, dv, o, h0, dhT, dh0, hT;   // byte offsets from the start of the pad region
-    size_t g, b, w, dg, db, dw;                              // channel-wise calls only: the gate vectors and their gradients
+    size_t g, b, w, dg, db, dw;                              // the gate vectors and their gradients
     size_t end;
 };
-PadPlan plan_for(const gdn_desc& d, bool channelwise) {
+PadPlan plan_for(const gdn_desc& d) {
     PadPlan P{};
     const size_t rows = (size_t)d.B * d.T * d.H, tok = align_up(rows * 128 * 2, 256), st = align_up((size_t)d.N * d.H * 128 * 128 * 4, 256);
-    const size_t gate = channelwise ? align_up(rows * 128 * 4, 256) : 0;
+    const size_t gate = align_up(rows * 128 * 4, 256);
     size_t o = 0;
     auto take = [&](size_t bytes) { const size_t r = o; o += bytes; return r; };
     P.q = take(d.d_k == 64 ? tok : 0); P.k = take(d.d_k == 64 ? tok : 0); P.dq = take(d.d_k == 64 ? tok : 0); P.dk = take(d.d_k == 64 ? tok : 0);
@@ -92,15 +92,14 @@ gdn_desc tc_padded_desc(const gdn_desc& d) {
     w.d_k = w.d_v = 128;
     return w;
 }
-size_t tc_padded_extra_bytes(const gdn_desc& d, bool channelwise) { return plan_for(d, channelwise).end; }
+size_t tc_padded_extra_bytes(const gdn_desc& d) { return plan_for(d).end; }
 
 // `inner` is the layout of the widened problem; the pad region starts at inner.total.
-// With `channelwise` the widened problem is a channel-wise call: its gate vectors are widened and their gradients
-// narrowed as well (a padded key channel has decay 1 and erase gate 0, a padded value channel write gate 0; with zero
+// The gate vectors are widened and their gradients narrowed as well (a padded key channel has decay 1 and erase gate 0, a padded value channel write gate 0; with zero
 // keys, queries and values there, every product is what it was).
-cudaError_t tc_padded_launch(const Problem& p, const WsLayout& inner, bool bwd, bool skip_recompute, bool channelwise, cudaStream_t st) {
+cudaError_t tc_padded_launch(const Problem& p, const WsLayout& inner, bool bwd, bool skip_recompute, cudaStream_t st) {
     const gdn_desc& d = p.d;
-    const PadPlan pl = plan_for(d, channelwise);
+    const PadPlan pl = plan_for(d);
     char* pad = p.ws + align_up(inner.total, 256);
     const size_t rows = (size_t)p.Ttot * d.H, chains = (size_t)d.N * d.H;
     Problem w = p;
@@ -125,12 +124,12 @@ cudaError_t tc_padded_launch(const Problem& p, const WsLayout& inner, bool bwd, 
         return reinterpret_cast<const float*>(pad + off);
     };
     const bool fresh = bwd && skip_recompute;   // the widened forward inputs are still in the workspace
-    if (channelwise && d.d_k == 64) {
+    if (d.d_k == 64) {
         if (!fresh) { w.gv = widen_gate(p.gv, pl.g); w.bv = widen_gate(p.bv, pl.b); }
         else { w.gv = reinterpret_cast<const float*>(pad + pl.g); w.bv = reinterpret_cast<const float*>(pad + pl.b); }
         if (bwd) { w.dgv = reinterpret_cast<float*>(pad + pl.dg); w.dbv = reinterpret_cast<float*>(pad + pl.db); }
     }
-    if (channelwise && d.d_v == 64) {
+    if (d.d_v == 64) {
         if (!fresh) w.wv = widen_gate(p.wv, pl.w); else w.wv = reinterpret_cast<const float*>(pad + pl.w);
         if (bwd) w.dwv = reinterpret_cast<float*>(pad + pl.dw);
     }
@@ -151,8 +150,7 @@ cudaError_t tc_padded_launch(const Problem& p, const WsLayout& inner, bool bwd, 
     } else if (p.hT) {
         w.hT = reinterpret_cast<float*>(pad + pl.hT);
     }
-    cudaError_t e = channelwise ? (bwd ? vec_launch_bwd(w, skip_recompute, st) : vec_launch_fwd(w, st))
-                                : (bwd ? tc_launch_bwd(w, skip_recompute, st) : tc_launch_fwd(w, st));
+    const cudaError_t e = bwd ? vec_launch_bwd(w, skip_recompute, st) : vec_launch_fwd(w, st);
     if (e != cudaSuccess) return e;
     auto narrow = [&](const void* src, void* dst) {
         if (!dst || rows == 0) return;
@@ -172,8 +170,8 @@ cudaError_t tc_padded_launch(const Problem& p, const WsLayout& inner, bool bwd, 
     if (bwd) {
         if (d.d_k == 64) { narrow(w.dq, p.dq); narrow(w.dk, p.dk); }
         if (d.d_v == 64) narrow(w.dv, p.dv);
-        if (channelwise && d.d_k == 64) { narrow_gate(w.dgv, p.dgv); narrow_gate(w.dbv, p.dbv); }
-        if (channelwise && d.d_v == 64) narrow_gate(w.dwv, p.dwv);
+        if (d.d_k == 64) { narrow_gate(w.dgv, p.dgv); narrow_gate(w.dbv, p.dbv); }
+        if (d.d_v == 64) narrow_gate(w.dwv, p.dwv);
         narrow_state(w.dh0, p.dh0);
     } else {
         if (d.d_v == 64) narrow(w.o, p.o);

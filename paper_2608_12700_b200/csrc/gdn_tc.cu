@@ -38,7 +38,7 @@ constexpr int kIntraThreads = kWideThreads + 32;   // ... plus one warp whose fi
                                                    // issues bulk copies and takes no part in the named barrier
 struct TcParams {
     Problem p;
-    CUtensorMap tm_q, tm_k, tm_v, tm_do;   // [T_total, H * 128] bf16, boxes of 64 rows x 64 columns
+    CUtensorMap tm_q, tm_k, tm_v, tm_do;   // [T_total, H, d] bf16, boxes of 64 tokens x 64 features of a head
     CUtensorMap tm_dq, tm_dk, tm_dv;       // same geometry, for the gradient stores of full chunks
     CUtensorMap tm_o;                      // same geometry, for the forward output (forward calls that want it)
     int with_bwd;                          // prep: also produce E
@@ -117,12 +117,12 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     bool ok = true;
     const uint32_t VO_BYTES = bwd ? 32768 : 16384;
     auto load_piece = [&](int piece, const ChunkInfo& c) {   // 0,1: Q  2,3: K  4,5: V  6,7: dO   (column halves)
-        const int cb = piece & 1, xq = c.hd * D + cb * 64;
+        const int cb = piece & 1;
         switch (piece >> 1) {
-            case 0: tma_load_2d(sm + QK + cb * 16384, &P.tm_q, xq, c.tok0, &bar_qk); break;
-            case 1: tma_load_2d(sm + QK + cb * 16384 + 8192, &P.tm_k, xq, c.tok0, &bar_qk); break;
-            case 2: tma_load_2d(sm + VO + cb * 16384, &P.tm_v, xq, c.tok0, &bar_vo); break;
-            case 3: if (bwd) tma_load_2d(sm + VO + cb * 16384 + 8192, &P.tm_do, xq, c.tok0, &bar_vo); break;
+            case 0: tma_load_3d(sm + QK + cb * 16384, &P.tm_q, cb * 64, c.hd, c.tok0, &bar_qk); break;
+            case 1: tma_load_3d(sm + QK + cb * 16384 + 8192, &P.tm_k, cb * 64, c.hd, c.tok0, &bar_qk); break;
+            case 2: tma_load_3d(sm + VO + cb * 16384, &P.tm_v, cb * 64, c.hd, c.tok0, &bar_vo); break;
+            case 3: if (bwd) tma_load_3d(sm + VO + cb * 16384 + 8192, &P.tm_do, cb * 64, c.hd, c.tok0, &bar_vo); break;
             default: break;
         }
     };
@@ -142,12 +142,12 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
                 if (!(lok = mbar_wait(&bar_ld0, ph))) break;
                 if (has_next) {
                     for (int cb = 0; cb < 2; ++cb) {
-                        prefetch_l2_tma_2d(&P.tm_v, nx.hd * D + cb * 64, nx.tok0);
-                        if (bwd) prefetch_l2_tma_2d(&P.tm_do, nx.hd * D + cb * 64, nx.tok0);
+                        prefetch_l2_tma_3d(&P.tm_v, cb * 64, nx.hd, nx.tok0);
+                        if (bwd) prefetch_l2_tma_3d(&P.tm_do, cb * 64, nx.hd, nx.tok0);
                     }
                     for (int cb = 0; cb < 2; ++cb) {
-                        prefetch_l2_tma_2d(&P.tm_q, nx.hd * D + cb * 64, nx.tok0);
-                        prefetch_l2_tma_2d(&P.tm_k, nx.hd * D + cb * 64, nx.tok0);
+                        prefetch_l2_tma_3d(&P.tm_q, cb * 64, nx.hd, nx.tok0);
+                        prefetch_l2_tma_3d(&P.tm_k, cb * 64, nx.hd, nx.tok0);
                     }
                 }
                 // T is staged
@@ -577,10 +577,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
     float st[NSH];
     {
         const float* init = reverse ? p.dhT : p.h0;
-        const size_t soff = ((size_t)n * p.d.H + hd) * D * D + (size_t)r * D + gc0;
+        const bool inside = r < p.d.d_k && gc0 < p.d.d_v;   // (a head dimension of 64: the rest of the state is zero)
+        const size_t soff = (((size_t)n * p.d.H + hd) * p.d.d_k + r) * p.d.d_v + gc0;
 #pragma unroll
         for (int k = 0; k < NSH / 4; ++k) {
-            float4 v = init ? *reinterpret_cast<const float4*>(init + soff + 4 * k) : make_float4(0.f, 0.f, 0.f, 0.f);
+            float4 v = init && inside ? *reinterpret_cast<const float4*>(init + soff + 4 * k) : make_float4(0.f, 0.f, 0.f, 0.f);
             st[4 * k] = v.x; st[4 * k + 1] = v.y; st[4 * k + 2] = v.z; st[4 * k + 3] = v.w;
         }
     }
@@ -638,9 +639,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
     }
     float* fin = reverse ? p.dh0 : p.hT;
     if (fin && ok) {
-        const size_t soff = ((size_t)n * p.d.H + hd) * D * D + (size_t)r * D + gc0;
+        const bool inside = r < p.d.d_k && gc0 < p.d.d_v;   // (a head dimension of 64: the rest of the state is zero)
+        const size_t soff = (((size_t)n * p.d.H + hd) * p.d.d_k + r) * p.d.d_v + gc0;
 #pragma unroll
-        for (int k = 0; k < NSH / 4; ++k) *reinterpret_cast<float4*>(fin + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
+        for (int k = 0; k < NSH / 4; ++k) if (inside) *reinterpret_cast<float4*>(fin + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
     }
     if (warp == 0) bulk_wait_read<0>();
     tc_fence_before();
@@ -740,8 +742,8 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
             // forward: Kb = Gam_e . k- (second product); reverse: k- itself, against the state scaled by Gam_e (below)
             bulk_load(slot + KT, p.ws + (reverse ? p.L.img_Km : p.L.img_K) + ch * 16384, 16384, &bar_full[stage]);
         } else {
-            tma_load_2d(slot + KT, &P.tm_k, hd * D, sg.chunk_tok0(c), &bar_full[stage]);
-            tma_load_2d(slot + KT + 8192, &P.tm_k, hd * D + 64, sg.chunk_tok0(c), &bar_full[stage]);
+            tma_load_3d(slot + KT, &P.tm_k, 0, hd, sg.chunk_tok0(c), &bar_full[stage]);
+            tma_load_3d(slot + KT + 8192, &P.tm_k, 64, hd, sg.chunk_tok0(c), &bar_full[stage]);
         }
         bulk_load(slot + XT, x_base + ch * x_chunk, x_bytes, &bar_full[stage]);
     };
@@ -761,10 +763,11 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     float st[NSH];
     {
         const float* init = reverse ? p.dhT : p.h0;
-        const size_t soff = ((size_t)n * H + hd) * D * D + (size_t)r * D + part * NS + lc0;
+        const bool inside = r < p.d.d_k && part * NS + lc0 < p.d.d_v;   // (a head dimension of 64: the rest of the state is zero)
+        const size_t soff = (((size_t)n * H + hd) * p.d.d_k + r) * p.d.d_v + part * NS + lc0;
 #pragma unroll
         for (int k = 0; k < NSH / 4; ++k) {
-            float4 v = init ? *reinterpret_cast<const float4*>(init + soff + 4 * k) : make_float4(0.f, 0.f, 0.f, 0.f);
+            float4 v = init && inside ? *reinterpret_cast<const float4*>(init + soff + 4 * k) : make_float4(0.f, 0.f, 0.f, 0.f);
             st[4 * k] = v.x; st[4 * k + 1] = v.y; st[4 * k + 2] = v.z; st[4 * k + 3] = v.w;
         }
     }
@@ -871,9 +874,10 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     }
     float* fin = reverse ? p.dh0 : p.hT;
     if (fin && ok) {
-        const size_t soff = ((size_t)n * H + hd) * D * D + (size_t)r * D + part * NS + lc0;
+        const bool inside = r < p.d.d_k && part * NS + lc0 < p.d.d_v;   // (a head dimension of 64: the rest of the state is zero)
+        const size_t soff = (((size_t)n * H + hd) * p.d.d_k + r) * p.d.d_v + part * NS + lc0;
 #pragma unroll
-        for (int k = 0; k < NSH / 4; ++k) *reinterpret_cast<float4*>(fin + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
+        for (int k = 0; k < NSH / 4; ++k) if (inside) *reinterpret_cast<float4*>(fin + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
     }
     if (warp == 0) bulk_wait_read<0>();
     tc_fence_before();
@@ -1040,18 +1044,18 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     //      T, Q             once the products of phase 4 are done; Q also read by the last readout
     constexpr uint32_t A_BYTES = 16384 + 32768 + 32768 + 16384 + 16384 + 8192, B_BYTES = 8192 + 16384 + 16384, U_BYTES = 16384;
     auto load_piece = [&](int piece, const ChunkInfo& c) {
-        const int cb = piece & 1, xq = c.hd * D + cb * 64;
+        const int cb = piece & 1;
         switch (piece) {
-            case 0: case 1: tma_load_2d(sm + KT + cb * 8192, &P.tm_k, xq, c.tok0, &bar_a); break;
-            case 2: case 3: tma_load_2d(sm + OX + cb * 16384, &P.tm_do, xq, c.tok0, &bar_a); break;
+            case 0: case 1: tma_load_3d(sm + KT + cb * 8192, &P.tm_k, cb * 64, c.hd, c.tok0, &bar_a); break;
+            case 2: case 3: tma_load_3d(sm + OX + cb * 16384, &P.tm_do, cb * 64, c.hd, c.tok0, &bar_a); break;
             case 4: bulk_load(sm + DH, p.ws + p.L.dhn + (size_t)c.ch * 32768, 32768, &bar_a); break;
             case 5: bulk_load(sm + HH, p.ws + p.L.hc + (size_t)c.ch * 32768, 32768, &bar_a); break;
             case 6: bulk_load(sm + W0, p.ws + p.L.W + (size_t)c.ch * 16384, 8192, &bar_a); break;
             case 7: bulk_load(sm + W1, p.ws + p.L.W + (size_t)c.ch * 16384 + 8192, 8192, &bar_a); break;
             case 8: bulk_load(sm + PT, p.ws + p.L.Pm + (size_t)c.ch * 8192, 8192, &bar_a); break;
             case 9: bulk_load(sm + UTT, p.ws + p.L.Ut + (size_t)c.ch * 16384, 16384, &bar_u); break;
-            case 10: case 11: tma_load_2d(sm + QT + cb * 8192, &P.tm_q, xq, c.tok0, &bar_b); break;
-            case 12: case 13: tma_load_2d(sm + VT + cb * 8192, &P.tm_v, xq, c.tok0, &bar_b); break;
+            case 10: case 11: tma_load_3d(sm + QT + cb * 8192, &P.tm_q, cb * 64, c.hd, c.tok0, &bar_b); break;
+            case 12: case 13: tma_load_3d(sm + VT + cb * 8192, &P.tm_v, cb * 64, c.hd, c.tok0, &bar_b); break;
             case 14: bulk_load(sm + TT, p.ws + p.L.Tm + (size_t)c.ch * 8192, 8192, &bar_b); break;
             default: break;
         }
@@ -1075,10 +1079,10 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
                 const bool early = has_next && item != (int)blockIdx.x;
                 if (!(lok = mbar_wait(&bar_ld0, ph))) break;   // the trip is under way: the late loads of the next one -> L2
                 if (early) {
-                    for (int cb = 0; cb < 2; ++cb) prefetch_l2_tma_2d(&P.tm_k, nx.hd * D + cb * 64, nx.tok0);
+                    for (int cb = 0; cb < 2; ++cb) prefetch_l2_tma_3d(&P.tm_k, cb * 64, nx.hd, nx.tok0);
                     prefetch_l2_bulk(p.ws + p.L.Pm + (size_t)nx.ch * 8192, 8192);
                     prefetch_l2_bulk(p.ws + p.L.Tm + (size_t)nx.ch * 8192, 8192);
-                    for (int cb = 0; cb < 2; ++cb) prefetch_l2_tma_2d(&P.tm_do, nx.hd * D + cb * 64, nx.tok0);
+                    for (int cb = 0; cb < 2; ++cb) prefetch_l2_tma_3d(&P.tm_do, cb * 64, nx.hd, nx.tok0);
                 }
                 if (!(lok = mbar_wait(&bar_e0, ph))) break;    // U~^T has been read by the first readout
                 if (early) { mbar_expect_tx(&bar_u, U_BYTES); pend_u = true; load_piece(9, nx); }
@@ -1086,7 +1090,7 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
                 if (early) { mbar_expect_tx(&bar_a, A_BYTES); pend_a = true; load_piece(4, nx); }   // (the first piece announces the group)
                 if (!(lok = mbar_wait(&bar_st1, ph))) break;   // dv is staged
                 if (full) {
-                    for (int cb = 0; cb < 2; ++cb) tma_store_2d(&P.tm_dv, x.hd * D + cb * 64, x.tok0, sm + STG_V + cb * 8192);
+                    for (int cb = 0; cb * 64 < p.d.d_v; ++cb) tma_store_3d(&P.tm_dv, cb * 64, x.hd, x.tok0, sm + STG_V + cb * 8192);
                     bulk_commit();
                 }
                 if (!(lok = mbar_wait(&bar_e2, ph))) break;    // dO, h and dXv (over W^T)
@@ -1117,9 +1121,9 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
                 }
                 if (!(lok = mbar_wait(&bar_st2, ph))) break;   // dq, dk are staged
                 if (full) {
-                    for (int cb = 0; cb < 2; ++cb) {
-                        tma_store_2d(&P.tm_dq, x.hd * D + cb * 64, x.tok0, sm + STG_Q + cb * 8192);
-                        tma_store_2d(&P.tm_dk, x.hd * D + cb * 64, x.tok0, sm + STG_K + cb * 8192);
+                    for (int cb = 0; cb * 64 < p.d.d_k; ++cb) {
+                        tma_store_3d(&P.tm_dq, cb * 64, x.hd, x.tok0, sm + STG_Q + cb * 8192);
+                        tma_store_3d(&P.tm_dk, cb * 64, x.hd, x.tok0, sm + STG_K + cb * 8192);
                     }
                     bulk_commit();
                 }
@@ -1315,8 +1319,6 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     }
     if (gates && has_next) fetch_gates(xn);
     GDN_WAIT_MMA(23)
-    // (addresses of the ragged-tail flushes are formed where they are used: nothing of them lives across the phases)
-    auto grad_rows = [&](void* base) { return reinterpret_cast<__nv_bfloat16*>(base) + ((size_t)x.tok0 * H + x.hd) * D; };
     if (ok && worker) {
         float v2[2][8];
         tmem_ld8(tmem + lane_base + C_DP + i0, v2[0]);
@@ -1361,7 +1363,7 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     fence_async_smem();
     cta_sync();
     if (threadIdx.x == 32) mbar_arrive(&bar_st1);   // dv is staged: the loader stores it (async proxy)
-    if (ok && !full) flush_rows(sm + STG_V, grad_rows(p.dv), (size_t)H * D, x.len, kWideThreads);   // rows beyond the sequence must not be written
+    if (ok && !full) flush_rows(sm + STG_V, p.dv, x, H, p.d.d_v, kWideThreads);   // rows beyond the sequence must not be written
 
     // ---- phase 3: dA = -stril(dXv U^T) ; under its readout [dO; dXv] h^T and dPD^T Q (rows on lanes 64..127)
     if (ok && issuer) {
@@ -1486,8 +1488,8 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     cta_sync();   // every reader of this trip's tiles and scratch is done
     if (threadIdx.x == 32) mbar_arrive(&bar_st2);   // dq, dk are staged: the loader stores them
     if (ok && !full) {
-        flush_rows(sm + STG_Q, grad_rows(p.dq), (size_t)H * D, x.len, kWideThreads);
-        flush_rows(sm + STG_K, grad_rows(p.dk), (size_t)H * D, x.len, kWideThreads);
+        flush_rows(sm + STG_Q, p.dq, x, H, p.d.d_k, kWideThreads);
+        flush_rows(sm + STG_K, p.dk, x, H, p.d.d_k, kWideThreads);
     }
     if (!ok) break;
     }
@@ -1552,8 +1554,8 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
             if (CW) {
                 bulk_load(sm + QK + cb * 16384, p.ws + p.L.img_QKp + (size_t)c.ch * 32768 + cb * 16384, 8192, &bar_in);
             } else {
-                tma_load_2d(sm + QK + cb * 16384, &P.tm_q, c.hd * D + cb * 64, c.tok0, &bar_in);
-                tma_load_2d(sm + QK + cb * 16384 + 8192, &P.tm_k, c.hd * D + cb * 64, c.tok0, &bar_in);
+                tma_load_3d(sm + QK + cb * 16384, &P.tm_q, cb * 64, c.hd, c.tok0, &bar_in);
+                tma_load_3d(sm + QK + cb * 16384 + 8192, &P.tm_k, cb * 64, c.hd, c.tok0, &bar_in);
             }
         }
         pending = true;
@@ -1664,11 +1666,11 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
         if (ok) {
             if (x.len == kC) {
                 if (threadIdx.x == 0) {
-                    for (int cb = 0; cb < 2; ++cb) tma_store_2d(&P.tm_o, x.hd * D + cb * 64, x.tok0, sm + STG + cb * 8192);
+                    for (int cb = 0; cb * 64 < p.d.d_v; ++cb) tma_store_3d(&P.tm_o, cb * 64, x.hd, x.tok0, sm + STG + cb * 8192);
                     bulk_commit();
                 }
             } else {
-                flush_rows(sm + STG, reinterpret_cast<__nv_bfloat16*>(p.o) + ((size_t)x.tok0 * H + x.hd) * D, (size_t)H * D, x.len);
+                flush_rows(sm + STG, p.o, x, H, p.d.d_v, kThreads);
                 __syncthreads();
             }
             if (threadIdx.x == 0) {
@@ -1696,7 +1698,7 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
 // host side
 // ------------------------------------------------------------------------------------------------
 bool tc_supported(const gdn_desc& d) {
-    return d.dtype == GDN_BF16 && d.d_k == 128 && d.d_v == 128 && d.chunk == kC;
+    return d.dtype == GDN_BF16 && (d.d_k == 64 || d.d_k == 128) && (d.d_v == 64 || d.d_v == 128) && d.chunk == kC;
 }
 
 thread_local int g_inject_timeout = 0;   // set by gdn_debug_inject_timeout, consumed by the next gdn_bwd of this family
@@ -1716,17 +1718,11 @@ static bool fill_params(TcParams& P, const Problem& p, bool with_bwd, int scan_d
     P.scan_dirs = scan_dirs;
     P.lowrank = tc_carries_lowrank(p.d) ? 1 : 0;
     P.withhold = 0;
-    const uint64_t rows = (uint64_t)p.Ttot, cols = (uint64_t)p.d.H * D, pitch = cols * 2;
-    if (!tc::make_tmap_bf16_2d(&P.tm_q, p.q, rows, cols, pitch, 64)) return false;
-    if (!tc::make_tmap_bf16_2d(&P.tm_k, p.k, rows, cols, pitch, 64)) return false;
-    if (!tc::make_tmap_bf16_2d(&P.tm_v, p.v, rows, cols, pitch, 64)) return false;
-    if (!tc::make_tmap_bf16_2d(&P.tm_do, with_bwd ? p.dO : p.v, rows, cols, pitch, 64)) return false;
-    if (!with_bwd && p.o && !tc::make_tmap_bf16_2d(&P.tm_o, p.o, rows, cols, pitch, 64)) return false;
-    if (with_bwd) {
-        if (!tc::make_tmap_bf16_2d(&P.tm_dq, p.dq, rows, cols, pitch, 64)) return false;
-        if (!tc::make_tmap_bf16_2d(&P.tm_dk, p.dk, rows, cols, pitch, 64)) return false;
-        if (!tc::make_tmap_bf16_2d(&P.tm_dv, p.dv, rows, cols, pitch, 64)) return false;
-    }
+    auto map = [&](CUtensorMap* m, const void* base, int d) { return tc::make_tmap_bf16_heads(m, base, p.Ttot, p.d.H, d); };
+    if (!map(&P.tm_q, p.q, p.d.d_k) || !map(&P.tm_k, p.k, p.d.d_k) || !map(&P.tm_v, p.v, p.d.d_v)) return false;
+    if (!map(&P.tm_do, with_bwd ? p.dO : p.v, p.d.d_v)) return false;
+    if (!with_bwd && p.o && !map(&P.tm_o, p.o, p.d.d_v)) return false;
+    if (with_bwd && (!map(&P.tm_dq, p.dq, p.d.d_k) || !map(&P.tm_dk, p.dk, p.d.d_k) || !map(&P.tm_dv, p.dv, p.d.d_v))) return false;
     return true;
 }
 
@@ -1812,8 +1808,7 @@ cudaError_t tc_launch_out_channelwise(const Problem& p, cudaStream_t st) {
     static SmemLimitOnce done;
     TcParams P{};
     P.p = p;
-    const uint64_t rows = (uint64_t)p.Ttot, cols = (uint64_t)p.d.H * D;
-    if (!tc::make_tmap_bf16_2d(&P.tm_o, p.o, rows, cols, cols * 2, 64)) return cudaErrorUnknown;
+    if (!tc::make_tmap_bf16_heads(&P.tm_o, p.o, p.Ttot, p.d.H, p.d.d_v)) return cudaErrorUnknown;
     const int items = p.L.max_chunks * p.d.H, ctas = 2 * sm_count();
     return launch_chunk_kernel(tc_out_kernel<true>, done, outk::SMEM_BYTES, ST_OUT, items < ctas ? items : ctas, kThreads, P, st);
 }
@@ -1835,7 +1830,7 @@ cudaError_t tc_launch_scan_channelwise(const Problem& p, int dirs, cudaStream_t 
 
 // A call with no tokens still owes the pass-through of the states.
 static cudaError_t empty_call(const Problem& p, bool bwd, cudaStream_t st) {
-    const size_t bytes = (size_t)p.d.N * p.d.H * D * D * sizeof(float);
+    const size_t bytes = (size_t)p.d.N * p.d.H * p.d.d_k * p.d.d_v * sizeof(float);
     float* dst = bwd ? p.dh0 : p.hT;
     const float* src = bwd ? p.dhT : p.h0;
     if (!dst) return cudaSuccess;

@@ -92,15 +92,14 @@ __device__ __forceinline__ float reduce8(float (&v)[8], int lane) {
     return r;
 }
 
-// Copy a staged [64 tokens][128 features] bf16 tile to a [T, H, 128] tensor with 16-byte stores (rows < len only).
-__device__ __forceinline__ void flush_rows(const unsigned char* tile, __nv_bfloat16* gbase, size_t row_pitch, int len, int nthr) {
+// Copy the first `d` features of a staged [64 tokens][128 features] bf16 tile to a [T, H, d] tensor with 16-byte stores (rows
+// < len only).
+__device__ __forceinline__ void flush_rows(const unsigned char* tile, void* base, const ChunkInfo& x, int H, int d, int nthr) {
+    __nv_bfloat16* g = reinterpret_cast<__nv_bfloat16*>(base) + ((size_t)x.tok0 * H + x.hd) * d;
     for (int t = threadIdx.x; t < kC * 16; t += nthr) {
         const int i = t >> 4, chk = t & 15;
-        if (i < len) *reinterpret_cast<uint4*>(gbase + (size_t)i * row_pitch + chk * 8) = *reinterpret_cast<const uint4*>(tile + tile_chunk_off(64, i, chk));
+        if (i < x.len && chk * 8 < d) *reinterpret_cast<uint4*>(g + (size_t)i * H * d + chk * 8) = *reinterpret_cast<const uint4*>(tile + tile_chunk_off(64, i, chk));
     }
-}
-__device__ __forceinline__ void flush_rows(const unsigned char* tile, __nv_bfloat16* gbase, size_t row_pitch, int len) {
-    flush_rows(tile, gbase, row_pitch, len, (int)blockDim.x);
 }
 
 // dg_j = sum_{i >= j} dgam_i inside a chunk (gam_i = sum_{j <= i} g_j), by one warp: lane l owns tokens l and l + 32.

@@ -69,8 +69,8 @@ __global__ void __launch_bounds__(split::kT, 2) tc_factors_kernel(const __grid_c
     auto issue_loads = [&](const ChunkInfo& c) {   // thread 0
         mbar_expect_tx(&bar_in, 32768);
         for (int cb = 0; cb < 2; ++cb) {
-            tma_load_2d(sm + KV + cb * 16384, &P.tm_k, c.hd * D + cb * 64, c.tok0, &bar_in);
-            tma_load_2d(sm + KV + cb * 16384 + 8192, &P.tm_v, c.hd * D + cb * 64, c.tok0, &bar_in);
+            tma_load_3d(sm + KV + cb * 16384, &P.tm_k, cb * 64, c.hd, c.tok0, &bar_in);
+            tma_load_3d(sm + KV + cb * 16384 + 8192, &P.tm_v, cb * 64, c.hd, c.tok0, &bar_in);
         }
         pending = true;
     };
@@ -275,9 +275,9 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
     auto issue_loads = [&](const ChunkInfo& c) {   // thread 0
         mbar_expect_tx(&bar_in, 65536);
         for (int cb = 0; cb < 2; ++cb) {
-            tma_load_2d(sm + QK + cb * 16384, &P.tm_q, c.hd * D + cb * 64, c.tok0, &bar_in);
-            tma_load_2d(sm + QK + cb * 16384 + 8192, &P.tm_k, c.hd * D + cb * 64, c.tok0, &bar_in);
-            tma_load_2d(sm + DOT + cb * 8192, &P.tm_do, c.hd * D + cb * 64, c.tok0, &bar_in);
+            tma_load_3d(sm + QK + cb * 16384, &P.tm_q, cb * 64, c.hd, c.tok0, &bar_in);
+            tma_load_3d(sm + QK + cb * 16384 + 8192, &P.tm_k, cb * 64, c.hd, c.tok0, &bar_in);
+            tma_load_3d(sm + DOT + cb * 8192, &P.tm_do, cb * 64, c.hd, c.tok0, &bar_in);
         }
         bulk_load(sm + WT, p.ws + p.L.W + (size_t)c.ch * 16384, 16384, &bar_in);
         pending = true;
@@ -468,11 +468,10 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
     auto issue_loads = [&](const ChunkInfo& c, bool withhold) {   // thread 0
         mbar_expect_tx(&bar_in, 65536);
         for (int cb = 0; cb < 2; ++cb) {
-            const int xq = c.hd * D + cb * 64;
-            if (!(withhold && cb == 0)) tma_load_2d(sm + QK + cb * 16384, &P.tm_q, xq, c.tok0, &bar_in);
-            tma_load_2d(sm + QK + cb * 16384 + 8192, &P.tm_k, xq, c.tok0, &bar_in);
-            tma_load_2d(sm + VO + cb * 16384, &P.tm_v, xq, c.tok0, &bar_in);
-            tma_load_2d(sm + VO + cb * 16384 + 8192, &P.tm_do, xq, c.tok0, &bar_in);
+            if (!(withhold && cb == 0)) tma_load_3d(sm + QK + cb * 16384, &P.tm_q, cb * 64, c.hd, c.tok0, &bar_in);
+            tma_load_3d(sm + QK + cb * 16384 + 8192, &P.tm_k, cb * 64, c.hd, c.tok0, &bar_in);
+            tma_load_3d(sm + VO + cb * 16384, &P.tm_v, cb * 64, c.hd, c.tok0, &bar_in);
+            tma_load_3d(sm + VO + cb * 16384 + 8192, &P.tm_do, cb * 64, c.hd, c.tok0, &bar_in);
         }
         pending = true;
     };
