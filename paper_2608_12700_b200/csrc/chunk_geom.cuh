@@ -31,6 +31,14 @@ __device__ __forceinline__ void chunk_entry(const Problem& p, ChunkInfo& x, int 
         x.len = min(kC, p.d.T - pos * kC);
     }
 }
+// ... and from the table, for calls that build it whatever the sequences (the channel-wise ones).
+__device__ __forceinline__ void chunk_entry_tab(const Problem& p, ChunkInfo& x, int item) {
+    x.c = item / p.d.H;
+    x.hd = item % p.d.H;
+    x.ch = item;
+    x.tok0 = reinterpret_cast<const int32_t*>(p.ws + p.L.chunk_tok0)[x.c];
+    x.len = reinterpret_cast<const int32_t*>(p.ws + p.L.chunk_len)[x.c];
+}
 // The same geometry for kernels that walk along whole sequences.
 struct ChunkGeom {
     const int32_t *first, *tok0, *len;   // tables (packed sequences), else null

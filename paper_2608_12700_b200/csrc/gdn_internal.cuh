@@ -18,8 +18,9 @@ struct WsHeader {
     int32_t status;    // device-side gdn_status (0 = ok)
     int32_t n_chunks;  // chunks actually present (<= max_chunks)
     int32_t detail;    // where a bounded wait gave up / offending sequence index
-    int32_t cw_fallback;   // channel-wise calls: 1 if the last call on this workspace was computed by the fall-back kernels
-                           // (then the workspace holds their fp32 data, not tile images); kept across calls
+    int32_t cw_fallback;   // channel-wise calls on the tensor-core route: 1 if the gates of the call leave its range (set by its first
+                           // stage, cleared by the table kernel).  The tensor-core kernels then stand down and the FFMA kernels enqueued
+                           // behind them compute the call, and the backward on the workspace of such a forward.
     int32_t pad[60];
 };
 static_assert(sizeof(WsHeader) == 256, "header size");
@@ -43,9 +44,9 @@ struct WsLayout {
     size_t E;              // [CH, d_k, d_v]           scale (Gam Q - P W)^T dO
     size_t dhn;            // [CH, d_k, d_v]           gradient w.r.t. the state leaving the chunk
     size_t Pm;             // [CH, 64, 64]             P = tril(Q K^T . D) (tcgen05 d = 128 family: made once, by tc_prep)
-    size_t img_W, img_U, img_K, img_E;   // channel-wise path on the tensor cores (bf16, d = 128): bf16 tile images of W^T,
-                                         // U~^T, the scaled keys Kb (16 KB per chunk-head each) and E (32 KB); else unused
-    size_t img_QKp, img_Km, img_Vt, img_dO;   // ... of [Q~; K+] (32 KB), K-, V~ and scale dO (16 KB each)
+    size_t img_W, img_U, img_E;    // channel-wise path on the tensor cores (bf16, d = 128): bf16 tile images of W^T, U~^T (16 KB
+                                   // per chunk-head each) and E (32 KB); else unused
+    size_t img_QKp, img_Km, img_Vt;   // ... of [Q~; K+] (32 KB), K- and V~ (16 KB each)
     int tc_scans;                        // ... and T, P, hc, dhn are bf16 tile images as well (8, 8, 32, 32 KB)
     size_t Kb, U, dU;      // FFMA families (fp32): keys scaled to the chunk end [CH, 64, d_k]; U = U~ - W h and dU [CH, 64, d_v]
     size_t scratch;        // kernel-private staging, per chunk-head
@@ -136,7 +137,6 @@ inline WsLayout make_layout_vec(const gdn_desc& d) {
     L.Nm = L.Bf = o;
     L.img_W = take(L.tc_scans ? CH * 16384 : 0);
     L.img_U = take(L.tc_scans ? CH * 16384 : 0);
-    L.img_K = take(L.tc_scans ? CH * 16384 : 0);
     L.img_QKp = take(L.tc_scans ? CH * 32768 : 0);
     L.img_Km = take(L.tc_scans ? CH * 16384 : 0);
     L.img_Vt = take(L.tc_scans ? CH * 16384 : 0);
@@ -146,7 +146,6 @@ inline WsLayout make_layout_vec(const gdn_desc& d) {
     L.fwd_end = o;
     L.E = take(4 * CH * d.d_k * d.d_v);
     L.img_E = take(L.tc_scans ? CH * 32768 : 0);
-    L.img_dO = take(L.tc_scans ? CH * 16384 : 0);
     L.dhn = take(4 * CH * d.d_k * d.d_v);
     L.dU = take(4 * CH * kC * d.d_v);
     L.scratch = L.total = o;
@@ -251,6 +250,7 @@ bool tc_supported(const gdn_desc& d);
 bool tc_carries_lowrank(const gdn_desc& d);
 cudaError_t tc_launch_scan_channelwise(const Problem& p, int dirs, cudaStream_t st);   // carries of the channel-wise path
 cudaError_t tc_launch_out_channelwise(const Problem& p, cudaStream_t st);              // its forward output (p.o non-null)
+int tc_sm_count();                                                                     // SMs of the current device
 cudaError_t tc_launch_fwd(const Problem& p, cudaStream_t st);
 cudaError_t tc_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st);
 

@@ -47,6 +47,7 @@ __global__ void table_kernel(Problem p) {
             acc += (int)((e - a + kC - 1) / kC);
         }
         if (good && cu(N) != p.Ttot) { good = 0; bad_at = N; }
+        hdr->cw_fallback = 0;
         if (good) {
             seq_first[N] = acc;
             hdr->status = GDN_OK;

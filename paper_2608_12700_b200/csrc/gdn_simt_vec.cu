@@ -31,18 +31,11 @@ using namespace ffma;
 
 constexpr int kB = 16, kNB = kC / kB;   // tokens of a block, blocks of a chunk
 
-// Whether this launch has work: normally when no earlier stage has reported an error; a launch of the fall-back sequence
-// only when the tensor-core route has refused the gates of this call (decided on the device, no host round trip).
+// Whether this launch has work: no earlier stage has reported an error, and, for a launch of the fall-back sequence, the
+// tensor-core route has refused the gates of this call (decided on the device, no host round trip).
 __device__ __forceinline__ bool vec_go(const Problem& p) {
-    const int st = reinterpret_cast<const WsHeader*>(p.ws)->status;
-    return p.fallback ? st == GDN_ERR_DECAY_RANGE : st == GDN_OK;
-}
-__global__ void vec_clear_refusal_kernel(Problem p) {
-    wait_prerequisites();
-    WsHeader* hdr = reinterpret_cast<WsHeader*>(p.ws);
-    const bool refused = hdr->status == GDN_ERR_DECAY_RANGE;
-    hdr->cw_fallback = refused ? 1 : 0;   // a backward on this workspace "fresh from the forward" must know whose data it holds
-    if (refused) { hdr->status = GDN_OK; hdr->detail = 0; }
+    const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
+    return hdr->status == GDN_OK && (!p.fallback || hdr->cw_fallback);
 }
 
 // References of the four blocks and their exponentials: ref_0 = 0 (the chunk start), ref_I = gam of token 16 I - 1.
@@ -659,18 +652,15 @@ cudaError_t ffma_bwd(const Problem& q, bool skip_recompute, cudaStream_t st) {
 }
 
 // bf16 I/O at d = 128 runs on the tensor cores (gdn_tc_cw.cu).  That route refuses gates whose chunk-cumulative log decay
-// leaves its range, through the status word; the FFMA sequence is therefore enqueued behind it in fall-back mode: its
-// launches return at once unless the status word says so, in which case they compute the call (with the decay inside the
-// contractions there is no range limit) and clear the refusal.  No host round trip, the same launches every call.
+// leaves its range, through the workspace header; the FFMA sequence is therefore enqueued behind it in fall-back mode: its
+// launches return at once unless the header says so, in which case they compute the call (with the decay inside the
+// contractions there is no range limit).  No host round trip, the same launches every call.
 template <typename IO, int DK, int DV>
 cudaError_t ffma_fallback(const Problem& p, bool bwd, bool skip_recompute, cudaStream_t st) {
     Problem q = p;
     q.fallback = 1;
     q.L.tc_scans = 0;
-    cudaError_t e = bwd ? ffma_bwd<IO, DK, DV>(q, skip_recompute, st) : ffma_fwd<IO, DK, DV>(q, st);
-    if (e != cudaSuccess) return e;
-    { StageScope t(ST_FALLBACK, st); launch_kernel(vec_clear_refusal_kernel, 1, 1, 0, st, q); }
-    return cudaGetLastError();
+    return bwd ? ffma_bwd<IO, DK, DV>(q, skip_recompute, st) : ffma_fwd<IO, DK, DV>(q, st);
 }
 
 template <typename IO, int DK, int DV>

@@ -685,7 +685,7 @@ template <int S> struct Cfg {
 
 // One direction of one chain (the direction is a compile-time constant: the two differ in operands and readouts).
 // CW = carries of the channel-wise path (per-channel gates): the decay of the state is a vector (one factor per state
-// row, i.e. per thread), and the key tile arrives already scaled, Kb_j = exp(gam_e - gam_j) . k_j, as a tile image from the
+// row, i.e. per thread), and the key tile arrives as K- = k / Gam, a tile image from the
 // workspace together with images of W^T, U~^T and E (written by the channel-wise preparation kernels), so the readout of the
 // first product applies no per-token factor.
 template <bool reverse, bool CW, int S>
@@ -739,8 +739,8 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         mbar_expect_tx(&bar_full[stage], 32768 + x_bytes);
         bulk_load(slot + WT, w_base + ch * 16384, 16384, &bar_full[stage]);
         if constexpr (CW) {
-            // forward: Kb = Gam_e . k- (second product); reverse: k- itself, against the state scaled by Gam_e (below)
-            bulk_load(slot + KT, p.ws + (reverse ? p.L.img_Km : p.L.img_K) + ch * 16384, 16384, &bar_full[stage]);
+            // k- itself, in both directions: the decay to the chunk end is applied to the state (row by row, below)
+            bulk_load(slot + KT, p.ws + p.L.img_Km + ch * 16384, 16384, &bar_full[stage]);
         } else {
             tma_load_3d(slot + KT, &P.tm_k, 0, hd, sg.chunk_tok0(c), &bar_full[stage]);
             tma_load_3d(slot + KT + 8192, &P.tm_k, 64, hd, sg.chunk_tok0(c), &bar_full[stage]);
@@ -868,7 +868,10 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
             if (reverse) chunk_load(ring + XT, 128, r, (lc0 >> 3) + k, ad);
             tmem_wait_ld();
 #pragma unroll
-            for (int j = 0; j < 8; ++j) st[8 * k + j] = fmaf(Ge, st[8 * k + j], reverse ? ad[j] + d2[j] : d2[j]);
+            for (int j = 0; j < 8; ++j) {
+                if (CW && !reverse) st[8 * k + j] = Ge * (st[8 * k + j] + d2[j]);   // Gam_e h + (Gam_e . K-)^T U
+                else st[8 * k + j] = fmaf(Ge, st[8 * k + j], reverse ? ad[j] + d2[j] : d2[j]);
+            }
         }
         tc_fence_before();
     }
@@ -913,7 +916,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_cw_kernel(const __grid_co
     __shared__ uint64_t bar_full[Cfg<S>::STAGES], bar_mma;
     __shared__ uint32_t tmem_slot;
     const int bid = (int)blockIdx.x;
-    if (reinterpret_cast<const WsHeader*>(P.p.ws)->status != GDN_OK) return;
+    const WsHeader* hdr = reinterpret_cast<const WsHeader*>(P.p.ws);
+    if (hdr->status != GDN_OK || hdr->cw_fallback) return;
     const int rev = (S == 1 && P.scan_dirs == 2) ? (bid & 1) : P.scan_dirs;
     const int chain = (S == 2 || P.scan_dirs == 2) ? (bid >> 1) : bid;
     const int part = S == 2 ? (bid & 1) : 0;
@@ -1527,7 +1531,8 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
     using namespace outk;
     const Problem& p = P.p;
     const int H = p.d.H;
-    if (reinterpret_cast<const WsHeader*>(p.ws)->status != GDN_OK) return;
+    const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
+    if (hdr->status != GDN_OK || (CW && hdr->cw_fallback)) return;
     const int n_items = n_chunks_of(p) * H;
     if ((int)blockIdx.x >= n_items) return;
     extern __shared__ unsigned char smem_raw[];
@@ -1802,6 +1807,8 @@ static cudaError_t launch_out(const TcParams& P, cudaStream_t st) {
     const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count();
     return launch_chunk_kernel(tc_out_kernel<false>, done, outk::SMEM_BYTES, ST_OUT, items < ctas ? items : ctas, kThreads, P, st);
 }
+
+int tc_sm_count() { return sm_count(); }
 
 // Forward output of the channel-wise path from the tile images its preparation kernels and carries left in the workspace.
 cudaError_t tc_launch_out_channelwise(const Problem& p, cudaStream_t st) {

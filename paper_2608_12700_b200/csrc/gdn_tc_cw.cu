@@ -6,7 +6,7 @@
 // factor exp(gam_i - gam_j) of a token pair splits into a row part and a column part, and the keys and queries are
 // scaled once, element by element, before any product:
 //     q~_i = Gam_i . q_i      k+_i = Gam_i . b_i . k_i   (row role)      k-_j = k_j / Gam_j   (column role)
-//     v~_i = w_i . v_i        Kb_j = Gam_e . k-_j        (carries)        dO'  = scale dO
+//     v~_i = w_i . v_i                                                    dO'  = scale dO (the factor is applied to fp32 accumulators)
 // In these variables the chunk is a decay-free delta rule whose token-token matrices carry plain triangular masks:
 //     A = stril(K+ K-^T)   P = tril(Q~ K-^T)   T = (I + A)^-1   W = T K+   U~ = T V~   E = (Q~ - P W)^T dO'
 //     U = U~ - W h   dU = P^T dO' + K- dh''   (dh'' = Diag(Gam_e) dh')
@@ -51,11 +51,7 @@ __device__ __forceinline__ bool chunk_ctx(const Problem& p, ChunkCtx& x) {
 // ------------------------------------------------------------------------------------------------
 // cw_scale
 // ------------------------------------------------------------------------------------------------
-// mode 0: the forward's images; 1: those and dO' (closed backward); 2: dO' alone, for a backward on a workspace fresh
-// from the forward (every other image, gam and the factors are still there).  If that forward was computed by the
-// fall-back kernels (its gates were refused; the header remembers), the workspace holds their fp32 data instead: the
-// refusal is raised again and the fall-back sequence computes this call too.
-__global__ void __launch_bounds__(kT) cw_scale_kernel(Problem p, int mode) {
+__global__ void __launch_bounds__(kT) cw_scale_kernel(Problem p) {
     wait_prerequisites();
     ChunkCtx x;
     if (!chunk_ctx(p, x)) return;
@@ -63,28 +59,6 @@ __global__ void __launch_bounds__(kT) cw_scale_kernel(Problem p, int mode) {
     __shared__ int bad;
     const int H = p.d.H;
     const size_t base = ((size_t)x.tok0 * H + x.hd) * D, rs = (size_t)H * D;
-    const bool with_bwd = mode != 0;
-    const __nv_bfloat16* op = with_bwd ? reinterpret_cast<const __nv_bfloat16*>(p.dO) + base : nullptr;
-    if (mode == 2) {
-        WsHeader* hdr = reinterpret_cast<WsHeader*>(p.ws);
-        if (hdr->cw_fallback) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) { hdr->status = GDN_ERR_DECAY_RANGE; hdr->detail = -1; }
-            return;
-        }
-        char* iDO = p.ws + p.L.img_dO + (size_t)x.ch * 16384;
-        const float sc = p.d.scale;
-        for (int t = threadIdx.x; t < kC * 16; t += kT) {
-            const int i = t >> 4, ch = t & 15;
-            float o8[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) o8[j] = 0.f;
-            if (i < x.len) unpack8(*reinterpret_cast<const uint4*>(op + i * rs + ch * 8), o8);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) o8[j] *= sc;
-            *reinterpret_cast<uint4*>(iDO + tile_chunk_off(64, i, ch)) = pack8(o8);
-        }
-        return;
-    }
     const __nv_bfloat16* qp = reinterpret_cast<const __nv_bfloat16*>(p.q) + base;
     const __nv_bfloat16* kp = reinterpret_cast<const __nv_bfloat16*>(p.k) + base;
     const __nv_bfloat16* vp = reinterpret_cast<const __nv_bfloat16*>(p.v) + base;
@@ -111,8 +85,7 @@ __global__ void __launch_bounds__(kT) cw_scale_kernel(Problem p, int mode) {
     if (bad) {
         if (threadIdx.x == 0) {
             WsHeader* hdr = reinterpret_cast<WsHeader*>(p.ws);
-            hdr->status = GDN_ERR_DECAY_RANGE;
-            hdr->detail = x.ch;
+            hdr->cw_fallback = 1;
         }
         return;
     }
@@ -120,21 +93,17 @@ __global__ void __launch_bounds__(kT) cw_scale_kernel(Problem p, int mode) {
     for (int t = threadIdx.x; t < kC * D; t += kT) wsG[t] = gam[(t / D) * (D + 1) + t % D];
     char* iQKp = p.ws + p.L.img_QKp + (size_t)x.ch * 32768;
     char* iKm = p.ws + p.L.img_Km + (size_t)x.ch * 16384;
-    char* iKb = p.ws + p.L.img_K + (size_t)x.ch * 16384;
     char* iVt = p.ws + p.L.img_Vt + (size_t)x.ch * 16384;
-    char* iDO = p.ws + p.L.img_dO + (size_t)x.ch * 16384;
-    const float sc = p.d.scale;
     for (int t = threadIdx.x; t < kC * 16; t += kT) {   // one 16-byte piece (8 features) of one token row
         const int i = t >> 4, ch = t & 15;
-        float q8[8], k8[8], v8[8], o8[8], a[8], b[8], c[8], d8[8], b8[8], w8[8];
+        float q8[8], k8[8], v8[8], a[8], b[8], c[8], b8[8], w8[8];
         const bool live = i < x.len;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) { q8[j] = k8[j] = v8[j] = o8[j] = b8[j] = w8[j] = 0.f; }
+        for (int j = 0; j < 8; ++j) { q8[j] = k8[j] = v8[j] = b8[j] = w8[j] = 0.f; }
         if (live) {
             unpack8(*reinterpret_cast<const uint4*>(qp + i * rs + ch * 8), q8);
             unpack8(*reinterpret_cast<const uint4*>(kp + i * rs + ch * 8), k8);
             unpack8(*reinterpret_cast<const uint4*>(vp + i * rs + ch * 8), v8);
-            if (with_bwd) unpack8(*reinterpret_cast<const uint4*>(op + i * rs + ch * 8), o8);
             const float4* bp = reinterpret_cast<const float4*>(p.bv + base + i * rs + ch * 8);
             const float4* wp = reinterpret_cast<const float4*>(p.wv + base + i * rs + ch * 8);
             const float4 b0 = bp[0], b1 = bp[1], w0 = wp[0], w1 = wp[1];
@@ -144,149 +113,129 @@ __global__ void __launch_bounds__(kT) cw_scale_kernel(Problem p, int mode) {
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const int r = ch * 8 + j;
-            const float g = gam[i * (D + 1) + r], ge = gam[(kC - 1) * (D + 1) + r];
+            const float g = gam[i * (D + 1) + r];
             const float G = expf(g);
             const float bb = b8[j], ww = w8[j];
             a[j] = G * q8[j];                 // q~
             b[j] = G * bb * k8[j];            // k+
             c[j] = expf(-g) * k8[j];          // k-
-            d8[j] = expf(ge - g) * k8[j];     // Kb
             v8[j] *= ww;                      // v~
-            o8[j] *= sc;                      // dO'
         }
         *reinterpret_cast<uint4*>(iQKp + tile_chunk_off(128, i, ch)) = pack8(a);
         *reinterpret_cast<uint4*>(iQKp + tile_chunk_off(128, 64 + i, ch)) = pack8(b);
         *reinterpret_cast<uint4*>(iKm + tile_chunk_off(64, i, ch)) = pack8(c);
-        *reinterpret_cast<uint4*>(iKb + tile_chunk_off(64, i, ch)) = pack8(d8);
         *reinterpret_cast<uint4*>(iVt + tile_chunk_off(64, i, ch)) = pack8(v8);
-        if (with_bwd) *reinterpret_cast<uint4*>(iDO + tile_chunk_off(64, i, ch)) = pack8(o8);
     }
 }
 
+// Whether the tensor-core kernels of the call have work: no error so far, and no gates beyond their range (then the FFMA
+// sequence enqueued behind them computes the call).
+__device__ __forceinline__ bool cw_go(const WsHeader* hdr) { return hdr->status == GDN_OK && !hdr->cw_fallback; }
+
+struct CwParams {
+    Problem p;
+    CUtensorMap tm_do;   // [T_total, H, 128] bf16, boxes of 64 tokens x 64 features of a head
+    int with_bwd;        // prep: also produce E
+};
+
 // ------------------------------------------------------------------------------------------------
-// cw_prep
+// cw_prep: P, T, W^T, U~^T and, for a backward, E = scale (Q~ - P W)^T dO.  Two CTAs per SM, as tc_prep_lr: a chain of four
+// dependent phases, whose waits the neighbour fills: 95 -> 70 us on 4 x 16 heads of 2048 tokens against one CTA with look-ahead.
+// K- is needed by the first product only and shares its place with the fp32
+// blocks of the inversion and the staged E, so it is loaded at the top of its trip.
 // ------------------------------------------------------------------------------------------------
 namespace prepcw {
-constexpr uint32_t QKP = 0;                 // [Q~ rows 0..63 ; K+ rows 64..127] x 128                               32 KB
-constexpr uint32_t KM = 32768;              // K- [64][128]                                     16 KB
-constexpr uint32_t VT = KM + 16384;         // V~ [64][128]                                     16 KB
-constexpr uint32_t DOT = VT + 16384;        // dO' [64][128]                                    16 KB
-constexpr uint32_t XA = DOT + 16384;        // fp32 A [64][kLdi]
-constexpr uint32_t XT = XA + 17408;         // fp32 T
-constexpr uint32_t TT = XT + 17408;         // T  bf16 [64][64]                                  8 KB
-constexpr uint32_t PT = TT + 8192;          // P  bf16 [64][64]                                  8 KB
-constexpr uint32_t WT = PT + 8192;          // W^T  [128][64]                                   16 KB
-constexpr uint32_t UTT = WT + 16384;        // U~^T [128][64]                                   16 KB
-constexpr uint32_t PDOT = UTT + 16384;      // (P^T dO')^T [128][64]                            16 KB
-constexpr uint32_t EST = XA;                // staged E image [128][128] over the fp32 A and T blocks                       32 KB
-constexpr uint32_t SMEM_BYTES = PDOT + 16384 + 1024;
-constexpr uint32_t C_S1 = 0, C_W = 64, C_U = 128, C_PDO = 192, C_E = 256;   // TMEM columns (512 allocated)
-static_assert(EST % 1024 == 0 && EST + 32768 <= TT, "the E image fits over the fp32 A and T blocks");
-static_assert(TT % 1024 == 0 && SMEM_BYTES <= 225 * 1024, "tile alignment and shared memory budget");
+constexpr uint32_t QKP = 0;                 // [Q~ rows 0..63 ; K+ rows 64..127] x 128                              32 KB
+constexpr uint32_t VO = 32768;              // [V~ ; dO] x 128                                                      32 KB
+constexpr uint32_t XA = VO + 32768;         // K- [64][128]; then fp32 A [64][kLdi]; then T and W^T; finally the E image
+constexpr uint32_t XT = XA + 17408;         // fp32 T [64][kLdi]
+constexpr uint32_t PT = XT + 17408;         // P = tril(Q~ K-^T)                                                     8 KB
+constexpr uint32_t KM = XA, TT = XA, WT = XA + 8192, ES = XA;
+// U~^T [128][64] over V~ and (P^T dO)^T [128][64] over K+: two pieces of 64 rows each, 16 KB apart
+constexpr uint32_t UTT = VO, PDOT = QKP + 8192;
+constexpr uint32_t SMEM_BYTES = PT + 8192 + 1024 /* alignment slack */;
+constexpr uint32_t C_S1 = 0, C_PDO = 64, C_W = 128, C_U = 192, C_E = 0;   // TMEM columns (256 allocated; E over S1 and P^T dO)
+static_assert(ES + 32768 <= PT && PT % 1024 == 0, "T, W^T and the E image fit over the fp32 blocks");
+static_assert(2 * (SMEM_BYTES + 4096) <= 228 * 1024, "two CTAs per SM");
 }  // namespace prepcw
 
-// mode 0: the forward's share (P, A, T, W, U~); 1: that and E (closed backward); 2: E alone from the stored P and W^T
-// (backward on a workspace fresh from the forward: no product, inversion or store of the forward is repeated).
-__global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
+__global__ void __launch_bounds__(kT, 2) cw_prep_kernel(const __grid_constant__ CwParams P) {
     wait_prerequisites();
     using namespace prepcw;
+    const Problem& p = P.p;
     const int H = p.d.H;
     const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
-    if (hdr->status != GDN_OK) return;
+    if (!cw_go(hdr)) return;
     const int n_items = hdr->n_chunks * H;
     if ((int)blockIdx.x >= n_items) return;
+    const bool bwd = P.with_bwd != 0;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sm = align1024(smem_raw);
-    __shared__ uint64_t bar_in, bar_mma;
+    __shared__ uint64_t bar_in, bar_k, bar_mma;
     __shared__ uint32_t tmem_slot;
     const int warp = warp_id(), lane = threadIdx.x & 31;
     const int q4 = warp & 3, grp = warp >> 2;
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
-    if (threadIdx.x == 0) { mbar_init(&bar_in, 1); mbar_init(&bar_mma, 1); fence_mbar_init(); }
-    if (warp == 0) { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
+    if (threadIdx.x == 0) { mbar_init(&bar_in, 1); mbar_init(&bar_k, 1); mbar_init(&bar_mma, 1); fence_mbar_init(); }
+    if (warp == 0) { tmem_alloc(&tmem_slot, 256); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
     float* Af = reinterpret_cast<float*>(sm + XA);
     float* Tf = reinterpret_cast<float*>(sm + XT);
-    const bool bwd = mode != 0, fresh = mode == 2;
+    const float sc = p.d.scale;
     bool ok = true, pending = false;
-    uint32_t mma_phase = 0, in_phase = 0, pending_phase = 0;   // (pending_phase: the phase of bar_in the loads in flight belong to)
-    // The tiles of a trip arrive in two pieces on one mbarrier phase, each issued during the trip before as soon as the
-    // last product that reads its region is done (E is staged over the fp32 A and T blocks, never over an input tile):
-    //   closed / forward:  a = K-                     after step 1      b = [Q~; K+], V~, dO'     after step 2
-    //   fresh workspace:   a = Q~, dO', stored P      after its first products      b = stored W^T   after step 3
-    auto load_a = [&](size_t c, uint32_t phase) {   // thread 0; the first piece announces the whole trip's bytes
-        pending_phase = phase;
+    uint32_t mma_phase = 0, in_phase = 0;
+    // [Q~; K+], V~ and dO of a trip are dead once its last product is done: the next trip's are loaded right then, under the
+    // readout of E and its store.
+    auto issue_loads = [&](const ChunkInfo& c) {   // thread 0
+        mbar_expect_tx(&bar_in, 49152 + (bwd ? 16384 : 0));
+        bulk_load(sm + QKP, p.ws + p.L.img_QKp + (size_t)c.ch * 32768, 32768, &bar_in);
+        for (int cb = 0; cb < 2; ++cb) {
+            bulk_load(sm + VO + cb * 16384, p.ws + p.L.img_Vt + (size_t)c.ch * 16384 + cb * 8192, 8192, &bar_in);
+            if (bwd) tma_load_3d(sm + VO + cb * 16384 + 8192, &P.tm_do, cb * 64, c.hd, c.tok0, &bar_in);
+        }
+        prefetch_l2_bulk(p.ws + p.L.img_Km + (size_t)c.ch * 16384, 16384);
         pending = true;
-        if (fresh) {
-            mbar_expect_tx(&bar_in, 16384 + 16384 + 8192 + 16384);
-            for (int cb = 0; cb < 2; ++cb) bulk_load(sm + QKP + cb * 16384, p.ws + p.L.img_QKp + c * 32768 + cb * 16384, 8192, &bar_in);
-            bulk_load(sm + DOT, p.ws + p.L.img_dO + c * 16384, 16384, &bar_in);
-            bulk_load(sm + PT, p.ws + p.L.Pm + c * 8192, 8192, &bar_in);
-        } else {
-            mbar_expect_tx(&bar_in, 65536 + (bwd ? 16384 : 0));
-            bulk_load(sm + KM, p.ws + p.L.img_Km + c * 16384, 16384, &bar_in);
-        }
     };
-    auto load_b = [&](size_t c) {
-        if (fresh) {
-            bulk_load(sm + WT, p.ws + p.L.img_W + c * 16384, 16384, &bar_in);
-        } else {
-            bulk_load(sm + QKP, p.ws + p.L.img_QKp + c * 32768, 32768, &bar_in);
-            bulk_load(sm + VT, p.ws + p.L.img_Vt + c * 16384, 16384, &bar_in);
-            if (bwd) bulk_load(sm + DOT, p.ws + p.L.img_dO + c * 16384, 16384, &bar_in);
-        }
-    };
-    if (threadIdx.x == 0) { load_a(blockIdx.x, 0); load_b(blockIdx.x); }
+    ChunkInfo x;
+    chunk_entry_tab(p, x, blockIdx.x);
+    if (threadIdx.x == 0) issue_loads(x);
 #pragma unroll 1
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, in_phase ^= 1) {
-        const size_t ch = (size_t)item, chn = ch + gridDim.x;
         const bool has_next = item + (int)gridDim.x < n_items;
-        if (warp == 0) bulk_wait_read<0>();   // the previous trip's stores have read their tiles (rewritten from here on)
+        ChunkInfo xn = x;
+        if (has_next) chunk_entry_tab(p, xn, item + gridDim.x);
+        if (warp == 0 && elect_one()) {
+            bulk_wait_read<0>();   // the previous trip's stores have read P and the E image: rewritten from here on
+            mbar_expect_tx(&bar_k, 16384);
+            bulk_load(sm + KM, p.ws + p.L.img_Km + (size_t)x.ch * 16384, 16384, &bar_k);
+        }
         if (ok) {
             ok = mbar_wait(&bar_in, in_phase);
-            if (!ok && threadIdx.x == 0) report_timeout(p.ws, 40);
             if (ok && threadIdx.x == 0) pending = false;
         }
-        __syncthreads();
-        if (fresh) {
-            // (P^T dO')^T and Q~^T dO' from the loaded tiles; then E = Q~^T dO' - W^T (P^T dO') as in the closed arm
-            if (warp == 0 && elect_one() && ok) {
-                tc_fence_after();
-                mma_tile<128, 64, 64>(tmem + C_PDO, op_mn_major(sm + DOT, 64), op_mn_major(sm + PT, 64), false);
-                mma_tile<128, 128, 64>(tmem + C_E, op_mn_major(sm + QKP, 128, 0), op_mn_major(sm + DOT, 64), false);
-                mma_commit(&bar_mma);
-            }
-            GDN_WAIT_MMA(45)
-            if (ok && has_next && threadIdx.x == 0) load_a(chn, in_phase ^ 1);   // Q~, dO' and P have been read for the last time
-            if (ok) {
-                const int f = q4 * 32 + lane, i0 = grp * 32;
-#pragma unroll 1
-                for (int part = 0; part < 4; ++part) {
-                    const int ib = i0 + part * 8;
-                    float v[8];
-                    tmem_ld8(tmem + lane_base + C_PDO + ib, v);
-                    tmem_wait_ld();
-                    chunk_store(sm + PDOT, 128, f, ib >> 3, v);
-                }
-            }
-            tc_fence_before();
+        {   // (waited for in any case: it is in flight)
+            const bool okk = mbar_wait(&bar_k, in_phase);
+            ok = ok && okk;
+            if (!ok && threadIdx.x == 0) report_timeout(p.ws, 40);
+        }
+        if (ok && bwd && x.len < kC) {   // rows beyond the sequence belong to somebody else (the images have zeros there)
+            zero_tail_rows(sm + VO, 128, 64, x.len, kT);
             fence_async_smem();
-            __syncthreads();
-        } else {
-        // ---- step 1: S1 = [Q~; K+] K-^T  (rows 0..63: P before masking, rows 64..127: A)
+        }
+        __syncthreads();
+        // ---- phase 1: S1 = [Q~; K+] K-^T  (rows 0..63: P before masking, rows 64..127: A)
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 128>(tmem + C_S1, op_k_major(sm + QKP, 128, 0), op_k_major(sm + KM, 64), false);
             mma_commit(&bar_mma);
         }
         GDN_WAIT_MMA(41)
-        if (ok && has_next && threadIdx.x == 0) load_a(chn, in_phase ^ 1);   // K- has been read for the last time
         if (ok) {
             const int i = (q4 & 1) * 32 + lane, j0 = grp * 32;
-#pragma unroll 1
+#pragma unroll 2
             for (int part = 0; part < 4; ++part) {
                 float v[8];
                 const int jb = j0 + part * 8;
@@ -307,115 +256,245 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
         tc_fence_before();
         fence_async_smem();
         __syncthreads();
-        // (P^T dO')^T and Q~^T dO' need nothing of the inversion: they run under it, covered by the next commit
-        if (warp == 0 && elect_one() && ok && bwd) {
+        // (P^T dO)^T needs nothing of the inversion: it runs under it, covered by the next commit
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
-            mma_tile<128, 64, 64>(tmem + C_PDO, op_mn_major(sm + DOT, 64), op_mn_major(sm + PT, 64), false);
-            mma_tile<128, 128, 64>(tmem + C_E, op_mn_major(sm + QKP, 128, 0), op_mn_major(sm + DOT, 64), false);
+            if (bwd) mma_tile<128, 64, 64>(tmem + C_PDO, op_mn_major(sm + VO, 128, 64), op_mn_major(sm + PT, 64), false);
+            bulk_store(p.ws + p.L.Pm + (size_t)x.ch * 8192, sm + PT, 8192);
+            bulk_commit();
         }
-        // ---- T = (I + A)^-1, blocked, fp32
         invert64(Af, Tf, [] { __syncthreads(); });
-        {   // T -> bf16 tile: a thread converts two rows of one 8-column piece
+        {   // T -> bf16 tile over A: every row is in registers before the first one is written
             const int cch = threadIdx.x & 7;
+            float a[2][8];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int i = (threadIdx.x >> 3) + 32 * h;
-                float a[8];
-                if ((cch >> 1) <= (i >> 4)) {   // blocks above the block diagonal are zero and were never written
-                    ld8s(Tf + i * kLdi + cch * 8, a);
+                if ((cch >> 1) <= (i >> 4)) {   // (beyond the block diagonal: zero)
+                    ld8s(Tf + i * kLdi + cch * 8, a[h]);
                 } else {
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) a[k] = 0.f;
+                    for (int k = 0; k < 8; ++k) a[h][k] = 0.f;
                 }
-                chunk_store(sm + TT, 64, i, cch, a);
             }
+            __syncthreads();
+#pragma unroll
+            for (int h = 0; h < 2; ++h) chunk_store(sm + TT, 64, (threadIdx.x >> 3) + 32 * h, cch, a[h]);
         }
         fence_async_smem();
         __syncthreads();
-        // ---- step 2: W^T = K+^T T^T ; U~^T = V~^T T^T
+        // ---- phase 2: W^T = K+^T T^T ; U~^T = V~^T T^T
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 64>(tmem + C_W, op_mn_major(sm + QKP, 128, 64), op_k_major(sm + TT, 64), false);
-            mma_tile<128, 64, 64>(tmem + C_U, op_mn_major(sm + VT, 64), op_k_major(sm + TT, 64), false);
+            mma_tile<128, 64, 64>(tmem + C_U, op_mn_major(sm + VO, 128, 0), op_k_major(sm + TT, 64), false);
             mma_commit(&bar_mma);
+            bulk_store(p.ws + p.L.Tm + (size_t)x.ch * 8192, sm + TT, 8192);
+            bulk_commit();
         }
         GDN_WAIT_MMA(42)
-        if (ok && has_next && threadIdx.x == 0) load_b(chn);   // [Q~; K+], V~ and dO' have been read for the last time
         if (ok) {
             const int f = q4 * 32 + lane, i0 = grp * 32;
+            unsigned char* ut = sm + UTT + (f >> 6) * 16384;      // this feature's half of the two-piece tiles
+            unsigned char* pd = sm + PDOT + (f >> 6) * 16384;
 #pragma unroll 1
             for (int part = 0; part < 4; ++part) {
                 const int ib = i0 + part * 8;
-                float v[8];
-                tmem_ld8(tmem + lane_base + C_W + ib, v);
+                float a[8], b[8], c[8];
+                tmem_ld8(tmem + lane_base + C_W + ib, a);
+                tmem_ld8(tmem + lane_base + C_U + ib, b);
+                tmem_ld8(tmem + lane_base + C_PDO + ib, c);
                 tmem_wait_ld();
-                chunk_store(sm + WT, 128, f, ib >> 3, v);
-                tmem_ld8(tmem + lane_base + C_U + ib, v);
-                tmem_wait_ld();
-                chunk_store(sm + UTT, 128, f, ib >> 3, v);
-                if (bwd) {
-                    tmem_ld8(tmem + lane_base + C_PDO + ib, v);
-                    tmem_wait_ld();
-                    chunk_store(sm + PDOT, 128, f, ib >> 3, v);
-                }
+                chunk_store(sm + WT, 128, f, ib >> 3, a);
+                chunk_store(ut, 64, f & 63, ib >> 3, b);
+                if (bwd) chunk_store(pd, 64, f & 63, ib >> 3, c);
             }
         }
         tc_fence_before();
         fence_async_smem();
         __syncthreads();
-        }   // (!fresh)
-        // ---- step 3: E = Q~^T dO' - W^T (P^T dO')
-        if (bwd) {
-            if (warp == 0 && elect_one() && ok) {
-                tc_fence_after();
-                mma_tile<128, 128, 64>(tmem + C_E, op_k_major(sm + WT, 128), op_k_major(sm + PDOT, 128), true, /*neg_a=*/true);
-                mma_commit(&bar_mma);
-            }
-            GDN_WAIT_MMA(43)
-            if (ok && fresh && has_next && threadIdx.x == 0) load_b(chn);   // W^T has been read for the last time
-            if (ok) {   // E -> bf16 tile image, staged over the fp32 A and T blocks (dead since T was converted)
-                const int r = q4 * 32 + lane, c0 = grp * 64;
-#pragma unroll 1
-                for (int part = 0; part < 8; ++part) {
-                    const int cb = c0 + part * 8;
-                    float v[8];
-                    tmem_ld8(tmem + lane_base + C_E + cb, v);
-                    tmem_wait_ld();
-                    chunk_store(sm + EST, 128, r, cb >> 3, v);
-                }
-            }
-            tc_fence_before();
-            fence_async_smem();
-            __syncthreads();
-        }
+        // ---- phase 3: E = Q~^T dO - W^T (P^T dO)   (the second operand of the second product in two pieces: 64 columns each)
         if (warp == 0 && elect_one() && ok) {
-            if (!fresh) {
-                bulk_store(p.ws + p.L.Tm + ch * 8192, sm + TT, 8192);
-                bulk_store(p.ws + p.L.Pm + ch * 8192, sm + PT, 8192);
-                bulk_store(p.ws + p.L.img_W + ch * 16384, sm + WT, 16384);
-                bulk_store(p.ws + p.L.img_U + ch * 16384, sm + UTT, 16384);
+            tc_fence_after();
+            if (bwd) {
+                mma_tile<128, 128, 64>(tmem + C_E, op_mn_major(sm + QKP, 128, 0), op_mn_major(sm + VO, 128, 64), false);
+                mma_tile<128, 64, 64>(tmem + C_E, op_k_major(sm + WT, 128), op_k_major(sm + PDOT, 64), true, /*neg_a=*/true);
+                mma_tile<128, 64, 64>(tmem + C_E + 64, op_k_major(sm + WT, 128), op_k_major(sm + PDOT + 16384, 64), true, /*neg_a=*/true);
             }
-            if (bwd) bulk_store(p.ws + p.L.img_E + ch * 32768, sm + EST, 32768);
+            bulk_store(p.ws + p.L.img_W + (size_t)x.ch * 16384, sm + WT, 16384);
+            bulk_store(p.ws + p.L.img_U + (size_t)x.ch * 16384, sm + UTT, 8192);
+            bulk_store(p.ws + p.L.img_U + (size_t)x.ch * 16384 + 8192, sm + UTT + 16384, 8192);
+            bulk_commit();
+            bulk_wait_read<0>();   // T, W^T and U~^T have left: the E image and the next inputs go over them
+            mma_commit(&bar_mma);
+        }
+        GDN_WAIT_MMA(43)
+        if (ok && has_next && threadIdx.x == 0) issue_loads(xn);   // every input tile has been read for the last time
+        if (ok && bwd) {   // E -> bf16 tile image
+            const int rr = q4 * 32 + lane, c0 = grp * 64;
+#pragma unroll 2
+            for (int part = 0; part < 8; ++part) {
+                const int cb = c0 + part * 8;
+                float v[8];
+                tmem_ld8(tmem + lane_base + C_E + cb, v);
+                tmem_wait_ld();
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] *= sc;
+                chunk_store(sm + ES, 128, rr, cb >> 3, v);
+            }
+        }
+        tc_fence_before();
+        fence_async_smem();
+        __syncthreads();
+        if (warp == 0 && elect_one() && ok && bwd) {
+            bulk_store(p.ws + p.L.img_E + (size_t)x.ch * 32768, sm + ES, 32768);
             bulk_commit();
         }
         if (!ok) break;
+        x = xn;
     }
     if (warp == 0) bulk_wait_read<0>();
-    if (threadIdx.x == 0 && pending) (void)mbar_wait(&bar_in, pending_phase);   // after a timeout a load may still be in flight
+    if (threadIdx.x == 0 && pending) (void)mbar_wait(&bar_in, in_phase);   // after a timeout a load may still be in flight
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, 512);
+    if (warp == 0) tmem_dealloc(tmem, 256);
+}
+
+// ------------------------------------------------------------------------------------------------
+// cw_eprep: E alone, from the stored P and W^T (backward on a workspace fresh from the forward).  Two CTAs per SM.
+// ------------------------------------------------------------------------------------------------
+namespace eprepcw {
+constexpr uint32_t QT = 0;                  // Q~ [64][128]                                  16 KB
+constexpr uint32_t DOT = 16384;             // dO [64][128]                                  16 KB
+constexpr uint32_t WT = 32768;              // W^T [128][64]                                 16 KB
+constexpr uint32_t PT = 49152;              // P [64][64]                                     8 KB
+constexpr uint32_t PDOT = PT + 8192;        // (P^T dO)^T [128][64]                          16 KB
+constexpr uint32_t ES = PDOT + 16384;       // staged E image [128][128]                     32 KB
+constexpr uint32_t SMEM_BYTES = ES + 32768 + 1024 /* alignment slack */;
+constexpr uint32_t C_PDO = 0, C_E = 128;    // TMEM columns (256 allocated)
+static_assert(2 * (SMEM_BYTES + 4096) <= 228 * 1024, "two CTAs per SM");
+}  // namespace eprepcw
+
+__global__ void __launch_bounds__(kT, 2) cw_eprep_kernel(const __grid_constant__ CwParams P) {
+    wait_prerequisites();
+    using namespace eprepcw;
+    const Problem& p = P.p;
+    const int H = p.d.H;
+    const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
+    if (!cw_go(hdr)) return;
+    const int n_items = hdr->n_chunks * H;
+    if ((int)blockIdx.x >= n_items) return;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* sm = align1024(smem_raw);
+    __shared__ uint64_t bar_in, bar_mma;
+    __shared__ uint32_t tmem_slot;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
+    const int q4 = warp & 3, grp = warp >> 2;
+    const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
+    if (threadIdx.x == 0) { mbar_init(&bar_in, 1); mbar_init(&bar_mma, 1); fence_mbar_init(); }
+    if (warp == 0) { tmem_alloc(&tmem_slot, 256); tmem_relinquish(); }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+    const float sc = p.d.scale;
+    bool ok = true, pending = false;
+    uint32_t mma_phase = 0, in_phase = 0;
+    auto issue_loads = [&](const ChunkInfo& c) {   // thread 0: every tile of a trip is dead once its last product is done
+        mbar_expect_tx(&bar_in, 57344);
+        for (int cb = 0; cb < 2; ++cb) {
+            bulk_load(sm + QT + cb * 8192, p.ws + p.L.img_QKp + (size_t)c.ch * 32768 + cb * 16384, 8192, &bar_in);
+            tma_load_3d(sm + DOT + cb * 8192, &P.tm_do, cb * 64, c.hd, c.tok0, &bar_in);
+        }
+        bulk_load(sm + PT, p.ws + p.L.Pm + (size_t)c.ch * 8192, 8192, &bar_in);
+        bulk_load(sm + WT, p.ws + p.L.img_W + (size_t)c.ch * 16384, 16384, &bar_in);
+        pending = true;
+    };
+    ChunkInfo x;
+    chunk_entry_tab(p, x, blockIdx.x);
+    if (threadIdx.x == 0) issue_loads(x);
+#pragma unroll 1
+    for (int item = blockIdx.x; item < n_items; item += gridDim.x, in_phase ^= 1) {
+        const bool has_next = item + (int)gridDim.x < n_items;
+        ChunkInfo xn = x;
+        if (has_next) chunk_entry_tab(p, xn, item + gridDim.x);
+        if (ok) {
+            ok = mbar_wait(&bar_in, in_phase);
+            if (!ok && threadIdx.x == 0) report_timeout(p.ws, 46);
+            if (ok && threadIdx.x == 0) pending = false;
+        }
+        if (ok && x.len < kC) {
+            zero_tail_rows(sm + DOT, 64, 0, x.len, kT);
+            fence_async_smem();
+        }
+        __syncthreads();
+        if (warp == 0 && elect_one() && ok) {   // (P^T dO)^T ; Q~^T dO
+            tc_fence_after();
+            mma_tile<128, 64, 64>(tmem + C_PDO, op_mn_major(sm + DOT, 64), op_mn_major(sm + PT, 64), false);
+            mma_commit(&bar_mma);
+            mma_tile<128, 128, 64>(tmem + C_E, op_mn_major(sm + QT, 64), op_mn_major(sm + DOT, 64), false);
+        }
+        GDN_WAIT_MMA(47)
+        if (ok) {
+            const int f = q4 * 32 + lane, i0 = grp * 32;
+#pragma unroll 2
+            for (int part = 0; part < 4; ++part) {
+                float v[8];
+                tmem_ld8(tmem + lane_base + C_PDO + i0 + part * 8, v);
+                tmem_wait_ld();
+                chunk_store(sm + PDOT, 128, f, (i0 >> 3) + part, v);
+            }
+        }
+        tc_fence_before();
+        fence_async_smem();
+        __syncthreads();
+        if (warp == 0 && elect_one() && ok) {   // E -= W^T (P^T dO)
+            tc_fence_after();
+            mma_tile<128, 128, 64>(tmem + C_E, op_k_major(sm + WT, 128), op_k_major(sm + PDOT, 128), true, /*neg_a=*/true);
+            bulk_wait_read<0>();   // the previous trip's store has read the E image
+            mma_commit(&bar_mma);
+        }
+        GDN_WAIT_MMA(48)
+        if (ok && has_next && threadIdx.x == 0) issue_loads(xn);
+        if (ok) {
+            const int rr = q4 * 32 + lane, c0 = grp * 64;
+#pragma unroll 2
+            for (int part = 0; part < 8; ++part) {
+                const int cb = c0 + part * 8;
+                float v[8];
+                tmem_ld8(tmem + lane_base + C_E + cb, v);
+                tmem_wait_ld();
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] *= sc;
+                chunk_store(sm + ES, 128, rr, cb >> 3, v);
+            }
+        }
+        tc_fence_before();
+        fence_async_smem();
+        __syncthreads();
+        if (warp == 0 && elect_one() && ok) {
+            bulk_store(p.ws + p.L.img_E + (size_t)x.ch * 32768, sm + ES, 32768);
+            bulk_commit();
+        }
+        if (!ok) break;
+        x = xn;
+    }
+    if (warp == 0) bulk_wait_read<0>();
+    if (threadIdx.x == 0 && pending) (void)mbar_wait(&bar_in, in_phase);   // after a timeout a load may still be in flight
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, 256);
 }
 
 // ------------------------------------------------------------------------------------------------
 // cw_intra: every gradient of one (chunk, head).
 //
 // Four dependent steps (products; [readout] what the threads make of them):
-//   1  (W h)^T ; (K- dh'')^T ; (P^T dO')^T            [U = U~ - W h ; dU = P^T dO' + K- dh'']
-//   2  dP = dO' U^T ; dXv^T = dU^T T ; under the readout dQ~^T = h dO'^T ; dK-^T = dh'' U^T        [tril ; dv, dw]
-//   3  dA = dXv U^T (K#2) ; under the readout dK+^T = -h dXv^T ; dQ~^T += K-^T dP^T ; Q~^T dP      [-stril]
+//   1  (W h)^T ; (K- dh'')^T ; (P^T dO)^T             [U = U~ - W h ; dU = scale P^T dO + K- dh'']
+//   2  dP = dO U^T ; dXv^T = dU^T T ; under the readout h dO^T ; dK-^T = dh'' U^T        [scale tril ; dv, dw]
+//   3  dA = dXv U^T (K#2) ; under the readout dK+^T = -h dXv^T ; K-^T dP^T ; Q~^T dP               [-stril]
 //   4  dK+^T += K-^T dA^T ; (Q~^T dP) += K+^T dA                                                   [dq, dk, db, dg]
-// What bounds it is HBM: 176 KB of operand images, 144 KB of gates, inputs and gammas, 144 KB of gradients per chunk-head.  The
+// What bounds it is HBM: 176 KB of operands, 144 KB of gates, inputs and gammas, 144 KB of gradients per chunk-head.  The
 // gradients are made with features on the TMEM lanes and tokens on the columns: a warp's accesses to the gate vectors and
 // gradients are then whole 128-byte lines, all lanes work (a 64-row accumulator fills half of them), and the sums of dg
 // over the tokens of a chunk run along a thread's own columns.  So nothing passes through HBM between the products and the
@@ -426,7 +505,7 @@ __global__ void __launch_bounds__(kT, 1) cw_prep_kernel(Problem p, int mode) {
 namespace intracw {
 constexpr uint32_t QKM = 0;                 // [Q~ rows 0..63 ; K- rows 64..127] x 128         32 KB
 constexpr uint32_t KP = 32768;              // K+ [64][128]                                     16 KB
-constexpr uint32_t DOT = KP + 16384;        // dO' [64][128]                                    16 KB
+constexpr uint32_t DOT = KP + 16384;        // dO  [64][128]                                    16 KB
 constexpr uint32_t WT = DOT + 16384;        // W^T  [128][64]                                   16 KB
 constexpr uint32_t UTT = WT + 16384;        // U~^T [128][64]                                   16 KB
 constexpr uint32_t TT = UTT + 16384;        // T [64][64]; later dA                              8 KB
@@ -440,6 +519,7 @@ constexpr uint32_t DA = TT, DP = PT, DXVT = DUT;   // (dA over T, dP over P, dXv
 // TMEM columns (512 allocated, fixed offsets): eight accumulators of 64 columns, features on the lanes except dP and dA
 // (token rows on lanes 0..15 of each quadrant).
 constexpr uint32_t C_A = 0, C_B = 64, C_PDO = 128, C_PP = 192, C_DQ = 256, C_KM = 320, C_KP = 384, C_KM2 = 448;
+constexpr uint32_t C_DQ2 = C_B;             // (K-^T dP^T, over an accumulator of step 1)
 constexpr int kWorkers = 512;               // 16 readout warps: lane quadrant = warp % 4, tokens 16 (warp / 4) ..
                                             // (a seventeenth warp would cost every thread 32 of its 128 registers; warp 0 issues
                                             // the products, warp 1 the loads)
@@ -447,12 +527,13 @@ constexpr int kTok = 16;                    // tokens of a thread
 static_assert(SMEM_BYTES <= 220 * 1024, "shared memory budget");
 }  // namespace intracw
 
-__global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem p) {
+__global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(const __grid_constant__ CwParams P) {
     wait_prerequisites();
     using namespace intracw;
+    const Problem& p = P.p;
     const int H = p.d.H;
     const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
-    if (hdr->status != GDN_OK) return;
+    if (!cw_go(hdr)) return;
     const int n_items = hdr->n_chunks * H;
     if ((int)blockIdx.x >= n_items) return;
     extern __shared__ unsigned char smem_raw[];
@@ -475,12 +556,13 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
     const int f = q4 * 32 + lane;             // feature row of the M = 128 accumulators
     const int tr = q4 * 16 + (lane & 15);     // token row of the M = 64 accumulators (lanes 0..15 of the quadrant)
     const int i0 = grp * kTok;                // first of this thread's 16 tokens
+    const float sc = p.d.scale;
     const bool ga = lane < 16;
     bool ok = true;
     uint32_t mma_phase = 0, in_phase = 0;
     // The tiles of a trip arrive in groups, each loaded during the previous trip as soon as the last product that reads its
     // region is done (look-ahead without a second buffer):
-    //   b  W^T, U~^T     after the first readout          a  dO' after step 2, P after step 4
+    //   b  W^T, U~^T     after the first readout          a  dO after step 2, P after step 4
     //   s  dh'' after step 2, h after step 4              k  Q~, K-, K+, T after step 4
     bool pend_s = false, pend_a = false, pend_b = false, pend_k = false;   // the elected lane of warp 1
     auto load_s1 = [&](size_t c) {
@@ -489,9 +571,11 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
         pend_s = true;
     };
     auto load_s2 = [&](size_t c) { bulk_load(sm + HH, p.ws + p.L.hc + c * 32768, 32768, &bar_s); };
-    auto load_a1 = [&](size_t c) {
+    auto load_a1 = [&](int c) {
+        ChunkInfo y;
+        chunk_entry_tab(p, y, c);
         mbar_expect_tx(&bar_a, 24576);
-        bulk_load(sm + DOT, p.ws + p.L.img_dO + c * 16384, 16384, &bar_a);
+        for (int cb = 0; cb < 2; ++cb) tma_load_3d(sm + DOT + cb * 8192, &P.tm_do, cb * 64, y.hd, y.tok0, &bar_a);
         pend_a = true;
     };
     auto load_a2 = [&](size_t c) { bulk_load(sm + PT, p.ws + p.L.Pm + c * 8192, 8192, &bar_a); };
@@ -513,23 +597,17 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
         bulk_load(sm + TT, p.ws + p.L.Tm + c * 8192, 8192, &bar_k);
         pend_k = true;
     };
-    auto chunk_of = [&](int it) {
-        ChunkInfo x;
-        x.c = it / H; x.hd = it % H; x.ch = it;
-        x.tok0 = reinterpret_cast<const int32_t*>(p.ws + p.L.chunk_tok0)[x.c];
-        x.len = reinterpret_cast<const int32_t*>(p.ws + p.L.chunk_len)[x.c];
-        return x;
-    };
     if (warp == 1 && elect_one()) {
         const size_t c = blockIdx.x;
-        load_s1(c); load_s2(c); load_k(c); load_b(c); load_a1(c); load_a2(c);
+        load_s1(c); load_s2(c); load_k(c); load_b(c); load_a1((int)c); load_a2(c);
     }
 #pragma unroll 1
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, in_phase ^= 1) {
         const size_t ch = (size_t)item;
         const bool has_next = item + (int)gridDim.x < n_items;
         const size_t chn = ch + gridDim.x;
-        const ChunkInfo x = chunk_of(item);
+        ChunkInfo x;
+        chunk_entry_tab(p, x, item);
         const size_t rs = (size_t)H * D, base = ((size_t)x.tok0 * H + x.hd) * D + (size_t)i0 * rs + f;   // this thread's channel of its first token
         const int live = x.len - i0;          // tokens of this thread inside the sequence (may be negative)
         const bool whole = live >= kTok;      // (two copies of the accesses: a condition at each of them costs more than it skips)
@@ -537,6 +615,10 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
             ok = mbar_wait(&bar_s, in_phase) && mbar_wait(&bar_k, in_phase) && mbar_wait(&bar_b, in_phase) && mbar_wait(&bar_a, in_phase);
             if (!ok && threadIdx.x == 0) report_timeout(p.ws, 44);
             if (ok) pend_s = pend_k = pend_a = pend_b = false;
+        }
+        if (ok && x.len < kC) {   // rows beyond the sequence belong to somebody else (the images have zeros there)
+            zero_tail_rows(sm + DOT, 64, 0, x.len, kWorkers);
+            fence_async_smem();
         }
         __syncthreads();
         // ---- step 1
@@ -559,7 +641,7 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
             }
         }
         GDN_WAIT_MMA(45)
-        if (ok) {   // U^T = U~^T - (W h)^T ; dU^T = (P^T dO')^T + (K- dh'')^T
+        if (ok) {   // U^T = U~^T - (W h)^T ; dU^T = scale (P^T dO)^T + (K- dh'')^T
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 const int ib = i0 + part * 8;
@@ -570,7 +652,7 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
                 chunk_load(sm + UTT, 128, f, ib >> 3, u);
                 tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 8; ++j) { u[j] -= t[j]; pd[j] += kb[j]; }
+                for (int j = 0; j < 8; ++j) { u[j] -= t[j]; pd[j] = fmaf(sc, pd[j], kb[j]); }
                 chunk_store(sm + UT, 128, f, ib >> 3, u);
                 chunk_store(sm + DUT, 128, f, ib >> 3, pd);
             }
@@ -622,13 +704,13 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
                 }
             }
 #pragma unroll
-            for (int part = 0; part < 2; ++part) {   // dP = tril(dO' U^T), rows on lanes 0..15
+            for (int part = 0; part < 2; ++part) {   // dP = scale tril(dO U^T), rows on lanes 0..15
                 const int jb = i0 + part * 8;
                 tmem_ld8(tmem + lane_base + C_PP + jb, v);
                 tmem_wait_ld();
                 if (ga) {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) v[j] = (jb + j <= tr) ? v[j] : 0.f;
+                    for (int j = 0; j < 8; ++j) v[j] = (jb + j <= tr) ? sc * v[j] : 0.f;
                     chunk_store(sm + DP, 64, tr, jb >> 3, v);
                 }
             }
@@ -642,11 +724,11 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
             mma_tile<64, 64, 128>(tmem + C_PP, op_mn_major(sm + DXVT, 128), op_mn_major(sm + UT, 128), false);
             mma_commit(&bar_mma);
             mma_tile<128, 64, 128>(tmem + C_KP, op_k_major(sm + HH, 128), op_mn_major(sm + DXVT, 128), false, /*neg_a=*/true);
-            mma_tile<128, 64, 64>(tmem + C_DQ, op_mn_major(sm + QKM, 128, 64), op_k_major(sm + DP, 64), true);
+            mma_tile<128, 64, 64>(tmem + C_DQ2, op_mn_major(sm + QKM, 128, 64), op_k_major(sm + DP, 64), false);
             mma_tile<128, 64, 64>(tmem + C_KM2, op_mn_major(sm + QKM, 128, 0), op_mn_major(sm + DP, 64), false);
         }
         GDN_WAIT_MMA(47)
-        if (warp == 1 && elect_one() && ok && has_next) { load_a1(chn); load_s1(chn); }   // dO' and dh'' have been read for the last time
+        if (warp == 1 && elect_one() && ok && has_next) { load_a1((int)chn); load_s1(chn); }   // dO and dh'' have been read for the last time
         if (ok) {   // dA = -stril(.)  (over T, which step 2 has read)
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
@@ -705,8 +787,9 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
             float* dbp = p.dbv + base;
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
-                float dq[8], kr[8], km[8], km2[8];
+                float dq[8], dq2[8], kr[8], km[8], km2[8];
                 tmem_ld8(tmem + lane_base + C_DQ + i0 + part * 8, dq);
+                tmem_ld8(tmem + lane_base + C_DQ2 + i0 + part * 8, dq2);
                 tmem_ld8(tmem + lane_base + C_KP + i0 + part * 8, kr);
                 tmem_ld8(tmem + lane_base + C_KM + i0 + part * 8, km);
                 tmem_ld8(tmem + lane_base + C_KM2 + i0 + part * 8, km2);
@@ -716,7 +799,7 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
                 for (int j = 0; j < 8; ++j) {
                     const float G = expf(g8[j]), iG = expf(-g8[j]);
                     const float q = __uint_as_float(q8[j] << 16), k = __uint_as_float(k8[j] << 16);
-                    dq[j] *= G;                                      // dq = Gam . dQ~
+                    dq[j] = G * fmaf(sc, dq[j], dq2[j]);             // dq = Gam . dQ~
                     const float row = G * kr[j];                     // what multiplies b . k in the row role
                     const float ucol = iG * km[j];
                     const float col = fmaf(iG, km2[j], ucol);        // column role
@@ -774,29 +857,34 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(Problem 
 
 // Host side: the channel-wise calls on this route (bf16 I/O, d_k = d_v = 128).
 cudaError_t cw_tc_launch(const Problem& p, bool bwd, bool skip_recompute, cudaStream_t st) {
-    static SmemLimitOnce once_scale, once_prep, once_intra;
+    static SmemLimitOnce once_scale, once_prep, once_eprep, once_intra;
     const int CH = p.L.max_chunks * p.d.H, chains = p.d.N * p.d.H;
-    cudaError_t e = launch_table(p, st);
-    if (e != cudaSuccess) return e;
-    if (CH > 0) {
-        int dev = 0, sms = 148;
-        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int grid = CH < sms ? CH : sms;
-        const uint32_t sm_scale = sizeof(float) * kC * (D + 1);
-        if ((e = once_scale.ensure(cw_scale_kernel, sm_scale)) != cudaSuccess) return e;
-        if ((e = once_prep.ensure(cw_prep_kernel, prepcw::SMEM_BYTES)) != cudaSuccess) return e;
-        const int mode = bwd ? (skip_recompute ? 2 : 1) : 0;
-        { StageScope t(ST_SCALE, st); launch_kernel(cw_scale_kernel, CH, kT, sm_scale, st, p, mode); }
-        { StageScope t(ST_PREP, st); launch_kernel(cw_prep_kernel, grid, kT, prepcw::SMEM_BYTES, st, p, mode); }
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    cudaError_t e;
+    const bool fresh = bwd && skip_recompute;   // the chunk table, the images, gam and the factors are still there
+    if (!fresh && (e = launch_table(p, st)) != cudaSuccess) return e;
+    const int sms = tc_sm_count(), grid = CH < sms ? CH : sms, grid2 = CH < 2 * sms ? CH : 2 * sms;
+    CwParams P;
+    P.p = p;
+    P.with_bwd = bwd ? 1 : 0;
+    if (p.Ttot > 0) {
+        if (!make_tmap_bf16_heads(&P.tm_do, bwd ? p.dO : p.v, p.Ttot, p.d.H, D)) return cudaErrorUnknown;
+        if (fresh) {
+            if ((e = once_eprep.ensure(cw_eprep_kernel, eprepcw::SMEM_BYTES)) != cudaSuccess) return e;
+            StageScope t(ST_EPREP, st);
+            e = launch_kernel(cw_eprep_kernel, grid2, kT, eprepcw::SMEM_BYTES, st, P);
+        } else {
+            const uint32_t sm_scale = sizeof(float) * kC * (D + 1);
+            if ((e = once_scale.ensure(cw_scale_kernel, sm_scale)) != cudaSuccess) return e;
+            if ((e = once_prep.ensure(cw_prep_kernel, prepcw::SMEM_BYTES)) != cudaSuccess) return e;
+            { StageScope t(ST_SCALE, st); launch_kernel(cw_scale_kernel, CH, kT, sm_scale, st, p); }
+            { StageScope t(ST_PREP, st); e = launch_kernel(cw_prep_kernel, grid2, kT, prepcw::SMEM_BYTES, st, P); }
+        }
+        if (e != cudaSuccess) return e;
     }
     if (chains > 0 && (e = tc_launch_scan_channelwise(p, bwd ? (skip_recompute ? 1 : 2) : 0, st)) != cudaSuccess) return e;
-    if (bwd && CH > 0) {
-        int dev = 0, sms = 148;
-        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int grid = CH < sms ? CH : sms;
+    if (bwd && p.Ttot > 0) {
         if ((e = once_intra.ensure(cw_intra_kernel, intracw::SMEM_BYTES)) != cudaSuccess) return e;
-        { StageScope t(ST_INTRA, st); launch_kernel(cw_intra_kernel, grid, intracw::kWorkers, intracw::SMEM_BYTES, st, p); }
+        { StageScope t(ST_INTRA, st); launch_kernel(cw_intra_kernel, grid, intracw::kWorkers, intracw::SMEM_BYTES, st, P); }
     }
     return cudaGetLastError();
 }
