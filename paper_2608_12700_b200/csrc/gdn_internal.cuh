@@ -73,6 +73,7 @@ inline WsLayout make_layout(const gdn_desc& d, size_t elem, size_t elem_add, siz
     L.Tm = take(elem * CH * kC * kC);
     L.W = take(elem * CH * kC * d.d_k);
     L.Ut = take(elem * CH * kC * d.d_v);
+    L.Pm = take(elem * CH * kC * kC);
     L.has_operator = with_operator ? 1 : 0;
     L.Nm = take(with_operator ? elem * CH * d.d_k * d.d_k : 0);
     L.Bf = take(with_operator ? elem_add * CH * d.d_k * d.d_v : 0);
@@ -80,7 +81,6 @@ inline WsLayout make_layout(const gdn_desc& d, size_t elem, size_t elem_add, siz
     L.fwd_end = o;
     L.E = take(elem_add * CH * d.d_k * d.d_v);
     L.dhn = take(elem * CH * d.d_k * d.d_v);
-    L.Pm = take(elem * CH * kC * kC);
     L.scratch_per_ch = scratch_per_ch;
     L.scratch = take(scratch_per_ch * CH);
     L.total = o;

@@ -43,7 +43,7 @@ struct TcParams {
     CUtensorMap tm_o;                      // same geometry, for the forward output (forward calls that want it)
     int with_bwd;                          // prep: also produce E
     int scan_dirs;                         // scan: 0 = forward carry only, 1 = reverse only, 2 = both
-    int lowrank;                           // carries in low-rank form (tc_scan_lr): prepared by tc_prep_lr / tc_factors without Nm, Bf
+    int lowrank;                           // carries in low-rank form (tc_scan_lr): prepared by tc_prep_lr without Nm, Bf
     int withhold;                          // debugging hook: tc_prep leaves out one of its first loads, so that the wait
                                            // for it runs out (exercises the time-out path without any fault)
 };
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
                 // T is staged
                 if (!(lok = mbar_wait(&bar_t, ph))) break;
                 bulk_store(p.ws + p.L.Tm + (size_t)x.ch * 8192, sm + TT, 8192);
-                if (bwd) bulk_store(p.ws + p.L.Pm + (size_t)x.ch * 8192, sm + PT, 8192);   // the gradient stage reads P from here
+                bulk_store(p.ws + p.L.Pm + (size_t)x.ch * 8192, sm + PT, 8192);   // the forward output and the gradient stage read P from here
                 bulk_commit();
                 // W^T, U~^T are staged and V, dO have been read for the last time
                 if (!(lok = mbar_wait(&bar_vofree, ph))) break;
@@ -1509,19 +1509,19 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
 // loaded as soon as the last product (or store) that reads their region is done.  Q h and P U are formed token-major
 // (M = 64: a thread owns a token row), so the output tile is staged with 16-byte stores and leaves by TMA.
 // CW: the channel-wise path.  Its preparation kernels leave Q~ = Gam.q, P = tril(Q~ K-^T), W^T, U~^T and the per-chunk
-// states in the workspace as tile images, the decay is inside Q~ and P, so o = scale (Q~ h + P (U~ - W h)): no product
-// Q K^T, no gates, and P U accumulates onto Q~ h.  P arrives in the half of the [Q ; K] tile that K would occupy.
+// states in the workspace as tile images, the decay is inside Q~ and P, so o = scale (Q~ h + P (U~ - W h)): no
+// gates here, and P U accumulates onto Q~ h.
 // ------------------------------------------------------------------------------------------------
 namespace outk {
-constexpr uint32_t QK = 0;                  // [Q rows 0..63 ; K rows 64..127] x 128              32 KB
-constexpr uint32_t WT = 32768;              // W^T [128][64]; after the first products: P [64][64]  16 KB
+constexpr uint32_t QT = 0;                  // Q or Q~ [64][128]                                     16 KB
+constexpr uint32_t PT = 16384;              // P [64][64]                                             8 KB
+constexpr uint32_t WT = PT + 8192;          // W^T [128][64]                                         16 KB
 constexpr uint32_t UTT = WT + 16384;        // U~^T [128][64]; U^T in place                         16 KB
 constexpr uint32_t HH = UTT + 16384;        // h [128][128]; after the first products: staged o     32 KB
-constexpr uint32_t PT = WT, STG = HH;
+constexpr uint32_t STG = HH;
 constexpr uint32_t SMEM_BYTES = HH + 32768 + 1024 /* alignment slack */;
-constexpr uint32_t C_P = 0, C_WH = 64, C_QH = 128, C_PU = 0;   // TMEM columns (256 allocated)
-constexpr uint32_t PT_CW = QK + 8192;        // channel-wise: P, loaded, in rows 64..127 of the first column block of [Q ; K]
-constexpr uint32_t IN_BYTES = 32768 + 16384 + 16384 + 32768, IN_BYTES_CW = 16384 + 8192 + 16384 + 16384 + 32768;
+constexpr uint32_t C_WH = 0, C_QH = 128, C_PU = 0;   // TMEM columns (256 allocated; P U over (W h)^T, which is read by then)
+constexpr uint32_t IN_BYTES = 16384 + 8192 + 16384 + 16384 + 32768;
 static_assert(2 * (SMEM_BYTES + 4096) <= 228 * 1024, "two CTAs per SM");
 }  // namespace outk
 
@@ -1537,7 +1537,7 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
     if ((int)blockIdx.x >= n_items) return;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sm = align1024(smem_raw);
-    __shared__ __align__(16) float gl[kC], Gam[kC];
+    __shared__ float Gam[kC];
     __shared__ uint64_t bar_in, bar_mma;
     __shared__ uint32_t tmem_slot;
     const int warp = warp_id(), lane = threadIdx.x & 31;
@@ -1552,23 +1552,19 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
     bool ok = true, pending = false;
     uint32_t mma_phase = 0, in_phase = 0, pending_phase = 0;   // (pending_phase: the phase of bar_in the loads in flight belong to)
     // One mbarrier phase per trip collects all five tiles; they are issued in three pieces, each when its region is free.
-    auto load_qk = [&](const ChunkInfo& c, uint32_t phase) {   // thread 0; first piece of a trip: announces the whole trip's bytes
+    auto load_q = [&](const ChunkInfo& c, uint32_t phase) {   // thread 0; first piece of a trip: announces the whole trip's bytes
         pending_phase = phase;
-        mbar_expect_tx(&bar_in, CW ? IN_BYTES_CW : IN_BYTES);
+        mbar_expect_tx(&bar_in, IN_BYTES);
         for (int cb = 0; cb < 2; ++cb) {
-            if (CW) {
-                bulk_load(sm + QK + cb * 16384, p.ws + p.L.img_QKp + (size_t)c.ch * 32768 + cb * 16384, 8192, &bar_in);
-            } else {
-                tma_load_3d(sm + QK + cb * 16384, &P.tm_q, cb * 64, c.hd, c.tok0, &bar_in);
-                tma_load_3d(sm + QK + cb * 16384 + 8192, &P.tm_k, cb * 64, c.hd, c.tok0, &bar_in);
-            }
+            if (CW) bulk_load(sm + QT + cb * 8192, p.ws + p.L.img_QKp + (size_t)c.ch * 32768 + cb * 16384, 8192, &bar_in);
+            else tma_load_3d(sm + QT + cb * 8192, &P.tm_q, cb * 64, c.hd, c.tok0, &bar_in);
         }
+        bulk_load(sm + WT, p.ws + (CW ? p.L.img_W : p.L.W) + (size_t)c.ch * 16384, 16384, &bar_in);
         pending = true;
     };
-    auto load_wu = [&](const ChunkInfo& c) {   // (channel-wise: and P, whose place the second product reads)
-        bulk_load(sm + WT, p.ws + (CW ? p.L.img_W : p.L.W) + (size_t)c.ch * 16384, 16384, &bar_in);
+    auto load_up = [&](const ChunkInfo& c) {
         bulk_load(sm + UTT, p.ws + (CW ? p.L.img_U : p.L.Ut) + (size_t)c.ch * 16384, 16384, &bar_in);
-        if (CW) bulk_load(sm + PT_CW, p.ws + p.L.Pm + (size_t)c.ch * 8192, 8192, &bar_in);
+        bulk_load(sm + PT, p.ws + p.L.Pm + (size_t)c.ch * 8192, 8192, &bar_in);
     };
     auto load_h = [&](const ChunkInfo& c) { bulk_load(sm + HH, p.ws + p.L.hc + (size_t)c.ch * 32768, 32768, &bar_in); };
     auto fetch_gamma = [&](const ChunkInfo& c) {   // threads 0..63: cumulative log decay of their token
@@ -1576,7 +1572,7 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
     };
     ChunkInfo x;
     chunk_entry(p, x, blockIdx.x);
-    if (threadIdx.x == 0) { load_qk(x, 0); load_wu(x); load_h(x); }
+    if (threadIdx.x == 0) { load_q(x, 0); load_up(x); load_h(x); }
     float gnext = (!CW && threadIdx.x < kC) ? fetch_gamma(x) : 0.f;
     const int f = q4 * 32 + lane;            // feature row of the transposed accumulator (W h)^T
     const int tr = q4 * 16 + (lane & 15);    // token row of the M = 64 accumulators (lanes 0..15 of a quadrant hold them)
@@ -1588,7 +1584,6 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
         ChunkInfo xn = x;
         if (has_next) chunk_entry(p, xn, item + gridDim.x);
         if (!CW && threadIdx.x < kC) {
-            gl[threadIdx.x] = gnext * kLog2e;
             Gam[threadIdx.x] = expf(gnext);
         }
         if (ok) {
@@ -1597,41 +1592,28 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
             if (ok && threadIdx.x == 0) pending = false;
         }
         if (!CW && ok && x.len < kC) {   // ragged tail: rows beyond the sequence belong to somebody else (the images are padded)
-            zero_tail_rows(sm + QK, 128, 0, x.len);
-            zero_tail_rows(sm + QK, 128, 64, x.len);
+            zero_tail_rows(sm + QT, 64, 0, x.len);
             fence_async_smem();
         }
         __syncthreads();
-        // ---- step 1: Q K^T ; (W h)^T ; Q h
+        // ---- step 1: (W h)^T ; under its readout Q h
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
-            if (!CW) mma_tile<64, 64, 128>(tmem + C_P, op_k_major(sm + QK, 128, 0), op_k_major(sm + QK, 128, 64), false);
             mma_tile<128, 64, 128>(tmem + C_WH, op_mn_major(sm + HH, 128), op_mn_major(sm + WT, 128), false);
-            mma_tile<64, 128, 128>(tmem + C_QH, op_k_major(sm + QK, 128, 0), op_mn_major(sm + HH, 128), false);
             mma_commit(&bar_mma);
+            mma_tile<64, 128, 128>(tmem + C_QH, op_k_major(sm + QT, 64), op_mn_major(sm + HH, 128), false);
         }
         GDN_WAIT_MMA(31)
-        if (ok && has_next) {   // Q and K have been read for the last time
-            if (threadIdx.x == 0) load_qk(xn, in_phase ^ 1);
-            if (!CW && threadIdx.x < kC) gnext = fetch_gamma(xn);
-        }
-        if (ok) {   // P = tril(Q K^T . D) over W^T (dead), U = U~ - W h in place
-            const int i0 = half * 32, j0 = half * 32;
-#pragma unroll 1
+        if (!CW && ok && has_next && threadIdx.x < kC) gnext = fetch_gamma(xn);
+        if (ok) {   // U = U~ - W h in place
+            const int i0 = half * 32;
+#pragma unroll 2
             for (int part = 0; part < 4; ++part) {
-                float v[8], u[8], t[8];
-                const int jb = j0 + part * 8, ib = i0 + part * 8;
-                if (!CW) tmem_ld8(tmem + lane_base + C_P + jb, v);
+                float u[8], t[8];
+                const int ib = i0 + part * 8;
                 tmem_ld8(tmem + lane_base + C_WH + ib, t);
                 chunk_load(sm + UTT, 128, f, ib >> 3, u);
                 tmem_wait_ld();
-                if (!CW && ga) {
-                    float g8[8];
-                    ld8s(gl + jb, g8);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) v[j] = (jb + j <= tr) ? v[j] * ex2(gl[tr] - g8[j]) : 0.f;
-                    chunk_store(sm + PT, 64, tr, jb >> 3, v);
-                }
 #pragma unroll
                 for (int i = 0; i < 8; ++i) u[i] -= t[i];
                 chunk_store(sm + UTT, 128, f, ib >> 3, u);
@@ -1640,15 +1622,15 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
         tc_fence_before();
         fence_async_smem();
         __syncthreads();
-        // ---- step 2: P U (token-major, over the columns of the first two accumulators)
+        // ---- step 2: P U (token-major)
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
-            if (CW) mma_tile<64, 128, 64>(tmem + C_QH, op_k_major(sm + PT_CW, 64), op_k_major(sm + UTT, 128), true);
+            if (CW) mma_tile<64, 128, 64>(tmem + C_QH, op_k_major(sm + PT, 64), op_k_major(sm + UTT, 128), true);
             else mma_tile<64, 128, 64>(tmem + C_PU, op_k_major(sm + PT, 64), op_k_major(sm + UTT, 128), false);
             mma_commit(&bar_mma);
         }
         GDN_WAIT_MMA(32)
-        if (ok && has_next && threadIdx.x == 0) load_wu(xn);   // P (over W^T) and U^T have been read for the last time
+        if (ok && has_next && threadIdx.x == 0) { load_q(xn, in_phase ^ 1); load_up(xn); }   // every tile has been read for the last time
         if (ok) {   // o = scale (Gam . (Q h) + P U): the sixteen low lanes of a warp own a token row and 64 columns each
             const float coef = CW ? sc : sc * Gam[tr];
 #pragma unroll 1
@@ -1761,12 +1743,7 @@ static int sm_count() {
     return cached[dev];
 }
 
-// The two small preparation kernels, two CTAs per SM.
-static cudaError_t launch_factors(const TcParams& P, cudaStream_t st) {
-    static SmemLimitOnce done;
-    const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count();
-    return launch_chunk_kernel(tc_factors_kernel, done, factors::SMEM_BYTES, ST_PREP, items < ctas ? items : ctas, split::kT, P, st);
-}
+// The small preparation kernels, two CTAs per SM.
 static cudaError_t launch_eprep(const TcParams& P, cudaStream_t st) {
     static SmemLimitOnce done;
     const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count();
@@ -1776,7 +1753,7 @@ static cudaError_t launch_eprep(const TcParams& P, cudaStream_t st) {
 static cudaError_t launch_prep_lr(const TcParams& P, cudaStream_t st) {
     static SmemLimitOnce done;
     const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count();
-    return launch_chunk_kernel(tc_prep_lr_kernel, done, both::SMEM_BYTES, ST_PREP, items < ctas ? items : ctas, split::kT, P, st);
+    return launch_chunk_kernel(tc_prep_lr_kernel, done, preplr::SMEM_BYTES, ST_PREP, items < ctas ? items : ctas, split::kT, P, st);
 }
 
 static cudaError_t launch_scan(const TcParams& P, cudaStream_t st) {
@@ -1849,15 +1826,15 @@ static cudaError_t launch_table_if_needed(const Problem& p, cudaStream_t st) {
     return (p.cu || p.Ttot == 0) ? launch_table(p, st) : cudaSuccess;
 }
 
-// Carries in low-rank form take the chunk factors from tc_factors; in operator form they also need Nm and Bf, which
-// only the fused tc_prep makes.
+// Carries in low-rank form take the chunk factors from tc_prep_lr; in operator form they also need Nm and Bf, which only
+// tc_prep makes.
 cudaError_t tc_launch_fwd(const Problem& p, cudaStream_t st) {
     TcParams P;
     cudaError_t e = launch_table_if_needed(p, st);
     if (e != cudaSuccess) return e;
     if (p.Ttot == 0) return empty_call(p, false, st);
     if (!fill_params(P, p, false, 0)) return cudaErrorUnknown;
-    if ((e = P.lowrank ? launch_factors(P, st) : launch_prep(P, st)) != cudaSuccess) return e;
+    if ((e = P.lowrank ? launch_prep_lr(P, st) : launch_prep(P, st)) != cudaSuccess) return e;
     if ((e = launch_scan(P, st)) != cudaSuccess) return e;
     return p.o ? launch_out(P, st) : cudaSuccess;
 }
@@ -1878,8 +1855,6 @@ cudaError_t tc_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st
         P.withhold = 1;
         if ((e = cudaMemcpyToSymbolAsync(g_wait_limit_ns, &ns, sizeof(ns), 0, cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
     }
-    // (the closed arm keeps fused kernels: they read k once and never move W through HBM on its way to E; measured on
-    // B = 4, T = 2048, H = 16: tc_prep_lr 77 us, tc_factors + tc_eprep 62 + 45 us)
     if ((e = skip_recompute ? launch_eprep(P, st) : P.lowrank ? launch_prep_lr(P, st) : launch_prep(P, st)) != cudaSuccess) return e;
     if ((e = launch_scan(P, st)) != cudaSuccess) return e;
     e = launch_intra(P, st);
