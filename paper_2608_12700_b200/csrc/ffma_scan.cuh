@@ -172,9 +172,8 @@ __device__ __forceinline__ void scan_chain(const Problem& p, int chain, int part
 
 // Block index -> (chain, direction, column slice).  dirs: 0 forward, 1 reverse, 2 both in one launch.
 template <int DK, int DV, bool VEC>
-__device__ __forceinline__ void scan_block(const Problem& p, int dirs, float* sm) {
+__device__ __forceinline__ void scan_block(const Problem& p, int dirs, float* sm, int b) {
     constexpr int PARTS = DV / kScanCols;
-    int b = blockIdx.x;
     const int part = b % PARTS;
     b /= PARTS;
     const bool reverse = dirs == 2 ? (b & 1) != 0 : dirs == 1;

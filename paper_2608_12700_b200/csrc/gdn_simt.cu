@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kThreads) scan_kernel(Problem p, int dirs) {
     wait_prerequisites();
     extern __shared__ __align__(16) float sm[];
     if (reinterpret_cast<const WsHeader*>(p.ws)->status != GDN_OK) return;
-    scan_block<DK, DV, false>(p, dirs, sm);
+    scan_block<DK, DV, false>(p, dirs, sm, (int)blockIdx.x);
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -38,6 +38,16 @@ __device__ __forceinline__ bool vec_go(const Problem& p) {
     return hdr->status == GDN_OK && (!p.fallback || hdr->cw_fallback);
 }
 
+// The (chunk, head) items of a block.
+template <class Body>
+__device__ __forceinline__ void for_chunks(const Problem& p, Body body) {
+    ChunkInfo x;
+    for (int item = blockIdx.x; chunk_info(p, x, item); item += gridDim.x) {
+        body(x);
+        __syncthreads();
+    }
+}
+
 // References of the four blocks and their exponentials: ref_0 = 0 (the chunk start), ref_I = gam of token 16 I - 1.
 template <int DK>
 struct Refs { float ref[kNB][DK], eref[kNB][DK]; };
@@ -89,11 +99,7 @@ struct PrepTiles {
 };
 
 template <typename IO, int DK, int DV>
-__global__ void __launch_bounds__(kThreads, 1) vprep_kernel(Problem p, int mode) {
-    wait_prerequisites();
-    if (!p.fallback) init_header_if_untabled(p);
-    ChunkInfo x;
-    if ((p.fallback && !vec_go(p)) || !chunk_info(p, x)) return;
+__device__ __forceinline__ void vprep_chunk(const Problem& p, int mode, const ChunkInfo& x) {
     using L = PrepTiles<DK, DV>;
     constexpr int PK = pitch(DK), PV = pitch(DV);
     extern __shared__ __align__(16) float sm[];
@@ -287,6 +293,14 @@ __global__ void __launch_bounds__(kThreads, 1) vprep_kernel(Problem p, int mode)
     }
 }
 
+template <typename IO, int DK, int DV>
+__global__ void __launch_bounds__(kThreads, 1) vprep_kernel(Problem p, int mode) {
+    wait_prerequisites();
+    if (!p.fallback) init_header_if_untabled(p);
+    else if (!vec_go(p)) return;
+    for_chunks(p, [&](const ChunkInfo& x) { vprep_chunk<IO, DK, DV>(p, mode, x); });
+}
+
 // ------------------------------------------------------------------------------------------------
 // vscan: forward and reverse carries (ffma_scan.cuh).
 // ------------------------------------------------------------------------------------------------
@@ -295,7 +309,11 @@ __global__ void __launch_bounds__(kThreads) vscan_kernel(Problem p, int dirs) {
     wait_prerequisites();
     extern __shared__ __align__(16) float sm[];
     if (!vec_go(p)) return;
-    scan_block<DK, DV, true>(p, dirs, sm);
+    const int blocks = p.d.N * p.d.H * (dirs == 2 ? 2 : 1) * (DV / kScanCols);
+    for (int b = blockIdx.x; b < blocks; b += gridDim.x) {
+        scan_block<DK, DV, true>(p, dirs, sm, b);
+        __syncthreads();
+    }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -305,10 +323,7 @@ template <int DK, int DV>
 constexpr size_t vout_smem() { return sizeof(float) * (kC * pitch(DK) + DK * pitch(DV) + kC * pitch(DV) + kC * kPc); }
 
 template <typename IO, int DK, int DV>
-__global__ void __launch_bounds__(kThreads, 1) vout_kernel(Problem p) {
-    wait_prerequisites();
-    ChunkInfo x;
-    if (!vec_go(p) || !chunk_info(p, x)) return;
+__device__ __forceinline__ void vout_chunk(const Problem& p, const ChunkInfo& x) {
     constexpr int PK = pitch(DK), PV = pitch(DV), R = Out<DV>::R;
     extern __shared__ __align__(16) float sm[];
     float* sQ = sm;
@@ -342,6 +357,13 @@ __global__ void __launch_bounds__(kThreads, 1) vout_kernel(Problem p) {
             for (int y = 0; y < 4; ++y) stf(op + o.row(r) * rv + o.c + 8 * y, sc * acc[r][y]);
 }
 
+template <typename IO, int DK, int DV>
+__global__ void __launch_bounds__(kThreads, 1) vout_kernel(Problem p) {
+    wait_prerequisites();
+    if (!vec_go(p)) return;
+    for_chunks(p, [&](const ChunkInfo& x) { vout_chunk<IO, DK, DV>(p, x); });
+}
+
 // ------------------------------------------------------------------------------------------------
 // vintra: token gradients of one (chunk, head).  K#2 in its short form: dXv = T^T dU, dXk = -dXv h^T, dA = -stril(dXv U^T).
 //     dq_i = scale Gam_i (dO h^T)_i + sum_{j <= i} dP_ij e^{gam_i - gam_j} k_j
@@ -373,10 +395,7 @@ struct IntraTiles {
 };
 
 template <typename IO, int DK, int DV>
-__global__ void __launch_bounds__(kThreads, 1) vintra_kernel(Problem p) {
-    wait_prerequisites();
-    ChunkInfo x;
-    if (!vec_go(p) || !chunk_info(p, x)) return;
+__device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& x) {
     using L = IntraTiles<DK, DV>;
     constexpr int PK = pitch(DK), PV = pitch(DV), NH = DK / 64;
     extern __shared__ __align__(16) float sm[];
@@ -605,13 +624,24 @@ __global__ void __launch_bounds__(kThreads, 1) vintra_kernel(Problem p) {
     }
 }
 
+template <typename IO, int DK, int DV>
+__global__ void __launch_bounds__(kThreads, 1) vintra_kernel(Problem p) {
+    wait_prerequisites();
+    if (!vec_go(p)) return;
+    for_chunks(p, [&](const ChunkInfo& x) { vintra_chunk<IO, DK, DV>(p, x); });
+}
+
+// Blocks of a launch over `items`: one each, or, for the fall-back sequence, one per SM (it rarely has work, and a grid of
+// thousands of blocks that return at once takes microseconds: three launches behind a call of 2112 chunk-heads, see launch).
+int grid_of(const Problem& p, int items) { return p.fallback && items > tc_sm_count() ? tc_sm_count() : items; }
+
 template <int DK, int DV>
 cudaError_t launch_vscan(const Problem& p, int dirs, cudaStream_t st) {
     static SmemLimitOnce once;
     const cudaError_t e = once.ensure(vscan_kernel<DK, DV>, (uint32_t)scan_smem<DK>());
     if (e != cudaSuccess) return e;
     const int ctas = p.d.N * p.d.H * (dirs == 2 ? 2 : 1) * (DV / kScanCols);
-    { StageScope t(p.fallback ? ST_FALLBACK : dirs == 2 ? ST_SCANS : dirs == 1 ? ST_RSCAN : ST_FSCAN, st); launch_kernel(vscan_kernel<DK, DV>, ctas, kThreads, scan_smem<DK>(), st, p, dirs); }
+    { StageScope t(p.fallback ? ST_FALLBACK : dirs == 2 ? ST_SCANS : dirs == 1 ? ST_RSCAN : ST_FSCAN, st); launch_kernel(vscan_kernel<DK, DV>, grid_of(p, ctas), kThreads, scan_smem<DK>(), st, p, dirs); }
     return cudaGetLastError();
 }
 template <typename IO, int DK, int DV>
@@ -620,7 +650,7 @@ cudaError_t launch_vprep(const Problem& p, PrepMode mode, cudaStream_t st) {
     constexpr size_t sm = PrepTiles<DK, DV>::BYTES;
     const cudaError_t e = once.ensure(vprep_kernel<IO, DK, DV>, (uint32_t)sm);
     if (e != cudaSuccess) return e;
-    { StageScope t(p.fallback ? ST_FALLBACK : mode == PREP_BWD ? ST_EPREP : ST_PREP, st); launch_kernel(vprep_kernel<IO, DK, DV>, p.L.max_chunks * p.d.H, kThreads, sm, st, p, mode); }
+    { StageScope t(p.fallback ? ST_FALLBACK : mode == PREP_BWD ? ST_EPREP : ST_PREP, st); launch_kernel(vprep_kernel<IO, DK, DV>, grid_of(p, p.L.max_chunks * p.d.H), kThreads, sm, st, p, mode); }
     return cudaGetLastError();
 }
 
@@ -634,7 +664,7 @@ cudaError_t ffma_fwd(const Problem& q, cudaStream_t st) {
     if ((e = launch_vscan<DK, DV>(q, 0, st)) != cudaSuccess || !q.o) return e;
     static SmemLimitOnce once;
     if ((e = once.ensure(vout_kernel<IO, DK, DV>, (uint32_t)vout_smem<DK, DV>())) != cudaSuccess) return e;
-    { StageScope t(q.fallback ? ST_FALLBACK : ST_OUT, st); launch_kernel(vout_kernel<IO, DK, DV>, q.L.max_chunks * q.d.H, kThreads, vout_smem<DK, DV>(), st, q); }
+    { StageScope t(q.fallback ? ST_FALLBACK : ST_OUT, st); launch_kernel(vout_kernel<IO, DK, DV>, grid_of(q, q.L.max_chunks * q.d.H), kThreads, vout_smem<DK, DV>(), st, q); }
     return cudaGetLastError();
 }
 
@@ -647,7 +677,7 @@ cudaError_t ffma_bwd(const Problem& q, bool skip_recompute, cudaStream_t st) {
     static SmemLimitOnce once;
     constexpr size_t sm = IntraTiles<DK, DV>::BYTES;
     if ((e = once.ensure(vintra_kernel<IO, DK, DV>, (uint32_t)sm)) != cudaSuccess) return e;
-    { StageScope t(q.fallback ? ST_FALLBACK : ST_INTRA, st); launch_kernel(vintra_kernel<IO, DK, DV>, q.L.max_chunks * q.d.H, kThreads, sm, st, q); }
+    { StageScope t(q.fallback ? ST_FALLBACK : ST_INTRA, st); launch_kernel(vintra_kernel<IO, DK, DV>, grid_of(q, q.L.max_chunks * q.d.H), kThreads, sm, st, q); }
     return cudaGetLastError();
 }
 
