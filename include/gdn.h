@@ -58,9 +58,9 @@ typedef enum gdn_status {
     GDN_ERR_WORKSPACE_TOO_SMALL = 6,
     GDN_ERR_CUDA = 7,               /* a CUDA runtime call or launch failed                            */
     GDN_ERR_DEVICE_TIMEOUT = 8,     /* device-side: a bounded wait gave up                             */
-    GDN_ERR_DECAY_RANGE = 9         /* device-side and transient: the tensor-core kernels of a channel-wise call  */
-                                    /* stood down (cumulative log decay of a chunk outside [-80, 80]); the same   */
-                                    /* call then runs on the FFMA kernels and clears it.  Never left behind.      */
+    GDN_ERR_DECAY_RANGE = 9         /* names the case in which the tensor-core kernels of a channel-wise call     */
+                                    /* stand down (cumulative log decay of a chunk outside [-80, 80]); the same   */
+                                    /* call then runs on the FFMA kernels.  Never returned nor left behind.       */
 } gdn_status;
 
 typedef enum gdn_dtype { GDN_F32 = 0, GDN_BF16 = 1 } gdn_dtype;
@@ -156,7 +156,7 @@ const char* gdn_status_string(gdn_status s);
 
 /* Name of the kernel family a descriptor dispatches to ("simt_f32", "simt_bf16", "tcgen05_bf16",
  * "tcgen05_bf16_scalar_gate", "tcgen05_bf16_padded": bf16 shapes with one or both head dimensions at 64 that have no
- * kernels of their own, zero-padded onto the d = 128 tensor-core kernels inside the workspace),
+ * kernels of their own; the d = 128 tensor-core kernels read the missing features as zeros),
  * or NULL for an unsupported descriptor.  Diagnostic only (the paper has no counterpart). */
 const char* gdn_kernel_path(const gdn_desc* desc);
 /* The same for the channel-wise calls: "tcgen05_bf16_channelwise" (bf16, d_k = d_v = 128),

@@ -12,17 +12,17 @@
 //     U = U~ - W h   dU = P^T dO' + K- dh''   (dh'' = Diag(Gam_e) dh')
 //     dP = tril(dO' U^T)   dW = -dU h^T   dXk = T^T dW   dXv = T^T dU   dA = -stril(dXk W^T + dXv U~^T)
 //     dQ~ = dO' h^T + dP K-     dK+ = dXk + dA K-     dK- = U dh''^T + dP^T Q~ + dA^T K+
-// and the gradients of the caller's tensors follow element by element.  Three kernels beside the carries
+// and the gradients of the caller's tensors follow element by element.  Beside the carries
 // (tc_scan_cw in gdn_tc.cu):
 //   cw_scale  scaled operand tiles as bf16 tile images, gam; checks that |gam| stays below 80 (beyond that the split
-//             would need reference points inside the chunk): otherwise it records GDN_ERR_DECAY_RANGE, the kernels below
+//             would need reference points inside the chunk): otherwise it sets the fall-back word of the workspace header, the kernels below
 //             stand down, and the FFMA sequence enqueued behind them computes the call (gdn_simt_vec.cu)
 //   cw_prep   [Q~;K+] K-^T, fp32 blocked inversion, W^T, U~^T, (P^T dO')^T, E               (tcgen05)
 //   cw_intra  the thirteen products of the gradient stage in four dependent steps (K#2 reuses T), and from them dq, dk, dv,
 //             db, dw, and dg by a reverse cumulative sum per channel                                  (tcgen05)
-// The tensor-core kernels are written straight-line (one CTA per SM walks over chunk-heads; one thread issues every
-// product and copy; CTA-wide barriers between the steps): the plain statement of the channel-wise path on tcgen05,
-// not a tuned one.  Accumulators live in one TMEM reservation at fixed column offsets; every wait is bounded.
+// The tensor-core kernels are written straight-line (a CTA walks over chunk-heads; one thread issues every product and
+// copy; CTA-wide barriers between the steps).  Accumulators live in one TMEM reservation at fixed column offsets; every wait
+// is bounded.
 #include "tc_common.cuh"
 #include "tc_inverse.cuh"
 
