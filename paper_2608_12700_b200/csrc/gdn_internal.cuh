@@ -32,7 +32,8 @@ struct WsLayout {
     size_t chunk_seq;      // int32 [max_chunks]
     size_t chunk_tok0;     // int32 [max_chunks]   global token index of the chunk's first row
     size_t chunk_len;      // int32 [max_chunks]   valid rows (1..64)
-    size_t gamma;          // f32 [CH, 64]         chunk-local cumulative log decay
+    size_t gamma;          // f32 [CH, 64]         chunk-local cumulative log decay (channel-wise calls: [CH, 64, d_k])
+    size_t ref;            // int32 [CH, d_k]      channel-wise path on the tensor cores: the reference of a chunk's decays is 2^ref
     size_t Tm;             // f32|bf16 [CH, 64, 64]    T = (I + A)^-1
     size_t W;              // [CH, 64, d_k]
     size_t Ut;             // [CH, 64, d_v]            U~ = T Diag(w) V
@@ -135,6 +136,7 @@ inline WsLayout make_layout_vec(const gdn_desc& d) {
     L.Ut = take(4 * CH * kC * d.d_v);
     L.Pm = take(4 * CH * kC * kC);
     L.Nm = L.Bf = o;
+    L.ref = take(L.tc_scans ? 4 * CH * d.d_k : 0);
     L.img_W = take(L.tc_scans ? CH * 16384 : 0);
     L.img_U = take(L.tc_scans ? CH * 16384 : 0);
     L.img_QKp = take(L.tc_scans ? CH * 32768 : 0);

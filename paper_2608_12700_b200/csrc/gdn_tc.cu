@@ -685,9 +685,11 @@ template <int S> struct Cfg {
 
 // One direction of one chain (the direction is a compile-time constant: the two differ in operands and readouts).
 // CW = carries of the channel-wise path (per-channel gates): the decay of the state is a vector (one factor per state
-// row, i.e. per thread), and the key tile arrives as K- = k / Gam, a tile image from the
+// row, i.e. per thread), and the key tile arrives as K- = S k / Gam, a tile image from the
 // workspace together with images of W^T, U~^T and E (written by the channel-wise preparation kernels), so the readout of the
-// first product applies no per-token factor.
+// first product applies no per-token factor.  Those images are relative to a reference S = 2^ref of the chunk (gdn_tc_cw.cu), and
+// so is the state that enters a chunk's products: S h forward, (Gam_e / S) dh' in reverse.  The increment that the second
+// product leaves is scaled by the other of the two factors.
 template <bool reverse, bool CW, int S>
 __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int part, float* ge, float (*ee2)[kC], uint64_t* bar_full,
                                               uint64_t& bar_mma, uint32_t& tmem_slot) {
@@ -739,7 +741,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         mbar_expect_tx(&bar_full[stage], 32768 + x_bytes);
         bulk_load(slot + WT, w_base + ch * 16384, 16384, &bar_full[stage]);
         if constexpr (CW) {
-            // k- itself, in both directions: the decay to the chunk end is applied to the state (row by row, below)
+            // k-, in both directions: what is left of the decay is applied to the state (row by row, below)
             bulk_load(slot + KT, p.ws + p.L.img_Km + ch * 16384, 16384, &bar_full[stage]);
         } else {
             tma_load_3d(slot + KT, &P.tm_k, 0, hd, sg.chunk_tok0(c), &bar_full[stage]);
@@ -774,7 +776,15 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     __syncthreads();
     bool ok = true;
     uint32_t mma_phase = 0;
-    float cw_gam = (CW && nsteps > 0) ? gamma[(((size_t)chunk_of(0) * H + hd) * kC + kC - 1) * D + r] : 0.f;
+    // channel-wise: log decay over the chunk and reference of this thread's state row, fetched a step ahead
+    float cw_gam = 0.f;
+    int cw_ref = 0;
+    auto cw_fetch = [&](int s) {
+        const size_t ch = (size_t)chunk_of(s) * H + hd;
+        cw_gam = gamma[(ch * kC + kC - 1) * D + r];
+        cw_ref = reinterpret_cast<const int32_t*>(p.ws + p.L.ref)[ch * D + r];
+    };
+    if (CW && nsteps > 0) cw_fetch(0);
 #pragma unroll 1
     for (int s = 0; s < nsteps; ++s) {
         unsigned char* Ht = sm + HT + (s & 1) * HT_BYTES;
@@ -782,18 +792,19 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         const size_t ch = (size_t)c * H + hd;
         unsigned char* ring = sm + stage * STAGE_BYTES;
         const float* ee = ee2[s & 1];
-        // decay of the state over the chunk: a scalar, or (channel-wise) the factor of this thread's state row, whose log
-        // was fetched during the step before (the reverse chain needs it at the top of the step)
+        // decay of the state over the chunk: a scalar, or (channel-wise) the factor of this thread's state row; channel-wise also
+        // the factors of the state on its way into the products and of the increment
         const float Ge = CW ? expf(cw_gam) : (s < GE_CAP ? ge[s] : expf(gamma[ch * kC + kC - 1]));
-        if (CW && s + 1 < nsteps) cw_gam = gamma[(((size_t)chunk_of(s + 1) * H + hd) * kC + kC - 1) * D + r];
-        // state -> bf16: operand of the first product, and the per-chunk state the gradient stage reads.  Channel-wise,
-        // reverse: stored as dh'' = Diag(Gam_e) dh', the form the gradient stage works with ((Kb dh') = k- dh'').
+        const float S_ref = pow2(cw_ref), G_end = Ge * pow2(-cw_ref);   // (channel-wise only)
+        const float Gin = reverse ? G_end : S_ref, Gout = reverse ? S_ref : G_end;
+        if (CW && s + 1 < nsteps) cw_fetch(s + 1);
+        // state -> bf16: operand of the first product, and the per-chunk state the gradient stage reads
 #pragma unroll
         for (int k = 0; k < NSH / 8; ++k) {
-            if constexpr (CW && reverse) {
+            if constexpr (CW) {
                 float sc8[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) sc8[j] = Ge * st[8 * k + j];
+                for (int j = 0; j < 8; ++j) sc8[j] = Gin * st[8 * k + j];
                 *reinterpret_cast<uint4*>(Ht + tile_chunk_off(128, r, (lc0 >> 3) + k)) = pack8(sc8);
             } else {
                 *reinterpret_cast<uint4*>(Ht + tile_chunk_off(128, r, (lc0 >> 3) + k)) = pack8(st + 8 * k);
@@ -869,8 +880,8 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
             tmem_wait_ld();
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                if (CW && !reverse) st[8 * k + j] = Ge * (st[8 * k + j] + d2[j]);   // Gam_e h + (Gam_e . K-)^T U
-                else st[8 * k + j] = fmaf(Ge, st[8 * k + j], reverse ? ad[j] + d2[j] : d2[j]);
+                const float inc = reverse ? ad[j] + d2[j] : d2[j];
+                st[8 * k + j] = fmaf(Ge, st[8 * k + j], CW ? Gout * inc : inc);
             }
         }
         tc_fence_before();
@@ -1508,9 +1519,9 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
 // steps of one chunk-head while its neighbour is in another step of another one.  The tiles of the next trip are
 // loaded as soon as the last product (or store) that reads their region is done.  Q h and P U are formed token-major
 // (M = 64: a thread owns a token row), so the output tile is staged with 16-byte stores and leaves by TMA.
-// CW: the channel-wise path.  Its preparation kernels leave Q~ = Gam.q, P = tril(Q~ K-^T), W^T, U~^T and the per-chunk
-// states in the workspace as tile images, the decay is inside Q~ and P, so o = scale (Q~ h + P (U~ - W h)): no
-// gates here, and P U accumulates onto Q~ h.
+// CW: the channel-wise path.  Its preparation kernels leave Q~, P = tril(Q~ K-^T), W^T, U~^T and the per-chunk
+// states h~ in the workspace as tile images, the decay is inside them, so o = scale (Q~ h~ + P (U~ - W h~)): no
+// gates here, and P U accumulates onto Q~ h~.
 // ------------------------------------------------------------------------------------------------
 namespace outk {
 constexpr uint32_t QT = 0;                  // Q or Q~ [64][128]                                     16 KB

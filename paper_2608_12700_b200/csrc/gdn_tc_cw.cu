@@ -2,19 +2,24 @@
 // d_k = d_v = 128.
 //
 // "The channel-wise path folds the per-channel decay Diag(e^{g_t}) inside those contractions" (Appendix A): with the
-// chunk-local cumulative log decay gam_i in R^{d_k} (reference: the chunk start, so gam <= 0 for a decaying gate) every
-// factor exp(gam_i - gam_j) of a token pair splits into a row part and a column part, and the keys and queries are
-// scaled once, element by element, before any product:
-//     q~_i = Gam_i . q_i      k+_i = Gam_i . b_i . k_i   (row role)      k-_j = k_j / Gam_j   (column role)
+// chunk-local cumulative log decay gam_i in R^{d_k}, Gam_i = exp(gam_i), and a reference S in R^{d_k} of the chunk, every factor
+// exp(gam_i - gam_j) of a token pair splits into a row part and a column part, and the keys and queries are scaled once, element by
+// element, before any product.  With G_i = Gam_i / S:
+//     q~_i = G_i . q_i        k+_i = G_i . b_i . k_i   (row role)        k-_j = k_j / G_j   (column role)
 //     v~_i = w_i . v_i                                                    dO'  = scale dO (the factor is applied to fp32 accumulators)
-// In these variables the chunk is a decay-free delta rule whose token-token matrices carry plain triangular masks:
+// In these variables, and with the states h~ = Diag(S) h and dh'' = Diag(G_e) dh' (e: the chunk's end), the chunk is a decay-free
+// delta rule whose token-token matrices carry plain triangular masks:
 //     A = stril(K+ K-^T)   P = tril(Q~ K-^T)   T = (I + A)^-1   W = T K+   U~ = T V~   E = (Q~ - P W)^T dO'
-//     U = U~ - W h   dU = P^T dO' + K- dh''   (dh'' = Diag(Gam_e) dh')
-//     dP = tril(dO' U^T)   dW = -dU h^T   dXk = T^T dW   dXv = T^T dU   dA = -stril(dXk W^T + dXv U~^T)
-//     dQ~ = dO' h^T + dP K-     dK+ = dXk + dA K-     dK- = U dh''^T + dP^T Q~ + dA^T K+
-// and the gradients of the caller's tensors follow element by element.  Beside the carries
-// (tc_scan_cw in gdn_tc.cu):
-//   cw_scale  scaled operand tiles as bf16 tile images, gam; checks that |gam| stays below 80 (beyond that the split
+//     U = U~ - W h~   dU = P^T dO' + K- dh''
+//     dP = tril(dO' U^T)   dW = -dU h~^T   dXk = T^T dW   dXv = T^T dU   dA = -stril(dXk W^T + dXv U~^T)
+//     dQ~ = dO' h~^T + dP K-    dK+ = dXk + dA K-     dK- = U dh''^T + dP^T Q~ + dA^T K+
+//     h' = Gam_e . h + G_e . (K-^T U)        dh = Gam_e . dh' + S . (E - W^T (K- dh''))                (the carries)
+// and the gradients of the caller's tensors follow element by element.  S = 2^ref, per channel, lies in the middle of the range
+// that gam and the chunk start (gam = 0) span: a chunk that decays by e^-80 then scales its operands and states by factors
+// between e^-40 and e^40.  With S = 1, K- reached e^80 and dh'' e^-80 of the values: an increment K-^T U beyond fp32 for values
+// of 1e5, a subnormal dh'' for gradients of 1e-6.  A power of two, because every operand is then the same number
+// with another exponent, and no rounding depends on S.  Beside the carries (tc_scan_cw in gdn_tc.cu):
+//   cw_scale  scaled operand tiles as bf16 tile images, gam, ref; checks that |gam| stays below 80 (beyond that the split
 //             would need reference points inside the chunk): otherwise it sets the fall-back word of the workspace header, the kernels below
 //             stand down, and the FFMA sequence enqueued behind them computes the call (gdn_simt_vec.cu)
 //   cw_prep   [Q~;K+] K-^T, fp32 blocked inversion, W^T, U~^T, (P^T dO')^T, E               (tcgen05)
@@ -33,7 +38,7 @@ using namespace tc;
 
 constexpr int D = 128;
 constexpr int kT = 256;               // 8 warps: TMEM lane quadrant = warp % 4, column half = warp / 4
-constexpr float kMaxDecay = 80.f;     // bound on |gam| inside a chunk (exp(80) is still a bf16 number)
+constexpr float kMaxDecay = 80.f;     // bound on |gam| inside a chunk (|log G| is no larger: exp(80) is still a bf16 number)
 
 // (chunk, head) of an elementwise CTA, from the chunk table (which these calls always build)
 struct ChunkCtx { int hd, ch, tok0, len; };
@@ -57,6 +62,7 @@ __global__ void __launch_bounds__(kT) cw_scale_kernel(Problem p) {
     if (!chunk_ctx(p, x)) return;
     extern __shared__ __align__(16) float gam[];   // [64][D + 1]
     __shared__ int bad;
+    __shared__ int ref[D];
     const int H = p.d.H;
     const size_t base = ((size_t)x.tok0 * H + x.hd) * D, rs = (size_t)H * D;
     const __nv_bfloat16* qp = reinterpret_cast<const __nv_bfloat16*>(p.q) + base;
@@ -66,7 +72,7 @@ __global__ void __launch_bounds__(kT) cw_scale_kernel(Problem p) {
     __syncthreads();
     if (threadIdx.x < D) {
         const int r = threadIdx.x;
-        float s = 0.f, worst = 0.f;
+        float s = 0.f, lo = 0.f, hi = 0.f;   // (the chunk start counts: the states enter there)
 #pragma unroll 1
         for (int i0 = 0; i0 < kC; i0 += 16) {   // sixteen loads in flight, then their running sum in token order
             float g16[16];
@@ -76,10 +82,12 @@ __global__ void __launch_bounds__(kT) cw_scale_kernel(Problem p) {
             for (int k = 0; k < 16; ++k) {
                 s += g16[k];
                 gam[(i0 + k) * (D + 1) + r] = s;
-                worst = fmaxf(worst, fabsf(s));
+                lo = fminf(lo, s);
+                hi = fmaxf(hi, s);
             }
         }
-        if (!(worst <= kMaxDecay)) bad = 1;   // (also catches a NaN gate: it cannot be scaled apart either)
+        if (lo < -kMaxDecay || hi > kMaxDecay) bad = 1;   // (a NaN gate passes and comes out as NaN)
+        ref[r] = __float2int_rn(0.5f * kLog2e * (lo + hi));
     }
     __syncthreads();
     if (bad) {
@@ -91,6 +99,7 @@ __global__ void __launch_bounds__(kT) cw_scale_kernel(Problem p) {
     }
     float* wsG = reinterpret_cast<float*>(p.ws + p.L.gamma) + (size_t)x.ch * kC * D;
     for (int t = threadIdx.x; t < kC * D; t += kT) wsG[t] = gam[(t / D) * (D + 1) + t % D];
+    if (threadIdx.x < D) reinterpret_cast<int32_t*>(p.ws + p.L.ref)[(size_t)x.ch * D + threadIdx.x] = ref[threadIdx.x];
     char* iQKp = p.ws + p.L.img_QKp + (size_t)x.ch * 32768;
     char* iKm = p.ws + p.L.img_Km + (size_t)x.ch * 16384;
     char* iVt = p.ws + p.L.img_Vt + (size_t)x.ch * 16384;
@@ -114,11 +123,11 @@ __global__ void __launch_bounds__(kT) cw_scale_kernel(Problem p) {
         for (int j = 0; j < 8; ++j) {
             const int r = ch * 8 + j;
             const float g = gam[i * (D + 1) + r];
-            const float G = expf(g);
+            const float G = expf(g) * pow2(-ref[r]);
             const float bb = b8[j], ww = w8[j];
             a[j] = G * q8[j];                 // q~
             b[j] = G * bb * k8[j];            // k+
-            c[j] = expf(-g) * k8[j];          // k-
+            c[j] = expf(-g) * pow2(ref[r]) * k8[j];   // k-
             v8[j] *= ww;                      // v~
         }
         *reinterpret_cast<uint4*>(iQKp + tile_chunk_off(128, i, ch)) = pack8(a);
@@ -490,6 +499,7 @@ __global__ void __launch_bounds__(kT, 2) cw_eprep_kernel(const __grid_constant__
 // cw_intra: every gradient of one (chunk, head).
 //
 // Four dependent steps (products; [readout] what the threads make of them):
+// (h and Gam stand for h~ and G of the head of this file.)
 //   1  (W h)^T ; (K- dh'')^T ; (P^T dO)^T             [U = U~ - W h ; dU = scale P^T dO + K- dh'']
 //   2  dP = dO U^T ; dXv^T = dU^T T ; under the readout h dO^T ; dK-^T = dh'' U^T        [scale tril ; dv, dw]
 //   3  dA = dXv U^T (K#2) ; under the readout dK+^T = -h dXv^T ; K-^T dP^T ; Q~^T dP               [-stril]
@@ -510,8 +520,8 @@ constexpr uint32_t WT = DOT + 16384;        // W^T  [128][64]                   
 constexpr uint32_t UTT = WT + 16384;        // U~^T [128][64]                                   16 KB
 constexpr uint32_t TT = UTT + 16384;        // T [64][64]; later dA                              8 KB
 constexpr uint32_t PT = TT + 8192;          // P [64][64]; later dP                              8 KB
-constexpr uint32_t HH = PT + 8192;          // h [128][128]                                     32 KB
-constexpr uint32_t DH = HH + 32768;         // dh'' = Diag(Gam_e) dh' [128][128]                32 KB
+constexpr uint32_t HH = PT + 8192;          // h~ [128][128]                                    32 KB
+constexpr uint32_t DH = HH + 32768;         // dh'' [128][128]                                  32 KB
 constexpr uint32_t UT = DH + 32768;         // U^T  [128][64]                                   16 KB
 constexpr uint32_t DUT = UT + 16384;        // dU^T [128][64]; later dXv^T [128][64]            16 KB
 constexpr uint32_t SMEM_BYTES = DUT + 16384 + 1024;
@@ -611,7 +621,7 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(const __
         const size_t rs = (size_t)H * D, base = ((size_t)x.tok0 * H + x.hd) * D + (size_t)i0 * rs + f;   // this thread's channel of its first token
         const int live = x.len - i0;          // tokens of this thread inside the sequence (may be negative)
         const bool whole = live >= kTok;      // (two copies of the accesses: a condition at each of them costs more than it skips)
-        if (ok) {   // everything step 1 reads (the reverse carry left dh'' = Diag(Gam_e) dh', the form used here)
+        if (ok) {   // everything step 1 reads (the carries left h~ and dh'', the forms used here)
             ok = mbar_wait(&bar_s, in_phase) && mbar_wait(&bar_k, in_phase) && mbar_wait(&bar_b, in_phase) && mbar_wait(&bar_a, in_phase);
             if (!ok && threadIdx.x == 0) report_timeout(p.ws, 44);
             if (ok) pend_s = pend_k = pend_a = pend_b = false;
@@ -757,6 +767,7 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(const __
         const uint16_t* qp = reinterpret_cast<const uint16_t*>(p.q) + base;
         const uint16_t* kp = reinterpret_cast<const uint16_t*>(p.k) + base;
         const float* bp = p.bv + base;
+        const int ref = reinterpret_cast<const int32_t*>(p.ws + p.L.ref)[ch * D + f];
         float g8[8], b8[8];
         uint32_t q8[8], k8[8];
         auto fetch = [&](int i1) {   // eight tokens' gates and inputs of this channel
@@ -778,6 +789,7 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(const __
             }
         };
         fetch(0);   // while the products run
+        const float S = pow2(ref), iS = pow2(-ref);
         GDN_WAIT_MMA(49)
         if (warp == 1 && elect_one() && ok && has_next) { load_k(chn); load_s2(chn); load_a2(chn); }   // every tile has been read for the last time
         float dgm[kTok];
@@ -797,7 +809,7 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(const __
                 float dk[8], db[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const float G = expf(g8[j]), iG = expf(-g8[j]);
+                    const float G = expf(g8[j]) * iS, iG = expf(-g8[j]) * S;
                     const float q = __uint_as_float(q8[j] << 16), k = __uint_as_float(k8[j] << 16);
                     dq[j] = G * fmaf(sc, dq[j], dq2[j]);             // dq = Gam . dQ~
                     const float row = G * kr[j];                     // what multiplies b . k in the row role

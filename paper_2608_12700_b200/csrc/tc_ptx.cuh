@@ -273,6 +273,8 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 }
 
 // ---------------------------------------------------------------- small conversions
+// 2^e, exactly, for -126 <= e <= 127
+__device__ __forceinline__ float pow2(int e) { return __int_as_float((127 + e) << 23); }
 // 2^x, hardware approximation (about 2 ulp); callers pass non-positive arguments only.
 __device__ __forceinline__ float ex2(float x) {
     float y;

@@ -112,3 +112,32 @@ def test_channelwise_gates_at_zero_and_one_and_zero_keys(family):
     wl.k[64:128] = 0.0
     wl.k[::7] = 0.0
     cw_check(wl)
+
+
+@pytest.mark.parametrize("family", CW_FAMILIES)
+@pytest.mark.parametrize("decay", ["steady", "one_token"])
+@pytest.mark.parametrize("values,grads", [(2.0 ** 17, 1.0), (1.0, 2.0 ** -20), (2.0 ** -20, 2.0 ** -20)])
+def test_channelwise_decay_at_the_edge_of_the_range(family, decay, values, grads):
+    """Half of the key channels lose a factor e^-79 in every whole chunk, just inside what the tensor-core route accepts, evenly or
+    at one token, with values and states around 1e5 or 1e-6 and incoming gradients around 1e-6 (a mean loss): the results scale
+    with them, so neither an overflow nor an underflow of a scaled operand may show.  Outputs, closed and fresh gradients."""
+    wl = cw_workload(family, "cw_edge")
+    wl.gv[:, :, 1::2] = -79.0 / 64 if decay == "steady" else 0.0
+    if decay == "one_token":
+        for n in range(wl.N):
+            wl.gv[wl.cu_seqlens[n] + 20:wl.cu_seqlens[n + 1]:64, :, 1::2] = -79.0
+    wl.v *= values
+    wl.h0 *= values
+    wl.dO *= grads
+    wl.dhT *= grads
+    cw_check(wl)
+    ref = oracle.vec_bwd_workload(wl)
+    buf = runner.to_device_channelwise(wl, want_o=True)
+    runner.run_fwd_channelwise(buf)
+    got = runner.fetch(buf)
+    for n in ("o", "hT"):
+        assert rel(got[n], ref[n]) <= TOL[wl.dtype], (n, rel(got[n], ref[n]))
+    runner.run_bwd_channelwise(buf, fresh=1)
+    got = runner.fetch(buf)
+    for n in ("dq", "dk", "dv", "dg", "db", "dw", "dh0"):
+        assert rel(got[n], ref[n]) <= TOL[wl.dtype], (n, rel(got[n], ref[n]))
