@@ -17,9 +17,10 @@ __global__ void widen_rows_kernel(const uint4* src, uint4* dst, size_t rows) {
         dst[t] = c < 8 ? src[r * 8 + c] : make_uint4(0, 0, 0, 0);
     }
 }
-// rows of 128 bf16 -> their first 64
-__global__ void narrow_rows_kernel(const uint4* src, uint4* dst, size_t rows) {
+// rows of 128 bf16 -> their first 64 (results: like every other output, not after an error)
+__global__ void narrow_rows_kernel(const WsHeader* hdr, const uint4* src, uint4* dst, size_t rows) {
     wait_prerequisites();
+    if (hdr->status != GDN_OK) return;
     for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < rows * 8; t += (size_t)gridDim.x * blockDim.x)
         dst[t] = src[(t >> 3) * 16 + (t & 7)];
 }
@@ -32,8 +33,9 @@ __global__ void widen_state_kernel(const float* src, float* dst, size_t n, int d
         dst[t] = (r < dk && c < dv) ? src[(s * dk + r) * dv + c] : 0.f;
     }
 }
-__global__ void narrow_state_kernel(const float* src, float* dst, size_t n, int dk, int dv) {
+__global__ void narrow_state_kernel(const WsHeader* hdr, const float* src, float* dst, size_t n, int dk, int dv) {
     wait_prerequisites();
+    if (hdr->status != GDN_OK) return;
     for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * dk * dv; t += (size_t)gridDim.x * blockDim.x) {
         const size_t s = t / ((size_t)dk * dv);
         const int r = (int)((t / dv) % dk), c = (int)(t % dv);
@@ -50,8 +52,9 @@ __global__ void widen_rows_f32_kernel(const float4* src, float4* dst, size_t row
         dst[t] = c < 16 ? src[r * 16 + c] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
-__global__ void narrow_rows_f32_kernel(const float4* src, float4* dst, size_t rows) {
+__global__ void narrow_rows_f32_kernel(const WsHeader* hdr, const float4* src, float4* dst, size_t rows) {
     wait_prerequisites();
+    if (hdr->status != GDN_OK) return;
     for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < rows * 16; t += (size_t)gridDim.x * blockDim.x)
         dst[t] = src[(t >> 4) * 32 + (t & 15)];
 }
@@ -152,20 +155,21 @@ cudaError_t tc_padded_launch(const Problem& p, const WsLayout& inner, bool bwd, 
     }
     const cudaError_t e = bwd ? vec_launch_bwd(w, skip_recompute, st) : vec_launch_fwd(w, st);
     if (e != cudaSuccess) return e;
+    const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
     auto narrow = [&](const void* src, void* dst) {
         if (!dst || rows == 0) return;
         StageScope t(ST_TABLE, st);
-        launch_kernel(narrow_rows_kernel, grid_for(rows * 8), 256, 0, st, static_cast<const uint4*>(src), static_cast<uint4*>(dst), rows);
+        launch_kernel(narrow_rows_kernel, grid_for(rows * 8), 256, 0, st, hdr, static_cast<const uint4*>(src), static_cast<uint4*>(dst), rows);
     };
     auto narrow_state = [&](const float* src, float* dst) {
         if (!dst) return;
         StageScope t(ST_TABLE, st);
-        launch_kernel(narrow_state_kernel, grid_for(chains * d.d_k * d.d_v), 256, 0, st, src, dst, chains, d.d_k, d.d_v);
+        launch_kernel(narrow_state_kernel, grid_for(chains * d.d_k * d.d_v), 256, 0, st, hdr, src, dst, chains, d.d_k, d.d_v);
     };
     auto narrow_gate = [&](const float* src, float* dst) {
         if (!dst || rows == 0) return;
         StageScope t(ST_TABLE, st);
-        launch_kernel(narrow_rows_f32_kernel, grid_for(rows * 16), 256, 0, st, reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(dst), rows);
+        launch_kernel(narrow_rows_f32_kernel, grid_for(rows * 16), 256, 0, st, hdr, reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(dst), rows);
     };
     if (bwd) {
         if (d.d_k == 64) { narrow(w.dq, p.dq); narrow(w.dk, p.dk); }

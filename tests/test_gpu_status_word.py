@@ -1,0 +1,44 @@
+"""The status word of a workspace: after a device-side error a call leaves its outputs unwritten.  Every kernel family."""
+import pytest
+import torch
+
+from paper_2608_12700_b200 import binding, runner, synth
+
+pytestmark = pytest.mark.gpu
+
+BAD_SEQLENS = 5
+
+FAMILIES = {   # (per-channel gates, forced family, descriptor)
+    "operator_form": (False, 2, dict(dtype="bf16", d_k=128, d_v=128)),
+    "low_rank_form": (False, 3, dict(dtype="bf16", d_k=128, d_v=128)),
+    "narrow_values": (False, 0, dict(dtype="bf16", d_k=128, d_v=64)),
+    "scalar_gate_d64": (False, 0, dict(dtype="bf16", d_k=64, d_v=64, delta_rule=0)),
+    "ffma": (False, 0, dict(dtype="f32", d_k=64, d_v=128)),
+    "channelwise": (True, 0, dict(dtype="bf16", d_k=128, d_v=128)),
+    "channelwise_padded": (True, 0, dict(dtype="bf16", d_k=64, d_v=64)),
+    "channelwise_ffma": (True, 0, dict(dtype="f32", d_k=64, d_v=64)),
+}
+
+
+@pytest.fixture(params=sorted(FAMILIES))
+def family(request):
+    channelwise, forced, kw = FAMILIES[request.param]
+    binding.gdn_debug_force_family(forced)
+    yield channelwise, kw
+    binding.gdn_debug_force_family(0)
+
+
+@pytest.mark.parametrize("bad", [[0, 180, 164, 194], [0, 100, 164, 190], [3, 100, 164, 194]], ids=["decreasing", "short", "offset"])
+def test_malformed_cu_seqlens_leave_the_outputs_unwritten(family, bad):
+    channelwise, fam = family
+    wl = (synth.make_channelwise if channelwise else synth.make_workload)("status", lengths=[100, 64, 30], H=2, states=True, seed=190, **fam)
+    buf = (runner.to_device_channelwise if channelwise else runner.to_device)(wl, want_o=True)
+    buf.inputs["cu_seqlens"] = torch.tensor(bad, dtype=torch.int32, device="cuda")
+    for run, outputs in ((runner.run_bwd_channelwise if channelwise else runner.run_bwd, ("dq", "dk", "dv", "dg", "dbeta", "db", "dw", "dh0")),
+                         (runner.run_fwd_channelwise if channelwise else runner.run_fwd, ("o", "hT"))):
+        outs = [buf.outputs[n] for n in outputs if buf.outputs.get(n) is not None]
+        for v in outs:
+            v.fill_(7.0)
+        run(buf)
+        assert binding.gdn_last_device_status(buf.workspace) == BAD_SEQLENS
+        assert all(torch.all(v == 7.0) for v in outs)
