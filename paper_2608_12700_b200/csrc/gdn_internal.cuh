@@ -19,8 +19,9 @@ struct WsHeader {
     int32_t n_chunks;  // chunks actually present (<= max_chunks)
     int32_t detail;    // where a bounded wait gave up / offending sequence index
     int32_t cw_fallback;   // channel-wise calls on the tensor-core route: 1 if the gates of the call leave its range (set by its first
-                           // stage, cleared by the table kernel).  The tensor-core kernels then stand down and the FFMA kernels enqueued
-                           // behind them compute the call, and the backward on the workspace of such a forward.
+                           // stage, cleared by the table kernel of a call that does not consume a forward's workspace).  The
+                           // tensor-core kernels then stand down and the FFMA kernels enqueued behind them compute the call, and
+                           // the backward on the workspace of such a forward.
     int32_t pad[60];
 };
 static_assert(sizeof(WsHeader) == 256, "header size");
@@ -233,7 +234,9 @@ gdn_status check_bwd_args(const gdn_desc* desc, const void* q, const void* k, co
 
 // Kernel families (each defined in its own translation unit).  They enqueue on `st` and return the
 // first CUDA error seen.
-cudaError_t launch_table(const Problem& p, cudaStream_t st);
+// Chunk table of a call with packed sequences (or without tokens); it validates cu_seqlens, so it runs in every such call, ahead
+// of whatever reads them.  `fresh`: the workspace is the forward's, whose fall-back word stays as it is.
+cudaError_t launch_table(const Problem& p, cudaStream_t st, bool fresh = false);
 cudaError_t simt_launch_fwd(const Problem& p, cudaStream_t st);
 cudaError_t simt_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st);
 

@@ -26,7 +26,7 @@ using namespace ffma;
 // ------------------------------------------------------------------------------------------------
 // Chunk table.  One block.  Validates cu_seqlens; on failure records the status and leaves no work.
 // ------------------------------------------------------------------------------------------------
-__global__ void table_kernel(Problem p) {
+__global__ void table_kernel(Problem p, int fresh) {
     wait_prerequisites();
     WsHeader* hdr = reinterpret_cast<WsHeader*>(p.ws);
     int32_t* seq_first = reinterpret_cast<int32_t*>(p.ws + p.L.seq_first);
@@ -47,7 +47,7 @@ __global__ void table_kernel(Problem p) {
             acc += (int)((e - a + kC - 1) / kC);
         }
         if (good && cu(N) != p.Ttot) { good = 0; bad_at = N; }
-        hdr->cw_fallback = 0;
+        if (!fresh) hdr->cw_fallback = 0;
         if (good) {
             seq_first[N] = acc;
             hdr->status = GDN_OK;
@@ -598,7 +598,7 @@ cudaError_t launch_fwd_t(const Problem& p, cudaStream_t st) {
 template <typename IO, int DK, int DV>
 cudaError_t launch_bwd_t(const Problem& p, bool skip_recompute, cudaStream_t st) {
     cudaError_t e;
-    if (p.cu && !skip_recompute && (e = launch_table(p, st)) != cudaSuccess) return e;
+    if (p.cu && (e = launch_table(p, st, skip_recompute)) != cudaSuccess) return e;
     if ((e = launch_prep_t<IO, DK, DV>(p, skip_recompute ? PREP_BWD : PREP_FWD_BWD, st)) != cudaSuccess) return e;
     if ((e = launch_scan_t<DK, DV>(p, skip_recompute ? 1 : 2, st)) != cudaSuccess) return e;
     static SmemLimitOnce once;
@@ -609,9 +609,9 @@ cudaError_t launch_bwd_t(const Problem& p, bool skip_recompute, cudaStream_t st)
 
 }  // namespace
 
-cudaError_t launch_table(const Problem& p, cudaStream_t st) {
+cudaError_t launch_table(const Problem& p, cudaStream_t st, bool fresh) {
     StageScope t(ST_TABLE, st);
-    launch_kernel(table_kernel, 1, 256, 0, st, p);
+    launch_kernel(table_kernel, 1, 256, 0, st, p, fresh ? 1 : 0);
     return cudaGetLastError();
 }
 

@@ -872,8 +872,8 @@ cudaError_t cw_tc_launch(const Problem& p, bool bwd, bool skip_recompute, cudaSt
     static SmemLimitOnce once_scale, once_prep, once_eprep, once_intra;
     const int CH = p.L.max_chunks * p.d.H, chains = p.d.N * p.d.H;
     cudaError_t e;
-    const bool fresh = bwd && skip_recompute;   // the chunk table, the images, gam and the factors are still there
-    if (!fresh && (e = launch_table(p, st)) != cudaSuccess) return e;
+    const bool fresh = bwd && skip_recompute;   // the images, gam and the factors are still there
+    if ((!fresh || p.cu) && (e = launch_table(p, st, fresh)) != cudaSuccess) return e;
     const int sms = tc_sm_count(), grid = CH < sms ? CH : sms, grid2 = CH < 2 * sms ? CH : 2 * sms;
     CwParams P;
     P.p = p;

@@ -1,4 +1,6 @@
-"""The status word of a workspace: after a device-side error a call leaves its outputs unwritten.  Every kernel family."""
+"""The status word of a workspace: after a device-side error a call leaves its outputs unwritten, and malformed cu_seqlens are
+refused before any kernel reads them, in a backward on the forward's workspace too.  Every kernel family."""
+import numpy as np
 import pytest
 import torch
 
@@ -42,3 +44,41 @@ def test_malformed_cu_seqlens_leave_the_outputs_unwritten(family, bad):
         run(buf)
         assert binding.gdn_last_device_status(buf.workspace) == BAD_SEQLENS
         assert all(torch.all(v == 7.0) for v in outs)
+
+
+def forward(family, **kw):
+    """Buffers after a forward, outputs of the backward filled with 7, and the backward on that workspace."""
+    channelwise, fam = family
+    make = synth.make_channelwise if channelwise else synth.make_workload
+    wl = make("status", H=2, states=True, seed=190, **fam, **kw)
+    buf = (runner.to_device_channelwise if channelwise else runner.to_device)(wl, want_o=True)
+    (runner.run_fwd_channelwise if channelwise else runner.run_fwd)(buf)
+    for n, v in buf.outputs.items():
+        if v is not None and n not in ("o", "hT"):
+            v.fill_(7.0)
+    run = runner.run_bwd_channelwise if channelwise else runner.run_bwd
+    return wl, buf, lambda: run(buf, fresh=1)
+
+
+def assert_unwritten(buf):
+    for n, v in buf.outputs.items():
+        if v is not None and n not in ("o", "hT"):
+            assert torch.all(v == 7.0), n
+
+
+def test_malformed_cu_seqlens_are_refused_on_a_forwards_workspace(family):
+    wl, buf, bwd = forward(family, lengths=[100, 64, 30])
+    good = buf.inputs["cu_seqlens"]
+    for bad in ([0, 180, 164, 194], [0, 100, 164, 190], [3, 100, 164, 194]):   # decreasing; short of T; not from 0
+        buf.inputs["cu_seqlens"] = torch.tensor(bad, dtype=torch.int32, device="cuda")
+        bwd()
+        assert binding.gdn_last_device_status(buf.workspace) == BAD_SEQLENS
+        assert_unwritten(buf)
+    # the forward's data is whole: with its own cu_seqlens the backward runs, and as if nothing had happened
+    buf.inputs["cu_seqlens"] = good
+    bwd()
+    got = runner.fetch(buf)
+    channelwise, _ = family
+    whole = (runner.backward_channelwise if channelwise else runner.backward)(wl)
+    for n in whole:
+        assert np.array_equal(whole[n], got[n]), n
