@@ -99,7 +99,9 @@ gdn_status gdn_fwd_recompute(const gdn_desc* desc,
  *     dbeta        required iff delta_rule dh0     optional (NULL: not written)
  *     dhT          optional (NULL = zero)  h0      optional (NULL = zero)
  * workspace_is_fresh_from_fwd != 0 asserts that `workspace` was filled by gdn_fwd_recompute with the same
- * desc, q, k, v, g, beta, h0 and cu_seqlens and not touched since; the recompute stage is then skipped. */
+ * desc, q, k, v, g, beta, h0 and cu_seqlens and not touched since; the recompute stage is then skipped.  A wait that
+ * ran out, or malformed cu_seqlens in the forward, stand in its status word until the next forward: such a backward computes
+ * nothing from what was left there. */
 gdn_status gdn_bwd(const gdn_desc* desc,
                    const void* q, const void* k, const void* v,
                    const float* g, const float* beta, const float* h0,

@@ -22,7 +22,9 @@ struct WsHeader {
                            // stage, cleared by the table kernel of a call that does not consume a forward's workspace).  The
                            // tensor-core kernels then stand down and the FFMA kernels enqueued behind them compute the call, and
                            // the backward on the workspace of such a forward.
-    int32_t pad[60];
+    int32_t fresh_refused;   // 1 if a status of GDN_ERR_BAD_SEQLENS comes from a backward on the forward's workspace, not from the
+                             // forward: the forward's data is whole, and the next such backward may have better cu_seqlens
+    int32_t pad[59];
 };
 static_assert(sizeof(WsHeader) == 256, "header size");
 
@@ -235,7 +237,7 @@ gdn_status check_bwd_args(const gdn_desc* desc, const void* q, const void* k, co
 // Kernel families (each defined in its own translation unit).  They enqueue on `st` and return the
 // first CUDA error seen.
 // Chunk table of a call with packed sequences (or without tokens); it validates cu_seqlens, so it runs in every such call, ahead
-// of whatever reads them.  `fresh`: the workspace is the forward's, whose fall-back word stays as it is.
+// of whatever reads them.  `fresh`: the workspace is the forward's, whose status and fall-back words stay as they are.
 cudaError_t launch_table(const Problem& p, cudaStream_t st, bool fresh = false);
 cudaError_t simt_launch_fwd(const Problem& p, cudaStream_t st);
 cudaError_t simt_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st);

@@ -24,7 +24,8 @@ namespace {
 using namespace ffma;
 
 // ------------------------------------------------------------------------------------------------
-// Chunk table.  One block.  Validates cu_seqlens; on failure records the status and leaves no work.
+// Chunk table.  One block.  Validates cu_seqlens; on failure records the status and leaves no work.  In a backward on the
+// forward's workspace (fresh) an error that the forward left stands: nothing is to be computed from what it left.
 // ------------------------------------------------------------------------------------------------
 __global__ void table_kernel(Problem p, int fresh) {
     wait_prerequisites();
@@ -36,7 +37,9 @@ __global__ void table_kernel(Problem p, int fresh) {
     const int N = p.d.N;
     __shared__ int ok;
     auto cu = [&](int n) -> long long { return p.cu ? (long long)p.cu[n] : (long long)n * p.d.T; };
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && fresh && hdr->status != GDN_OK && !(hdr->status == GDN_ERR_BAD_SEQLENS && hdr->fresh_refused)) {
+        ok = 0;
+    } else if (threadIdx.x == 0) {
         int good = 1, bad_at = -1;
         if (cu(0) != 0) { good = 0; bad_at = 0; }
         int acc = 0;
@@ -48,6 +51,7 @@ __global__ void table_kernel(Problem p, int fresh) {
         }
         if (good && cu(N) != p.Ttot) { good = 0; bad_at = N; }
         if (!fresh) hdr->cw_fallback = 0;
+        hdr->fresh_refused = fresh && !good;
         if (good) {
             seq_first[N] = acc;
             hdr->status = GDN_OK;
@@ -138,7 +142,7 @@ template <typename IO, int DK, int DV>
 __global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) {
     wait_prerequisites();
     const bool fwd = mode != PREP_BWD, bwd = mode != PREP_FWD;
-    init_header_if_untabled(p);
+    if (fwd) init_header_if_untabled(p);   // (the backward's part alone: the status word is the forward's)
     ChunkInfo x;
     if (!chunk_info(p, x)) return;   // (no chunk at all when the table was refused)
     constexpr int PK = pitch(DK), PV = pitch(DV);

@@ -296,8 +296,8 @@ __device__ __forceinline__ void vprep_chunk(const Problem& p, int mode, const Ch
 template <typename IO, int DK, int DV>
 __global__ void __launch_bounds__(kThreads, 1) vprep_kernel(Problem p, int mode) {
     wait_prerequisites();
-    if (!p.fallback) init_header_if_untabled(p);
-    else if (!vec_go(p)) return;
+    if (p.fallback) { if (!vec_go(p)) return; }
+    else if (mode != PREP_BWD) init_header_if_untabled(p);   // (the backward's part alone: the status word is the forward's)
     for_chunks(p, [&](const ChunkInfo& x) { vprep_chunk<IO, DK, DV>(p, mode, x); });
 }
 

@@ -1833,15 +1833,15 @@ static cudaError_t empty_call(const Problem& p, bool bwd, cudaStream_t st) {
 }
 
 // The chunk table is needed for packed sequences only (and for an empty call, whose only kernel it is).
-static cudaError_t launch_table_if_needed(const Problem& p, cudaStream_t st) {
-    return (p.cu || p.Ttot == 0) ? launch_table(p, st) : cudaSuccess;
+static cudaError_t launch_table_if_needed(const Problem& p, bool fresh, cudaStream_t st) {
+    return (p.cu || p.Ttot == 0) ? launch_table(p, st, fresh) : cudaSuccess;
 }
 
 // Carries in low-rank form take the chunk factors from tc_prep_lr; in operator form they also need Nm and Bf, which only
 // tc_prep makes.
 cudaError_t tc_launch_fwd(const Problem& p, cudaStream_t st) {
     TcParams P;
-    cudaError_t e = launch_table_if_needed(p, st);
+    cudaError_t e = launch_table_if_needed(p, false, st);
     if (e != cudaSuccess) return e;
     if (p.Ttot == 0) return empty_call(p, false, st);
     if (!fill_params(P, p, false, 0)) return cudaErrorUnknown;
@@ -1850,12 +1850,12 @@ cudaError_t tc_launch_fwd(const Problem& p, cudaStream_t st) {
     return p.o ? launch_out(P, st) : cudaSuccess;
 }
 
-// With a workspace fresh from gdn_fwd_recompute nothing of the forward is repeated: T, W, U~ and the per-chunk states
-// are taken from it, and only what needs dO is built (P, E; tc_eprep), followed by the reverse carry and the
-// gradient stage.
+// With a workspace fresh from gdn_fwd_recompute nothing of the forward is repeated: P, T, W, U~ and the per-chunk states
+// are taken from it, and only what needs dO is built (E; tc_eprep), followed by the reverse carry and the
+// gradient stage.  A status that the forward left stands.
 cudaError_t tc_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st) {
     TcParams P;
-    cudaError_t e = launch_table_if_needed(p, st);
+    cudaError_t e = launch_table_if_needed(p, skip_recompute, st);
     if (e != cudaSuccess) return e;
     if (p.Ttot == 0) return empty_call(p, true, st);
     if (!fill_params(P, p, true, skip_recompute ? 1 : 2)) return cudaErrorUnknown;

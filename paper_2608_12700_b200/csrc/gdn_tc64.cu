@@ -594,13 +594,14 @@ static bool fill_params64(Tc64Params& P, const Problem& p, bool with_bwd) {
     return true;
 }
 
-static cudaError_t tc64_prologue(const Problem& p, cudaStream_t st) {
+// fresh: gamma and the status word are those of the forward whose workspace the call consumes.
+static cudaError_t tc64_prologue(const Problem& p, bool fresh, cudaStream_t st) {
     // the chunk table is needed for packed sequences only (and for an empty call, whose only kernel it is)
     if (p.cu || p.Ttot == 0) {
-        const cudaError_t e = launch_table(p, st);
+        const cudaError_t e = launch_table(p, st, fresh);
         if (e != cudaSuccess) return e;
     }
-    if (p.L.max_chunks > 0 && p.Ttot > 0) {
+    if (!fresh && p.L.max_chunks > 0 && p.Ttot > 0) {
         StageScope t(ST_PREP, st);
         launch_kernel(tc64_gamma_kernel, dim3(p.L.max_chunks, (p.d.H + 31) / 32), 256, 0, st, p);
     }
@@ -623,7 +624,7 @@ static cudaError_t tc64_fwd_pass(const Tc64Params& P, cudaStream_t st) {
 
 cudaError_t tc64_launch_fwd(const Problem& p, cudaStream_t st) {
     Tc64Params P;
-    cudaError_t e = tc64_prologue(p, st);
+    cudaError_t e = tc64_prologue(p, false, st);
     if (e != cudaSuccess) return e;
     if (p.Ttot == 0) {
         const size_t bytes = (size_t)p.d.N * p.d.H * D6 * D6 * sizeof(float);
@@ -636,7 +637,7 @@ cudaError_t tc64_launch_fwd(const Problem& p, cudaStream_t st) {
 
 cudaError_t tc64_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st) {
     Tc64Params P;
-    cudaError_t e = tc64_prologue(p, st);
+    cudaError_t e = tc64_prologue(p, skip_recompute, st);
     if (e != cudaSuccess) return e;
     if (p.Ttot == 0) {
         const size_t bytes = (size_t)p.d.N * p.d.H * D6 * D6 * sizeof(float);

@@ -1,5 +1,6 @@
 """The status word of a workspace: after a device-side error a call leaves its outputs unwritten, and malformed cu_seqlens are
-refused before any kernel reads them, in a backward on the forward's workspace too.  Every kernel family."""
+refused before any kernel reads them, in a backward on the forward's workspace too; such a backward computes nothing after an
+error of the forward (the word is written by the host here, in place of a wait that ran out).  Every kernel family."""
 import numpy as np
 import pytest
 import torch
@@ -8,7 +9,7 @@ from paper_2608_12700_b200 import binding, runner, synth
 
 pytestmark = pytest.mark.gpu
 
-BAD_SEQLENS = 5
+BAD_SEQLENS, TIMEOUT = 5, 8
 
 FAMILIES = {   # (per-channel gates, forced family, descriptor)
     "operator_form": (False, 2, dict(dtype="bf16", d_k=128, d_v=128)),
@@ -82,3 +83,24 @@ def test_malformed_cu_seqlens_are_refused_on_a_forwards_workspace(family):
     whole = (runner.backward_channelwise if channelwise else runner.backward)(wl)
     for n in whole:
         assert np.array_equal(whole[n], got[n]), n
+
+
+@pytest.mark.parametrize("seqs", [dict(lengths=[100, 64, 30]), dict(B=2, T=100)], ids=["packed", "equal"])
+def test_an_error_of_the_forward_stands_in_the_backward_on_its_workspace(family, seqs):
+    wl, buf, bwd = forward(family, **seqs)
+    buf.workspace[:4].view(torch.int32).fill_(TIMEOUT)
+    bwd()
+    assert binding.gdn_last_device_status(buf.workspace) == TIMEOUT
+    assert_unwritten(buf)
+
+
+def test_malformed_cu_seqlens_in_the_forward_leave_nothing_for_the_backward(family):
+    wl, buf, bwd = forward(family, lengths=[100, 64, 30])
+    good = buf.inputs["cu_seqlens"]
+    buf.inputs["cu_seqlens"] = torch.tensor([0, 100, 164, 190], dtype=torch.int32, device="cuda")
+    (runner.run_fwd_channelwise if family[0] else runner.run_fwd)(buf)
+    assert binding.gdn_last_device_status(buf.workspace) == BAD_SEQLENS
+    buf.inputs["cu_seqlens"] = good
+    bwd()
+    assert binding.gdn_last_device_status(buf.workspace) == BAD_SEQLENS
+    assert_unwritten(buf)
