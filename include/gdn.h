@@ -150,7 +150,8 @@ gdn_status gdn_bwd_channelwise(const gdn_desc* desc,
 /* Synchronises the stream, reads the device-side status word of the last call that used `workspace`
  * and returns it (GDN_OK, GDN_ERR_BAD_SEQLENS or GDN_ERR_DEVICE_TIMEOUT; GDN_ERR_CUDA if the stream
  * itself reports an error).  Error reporting of this library (the paper has no counterpart).  After
- * a device-side error the kernels of that call stop early and leave the outputs unwritten. */
+ * a device-side error the remaining kernels of that call leave its outputs unwritten (a wait that runs out in the last of
+ * them, the gradient stage, leaves the outputs partly written). */
 gdn_status gdn_last_device_status(const void* workspace, void* cuda_stream);
 
 /* Static, NUL-terminated description of a status code (the paper has no counterpart). */
@@ -233,7 +234,7 @@ gdn_status gdn_debug_force_family(int32_t family);
  * leaves out one of its input loads, so the wait for it runs out.  The CTAs leave through their normal teardown
  * (tensor memory released, no copy in flight), the remaining kernels of the call see the status word and write
  * nothing, gdn_bwd itself returns GDN_OK and gdn_last_device_status reports GDN_ERR_DEVICE_TIMEOUT.  The next call
- * is a normal one.  0 cancels a pending request. */
+ * is a normal one.  2 and 3: the same in the carries and in the gradient stage.  0 cancels a pending request. */
 gdn_status gdn_debug_inject_timeout(int32_t on);
 
 #ifdef __cplusplus

@@ -250,7 +250,8 @@ cudaError_t cw_tc_launch(const Problem& p, bool bwd, bool skip_recompute, cudaSt
 
 // tcgen05 family (bf16 I/O; tiles of 128 features, a head dimension of 64 fills half of them).
 extern thread_local int g_force_carries;   // form of the inter-chunk carries: 0 = chosen by shape, 1 = operator form, 2 = low-rank
-extern thread_local int g_inject_timeout;   // debugging hook: the next gdn_bwd of this family provokes a device-side time-out
+extern thread_local int g_inject_timeout;   // debugging hook: the next gdn_bwd of this family provokes a device-side time-out (which
+                                            // kernel's: see TcParams::withhold)
 bool tc_supported(const gdn_desc& d);
 // Form of the carries for a descriptor: one rule for the forward, the backward and a backward that consumes a workspace
 // fresh from the forward, so that the layout of a workspace does not depend on which call sized it.

@@ -36,6 +36,7 @@ constexpr int kTG = kC / kGroups;             // token columns per group (16)
 constexpr int kIntraThreads = kWideThreads + 32;   // ... plus one warp whose first lane only issues MMAs; the kernels are
                                                    // launched with one more warp on top (kIntraThreads + 32) that only
                                                    // issues bulk copies and takes no part in the named barrier
+enum { WITHHOLD_PREP = 1, WITHHOLD_CARRY = 2, WITHHOLD_GRADIENT = 3 };   // values of TcParams::withhold and of gdn_debug_inject_timeout
 struct TcParams {
     Problem p;
     CUtensorMap tm_q, tm_k, tm_v, tm_do;   // [T_total, H, d] bf16, boxes of 64 tokens x 64 features of a head
@@ -44,8 +45,8 @@ struct TcParams {
     int with_bwd;                          // prep: also produce E
     int scan_dirs;                         // scan: 0 = forward carry only, 1 = reverse only, 2 = both
     int lowrank;                           // carries in low-rank form (tc_scan_lr): prepared by tc_prep_lr without Nm, Bf
-    int withhold;                          // debugging hook: tc_prep leaves out one of its first loads, so that the wait
-                                           // for it runs out (exercises the time-out path without any fault)
+    int withhold;                          // debugging hook: a kernel leaves out one of its first loads, so that the wait for
+                                           // it runs out (exercises the time-out path without any fault)
 };
 
 // ------------------------------------------------------------------------------------------------
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     if (warp == 0) { fetch_gates(xn); make_gates(0, xn.ch); }
     // first trip: the inputs are loaded at once, one instruction per warp
     if (issuer) { mbar_expect_tx(&bar_qk, 32768); mbar_expect_tx(&bar_vo, VO_BYTES); }
-    if (lane == 0 && warp < 8 && !(P.withhold && warp == 0)) load_piece(warp, xn);
+    if (lane == 0 && warp < 8 && !(P.withhold == WITHHOLD_PREP && warp == 0)) load_piece(warp, xn);
 #pragma unroll 1
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, in_phase ^= 1) {
     const ChunkInfo x = xn;
@@ -474,7 +475,10 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     fence_async_smem();
     cta_sync();
     if (threadIdx.x == 32) mbar_arrive(&bar_st);   // the three images are staged: the loader stores them
-    if (!ok) break;
+    if (!ok) {   // a load of this trip may still be in flight: wait for it (bounded) before the CTA retires
+        if (threadIdx.x == 0) { (void)mbar_wait(&bar_vo, in_phase); (void)mbar_wait(&bar_qk, in_phase); }
+        break;
+    }
     }
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
@@ -554,7 +558,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
         const int stage = s % STAGES;
         const size_t ch = (size_t)chunk_of(s) * p.d.H + hd;
         mbar_expect_tx(&bar_full[stage], STAGE_BYTES);
-        bulk_load(sm + stage * STAGE_BYTES + NM, nm_base + ch * 32768, 32768, &bar_full[stage]);
+        if (!(P.withhold == WITHHOLD_CARRY && s == 0)) bulk_load(sm + stage * STAGE_BYTES + NM, nm_base + ch * 32768, 32768, &bar_full[stage]);
         bulk_load(sm + stage * STAGE_BYTES + ADD, add_base + ch * 32768, ADD_BYTES, &bar_full[stage]);
         // The ring gives a load one step of lead, less than an HBM round trip; pull the step after next into L2 now.
         if (s + PREFETCH_AHEAD < nsteps) {
@@ -588,8 +592,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
     __syncthreads();
     bool ok = true;
     uint32_t mma_phase = 0;
+    int s = 0;
 #pragma unroll 1
-    for (int s = 0; s < nsteps; ++s) {
+    for (; s < nsteps; ++s) {
         unsigned char* Ht = sm + HT + (s & 1) * HT_BYTES;
         const size_t ch = (size_t)chunk_of(s) * p.d.H + hd;
         const int stage = s % STAGES;
@@ -645,6 +650,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
         for (int k = 0; k < NSH / 4; ++k) if (inside) *reinterpret_cast<float4*>(fin + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
     }
     if (warp == 0) bulk_wait_read<0>();
+    if (threadIdx.x == 32) drain_ring<STAGES>(bar_full, s, nsteps);
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, NS);
@@ -739,7 +745,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         const size_t ch = (size_t)c * H + hd;
         unsigned char* slot = sm + stage * STAGE_BYTES;
         mbar_expect_tx(&bar_full[stage], 32768 + x_bytes);
-        bulk_load(slot + WT, w_base + ch * 16384, 16384, &bar_full[stage]);
+        if (!(P.withhold == WITHHOLD_CARRY && s == 0)) bulk_load(slot + WT, w_base + ch * 16384, 16384, &bar_full[stage]);
         if constexpr (CW) {
             // k-, in both directions: what is left of the decay is applied to the state (row by row, below)
             bulk_load(slot + KT, p.ws + p.L.img_Km + ch * 16384, 16384, &bar_full[stage]);
@@ -785,8 +791,9 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         cw_ref = reinterpret_cast<const int32_t*>(p.ws + p.L.ref)[ch * D + r];
     };
     if (CW && nsteps > 0) cw_fetch(0);
+    int s = 0;
 #pragma unroll 1
-    for (int s = 0; s < nsteps; ++s) {
+    for (; s < nsteps; ++s) {
         unsigned char* Ht = sm + HT + (s & 1) * HT_BYTES;
         const int c = chunk_of(s), stage = s % STAGES, len = sg.chunk_len(c);
         const size_t ch = (size_t)c * H + hd;
@@ -894,6 +901,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         for (int k = 0; k < NSH / 4; ++k) if (inside) *reinterpret_cast<float4*>(fin + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
     }
     if (warp == 0) bulk_wait_read<0>();
+    if (threadIdx.x == 32) drain_ring<STAGES>(bar_full, s, nsteps);
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, C::TMEM_COLS);
@@ -1219,7 +1227,7 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     };
     // first trip: every group is loaded at once, one instruction per warp
     if (issuer) { mbar_expect_tx(&bar_a, A_BYTES); mbar_expect_tx(&bar_b, B_BYTES); mbar_expect_tx(&bar_u, U_BYTES); }
-    if (lane == 0 && warp < 15) load_piece(warp, xn);
+    if (lane == 0 && warp < 15 && !(P.withhold == WITHHOLD_GRADIENT && warp == 9)) load_piece(warp, xn);
     if (gates) { fetch_gates(xn); make_gates(0); }
 #pragma unroll 1
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, in_phase ^= 1) {
@@ -1506,7 +1514,10 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
         flush_rows(sm + STG_Q, p.dq, x, H, p.d.d_k, kWideThreads);
         flush_rows(sm + STG_K, p.dk, x, H, p.d.d_k, kWideThreads);
     }
-    if (!ok) break;
+    if (!ok) {   // a load of this trip may still be in flight: wait for it (bounded) before the CTA retires
+        if (threadIdx.x == 0) { (void)mbar_wait(&bar_a, in_phase); (void)mbar_wait(&bar_u, in_phase); (void)mbar_wait(&bar_b, in_phase); }
+        break;
+    }
     }
     if (ok && have_prev && gates) finish_gates();
     if (warp == 0) tmem_dealloc(tmem, 512);
@@ -1860,10 +1871,10 @@ cudaError_t tc_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st
     if (p.Ttot == 0) return empty_call(p, true, st);
     if (!fill_params(P, p, true, skip_recompute ? 1 : 2)) return cudaErrorUnknown;
     const bool inject = g_inject_timeout && !skip_recompute;
-    if (inject) {   // debugging hook, this call only: a millisecond of patience, and tc_prep withholds one load
+    if (inject) {   // debugging hook, this call only: a millisecond of patience, and one kernel withholds a load
         const unsigned long long ns = 1000000ull;
+        P.withhold = g_inject_timeout;
         g_inject_timeout = 0;
-        P.withhold = 1;
         if ((e = cudaMemcpyToSymbolAsync(g_wait_limit_ns, &ns, sizeof(ns), 0, cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
     }
     if ((e = skip_recompute ? launch_eprep(P, st) : P.lowrank ? launch_prep_lr(P, st) : launch_prep(P, st)) != cudaSuccess) return e;

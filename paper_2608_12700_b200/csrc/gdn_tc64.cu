@@ -156,8 +156,9 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
     __syncthreads();
     bool ok = true;
     uint32_t mma_phase = 0;
+    int s = 0;
 #pragma unroll 1
-    for (int s = 0; s < nsteps; ++s) {
+    for (; s < nsteps; ++s) {
         const int c = c0 + s, stage = s % STAGES, len = cg.chunk_len(c);
         const size_t ch = (size_t)c * H + hd;
         unsigned char* tiles = sm + stage * STAGE_BYTES;
@@ -265,6 +266,7 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
         }
     }
     if (warp == 0) bulk_wait_read<0>();
+    if (threadIdx.x == 0) drain_ring<STAGES>(bar_full, s, nsteps);
     if (p.hT && ok) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) *reinterpret_cast<float4*>(p.hT + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
@@ -350,8 +352,9 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
     if (loader) {
         if (lane == 0) {
             for (int s = 0; s < STAGES && s < nsteps; ++s) fill(s);
+            int s = 0;
 #pragma unroll 1
-            for (int s = 0; s < nsteps; ++s) {
+            for (; s < nsteps; ++s) {
                 if (!mbar_wait(&bar_st, s & 1)) break;          // step s has staged its gradient rows (or flushed them)
                 const int c = c1 - 1 - s;
                 if (cg.chunk_len(c) == kC) {
@@ -366,6 +369,7 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
                 if (s + STAGES < nsteps) fill(s + STAGES);
             }
             bulk_wait_read<0>();
+            drain_ring<STAGES>(bar_full, s, nsteps);
         }
         return;
     }

@@ -118,6 +118,15 @@ __device__ __forceinline__ void write_dg_suffix(const float* v0, const float* v1
     if (lane + 32 < len) dg[(size_t)(lane + 32) * stride] = b;
 }
 
+// After a wait gave up in step `s` of a chain: waits (bounded) for the loads of the ring that are in flight, so that the CTA does
+// not retire under them.  By one thread.  (Without a time-out s = nsteps and there is nothing to wait for; at most one of the
+// waits is for a load that was never issued.)
+template <int STAGES>
+__device__ __forceinline__ void drain_ring(uint64_t* bar_full, int s, int nsteps) {
+#pragma unroll 1
+    for (int k = s; k < nsteps && k < s + STAGES; ++k) (void)mbar_wait(&bar_full[k % STAGES], (k / STAGES) & 1);
+}
+
 // Wait for the MMAs committed to `bar`; on a timeout record it once.
 #define GDN_WAIT_MMA(where)                                                    \
     if (ok) {                                                                  \

@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
     };
     ChunkInfo x;
     chunk_entry(p, x, blockIdx.x);
-    if (threadIdx.x == 0) issue_loads(x, P.withhold != 0);
+    if (threadIdx.x == 0) issue_loads(x, P.withhold == WITHHOLD_PREP);
     if (warp == 0) fetch_gates(x);
 #pragma unroll 1
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, in_phase ^= 1) {

@@ -35,6 +35,31 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_correct(lengths, 
     assert binding.gdn_last_device_status(buf.workspace) == binding.GDN_OK
 
 
+@pytest.mark.parametrize("form", [2, 3], ids=["operator", "low_rank"])
+@pytest.mark.parametrize("where", [1, 2, 3], ids=["preparation", "carries", "gradients"])
+@pytest.mark.parametrize("shape", [dict(lengths=[200, 64, 75], H=2), dict(B=3, T=700, H=10)], ids=["small", "several_trips"])
+def test_every_kernel_leaves_through_its_teardown(shape, where, form):
+    """One wait at a time, in the preparation, the carries (one and two CTAs per chain) and the gradient stage, in both forms of the
+    carries; the larger shape has 330 chunk-heads (every CTA of the persistent kernels has further trips) and 30 chains."""
+    try:
+        binding.gdn_debug_force_family(form)
+        wl = synth.make_workload("timeout_where", dtype="bf16", d_k=128, d_v=128, states=True, seed=92, **shape)
+        buf = runner.to_device(wl)
+        for v in buf.outputs.values():
+            if v is not None:
+                v.fill_(7.0)
+        binding.gdn_debug_inject_timeout(where)
+        runner.run_bwd(buf)
+        assert binding.gdn_last_device_status(buf.workspace) == GDN_ERR_DEVICE_TIMEOUT
+        if where < 3:   # the gradient stage saw the status and wrote nothing
+            for n in ("dq", "dk", "dv", "dg", "dbeta") + (("dh0",) if where == 2 else ()):
+                assert torch.all(buf.outputs[n] == 7.0), n
+        runner.run_bwd(buf)
+        check_against_oracle(wl, runner.fetch(buf))
+    finally:
+        binding.gdn_debug_force_family(0)
+
+
 def test_a_cancelled_request_changes_nothing():
     wl = synth.make_workload("timeout_cancel", dtype="bf16", lengths=[100], H=1, d_k=128, d_v=128, states=True, seed=91)
     binding.gdn_debug_inject_timeout(True)
