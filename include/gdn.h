@@ -126,7 +126,8 @@ gdn_status gdn_bwd(const gdn_desc* desc,
  * layout; its status word is read with gdn_last_device_status.  With bf16 I/O these calls run on the tensor cores
  * (tcgen05; kernels for d_k = d_v = 128, a head dimension of 64 is zero-padded to 128 inside the workspace, gate
  * vectors included, which is exact): keys and queries are scaled by the chunk-local cumulative decay element by element, which
- * requires |sum of g over any prefix of a 64-token chunk| <= 80 per channel; a call whose gates leave that range is
+ * requires |sum of g over any prefix of a 64-token chunk| <= 80 per channel, and such sums no more than 92 apart (which takes
+ * gates of both signs); a call whose gates leave that range is
  * computed by the FFMA kernels instead (which evaluate the decay inside the contractions and have no such limit): the
  * decision is taken on the device, the call enqueues the same launches either way and needs no host round trip.  fp32
  * I/O runs on fp32 FFMA kernels throughout (with bf16 I/O they take bf16 inputs and give bf16 dq, dk, dv; all their

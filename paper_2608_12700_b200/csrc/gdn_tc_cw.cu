@@ -19,8 +19,8 @@
 // between e^-40 and e^40.  With S = 1, K- reached e^80 and dh'' e^-80 of the values: an increment K-^T U beyond fp32 for values
 // of 1e5, a subnormal dh'' for gradients of 1e-6.  A power of two, because every operand is then the same number
 // with another exponent, and no rounding depends on S.  Beside the carries (tc_scan_cw in gdn_tc.cu):
-//   cw_scale  scaled operand tiles as bf16 tile images, gam, ref; checks that |gam| stays below 80 (beyond that the split
-//             would need reference points inside the chunk): otherwise it sets the fall-back word of the workspace header, the kernels below
+//   cw_scale  scaled operand tiles as bf16 tile images, gam, ref; checks that gam stays in range (beyond it the split would
+//             need reference points inside the chunk): otherwise it sets the fall-back word of the workspace header, the kernels below
 //             stand down, and the FFMA sequence enqueued behind them computes the call (gdn_simt_vec.cu)
 //   cw_prep   [Q~;K+] K-^T, fp32 blocked inversion, W^T, U~^T, (P^T dO')^T, E               (tcgen05)
 //   cw_intra  the thirteen products of the gradient stage in four dependent steps (K#2 reuses T), and from them dq, dk, dv,
@@ -38,7 +38,9 @@ using namespace tc;
 
 constexpr int D = 128;
 constexpr int kT = 256;               // 8 warps: TMEM lane quadrant = warp % 4, column half = warp / 4
-constexpr float kMaxDecay = 80.f;     // bound on |gam| inside a chunk (|log G| is no larger: exp(80) is still a bf16 number)
+constexpr float kMaxDecay = 80.f;     // bound on |gam| inside a chunk, hence |log2 S| <= 58
+constexpr float kMaxSwing = 92.f;     // ... and on the range of gam and 0, hence |log2 G| <= 67: G, 1 / G and the factors of the carries (G_e
+                                      // times another chunk's S) are normal numbers.  Gates that only decay never come near it.
 
 // (chunk, head) of an elementwise CTA, from the chunk table (which these calls always build)
 struct ChunkCtx { int hd, ch, tok0, len; };
@@ -86,7 +88,7 @@ __global__ void __launch_bounds__(kT) cw_scale_kernel(Problem p) {
                 hi = fmaxf(hi, s);
             }
         }
-        if (lo < -kMaxDecay || hi > kMaxDecay) bad = 1;   // (a NaN gate passes and comes out as NaN)
+        if (lo < -kMaxDecay || hi > kMaxDecay || hi - lo > kMaxSwing) bad = 1;   // (a NaN gate passes and comes out as NaN)
         ref[r] = __float2int_rn(0.5f * kLog2e * (lo + hi));
     }
     __syncthreads();

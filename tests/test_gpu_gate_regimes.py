@@ -141,3 +141,30 @@ def test_channelwise_decay_at_the_edge_of_the_range(family, decay, values, grads
     got = runner.fetch(buf)
     for n in ("dq", "dk", "dv", "dg", "db", "dw", "dh0"):
         assert rel(got[n], ref[n]) <= TOL[wl.dtype], (n, rel(got[n], ref[n]))
+
+
+@pytest.mark.parametrize("family", CW_FAMILIES)
+@pytest.mark.parametrize("rise,fall", [(10.0, -88.0), (40.0, -85.0), (50.0, -100.0), (-79.0, 0.0)])
+def test_channelwise_gates_of_both_signs(family, rise, fall):
+    """Channels that grow for the first 24 tokens of a chunk and then decay, to just inside and to beyond what the tensor-core route
+    accepts (sums in [-80, 80] no more than 92 apart), and chunks that decay by e^-79 beside chunks that do not at all (the
+    references of neighbouring chunks differ by 2^57).  Growth by more than e^10 without the delta rule, whose products of growing
+    keys leave fp32.  Where gates grow, states and outputs of other channels are small beside theirs: whole tensors are compared,
+    not blocks."""
+    wl = cw_workload(family, "cw_signs")
+    if rise > 10.0:
+        wl.bv[:] = 0.0
+    for n in range(wl.N):
+        pos = np.arange(wl.cu_seqlens[n + 1] - wl.cu_seqlens[n])
+        g = np.where(pos % 64 < 24, rise / 24, fall / 40)
+        if fall == 0.0:
+            g = np.where(pos // 64 % 2 == 0, rise / 64, 0.0)
+        wl.gv[wl.cu_seqlens[n]:wl.cu_seqlens[n + 1], :, 1::2] = g[:, None, None]
+    ref = oracle.vec_bwd_workload(wl)
+    buf = runner.to_device_channelwise(wl, want_o=True)
+    runner.run_fwd_channelwise(buf)
+    got = runner.fetch(buf)
+    runner.run_bwd_channelwise(buf)
+    got.update({n: x for n, x in runner.fetch(buf).items() if n not in ("o", "hT")})
+    for n in ("o", "hT", "dq", "dk", "dv", "dg", "db", "dw", "dh0"):
+        assert rel(got[n], ref[n]) <= TOL[wl.dtype], (n, rel(got[n], ref[n]))
