@@ -191,6 +191,28 @@ def test_tensor_core_route_with_several_trips_per_cta_and_equal_lengths():
     print(wl.name, errs)
 
 
+@pytest.mark.parametrize("shape", [dict(B=3, T=700), dict(lengths=[700, 0, 701, 64, 635])], ids=["equal", "packed"])
+def test_fall_back_with_several_items_per_block(shape):
+    """The fall-back sequence has one block per SM, each walking over its chunk-heads and slices of the carries: here several of
+    each per block, so shared memory is used again from item to item.  A single channel of a single chunk leaves the range."""
+    wl = synth.make_channelwise("cw_fallback_trips", member="gdn", dtype="bf16", H=10, d_k=128, d_v=128, states=True, seed=72, **shape)
+    wl.gv[130:170, 4, 77] = -3.0
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert (wl.T_total // 64) * wl.H > 2 * sms and wl.N * wl.H * 128 // 16 > sms   # (16 state columns per block of a carry, per direction)
+    buf = runner.to_device_channelwise(wl, want_o=True)
+    runner.run_bwd_channelwise(buf)
+    got = runner.fetch(buf)
+    errs, ref = check(wl, got)
+    assert max(errs[n] for n in ("dg", "db", "dw", "dh0")) < 1e-5     # fp32 arithmetic: the fall-back did run
+    runner.run_fwd_channelwise(buf)
+    f = runner.fetch(buf)
+    assert rel(f["o"], ref["o"]) < TOL["bf16"] and rel(f["hT"], ref["hT"]) < 1e-5
+    runner.run_bwd_channelwise(buf, fresh=1)
+    fresh = runner.fetch(buf)
+    for n in GRADS:
+        assert np.array_equal(fresh[n], got[n]), n
+
+
 @pytest.mark.parametrize("dtype,d", [("bf16", 128), ("f32", 64)])
 def test_no_tokens_passes_the_state_gradient_through(dtype, d):
     wl = synth.make_channelwise("cw_empty", dtype=dtype, lengths=[0, 0], H=2, d_k=d, d_v=d, states=True, seed=71)
