@@ -19,7 +19,7 @@ struct Rec { Stage s; cudaEvent_t a, b; };
 std::vector<Rec> g_recs;          // recorded since the last read
 std::vector<cudaEvent_t> g_pool;  // reusable events
 cudaEvent_t g_open = nullptr;
-const char* kStageNames[ST_COUNT] = {"table", "prep", "fscan", "out", "eprep", "rscan", "intra", "scans", "scale", "post", "fallback"};
+const char* kStageNames[ST_COUNT] = {"table", "prep", "fscan", "out", "eprep", "rscan", "intra", "scans", "scale", "fallback"};
 cudaEvent_t take_event() {
     if (!g_pool.empty()) { cudaEvent_t e = g_pool.back(); g_pool.pop_back(); return e; }
     cudaEvent_t e = nullptr;
@@ -68,11 +68,10 @@ Path pick_path(const gdn_desc& d) {
 }
 
 WsLayout layout_for(const gdn_desc& d) {
-    // tcgen05 path: every factor, state and additive term of the carries is a bf16 tile image.
     // The d = 128 family keeps the chunk operator Nm and the additive term Bf only when its carries use them.
     // A head dimension of 64 takes the workspace of 128: its tiles are half zero.
-    if (pick_path(d) == Path::TcBf16 || pick_path(d) == Path::TcBf16Padded) return make_layout(tc_padded_desc(d), 2, 2, 0, !tc_carries_lowrank(d));
-    if (pick_path(d) == Path::Tc64Bf16) return make_layout(d, 2, 2, 0);
+    if (pick_path(d) == Path::TcBf16 || pick_path(d) == Path::TcBf16Padded) return make_layout_tc(tc_padded_desc(d), !tc_carries_lowrank(d));
+    if (pick_path(d) == Path::Tc64Bf16) return make_layout_tc(d, true);
     return make_layout_ffma(d);   // the FFMA kernels keep everything in fp32, whatever the I/O dtype
 }
 
@@ -264,8 +263,7 @@ gdn_status gdn_last_device_status(const void* workspace, void* cuda_stream) {
     int32_t word = 0;
     if (cudaMemcpyAsync(&word, workspace, sizeof(word), cudaMemcpyDeviceToHost, st) != cudaSuccess) return GDN_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return GDN_ERR_CUDA;
-    if (word == GDN_OK || word == GDN_ERR_BAD_SEQLENS || word == GDN_ERR_DEVICE_TIMEOUT || word == GDN_ERR_DECAY_RANGE)
-        return (gdn_status)word;
+    if (word == GDN_OK || word == GDN_ERR_BAD_SEQLENS || word == GDN_ERR_DEVICE_TIMEOUT) return (gdn_status)word;
     return GDN_ERR_CUDA;
 }
 

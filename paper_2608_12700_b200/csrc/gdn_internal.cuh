@@ -53,16 +53,13 @@ struct WsLayout {
     size_t img_QKp, img_Km, img_Vt;   // ... of [Q~; K+] (32 KB), K- and V~ (16 KB each)
     int tc_scans;                        // ... and T, P, hc, dhn are bf16 tile images as well (8, 8, 32, 32 KB)
     size_t Kb, U, dU;      // FFMA families (fp32): keys scaled to the chunk end [CH, 64, d_k]; U = U~ - W h and dU [CH, 64, d_v]
-    size_t scratch;        // kernel-private staging, per chunk-head
-    size_t scratch_per_ch; // bytes of scratch per chunk-head
     size_t total;
 };
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// elem = bytes per element of the chunk factors and stored states (T, W, U~, Nm, hc, dhn): 4 on the fp32
-// path, 2 for the bf16 tile images of the tcgen05 path.  elem_add = bytes per element of Bf and E.
-inline WsLayout make_layout(const gdn_desc& d, size_t elem, size_t elem_add, size_t scratch_per_ch, bool with_operator = true) {
+// Layout of the scalar-gate tcgen05 families: every factor, state and additive term of the carries is a bf16 tile image.
+inline WsLayout make_layout_tc(const gdn_desc& d, bool with_operator) {
     WsLayout L{};
     const size_t Ttot = (size_t)d.B * (size_t)d.T;
     L.max_chunks = (int)((Ttot + kC - 1) / kC + (size_t)d.N);
@@ -74,19 +71,17 @@ inline WsLayout make_layout(const gdn_desc& d, size_t elem, size_t elem_add, siz
     L.chunk_tok0 = take(4 * (size_t)L.max_chunks);
     L.chunk_len = take(4 * (size_t)L.max_chunks);
     L.gamma = take(4 * CH * kC);
-    L.Tm = take(elem * CH * kC * kC);
-    L.W = take(elem * CH * kC * d.d_k);
-    L.Ut = take(elem * CH * kC * d.d_v);
-    L.Pm = take(elem * CH * kC * kC);
+    L.Tm = take(2 * CH * kC * kC);
+    L.W = take(2 * CH * kC * d.d_k);
+    L.Ut = take(2 * CH * kC * d.d_v);
+    L.Pm = take(2 * CH * kC * kC);
     L.has_operator = with_operator ? 1 : 0;
-    L.Nm = take(with_operator ? elem * CH * d.d_k * d.d_k : 0);
-    L.Bf = take(with_operator ? elem_add * CH * d.d_k * d.d_v : 0);
-    L.hc = take(elem * CH * d.d_k * d.d_v);
+    L.Nm = take(with_operator ? 2 * CH * d.d_k * d.d_k : 0);
+    L.Bf = take(with_operator ? 2 * CH * d.d_k * d.d_v : 0);
+    L.hc = take(2 * CH * d.d_k * d.d_v);
     L.fwd_end = o;
-    L.E = take(elem_add * CH * d.d_k * d.d_v);
-    L.dhn = take(elem * CH * d.d_k * d.d_v);
-    L.scratch_per_ch = scratch_per_ch;
-    L.scratch = take(scratch_per_ch * CH);
+    L.E = take(2 * CH * d.d_k * d.d_v);
+    L.dhn = take(2 * CH * d.d_k * d.d_v);
     L.total = o;
     return L;
 }
@@ -115,7 +110,7 @@ inline WsLayout make_layout_ffma(const gdn_desc& d) {
     L.E = take(4 * CH * d.d_k * d.d_v);
     L.dhn = take(4 * CH * d.d_k * d.d_v);
     L.dU = take(4 * CH * kC * d.d_v);
-    L.scratch = L.total = o;
+    L.total = o;
     return L;
 }
 
@@ -153,7 +148,7 @@ inline WsLayout make_layout_vec(const gdn_desc& d) {
     L.img_E = take(L.tc_scans ? CH * 32768 : 0);
     L.dhn = take(4 * CH * d.d_k * d.d_v);
     L.dU = take(4 * CH * kC * d.d_v);
-    L.scratch = L.total = o;
+    L.total = o;
     return L;
 }
 
@@ -176,7 +171,7 @@ struct Problem {
 
 // Launch bookkeeping: every kernel launch goes through stage_begin / stage_end so that launches can be
 // counted and, when enabled, timed per stage with CUDA events on the launching stream.
-enum Stage { ST_TABLE = 0, ST_PREP, ST_FSCAN, ST_OUT, ST_EPREP, ST_RSCAN, ST_INTRA, ST_SCANS, ST_SCALE, ST_POST, ST_FALLBACK, ST_COUNT };
+enum Stage { ST_TABLE = 0, ST_PREP, ST_FSCAN, ST_OUT, ST_EPREP, ST_RSCAN, ST_INTRA, ST_SCANS, ST_SCALE, ST_FALLBACK, ST_COUNT };
 void stage_begin(Stage s, cudaStream_t st);
 void stage_end(Stage s, cudaStream_t st);
 struct StageScope {

@@ -42,12 +42,6 @@ __device__ __forceinline__ void ld8s(const float* p, float* v) {
     *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(p);
     *reinterpret_cast<float4*>(v + 4) = *reinterpret_cast<const float4*>(p + 4);
 }
-__device__ __forceinline__ float tile_get(const unsigned char* tile, int R, int r, int c) {
-    return __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(tile + tile_off(R, r, c)));
-}
-__device__ __forceinline__ void tile_put(unsigned char* tile, int R, int r, int c, float x) {
-    *reinterpret_cast<__nv_bfloat16*>(tile + tile_off(R, r, c)) = __float2bfloat16_rn(x);
-}
 
 // Zero rows [row0 + len, row0 + 64) of a tile with R rows and 128 columns (threads 0 .. nthr-1 of the CTA take part).
 __device__ __forceinline__ void zero_tail_rows(unsigned char* tile, int R, int row0, int len, int nthr) {
@@ -64,32 +58,6 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-// Each lane holds 8 values (one per token of a group of 8); returns, on every lane, the sum over the 32 lanes of
-// the value belonging to token (lane % 8).  Fixed order: bit-identical from run to run.
-__device__ __forceinline__ float reduce8(float (&v)[8], int lane) {
-    bool up = (lane & 4) != 0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float send = up ? v[k] : v[k + 4], keep = up ? v[k + 4] : v[k];
-        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-    }
-    up = (lane & 2) != 0;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const float send = up ? v[k] : v[k + 2], keep = up ? v[k + 2] : v[k];
-        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-    }
-    up = (lane & 1) != 0;
-    {
-        const float send = up ? v[0] : v[1], keep = up ? v[1] : v[0];
-        v[0] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
-    }
-    float r = v[0];
-    r += __shfl_xor_sync(0xffffffffu, r, 8);
-    r += __shfl_xor_sync(0xffffffffu, r, 16);
-    return r;
 }
 
 // Copy the first `d` features of a staged [64 tokens][128 features] bf16 tile to a [T, H, d] tensor with 16-byte stores (rows

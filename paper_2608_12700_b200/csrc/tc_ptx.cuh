@@ -17,10 +17,6 @@ namespace tc {
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // ---------------------------------------------------------------- tile addressing
-// Byte offset of element (r, c) inside a tile with R rows.
-__device__ __forceinline__ uint32_t tile_off(int R, int r, int c) {
-    return (uint32_t)((c >> 6) * R * 128 + r * 128 + ((((c & 63) >> 3) ^ (r & 7)) << 4) + ((c & 7) << 1));
-}
 // Byte offset of the 16-byte chunk holding columns [8*ch, 8*ch + 8) of row r.
 __device__ __forceinline__ uint32_t tile_chunk_off(int R, int r, int ch) {
     return (uint32_t)((ch >> 3) * R * 128 + r * 128 + (((ch & 7) ^ (r & 7)) << 4));
@@ -150,8 +146,6 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 // Wait until at most N of this thread's bulk groups still read their shared-memory source.
 template <int N>
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
-template <int N>
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group %0;" ::"n"(N) : "memory"); }
 
 // ---------------------------------------------------------------- tensor memory
 // One warp allocates `cols` (power of two >= 32) columns; the base address is written to *slot (shared).
