@@ -1793,9 +1793,10 @@ static cudaError_t launch_eprep(const TcParams& P, cudaStream_t st) {
 }
 
 static cudaError_t launch_prep_lr(const TcParams& P, cudaStream_t st) {
-    static SmemLimitOnce done;
-    const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count();
-    return launch_chunk_kernel(tc_prep_lr_kernel, done, preplr::SMEM_BYTES, ST_PREP, items < ctas ? items : ctas, split::kT, P, st);
+    static SmemLimitOnce done, done_fwd;
+    const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count(), grid = items < ctas ? items : ctas;
+    return P.with_bwd ? launch_chunk_kernel(tc_prep_lr_kernel<true>, done, preplr::SMEM_BYTES, ST_PREP, grid, split::kT, P, st)
+                      : launch_chunk_kernel(tc_prep_lr_kernel<false>, done_fwd, preplr::SMEM_BYTES, ST_PREP, grid, split::kT, P, st);
 }
 
 static cudaError_t launch_scan(const TcParams& P, cudaStream_t st) {

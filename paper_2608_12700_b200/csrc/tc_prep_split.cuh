@@ -177,6 +177,8 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
 // Against one CTA per SM with sixteen readout warps, a loader and an issuer warp (the form tc_prep still has), two CTAs fill each
 // other's waits: 4 x 16 heads of 2048 tokens 94 -> 77 us (both bound by the chain of dependent phases of a chunk-head), 32 heads
 // of 32768 packed tokens 695 -> 564 us (144 KB of traffic per chunk-head at 4.2 TB/s).
+// The forward has an instance of its own: without the backward's part of the readouts gdn_fwd_recompute takes 1.2 us less (4 x 16
+// heads of 2048 tokens, no output: 123.9 -> 122.6 us).
 // P is the forward's to make, although only its output and the backward use it: Q K^T rides along with K K^T in one M = 128
 // product, and neither of those has to load K and wait for a product of its own (tc_out, tc_eprep).
 // ------------------------------------------------------------------------------------------------
@@ -195,6 +197,7 @@ static_assert(TPP + 8192 <= PT && ES + 32768 <= PT && PT % 1024 == 0, "T tiles a
 static_assert(2 * (SMEM_BYTES + 4096) <= 228 * 1024, "two CTAs per SM");
 }  // namespace preplr
 
+template <bool bwd>   // with the backward's share
 __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_constant__ TcParams P) {
     wait_prerequisites();
     using namespace preplr;
@@ -222,7 +225,6 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
     float* Af = reinterpret_cast<float*>(sm + XA);
     float* Tf = reinterpret_cast<float*>(sm + XT);
     const float sc = p.d.scale;
-    const bool bwd = P.with_bwd != 0;
     bool ok = true, pending = false;
     uint32_t mma_phase = 0, in_phase = 0;
     // Every input tile of a trip is dead once its last product is done: the next trip's are loaded right then, under the
@@ -384,7 +386,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
                 float a[8], b[8], c[8];
                 tmem_ld8(tmem + lane_base + C_W + ib, a);
                 tmem_ld8(tmem + lane_base + C_U + ib, b);
-                tmem_ld8(tmem + lane_base + C_PDO + ib, c);
+                if (bwd) tmem_ld8(tmem + lane_base + C_PDO + ib, c);
                 tmem_wait_ld();
                 chunk_store(sm + WT, 128, f, ib >> 3, a);
                 chunk_store(ut, 64, f & 63, ib >> 3, b);
