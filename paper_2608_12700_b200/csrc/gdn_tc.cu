@@ -986,15 +986,15 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_cw_kernel(const __grid_co
 // instruction issue; HBM needs 10 k of the cycles.  The forms of the products follow from that:
 // * Phase 1 is transposed (features on TMEM lanes) because its results feed later products.
 // * The two pairs of products with a common second operand, dO h^T with dXv h^T and dPD K with G K, are stacked along M: one
-//   instruction of M = 128 costs little more than one of M = 64 (97 against 86 cycles at N = 128), and the last readout finds a
+//   instruction of M = 128 costs what one of M = 64 does (66 cycles at N = 128), and the last readout finds a
 //   token of dq on each of lanes 0..63 and one of dk on each of lanes 64..127, where 64-row accumulators would leave half of
 //   the lanes of every warp idle.  The two products of dk^col are issued with M = 128 as well, their A operand shifted by one
 //   64-column block so that the 64 rows that count land on lanes 64..127, beside the other half of dk (the rows on lanes
 //   0..63 are made from whatever lies there and are never read).
 // * T^T dU is issued as two 64-column halves, one on lanes 0..15 and one on lanes 16..31 of each quadrant.
-// Measured on 4 x 16 heads of 2048 tokens (2048 chunk-heads): 108 us, 13.5 k cycles per chunk-head; with separate M = 64
-// products, gate gradients finished by two of the readout warps and dq assembled in a readout of its own it was 142 us (17.7 k).
-// 8 packed sequences, 32768 tokens, 32 heads: 971 -> 757 us.
+// Measured on 4 x 16 heads of 2048 tokens (2048 chunk-heads): 116 us, 14.7 k cycles per chunk-head; with separate M = 64
+// products, gate gradients finished by two of the readout warps and dq assembled in a readout of its own it was 144 us.
+// 8 packed sequences, 32768 tokens, 32 heads: 971 -> 763 us.
 // ------------------------------------------------------------------------------------------------
 namespace intra {
 constexpr uint32_t OX = 0;                 // rows 0..63 dO, rows 64..127 dXv  x 128            32 KB
@@ -1546,7 +1546,7 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
 // ------------------------------------------------------------------------------------------------
 // tc_out (optional forward output): o = scale (Diag(Gam) Q h + P (U~ - W h)),  P = tril(Q K^T . D)
 //
-// Persistent, two CTAs per SM (96 KB of shared memory, 256 TMEM columns each): a CTA walks through the dependent
+// Persistent, two CTAs per SM (89 KB of shared memory, 256 TMEM columns each): a CTA walks through the dependent
 // steps of one chunk-head while its neighbour is in another step of another one.  The tiles of the next trip are
 // loaded as soon as the last product (or store) that reads their region is done.  Q h and P U are formed token-major
 // (M = 64: a thread owns a token row), so the output tile is staged with 16-byte stores and leaves by TMA.
@@ -1733,10 +1733,12 @@ bool tc_supported(const gdn_desc& d) {
 thread_local int g_inject_timeout = 0;   // set by gdn_debug_inject_timeout, consumed by the next gdn_bwd of this family
 
 static int sm_count();
-// When one CTA per (chain, direction) of the backward fills more than half of the SMs the carries are bound by HBM
-// bandwidth, and the low-rank form moves less.  With fewer chains a step's latency counts, and the operator form needs one
-// product per step.  The rule looks at the chains only, so the forward, the backward and a backward on a workspace fresh
-// from the forward agree on the form (and on the workspace layout that follows from it).
+// Up to 37 chains (on 148 SMs) the operator form gives each direction of a chain two CTAs, and its one product per step wins; from
+// 38 on it would have one, and the low-rank form moves less.  Backward, us, operator / low-rank: 4 chains of 6 chunks 32.1 / 38.4,
+// 16 of 256 606 / 739, 37 of 32 172.7 / 175.0; 38 of 32 198.2 / 184.7, 64 of 32 290 / 260, 64 of 256 2270 / 1948; the line lies
+// there from 1 chunk to 256.  (A forward with its output and the backward on its workspace, each with one direction per launch,
+// would change sides near 64 chains: 38 of 32 250 / 266.)  The rule looks at the chains only, so the forward, the backward and
+// a backward on a workspace fresh from the forward agree on the form (and on the workspace layout that follows from it).
 bool tc_carries_lowrank(const gdn_desc& d) {
     if (g_force_carries) return g_force_carries == 2;
     return 4 * (long long)d.N * d.H > sm_count();

@@ -511,7 +511,7 @@ __global__ void __launch_bounds__(kT, 2) cw_eprep_kernel(const __grid_constant__
 // gradients are then whole 128-byte lines, all lanes work (a 64-row accumulator fills half of them), and the sums of dg
 // over the tokens of a chunk run along a thread's own columns.  So nothing passes through HBM between the products and the
 // elementwise part: with fp32 scratch and a kernel of its own (256 KB more traffic per chunk-head) the two took 300 us on
-// 4 x 16 heads of 2048 tokens, this kernel 208 us.
+// 4 x 16 heads of 2048 tokens, this kernel 211 us.
 // (L2 prefetches of what the elementwise part reads, a trip ahead, made it slower: 481 -> 495 us for the call.)
 // ------------------------------------------------------------------------------------------------
 namespace intracw {

@@ -175,8 +175,8 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
 // tc_prep_lr: gamma, P = tril(Q K^T . D), T = (I + A)^-1, W^T, U~^T and, for a backward that recomputes the forward,
 // E = scale (Diag(Gam) Q - P W)^T dO.
 // Against one CTA per SM with sixteen readout warps, a loader and an issuer warp (the form tc_prep still has), two CTAs fill each
-// other's waits: 4 x 16 heads of 2048 tokens 94 -> 77 us (both bound by the chain of dependent phases of a chunk-head), 32 heads
-// of 32768 packed tokens 695 -> 564 us (144 KB of traffic per chunk-head at 4.2 TB/s).
+// other's waits: 4 x 16 heads of 2048 tokens 98 -> 79 us (both bound by the chain of dependent phases of a chunk-head), 32 heads
+// of 32768 packed tokens 695 -> 562 us (144 KB of traffic per chunk-head at 4.2 TB/s).
 // The forward has an instance of its own: without the backward's part of the readouts gdn_fwd_recompute takes 1.2 us less (4 x 16
 // heads of 2048 tokens, no output: 123.9 -> 122.6 us).
 // P is the forward's to make, although only its output and the backward use it: Q K^T rides along with K K^T in one M = 128

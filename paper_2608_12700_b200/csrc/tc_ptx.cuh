@@ -238,9 +238,8 @@ __device__ __forceinline__ void mma_issue(uint32_t tmem_d, uint64_t adesc, uint6
         : "memory");
 }
 // Products are issued by one elected lane of a warp, under a condition that the compiler can see is uniform for the warp:
-// if (warp_id() == w && elect_one()).  Descriptors then live in uniform registers, where the instruction wants them, and an
-// M64 x N64 instruction costs 34 cycles instead of 47 (issued behind threadIdx.x == 0 each of them moves its descriptors there
-// first; larger shapes are bound by the pipe either way, but the issuer needs fewer of the slots that the readout warps want).
+// if (warp_id() == w && elect_one()).  An M64 x N64 instruction then costs 34 cycles, against 47 behind threadIdx.x == 0; larger
+// shapes take the same time either way.
 // All 32 lanes have to reach elect_one() together; it always elects the same one.  Whole calls: 8 x 32 heads of 4096 tokens of
 // the scalar-gate recurrence 481 -> 462 us, 4 heads of 640 tokens of it 64 -> 58 us, 6 x 16 x 1500 forward and backward
 // 372 -> 370 us.  (tc_intra keeps threadIdx.x: the uniform warp index cost it registers it does not have, 64 bytes of spills.)
@@ -251,7 +250,7 @@ __device__ __forceinline__ bool elect_one() {
     return p != 0;
 }
 // D[M x N] (+)= A[M x Kt] * B[Kt x N]: one thread issues Kt / 16 instructions, fully unrolled so that each costs two
-// integer adds besides the tcgen05.mma itself (the tensor pipe accepts one such instruction every ~50-60 cycles).
+// integer adds besides the tcgen05.mma itself (which takes 34 cycles at M64 x N64, 50 at M128 x N64, 66 at N128, 130 at M128 x N256).
 template <int M, int N, int Kt>
 __device__ __forceinline__ void mma_tile(uint32_t tmem_d, const Operand& a, const Operand& b, bool accumulate, bool neg_a = false) {
     const uint32_t idesc = make_idesc(M, N, a.mn_major, b.mn_major, neg_a);
