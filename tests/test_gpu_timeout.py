@@ -1,6 +1,6 @@
 """Failure detection on the device: every wait in the kernels is bounded, and a wait that runs out is reported
 through the workspace's status word instead of hanging or trapping.  The test makes one wait run out on the host's
-terms (a debugging hook shortens the limit to a millisecond for one call and has the first kernel leave out one of
+terms (a debugging hook shortens the limit to a millisecond for one call and has one of the kernels leave out one of
 its loads); nothing faults, and the same buffers give correct gradients on the next call."""
 import numpy as np
 import pytest
