@@ -156,16 +156,16 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
     __syncthreads();
     bool ok = true;
     uint32_t mma_phase = 0;
-    int s = 0;
+    auto give_up = [&](int s) { if (threadIdx.x == 0) drain_ring<STAGES>(bar_full, s, nsteps); };
 #pragma unroll 1
-    for (; s < nsteps; ++s) {
+    for (int s = 0; s < nsteps; ++s) {
         const int c = c0 + s, stage = s % STAGES, len = cg.chunk_len(c);
         const size_t ch = (size_t)c * H + hd;
         unsigned char* tiles = sm + stage * STAGE_BYTES;
         unsigned char* HT = sm + C::HT + (s & 1) * 8192;
         const float *gl = gl2[s & 1], *Gam = Gam2[s & 1], *ee = ee2[s & 1];
         ok = mbar_wait(&bar_full[stage], (s / STAGES) & 1);
-        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 40); break; }
+        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 40); give_up(s); break; }
         if (len < kC) {
             zero_tail_rows64(tiles + KT, len);
             zero_tail_rows64(tiles + VT, len);
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
             mma_commit(&bar_mma);
         }
         GDN_WAIT_MMA(41)
-        if (!ok) break;
+        if (!ok) { give_up(s); break; }
         // without o the slot's K and V have now been read for the last time: refill it while the state is updated
         if (!O && threadIdx.x == 96 && s + STAGES < nsteps) fill(s + STAGES);
         if (O) {   // o = scale (Gam_i (Q h)_i + (P V)_i)
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
                 mma_commit(&bar_mma);
             }
             GDN_WAIT_MMA(42)
-            if (!ok) break;
+            if (!ok) { give_up(s); break; }
             __nv_bfloat16* go = reinterpret_cast<__nv_bfloat16*>(p.o) + ((size_t)(cg.chunk_tok0(c) + r) * H + hd) * D6;
 #pragma unroll 1
             for (int part = 0; part < 4; ++part) {
@@ -266,7 +266,6 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
         }
     }
     if (warp == 0) bulk_wait_read<0>();
-    if (threadIdx.x == 0) drain_ring<STAGES>(bar_full, s, nsteps);
     if (p.hT && ok) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) *reinterpret_cast<float4*>(p.hT + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
