@@ -711,6 +711,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     const int H = p.d.H, n = chain / H, hd = chain % H;
     const SeqGeom sg = seq_geom(p, n);
     const int c0 = sg.c0, nsteps = sg.n_chunks, c1 = c0 + nsteps;
+    auto chunk_of = [&](int s) { return reverse ? (c1 - 1 - s) : (c0 + s); };
 
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sm = align1024(smem_raw);
@@ -724,6 +725,18 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     const int r1 = S == 1 ? r : q4 * 16 + (lane & 15);
     const bool act1 = S == 1 || lane < 16;
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
+    // channel-wise: log decay over the chunk and reference of this thread's state row, fetched a step ahead
+    struct { float gam; int ref; } cw_next{0.f, 0};
+    auto cw_fetch = [&](int s) {
+        if (CW && s < nsteps) {
+            const size_t ch = (size_t)chunk_of(s) * H + hd;
+            cw_next.gam = reinterpret_cast<const float*>(p.ws + p.L.gamma)[(ch * kC + kC - 1) * D + r];
+            cw_next.ref = reinterpret_cast<const int32_t*>(p.ws + p.L.ref)[ch * D + r];
+        } else {
+            cw_next.ref = 0;
+        }
+    };
+    cw_fetch(0);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) mbar_init(&bar_full[s], 1);
@@ -736,7 +749,6 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
-    auto chunk_of = [&](int s) { return reverse ? (c1 - 1 - s) : (c0 + s); };
     const char* w_base = p.ws + (CW ? p.L.img_W : p.L.W);
     // this CTA's part of the additive image: rows part * NS.. of U~^T [d_v][tokens], column block `part` of E [d_k][d_v]
     const uint32_t x_chunk = reverse ? 32768u : 16384u, x_bytes = x_chunk / S;
@@ -786,22 +798,11 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     __syncthreads();
     bool ok = true;
     uint32_t mma_phase = 0;
-    // channel-wise: log decay over the chunk and reference of this thread's state row, fetched a step ahead
-    float cw_gam = 0.f;
-    int cw_ref = 0;
-    auto cw_fetch = [&](int s) {
-        const size_t ch = (size_t)chunk_of(s) * H + hd;
-        cw_gam = gamma[(ch * kC + kC - 1) * D + r];
-        cw_ref = reinterpret_cast<const int32_t*>(p.ws + p.L.ref)[ch * D + r];
-    };
-    int ref_prev = 0;   // (reverse)
-    if (CW && nsteps > 0) {
-        cw_fetch(0);
-        if (!reverse) {
-            const float S_ref = pow2(cw_ref);
+    int cw_ref = 0;   // reverse: reference of the step before
+    if (CW && !reverse) {
+        const float S_ref = pow2(cw_next.ref);
 #pragma unroll
-            for (int k = 0; k < NSH; ++k) st[k] *= S_ref;
-        }
+        for (int k = 0; k < NSH; ++k) st[k] *= S_ref;
     }
     int s = 0;
 #pragma unroll 1
@@ -812,13 +813,10 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         unsigned char* ring = sm + stage * STAGE_BYTES;
         const float* ee = ee2[s & 1];
         // decay of the state over the chunk: a scalar, or (channel-wise) the factor of this thread's state row
-        float Ge = CW ? expf(cw_gam) : (s < GE_CAP ? ge[s] : expf(gamma[ch * kC + kC - 1]));
-        const int ref = cw_ref;
-        if (CW && reverse) { Ge *= pow2(ref_prev - ref); ref_prev = ref; }   // A
-        if (CW) {
-            if (s + 1 < nsteps) cw_fetch(s + 1);
-            else cw_ref = 0;
-        }
+        float Ge = CW ? expf(cw_next.gam) : (s < GE_CAP ? ge[s] : expf(gamma[ch * kC + kC - 1]));
+        const int ref = cw_next.ref;
+        if (CW && reverse) { Ge *= pow2(cw_ref - ref); cw_ref = ref; }   // A
+        if (CW) cw_fetch(s + 1);
         // state -> bf16: operand of the first product, and the per-chunk state the gradient stage reads
 #pragma unroll
         for (int k = 0; k < NSH / 8; ++k) {
@@ -893,7 +891,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         mma_phase ^= 1;
         if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 13); break; }
         tc_fence_after();
-        if (CW && !reverse) Ge *= pow2(cw_ref - ref);   // A
+        if (CW && !reverse) Ge *= pow2(cw_next.ref - ref);   // A
 #pragma unroll
         for (int k = 0; k < NSH / 8; ++k) {
             float d2[8], ad[8];
@@ -910,7 +908,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     }
     float* fin = reverse ? p.dh0 : p.hT;
     if (CW && reverse) {
-        const float S_ref = pow2(ref_prev);
+        const float S_ref = pow2(cw_ref);
 #pragma unroll
         for (int k = 0; k < NSH; ++k) st[k] *= S_ref;
     }
