@@ -61,7 +61,8 @@ __device__ __forceinline__ ChunkGeom chunk_geom(const Problem& p) {
     return g;
 }
 // One sequence, for the kernels that walk along it: its chunks are consecutive, each starts 64 tokens after the one
-// before, only the last can be short.  (cu_seqlens has been validated by the table kernel by the time it is read here.)
+// before, only the last can be short.  (Packed sequences: from the table, never from the caller's cu_seqlens, which in a backward on
+// the forward's workspace may no longer be what they were.)
 struct SeqGeom {
     int c0, n_chunks, tok0, len;   // first chunk, number of chunks, first token, tokens
     __device__ __forceinline__ int chunk_tok0(int c) const { return tok0 + (c - c0) * kC; }
@@ -69,9 +70,10 @@ struct SeqGeom {
 };
 __device__ __forceinline__ SeqGeom seq_geom(const Problem& p, int n) {
     SeqGeom g;
-    if (p.cu) {
-        g.tok0 = p.cu[n];
-        g.len = p.cu[n + 1] - g.tok0;
+    if (p.cu && p.Ttot > 0) {
+        const int32_t* tok0 = reinterpret_cast<const int32_t*>(p.ws + p.L.seq_tok0);
+        g.tok0 = tok0[n];
+        g.len = tok0[n + 1] - g.tok0;
         g.c0 = reinterpret_cast<const int32_t*>(p.ws + p.L.seq_first)[n];
     } else {
         g.tok0 = n * p.d.T;
@@ -94,6 +96,27 @@ __device__ __forceinline__ void init_header_if_untabled(const Problem& p) {
         hdr->status = GDN_OK;
         hdr->n_chunks = n_chunks_of(p);
         hdr->detail = 0;
+        hdr->seqlens_ok = 1;
+    }
+}
+// Called by all threads at the top of the first kernel of a backward on the forward's workspace, in the families that do not build
+// the table again: the cu_seqlens have to be the forward's.  One block looks, the last one, which has no chunk to work on in a grid
+// of max_chunks x heads (the bound allows one chunk more than there can be); the others work from the table meanwhile, and the kernels
+// behind, which write the outputs, see the status.  (As a launch of the table kernel ahead of it the check took 2.5 us.)
+__device__ __forceinline__ bool status_from_fresh(const WsHeader* hdr) { return hdr->status == GDN_ERR_BAD_SEQLENS && hdr->seqlens_ok; }
+__device__ __forceinline__ void check_fresh_seqlens(const Problem& p) {
+    if (!p.cu || blockIdx.x != gridDim.x - 1) return;
+    const int32_t* tok0 = reinterpret_cast<const int32_t*>(p.ws + p.L.seq_tok0);
+    int same = 1, at = p.d.N;
+    for (int n = threadIdx.x; n <= p.d.N; n += blockDim.x)
+        if (p.cu[n] != (p.Ttot > 0 ? tok0[n] : 0)) { same = 0; at = n; }
+    const int all = __syncthreads_and(same);
+    WsHeader* hdr = reinterpret_cast<WsHeader*>(p.ws);
+    if (all ? threadIdx.x == 0 : !same) {   // (several threads may find a difference: any of them will do)
+        if (hdr->status == GDN_OK || status_from_fresh(hdr)) {
+            hdr->status = all ? GDN_OK : GDN_ERR_BAD_SEQLENS;
+            hdr->detail = all ? 0 : at;
+        }
     }
 }
 

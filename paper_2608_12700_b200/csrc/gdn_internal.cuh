@@ -22,8 +22,8 @@ struct WsHeader {
                            // stage, cleared by the table kernel of a call that does not consume a forward's workspace).  The
                            // tensor-core kernels then stand down and the FFMA kernels enqueued behind them compute the call, and
                            // the backward on the workspace of such a forward.
-    int32_t fresh_refused;   // 1 if a status of GDN_ERR_BAD_SEQLENS comes from a backward on the forward's workspace, not from the
-                             // forward: the forward's data is whole, and the next such backward may have better cu_seqlens
+    int32_t seqlens_ok;    // 1 if the sequences that the workspace was filled for were valid: a status of GDN_ERR_BAD_SEQLENS then comes from a
+                           // backward on the forward's workspace, whose data is whole, and the next such backward may have better ones
     int32_t pad[59];
 };
 static_assert(sizeof(WsHeader) == 256, "header size");
@@ -32,7 +32,8 @@ static_assert(sizeof(WsHeader) == 256, "header size");
 struct WsLayout {
     int max_chunks;        // bound on the number of chunks: sum over sequences of ceil(len/64) <= ceil(T_total/64) + N
     size_t seq_first;      // int32 [N + 1]   first chunk index of each sequence
-    size_t chunk_seq;      // int32 [max_chunks]
+    size_t seq_tok0;       // int32 [N + 1]   first token of each sequence: cu_seqlens as validated (no tokens: not written; the region has
+                           //                 room for max_chunks entries, which is N then)
     size_t chunk_tok0;     // int32 [max_chunks]   global token index of the chunk's first row
     size_t chunk_len;      // int32 [max_chunks]   valid rows (1..64)
     size_t gamma;          // f32 [CH, 64]         chunk-local cumulative log decay (channel-wise calls: [CH, 64, d_k])
@@ -67,7 +68,7 @@ inline WsLayout make_layout_tc(const gdn_desc& d, bool with_operator) {
     size_t o = sizeof(WsHeader);
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
     L.seq_first = take(4 * ((size_t)d.N + 1));
-    L.chunk_seq = take(4 * (size_t)L.max_chunks);
+    L.seq_tok0 = take(4 * (size_t)L.max_chunks);
     L.chunk_tok0 = take(4 * (size_t)L.max_chunks);
     L.chunk_len = take(4 * (size_t)L.max_chunks);
     L.gamma = take(4 * CH * kC);
@@ -95,7 +96,7 @@ inline WsLayout make_layout_ffma(const gdn_desc& d) {
     size_t o = sizeof(WsHeader);
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
     L.seq_first = take(4 * ((size_t)d.N + 1));
-    L.chunk_seq = take(4 * (size_t)L.max_chunks);
+    L.seq_tok0 = take(4 * (size_t)L.max_chunks);
     L.chunk_tok0 = take(4 * (size_t)L.max_chunks);
     L.chunk_len = take(4 * (size_t)L.max_chunks);
     L.gamma = take(4 * CH * kC);
@@ -125,7 +126,7 @@ inline WsLayout make_layout_vec(const gdn_desc& d) {
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
     L.tc_scans = vec_tc_scans(d) ? 1 : 0;
     L.seq_first = take(4 * ((size_t)d.N + 1));
-    L.chunk_seq = take(4 * (size_t)L.max_chunks);
+    L.seq_tok0 = take(4 * (size_t)L.max_chunks);
     L.chunk_tok0 = take(4 * (size_t)L.max_chunks);
     L.chunk_len = take(4 * (size_t)L.max_chunks);
     L.gamma = take(4 * CH * kC * d.d_k);
@@ -231,8 +232,8 @@ gdn_status check_bwd_args(const gdn_desc* desc, const void* q, const void* k, co
 
 // Kernel families (each defined in its own translation unit).  They enqueue on `st` and return the
 // first CUDA error seen.
-// Chunk table of a call with packed sequences (or without tokens); it validates cu_seqlens, so it runs in every such call, ahead
-// of whatever reads them.  `fresh`: the workspace is the forward's, whose status and fall-back words stay as they are.
+// Chunk table of a call with packed sequences (or without tokens).  It validates cu_seqlens; nothing else reads them but
+// check_fresh_seqlens.  `fresh`: the workspace is the forward's, whose status and fall-back words stay as they are.
 cudaError_t launch_table(const Problem& p, cudaStream_t st, bool fresh = false);
 cudaError_t simt_launch_fwd(const Problem& p, cudaStream_t st);
 cudaError_t simt_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st);

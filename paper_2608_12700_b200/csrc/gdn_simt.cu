@@ -31,13 +31,16 @@ __global__ void table_kernel(Problem p, int fresh) {
     wait_prerequisites();
     WsHeader* hdr = reinterpret_cast<WsHeader*>(p.ws);
     int32_t* seq_first = reinterpret_cast<int32_t*>(p.ws + p.L.seq_first);
-    int32_t* chunk_seq = reinterpret_cast<int32_t*>(p.ws + p.L.chunk_seq);
+    int32_t* seq_tok0 = reinterpret_cast<int32_t*>(p.ws + p.L.seq_tok0);
     int32_t* chunk_tok0 = reinterpret_cast<int32_t*>(p.ws + p.L.chunk_tok0);
     int32_t* chunk_len = reinterpret_cast<int32_t*>(p.ws + p.L.chunk_len);
     const int N = p.d.N;
     __shared__ int ok;
     auto cu = [&](int n) -> long long { return p.cu ? (long long)p.cu[n] : (long long)n * p.d.T; };
-    if (threadIdx.x == 0 && fresh && hdr->status != GDN_OK && !(hdr->status == GDN_ERR_BAD_SEQLENS && hdr->fresh_refused)) {
+    // (all threads: the loads of the one that goes through the sequences below then find them in the cache)
+    if (p.Ttot > 0)
+        for (int n = threadIdx.x; n <= N; n += blockDim.x) seq_tok0[n] = (int)cu(n);
+    if (threadIdx.x == 0 && fresh && hdr->status != GDN_OK && !status_from_fresh(hdr)) {
         ok = 0;
     } else if (threadIdx.x == 0) {
         int good = 1, bad_at = -1;
@@ -51,7 +54,7 @@ __global__ void table_kernel(Problem p, int fresh) {
         }
         if (good && cu(N) != p.Ttot) { good = 0; bad_at = N; }
         if (!fresh) hdr->cw_fallback = 0;
-        hdr->fresh_refused = fresh && !good;
+        if (!fresh) hdr->seqlens_ok = good;
         if (good) {
             seq_first[N] = acc;
             hdr->status = GDN_OK;
@@ -77,7 +80,6 @@ __global__ void table_kernel(Problem p, int fresh) {
         const int n = lo;
         const long long a = cu(n), e = cu(n + 1);
         const long long t0 = a + (long long)(c - seq_first[n]) * kC;
-        chunk_seq[c] = n;
         chunk_tok0[c] = (int)t0;
         chunk_len[c] = (int)((e - t0) < kC ? (e - t0) : kC);
     }
@@ -142,7 +144,7 @@ template <typename IO, int DK, int DV>
 __global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) {
     wait_prerequisites();
     const bool fwd = mode != PREP_BWD, bwd = mode != PREP_FWD;
-    if (fwd) init_header_if_untabled(p);   // (the backward's part alone: the status word is the forward's)
+    if (fwd) init_header_if_untabled(p); else check_fresh_seqlens(p);   // (the backward's part alone: the status word is the forward's)
     ChunkInfo x;
     if (!chunk_info(p, x)) return;   // (no chunk at all when the table was refused)
     constexpr int PK = pitch(DK), PV = pitch(DV);
@@ -602,7 +604,7 @@ cudaError_t launch_fwd_t(const Problem& p, cudaStream_t st) {
 template <typename IO, int DK, int DV>
 cudaError_t launch_bwd_t(const Problem& p, bool skip_recompute, cudaStream_t st) {
     cudaError_t e;
-    if (p.cu && (e = launch_table(p, st, skip_recompute)) != cudaSuccess) return e;
+    if (p.cu && !skip_recompute && (e = launch_table(p, st)) != cudaSuccess) return e;
     if ((e = launch_prep_t<IO, DK, DV>(p, skip_recompute ? PREP_BWD : PREP_FWD_BWD, st)) != cudaSuccess) return e;
     if ((e = launch_scan_t<DK, DV>(p, skip_recompute ? 1 : 2, st)) != cudaSuccess) return e;
     static SmemLimitOnce once;

@@ -297,7 +297,8 @@ template <typename IO, int DK, int DV>
 __global__ void __launch_bounds__(kThreads, 1) vprep_kernel(Problem p, int mode) {
     wait_prerequisites();
     if (p.fallback) { if (!vec_go(p)) return; }
-    else if (mode != PREP_BWD) init_header_if_untabled(p);   // (the backward's part alone: the status word is the forward's)
+    else if (mode != PREP_BWD) init_header_if_untabled(p);
+    else check_fresh_seqlens(p);   // (the backward's part alone: the status word is the forward's)
     for_chunks(p, [&](const ChunkInfo& x) { vprep_chunk<IO, DK, DV>(p, mode, x); });
 }
 
@@ -671,7 +672,7 @@ cudaError_t ffma_fwd(const Problem& q, cudaStream_t st) {
 template <typename IO, int DK, int DV>
 cudaError_t ffma_bwd(const Problem& q, bool skip_recompute, cudaStream_t st) {
     cudaError_t e;
-    if (q.cu && !q.fallback && (e = launch_table(q, st, skip_recompute)) != cudaSuccess) return e;
+    if (q.cu && !q.fallback && !skip_recompute && (e = launch_table(q, st)) != cudaSuccess) return e;
     if ((e = launch_vprep<IO, DK, DV>(q, skip_recompute ? PREP_BWD : PREP_FWD_BWD, st)) != cudaSuccess) return e;
     if ((e = launch_vscan<DK, DV>(q, skip_recompute ? 1 : 2, st)) != cudaSuccess) return e;
     static SmemLimitOnce once;

@@ -392,7 +392,10 @@ __global__ void __launch_bounds__(kT, 2) cw_eprep_kernel(const __grid_constant__
     const Problem& p = P.p;
     const int H = p.d.H;
     const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
-    if (!cw_go(hdr)) return;
+    check_fresh_seqlens(p);
+    // (its verdict may come at any moment and concerns the kernels behind this one: either status is a go here, for every thread)
+    const int32_t status = hdr->status;
+    if (!(status == GDN_OK || (status == GDN_ERR_BAD_SEQLENS && hdr->seqlens_ok)) || hdr->cw_fallback) return;
     const int n_items = hdr->n_chunks * H;
     if ((int)blockIdx.x >= n_items) return;
     extern __shared__ unsigned char smem_raw[];
@@ -874,8 +877,8 @@ cudaError_t cw_tc_launch(const Problem& p, bool bwd, bool skip_recompute, cudaSt
     static SmemLimitOnce once_scale, once_prep, once_eprep, once_intra;
     const int CH = p.L.max_chunks * p.d.H, chains = p.d.N * p.d.H;
     cudaError_t e;
-    const bool fresh = bwd && skip_recompute;   // the images, gam and the factors are still there
-    if ((!fresh || p.cu) && (e = launch_table(p, st, fresh)) != cudaSuccess) return e;
+    const bool fresh = bwd && skip_recompute;   // the chunk table, the images, gam and the factors are still there
+    if ((!fresh || p.Ttot == 0) && (e = launch_table(p, st, fresh)) != cudaSuccess) return e;
     const int sms = tc_sm_count(), grid = CH < sms ? CH : sms, grid2 = CH < 2 * sms ? CH : 2 * sms;
     CwParams P;
     P.p = p;

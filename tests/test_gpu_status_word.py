@@ -75,7 +75,10 @@ def test_malformed_cu_seqlens_are_refused_on_a_forwards_workspace(family):
         bwd()
         assert binding.gdn_last_device_status(buf.workspace) == BAD_SEQLENS
         assert_unwritten(buf)
-    # the forward's data is whole: with its own cu_seqlens the backward runs, and as if nothing had happened
+    # the forward's data is whole: with its own cu_seqlens the backward runs (twice: after a refusal, and after a good call), and as if
+    # nothing had happened
+    buf.inputs["cu_seqlens"] = good
+    bwd()
     buf.inputs["cu_seqlens"] = good
     bwd()
     got = runner.fetch(buf)
