@@ -288,12 +288,12 @@ __global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) 
 // ------------------------------------------------------------------------------------------------
 // Forward and reverse carries (ffma_scan.cuh).
 // ------------------------------------------------------------------------------------------------
-template <int DK, int DV>
-__global__ void __launch_bounds__(kThreads) scan_kernel(Problem p, int dirs) {
+template <int DK, int DV, int CS>
+__global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_kernel(const __grid_constant__ Problem p, int dirs) {
     wait_prerequisites();
     extern __shared__ __align__(16) float sm[];
     if (reinterpret_cast<const WsHeader*>(p.ws)->status != GDN_OK) return;
-    scan_block<DK, DV, false>(p, dirs, sm, (int)blockIdx.x);
+    scan_block<DK, DV, CS, false>(p, dirs, sm, (int)blockIdx.x);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -570,14 +570,21 @@ __global__ void __launch_bounds__(kThreads, DK + DV == 128 ? 2 : 1) intra_kernel
     }
 }
 
+template <int DK, int DV, int CS>
+cudaError_t launch_scan_cs(const Problem& p, int dirs, cudaStream_t st) {
+    static SmemLimitOnce once;
+    const cudaError_t e = once.ensure(scan_kernel<DK, DV, CS>, (uint32_t)ScanShape<DK, CS>::BYTES);
+    if (e != cudaSuccess) return e;
+    { StageScope t(dirs == 2 ? ST_SCANS : dirs == 1 ? ST_RSCAN : ST_FSCAN, st); launch_kernel(scan_kernel<DK, DV, CS>, scan_blocks(p, dirs, CS), kThreads, ScanShape<DK, CS>::BYTES, st, p, dirs); }
+    return cudaGetLastError();
+}
 template <int DK, int DV>
 cudaError_t launch_scan_t(const Problem& p, int dirs, cudaStream_t st) {
-    static SmemLimitOnce once;
-    const cudaError_t e = once.ensure(scan_kernel<DK, DV>, (uint32_t)scan_smem<DK>());
-    if (e != cudaSuccess) return e;
-    const int ctas = p.d.N * p.d.H * (dirs == 2 ? 2 : 1) * (DV / kScanCols);
-    { StageScope t(dirs == 2 ? ST_SCANS : dirs == 1 ? ST_RSCAN : ST_FSCAN, st); launch_kernel(scan_kernel<DK, DV>, ctas, kThreads, scan_smem<DK>(), st, p, dirs); }
-    return cudaGetLastError();
+    switch (scan_columns(p, dirs)) {
+        case 4: return launch_scan_cs<DK, DV, 4>(p, dirs, st);
+        case 8: return launch_scan_cs<DK, DV, 8>(p, dirs, st);
+        default: return launch_scan_cs<DK, DV, 16>(p, dirs, st);
+    }
 }
 
 template <typename IO, int DK, int DV>

@@ -305,15 +305,19 @@ __global__ void __launch_bounds__(kThreads, 1) vprep_kernel(Problem p, int mode)
 // ------------------------------------------------------------------------------------------------
 // vscan: forward and reverse carries (ffma_scan.cuh).
 // ------------------------------------------------------------------------------------------------
-template <int DK, int DV>
-__global__ void __launch_bounds__(kThreads) vscan_kernel(Problem p, int dirs) {
+// (WALK: a block goes over the items, as the fall-back launches do; the loop costs 60 registers, hence an instance of its own.)
+template <int DK, int DV, int CS, bool WALK>
+__global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) vscan_kernel(const __grid_constant__ Problem p, int dirs) {
     wait_prerequisites();
     extern __shared__ __align__(16) float sm[];
     if (!vec_go(p)) return;
-    const int blocks = p.d.N * p.d.H * (dirs == 2 ? 2 : 1) * (DV / kScanCols);
-    for (int b = blockIdx.x; b < blocks; b += gridDim.x) {
-        scan_block<DK, DV, true>(p, dirs, sm, b);
-        __syncthreads();
+    if constexpr (!WALK) {
+        scan_block<DK, DV, CS, true>(p, dirs, sm, blockIdx.x);
+    } else {
+        for (int b = blockIdx.x; b < scan_blocks(p, dirs, CS); b += gridDim.x) {
+            scan_block<DK, DV, CS, true>(p, dirs, sm, b);
+            __syncthreads();
+        }
     }
 }
 
@@ -636,14 +640,21 @@ __global__ void __launch_bounds__(kThreads, 1) vintra_kernel(Problem p) {
 // thousands of blocks that return at once takes microseconds: three launches behind a call of 2112 chunk-heads, see launch).
 int grid_of(const Problem& p, int items) { return p.fallback && items > tc_sm_count() ? tc_sm_count() : items; }
 
+template <int DK, int DV, int CS, bool WALK>
+cudaError_t launch_vscan_cs(const Problem& p, int dirs, cudaStream_t st) {
+    static SmemLimitOnce once;
+    const auto kernel = vscan_kernel<DK, DV, CS, WALK>;
+    const cudaError_t e = once.ensure(kernel, (uint32_t)ScanShape<DK, CS>::BYTES);
+    if (e != cudaSuccess) return e;
+    { StageScope t(p.fallback ? ST_FALLBACK : dirs == 2 ? ST_SCANS : dirs == 1 ? ST_RSCAN : ST_FSCAN, st); launch_kernel(kernel, grid_of(p, scan_blocks(p, dirs, CS)), kThreads, ScanShape<DK, CS>::BYTES, st, p, dirs); }
+    return cudaGetLastError();
+}
 template <int DK, int DV>
 cudaError_t launch_vscan(const Problem& p, int dirs, cudaStream_t st) {
-    static SmemLimitOnce once;
-    const cudaError_t e = once.ensure(vscan_kernel<DK, DV>, (uint32_t)scan_smem<DK>());
-    if (e != cudaSuccess) return e;
-    const int ctas = p.d.N * p.d.H * (dirs == 2 ? 2 : 1) * (DV / kScanCols);
-    { StageScope t(p.fallback ? ST_FALLBACK : dirs == 2 ? ST_SCANS : dirs == 1 ? ST_RSCAN : ST_FSCAN, st); launch_kernel(vscan_kernel<DK, DV>, grid_of(p, ctas), kThreads, scan_smem<DK>(), st, p, dirs); }
-    return cudaGetLastError();
+    const int cs = scan_columns(p, dirs);
+    if constexpr (DK == 128 && DV == 128)
+        if (p.fallback && scan_blocks(p, dirs, cs) > tc_sm_count()) return launch_vscan_cs<DK, DV, 16, true>(p, dirs, st);
+    return cs == 4 ? launch_vscan_cs<DK, DV, 4, false>(p, dirs, st) : cs == 8 ? launch_vscan_cs<DK, DV, 8, false>(p, dirs, st) : launch_vscan_cs<DK, DV, 16, false>(p, dirs, st);
 }
 template <typename IO, int DK, int DV>
 cudaError_t launch_vprep(const Problem& p, PrepMode mode, cudaStream_t st) {

@@ -61,3 +61,29 @@ def test_channelwise_tile_edges(dk, dv, lengths, decay):
     fresh = runner.fetch(buf)
     for n in ("dq", "dk", "dv", "dg", "db", "dw", "dh0"):
         assert np.array_equal(fresh[n], got[n]), n
+
+
+@pytest.mark.parametrize("dk,dv", [(64, 64), (128, 128), (128, 64), (64, 128)])
+@pytest.mark.parametrize("heads", [1, 2, 4, 9])
+def test_columns_per_cta_of_the_carries(dk, dv, heads):
+    """The carries take 4, 8 or 16 state columns per CTA, by the number of chains: each of them, in one direction and in both,
+    with scalar and with per-channel gates (the same code with another decay)."""
+    lengths = [130, 65]
+    wl = synth.make_workload("columns", dtype="f32", lengths=lengths, H=heads, d_k=dk, d_v=dv, seed=312, states=True)
+    ref = oracle_grads(wl)
+    buf = runner.to_device(wl, want_o=True)
+    runner.run_bwd(buf)
+    got = runner.fetch(buf)
+    check_against_oracle(wl, got, tol=3e-6, ref=ref, block_tol=9e-6)
+    runner.run_fwd(buf)
+    runner.run_bwd(buf, fresh=1)
+    f = runner.fetch(buf)
+    assert rel(f["o"], ref["o"]) < 3e-6 and rel(f["hT"], ref["hT"]) < 3e-6
+    check_against_oracle(wl, f, tol=3e-6, ref=ref, block_tol=9e-6)
+    wl = synth.make_channelwise("columns", member="gdn", dtype="f32", lengths=lengths, H=heads, d_k=dk, d_v=dv, seed=313, states=True)
+    ref = oracle.vec_bwd_workload(wl)
+    buf = runner.to_device_channelwise(wl, want_o=True)
+    runner.run_bwd_channelwise(buf)
+    got = runner.fetch(buf)
+    for n in ("dq", "dk", "dv", "dg", "db", "dw", "dh0"):
+        assert rel(got[n], ref[n]) < 3e-6, (n, rel(got[n], ref[n]))
