@@ -50,7 +50,7 @@ __device__ __forceinline__ void for_chunks(const Problem& p, Body body) {
 
 // References of the four blocks and their exponentials: ref_0 = 0 (the chunk start), ref_I = gam of token 16 I - 1.
 template <int DK>
-struct Refs { float ref[kNB][DK], eref[kNB][DK]; };
+struct __align__(16) Refs { float ref[kNB][DK], eref[kNB][DK]; };
 template <int DK>
 __device__ __forceinline__ void make_refs(Refs<DK>& s, const float* G) {
     for (int t = threadIdx.x; t < kNB * DK; t += kThreads) {
@@ -60,25 +60,42 @@ __device__ __forceinline__ void make_refs(Refs<DK>& s, const float* G) {
         s.eref[I][r] = expf(v);
     }
 }
+// The elementwise passes go over four channels of a token at a time; what they read from global memory is fetched ahead of the pass,
+// all of it at once: with a load per element between the stores a pass of a chunk waited out 32 latencies, one behind the other.
+__device__ __forceinline__ float4 exp4(const float4& a, const float4& b) { return make_float4(expf(a.x - b.x), expf(a.y - b.y), expf(a.z - b.z), expf(a.w - b.w)); }
+__device__ __forceinline__ float4 mul4(const float4& a, const float4& b) { return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w); }
+__device__ __forceinline__ void st4(float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; }
+// v[i4 + y], i4 a multiple of four that is not known at compile time
+__device__ __forceinline__ float pick(const float (&v)[kB], int i4, int y) { return (i4 & 8) ? (i4 & 4 ? v[12 + y] : v[8 + y]) : (i4 & 4 ? v[4 + y] : v[y]); }
+template <int D>
+struct Quads {   // the quads of a [64 x D] tile, N per thread
+    static constexpr int N = kC * D / 4 / kThreads;
+    static __device__ __forceinline__ int row(int n) { return (threadIdx.x + n * kThreads) / (D / 4); }
+    static __device__ __forceinline__ int col(int n) { return (threadIdx.x + n * kThreads) % (D / 4) * 4; }
+};
+// Rows [0, 64) of a [T, H, D] tensor, this thread's quads; zero beyond `len`.
+template <int D, typename IO>
+__device__ __forceinline__ void fetch_quads(float4 (&v)[Quads<D>::N], const IO* src, size_t row_pitch, int len) {
+    using Qd = Quads<D>;
+#pragma unroll
+    for (int n = 0; n < Qd::N; ++n) v[n] = Qd::row(n) < len ? ld4(src + Qd::row(n) * row_pitch + Qd::col(n)) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
 // Rows of a tile times exp(gam - ref of their block), in place.
 template <int DK>
 __device__ __forceinline__ void scale_rows(float* X, const float* G, const Refs<DK>& s) {
-    for (int t = threadIdx.x; t < kC * DK; t += kThreads) {
-        const int i = t / DK, r = t % DK;
-        X[i * pitch(DK) + r] *= expf(G[i * pitch(DK) + r] - s.ref[i / kB][r]);
+    using Qd = Quads<DK>;
+#pragma unroll 2
+    for (int n = 0; n < Qd::N; ++n) {
+        const int i = Qd::row(n), c = Qd::col(n), o = i * pitch(DK) + c;
+        st4(X + o, mul4(ld4(X + o), exp4(ld4(G + o), ld4(s.ref[i / kB] + c))));
     }
 }
 // The scaled copies of the keys, k_j exp(ref_I - gam_j) for j < 16 I, I = 1 .. 3, one behind the other (96 rows).
 __host__ __device__ constexpr int copy_row(int I) { return kB * (I * (I - 1) / 2); }   // first row of copy I
-template <int DK, class KF>
-__device__ __forceinline__ void make_copies(float* C, const float* G, const Refs<DK>& s, KF key) {
-    for (int t = threadIdx.x; t < (kC - kB) * DK; t += kThreads) {
-        const int j = t / DK, r = t % DK;
-        const float k = key(j, r), g = G[j * pitch(DK) + r];
-#pragma unroll
-        for (int I = 1; I < kNB; ++I)
-            if (j < I * kB) C[(copy_row(I) + j) * pitch(DK) + r] = k * expf(s.ref[I][r] - g);
-    }
+template <int DK>
+__device__ __forceinline__ void make_copies(float* C, int j, int c, const float4& k, const float4& g, const Refs<DK>& s) {
+#pragma unroll 1
+    for (int I = j / kB + 1; I < kNB; ++I) st4(C + (copy_row(I) + j) * pitch(DK) + c, mul4(k, exp4(ld4(s.ref[I] + c), g)));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -122,38 +139,45 @@ __device__ __forceinline__ void vprep_chunk(const Problem& p, int mode, const Ch
         load_rows<DK>(K, rows_of<IO>(p.k, x, H, DK), rk, x.len);
         cp_commit();
         // chunk-local cumulative log decay per channel; rows beyond the sequence repeat the last valid one
+        using Qd = Quads<DK>;
+        load_rows<DK>(R, p.bv + base_k, rk, x.len);
+        cp_commit();
         if (tid < DK) {
             float s = 0.f;
 #pragma unroll 1
-            for (int i0 = 0; i0 < kC; i0 += 16) {   // sixteen loads in flight, then their running sum in token order
-                float g[16];
+            for (int i0 = 0; i0 < kC; i0 += 32) {   // 32 loads in flight, then their running sum in token order
+                float g[32];
 #pragma unroll
-                for (int k = 0; k < 16; ++k) g[k] = i0 + k < x.len ? p.gv[base_k + (size_t)(i0 + k) * rk + tid] : 0.f;
+                for (int k = 0; k < 32; ++k) g[k] = i0 + k < x.len ? p.gv[base_k + (size_t)(i0 + k) * rk + tid] : 0.f;
 #pragma unroll
-                for (int k = 0; k < 16; ++k) { s += g[k]; G[(i0 + k) * PK + tid] = s; }
+                for (int k = 0; k < 32; ++k) { s += g[k]; G[(i0 + k) * PK + tid] = s; }
             }
         }
-        for (int e = tid; e < 2 * kC * kPc; e += kThreads) A[e] = 0.f;   // (A and P lie behind each other)
+        for (int e = tid; e < 2 * kC * kPc / 4; e += kThreads) st4(A + 4 * e, make_float4(0.f, 0.f, 0.f, 0.f));   // (A and P lie behind each other)
         cp_wait<0>();
         __syncthreads();
         make_refs(refs, G);
-        for (int e = tid; e < kC * DK; e += kThreads) {
-            const int i = e / DK, r = e % DK;
-            const float k = K[i * PK + r];
-            R[i * PK + r] = i < x.len ? p.bv[base_k + i * rk + r] * k : 0.f;
-            wsG[e] = G[i * PK + r];
-            block_of(p, p.L.Kb, x.ch, kC * DK)[e] = k * expf(G[(kC - 1) * PK + r] - G[i * PK + r]);
+        float* wsKb = block_of(p, p.L.Kb, x.ch, kC * DK);
+#pragma unroll 2
+        for (int n = 0; n < Qd::N; ++n) {
+            const int o = Qd::row(n) * PK + Qd::col(n), e = (tid + n * kThreads) * 4;
+            const float4 k = ld4(K + o), g = ld4(G + o);
+            st4(R + o, mul4(ld4(R + o), k));
+            st4(wsG + e, g);
+            st4(wsKb + e, mul4(k, exp4(ld4(G + (kC - 1) * PK + Qd::col(n)), g)));
         }
         __syncthreads();
-        // pairs inside a block: 2 x 2 of them per thread, the 36 pieces of a block that reach the diagonal
-        if (tid < kNB * 36) {
-            const int I = tid / 36;
-            int n = tid % 36, a = 0;
+        // pairs inside a block, in pieces of 2 x 2: the 36 of a block that reach the diagonal; four lanes share one, a quarter of the channels each
+        const int z4 = tid & 3;
+#pragma unroll 1
+        for (int piece = tid >> 2; piece < kNB * 36; piece += kThreads / 4) {   // (a multiple of the eight pieces of a warp)
+            const int I = piece / 36;
+            int n = piece % 36, a = 0;
             while (n > a) { n -= a + 1; ++a; }   // piece (a, n), n <= a
             const int i = I * kB + 2 * a, j = I * kB + 2 * n;
             float aa[2][2] = {}, pp[2][2] = {};
 #pragma unroll 1
-            for (int r = 0; r < DK; r += 4) {
+            for (int r = 4 * z4; r < DK; r += 16) {
                 float gi[2][4], gj[2][4], q[2][4], b[2][4], k[2][4];
 #pragma unroll
                 for (int y = 0; y < 2; ++y) {
@@ -178,14 +202,25 @@ __device__ __forceinline__ void vprep_chunk(const Problem& p, int mode, const Ch
             for (int y = 0; y < 2; ++y)
 #pragma unroll
                 for (int w = 0; w < 2; ++w) {
+#pragma unroll
+                    for (int o = 1; o < 4; o <<= 1) {
+                        aa[y][w] += __shfl_xor_sync(0xffffffffu, aa[y][w], o);
+                        pp[y][w] += __shfl_xor_sync(0xffffffffu, pp[y][w], o);
+                    }
+                    if (z4 != 2 * y + w) continue;
                     if (j + w < i + y) A[(i + y) * kPc + j + w] = aa[y][w];
                     if (j + w <= i + y) Pm[(i + y) * kPc + j + w] = pp[y][w];
                 }
         }
         __syncthreads();
-        make_copies<DK>(C, G, refs, [&](int j, int r) { return K[j * PK + r]; });
-        scale_rows<DK>(Q, G, refs);
-        scale_rows<DK>(R, G, refs);
+#pragma unroll 2
+        for (int n = 0; n < Qd::N; ++n) {
+            const int i = Qd::row(n), c = Qd::col(n), o = i * PK + c;
+            const float4 g = ld4(G + o), e = exp4(g, ld4(refs.ref[i / kB] + c));
+            make_copies<DK>(C, i, c, ld4(K + o), g, refs);
+            st4(Q + o, mul4(ld4(Q + o), e));
+            st4(R + o, mul4(ld4(R + o), e));
+        }
         __syncthreads();
         // pairs of blocks J < I: A and P, 16 threads a 16 x 16 block, 4 x 4 each
         if (tid < 192) {
@@ -200,24 +235,29 @@ __device__ __forceinline__ void vprep_chunk(const Problem& p, int mode, const Ch
 #pragma unroll
                 for (int y = 0; y < 4; ++y) dst[r * kPc + 4 * y] = acc[r][y];
         }
-        for (int e = tid; e < kC * DK; e += kThreads) {   // Gam . b . K, the right-hand side of W
-            const int i = e / DK, r = e % DK;
-            K[i * PK + r] = R[i * PK + r] * refs.eref[i / kB][r];
+#pragma unroll 2
+        for (int n = 0; n < Qd::N; ++n) {   // Gam . b . K, the right-hand side of W
+            const int i = Qd::row(n), c = Qd::col(n), o = i * PK + c;
+            st4(K + o, mul4(ld4(R + o), ld4(refs.eref[i / kB] + c)));
         }
+        using Qv = Quads<DV>;
+        float4 wq[Qv::N];
+        fetch_quads<DV>(wq, p.wv + base_v, rv, x.len);
         __syncthreads();
         load_rows<DV>(R, rows_of<IO>(p.v, x, H, DV), rv, x.len);
         cp_commit();
         if (bwd) load_rows<DV>(O, rows_of<IO>(p.dO, x, H, DV), rv, x.len);
         cp_commit();
-        for (int e = tid; e < kC * kC; e += kThreads) wsP[e] = Pm[(e / kC) * kPc + e % kC];
+        for (int e = 4 * tid; e < kC * kC; e += 4 * kThreads) st4(wsP + e, ld4(Pm + (e / kC) * kPc + e % kC));
         invert(A, T);
         cp_wait<1>();
         __syncthreads();
         float* wsT = block_of(p, p.L.Tm, x.ch, kC * kC);
-        for (int e = tid; e < kC * kC; e += kThreads) wsT[e] = T[(e / kC) * kPc + e % kC];
-        for (int e = tid; e < kC * DV; e += kThreads) {
-            const int i = e / DV, r = e % DV;
-            if (i < x.len) R[i * PV + r] *= p.wv[base_v + i * rv + r];
+        for (int e = 4 * tid; e < kC * kC; e += 4 * kThreads) st4(wsT + e, ld4(T + (e / kC) * kPc + e % kC));
+#pragma unroll
+        for (int n = 0; n < Qv::N; ++n) {
+            float* v = R + Qv::row(n) * PV + Qv::col(n);
+            st4(v, mul4(ld4(v), wq[n]));
         }
         __syncthreads();
         float* wsU = block_of(p, p.L.Ut, x.ch, kC * DV);
@@ -343,10 +383,16 @@ __device__ __forceinline__ void vout_chunk(const Problem& p, const ChunkInfo& x)
     load_block<kC, DV>(sU, block_of(p, p.L.U, x.ch, kC * DV));
     load_block<kC, kC>(Pm, block_of(p, p.L.Pm, x.ch, kC * kC));
     cp_commit();
+    float4 gq[Quads<DK>::N];
+    fetch_quads<DK>(gq, block_of(p, p.L.gamma, x.ch, kC * DK), DK, kC);
     cp_wait<0>();
     __syncthreads();
-    const float* wsG = block_of(p, p.L.gamma, x.ch, kC * DK);
-    for (int e = threadIdx.x; e < kC * DK; e += kThreads) sQ[(e / DK) * PK + e % DK] *= expf(wsG[e]);
+    using Qd = Quads<DK>;
+#pragma unroll
+    for (int n = 0; n < Qd::N; ++n) {
+        float* q = sQ + Qd::row(n) * PK + Qd::col(n);
+        st4(q, mul4(ld4(q), exp4(gq[n], make_float4(0.f, 0.f, 0.f, 0.f))));
+    }
     __syncthreads();
     float acc[R][4];
     zero(acc);
@@ -407,7 +453,7 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
     float *s0 = sm + L::S0, *s1 = sm + L::S1, *sU = sm + L::U, *sH = sm + L::H, *sT = sm + L::T, *sP = sm + L::P;
     float *G = sm + L::G, *Q = sm + L::Q, *R = sm + L::R, *C = sm + L::C;
     __shared__ Refs<DK> refs;
-    __shared__ float ends[DK], blk[kNB][DK];   // chunk-end term of dg; first: its parts by row blocks; later: block sums of dgam
+    __shared__ __align__(16) float ends[DK], blk[kNB][DK];   // chunk-end term of dg; first: its parts by row blocks; later: block sums of dgam
     const int H = p.d.H, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const Thread t;
     const size_t rk = (size_t)H * DK, rv = (size_t)H * DV;
@@ -443,11 +489,19 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
     __syncthreads();
     {   // dXv = T^T dU, in place; dv = w . dXv, dw = v . dXv
         const Out<DV> o(t);
-        float acc[Out<DV>::R][4];
-        tri_product<DV, A_COL, A_UPPER>(t, sT, s1, PV, acc);
-        __syncthreads();
+        float acc[Out<DV>::R][4], vv[Out<DV>::R][4], ww[Out<DV>::R][4];
         const IO* vp = reinterpret_cast<const IO*>(p.v) + base_v;
         IO* dvp = reinterpret_cast<IO*>(p.dv) + base_v;
+#pragma unroll
+        for (int r = 0; r < Out<DV>::R; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const bool live = o.row(r) < x.len;
+                vv[r][y] = live ? ldf(vp + o.row(r) * rv + o.c + 8 * y) : 0.f;
+                ww[r][y] = live ? p.wv[base_v + o.row(r) * rv + o.c + 8 * y] : 0.f;
+            }
+        tri_product<DV, A_COL, A_UPPER>(t, sT, s1, PV, acc);
+        __syncthreads();
 #pragma unroll
         for (int r = 0; r < Out<DV>::R; ++r)
 #pragma unroll
@@ -455,8 +509,8 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
                 const int i = o.row(r), c = o.c + 8 * y;
                 s1[i * PV + c] = acc[r][y];
                 if (i < x.len) {
-                    stf(dvp + i * rv + c, p.wv[base_v + i * rv + c] * acc[r][y]);
-                    p.dwv[base_v + i * rv + c] = ldf(vp + i * rv + c) * acc[r][y];
+                    stf(dvp + i * rv + c, ww[r][y] * acc[r][y]);
+                    p.dwv[base_v + i * rv + c] = vv[r][y] * acc[r][y];
                 }
             }
     }
@@ -490,6 +544,11 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
     float col[NH][4][4];
 #pragma unroll
     for (int n = 0; n < NH; ++n) {
+        float kr[4][4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) kr[r][y] = t.rn + r < x.len ? ldf(kp + (t.rn + r) * rk + n * 64 + t.cn + 8 * y) : 0.f;
         zero(col[n]);
         mac<1, A_ROW, B_ROW>(col[n], sU, nullptr, PV, t.rn, sH + n * 64 * PV, PV, t.cn, 0, DV);
 #pragma unroll
@@ -503,7 +562,7 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
                 col[n][r][y] *= expf(G[(kC - 1) * PK + c] - g);
                 acc[n][r][y] *= sc * Gi;
                 acc[n][4 + r][y] *= -Gi;
-                if (i < x.len) s = fmaf(ldf(kp + i * rk + c), col[n][r][y], s);
+                s = fmaf(kr[r][y], col[n][r][y], s);
             }
             s += __shfl_xor_sync(0xffffffffu, s, 8);
             s += __shfl_xor_sync(0xffffffffu, s, 16);
@@ -511,23 +570,37 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
         }
     }
     // Gam_e rowdot(dh', h): one warp per state row (h from the workspace: its tile has been overwritten)
-    for (int r = warp; r < DK; r += kThreads / 32) {
-        float s = 0.f;
-        if (lane * 4 < DV) {
-            const float4 a = ld4(wsH + (size_t)r * DV + lane * 4), b = ld4(sH + r * PV + lane * 4);
-            s = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w)));
+    constexpr int HB = 8;   // rows whose loads are in flight at a time
+#pragma unroll 1
+    for (int r0 = warp * (DK / 8); r0 < (warp + 1) * (DK / 8); r0 += HB) {
+        float4 h4[HB];
+#pragma unroll
+        for (int k = 0; k < HB; ++k) h4[k] = lane * 4 < DV ? ld4(wsH + (size_t)(r0 + k) * DV + lane * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < HB; ++k) {
+            float s = 0.f;
+            if (lane * 4 < DV) {
+                const float4 a = h4[k], b = ld4(sH + (r0 + k) * PV + lane * 4);
+                s = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w)));
+            }
+            s = warp_total(s);
+            if (lane == 0) ends[r0 + k] = expf(G[(kC - 1) * PK + r0 + k]) * s;
         }
-        s = warp_total(s);
-        if (lane == 0) ends[r] = expf(G[(kC - 1) * PK + r]) * s;
     }
+    using Qd = Quads<DK>;
+    float4 kq[Qd::N], bq[Qd::N];
+    fetch_quads<DK>(kq, kp, rk, x.len);
+    fetch_quads<DK>(bq, p.bv + base_k, rk, x.len);
     __syncthreads();
     if (tid < DK) ends[tid] += (blk[0][tid] + blk[1][tid]) + (blk[2][tid] + blk[3][tid]);
-    for (int e = tid; e < kC * DK; e += kThreads) {
-        const int i = e / DK, r = e % DK;
-        R[i * PK + r] = i < x.len ? p.bv[base_k + i * rk + r] * ldf(kp + i * rk + r) * expf(G[i * PK + r] - refs.ref[i / kB][r]) : 0.f;
+#pragma unroll
+    for (int n = 0; n < Qd::N; ++n) {
+        const int i = Qd::row(n), c = Qd::col(n), o = i * PK + c;
+        const float4 g = ld4(G + o), e = exp4(g, ld4(refs.ref[i / kB] + c));
+        make_copies<DK>(C, i, c, kq[n], g, refs);
+        st4(R + o, mul4(mul4(bq[n], kq[n]), e));
+        st4(Q + o, mul4(ld4(Q + o), e));
     }
-    scale_rows<DK>(Q, G, refs);
-    make_copies<DK>(C, G, refs, [&](int j, int r) { return j < x.len ? ldf(kp + j * rk + r) : 0.f; });
     __syncthreads();
     // pairs of blocks J < I
 #pragma unroll
@@ -578,36 +651,58 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
 #pragma unroll 1
     for (int task = tid; task < kNB * DK; task += kThreads) {   // one channel of one block of tokens
         const int B = task / DK, r = task % DK, i0 = B * kB;
-        float q[kB], k[kB], b[kB], g[kB], dc[kB];
+        float k[kB], b[kB], g[kB], dc[kB];
+        float qn[4];   // q of four rows, fetched a group ahead
+        auto fetch_q = [&](int i4) {
+#pragma unroll
+            for (int y = 0; y < 4; ++y) qn[y] = i4 < kB && i0 + i4 + y < x.len ? ldf(qp + (i0 + i4 + y) * rk + r) : 0.f;
+        };
+        fetch_q(0);
 #pragma unroll
         for (int i = 0; i < kB; ++i) {
             const bool live = i0 + i < x.len;
-            q[i] = live ? ldf(qp + (i0 + i) * rk + r) : 0.f;
             k[i] = live ? ldf(kp + (i0 + i) * rk + r) : 0.f;
             b[i] = live ? p.bv[base_k + (i0 + i) * rk + r] : 0.f;
             g[i] = G[(i0 + i) * PK + r];
             dc[i] = R[(i0 + i) * PK + r];
         }
-        // a row at a time: its dq and row role are complete at once, the column roles collect
+        // four rows at a time (a rolled loop: the code of all 136 pairs is 30 KB, which a CTA would fetch for two passes): their dq and row
+        // role are complete at once, the column roles collect
+#pragma unroll 1
+        for (int i4 = 0; i4 < kB; i4 += 4) {
+            float gi[4], q[4], bk[4], ki[4], dq[4], row[4];
 #pragma unroll
-        for (int i = 0; i < kB; ++i) {
-            float dq = C[(i0 + i) * PK + r], row = Q[(i0 + i) * PK + r];
-            const float bk = b[i] * k[i];
-            const float* P_ = sP + (i0 + i) * kPc + i0;
-            const float* A_ = sT + (i0 + i) * kPc + i0;
+            for (int y = 0; y < 4; ++y) {
+                gi[y] = G[(i0 + i4 + y) * PK + r]; q[y] = qn[y]; ki[y] = pick(k, i4, y); bk[y] = pick(b, i4, y) * ki[y];
+                dq[y] = C[(i0 + i4 + y) * PK + r]; row[y] = Q[(i0 + i4 + y) * PK + r];
+            }
+            fetch_q(i4 + 4);
 #pragma unroll
-            for (int j = 0; j <= i; ++j) {
-                const float e = j < i ? expf(g[i] - g[j]) : 1.f, pe = P_[j] * e, ae = A_[j] * e;   // (dA_ii = 0)
-                dq = fmaf(pe, k[j], dq);
-                row = fmaf(ae, k[j], row);
-                dc[j] = fmaf(pe, q[i], fmaf(ae, bk, dc[j]));
+            for (int j4 = 0; j4 < kB; j4 += 4) {
+                if (j4 > i4) break;
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                    const float4 P4 = ld4(sP + (i0 + i4 + y) * kPc + i0 + j4), A4 = ld4(sT + (i0 + i4 + y) * kPc + i0 + j4);   // (zero above the diagonal, dA on it too)
+                    const float P_[4] = {P4.x, P4.y, P4.z, P4.w}, A_[4] = {A4.x, A4.y, A4.z, A4.w};
+#pragma unroll
+                    for (int z = 0; z < 4; ++z) {
+                        const float e = expf(j4 + z < i4 + y ? gi[y] - g[j4 + z] : 0.f), pe = P_[z] * e, ae = A_[z] * e;
+                        dq[y] = fmaf(pe, k[j4 + z], dq[y]);
+                        row[y] = fmaf(ae, k[j4 + z], row[y]);
+                        dc[j4 + z] = fmaf(pe, q[y], fmaf(ae, bk[y], dc[j4 + z]));
+                    }
+                }
             }
-            if (i0 + i < x.len) {
-                stf(dqp + (i0 + i) * rk + r, dq);
-                p.dbv[base_k + (i0 + i) * rk + r] = k[i] * row;
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int i = i0 + i4 + y;
+                if (i < x.len) {
+                    stf(dqp + i * rk + r, dq[y]);
+                    p.dbv[base_k + i * rk + r] = ki[y] * row[y];
+                }
+                Q[i * PK + r] = row[y];
+                C[i * PK + r] = fmaf(q[y], dq[y], bk[y] * row[y]);
             }
-            Q[(i0 + i) * PK + r] = row;
-            C[(i0 + i) * PK + r] = fmaf(q[i], dq, bk * row);
         }
         float run = 0.f;   // dgam, summed from the end of the block
 #pragma unroll
@@ -620,12 +715,15 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
     }
     __syncthreads();
     // dg_j = sum_{i >= j} dgam_i: the sum inside the block, the blocks behind it and the chunk end
-    for (int e = tid; e < kC * DK; e += kThreads) {
-        const int i = e / DK, r = e % DK;
-        if (i >= x.len) continue;
-        float s = ends[r];
-        for (int B = kNB - 1; B > i / kB; --B) s += blk[B][r];
-        p.dgv[base_k + i * rk + r] = s + C[i * PK + r];
+#pragma unroll 2
+    for (int n = 0; n < Qd::N; ++n) {
+        const int i = Qd::row(n), c = Qd::col(n);
+        float4 s = ld4(ends + c);
+#pragma unroll
+        for (int B = kNB - 1; B > 0; --B)
+            if (B > i / kB) { const float4 v = ld4(blk[B] + c); s = make_float4(s.x + v.x, s.y + v.y, s.z + v.z, s.w + v.w); }
+        const float4 v = ld4(C + i * PK + c);
+        if (i < x.len) st4(p.dgv + base_k + i * rk + c, make_float4(s.x + v.x, s.y + v.y, s.z + v.z, s.w + v.w));
     }
 }
 
