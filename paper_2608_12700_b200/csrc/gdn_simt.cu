@@ -356,29 +356,37 @@ __global__ void __launch_bounds__(kThreads, 1) out_kernel(Problem p) {
 //     dq = scale Gam (dO h^T) + dPD K        dk^row = G K + Gam dXk       dv = w dXv
 //     dk = b dk^row + dk^col                 dk^col = e (U dh'^T) + dPD^T Q + (b G)^T K
 //     dgam_i = <q, dq> + b <k, dk^row> - <k, dk^col>, and the last row adds sum_j e_j <k_j, (U dh'^T)_j> + Gam_e <dh', h>
-// Tiles: dO, U, dU (then dXv) and h first; K and Q over dO and dXv, dh' over h, once the products with h are done (their
-// results wait in registers: at d = 128 the seven tiles do not fit beside each other).
+// dPD, G and dXv are made once; dq and dk then in passes of 64 channels over the slices of h, dh', K and Q that these need (at d_v = 128
+// dh' comes over h, for the tiles do not fit beside each other).  The passes are a rolled loop: a CTA goes through the code once, and at
+// d = 128 what it waits for most is instructions.
 // ------------------------------------------------------------------------------------------------
 template <int DK, int DV>
-constexpr size_t intra_smem() {
-    constexpr int PM = pitch(DK > DV ? DK : DV);
-    return sizeof(float) * (2 * kC * PM + kC * pitch(DV) + DK * pitch(DV) + 3 * kC * kPc);
-}
+struct IntraTiles {
+    static constexpr int PV = pitch(DV);
+    static constexpr int O = 0;                  // dO
+    static constexpr int X = O + kC * PV;        // dU, then dXv
+    static constexpr int U = X + kC * PV;
+    static constexpr int T = U + kC * PV;        // T, then G
+    static constexpr int B = T + kC * kPc;       // Diag(b) G
+    static constexpr int P = B + kC * kPc;       // dPD
+    static constexpr int K = P + kC * kPc;       // slices of 64 channels
+    static constexpr int Q = K + kC * kPc;
+    static constexpr int H = Q + kC * kPc;       // h
+    static constexpr bool OWN = DV == 64;        // dh' has a tile of its own
+    static constexpr int D = OWN ? H + 64 * PV : H;
+    static constexpr size_t BYTES = sizeof(float) * (D + 64 * PV);
+};
 
 template <typename IO, int DK, int DV>
-__global__ void __launch_bounds__(kThreads, DK + DV == 128 ? 2 : 1) intra_kernel(Problem p) {
+__global__ void __launch_bounds__(kThreads, 1) intra_kernel(Problem p) {
     wait_prerequisites();
     ChunkInfo x;
     if (!chunk_head(p, x)) return;
-    constexpr int PK = pitch(DK), PV = pitch(DV), PM = pitch(DK > DV ? DK : DV), NH = DK / 64;
+    using L = IntraTiles<DK, DV>;
+    constexpr int PV = pitch(DV), NH = DK / 64;
     extern __shared__ __align__(16) float sm[];
-    float* s0 = sm;                  // dO, then K
-    float* s1 = s0 + kC * PM;        // dU, then dXv, then Q
-    float* sU = s1 + kC * PM;        // U
-    float* sH = sU + kC * PV;        // h, then dh'
-    float* sT = sH + DK * PV;        // T, then G
-    float* sB = sT + kC * kPc;       // Diag(b) G
-    float* sP = sB + kC * kPc;       // dPD
+    float *sO = sm + L::O, *sX = sm + L::X, *sU = sm + L::U, *sT = sm + L::T, *sB = sm + L::B, *sP = sm + L::P, *sK = sm + L::K, *sQ = sm + L::Q,
+          *sH = sm + L::H, *sD = sm + L::D;
     __shared__ Gates gs;
     __shared__ float red[4][4][kC];  // row dots <q, dq>, <k, dk^row>, <k, dk^col>, <v, dXv>: [which][column block][row]
     __shared__ float dgam[kC], part[2][kThreads / 32];
@@ -387,24 +395,31 @@ __global__ void __launch_bounds__(kThreads, DK + DV == 128 ? 2 : 1) intra_kernel
     const size_t rk = (size_t)H * DK, rv = (size_t)H * DV;
     const float sc = p.d.scale;
     const float* wsH = block_of(p, p.L.hc, x.ch, DK * DV);
+    const float* wsD = block_of(p, p.L.dhn, x.ch, DK * DV);
+    const IO* qp = rows_of<IO>(p.q, x, H, DK);
+    const IO* kp = rows_of<IO>(p.k, x, H, DK);
 
-    load_rows<DV>(s0, rows_of<IO>(p.dO, x, H, DV), rv, x.len);
+    load_rows<DV>(sO, rows_of<IO>(p.dO, x, H, DV), rv, x.len);
     load_block<kC, DV>(sU, block_of(p, p.L.U, x.ch, kC * DV));
     cp_commit();
-    load_block<kC, DV>(s1, block_of(p, p.L.dU, x.ch, kC * DV));
+    load_block<kC, DV>(sX, block_of(p, p.L.dU, x.ch, kC * DV));
     load_block<kC, kC>(sT, block_of(p, p.L.Tm, x.ch, kC * kC));
     cp_commit();
-    load_block<DK, DV>(sH, wsH);
+    load_block<64, DV>(sH, wsH);
+    cp_commit();
+    load_rows<64>(sK, kp, rk, x.len);
+    load_rows<64>(sQ, qp, rk, x.len);
+    if (L::OWN) load_block<64, DV>(sD, wsD);
     cp_commit();
     if (tid < 32) load_gates(p, x, gs, block_of(p, p.L.gamma, x.ch, kC));
-    cp_wait<2>();
+    cp_wait<3>();
     __syncthreads();
     // 64 x 64 matrices: warps whose 16 x 32 block lies above the diagonal have nothing to add up
     const bool below = (warp >> 2) * 32 <= (t.rn >> 4) * 16 + 15;
     {   // dPD = scale tril(dO U^T) . D; the decay exponent is only evaluated where it is non-positive
         float acc[4][4];
         zero(acc);
-        if (below) mac<1, A_ROW, B_ROW>(acc, s0, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
+        if (below) mac<1, A_ROW, B_ROW>(acc, sO, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
@@ -413,7 +428,7 @@ __global__ void __launch_bounds__(kThreads, DK + DV == 128 ? 2 : 1) intra_kernel
                 sP[i * kPc + j] = j <= i ? sc * acc[r][y] * expf(gs.gam[i] - gs.gam[j]) : 0.f;
             }
     }
-    cp_wait<1>();
+    cp_wait<2>();
     __syncthreads();
     {   // dXv = T^T dU, in place; dv = w dXv; <v, dXv>
         const Out<DV> o(t);
@@ -424,7 +439,7 @@ __global__ void __launch_bounds__(kThreads, DK + DV == 128 ? 2 : 1) intra_kernel
         for (int r = 0; r < R; ++r)
 #pragma unroll
             for (int y = 0; y < 4; ++y) vv[r][y] = o.row(r) < x.len ? ldf(vp + o.row(r) * rv + o.c + 8 * y) : 0.f;
-        tri_product<DV, A_COL, A_UPPER>(t, sT, s1, PV, acc);
+        tri_product<DV, A_COL, A_UPPER>(t, sT, sX, PV, acc);
         __syncthreads();
         IO* dvp = rows_of<IO>(p.dv, x, H, DV);
 #pragma unroll
@@ -434,7 +449,7 @@ __global__ void __launch_bounds__(kThreads, DK + DV == 128 ? 2 : 1) intra_kernel
             float dot = 0.f;
 #pragma unroll
             for (int y = 0; y < 4; ++y) {
-                s1[i * PV + o.c + 8 * y] = acc[r][y];
+                sX[i * PV + o.c + 8 * y] = acc[r][y];
                 dot = fmaf(vv[r][y], acc[r][y], dot);
                 if (i < x.len) stf(dvp + i * rv + o.c + 8 * y, w * acc[r][y]);
             }
@@ -442,12 +457,11 @@ __global__ void __launch_bounds__(kThreads, DK + DV == 128 ? 2 : 1) intra_kernel
             if ((lane & 7) == 0) red[3][DV == 128 ? warp >> 1 : warp >> 2][i] = dot;
         }
     }
-    cp_wait<0>();
     __syncthreads();
     {   // G = -stril(dXv U^T) . D and Diag(b) G (over T)
         float acc[4][4];
         zero(acc);
-        if (below) mac<1, A_ROW, B_ROW>(acc, s1, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
+        if (below) mac<1, A_ROW, B_ROW>(acc, sX, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
@@ -458,71 +472,88 @@ __global__ void __launch_bounds__(kThreads, DK + DV == 128 ? 2 : 1) intra_kernel
                 sB[i * kPc + j] = gs.bb[i] * g;
             }
     }
-    // [dO; dXv] h^T: rows 0..3 become dq, rows 4..7 dk^row
-    float acc[NH][8][4];
-#pragma unroll
-    for (int n = 0; n < NH; ++n) {
-        zero(acc[n]);
-        mac<2, A_ROW, B_ROW>(acc[n], s0, s1, PV, t.rn, sH + n * 64 * PV, PV, t.cn, 0, DV);
-    }
-    __syncthreads();
-    load_rows<DK>(s0, rows_of<IO>(p.k, x, H, DK), rk, x.len);
-    cp_commit();
-    load_rows<DK>(s1, rows_of<IO>(p.q, x, H, DK), rk, x.len);
-    load_block<DK, DV>(sH, block_of(p, p.L.dhn, x.ch, DK * DV));
-    cp_commit();
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const float a = sc * gs.Gam[t.rn + r], b = -gs.Gam[t.rn + r];
-#pragma unroll
-        for (int n = 0; n < NH; ++n)
-#pragma unroll
-            for (int y = 0; y < 4; ++y) { acc[n][r][y] *= a; acc[n][4 + r][y] *= b; }
-    }
-    cp_wait<1>();
-    __syncthreads();
-    // += [dPD; G] K
     const int w16 = (t.rn >> 4) * 16;
-#pragma unroll
-    for (int n = 0; n < NH; ++n) mac<2, A_ROW, B_COL>(acc[n], sP, sT, kPc, t.rn, s0 + n * 64, PK, t.cn, 0, w16 + 16);
-    cp_wait<0>();
-    __syncthreads();
-    // dk^col = e (U dh'^T) + dPD^T Q + (b G)^T K, then everything is written
-    IO* dqp = rows_of<IO>(p.dq, x, H, DK);
-    IO* dkp = rows_of<IO>(p.dk, x, H, DK);
-    float rsum = 0.f, dqq[4] = {}, drow[4] = {}, dcol[4] = {};
-#pragma unroll
+    float rsum = 0.f, hh = 0.f, dqq[4] = {}, drow[4] = {}, dcol[4] = {};
+#pragma unroll 1
     for (int n = 0; n < NH; ++n) {
-        float col[4][4];
+        // [dO; dXv] h^T: rows 0..3 become dq, rows 4..7 dk^row
+        float acc[8][4], col[4][4];
+        zero(acc);
         zero(col);
-        mac<1, A_ROW, B_ROW>(col, sU, nullptr, PV, t.rn, sH + n * 64 * PV, PV, t.cn, 0, DV);
+        if (n || !L::OWN) cp_wait<0>(); else cp_wait<1>();   // (the first slice of K and Q may still be under way; see below)
+        __syncthreads();
+        mac<2, A_ROW, B_ROW>(acc, sO, sX, PV, t.rn, sH, PV, t.cn, 0, DV);
+        float4 h4[64 * DV / 4 / kThreads];
+#pragma unroll
+        for (int m = 0; m < 64 * DV / 4 / kThreads; ++m) h4[m] = ld4(wsH + (size_t)n * 64 * DV + (tid + m * kThreads) * 4);
+        if (!L::OWN) {
+            __syncthreads();
+            load_block<64, DV>(sD, wsD + (size_t)n * 64 * DV);
+            cp_commit();
+        } else {
+            cp_wait<0>();
+            __syncthreads();
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const float a = sc * gs.Gam[t.rn + r], b = -gs.Gam[t.rn + r];
+#pragma unroll
+            for (int y = 0; y < 4; ++y) { acc[r][y] *= a; acc[4 + r][y] *= b; }
+        }
+        // += [dPD; G] K
+        mac<2, A_ROW, B_COL>(acc, sP, sT, kPc, t.rn, sK, kPc, t.cn, 0, w16 + 16);
+        if (!L::OWN) {
+            cp_wait<0>();
+            __syncthreads();
+        }
+        // dk^col = e (U dh'^T) + dPD^T Q + (b G)^T K, then everything is written
+        mac<1, A_ROW, B_ROW>(col, sU, nullptr, PV, t.rn, sD, PV, t.cn, 0, DV);
+#pragma unroll
+        for (int m = 0; m < 64 * DV / 4 / kThreads; ++m) {   // <dh', h> (h from the workspace: its tile may have been overwritten)
+            const int e = tid + m * kThreads;
+            const float4 b = ld4(sD + (e / (DV / 4)) * PV + (e % (DV / 4)) * 4);
+            hh = fmaf(h4[m].x, b.x, fmaf(h4[m].y, b.y, fmaf(h4[m].z, b.z, fmaf(h4[m].w, b.w, hh))));
+        }
+        if (n + 1 < NH) {   // the next slice of the states
+            __syncthreads();
+            load_block<64, DV>(sH, wsH + (size_t)(n + 1) * 64 * DV);
+            if (L::OWN) load_block<64, DV>(sD, wsD + (size_t)(n + 1) * 64 * DV);
+        }
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const float e = gs.ee[t.rn + r];
 #pragma unroll
             for (int y = 0; y < 4; ++y) {
                 col[r][y] *= e;
-                rsum = fmaf(s0[(t.rn + r) * PK + n * 64 + t.cn + 8 * y], col[r][y], rsum);
+                rsum = fmaf(sK[(t.rn + r) * kPc + t.cn + 8 * y], col[r][y], rsum);
             }
         }
-        mac<1, A_COL, B_COL>(col, sP, nullptr, kPc, t.rn, s1 + n * 64, PK, t.cn, w16, kC);
-        mac<1, A_COL, B_COL>(col, sB, nullptr, kPc, t.rn, s0 + n * 64, PK, t.cn, w16, kC);
+        mac<1, A_COL, B_COL>(col, sP, nullptr, kPc, t.rn, sQ, kPc, t.cn, w16, kC);
+        mac<1, A_COL, B_COL>(col, sB, nullptr, kPc, t.rn, sK, kPc, t.cn, w16, kC);
+        IO* dqp = rows_of<IO>(p.dq, x, H, DK) + n * 64;
+        IO* dkp = rows_of<IO>(p.dk, x, H, DK) + n * 64;
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const int i = t.rn + r;
             const float b = gs.bb[i];
 #pragma unroll
             for (int y = 0; y < 4; ++y) {
-                const int c = n * 64 + t.cn + 8 * y;
-                const float q = s1[i * PK + c], k = s0[i * PK + c];
-                dqq[r] = fmaf(q, acc[n][r][y], dqq[r]);
-                drow[r] = fmaf(k, acc[n][4 + r][y], drow[r]);
+                const int c = t.cn + 8 * y;
+                const float q = sQ[i * kPc + c], k = sK[i * kPc + c];
+                dqq[r] = fmaf(q, acc[r][y], dqq[r]);
+                drow[r] = fmaf(k, acc[4 + r][y], drow[r]);
                 dcol[r] = fmaf(k, col[r][y], dcol[r]);
                 if (i < x.len) {
-                    stf(dqp + i * rk + c, acc[n][r][y]);
-                    stf(dkp + i * rk + c, fmaf(b, acc[n][4 + r][y], col[r][y]));
+                    stf(dqp + i * rk + c, acc[r][y]);
+                    stf(dkp + i * rk + c, fmaf(b, acc[4 + r][y], col[r][y]));
                 }
             }
+        }
+        if (n + 1 < NH) {
+            __syncthreads();
+            load_rows<64>(sK, kp + (n + 1) * 64, rk, x.len);
+            load_rows<64>(sQ, qp + (n + 1) * 64, rk, x.len);
+            cp_commit();
         }
     }
 #pragma unroll
@@ -532,13 +563,6 @@ __global__ void __launch_bounds__(kThreads, DK + DV == 128 ? 2 : 1) intra_kernel
             const int cb = warp >> 2, i = t.rn + r;
             red[0][cb][i] = dqq[r]; red[1][cb][i] = drow[r]; red[2][cb][i] = dcol[r];
         }
-    }
-    // <dh', h> over the whole state (h from the workspace: its tile has been overwritten)
-    float hh = 0.f;
-#pragma unroll 4
-    for (int e = tid; e < DK * DV / 4; e += kThreads) {
-        const float4 a = ld4(wsH + (size_t)e * 4), b = ld4(sH + (e / (DV / 4)) * PV + (e % (DV / 4)) * 4);
-        hh = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, hh))));
     }
     rsum = warp_total(rsum);
     hh = warp_total(hh);
@@ -615,8 +639,8 @@ cudaError_t launch_bwd_t(const Problem& p, bool skip_recompute, cudaStream_t st)
     if ((e = launch_prep_t<IO, DK, DV>(p, skip_recompute ? PREP_BWD : PREP_FWD_BWD, st)) != cudaSuccess) return e;
     if ((e = launch_scan_t<DK, DV>(p, skip_recompute ? 1 : 2, st)) != cudaSuccess) return e;
     static SmemLimitOnce once;
-    if ((e = once.ensure(intra_kernel<IO, DK, DV>, (uint32_t)intra_smem<DK, DV>())) != cudaSuccess) return e;
-    { StageScope t(ST_INTRA, st); launch_kernel(intra_kernel<IO, DK, DV>, p.L.max_chunks * p.d.H, kThreads, intra_smem<DK, DV>(), st, p); }
+    if ((e = once.ensure(intra_kernel<IO, DK, DV>, (uint32_t)IntraTiles<DK, DV>::BYTES)) != cudaSuccess) return e;
+    { StageScope t(ST_INTRA, st); launch_kernel(intra_kernel<IO, DK, DV>, p.L.max_chunks * p.d.H, kThreads, IntraTiles<DK, DV>::BYTES, st, p); }
     return cudaGetLastError();
 }
 
