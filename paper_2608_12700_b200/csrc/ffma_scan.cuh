@@ -1,12 +1,12 @@
 // Inter-chunk carries of the FFMA families in low-rank form (fp32), for scalar and for per-channel gates:
 //     forward   U = U~ - W h (stored),          h' = Ge h + Kb^T U            (h stored per chunk)
-//     reverse   Y = Kb dh', dU += Y (stored),   dh = Ge dh' + E - W^T Y        (dh' stored per chunk; the paper's K#1)
+//     reverse   dU = scale P^T dO + Kb dh' (stored),   dh = Ge dh' + E - W^T dU   (dh' stored per chunk; the paper's K#1)
 // with Kb the keys scaled to the chunk end (made by the preparation kernel), Ge the decay of the state over the chunk (one
-// factor, or one per state row) and dU preset to scale P^T dO.  U and dU are what the gradient stage needs, so it repeats
-// neither product.
+// factor, or one per state row), E = scale (Gam . Q)^T dO, and dU preset to scale P^T dO.  U and dU are what the gradient stage
+// needs, so it repeats neither product; and because W^T meets the whole of dU here, E needs neither P nor W.
 //
 // The chain of chunks is serial, so a step is made short.  The state columns evolve independently and a CTA carries CS of them, in
-// passes of at most eight.  A warp owns eight tokens of the chunk: it makes their rows of U or Y (a contraction over the features, split
+// passes of at most eight.  A warp owns eight tokens of the chunk: it makes their rows of U or dU (a contraction over the features, split
 // over eight lanes and summed by exchanges) and multiplies them into the state at once (over its own eight tokens), so only the sum
 // of the eight warps' shares crosses the CTA: two barriers a step.  W and Kb come straight into the registers of the threads
 // that use them, each as soon as the step before has used its predecessor; no element of them is wanted twice.
@@ -63,10 +63,10 @@ __device__ __forceinline__ void scan_chain(const Problem& p, int chain, int part
     using Sl = Slice<DK, CB>;
     constexpr int MA = DK / 32;                       // 16-byte pieces of a row per lane in the first product
     constexpr int PW = DK * CB / kThreads;            // consecutive columns of the state that a thread keeps, per pass
-    constexpr int YW = CB / 4;                        // ... and of U or Y that a lane sums up
+    constexpr int YW = CB / 4;                        // ... and of U or dU that a lane sums up
     float* red = sm;                                  // [NP][SLICES] slices
     float* hs = red + NP * Sh::SLICES * Sl::FLOATS;   // [NP] slices: the state
-    float* ys = hs + NP * Sl::FLOATS;                 // [64][CB]: U or Y, every warp its own eight rows
+    float* ys = hs + NP * Sl::FLOATS;                 // [64][CB]: U or dU, every warp its own eight rows
     const int H = p.d.H, n = chain / H, hd = chain % H;
     const SeqGeom sg = seq_geom(p, n);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -176,20 +176,16 @@ __device__ __forceinline__ void scan_chain(const Problem& p, int chain, int part
                         acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
                     }
                 }
-                float y[YW], out[YW];
+                float y[YW];
 #pragma unroll
-                for (int c = 0; c < YW; ++c) {
-                    y[c] = acc[c];
-                    out[c] = REVERSE ? yadd[u][c] + y[c] : yadd[u][c] - y[c];
-                    if (!REVERSE) y[c] = out[c];
-                }
-                st_cols(wsY + (ch * kC + yrow) * DV + part * CS + u * CB + ycol, out);
+                for (int c = 0; c < YW; ++c) y[c] = REVERSE ? yadd[u][c] + acc[c] : yadd[u][c] - acc[c];
+                st_cols(wsY + (ch * kC + yrow) * DV + part * CS + u * CB + ycol, y);
                 st_cols(ys + yrow * CB + ycol, y);
             }
             if (more) load_yadd(s + 1, u);
             if (more && u == NP - 1) load_a(s + 1);
             __syncwarp();
-            {   // Kb^T U or W^T Y
+            {   // Kb^T U or W^T dU
                 float4 acc[4][NQ] = {};
 #pragma unroll
                 for (int t = 0; t < TB; ++t)

@@ -186,6 +186,9 @@ __device__ __forceinline__ void invert(const float* A, float* T) {
 
 // Which part of the preparation a launch makes: the forward's, that and the backward's, the backward's alone.
 enum PrepMode { PREP_FWD = 0, PREP_FWD_BWD = 1, PREP_BWD = 2 };
+// CTAs per chunk-head of the scalar-gate preparation: two as long as every one of them finds an SM of its own (2 heads of 128 tokens, d = 64,
+// closed backward: 23.7 -> 16.8 us).  With per-channel gates both chains need the decay within the blocks, and two CTAs gain nothing.
+inline int prep_parts(const Problem& p, PrepMode mode) { return mode != PREP_BWD && 2 * p.L.max_chunks * p.d.H <= tc_sm_count() ? 2 : 1; }
 
 // Sum over the eight lanes that share a row (fixed order).
 __device__ __forceinline__ float row_sum8(float v) {

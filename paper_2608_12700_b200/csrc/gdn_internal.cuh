@@ -46,7 +46,7 @@ struct WsLayout {
     int has_operator;
     size_t hc;             // [CH, d_k, d_v]           state entering the chunk
     size_t fwd_end;        // bytes needed by the forward recompute
-    size_t E;              // [CH, d_k, d_v]           scale (Gam Q - P W)^T dO
+    size_t E;              // [CH, d_k, d_v]           scale (Gam Q - P W)^T dO (FFMA families: scale (Gam Q)^T dO)
     size_t dhn;            // [CH, d_k, d_v]           gradient w.r.t. the state leaving the chunk
     size_t Pm;             // [CH, 64, 64]             P = tril(Q K^T . D) (tcgen05 d = 128 family: made once, by tc_prep)
     size_t img_W, img_U, img_E;    // channel-wise path on the tensor cores (bf16, d = 128): bf16 tile images of W^T, U~^T (16 KB

@@ -5,9 +5,9 @@
 //   table  : chunk table from cu_seqlens (packed sequences only)
 //   prep   : gamma = cumsum(g); A = stril(Diag(b)(K K^T . D)); P = tril(Q K^T . D); T = (I + A)^-1; W = T Diag(b Gam) K;
 //            Ut = T Diag(w) V; Kb = Diag(exp(gam_e - gam)) K; and for the backward
-//            dU0 = scale P^T dO, E = scale (Diag(Gam) Q - P W)^T dO (alone on a workspace fresh from the forward)
-//   scan   : h' = Gam_e h + Kb^T U with U = Ut - W h, and dh = Gam_e dh' + E - W^T (Kb dh') (the paper's K#1), both
-//            directions in one launch when both are wanted (ffma_scan.cuh)
+//            dU0 = scale P^T dO, E = scale (Diag(Gam) Q)^T dO (alone on a workspace fresh from the forward)
+//   scan   : h' = Gam_e h + Kb^T U with U = Ut - W h, and dh = Gam_e dh' + E - W^T dU with dU = dU0 + Kb dh' (the paper's
+//            K#1), both directions in one launch when both are wanted (ffma_scan.cuh)
 //   intra  : all token gradients of a chunk, including the VJP of the triangular solve (the paper's K#2)
 //   out    : forward output
 // One CTA handles one (chunk, head) in the parallel stages.  Operands are staged in shared memory, products are register
@@ -122,7 +122,7 @@ __device__ __forceinline__ void make_gates(const Problem& p, const ChunkInfo& x,
     }
     b += __shfl_sync(0xffffffffu, a, 31);
     const float gend = __shfl_sync(0xffffffffu, b, 31);
-    wsG[lane] = a; wsG[lane + 32] = b;
+    if (wsG) { wsG[lane] = a; wsG[lane + 32] = b; }
     finish_gates(s, lane, a, b, gend);
     load_erase_write(p, x, s, lane);
 }
@@ -134,28 +134,33 @@ __device__ __forceinline__ void load_gates(const Problem& p, const ChunkInfo& x,
 
 // ------------------------------------------------------------------------------------------------
 // prep
+//
+// Two chains of steps that share only Q, K and the gates: A -> T -> W, U~, and P -> dU0, E.  One CTA takes both (Q K^T and K K^T in one
+// pass over K), or, when that leaves half of the SMs idle, two CTAs one each (prep_parts).
 // ------------------------------------------------------------------------------------------------
 template <int DK, int DV>
-constexpr size_t prep_smem() {
-    return sizeof(float) * (kC * (2 * pitch(DK) + pitch(DK > DV ? DK : DV) + pitch(DV)) + 4 * kC * kPc);
-}
+constexpr size_t prep_smem() { return sizeof(float) * (kC * (2 * pitch(DK) + 2 * pitch(DV)) + 4 * kC * kPc); }
 
 template <typename IO, int DK, int DV>
-__global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) {
+__global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode, int parts) {
     wait_prerequisites();
-    const bool fwd = mode != PREP_BWD, bwd = mode != PREP_FWD;
+    const int item = parts == 2 ? blockIdx.x >> 1 : blockIdx.x;
+    const bool fwd = mode != PREP_BWD;
+    const bool solve = fwd && (parts == 1 || (blockIdx.x & 1) == 0);           // A, T, W, U~
+    const bool readout = parts == 1 || (blockIdx.x & 1) == 1;                  // P, Kb; with a backward dU0, E
+    const bool bwd = mode != PREP_FWD && readout;
     if (fwd) init_header_if_untabled(p); else check_fresh_seqlens(p);   // (the backward's part alone: the status word is the forward's)
     ChunkInfo x;
-    if (!chunk_info(p, x)) return;   // (no chunk at all when the table was refused)
+    if (!chunk_info(p, x, item)) return;   // (no chunk at all when the table was refused)
     constexpr int PK = pitch(DK), PV = pitch(DV);
     extern __shared__ __align__(16) float sm[];
-    float* sK = sm;                                   // K
-    float* sQ = sK + kC * PK;                         // Q, then X = Diag(Gam) Q - P W
-    float* sV = sQ + kC * PK;                         // V, then W
-    float* sO = sV + kC * pitch(DK > DV ? DK : DV);   // dO
-    float* A = sO + kC * PV;                          // A, then T Diag(w)
+    float* sK = sm;                  // K
+    float* sQ = sK + kC * PK;        // Q, then Diag(Gam) Q
+    float* sV = sQ + kC * PK;        // V
+    float* sO = sV + kC * PV;        // dO
+    float* A = sO + kC * PV;         // A, then T Diag(w)
     float* T = A + kC * kPc;
-    float* S = T + kC * kPc;                          // T Diag(b Gam)
+    float* S = T + kC * kPc;         // T Diag(b Gam)
     float* Pm = S + kC * kPc;
     __shared__ Gates gs;
     const int H = p.d.H, tid = threadIdx.x;
@@ -164,52 +169,60 @@ __global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) 
     const Out<DV> ov(t);
     const size_t rk = (size_t)H * DK, rv = (size_t)H * DV;
     float* wsG = block_of(p, p.L.gamma, x.ch, kC);
-    float* wsW = block_of(p, p.L.W, x.ch, kC * DK);
     float* wsP = block_of(p, p.L.Pm, x.ch, kC * kC);
     const float sc = p.d.scale;
 
-    load_rows<DK>(sQ, rows_of<IO>(p.q, x, H, DK), rk, x.len);
+    if (readout) load_rows<DK>(sQ, rows_of<IO>(p.q, x, H, DK), rk, x.len);
     if (fwd) load_rows<DK>(sK, rows_of<IO>(p.k, x, H, DK), rk, x.len);
     cp_commit();
-    if (fwd) {
-        load_rows<DV>(sV, rows_of<IO>(p.v, x, H, DV), rv, x.len);
-    } else {
-        load_block<kC, DK>(sV, wsW);
-        load_block<kC, kC>(Pm, wsP);
-    }
+    if (solve) load_rows<DV>(sV, rows_of<IO>(p.v, x, H, DV), rv, x.len);
+    if (!fwd) load_block<kC, kC>(Pm, wsP);
     if (bwd) load_rows<DV>(sO, rows_of<IO>(p.dO, x, H, DV), rv, x.len);
     cp_commit();
-    if (tid < 32) { if (fwd) make_gates(p, x, gs, wsG); else load_gates(p, x, gs, wsG); }
+    if (tid < 32) { if (fwd) make_gates(p, x, gs, readout ? wsG : nullptr); else load_gates(p, x, gs, wsG); }
     if (fwd) {
         cp_wait<1>();
         __syncthreads();
-        // P = tril(Q K^T . D) and A = stril(Diag(b)(K K^T . D)) in one pass over K; the decay exponent is only evaluated where
-        // j <= i (non-positive)
+        // P = tril(Q K^T . D) and A = stril(Diag(b)(K K^T . D)); the decay exponent is only evaluated where j <= i (non-positive)
         {
             float acc[8][4];
             zero(acc);
-            mac<2, A_ROW, B_ROW>(acc, sQ, sK, PK, t.rn, sK, PK, t.cn, 0, DK);
+            if (parts == 1) mac<2, A_ROW, B_ROW>(acc, sQ, sK, PK, t.rn, sK, PK, t.cn, 0, DK);
+            else if ((tid >> 7) * 32 <= (t.rn >> 4) * 16 + 15) {   // (warps whose block lies above the diagonal have nothing to add up)
+                float one[4][4];
+                zero(one);
+                mac<1, A_ROW, B_ROW>(one, solve ? sK : sQ, nullptr, PK, t.rn, sK, PK, t.cn, 0, DK);
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int y = 0; y < 4; ++y) acc[r][y] = acc[4 + r][y] = one[r][y];
+            }
 #pragma unroll
             for (int r = 0; r < 4; ++r)
 #pragma unroll
                 for (int y = 0; y < 4; ++y) {
                     const int i = t.rn + r, j = t.cn + 8 * y;
                     const float D = j <= i ? expf(gs.gam[i] - gs.gam[j]) : 0.f;
-                    const float P_ = j <= i ? acc[r][y] * D : 0.f;
-                    Pm[i * kPc + j] = P_;
-                    wsP[i * kC + j] = P_;
-                    A[i * kPc + j] = j < i ? gs.bb[i] * acc[4 + r][y] * D : 0.f;
+                    if (readout) {
+                        const float P_ = j <= i ? acc[r][y] * D : 0.f;
+                        Pm[i * kPc + j] = P_;
+                        wsP[i * kC + j] = P_;
+                    }
+                    if (solve) A[i * kPc + j] = j < i ? gs.bb[i] * acc[4 + r][y] * D : 0.f;
                 }
         }
-        // Kb = Diag(exp(gam_e - gam)) K, for the carries
-        float* wsKb = block_of(p, p.L.Kb, x.ch, kC * DK);
-        for (int e = tid; e < kC * DK / 4; e += kThreads) {
-            const int i = e / (DK / 4), c = (e % (DK / 4)) * 4;
-            float4 k = ld4(sK + i * PK + c);
-            const float w = gs.ee[i];
-            *reinterpret_cast<float4*>(wsKb + (size_t)e * 4) = make_float4(w * k.x, w * k.y, w * k.z, w * k.w);
+        if (readout) {   // Kb = Diag(exp(gam_e - gam)) K, for the carries
+            float* wsKb = block_of(p, p.L.Kb, x.ch, kC * DK);
+            for (int e = tid; e < kC * DK / 4; e += kThreads) {
+                const int i = e / (DK / 4), c = (e % (DK / 4)) * 4;
+                float4 k = ld4(sK + i * PK + c);
+                const float w = gs.ee[i];
+                *reinterpret_cast<float4*>(wsKb + (size_t)e * 4) = make_float4(w * k.x, w * k.y, w * k.z, w * k.w);
+            }
         }
         __syncthreads();
+    }
+    if (solve) {
         invert(A, T);
         cp_wait<0>();
         __syncthreads();
@@ -222,7 +235,7 @@ __global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) 
             A[i * kPc + j] = v * gs.ww[j];
         }
         __syncthreads();
-        // Ut = T Diag(w) V, then W = T Diag(b Gam) K (over V)
+        // Ut = T Diag(w) V, W = T Diag(b Gam) K
         float* wsU = block_of(p, p.L.Ut, x.ch, kC * DV);
         {
             float acc[Out<DV>::R][4];
@@ -232,23 +245,28 @@ __global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) 
 #pragma unroll
                 for (int y = 0; y < 4; ++y) wsU[ov.row(r) * DV + ov.c + 8 * y] = acc[r][y];
         }
-        __syncthreads();
+        float* wsW = block_of(p, p.L.W, x.ch, kC * DK);
         {
             float acc[Out<DK>::R][4];
             tri_product<DK, A_ROW, A_LOWER>(t, S, sK, PK, acc);
 #pragma unroll
             for (int r = 0; r < Out<DK>::R; ++r)
 #pragma unroll
-                for (int y = 0; y < 4; ++y) {
-                    wsW[ok.row(r) * DK + ok.c + 8 * y] = acc[r][y];
-                    sV[ok.row(r) * PK + ok.c + 8 * y] = acc[r][y];
-                }
+                for (int y = 0; y < 4; ++y) wsW[ok.row(r) * DK + ok.c + 8 * y] = acc[r][y];
         }
-        if (!bwd) return;
-    } else {
-        cp_wait<0>();
     }
-    __syncthreads();
+    if (!bwd) return;
+    if (!solve) {
+        cp_wait<0>();
+        __syncthreads();
+    }
+    for (int e = tid; e < kC * DK / 4; e += kThreads) {   // Diag(Gam) Q, in place
+        const int i = e / (DK / 4);
+        float4* q = reinterpret_cast<float4*>(sQ + i * PK + (e % (DK / 4)) * 4);
+        const float4 v = *q;
+        const float G = gs.Gam[i];
+        *q = make_float4(G * v.x, G * v.y, G * v.z, G * v.w);
+    }
     // dU0 = scale P^T dO
     float* wsD = block_of(p, p.L.dU, x.ch, kC * DV);
     {
@@ -259,19 +277,8 @@ __global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode) 
 #pragma unroll
             for (int y = 0; y < 4; ++y) wsD[ov.row(r) * DV + ov.c + 8 * y] = sc * acc[r][y];
     }
-    {   // X = Diag(Gam) Q - P W, in place over Q
-        float acc[Out<DK>::R][4];
-        tri_product<DK, A_ROW, A_LOWER>(t, Pm, sV, PK, acc);
-#pragma unroll
-        for (int r = 0; r < Out<DK>::R; ++r) {
-            float* q = sQ + ok.row(r) * PK + ok.c;
-            const float G = gs.Gam[ok.row(r)];
-#pragma unroll
-            for (int y = 0; y < 4; ++y) q[8 * y] = G * q[8 * y] - acc[r][y];
-        }
-    }
     __syncthreads();
-    // E = scale X^T dO, 64 rows at a time
+    // E = scale (Diag(Gam) Q)^T dO, 64 rows at a time
     float* wsE = block_of(p, p.L.E, x.ch, DK * DV);
 #pragma unroll 1
     for (int r0 = 0; r0 < DK; r0 += 64) {
@@ -616,7 +623,8 @@ cudaError_t launch_prep_t(const Problem& p, PrepMode mode, cudaStream_t st) {
     static SmemLimitOnce once;
     const cudaError_t e = once.ensure(prep_kernel<IO, DK, DV>, (uint32_t)prep_smem<DK, DV>());
     if (e != cudaSuccess) return e;
-    { StageScope t(mode == PREP_BWD ? ST_EPREP : ST_PREP, st); launch_kernel(prep_kernel<IO, DK, DV>, p.L.max_chunks * p.d.H, kThreads, prep_smem<DK, DV>(), st, p, mode); }
+    const int parts = prep_parts(p, mode);
+    { StageScope t(mode == PREP_BWD ? ST_EPREP : ST_PREP, st); launch_kernel(prep_kernel<IO, DK, DV>, p.L.max_chunks * p.d.H * parts, kThreads, prep_smem<DK, DV>(), st, p, (int)mode, parts); }
     return cudaGetLastError();
 }
 

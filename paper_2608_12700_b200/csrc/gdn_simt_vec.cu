@@ -12,7 +12,7 @@
 //   table  : chunk table from cu_seqlens (shared with the scalar-gate family)
 //   vprep  : gam = cumsum(g) per channel;  A_ij = sum_r b_i k_i k_j e^{gam_i - gam_j} (j < i);  P_ij = sum_r q_i k_j
 //            e^{gam_i - gam_j} (j <= i);  T = (I + A)^-1;  W = T (Gam . b . K);  Ut = T (w . V);  Kb_j = e^{gam_e - gam_j} . k_j;
-//            and for the backward dU0 = scale P^T dO, E = scale (Gam . Q - P W)^T dO
+//            and for the backward dU0 = scale P^T dO, E = scale (Gam . Q)^T dO
 //   vscan  : the carries (ffma_scan.cuh; the state decays by one factor per row)
 //   vintra : every token gradient, including the VJP of the triangular solve from the stored T (K#2), the gate
 //            gradients per channel, and dg by a reverse cumulative sum inside the chunk
@@ -105,9 +105,9 @@ template <int DK, int DV>
 struct PrepTiles {
     static constexpr int PM = pitch(DK > DV ? DK : DV), COPY = 96 * pitch(DK);
     static constexpr int G = 0;                       // gam, then dO
-    static constexpr int Q = G + kC * PM;             // q, scaled, then X = Gam . Q - P W
+    static constexpr int Q = G + kC * PM;             // q, scaled, then Gam . Q
     static constexpr int K = Q + kC * pitch(DK);      // k, then Gam . b . K
-    static constexpr int R = K + kC * pitch(DK);      // b . k, scaled, then w . V, then W
+    static constexpr int R = K + kC * pitch(DK);      // b . k, scaled, then w . V
     static constexpr int C = R + kC * PM;             // scaled copies of the keys, then T
     static constexpr int A = C + COPY;
     static constexpr int P = A + kC * kPc;
@@ -130,7 +130,6 @@ __device__ __forceinline__ void vprep_chunk(const Problem& p, int mode, const Ch
     const Out<DV> ov(t);
     const size_t rk = (size_t)H * DK, rv = (size_t)H * DV, base_k = ((size_t)x.tok0 * H + x.hd) * DK, base_v = ((size_t)x.tok0 * H + x.hd) * DV;
     float* wsG = block_of(p, p.L.gamma, x.ch, kC * DK);
-    float* wsW = block_of(p, p.L.W, x.ch, kC * DK);
     float* wsP = block_of(p, p.L.Pm, x.ch, kC * kC);
     const float sc = p.d.scale;
 
@@ -269,22 +268,18 @@ __device__ __forceinline__ void vprep_chunk(const Problem& p, int mode, const Ch
 #pragma unroll
                 for (int y = 0; y < 4; ++y) wsU[ov.row(r) * DV + ov.c + 8 * y] = acc[r][y];
         }
-        __syncthreads();
+        float* wsW = block_of(p, p.L.W, x.ch, kC * DK);
         {
             float acc[Out<DK>::R][4];
             tri_product<DK, A_ROW, A_LOWER>(t, T, K, PK, acc);
 #pragma unroll
             for (int r = 0; r < Out<DK>::R; ++r)
 #pragma unroll
-                for (int y = 0; y < 4; ++y) {
-                    wsW[ok.row(r) * DK + ok.c + 8 * y] = acc[r][y];
-                    R[ok.row(r) * PK + ok.c + 8 * y] = acc[r][y];
-                }
+                for (int y = 0; y < 4; ++y) wsW[ok.row(r) * DK + ok.c + 8 * y] = acc[r][y];
         }
         if (!bwd) return;
     } else {
         load_block<kC, DK>(G, wsG);
-        load_block<kC, DK>(R, wsW);
         load_block<kC, kC>(Pm, wsP);
         cp_commit();
         cp_wait<0>();
@@ -298,6 +293,12 @@ __device__ __forceinline__ void vprep_chunk(const Problem& p, int mode, const Ch
     }
     cp_wait<0>();
     __syncthreads();
+    using Qd = Quads<DK>;
+#pragma unroll 2
+    for (int n = 0; n < Qd::N; ++n) {   // Gam . Q, in place
+        const int i = Qd::row(n), c = Qd::col(n), o = i * PK + c;
+        st4(Q + o, mul4(ld4(Q + o), ld4(refs.eref[i / kB] + c)));
+    }
     // dU0 = scale P^T dO
     float* wsD = block_of(p, p.L.dU, x.ch, kC * DV);
     {
@@ -308,18 +309,8 @@ __device__ __forceinline__ void vprep_chunk(const Problem& p, int mode, const Ch
 #pragma unroll
             for (int y = 0; y < 4; ++y) wsD[ov.row(r) * DV + ov.c + 8 * y] = sc * acc[r][y];
     }
-    {   // X = Gam . Q - P W, in place over Q
-        float acc[Out<DK>::R][4];
-        tri_product<DK, A_ROW, A_LOWER>(t, Pm, R, PK, acc);
-#pragma unroll
-        for (int r = 0; r < Out<DK>::R; ++r) {
-            float* q = Q + ok.row(r) * PK + ok.c;
-#pragma unroll
-            for (int y = 0; y < 4; ++y) q[8 * y] = fmaf(q[8 * y], refs.eref[ok.row(r) / kB][ok.c + 8 * y], -acc[r][y]);
-        }
-    }
     __syncthreads();
-    // E = scale X^T dO, 64 rows at a time
+    // E = scale (Gam . Q)^T dO, 64 rows at a time
     float* wsE = block_of(p, p.L.E, x.ch, DK * DV);
 #pragma unroll 1
     for (int r0 = 0; r0 < DK; r0 += 64) {
