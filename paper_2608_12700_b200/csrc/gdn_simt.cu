@@ -16,11 +16,14 @@
 // 22 us, the backward's share of it 21 us): eight warps on an SM issue in half of the cycles, between barriers.  With the operands of every FMA read from
 // global memory, and the solve and the sums over a chunk done by single threads, the same stages took 907, 165 and 102 us
 // (2 x 4 heads of 1000 tokens); the smallest call, 2 heads of 128 tokens at d = 64, went from 370 to 53 us.
+#include <cooperative_groups.h>
+
 #include "ffma_scan.cuh"
 
 namespace gdn {
 namespace {
 
+namespace cg = cooperative_groups;
 using namespace ffma;
 
 // ------------------------------------------------------------------------------------------------
@@ -384,6 +387,91 @@ struct IntraTiles {
     static constexpr size_t BYTES = sizeof(float) * (D + 64 * PV);
 };
 
+// dg_j = sum_{i >= j} dgam_i, by warp 0: lane l owns tokens l and l + 32; `end` is the chunk-end term.
+__device__ __forceinline__ void write_dg(const Problem& p, const ChunkInfo& x, const float* dgam, float end) {
+    const int lane = threadIdx.x;
+    float a = dgam[lane], b = dgam[lane + 32] + (lane == 31 ? end : 0.f);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float ta = __shfl_down_sync(0xffffffffu, a, o), tb = __shfl_down_sync(0xffffffffu, b, o);
+        if (lane + o < 32) { a += ta; b += tb; }
+    }
+    a += __shfl_sync(0xffffffffu, b, 0);
+    float* dg = p.dg + (size_t)x.tok0 * p.d.H + x.hd;
+    if (lane < x.len) dg[(size_t)lane * p.d.H] = a;
+    if (lane + 32 < x.len) dg[(size_t)(lane + 32) * p.d.H] = b;
+}
+
+// dPD, G and Diag(b) G, dXv (and with it, if `values`, dv and <v, dXv>), from the first two groups of loads; two more groups are under way behind them.
+template <typename IO, int DV>
+__device__ __forceinline__ void intra_factors(const Problem& p, const ChunkInfo& x, const Thread& t, const Gates& gs, const float* sO, float* sX,
+                                              const float* sU, float* sT, float* sB, float* sP, float (*dot_v)[kC], bool values) {
+    constexpr int PV = pitch(DV);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const size_t rv = (size_t)p.d.H * DV;
+    const float sc = p.d.scale;
+    cp_wait<3>();
+    __syncthreads();
+    // 64 x 64 matrices: warps whose 16 x 32 block lies above the diagonal have nothing to add up
+    const bool below = (warp >> 2) * 32 <= (t.rn >> 4) * 16 + 15;
+    {   // dPD = scale tril(dO U^T) . D; the decay exponent is only evaluated where it is non-positive
+        float acc[4][4];
+        zero(acc);
+        if (below) mac<1, A_ROW, B_ROW>(acc, sO, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int i = t.rn + r, j = t.cn + 8 * y;
+                sP[i * kPc + j] = j <= i ? sc * acc[r][y] * expf(gs.gam[i] - gs.gam[j]) : 0.f;
+            }
+    }
+    cp_wait<2>();
+    __syncthreads();
+    {   // dXv = T^T dU, in place; dv = w dXv; <v, dXv>
+        const Out<DV> o(t);
+        constexpr int R = Out<DV>::R;
+        float acc[R][4], vv[R][4];
+        const IO* vp = rows_of<IO>(p.v, x, p.d.H, DV);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) vv[r][y] = values && o.row(r) < x.len ? ldf(vp + o.row(r) * rv + o.c + 8 * y) : 0.f;
+        tri_product<DV, A_COL, A_UPPER>(t, sT, sX, PV, acc);
+        __syncthreads();
+        IO* dvp = rows_of<IO>(p.dv, x, p.d.H, DV);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int i = o.row(r);
+            const float w = gs.ww[i];
+            float dot = 0.f;
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                sX[i * PV + o.c + 8 * y] = acc[r][y];
+                dot = fmaf(vv[r][y], acc[r][y], dot);
+                if (values && i < x.len) stf(dvp + i * rv + o.c + 8 * y, w * acc[r][y]);
+            }
+            dot = row_sum8(dot);
+            if ((lane & 7) == 0) dot_v[DV == 128 ? warp >> 1 : warp >> 2][i] = dot;
+        }
+    }
+    __syncthreads();
+    {   // G = -stril(dXv U^T) . D and Diag(b) G (over T)
+        float acc[4][4];
+        zero(acc);
+        if (below) mac<1, A_ROW, B_ROW>(acc, sX, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int i = t.rn + r, j = t.cn + 8 * y;
+                const float g = j < i ? -acc[r][y] * expf(gs.gam[i] - gs.gam[j]) : 0.f;
+                sT[i * kPc + j] = g;
+                sB[i * kPc + j] = gs.bb[i] * g;
+            }
+    }
+}
+
 template <typename IO, int DK, int DV>
 __global__ void __launch_bounds__(kThreads, 1) intra_kernel(Problem p) {
     wait_prerequisites();
@@ -419,66 +507,7 @@ __global__ void __launch_bounds__(kThreads, 1) intra_kernel(Problem p) {
     if (L::OWN) load_block<64, DV>(sD, wsD);
     cp_commit();
     if (tid < 32) load_gates(p, x, gs, block_of(p, p.L.gamma, x.ch, kC));
-    cp_wait<3>();
-    __syncthreads();
-    // 64 x 64 matrices: warps whose 16 x 32 block lies above the diagonal have nothing to add up
-    const bool below = (warp >> 2) * 32 <= (t.rn >> 4) * 16 + 15;
-    {   // dPD = scale tril(dO U^T) . D; the decay exponent is only evaluated where it is non-positive
-        float acc[4][4];
-        zero(acc);
-        if (below) mac<1, A_ROW, B_ROW>(acc, sO, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int y = 0; y < 4; ++y) {
-                const int i = t.rn + r, j = t.cn + 8 * y;
-                sP[i * kPc + j] = j <= i ? sc * acc[r][y] * expf(gs.gam[i] - gs.gam[j]) : 0.f;
-            }
-    }
-    cp_wait<2>();
-    __syncthreads();
-    {   // dXv = T^T dU, in place; dv = w dXv; <v, dXv>
-        const Out<DV> o(t);
-        constexpr int R = Out<DV>::R;
-        float acc[R][4], vv[R][4];
-        const IO* vp = rows_of<IO>(p.v, x, H, DV);
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int y = 0; y < 4; ++y) vv[r][y] = o.row(r) < x.len ? ldf(vp + o.row(r) * rv + o.c + 8 * y) : 0.f;
-        tri_product<DV, A_COL, A_UPPER>(t, sT, sX, PV, acc);
-        __syncthreads();
-        IO* dvp = rows_of<IO>(p.dv, x, H, DV);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int i = o.row(r);
-            const float w = gs.ww[i];
-            float dot = 0.f;
-#pragma unroll
-            for (int y = 0; y < 4; ++y) {
-                sX[i * PV + o.c + 8 * y] = acc[r][y];
-                dot = fmaf(vv[r][y], acc[r][y], dot);
-                if (i < x.len) stf(dvp + i * rv + o.c + 8 * y, w * acc[r][y]);
-            }
-            dot = row_sum8(dot);
-            if ((lane & 7) == 0) red[3][DV == 128 ? warp >> 1 : warp >> 2][i] = dot;
-        }
-    }
-    __syncthreads();
-    {   // G = -stril(dXv U^T) . D and Diag(b) G (over T)
-        float acc[4][4];
-        zero(acc);
-        if (below) mac<1, A_ROW, B_ROW>(acc, sX, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int y = 0; y < 4; ++y) {
-                const int i = t.rn + r, j = t.cn + 8 * y;
-                const float g = j < i ? -acc[r][y] * expf(gs.gam[i] - gs.gam[j]) : 0.f;
-                sT[i * kPc + j] = g;
-                sB[i * kPc + j] = gs.bb[i] * g;
-            }
-    }
+    intra_factors<IO, DV>(p, x, t, gs, sO, sX, sU, sT, sB, sP, red[3], true);
     const int w16 = (t.rn >> 4) * 16;
     float rsum = 0.f, hh = 0.f, dqq[4] = {}, drow[4] = {}, dcol[4] = {};
 #pragma unroll 1
@@ -584,21 +613,153 @@ __global__ void __launch_bounds__(kThreads, 1) intra_kernel(Problem p) {
         dgam[i] = (red[0][0][i] + red[0][1][i]) + gs.bb[i] * db - (red[2][0][i] + red[2][1][i]);
     }
     __syncthreads();
-    if (warp == 0) {   // dg_j = sum_{i >= j} dgam_i: lane l owns tokens l and l + 32
+    if (warp == 0) {
         float rs = 0.f, hs = 0.f;
 #pragma unroll
         for (int w = 0; w < kThreads / 32; ++w) { rs += part[0][w]; hs += part[1][w]; }
-        float a = dgam[lane], b = dgam[lane + 32] + (lane == 31 ? rs + gs.Gam[kC - 1] * hs : 0.f);
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float ta = __shfl_down_sync(0xffffffffu, a, o), tb = __shfl_down_sync(0xffffffffu, b, o);
-            if (lane + o < 32) { a += ta; b += tb; }
-        }
-        a += __shfl_sync(0xffffffffu, b, 0);
-        float* dg = p.dg + (size_t)x.tok0 * H + x.hd;
-        if (lane < x.len) dg[(size_t)lane * H] = a;
-        if (lane + 32 < x.len) dg[(size_t)(lane + 32) * H] = b;
+        write_dg(p, x, dgam, rs + gs.Gam[kC - 1] * hs);
     }
+}
+
+// The same by a cluster of DK / 32 CTAs, each of which makes 32 channels of dq and dk (and all of the factors, the first of them dv): for calls
+// of so few chunk-heads that most SMs would idle.  Of a [64 x 32] result a half of the warps takes dq, the other the row role of k; dk^col
+// is U dh'^T by the first half and the rest by the second.  The row sums behind dbeta and dg meet in the first CTA's hands.
+// What bounds it: latency, as every kernel of one chunk-head per SM, and the factors, which every CTA makes for itself.  Gradient stage of 4
+// chunk-heads at d = 64 27.0 -> 25.0 us; backward of 2 heads of 1024 tokens at d = 128 (four CTAs each) 102 -> 77 us.
+template <int DV>
+struct IntraSplitTiles {
+    static constexpr int PV = pitch(DV), NC = 32, PC = pitch(NC);
+    static constexpr int O = 0, X = O + kC * PV, U = X + kC * PV, T = U + kC * PV, B = T + kC * kPc, P = B + kC * kPc;   // as above
+    static constexpr int K = P + kC * kPc, Q = K + kC * PC, C = Q + kC * PC;   // slices of 32 channels; C: e (U dh'^T)
+    static constexpr int H = C + kC * PC, D = H + NC * PV;
+    static constexpr size_t BYTES = sizeof(float) * (D + NC * PV);
+};
+
+template <typename IO, int DK, int DV>
+__global__ void __launch_bounds__(kThreads, 1) intra_split_kernel(Problem p) {
+    wait_prerequisites();
+    using L = IntraSplitTiles<DV>;
+    constexpr int PV = pitch(DV), PC = L::PC, NC = L::NC, S = DK / NC;
+    const int rank = blockIdx.x % S;
+    ChunkInfo x;
+    if (reinterpret_cast<const WsHeader*>(p.ws)->status != GDN_OK || !chunk_info(p, x, (int)blockIdx.x / S)) return;   // (the whole cluster)
+    extern __shared__ __align__(16) float sm[];
+    float *sO = sm + L::O, *sX = sm + L::X, *sU = sm + L::U, *sT = sm + L::T, *sB = sm + L::B, *sP = sm + L::P, *sK = sm + L::K, *sQ = sm + L::Q,
+          *sC = sm + L::C, *sH = sm + L::H, *sD = sm + L::D;
+    __shared__ Gates gs;
+    __shared__ float dot_v[4][kC], red[3][kC];   // <v, dXv> by column block; <q, dq>, <k, dk^row>, <k, dk^col> of this CTA's channels
+    __shared__ float dgam[kC], part[2][kThreads / 32];
+    const int H = p.d.H, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const Thread t;
+    const size_t rk = (size_t)H * DK, rv = (size_t)H * DV;
+    const float sc = p.d.scale;
+
+    load_rows<DV>(sO, rows_of<IO>(p.dO, x, H, DV), rv, x.len);
+    load_block<kC, DV>(sU, block_of(p, p.L.U, x.ch, kC * DV));
+    cp_commit();
+    load_block<kC, DV>(sX, block_of(p, p.L.dU, x.ch, kC * DV));
+    load_block<kC, kC>(sT, block_of(p, p.L.Tm, x.ch, kC * kC));
+    cp_commit();
+    load_block<NC, DV>(sH, block_of(p, p.L.hc, x.ch, DK * DV) + rank * NC * DV);
+    cp_commit();
+    load_rows<NC>(sK, rows_of<IO>(p.k, x, H, DK) + rank * NC, rk, x.len);
+    load_rows<NC>(sQ, rows_of<IO>(p.q, x, H, DK) + rank * NC, rk, x.len);
+    load_block<NC, DV>(sD, block_of(p, p.L.dhn, x.ch, DK * DV) + rank * NC * DV);
+    cp_commit();
+    if (tid < 32) load_gates(p, x, gs, block_of(p, p.L.gamma, x.ch, kC));
+    intra_factors<IO, DV>(p, x, t, gs, sO, sX, sU, sT, sB, sP, dot_v, rank == 0);
+    cp_wait<0>();
+    __syncthreads();
+    const bool row = warp >= 4;              // dO and dPD, or dXv and G
+    const int w16 = (t.rn >> 4) * 16, c = lane & 7;
+    float rsum = 0.f, hh = 0.f, acc[4][4], col[4][4];
+    zero(acc);
+    zero(col);
+    mac<1, A_ROW, B_ROW>(acc, row ? sX : sO, nullptr, PV, t.rn, sH, PV, c, 0, DV);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const float a = row ? -gs.Gam[t.rn + r] : sc * gs.Gam[t.rn + r];
+#pragma unroll
+        for (int y = 0; y < 4; ++y) acc[r][y] *= a;
+    }
+    mac<1, A_ROW, B_COL>(acc, row ? sT : sP, nullptr, kPc, t.rn, sK, PC, c, 0, w16 + 16);
+    if (!row) {
+        mac<1, A_ROW, B_ROW>(col, sU, nullptr, PV, t.rn, sD, PV, c, 0, DV);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const float e = gs.ee[t.rn + r];
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int o = (t.rn + r) * PC + c + 8 * y;
+                col[r][y] *= e;
+                rsum = fmaf(sK[o], col[r][y], rsum);
+                sC[o] = col[r][y];
+            }
+        }
+    } else {
+#pragma unroll 1
+        for (int m = 0; m < 2; ++m) mac<1, A_COL, B_COL>(col, m ? sB : sP, nullptr, kPc, t.rn, m ? sK : sQ, PC, c, w16, kC);
+    }
+    for (int e = tid; e < NC * DV / 4; e += kThreads) {   // <dh', h>
+        const int o = e / (DV / 4) * PV + e % (DV / 4) * 4;
+        const float4 a = ld4(sH + o), b = ld4(sD + o);
+        hh = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, hh))));
+    }
+    __syncthreads();
+    IO* out = rows_of<IO>(row ? p.dk : p.dq, x, H, DK) + rank * NC;
+    float d0[4] = {}, d1[4] = {};   // <q, dq>; or <k, dk^row> and <k, dk^col>
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = t.rn + r;
+        const float b = gs.bb[i];
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+            const int o = i * PC + c + 8 * y;
+            const float f = row ? sK[o] : sQ[o], v = acc[r][y];
+            d0[r] = fmaf(f, v, d0[r]);
+            float res = v;
+            if (row) {
+                const float cl = sC[o] + col[r][y];
+                d1[r] = fmaf(f, cl, d1[r]);
+                res = fmaf(b, v, cl);
+            }
+            if (i < x.len) stf(out + i * rk + c + 8 * y, res);
+        }
+        d0[r] = row_sum8(d0[r]);
+        d1[r] = row_sum8(d1[r]);
+        if (c == 0) {
+            red[row ? 1 : 0][i] = d0[r];
+            if (row) red[2][i] = d1[r];
+        }
+    }
+    rsum = warp_total(rsum);
+    hh = warp_total(hh);
+    if (lane == 0) { part[0][warp] = rsum; part[1][warp] = hh; }
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    if (rank == 0) {   // (in the order of the CTAs)
+        if (tid < kC) {
+            float v[3] = {};
+#pragma unroll
+            for (int q = 0; q < S; ++q)
+#pragma unroll
+                for (int w = 0; w < 3; ++w) v[w] += cluster.map_shared_rank(&red[0][0], q)[w * kC + tid];
+            float dw = dot_v[0][tid] + dot_v[1][tid];
+            if (DV == 128) dw += dot_v[2][tid] + dot_v[3][tid];
+            if (p.d.delta_rule && tid < x.len) p.dbeta[(size_t)(x.tok0 + tid) * H + x.hd] = v[1] + dw;
+            dgam[tid] = v[0] + gs.bb[tid] * v[1] - v[2];
+        }
+        __syncthreads();
+        if (warp == 0) {
+            float rs = 0.f, hs = 0.f;
+            for (int q = 0; q < S; ++q) {
+                const float* o = cluster.map_shared_rank(&part[0][0], q);
+                for (int w = 0; w < kThreads / 32; ++w) { rs += o[w]; hs += o[kThreads / 32 + w]; }
+            }
+            write_dg(p, x, dgam, rs + gs.Gam[kC - 1] * hs);
+        }
+    }
+    cluster.sync();   // the sums have been read: the CTAs may leave
 }
 
 template <int DK, int DV, int CS>
@@ -646,7 +807,13 @@ cudaError_t launch_bwd_t(const Problem& p, bool skip_recompute, cudaStream_t st)
     if (p.cu && !skip_recompute && (e = launch_table(p, st)) != cudaSuccess) return e;
     if ((e = launch_prep_t<IO, DK, DV>(p, skip_recompute ? PREP_BWD : PREP_FWD_BWD, st)) != cudaSuccess) return e;
     if ((e = launch_scan_t<DK, DV>(p, skip_recompute ? 1 : 2, st)) != cudaSuccess) return e;
-    static SmemLimitOnce once;
+    static SmemLimitOnce once, once_split;
+    constexpr int S = DK / IntraSplitTiles<DV>::NC;
+    if (S * p.L.max_chunks * p.d.H <= tc_sm_count()) {   // every CTA of a cluster on an SM of its own
+        if ((e = once_split.ensure(intra_split_kernel<IO, DK, DV>, (uint32_t)IntraSplitTiles<DV>::BYTES)) != cudaSuccess) return e;
+        { StageScope t(ST_INTRA, st); launch_kernel_cluster(intra_split_kernel<IO, DK, DV>, S * p.L.max_chunks * p.d.H, kThreads, IntraSplitTiles<DV>::BYTES, st, S, p); }
+        return cudaGetLastError();
+    }
     if ((e = once.ensure(intra_kernel<IO, DK, DV>, (uint32_t)IntraTiles<DK, DV>::BYTES)) != cudaSuccess) return e;
     { StageScope t(ST_INTRA, st); launch_kernel(intra_kernel<IO, DK, DV>, p.L.max_chunks * p.d.H, kThreads, IntraTiles<DK, DV>::BYTES, st, p); }
     return cudaGetLastError();

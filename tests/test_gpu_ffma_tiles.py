@@ -66,8 +66,8 @@ def test_channelwise_tile_edges(dk, dv, lengths, decay):
 @pytest.mark.parametrize("dk,dv", [(64, 64), (128, 128), (128, 64), (64, 128)])
 @pytest.mark.parametrize("heads", [1, 2, 4, 9, 12])
 def test_columns_per_cta_of_the_carries(dk, dv, heads):
-    """The carries take 4, 8 or 16 state columns per CTA, by the number of chains, and the scalar-gate preparation one or two CTAs per
-    chunk-head (two up to 74 of them, 12 heads are 84): each of them, in one direction and in both,
+    """The carries take 4, 8 or 16 state columns per CTA, by the number of chains, and the scalar-gate preparation and gradient stage
+    one or several CTAs per chunk-head (preparation two up to 74 of them; gradient stage d_k / 32 while they fit 148 SMs; 12 heads are 84): each of them, in one direction and in both,
     with scalar and with per-channel gates (the same code with another decay)."""
     lengths = [130, 65]
     wl = synth.make_workload("columns", dtype="f32", lengths=lengths, H=heads, d_k=dk, d_v=dv, seed=312, states=True)
