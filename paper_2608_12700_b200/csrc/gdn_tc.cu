@@ -45,6 +45,7 @@ struct TcParams {
     int with_bwd;                          // prep: also produce E
     int scan_dirs;                         // scan: 0 = forward carry only, 1 = reverse only, 2 = both
     int lowrank;                           // carries in low-rank form (tc_scan_lr): prepared by tc_prep_lr without Nm, Bf
+    int narrow_v;                          // d_v = 64: of the kernels whose CTAs carry 64 state columns only the first half is launched
     int withhold;                          // debugging hook: a kernel leaves out one of its first loads, so that the wait for
                                            // it runs out (exercises the time-out path without any fault)
 };
@@ -517,7 +518,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
     using C = Cfg<S>;
     constexpr int NS = C::NS, NSH = NS / 2, STAGES = C::STAGES, PREFETCH_AHEAD = C::PREFETCH_AHEAD;
     constexpr uint32_t STAGE_BYTES = C::STAGE_BYTES, ADD_BYTES = C::ADD_BYTES, HT = C::HT, HT_BYTES = C::HT_BYTES;
-    const int part = (int)blockIdx.x % S, bid = (int)blockIdx.x / S;   // column block of the state, (chain, direction)
+    const int blocks = S == 2 && P.narrow_v ? 1 : S;
+    const int part = (int)blockIdx.x % blocks, bid = (int)blockIdx.x / blocks;   // column block of the state, (chain, direction)
     const Problem& p = P.p;
     const WsHeader* hdr = reinterpret_cast<const WsHeader*>(p.ws);
     if (hdr->status != GDN_OK) return;
@@ -926,7 +928,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
 }
 
 // Block index -> (chain, direction, column block): with both directions in one launch the direction is the low bit
-// (S = 1 only); with S = 2 (one direction per launch) the low bit is the column block.
+// (S = 1, or narrow_v, where the second column block is not there); with S = 2 (one direction per launch) the low bit is the column block.
 template <int S>
 __global__ void __launch_bounds__(kThreads, 1) tc_scan_lr_kernel(const __grid_constant__ TcParams P) {
     wait_prerequisites();
@@ -937,9 +939,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_lr_kernel(const __grid_co
     __shared__ uint32_t tmem_slot;
     const int bid = (int)blockIdx.x;
     if (reinterpret_cast<const WsHeader*>(P.p.ws)->status != GDN_OK) return;
-    const int rev = (S == 1 && P.scan_dirs == 2) ? (bid & 1) : P.scan_dirs;
-    const int chain = (S == 2 || P.scan_dirs == 2) ? (bid >> 1) : bid;
-    const int part = S == 2 ? (bid & 1) : 0;
+    const bool halves = S == 2 && !P.narrow_v;
+    const int rev = (!halves && P.scan_dirs == 2) ? (bid & 1) : P.scan_dirs;
+    const int chain = (halves || P.scan_dirs == 2) ? (bid >> 1) : bid;
+    const int part = halves ? (bid & 1) : 0;
     if (rev) scan_lr_chain<true, false, S>(P, chain, part, ge, ee2, bar_full, bar_mma, tmem_slot);
     else scan_lr_chain<false, false, S>(P, chain, part, ge, ee2, bar_full, bar_mma, tmem_slot);
 }
@@ -1027,6 +1030,7 @@ constexpr int kThreadsAll = kIntraThreads + 64;     // 16 readout warps, issuer,
 constexpr int kBarThreads = kIntraThreads + 32;     // ... all but the loader meet at the named barrier
 }  // namespace intra
 
+template <int DV>
 __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const __grid_constant__ TcParams P) {
     wait_prerequisites();
     using namespace intra;
@@ -1083,20 +1087,21 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     //      P, K             once the products of phase 4 are done (e3); K also read by the last readout
     //   b  V                once the staged dv has left (needed by the second readout)
     //      T, Q             once the products of phase 4 are done; Q also read by the last readout
-    constexpr uint32_t A_BYTES = 16384 + 32768 + 32768 + 16384 + 16384 + 8192, B_BYTES = 8192 + 16384 + 16384, U_BYTES = 16384;
+    constexpr uint32_t STATE_BYTES = 256 * DV, VALUE_BYTES = 128 * DV;   // h or dh'; dO, V or U~ (d_v = 64: the first half of the tiles, the rest is never looked at)
+    constexpr uint32_t A_BYTES = 16384 + 2 * STATE_BYTES + VALUE_BYTES + 16384 + 8192, B_BYTES = 8192 + 16384 + VALUE_BYTES, U_BYTES = VALUE_BYTES;
     auto load_piece = [&](int piece, const ChunkInfo& c) {
         const int cb = piece & 1;
         switch (piece) {
             case 0: case 1: tma_load_3d(sm + KT + cb * 8192, &P.tm_k, cb * 64, c.hd, c.tok0, &bar_a); break;
-            case 2: case 3: tma_load_3d(sm + OX + cb * 16384, &P.tm_do, cb * 64, c.hd, c.tok0, &bar_a); break;
-            case 4: bulk_load(sm + DH, p.ws + p.L.dhn + (size_t)c.ch * 32768, 32768, &bar_a); break;
-            case 5: bulk_load(sm + HH, p.ws + p.L.hc + (size_t)c.ch * 32768, 32768, &bar_a); break;
+            case 2: case 3: if (cb * 64 < DV) tma_load_3d(sm + OX + cb * 16384, &P.tm_do, cb * 64, c.hd, c.tok0, &bar_a); break;
+            case 4: bulk_load(sm + DH, p.ws + p.L.dhn + (size_t)c.ch * 32768, STATE_BYTES, &bar_a); break;
+            case 5: bulk_load(sm + HH, p.ws + p.L.hc + (size_t)c.ch * 32768, STATE_BYTES, &bar_a); break;
             case 6: bulk_load(sm + W0, p.ws + p.L.W + (size_t)c.ch * 16384, 8192, &bar_a); break;
             case 7: bulk_load(sm + W1, p.ws + p.L.W + (size_t)c.ch * 16384 + 8192, 8192, &bar_a); break;
             case 8: bulk_load(sm + PT, p.ws + p.L.Pm + (size_t)c.ch * 8192, 8192, &bar_a); break;
-            case 9: bulk_load(sm + UTT, p.ws + p.L.Ut + (size_t)c.ch * 16384, 16384, &bar_u); break;
+            case 9: bulk_load(sm + UTT, p.ws + p.L.Ut + (size_t)c.ch * 16384, VALUE_BYTES, &bar_u); break;
             case 10: case 11: tma_load_3d(sm + QT + cb * 8192, &P.tm_q, cb * 64, c.hd, c.tok0, &bar_b); break;
-            case 12: case 13: tma_load_3d(sm + VT + cb * 8192, &P.tm_v, cb * 64, c.hd, c.tok0, &bar_b); break;
+            case 12: case 13: if (cb * 64 < DV) tma_load_3d(sm + VT + cb * 8192, &P.tm_v, cb * 64, c.hd, c.tok0, &bar_b); break;
             case 14: bulk_load(sm + TT, p.ws + p.L.Tm + (size_t)c.ch * 8192, 8192, &bar_b); break;
             default: break;
         }
@@ -1123,7 +1128,7 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
                     for (int cb = 0; cb < 2; ++cb) prefetch_l2_tma_3d(&P.tm_k, cb * 64, nx.hd, nx.tok0);
                     prefetch_l2_bulk(p.ws + p.L.Pm + (size_t)nx.ch * 8192, 8192);
                     prefetch_l2_bulk(p.ws + p.L.Tm + (size_t)nx.ch * 8192, 8192);
-                    for (int cb = 0; cb < 2; ++cb) prefetch_l2_tma_3d(&P.tm_do, cb * 64, nx.hd, nx.tok0);
+                    for (int cb = 0; cb * 64 < DV; ++cb) prefetch_l2_tma_3d(&P.tm_do, cb * 64, nx.hd, nx.tok0);
                 }
                 if (!(lok = mbar_wait(&bar_e0, ph))) break;    // U~^T has been read by the first readout
                 if (early) { mbar_expect_tx(&bar_u, U_BYTES); pend_u = true; load_piece(9, nx); }
@@ -1131,7 +1136,7 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
                 if (early) { mbar_expect_tx(&bar_a, A_BYTES); pend_a = true; load_piece(4, nx); }   // (the first piece announces the group)
                 if (!(lok = mbar_wait(&bar_st1, ph))) break;   // dv is staged
                 if (full) {
-                    for (int cb = 0; cb * 64 < p.d.d_v; ++cb) tma_store_3d(&P.tm_dv, cb * 64, x.hd, x.tok0, sm + STG_V + cb * 8192);
+                    for (int cb = 0; cb * 64 < DV; ++cb) tma_store_3d(&P.tm_dv, cb * 64, x.hd, x.tok0, sm + STG_V + cb * 8192);
                     bulk_commit();
                 }
                 if (!(lok = mbar_wait(&bar_e2, ph))) break;    // dO, h and dXv (over W^T)
@@ -1293,7 +1298,7 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     }
     const int i0 = grp * kTG;          // first of this thread's 16 tokens (or columns of a 64-column accumulator)
     float rs = 0.f;
-    if (ok && worker) {
+    if (ok && worker && (DV == 128 || q4 < 2)) {
         const int f = q4 * 32 + lane;      // feature (lane of the transposed accumulators)
         float t2[2][8], kb2[2][8], pd2[2][8];
 #pragma unroll
@@ -1339,18 +1344,18 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     // ---- phase 2: dO U^T and dXv = T^T dU (features 0..63 on lanes 0..15, 64..127 on lanes 16..31)
     if (ok && issuer) {
         tc_fence_after();
-        mma_tile<64, 64, 128>(tmem + C_DP, op_k_major(sm + OX, 128), op_mn_major(sm + UT, 128), false);
+        mma_tile<64, 64, DV>(tmem + C_DP, op_k_major(sm + OX, 128), op_mn_major(sm + UT, 128), false);
         mma_tile<64, 64, 64>(tmem + C_DX, op_mn_major(sm + TT, 64), op_k_major(sm + DUT, 128, 0), false);
-        mma_tile<64, 64, 64>(tmem + C_DX + LB, op_mn_major(sm + TT, 64), op_k_major(sm + DUT, 128, 64), false);
+        if (DV == 128) mma_tile<64, 64, 64>(tmem + C_DX + LB, op_mn_major(sm + TT, 64), op_k_major(sm + DUT, 128, 64), false);
         mma_commit(&bar_mma);
         // U dh'^T, rows on lanes 64..127, is first read after phase 4: it runs under the readout
-        mma_tile<128, 128, 128>(tmem + C_UH, op_mn_major(sm + UT - 16384, 128), op_k_major(sm + DH, 128), false);
+        mma_tile<128, 128, DV>(tmem + C_UH, op_mn_major(sm + UT - 16384, 128), op_k_major(sm + DH, 128), false);
     }
     // <dh', h> over the whole state, while the products run (both tiles share one format, so offsets pair up)
     float hh = 0.f;
     if (worker) {
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
+        for (int t = 0; t < DV / 32; ++t) {
             float a[8], b[8];
             unpack8(*reinterpret_cast<const uint4*>(sm + HH + (threadIdx.x + t * kWideThreads) * 16), a);
             unpack8(*reinterpret_cast<const uint4*>(sm + DH + (threadIdx.x + t * kWideThreads) * 16), b);
@@ -1385,6 +1390,7 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
         const float wg = gate_sets[in_phase][4][tr];
 #pragma unroll
         for (int part = 0; part < 2; ++part) {
+            if (DV == 64 && !ga) break;
             const int chk = (ga ? 0 : 8) + (i0 >> 3) + part;   // 8-feature piece
             float (&b)[8] = v2[part];
             float t8[8];
@@ -1397,7 +1403,7 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
             }
             chunk_store(sm + STG_V, 64, tr, chk, b);
         }
-        acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+        if (DV == 128) acc += __shfl_xor_sync(0xffffffffu, acc, 16);
         if (ga) red[1][grp][tr] = acc;
     }
     tc_fence_before();
@@ -1410,9 +1416,9 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     if (ok && issuer) {
         tc_fence_after();
         mma_commit(&bar_e1);   // U dh'^T is done: dh' has been read for the last time
-        mma_tile<64, 64, 128>(tmem + C_DA, op_k_major(sm + OX, 128, 64), op_mn_major(sm + UT, 128), false);
+        mma_tile<64, 64, DV>(tmem + C_DA, op_k_major(sm + OX, 128, 64), op_mn_major(sm + UT, 128), false);
         mma_commit(&bar_mma);
-        mma_tile<128, 128, 128>(tmem + C_A1, op_k_major(sm + OX, 128), op_k_major(sm + HH, 128), false);
+        mma_tile<128, 128, DV>(tmem + C_A1, op_k_major(sm + OX, 128), op_k_major(sm + HH, 128), false);
         mma_commit(&bar_e2);   // dO, dXv and h have been read for the last time
         mma_tile<128, 128, 64>(tmem + C_C2, op_mn_major(sm + PG - 8192, 64), op_mn_major(sm + QT, 64), false);
     }
@@ -1565,7 +1571,7 @@ constexpr uint32_t IN_BYTES = 16384 + 8192 + 16384 + 16384 + 32768;
 static_assert(2 * (SMEM_BYTES + 4096) <= 228 * 1024, "two CTAs per SM");
 }  // namespace outk
 
-template <bool CW>
+template <bool CW, int DV>
 __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_constant__ TcParams P) {
     wait_prerequisites();
     using namespace outk;
@@ -1594,7 +1600,7 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
     // One mbarrier phase per trip collects all five tiles; they are issued in three pieces, each when its region is free.
     auto load_q = [&](const ChunkInfo& c, uint32_t phase) {   // thread 0; first piece of a trip: announces the whole trip's bytes
         pending_phase = phase;
-        mbar_expect_tx(&bar_in, IN_BYTES);
+        mbar_expect_tx(&bar_in, IN_BYTES - (128 - DV) * 384);
         for (int cb = 0; cb < 2; ++cb) {
             if (CW) bulk_load(sm + QT + cb * 8192, p.ws + p.L.img_QKp + (size_t)c.ch * 32768 + cb * 16384, 8192, &bar_in);
             else tma_load_3d(sm + QT + cb * 8192, &P.tm_q, cb * 64, c.hd, c.tok0, &bar_in);
@@ -1603,10 +1609,10 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
         pending = true;
     };
     auto load_up = [&](const ChunkInfo& c) {
-        bulk_load(sm + UTT, p.ws + (CW ? p.L.img_U : p.L.Ut) + (size_t)c.ch * 16384, 16384, &bar_in);
+        bulk_load(sm + UTT, p.ws + (CW ? p.L.img_U : p.L.Ut) + (size_t)c.ch * 16384, 128 * DV, &bar_in);
         bulk_load(sm + PT, p.ws + p.L.Pm + (size_t)c.ch * 8192, 8192, &bar_in);
     };
-    auto load_h = [&](const ChunkInfo& c) { bulk_load(sm + HH, p.ws + p.L.hc + (size_t)c.ch * 32768, 32768, &bar_in); };
+    auto load_h = [&](const ChunkInfo& c) { bulk_load(sm + HH, p.ws + p.L.hc + (size_t)c.ch * 32768, 256 * DV, &bar_in); };
     auto fetch_gamma = [&](const ChunkInfo& c) {   // threads 0..63: cumulative log decay of their token
         return reinterpret_cast<const float*>(p.ws + p.L.gamma)[(size_t)c.ch * kC + threadIdx.x];
     };
@@ -1641,11 +1647,11 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
             tc_fence_after();
             mma_tile<128, 64, 128>(tmem + C_WH, op_mn_major(sm + HH, 128), op_mn_major(sm + WT, 128), false);
             mma_commit(&bar_mma);
-            mma_tile<64, 128, 128>(tmem + C_QH, op_k_major(sm + QT, 64), op_mn_major(sm + HH, 128), false);
+            mma_tile<64, DV, 128>(tmem + C_QH, op_k_major(sm + QT, 64), op_mn_major(sm + HH, 128), false);
         }
         GDN_WAIT_MMA(31)
         if (!CW && ok && has_next && threadIdx.x < kC) gnext = fetch_gamma(xn);
-        if (ok) {   // U = U~ - W h in place
+        if (ok && (DV == 128 || q4 < 2)) {   // U = U~ - W h in place
             const int i0 = half * 32;
 #pragma unroll 2
             for (int part = 0; part < 4; ++part) {
@@ -1665,17 +1671,17 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
         // ---- step 2: P U (token-major)
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
-            if (CW) mma_tile<64, 128, 64>(tmem + C_QH, op_k_major(sm + PT, 64), op_k_major(sm + UTT, 128), true);
-            else mma_tile<64, 128, 64>(tmem + C_PU, op_k_major(sm + PT, 64), op_k_major(sm + UTT, 128), false);
+            if (CW) mma_tile<64, DV, 64>(tmem + C_QH, op_k_major(sm + PT, 64), op_k_major(sm + UTT, 128), true);
+            else mma_tile<64, DV, 64>(tmem + C_PU, op_k_major(sm + PT, 64), op_k_major(sm + UTT, 128), false);
             mma_commit(&bar_mma);
         }
         GDN_WAIT_MMA(32)
         if (ok && has_next && threadIdx.x == 0) { load_q(xn, in_phase ^ 1); load_up(xn); }   // every tile has been read for the last time
-        if (ok) {   // o = scale (Gam . (Q h) + P U): the sixteen low lanes of a warp own a token row and 64 columns each
+        if (ok) {   // o = scale (Gam . (Q h) + P U): the sixteen low lanes of a warp own a token row and half of the columns each
             const float coef = CW ? sc : sc * Gam[tr];
 #pragma unroll 1
-            for (int part = 0; part < 8; ++part) {
-                const int cb = half * 64 + part * 8;
+            for (int part = 0; part < DV / 16; ++part) {
+                const int cb = half * (DV / 2) + part * 8;
                 float a[8], b[8];
                 tmem_ld8(tmem + lane_base + C_QH + cb, a);
                 if (!CW) tmem_ld8(tmem + lane_base + C_PU + cb, b);
@@ -1693,7 +1699,7 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
         if (ok) {
             if (x.len == kC) {
                 if (threadIdx.x == 0) {
-                    for (int cb = 0; cb * 64 < p.d.d_v; ++cb) tma_store_3d(&P.tm_o, cb * 64, x.hd, x.tok0, sm + STG + cb * 8192);
+                    for (int cb = 0; cb * 64 < DV; ++cb) tma_store_3d(&P.tm_o, cb * 64, x.hd, x.tok0, sm + STG + cb * 8192);
                     bulk_commit();
                 }
             } else {
@@ -1746,6 +1752,7 @@ static bool fill_params(TcParams& P, const Problem& p, bool with_bwd, int scan_d
     P.with_bwd = with_bwd ? 1 : 0;
     P.scan_dirs = scan_dirs;
     P.lowrank = tc_carries_lowrank(p.d) ? 1 : 0;
+    P.narrow_v = p.d.d_v == 64 ? 1 : 0;
     P.withhold = 0;
     auto map = [&](CUtensorMap* m, const void* base, int d) { return tc::make_tmap_bf16_heads(m, base, p.Ttot, p.d.H, d); };
     if (!map(&P.tm_q, p.q, p.d.d_k) || !map(&P.tm_k, p.k, p.d.d_k) || !map(&P.tm_v, p.v, p.d.d_v)) return false;
@@ -1787,45 +1794,51 @@ static int sm_count() {
 
 // The small preparation kernels, two CTAs per SM.
 static cudaError_t launch_eprep(const TcParams& P, cudaStream_t st) {
-    static SmemLimitOnce done;
+    static SmemLimitOnce done, done64;
     const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count();
-    return launch_chunk_kernel(tc_eprep_kernel, done, eprep::SMEM_BYTES, ST_EPREP, items < ctas ? items : ctas, split::kT, P, st);
+    if (P.narrow_v) return launch_chunk_kernel(tc_eprep_kernel<64>, done64, eprep::SMEM_BYTES, ST_EPREP, items < ctas ? items : ctas, split::kT, P, st);
+    return launch_chunk_kernel(tc_eprep_kernel<128>, done, eprep::SMEM_BYTES, ST_EPREP, items < ctas ? items : ctas, split::kT, P, st);
 }
 
-static cudaError_t launch_prep_lr(const TcParams& P, cudaStream_t st) {
+template <int DV>
+static cudaError_t launch_prep_lr_t(const TcParams& P, cudaStream_t st) {
     static SmemLimitOnce done, done_fwd;
     const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count(), grid = items < ctas ? items : ctas;
-    return P.with_bwd ? launch_chunk_kernel(tc_prep_lr_kernel<true>, done, preplr::SMEM_BYTES, ST_PREP, grid, split::kT, P, st)
-                      : launch_chunk_kernel(tc_prep_lr_kernel<false>, done_fwd, preplr::SMEM_BYTES, ST_PREP, grid, split::kT, P, st);
+    return P.with_bwd ? launch_chunk_kernel(tc_prep_lr_kernel<true, DV>, done, preplr::SMEM_BYTES, ST_PREP, grid, split::kT, P, st)
+                      : launch_chunk_kernel(tc_prep_lr_kernel<false, DV>, done_fwd, preplr::SMEM_BYTES, ST_PREP, grid, split::kT, P, st);
 }
+static cudaError_t launch_prep_lr(const TcParams& P, cudaStream_t st) { return P.narrow_v ? launch_prep_lr_t<64>(P, st) : launch_prep_lr_t<128>(P, st); }
 
 static cudaError_t launch_scan(const TcParams& P, cudaStream_t st) {
     static SmemLimitOnce done;
     static SmemLimitOnce done2;
     const int ctas = P.p.d.N * P.p.d.H * (P.scan_dirs == 2 ? 2 : 1);
+    const int half_ctas = P.narrow_v ? ctas : 2 * ctas;   // ... of the kernels whose CTAs carry 64 state columns each
     if (P.lowrank) {
         static SmemLimitOnce done_lr, done_lr2;
         // the reverse carry alone (backward on a fresh workspace) with few chains: two CTAs per chain, each carrying half of
         // the state columns (measured on 64 chains of 32 chunks: reverse 64 -> 58 us; the forward carry alone became
-        // slower that way, 62 -> 66 us, and keeps one CTA per chain)
-        if (P.scan_dirs == 1 && 2 * ctas <= sm_count())
-            return launch_chunk_kernel(tc_scan_lr_kernel<2>, done_lr2, scanlr::Cfg<2>::SMEM_BYTES, ST_SCANS, 2 * ctas, kThreads, P, st);
+        // slower that way, 62 -> 66 us, and keeps one CTA per chain).  d_v = 64: half of the columns are all there are.
+        if (P.narrow_v || (P.scan_dirs == 1 && half_ctas <= sm_count()))
+            return launch_chunk_kernel(tc_scan_lr_kernel<2>, done_lr2, scanlr::Cfg<2>::SMEM_BYTES, ST_SCANS, half_ctas, kThreads, P, st);
         return launch_chunk_kernel(tc_scan_lr_kernel<1>, done_lr, scanlr::Cfg<1>::SMEM_BYTES, ST_SCANS, ctas, kThreads, P, st);
     }
     // few chains: two CTAs per (chain, direction), each carrying half of the state columns
-    if (2 * ctas <= sm_count())
-        return launch_chunk_kernel(tc_scan_kernel<2>, done2, scan::Cfg<2>::SMEM_BYTES, ST_SCANS, 2 * ctas, kThreads, P, st);
+    if (half_ctas <= sm_count())
+        return launch_chunk_kernel(tc_scan_kernel<2>, done2, scan::Cfg<2>::SMEM_BYTES, ST_SCANS, half_ctas, kThreads, P, st);
     return launch_chunk_kernel(tc_scan_kernel<1>, done, scan::Cfg<1>::SMEM_BYTES, ST_SCANS, ctas, kThreads, P, st);
 }
 static cudaError_t launch_intra(const TcParams& P, cudaStream_t st) {
-    static SmemLimitOnce done;
+    static SmemLimitOnce done, done64;
     const int items = P.p.L.max_chunks * P.p.d.H, sms = sm_count();
-    return launch_chunk_kernel(tc_intra_kernel, done, intra::SMEM_BYTES, ST_INTRA, items < sms ? items : sms, intra::kThreadsAll, P, st);
+    if (P.narrow_v) return launch_chunk_kernel(tc_intra_kernel<64>, done64, intra::SMEM_BYTES, ST_INTRA, items < sms ? items : sms, intra::kThreadsAll, P, st);
+    return launch_chunk_kernel(tc_intra_kernel<128>, done, intra::SMEM_BYTES, ST_INTRA, items < sms ? items : sms, intra::kThreadsAll, P, st);
 }
 static cudaError_t launch_out(const TcParams& P, cudaStream_t st) {
-    static SmemLimitOnce done;
+    static SmemLimitOnce done, done64;
     const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count();
-    return launch_chunk_kernel(tc_out_kernel<false>, done, outk::SMEM_BYTES, ST_OUT, items < ctas ? items : ctas, kThreads, P, st);
+    if (P.narrow_v) return launch_chunk_kernel(tc_out_kernel<false, 64>, done64, outk::SMEM_BYTES, ST_OUT, items < ctas ? items : ctas, kThreads, P, st);
+    return launch_chunk_kernel(tc_out_kernel<false, 128>, done, outk::SMEM_BYTES, ST_OUT, items < ctas ? items : ctas, kThreads, P, st);
 }
 
 int tc_sm_count() { return sm_count(); }
@@ -1837,7 +1850,7 @@ cudaError_t tc_launch_out_channelwise(const Problem& p, cudaStream_t st) {
     P.p = p;
     if (!tc::make_tmap_bf16_heads(&P.tm_o, p.o, p.Ttot, p.d.H, p.d.d_v)) return cudaErrorUnknown;
     const int items = p.L.max_chunks * p.d.H, ctas = 2 * sm_count();
-    return launch_chunk_kernel(tc_out_kernel<true>, done, outk::SMEM_BYTES, ST_OUT, items < ctas ? items : ctas, kThreads, P, st);
+    return launch_chunk_kernel(tc_out_kernel<true, 128>, done, outk::SMEM_BYTES, ST_OUT, items < ctas ? items : ctas, kThreads, P, st);
 }
 
 // Carries of the channel-wise path: dirs = 0 forward, 1 reverse, 2 both in one launch.  Needs the tile images the

@@ -31,6 +31,7 @@ constexpr uint32_t C_PDO = 0, C_E = 128;    // TMEM columns (256 allocated)
 static_assert(2 * (SMEM_BYTES + 4096) <= 228 * 1024, "two CTAs per SM");
 }  // namespace eprep
 
+template <int DV>
 __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_constant__ TcParams P) {
     wait_prerequisites();
     using namespace eprep;
@@ -60,10 +61,10 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
     // Q, dO, P and W of a trip are dead once its last product is done: the next trip's are loaded right then, under the
     // readout of E and its store (E is staged over R and (P^T dO)^T, which are dead by then too, not over an input).
     auto issue_loads = [&](const ChunkInfo& c) {   // thread 0
-        mbar_expect_tx(&bar_in, 57344);
+        mbar_expect_tx(&bar_in, 40960 + 128 * DV);
         for (int cb = 0; cb < 2; ++cb) {
             tma_load_3d(sm + QT + cb * 8192, &P.tm_q, cb * 64, c.hd, c.tok0, &bar_in);
-            tma_load_3d(sm + DOT + cb * 8192, &P.tm_do, cb * 64, c.hd, c.tok0, &bar_in);
+            if (cb * 64 < DV) tma_load_3d(sm + DOT + cb * 8192, &P.tm_do, cb * 64, c.hd, c.tok0, &bar_in);
         }
         bulk_load(sm + PT, p.ws + p.L.Pm + (size_t)c.ch * 8192, 8192, &bar_in);
         bulk_load(sm + WT, p.ws + p.L.W + (size_t)c.ch * 16384, 16384, &bar_in);
@@ -132,8 +133,8 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
         // ---- phase 2: E = Q^T R - W^T (P^T dO)
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
-            mma_tile<128, 128, 64>(tmem + C_E, op_mn_major(sm + QT, 64), op_mn_major(sm + RT, 64), false);
-            mma_tile<128, 128, 64>(tmem + C_E, op_k_major(sm + WT, 128), op_k_major(sm + PDOT, 128), true, /*neg_a=*/true);
+            mma_tile<128, DV, 64>(tmem + C_E, op_mn_major(sm + QT, 64), op_mn_major(sm + RT, 64), false);
+            mma_tile<128, DV, 64>(tmem + C_E, op_k_major(sm + WT, 128), op_k_major(sm + PDOT, 128), true, /*neg_a=*/true);
             mma_commit(&bar_mma);
         }
         GDN_WAIT_MMA(27)
@@ -142,9 +143,9 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
             fetch_gamma(xn);
         }
         if (ok) {   // E -> bf16 tile image over R and (P^T dO)^T, which no product reads any more
-            const int r = q4 * 32 + lane, c0 = grp * 64;
+            const int r = q4 * 32 + lane, c0 = grp * (DV / 2);
 #pragma unroll 1
-            for (int part = 0; part < 8; ++part) {
+            for (int part = 0; part < DV / 16; ++part) {
                 const int cb = c0 + part * 8;
                 float v[8];
                 tmem_ld8(tmem + lane_base + C_E + cb, v);
@@ -158,7 +159,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
         fence_async_smem();
         __syncthreads();
         if (warp == 0 && elect_one() && ok) {
-            bulk_store(p.ws + p.L.E + (size_t)x.ch * 32768, sm + RT, 32768);
+            bulk_store(p.ws + p.L.E + (size_t)x.ch * 32768, sm + RT, 256 * DV);
             bulk_commit();
         }
         if (!ok) break;
@@ -197,7 +198,7 @@ static_assert(TPP + 8192 <= PT && ES + 32768 <= PT && PT % 1024 == 0, "T tiles a
 static_assert(2 * (SMEM_BYTES + 4096) <= 228 * 1024, "two CTAs per SM");
 }  // namespace preplr
 
-template <bool bwd>   // with the backward's share
+template <bool bwd, int DV>   // with the backward's share
 __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_constant__ TcParams P) {
     wait_prerequisites();
     using namespace preplr;
@@ -411,13 +412,13 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             if (bwd) {
-                mma_tile<128, 128, 64>(tmem + C_E, op_mn_major(sm + QK, 128, 0), op_mn_major(sm + VO, 128, 64), false);
+                mma_tile<128, DV, 64>(tmem + C_E, op_mn_major(sm + QK, 128, 0), op_mn_major(sm + VO, 128, 64), false);
                 mma_tile<128, 64, 64>(tmem + C_E, op_k_major(sm + WT, 128), op_k_major(sm + PDOT, 64), true, /*neg_a=*/true);
-                mma_tile<128, 64, 64>(tmem + C_E + 64, op_k_major(sm + WT, 128), op_k_major(sm + PDOT + 16384, 64), true, /*neg_a=*/true);
+                if (DV == 128) mma_tile<128, 64, 64>(tmem + C_E + 64, op_k_major(sm + WT, 128), op_k_major(sm + PDOT + 16384, 64), true, /*neg_a=*/true);
             }
             bulk_store(p.ws + p.L.W + (size_t)x.ch * 16384, sm + WT, 16384);
             bulk_store(p.ws + p.L.Ut + (size_t)x.ch * 16384, sm + UTT, 8192);
-            bulk_store(p.ws + p.L.Ut + (size_t)x.ch * 16384 + 8192, sm + UTT + 16384, 8192);
+            if (DV == 128) bulk_store(p.ws + p.L.Ut + (size_t)x.ch * 16384 + 8192, sm + UTT + 16384, 8192);
             bulk_commit();
             bulk_wait_read<0>();   // T, W^T and U~^T have left: the E image and the next inputs go over them
             mma_commit(&bar_mma);
@@ -428,9 +429,9 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
             if (warp == 0) fetch_gates(xn);
         }
         if (ok && bwd) {   // E -> bf16 tile image
-            const int r = q4 * 32 + lane, c0 = grp * 64;
+            const int r = q4 * 32 + lane, c0 = grp * (DV / 2);
 #pragma unroll 2
-            for (int part = 0; part < 8; ++part) {
+            for (int part = 0; part < DV / 16; ++part) {
                 const int cb = c0 + part * 8;
                 float v[8];
                 tmem_ld8(tmem + lane_base + C_E + cb, v);
@@ -444,7 +445,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
         fence_async_smem();
         __syncthreads();
         if (warp == 0 && elect_one() && ok && bwd) {
-            bulk_store(p.ws + p.L.E + (size_t)x.ch * 32768, sm + ES, 32768);
+            bulk_store(p.ws + p.L.E + (size_t)x.ch * 32768, sm + ES, 256 * DV);
             bulk_commit();
         }
         if (!ok) break;

@@ -110,3 +110,25 @@ def test_operator_form_with_one_cta_per_chain():
     finally:
         binding.gdn_debug_force_family(0)
     check_against_oracle(wl, got)
+
+
+@pytest.mark.parametrize("carries", [OPERATOR, LOW_RANK, 0], indirect=True)
+@pytest.mark.parametrize("d_k", [128, 64])
+@pytest.mark.parametrize("lengths,H", [([70, 130, 64], 2), ([1, 63, 0, 65], 1), ([65, 40], 40)])
+def test_values_of_64_features_leave_half_of_the_tiles_alone(carries, d_k, lengths, H):
+    """d_v = 64: the second halves of the value and state tiles are neither written nor read, so a workspace (and shared memory) full of
+    NaN patterns must not show, in any form of the carries and in either arm."""
+    wl = synth.make_workload("carry_narrow", dtype="bf16", lengths=lengths, H=H, d_k=d_k, d_v=64, states=True, seed=51)
+    ref = oracle_grads(wl)
+    buf = runner.to_device(wl, want_o=True)
+    buf.workspace.fill_(0xFF)
+    runner.run_bwd(buf)
+    got = runner.fetch(buf)
+    check_against_oracle(wl, got, ref=ref)
+    buf.workspace.fill_(0xFF)
+    runner.run_fwd(buf)
+    runner.run_bwd(buf, fresh=1)
+    fresh = runner.fetch(buf)
+    assert rel(fresh["o"], ref["o"]) < TOL["bf16"] and rel(fresh["hT"], ref["hT"]) < TOL["bf16"]
+    for name in ("dq", "dk", "dv", "dg", "dbeta", "dh0"):
+        assert np.array_equal(got[name], fresh[name]), name
