@@ -317,6 +317,7 @@ gdn_status gdn_debug_read(const gdn_desc* desc, const void* workspace, const cha
     if (!q) return GDN_ERR_BAD_SHAPE;
     if (!L.has_operator && (q->off == L.Nm || q->off == L.Bf) && (strcmp(what, "Nm") == 0 || strcmp(what, "Bf") == 0))
         return GDN_ERR_BAD_SHAPE;   // not stored: the carries of this descriptor run in low-rank form
+    if (pick_path(*desc) == Path::TcBf16 && tc_carries_lowrank(*desc) && strcmp(what, "E") == 0) return GDN_ERR_BAD_SHAPE;   // (dU lies there)
     if (cudaDeviceSynchronize() != cudaSuccess) return GDN_ERR_CUDA;
     const size_t n = (size_t)q->rows * q->cols;
     const char* base = static_cast<const char*>(workspace) + q->off;

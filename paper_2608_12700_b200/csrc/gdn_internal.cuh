@@ -40,13 +40,13 @@ struct WsLayout {
     size_t ref;            // int32 [CH, d_k]      channel-wise path on the tensor cores: the reference of a chunk's decays is 2^ref
     size_t Tm;             // f32|bf16 [CH, 64, 64]    T = (I + A)^-1
     size_t W;              // [CH, 64, d_k]
-    size_t Ut;             // [CH, 64, d_v]            U~ = T Diag(w) V
+    size_t Ut;             // [CH, 64, d_v]            U~ = T Diag(w) V (tcgen05 d = 128 family, low-rank carries: U = U~ - W h after the forward carry)
     size_t Nm;             // [CH, d_k, d_k]           Kb^T W        (these two only when the carries run in operator
     size_t Bf;             // [CH, d_k, d_v]           Kb^T U~        form: has_operator; otherwise they take no space)
     int has_operator;
     size_t hc;             // [CH, d_k, d_v]           state entering the chunk
     size_t fwd_end;        // bytes needed by the forward recompute
-    size_t E;              // [CH, d_k, d_v]           scale (Gam Q - P W)^T dO (FFMA families: scale (Gam Q)^T dO)
+    size_t E;              // [CH, d_k, d_v]           scale (Gam Q - P W)^T dO (FFMA families: scale (Gam Q)^T dO; tcgen05 d = 128 family, low-rank carries: dU [CH, 64, d_v])
     size_t dhn;            // [CH, d_k, d_v]           gradient w.r.t. the state leaving the chunk
     size_t Pm;             // [CH, 64, 64]             P = tril(Q K^T . D) (tcgen05 d = 128 family: made once, by tc_prep)
     size_t img_W, img_U, img_E;    // channel-wise path on the tensor cores (bf16, d = 128): bf16 tile images of W^T, U~^T (16 KB

@@ -6,6 +6,7 @@
 //   tc_scan  (one CTA per chain and direction)
 //                                      forward carry  h'  = Gam_e h  - Nm   h  + Bf   (stores h per chunk)
 //                                      reverse carry  dh  = Gam_e dh' - Nm^T dh' + E   (the paper's K#1; stores dh')
+//   tc_prep_lr, tc_scan_lr             the same with the carries in low-rank form, which leave U and dU per chunk as well
 //   tc_intra (one CTA per chunk-head)  every token gradient, including the VJP of the triangular solve (K#2)
 //   tc_out   (optional)                forward output o
 //
@@ -661,16 +662,287 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
 // ------------------------------------------------------------------------------------------------
 // tc_scan_lr: the same carries without the d x d operator of a chunk, for shapes whose carries are bound by HBM
 // bandwidth (one CTA per chain and direction fills the machine).  With e_j = exp(gam_e - gam_j):
-//   forward   h'  = Gam_e h   + K^T Diag(e) (U~ - W h)
-//   reverse   dh  = Gam_e dh' + E - W^T Diag(e) (K dh')
-// Two dependent products per step instead of one, but tc_prep neither forms nor writes Nm and Bf (64 KB per
-// chunk-head less to write and 16 KB less to read).  Per step a ring slot receives W^T, the K tile of the chunk and
-// U~^T (forward) or E (reverse); the first product leaves (W h)^T or (K dh')^T with features on TMEM lanes and tokens
-// on columns, the readout forms the scaled bf16 operand of the second product in the same orientation, the second
-// product yields the d_k x d_v increment of the state, which lives in fp32 registers as in tc_scan.
+//   forward   U  = U~ - W h (stored over U~),                 h' = Gam_e h   + K^T Diag(e) U
+//   reverse   dU = scale P^T dO + Diag(e) K dh' (stored),     dh = Gam_e dh' + (scale Diag(Gam) Q)^T dO - W^T dU
+// U and dU are what the forward output and the gradient stage need: both are operands of the second product here, so they cost a store of
+// 16 KB each and save those kernels a phase, and with the whole of dU under W^T the additive term of the reverse carry needs neither P
+// nor W: the preparation has no share in the backward, and a backward on a workspace fresh from the forward starts with the carry.
+// Per step a ring slot receives W^T, the K tile of the chunk and U~^T (forward) or Q, dO and P (reverse); the first product leaves
+// (W h)^T or (K dh')^T with features on TMEM lanes and tokens on columns, the readout forms the bf16 operand of the second product in the
+// same orientation, the second product yields the d_k x d_v increment of the state, which lives in fp32 registers as in tc_scan.  P^T dO
+// and Q^T dO do not depend on the state: they are issued behind the first product and run under its readout.
+// 4 x 16 heads of 2048 tokens, both directions: 93 us, 216 KB per chunk-head at 4.8 TB/s, which bounds it (with the additive term E from the
+// preparation, U and dU left to the consumers, 77; the preparation took 80 us for 64, the gradient stage 115 for 105, the output of 6 x 16
+// heads of 1500 tokens 51 for 44, and a backward on the forward's workspace had a kernel more, of 38 us).
 // ------------------------------------------------------------------------------------------------
 namespace scanlr {
-constexpr int GE_CAP = 2048;
+constexpr uint32_t WT = 0, KT = 16384, XT = 32768;   // ring slot: W^T | K | forward: this CTA's part of U~^T (16 KB / S), and room for U^T behind it
+constexpr uint32_t UT = 49152;
+constexpr uint32_t QT = 32768, PT = 49152, OT = 57344;   // reverse: Q | P | this CTA's columns of dO
+constexpr uint32_t C_D1 = 0, C_D3 = 64, C_D2 = 128;      // TMEM columns: first product (64), (P^T dO)^T (64), second product (128 / S)
+// S = number of CTAs that share a chain, each carrying 128 / S state columns (the columns of the state evolve
+// independently; W and K are needed whole by every one of them).  S = 2 serves calls that run one direction only with so
+// few chains that half of the SMs would idle (the forward, the backward on a fresh workspace): a step of a half is
+// shorter, and a step's latency is what bounds those launches.
+template <int S> struct Cfg {
+    static constexpr int NS = D / S;                          // state columns of this CTA = rows of the first product
+    static constexpr int NSH = NS / 2;                        // ... of one thread
+    static constexpr int STAGES = 2;
+    static constexpr uint32_t STAGE_BYTES = OT + 16384 / S;
+    static constexpr uint32_t HT = STAGES * STAGE_BYTES;      // two bf16 state tiles [128][NS]
+    static constexpr uint32_t HT_BYTES = 32768 / S;
+    static constexpr uint32_t GT = HT + 2 * HT_BYTES;         // operand of the second product, [NS features][64 tokens]
+    static constexpr uint32_t SMEM_BYTES = GT + 16384 / S + 1024;
+    static constexpr uint32_t TMEM_COLS = 256;
+    static_assert(SMEM_BYTES + 1536 <= 227 * 1024, "shared memory budget");
+    static_assert(UT + 16384 / S <= STAGE_BYTES && STAGE_BYTES % 1024 == 0, "U^T fits behind a forward slot's tiles");
+};
+struct Gates { float ee[2][kC], gq[2][kC], ge[2]; };   // e_j, scale Gam_j and Gam_e of a step, made during the step before it
+}  // namespace scanlr
+
+// One direction of one chain (the direction is a compile-time constant: the two differ in operands and readouts).
+template <bool reverse, int S>
+__device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int part, scanlr::Gates& gates, uint64_t* bar_full, uint64_t& bar_mma,
+                                              uint32_t& tmem_slot) {
+    using namespace scanlr;
+    using C = Cfg<S>;
+    constexpr int NS = C::NS, NSH = C::NSH, STAGES = C::STAGES;
+    constexpr uint32_t STAGE_BYTES = C::STAGE_BYTES, HT = C::HT, HT_BYTES = C::HT_BYTES, GT = C::GT, VALUE_BYTES = 16384 / S;
+    const Problem& p = P.p;
+    const int H = p.d.H, n = chain / H, hd = chain % H;
+    const SeqGeom sg = seq_geom(p, n);
+    const int c0 = sg.c0, nsteps = sg.n_chunks, c1 = c0 + nsteps;
+    auto chunk_of = [&](int s) { return reverse ? (c1 - 1 - s) : (c0 + s); };
+
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* sm = align1024(smem_raw);
+    const int warp = warp_id(), lane = threadIdx.x & 31;
+    const int q4 = warp & 3, hf = warp >> 2;
+    const int r = q4 * 32 + lane;              // TMEM lane of this thread: state row (d_k) or feature of the first product (d_v)
+    const int lc0 = hf * NSH;                  // first of its NSH state columns inside the CTA's block
+    const int tk0 = hf * 32;                   // first of its 32 tokens in the first product
+    // The first product has NS rows.  With 128 of them a thread's TMEM lane is its feature; with 64 (M = 64) the rows sit
+    // on lanes 0..15 of each quadrant and the other lanes of a warp have nothing to read out.
+    const int r1 = S == 1 ? r : q4 * 16 + (lane & 15);
+    const bool act1 = S == 1 || lane < 16;
+    const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
+    const float sc = p.d.scale;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) mbar_init(&bar_full[s], 1);
+        mbar_init(&bar_mma, 1);
+        fence_mbar_init();
+    }
+    if (warp == 0) { tmem_alloc(&tmem_slot, C::TMEM_COLS); tmem_relinquish(); }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+
+    // this CTA's rows of U~^T, then U^T, or of dU^T (both images [d_v][tokens])
+    char* y_base = p.ws + (reverse ? p.L.E : p.L.Ut) + part * VALUE_BYTES;
+    char* keep_base = p.ws + (reverse ? p.L.dhn : p.L.hc) + part * HT_BYTES;
+    const float* gamma = reinterpret_cast<const float*>(p.ws + p.L.gamma);
+    // (L2 prefetches running ahead of the ring, as in tc_scan, made this kernel slower: 79.7 -> 78.5 us without)
+    auto fill = [&](int s) {   // thread 32: bring chunk step s into ring slot s % STAGES
+        const int stage = s % STAGES, c = chunk_of(s), tok0 = sg.chunk_tok0(c);
+        const size_t ch = (size_t)c * H + hd;
+        unsigned char* slot = sm + stage * STAGE_BYTES;
+        uint64_t* bar = &bar_full[stage];
+        mbar_expect_tx(bar, 32768 + VALUE_BYTES + (reverse ? 24576 : 0));
+        if (!(P.withhold == WITHHOLD_CARRY && s == 0)) bulk_load(slot + WT, p.ws + p.L.W + ch * 16384, 16384, bar);
+        for (int cb = 0; cb < 2; ++cb) tma_load_3d(slot + KT + cb * 8192, &P.tm_k, cb * 64, hd, tok0, bar);
+        if (reverse) {
+            bulk_load(slot + PT, p.ws + p.L.Pm + ch * 8192, 8192, bar);
+            for (int cb = 0; cb < 2 / S; ++cb) tma_load_3d(slot + OT + cb * 8192, &P.tm_do, part * NS + cb * 64, hd, tok0, bar);
+            for (int cb = 0; cb < 2; ++cb) tma_load_3d(slot + QT + cb * 8192, &P.tm_q, cb * 64, hd, tok0, bar);
+        } else {
+            bulk_load(slot + XT, y_base + ch * 16384, VALUE_BYTES, bar);
+        }
+    };
+    if (threadIdx.x == 32) {
+        for (int s = 0; s < STAGES && s < nsteps; ++s) fill(s);
+    }
+    // the gate arrays of the first step; the cumulative decays of the second are fetched now
+    auto gate_row = [&](int s) { return gamma + ((size_t)chunk_of(s) * H + hd) * kC; };
+    auto make_gates = [&](int set, float g, float gend) {
+        gates.ee[set][threadIdx.x] = expf(gend - g);
+        if (reverse) gates.gq[set][threadIdx.x] = sc * expf(g);
+        if (threadIdx.x == 0) gates.ge[set] = expf(gend);
+    };
+    float gnext = 0.f, gend_next = 0.f;
+    if (threadIdx.x < kC && nsteps > 0) {
+        make_gates(0, gate_row(0)[threadIdx.x], gate_row(0)[kC - 1]);
+        if (nsteps > 1) { gnext = gate_row(1)[threadIdx.x]; gend_next = gate_row(1)[kC - 1]; }
+    }
+    float st[NSH];
+    {
+        const float* init = reverse ? p.dhT : p.h0;
+        const bool inside = r < p.d.d_k && part * NS + lc0 < p.d.d_v;   // (a head dimension of 64: the rest of the state is zero)
+        const size_t soff = (((size_t)n * H + hd) * p.d.d_k + r) * p.d.d_v + part * NS + lc0;
+#pragma unroll
+        for (int k = 0; k < NSH / 4; ++k) {
+            float4 v = init && inside ? *reinterpret_cast<const float4*>(init + soff + 4 * k) : make_float4(0.f, 0.f, 0.f, 0.f);
+            st[4 * k] = v.x; st[4 * k + 1] = v.y; st[4 * k + 2] = v.z; st[4 * k + 3] = v.w;
+        }
+    }
+    __syncthreads();
+    bool ok = true;
+    uint32_t mma_phase = 0;
+    int s = 0;
+#pragma unroll 1
+    for (; s < nsteps; ++s) {
+        unsigned char* Ht = sm + HT + (s & 1) * HT_BYTES;
+        const int c = chunk_of(s), stage = s % STAGES, len = sg.chunk_len(c);
+        const size_t ch = (size_t)c * H + hd;
+        unsigned char* ring = sm + stage * STAGE_BYTES;
+        const float* ee = gates.ee[s & 1];
+        // state -> bf16: operand of the first product, and the per-chunk state the gradient stage reads
+#pragma unroll
+        for (int k = 0; k < NSH / 8; ++k) *reinterpret_cast<uint4*>(Ht + tile_chunk_off(128, r, (lc0 >> 3) + k)) = pack8(st + 8 * k);
+        if (len < kC) {   // ragged tail: the rows beyond the sequence belong to somebody else
+            ok = mbar_wait_inline(&bar_full[stage], (s / STAGES) & 1);
+            if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 12); break; }
+            zero_tail_rows(ring + KT, 64, 0, len, kThreads);
+            if (reverse) {
+                zero_tail_rows(ring + QT, 64, 0, len, kThreads);
+                for (int t = threadIdx.x; t < (kC - len) * (NS / 8); t += kThreads)
+                    *reinterpret_cast<uint4*>(ring + OT + tile_chunk_off(64, len + t / (NS / 8), t % (NS / 8))) = make_uint4(0, 0, 0, 0);
+            }
+        }
+        fence_async_smem();
+        __syncthreads();
+        const float Ge = gates.ge[s & 1];   // decay of the state over the chunk
+        if (warp == 0 && elect_one()) {
+            ok = mbar_wait_inline(&bar_full[stage], (s / STAGES) & 1);
+            if (ok) {
+                tc_fence_after();
+                // forward (W h)^T = h^T W^T ; reverse (K dh')^T = dh'^T K^T : [d_v][tokens]
+                const Operand b = reverse ? op_k_major(ring + KT, 64) : op_mn_major(ring + WT, 128);
+                mma_tile<NS, 64, 128>(tmem + C_D1, op_mn_major(Ht, 128), b, false);
+                if (reverse) mma_tile<NS, 64, 64>(tmem + C_D3, op_mn_major(ring + OT, 64), op_mn_major(ring + PT, 64), false);   // (P^T dO)^T
+            } else {
+                report_timeout(p.ws, 10);
+            }
+            bulk_store(keep_base + ch * 32768, Ht, HT_BYTES);
+            bulk_commit();
+            bulk_wait_read<1>();   // (the stores of the step before have read their tiles: they are rewritten from here on)
+            mma_commit(&bar_mma);
+        } else if (threadIdx.x == 32) {
+            if (s >= 1 && s - 1 + STAGES < nsteps) fill(s - 1 + STAGES);
+        }
+        ok = mbar_wait_inline(&bar_full[stage], (s / STAGES) & 1);
+        if (reverse) {   // scale Diag(Gam) Q in place, under the first product; its product by dO runs under the readout
+            if (ok) {
+#pragma unroll
+                for (int it = 0; it < 4; ++it) {
+                    const int i = (threadIdx.x >> 4) + 16 * it;
+                    float v[8];
+                    chunk_load(ring + QT, 64, i, threadIdx.x & 15, v);
+                    const float G = gates.gq[s & 1][i];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) v[k] *= G;
+                    chunk_store(ring + QT, 64, i, threadIdx.x & 15, v);
+                }
+            }
+            fence_async_smem();
+            __syncthreads();
+            if (warp == 0 && elect_one() && ok) mma_tile<128, NS, 64>(tmem + C_D2, op_mn_major(ring + QT, 64), op_mn_major(ring + OT, 64), false);
+        }
+        if (ok) ok = mbar_wait_inline(&bar_mma, mma_phase);
+        mma_phase ^= 1;
+        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 11); break; }
+        tc_fence_after();
+        // operand of the second product, transposed: forward Diag(e) U (and U, for the workspace), reverse dU
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            float d1[8], u[8], e8[8];
+            tmem_ld8(tmem + lane_base + C_D1 + tk0 + 8 * k, d1);
+            if (reverse) {
+                tmem_ld8(tmem + lane_base + C_D3 + tk0 + 8 * k, u);
+            } else if (act1) {
+                chunk_load(ring + XT, NS, r1, (tk0 >> 3) + k, u);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) u[j] = 0.f;
+            }
+            ld8s(ee + tk0 + 8 * k, e8);
+            tmem_wait_ld();
+            if (reverse) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) d1[j] = fmaf(sc, u[j], e8[j] * d1[j]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) u[j] -= d1[j];
+                if (act1) chunk_store(ring + UT, NS, r1, (tk0 >> 3) + k, u);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) d1[j] = e8[j] * u[j];
+            }
+            if (act1) chunk_store(sm + GT, NS, r1, (tk0 >> 3) + k, d1);
+        }
+        tc_fence_before();
+        fence_async_smem();
+        __syncthreads();
+        if (warp == 0 && elect_one()) {
+            tc_fence_after();
+            if (reverse) mma_tile<128, NS, 64>(tmem + C_D2, op_k_major(ring + WT, 128), op_k_major(sm + GT, NS), true, /*neg_a=*/true);
+            else mma_tile<128, NS, 64>(tmem + C_D2, op_mn_major(ring + KT, 64), op_k_major(sm + GT, NS), false);
+            mma_commit(&bar_mma);
+            bulk_store(y_base + ch * 16384, reverse ? sm + GT : ring + UT, VALUE_BYTES);
+            bulk_commit();
+        }
+        if (threadIdx.x < kC && s + 1 < nsteps) {   // the gate arrays of the next step, while the product runs
+            make_gates((s + 1) & 1, gnext, gend_next);
+            if (s + 2 < nsteps) { gnext = gate_row(s + 2)[threadIdx.x]; gend_next = gate_row(s + 2)[kC - 1]; }
+        }
+        ok = mbar_wait_inline(&bar_mma, mma_phase);
+        mma_phase ^= 1;
+        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 13); break; }
+        tc_fence_after();
+#pragma unroll
+        for (int k = 0; k < NSH / 8; ++k) {
+            float d2[8];
+            tmem_ld8(tmem + lane_base + C_D2 + lc0 + 8 * k, d2);
+            tmem_wait_ld();
+#pragma unroll
+            for (int j = 0; j < 8; ++j) st[8 * k + j] = fmaf(Ge, st[8 * k + j], d2[j]);
+        }
+        tc_fence_before();
+    }
+    float* fin = reverse ? p.dh0 : p.hT;
+    if (fin && ok) {
+        const bool inside = r < p.d.d_k && part * NS + lc0 < p.d.d_v;   // (a head dimension of 64: the rest of the state is zero)
+        const size_t soff = (((size_t)n * H + hd) * p.d.d_k + r) * p.d.d_v + part * NS + lc0;
+#pragma unroll
+        for (int k = 0; k < NSH / 4; ++k) if (inside) *reinterpret_cast<float4*>(fin + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
+    }
+    if (warp == 0) bulk_wait_read<0>();
+    if (threadIdx.x == 32) drain_ring<STAGES>(bar_full, s, nsteps);
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, C::TMEM_COLS);
+}
+
+// Block index -> (chain, direction, column block): with both directions in one launch the direction is the low bit
+// (S = 1, or narrow_v, where the second column block is not there); with S = 2 (one direction per launch) the low bit is the column block.
+template <int S>
+__global__ void __launch_bounds__(kThreads, 1) tc_scan_lr_kernel(const __grid_constant__ TcParams P) {
+    wait_prerequisites();
+    using namespace scanlr;
+    __shared__ __align__(16) scanlr::Gates gates;
+    __shared__ uint64_t bar_full[Cfg<S>::STAGES], bar_mma;
+    __shared__ uint32_t tmem_slot;
+    const int bid = (int)blockIdx.x;
+    if (reinterpret_cast<const WsHeader*>(P.p.ws)->status != GDN_OK) return;
+    const bool halves = S == 2 && !P.narrow_v;
+    const int rev = (!halves && P.scan_dirs == 2) ? (bid & 1) : P.scan_dirs;
+    const int chain = (halves || P.scan_dirs == 2) ? (bid >> 1) : bid;
+    const int part = halves ? (bid & 1) : 0;
+    if (rev) scan_lr_chain<true, S>(P, chain, part, gates, bar_full, bar_mma, tmem_slot);
+    else scan_lr_chain<false, S>(P, chain, part, gates, bar_full, bar_mma, tmem_slot);
+}
+
+namespace scancw {
 constexpr uint32_t WT = 0, KT = 16384, XT = 32768;   // ring slot: W^T | K | this CTA's part of U~^T (16 KB / S) or E (32 KB / S)
 constexpr uint32_t C_D1 = 0, C_D2 = 64;              // TMEM columns: first product (64), second product (128 / S)
 // S = number of CTAs that share a chain, each carrying 128 / S state columns (the columns of the state evolve
@@ -687,12 +959,12 @@ template <int S> struct Cfg {
     static constexpr uint32_t GT = HT + 2 * HT_BYTES;         // operand of the second product, [NS features][64 tokens]
     static constexpr uint32_t SMEM_BYTES = GT + 16384 / S + 1024;
     static constexpr uint32_t TMEM_COLS = S == 1 ? 256 : 128;
-    static_assert(SMEM_BYTES + GE_CAP * 4 + 2048 <= 227 * 1024, "shared memory budget");
+    static_assert(SMEM_BYTES + 2048 <= 227 * 1024, "shared memory budget");
 };
-}  // namespace scanlr
+}  // namespace scancw
 
-// One direction of one chain (the direction is a compile-time constant: the two differ in operands and readouts).
-// CW = carries of the channel-wise path (per-channel gates): the decay of the state is a vector (one factor per state
+// The carries of the channel-wise path (per-channel gates, d_k = d_v = 128, bf16 I/O) on the same machinery, with the additive term E of
+// the preparation in reverse: the decay of the state is a vector (one factor per state
 // row, i.e. per thread), and the key tile arrives as K- = S k / Gam, a tile image from the
 // workspace together with images of W^T, U~^T and E (written by the channel-wise preparation kernels), so the readout of the
 // first product applies no per-token factor.  Those images are relative to a reference S = 2^ref of the chunk (gdn_tc_cw.cu), and
@@ -702,10 +974,10 @@ template <int S> struct Cfg {
 //   reverse   w = dh' / S'',       w'  = A w + E - W^T Y       with A = Gam_e S'' / S    (S'': of the chunk before in this order, 1 at first)
 // (A scaled copy of an unscaled state, and a factor of its own for the increment, took 40 to 50 ns a step: 8 heads of 8192 tokens
 // 383 -> 388 us.)
-template <bool reverse, bool CW, int S>
-__device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int part, float* ge, float (*ee2)[kC], uint64_t* bar_full,
+template <bool reverse, int S>
+__device__ __forceinline__ void scan_cw_chain(const TcParams& P, int chain, int part, uint64_t* bar_full,
                                               uint64_t& bar_mma, uint32_t& tmem_slot) {
-    using namespace scanlr;
+    using namespace scancw;
     using C = Cfg<S>;
     constexpr int NS = C::NS, NSH = C::NSH, STAGES = C::STAGES;
     constexpr uint32_t STAGE_BYTES = C::STAGE_BYTES, HT = C::HT, HT_BYTES = C::HT_BYTES, GT = C::GT;
@@ -730,7 +1002,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     // channel-wise: log decay over the chunk and reference of this thread's state row, fetched a step ahead
     struct { float gam; int ref; } cw_next{0.f, 0};
     auto cw_fetch = [&](int s) {
-        if (CW && s < nsteps) {
+        if (s < nsteps) {
             const size_t ch = (size_t)chunk_of(s) * H + hd;
             cw_next.gam = reinterpret_cast<const float*>(p.ws + p.L.gamma)[(ch * kC + kC - 1) * D + r];
             cw_next.ref = reinterpret_cast<const int32_t*>(p.ws + p.L.ref)[ch * D + r];
@@ -751,12 +1023,11 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
-    const char* w_base = p.ws + (CW ? p.L.img_W : p.L.W);
+    const char* w_base = p.ws + p.L.img_W;
     // this CTA's part of the additive image: rows part * NS.. of U~^T [d_v][tokens], column block `part` of E [d_k][d_v]
     const uint32_t x_chunk = reverse ? 32768u : 16384u, x_bytes = x_chunk / S;
-    const char* x_base = p.ws + (reverse ? (CW ? p.L.img_E : p.L.E) : (CW ? p.L.img_U : p.L.Ut)) + part * x_bytes;
+    const char* x_base = p.ws + (reverse ? p.L.img_E : p.L.img_U) + part * x_bytes;
     char* keep_base = p.ws + (reverse ? p.L.dhn : p.L.hc) + part * HT_BYTES;
-    const float* gamma = reinterpret_cast<const float*>(p.ws + p.L.gamma);
     // (L2 prefetches running ahead of the ring, as in tc_scan, made this kernel slower: 79.7 -> 78.5 us without)
     auto fill = [&](int s) {   // thread 32: bring chunk step s into ring slot s % STAGES
         const int stage = s % STAGES, c = chunk_of(s);
@@ -764,27 +1035,12 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         unsigned char* slot = sm + stage * STAGE_BYTES;
         mbar_expect_tx(&bar_full[stage], 32768 + x_bytes);
         if (!(P.withhold == WITHHOLD_CARRY && s == 0)) bulk_load(slot + WT, w_base + ch * 16384, 16384, &bar_full[stage]);
-        if constexpr (CW) {
-            // k-, in both directions: what is left of the decay is applied to the state (row by row, below)
-            bulk_load(slot + KT, p.ws + p.L.img_Km + ch * 16384, 16384, &bar_full[stage]);
-        } else {
-            tma_load_3d(slot + KT, &P.tm_k, 0, hd, sg.chunk_tok0(c), &bar_full[stage]);
-            tma_load_3d(slot + KT + 8192, &P.tm_k, 64, hd, sg.chunk_tok0(c), &bar_full[stage]);
-        }
+        // k-, in both directions: what is left of the decay is applied to the state (row by row, below)
+        bulk_load(slot + KT, p.ws + p.L.img_Km + ch * 16384, 16384, &bar_full[stage]);
         bulk_load(slot + XT, x_base + ch * x_chunk, x_bytes, &bar_full[stage]);
     };
     if (threadIdx.x == 32) {
         for (int s = 0; s < STAGES && s < nsteps; ++s) fill(s);
-    }
-    if constexpr (!CW)
-        for (int s = threadIdx.x; s < nsteps && s < GE_CAP; s += blockDim.x)
-            ge[s] = expf(gamma[((size_t)chunk_of(s) * H + hd) * kC + kC - 1]);
-    // e_j of the first step; the cumulative decays of the second are fetched now
-    auto gate_row = [&](int s) { return gamma + ((size_t)chunk_of(s) * H + hd) * kC; };
-    float gnext = 0.f, gend_next = 0.f;
-    if (!CW && threadIdx.x < kC && nsteps > 0) {
-        ee2[0][threadIdx.x] = expf(gate_row(0)[kC - 1] - gate_row(0)[threadIdx.x]);
-        if (nsteps > 1) { gnext = gate_row(1)[threadIdx.x]; gend_next = gate_row(1)[kC - 1]; }
     }
     float st[NSH];
     {
@@ -801,7 +1057,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     bool ok = true;
     uint32_t mma_phase = 0;
     int cw_ref = 0;   // reverse: reference of the step before
-    if (CW && !reverse) {
+    if (!reverse) {
         const float S_ref = pow2(cw_next.ref);
 #pragma unroll
         for (int k = 0; k < NSH; ++k) st[k] *= S_ref;
@@ -810,19 +1066,17 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
 #pragma unroll 1
     for (; s < nsteps; ++s) {
         unsigned char* Ht = sm + HT + (s & 1) * HT_BYTES;
-        const int c = chunk_of(s), stage = s % STAGES, len = sg.chunk_len(c);
+        const int c = chunk_of(s), stage = s % STAGES;
         const size_t ch = (size_t)c * H + hd;
         unsigned char* ring = sm + stage * STAGE_BYTES;
-        const float* ee = ee2[s & 1];
-        // decay of the state over the chunk: a scalar, or (channel-wise) the factor of this thread's state row
-        float Ge = CW ? expf(cw_next.gam) : (s < GE_CAP ? ge[s] : expf(gamma[ch * kC + kC - 1]));
+        float Ge = expf(cw_next.gam);   // decay of this thread's state row over the chunk
         const int ref = cw_next.ref;
-        if (CW && reverse) { Ge *= pow2(cw_ref - ref); cw_ref = ref; }   // A
-        if (CW) cw_fetch(s + 1);
+        if (reverse) { Ge *= pow2(cw_ref - ref); cw_ref = ref; }   // A
+        cw_fetch(s + 1);
         // state -> bf16: operand of the first product, and the per-chunk state the gradient stage reads
 #pragma unroll
         for (int k = 0; k < NSH / 8; ++k) {
-            if constexpr (CW && reverse) {
+            if constexpr (reverse) {
                 float sc8[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) sc8[j] = Ge * st[8 * k + j];
@@ -830,11 +1084,6 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
             } else {
                 *reinterpret_cast<uint4*>(Ht + tile_chunk_off(128, r, (lc0 >> 3) + k)) = pack8(st + 8 * k);
             }
-        }
-        if (!CW && len < kC) {   // ragged tail: the K rows beyond the sequence belong to somebody else
-            ok = mbar_wait_inline(&bar_full[stage], (s / STAGES) & 1);
-            if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 12); break; }
-            zero_tail_rows(ring + KT, 64, 0, len, kThreads);
         }
         fence_async_smem();
         __syncthreads();
@@ -863,17 +1112,16 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         // operand of the second product: forward Diag(e)(U~ - W h), reverse Diag(e)(K dh'), transposed
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            float d1[8], u[8], e8[8];
+            float d1[8], u[8];
             if constexpr (S == 2) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) u[j] = 0.f;
             }
             tmem_ld8(tmem + lane_base + C_D1 + tk0 + 8 * k, d1);
             if (!reverse && act1) chunk_load(ring + XT, NS, r1, (tk0 >> 3) + k, u);
-            ld8s(ee + tk0 + 8 * k, e8);
             tmem_wait_ld();
 #pragma unroll
-            for (int j = 0; j < 8; ++j) d1[j] = (CW ? 1.f : e8[j]) * (reverse ? d1[j] : (u[j] - d1[j]));
+            for (int j = 0; j < 8; ++j) d1[j] = reverse ? d1[j] : u[j] - d1[j];
             if (act1) chunk_store(sm + GT, NS, r1, (tk0 >> 3) + k, d1);
         }
         tc_fence_before();
@@ -885,15 +1133,11 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
             else mma_tile<128, NS, 64>(tmem + C_D2, op_mn_major(ring + KT, 64), op_k_major(sm + GT, NS), false);
             mma_commit(&bar_mma);
         }
-        if (!CW && threadIdx.x < kC && s + 1 < nsteps) {   // e_j of the next step, while the product runs
-            ee2[(s + 1) & 1][threadIdx.x] = expf(gend_next - gnext);
-            if (s + 2 < nsteps) { gnext = gate_row(s + 2)[threadIdx.x]; gend_next = gate_row(s + 2)[kC - 1]; }
-        }
         ok = mbar_wait_inline(&bar_mma, mma_phase);
         mma_phase ^= 1;
         if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 13); break; }
         tc_fence_after();
-        if (CW && !reverse) Ge *= pow2(cw_next.ref - ref);   // A
+        if (!reverse) Ge *= pow2(cw_next.ref - ref);   // A
 #pragma unroll
         for (int k = 0; k < NSH / 8; ++k) {
             float d2[8], ad[8];
@@ -902,14 +1146,14 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
             tmem_wait_ld();
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                if (CW && !reverse) st[8 * k + j] = Ge * (st[8 * k + j] + d2[j]);
-                else st[8 * k + j] = fmaf(Ge, st[8 * k + j], reverse ? ad[j] + d2[j] : d2[j]);
+                if (!reverse) st[8 * k + j] = Ge * (st[8 * k + j] + d2[j]);
+                else st[8 * k + j] = fmaf(Ge, st[8 * k + j], ad[j] + d2[j]);
             }
         }
         tc_fence_before();
     }
     float* fin = reverse ? p.dh0 : p.hT;
-    if (CW && reverse) {
+    if (reverse) {
         const float S_ref = pow2(cw_ref);
 #pragma unroll
         for (int k = 0; k < NSH; ++k) st[k] *= S_ref;
@@ -927,32 +1171,10 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     if (warp == 0) tmem_dealloc(tmem, C::TMEM_COLS);
 }
 
-// Block index -> (chain, direction, column block): with both directions in one launch the direction is the low bit
-// (S = 1, or narrow_v, where the second column block is not there); with S = 2 (one direction per launch) the low bit is the column block.
-template <int S>
-__global__ void __launch_bounds__(kThreads, 1) tc_scan_lr_kernel(const __grid_constant__ TcParams P) {
-    wait_prerequisites();
-    using namespace scanlr;
-    __shared__ float ge[GE_CAP];
-    __shared__ __align__(16) float ee2[2][kC];   // e_j of a step, made during the step before it
-    __shared__ uint64_t bar_full[Cfg<S>::STAGES], bar_mma;
-    __shared__ uint32_t tmem_slot;
-    const int bid = (int)blockIdx.x;
-    if (reinterpret_cast<const WsHeader*>(P.p.ws)->status != GDN_OK) return;
-    const bool halves = S == 2 && !P.narrow_v;
-    const int rev = (!halves && P.scan_dirs == 2) ? (bid & 1) : P.scan_dirs;
-    const int chain = (halves || P.scan_dirs == 2) ? (bid >> 1) : bid;
-    const int part = halves ? (bid & 1) : 0;
-    if (rev) scan_lr_chain<true, false, S>(P, chain, part, ge, ee2, bar_full, bar_mma, tmem_slot);
-    else scan_lr_chain<false, false, S>(P, chain, part, ge, ee2, bar_full, bar_mma, tmem_slot);
-}
-
-// The carries of the channel-wise path (per-channel gates, d_k = d_v = 128, bf16 I/O) on the same machinery.
 template <int S>
 __global__ void __launch_bounds__(kThreads, 1) tc_scan_cw_kernel(const __grid_constant__ TcParams P) {
     wait_prerequisites();
-    using namespace scanlr;
-    __shared__ __align__(16) float ee2[2][kC];   // (unused: the key tile arrives scaled)
+    using namespace scancw;
     __shared__ uint64_t bar_full[Cfg<S>::STAGES], bar_mma;
     __shared__ uint32_t tmem_slot;
     const int bid = (int)blockIdx.x;
@@ -961,8 +1183,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_cw_kernel(const __grid_co
     const int rev = (S == 1 && P.scan_dirs == 2) ? (bid & 1) : P.scan_dirs;
     const int chain = (S == 2 || P.scan_dirs == 2) ? (bid >> 1) : bid;
     const int part = S == 2 ? (bid & 1) : 0;
-    if (rev) scan_lr_chain<true, true, S>(P, chain, part, nullptr, ee2, bar_full, bar_mma, tmem_slot);
-    else scan_lr_chain<false, true, S>(P, chain, part, nullptr, ee2, bar_full, bar_mma, tmem_slot);
+    if (rev) scan_cw_chain<true, S>(P, chain, part, bar_full, bar_mma, tmem_slot);
+    else scan_cw_chain<false, S>(P, chain, part, bar_full, bar_mma, tmem_slot);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -973,7 +1195,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_cw_kernel(const __grid_co
 //   phase 2  dO U^T ; T^T dU ; under the readout U dh'^T   -> dPD = scale tril(dO U^T) . D ; dXv ; dv ; dw
 //   phase 3  dXv U^T ; under the readout [dO; dXv] h^T ; dPD^T Q   -> G = -stril(dXv U^T) . D ; Diag(b) G
 //   phase 4  [dPD; G] K ; += (Diag(b) G)^T K               -> dq ; dk ; db ; dgamma -> dg
-// (P = tril(Q K^T . D) comes from tc_prep, which forms it anyway.)
+// (P = tril(Q K^T . D) comes from tc_prep, which forms it anyway.)  With carries in low-rank form phase 1 is not there: U and dU come from the
+// carries (FACTORS), and sum_j r_j is made of U dh'^T in the last readout.
 // The vector-Jacobian product of the triangular solve (K#2) is taken in a shorter form than its definition
 // dW = -dU h^T, dXk = T^T dW, dXv = T^T dU, dA = -stril(dXk W^T + dXv U~^T):  T^T dW = -(T^T dU) h^T, so dXk = -dXv h^T,
 // and with it dXk W^T + dXv U~^T = dXv (U~ - W h)^T = dXv U^T.  dW is never formed, dXv follows dU directly (beside dP,
@@ -993,7 +1216,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_cw_kernel(const __grid_co
 //   64-column block so that the 64 rows that count land on lanes 64..127, beside the other half of dk (the rows on lanes
 //   0..63 are made from whatever lies there and are never read).
 // * T^T dU is issued as two 64-column halves, one on lanes 0..15 and one on lanes 16..31 of each quadrant.
-// Measured on 4 x 16 heads of 2048 tokens (2048 chunk-heads): 116 us, 14.7 k cycles per chunk-head; with separate M = 64
+// Measured on 4 x 16 heads of 2048 tokens (2048 chunk-heads): 105 us with FACTORS, 116 us (14.7 k cycles per chunk-head) with phase 1; with separate M = 64
 // products, gate gradients finished by two of the readout warps and dq assembled in a readout of its own it was 144 us.
 // 8 packed sequences, 32768 tokens, 32 heads: 971 -> 763 us.
 // ------------------------------------------------------------------------------------------------
@@ -1030,7 +1253,7 @@ constexpr int kThreadsAll = kIntraThreads + 64;     // 16 readout warps, issuer,
 constexpr int kBarThreads = kIntraThreads + 32;     // ... all but the loader meet at the named barrier
 }  // namespace intra
 
-template <int DV>
+template <int DV, bool FACTORS>   // FACTORS: the carries have left U and dU (low-rank form)
 __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const __grid_constant__ TcParams P) {
     wait_prerequisites();
     using namespace intra;
@@ -1050,6 +1273,10 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     __shared__ float scal[2][kWideThreads / 32];
     __shared__ uint64_t bar_a, bar_u, bar_b, bar_ld0, bar_e0, bar_e1, bar_e2, bar_e3, bar_st1, bar_st2, bar_v, bar_kq, bar_free, bar_mma;
     __shared__ uint32_t tmem_slot;
+    // where dq and dk are staged: over dU^T and U^T, or, when the next trip's are loaded over these as early as they can be, over the place of U~^T
+    // (not used then) and dXv (rows 64..127 of its tile)
+    constexpr uint32_t SQ = FACTORS ? UTT : STG_Q, SK = FACTORS ? OX : STG_K;
+    constexpr int SK_ROWS = FACTORS ? 128 : 64, SK_ROW0 = FACTORS ? 64 : 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int q4 = warp & 3, grp = warp >> 2;
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
@@ -1081,6 +1308,7 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     bool ok = true;
 
     // The tiles of a trip arrive in three groups, one mbarrier each, loaded during the previous trip as their regions fall free:
+    // (with FACTORS: u is dU^T (once T^T dU is done, e1), U^T (with h and dO, e2) and T; K comes with b; no U~^T, W^T, P)
     //   u  U~^T             once the first readout is done (e0)
     //   a  dh'              once U dh'^T is done (e1)
     //      h, dO, W^T       once [dO; dXv] h^T is done (e2)
@@ -1088,21 +1316,23 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     //   b  V                once the staged dv has left (needed by the second readout)
     //      T, Q             once the products of phase 4 are done; Q also read by the last readout
     constexpr uint32_t STATE_BYTES = 256 * DV, VALUE_BYTES = 128 * DV;   // h or dh'; dO, V or U~ (d_v = 64: the first half of the tiles, the rest is never looked at)
-    constexpr uint32_t A_BYTES = 16384 + 2 * STATE_BYTES + VALUE_BYTES + 16384 + 8192, B_BYTES = 8192 + 16384 + VALUE_BYTES, U_BYTES = VALUE_BYTES;
+    constexpr uint32_t A_BYTES = 2 * STATE_BYTES + VALUE_BYTES + (FACTORS ? 0 : 16384 + 16384 + 8192), B_BYTES = 16384 + VALUE_BYTES + (FACTORS ? 16384 : 8192),
+                       U_BYTES = FACTORS ? 2 * VALUE_BYTES + 8192 : VALUE_BYTES;
     auto load_piece = [&](int piece, const ChunkInfo& c) {
         const int cb = piece & 1;
         switch (piece) {
-            case 0: case 1: tma_load_3d(sm + KT + cb * 8192, &P.tm_k, cb * 64, c.hd, c.tok0, &bar_a); break;
+            case 0: case 1: tma_load_3d(sm + KT + cb * 8192, &P.tm_k, cb * 64, c.hd, c.tok0, FACTORS ? &bar_b : &bar_a); break;
             case 2: case 3: if (cb * 64 < DV) tma_load_3d(sm + OX + cb * 16384, &P.tm_do, cb * 64, c.hd, c.tok0, &bar_a); break;
             case 4: bulk_load(sm + DH, p.ws + p.L.dhn + (size_t)c.ch * 32768, STATE_BYTES, &bar_a); break;
             case 5: bulk_load(sm + HH, p.ws + p.L.hc + (size_t)c.ch * 32768, STATE_BYTES, &bar_a); break;
-            case 6: bulk_load(sm + W0, p.ws + p.L.W + (size_t)c.ch * 16384, 8192, &bar_a); break;
-            case 7: bulk_load(sm + W1, p.ws + p.L.W + (size_t)c.ch * 16384 + 8192, 8192, &bar_a); break;
-            case 8: bulk_load(sm + PT, p.ws + p.L.Pm + (size_t)c.ch * 8192, 8192, &bar_a); break;
-            case 9: bulk_load(sm + UTT, p.ws + p.L.Ut + (size_t)c.ch * 16384, VALUE_BYTES, &bar_u); break;
+            case 6: if (!FACTORS) bulk_load(sm + W0, p.ws + p.L.W + (size_t)c.ch * 16384, 8192, &bar_a); break;
+            case 7: if (!FACTORS) bulk_load(sm + W1, p.ws + p.L.W + (size_t)c.ch * 16384 + 8192, 8192, &bar_a); break;
+            case 8: if (!FACTORS) bulk_load(sm + PT, p.ws + p.L.Pm + (size_t)c.ch * 8192, 8192, &bar_a); break;
+            case 9: bulk_load(sm + (FACTORS ? UT : UTT), p.ws + p.L.Ut + (size_t)c.ch * 16384, VALUE_BYTES, &bar_u); break;
             case 10: case 11: tma_load_3d(sm + QT + cb * 8192, &P.tm_q, cb * 64, c.hd, c.tok0, &bar_b); break;
             case 12: case 13: if (cb * 64 < DV) tma_load_3d(sm + VT + cb * 8192, &P.tm_v, cb * 64, c.hd, c.tok0, &bar_b); break;
-            case 14: bulk_load(sm + TT, p.ws + p.L.Tm + (size_t)c.ch * 8192, 8192, &bar_b); break;
+            case 15: if (FACTORS) bulk_load(sm + DUT, p.ws + p.L.E + (size_t)c.ch * 16384, VALUE_BYTES, &bar_u); break;
+            case 14: bulk_load(sm + TT, p.ws + p.L.Tm + (size_t)c.ch * 8192, 8192, FACTORS ? &bar_u : &bar_b); break;
             default: break;
         }
     };
@@ -1126,14 +1356,15 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
                 if (!(lok = mbar_wait(&bar_ld0, ph))) break;   // the trip is under way: the late loads of the next one -> L2
                 if (early) {
                     for (int cb = 0; cb < 2; ++cb) prefetch_l2_tma_3d(&P.tm_k, cb * 64, nx.hd, nx.tok0);
-                    prefetch_l2_bulk(p.ws + p.L.Pm + (size_t)nx.ch * 8192, 8192);
+                    if (!FACTORS) prefetch_l2_bulk(p.ws + p.L.Pm + (size_t)nx.ch * 8192, 8192);
                     prefetch_l2_bulk(p.ws + p.L.Tm + (size_t)nx.ch * 8192, 8192);
                     for (int cb = 0; cb * 64 < DV; ++cb) prefetch_l2_tma_3d(&P.tm_do, cb * 64, nx.hd, nx.tok0);
                 }
-                if (!(lok = mbar_wait(&bar_e0, ph))) break;    // U~^T has been read by the first readout
-                if (early) { mbar_expect_tx(&bar_u, U_BYTES); pend_u = true; load_piece(9, nx); }
+                if (!FACTORS && !(lok = mbar_wait(&bar_e0, ph))) break;    // U~^T has been read by the first readout
+                if (early && !FACTORS) { mbar_expect_tx(&bar_u, U_BYTES); pend_u = true; load_piece(9, nx); }
                 if (!(lok = mbar_wait(&bar_e1, ph))) break;    // dh'
                 if (early) { mbar_expect_tx(&bar_a, A_BYTES); pend_a = true; load_piece(4, nx); }   // (the first piece announces the group)
+                if (early && FACTORS) { mbar_expect_tx(&bar_u, U_BYTES); pend_u = true; load_piece(15, nx); }   // dU
                 if (!(lok = mbar_wait(&bar_st1, ph))) break;   // dv is staged
                 if (full) {
                     for (int cb = 0; cb * 64 < DV; ++cb) tma_store_3d(&P.tm_dv, cb * 64, x.hd, x.tok0, sm + STG_V + cb * 8192);
@@ -1141,6 +1372,7 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
                 }
                 if (!(lok = mbar_wait(&bar_e2, ph))) break;    // dO, h and dXv (over W^T)
                 if (early) {
+                    if (FACTORS) load_piece(9, nx);
                     load_piece(5, nx);
                     load_piece(6, nx);
                     load_piece(7, nx);
@@ -1156,20 +1388,20 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
                     load_piece(13, nx);
                 }
                 if (!(lok = mbar_wait(&bar_e3, ph))) break;    // the products of phase 4 are done: Diag(b) G (over P), G (over T)
-                if (early) { load_piece(8, nx); }
+                if (early) { load_piece(FACTORS ? 14 : 8, nx); }
                 if (!(lok = mbar_wait(&bar_kq, ph))) break;    // ... and the readout holds its rows of K and Q
                 if (early) {
                     load_piece(0, nx);
                     load_piece(1, nx);
-                    load_piece(14, nx);
+                    if (!FACTORS) load_piece(14, nx);
                     load_piece(10, nx);
                     load_piece(11, nx);
                 }
                 if (!(lok = mbar_wait(&bar_st2, ph))) break;   // dq, dk are staged
                 if (full) {
                     for (int cb = 0; cb * 64 < p.d.d_k; ++cb) {
-                        tma_store_3d(&P.tm_dq, cb * 64, x.hd, x.tok0, sm + STG_Q + cb * 8192);
-                        tma_store_3d(&P.tm_dk, cb * 64, x.hd, x.tok0, sm + STG_K + cb * 8192);
+                        tma_store_3d(&P.tm_dq, cb * 64, x.hd, x.tok0, sm + SQ + cb * 8192);
+                        tma_store_3d(&P.tm_dk, cb * 64, x.hd, x.tok0, sm + SK + SK_ROW0 * 128 + cb * SK_ROWS * 128);
                     }
                     bulk_commit();
                 }
@@ -1179,7 +1411,7 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
                     mbar_expect_tx(&bar_u, U_BYTES);
                     pend_a = pend_b = pend_u = true;
 #pragma unroll 1
-                    for (int piece = 0; piece <= 14; ++piece) load_piece(piece, nx);
+                    for (int piece = 0; piece <= 15; ++piece) load_piece(piece, nx);
                 }
                 bulk_wait_read<0>();
                 mbar_arrive(&bar_free);   // the staging regions may be rewritten
@@ -1250,10 +1482,13 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     };
     // first trip: every group is loaded at once, one instruction per warp
     if (issuer) { mbar_expect_tx(&bar_a, A_BYTES); mbar_expect_tx(&bar_b, B_BYTES); mbar_expect_tx(&bar_u, U_BYTES); }
-    if (lane == 0 && warp < 15 && !(P.withhold == WITHHOLD_GRADIENT && warp == 9)) load_piece(warp, xn);
+    if (lane == 0 && warp < 16 && !(P.withhold == WITHHOLD_GRADIENT && warp == 9)) load_piece(warp, xn);
     if (gates) { fetch_gates(xn); make_gates(0); }
+    unsigned char* const sm_base = sm;
 #pragma unroll 1
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, in_phase ^= 1) {
+    unsigned char* sm = sm_base;
+    if (FACTORS) asm volatile("" : "+l"(sm));   // (addresses of tiles are made where they are used: kept over the trip they cost spills)
     const ChunkInfo x = xn;
     // this trip's gate arrays (the barrier before phase 1 publishes them)
     const float* gl = gate_sets[in_phase][0];
@@ -1264,15 +1499,27 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     const bool first = item == (int)blockIdx.x, full = x.len == kC;
     if (has_next) chunk_entry(p, xn, item + gridDim.x);
 
+    const int i0 = grp * kTG;          // first of this thread's 16 tokens (or columns of a 64-column accumulator)
+    float rs = 0.f;
+    if (FACTORS && gates && have_prev && ok) finish_gates();   // the previous chunk's gate gradients (what they are made of is rewritten below)
     if (ok) {
         ok = mbar_wait(&bar_a, in_phase);
         if (!ok && threadIdx.x == 0) report_timeout(p.ws, 20);
     }
+    if (FACTORS && ok) {
+        ok = mbar_wait(&bar_u, in_phase);
+        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 27);
+    }
+    if (FACTORS && ok && !first) {   // dXv goes where the previous trip's dk is staged, dq over its dq: the stores must have read them
+        ok = mbar_wait(&bar_free, in_phase ^ 1);
+        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 28);
+    }
     if (ok && !full) {
-        zero_tail_rows(sm + KT, 64, 0, x.len, kWideThreads);
+        if (!FACTORS) zero_tail_rows(sm + KT, 64, 0, x.len, kWideThreads);
         zero_tail_rows(sm + OX, 128, 0, x.len, kWideThreads);
         fence_async_smem();
     }
+    if constexpr (!FACTORS) {
     cta_sync();
 
     // ---- phase 1: (W h)^T, (K dh')^T, (P^T dO)^T
@@ -1296,8 +1543,6 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
         ok = mbar_wait(&bar_free, in_phase ^ 1);
         if (!ok && threadIdx.x == 0) report_timeout(p.ws, 28);
     }
-    const int i0 = grp * kTG;          // first of this thread's 16 tokens (or columns of a 64-column accumulator)
-    float rs = 0.f;
     if (ok && worker && (DV == 128 || q4 < 2)) {
         const int f = q4 * 32 + lane;      // feature (lane of the transposed accumulators)
         float t2[2][8], kb2[2][8], pd2[2][8];
@@ -1335,6 +1580,8 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     fence_async_smem();
     cta_sync();
     if (threadIdx.x == 32) mbar_arrive(&bar_e0);   // U~^T has been read
+    }
+    else { cta_sync(); }
 
     // Token-major accumulators with 64 rows (M = 64) occupy lanes 0..15 of each quadrant, or lanes 16..31 (address + 16 lanes).
     constexpr uint32_t LB = 16u << 16;
@@ -1362,8 +1609,21 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
 #pragma unroll
             for (int k = 0; k < 8; ++k) hh = fmaf(a[k], b[k], hh);
         }
+        if (FACTORS) {   // (the gate warp has read the previous trip's)
+            hh = warp_sum(hh);
+            if (lane == 0) scal[1][warp] = hh;
+        }
     }
+    if (FACTORS && threadIdx.x == 32) mbar_arrive(&bar_ld0);
     if (gates && has_next) fetch_gates(xn);
+    if (FACTORS && ok) {   // V is needed now, Q from phase 3 on, K from phase 4 on
+        ok = mbar_wait(&bar_b, in_phase);
+        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 31);
+        if (ok && !full) {
+            zero_tail_rows(sm + QT, 64, 0, x.len, kWideThreads);
+            zero_tail_rows(sm + KT, 64, 0, x.len, kWideThreads);
+        }
+    }
     GDN_WAIT_MMA(23)
     if (ok && worker) {
         float v2[2][8];
@@ -1488,11 +1748,11 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
                     b[j] = fmaf(coef, a[j], b[j]);
                     acc = fmaf(t8[j], b[j], acc);
                 }
-                chunk_store(sm + STG_Q, 64, i, cb >> 3, b);
+                chunk_store(sm + SQ, 64, i, cb >> 3, b);
             }
             red[0][grp][i] = acc;     // <q, dq>
         } else if (ok) {
-            float acc_col = 0.f, acc_db = 0.f;   // <k, dk^col> ; db = <k, G K + Gam dXk>
+            float acc_c = 0.f, acc_r = 0.f, acc_db = 0.f;   // <k, dk^col> in its two parts ; db = <k, G K + Gam dXk>
             const float e6 = ee[i], b6 = bb[i];
 #pragma unroll
             for (int part = 0; part < 4; ++part) {
@@ -1508,19 +1768,24 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
                 for (int j = 0; j < 8; ++j) {
                     const float kcol = fmaf(e6, d8[j], c8[j]);       // dk^col
                     const float t = fmaf(-G, b[j], a[j]);            // G K + Gam dXk
-                    acc_col = fmaf(kk[j], kcol, acc_col);
+                    acc_c = fmaf(kk[j], kcol, acc_c);
+                    if (FACTORS) acc_r = fmaf(kk[j], d8[j], acc_r);
                     acc_db = fmaf(kk[j], t, acc_db);
                     a[j] = fmaf(b6, t, kcol);
                 }
-                chunk_store(sm + STG_K, 64, i, cb >> 3, a);
+                chunk_store(sm + SK, SK_ROWS, SK_ROW0 + i, cb >> 3, a);
             }
             red[2][grp][i] = acc_db;
-            red[3][grp][i] = acc_col;
+            if (FACTORS) rs = e6 * acc_r;   // (its share of sum_j r_j; in the other form the first readout has made it)
+            red[3][grp][i] = acc_c;
         }
         // block totals of sum_j r_j and <dh', h>
         rs = warp_sum(rs);
-        hh = warp_sum(hh);
-        if (lane == 0) { scal[0][warp] = rs; scal[1][warp] = hh; }
+        if (!FACTORS) hh = warp_sum(hh);
+        if (lane == 0) {
+            scal[0][warp] = rs;
+            if (!FACTORS) scal[1][warp] = hh;
+        }
     }
     // The token-wise sums are turned into dbeta and dg by the gate warp during the next trip's first products.  It keeps what
     // the next trip overwrites: this chunk's gates and place.
@@ -1535,8 +1800,8 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     cta_sync();   // every reader of this trip's tiles and scratch is done
     if (threadIdx.x == 32) mbar_arrive(&bar_st2);   // dq, dk are staged: the loader stores them
     if (ok && !full) {
-        flush_rows(sm + STG_Q, p.dq, x, H, p.d.d_k, kWideThreads);
-        flush_rows(sm + STG_K, p.dk, x, H, p.d.d_k, kWideThreads);
+        flush_rows(sm + SQ, p.dq, x, H, p.d.d_k, kWideThreads);
+        flush_rows(sm + SK, p.dk, x, H, p.d.d_k, kWideThreads, SK_ROWS, SK_ROW0);
     }
     if (!ok) {   // a load of this trip may still be in flight: wait for it (bounded) before the CTA retires
         if (threadIdx.x == 0) { (void)mbar_wait(&bar_a, in_phase); (void)mbar_wait(&bar_u, in_phase); (void)mbar_wait(&bar_b, in_phase); }
@@ -1548,7 +1813,8 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
 }
 
 // ------------------------------------------------------------------------------------------------
-// tc_out (optional forward output): o = scale (Diag(Gam) Q h + P (U~ - W h)),  P = tril(Q K^T . D)
+// tc_out (optional forward output): o = scale (Diag(Gam) Q h + P U),  P = tril(Q K^T . D),  U = U~ - W h made here or, with carries in
+// low-rank form, left by the forward carry (FACTORS: one step instead of two; 6 x 16 heads of 1500 tokens 51 -> 44 us)
 //
 // Persistent, two CTAs per SM (89 KB of shared memory, 256 TMEM columns each): a CTA walks through the dependent
 // steps of one chunk-head while its neighbour is in another step of another one.  The tiles of the next trip are
@@ -1571,7 +1837,7 @@ constexpr uint32_t IN_BYTES = 16384 + 8192 + 16384 + 16384 + 32768;
 static_assert(2 * (SMEM_BYTES + 4096) <= 228 * 1024, "two CTAs per SM");
 }  // namespace outk
 
-template <bool CW, int DV>
+template <bool CW, int DV, bool FACTORS>   // FACTORS: the forward carry has left U where U~ was (low-rank form)
 __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_constant__ TcParams P) {
     wait_prerequisites();
     using namespace outk;
@@ -1600,12 +1866,12 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
     // One mbarrier phase per trip collects all five tiles; they are issued in three pieces, each when its region is free.
     auto load_q = [&](const ChunkInfo& c, uint32_t phase) {   // thread 0; first piece of a trip: announces the whole trip's bytes
         pending_phase = phase;
-        mbar_expect_tx(&bar_in, IN_BYTES - (128 - DV) * 384);
+        mbar_expect_tx(&bar_in, IN_BYTES - (128 - DV) * 384 - (FACTORS ? 16384 : 0));
         for (int cb = 0; cb < 2; ++cb) {
             if (CW) bulk_load(sm + QT + cb * 8192, p.ws + p.L.img_QKp + (size_t)c.ch * 32768 + cb * 16384, 8192, &bar_in);
             else tma_load_3d(sm + QT + cb * 8192, &P.tm_q, cb * 64, c.hd, c.tok0, &bar_in);
         }
-        bulk_load(sm + WT, p.ws + (CW ? p.L.img_W : p.L.W) + (size_t)c.ch * 16384, 16384, &bar_in);
+        if (!FACTORS) bulk_load(sm + WT, p.ws + (CW ? p.L.img_W : p.L.W) + (size_t)c.ch * 16384, 16384, &bar_in);
         pending = true;
     };
     auto load_up = [&](const ChunkInfo& c) {
@@ -1642,6 +1908,7 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
             fence_async_smem();
         }
         __syncthreads();
+        if constexpr (!FACTORS) {
         // ---- step 1: (W h)^T ; under its readout Q h
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
@@ -1650,7 +1917,6 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
             mma_tile<64, DV, 128>(tmem + C_QH, op_k_major(sm + QT, 64), op_mn_major(sm + HH, 128), false);
         }
         GDN_WAIT_MMA(31)
-        if (!CW && ok && has_next && threadIdx.x < kC) gnext = fetch_gamma(xn);
         if (ok && (DV == 128 || q4 < 2)) {   // U = U~ - W h in place
             const int i0 = half * 32;
 #pragma unroll 2
@@ -1668,9 +1934,12 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
         tc_fence_before();
         fence_async_smem();
         __syncthreads();
+        }
+        if (!CW && ok && has_next && threadIdx.x < kC) gnext = fetch_gamma(xn);
         // ---- step 2: P U (token-major)
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
+            if (FACTORS) mma_tile<64, DV, 128>(tmem + C_QH, op_k_major(sm + QT, 64), op_mn_major(sm + HH, 128), false);   // Q h
             if (CW) mma_tile<64, DV, 64>(tmem + C_QH, op_k_major(sm + PT, 64), op_k_major(sm + UTT, 128), true);
             else mma_tile<64, DV, 64>(tmem + C_PU, op_k_major(sm + PT, 64), op_k_major(sm + UTT, 128), false);
             mma_commit(&bar_mma);
@@ -1802,10 +2071,9 @@ static cudaError_t launch_eprep(const TcParams& P, cudaStream_t st) {
 
 template <int DV>
 static cudaError_t launch_prep_lr_t(const TcParams& P, cudaStream_t st) {
-    static SmemLimitOnce done, done_fwd;
-    const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count(), grid = items < ctas ? items : ctas;
-    return P.with_bwd ? launch_chunk_kernel(tc_prep_lr_kernel<true, DV>, done, preplr::SMEM_BYTES, ST_PREP, grid, split::kT, P, st)
-                      : launch_chunk_kernel(tc_prep_lr_kernel<false, DV>, done_fwd, preplr::SMEM_BYTES, ST_PREP, grid, split::kT, P, st);
+    static SmemLimitOnce done;
+    const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count();
+    return launch_chunk_kernel(tc_prep_lr_kernel<DV>, done, preplr::SMEM_BYTES, ST_PREP, items < ctas ? items : ctas, split::kT, P, st);
 }
 static cudaError_t launch_prep_lr(const TcParams& P, cudaStream_t st) { return P.narrow_v ? launch_prep_lr_t<64>(P, st) : launch_prep_lr_t<128>(P, st); }
 
@@ -1828,17 +2096,25 @@ static cudaError_t launch_scan(const TcParams& P, cudaStream_t st) {
         return launch_chunk_kernel(tc_scan_kernel<2>, done2, scan::Cfg<2>::SMEM_BYTES, ST_SCANS, half_ctas, kThreads, P, st);
     return launch_chunk_kernel(tc_scan_kernel<1>, done, scan::Cfg<1>::SMEM_BYTES, ST_SCANS, ctas, kThreads, P, st);
 }
-static cudaError_t launch_intra(const TcParams& P, cudaStream_t st) {
-    static SmemLimitOnce done, done64;
+template <int DV, bool FACTORS>
+static cudaError_t launch_intra_t(const TcParams& P, cudaStream_t st) {
+    static SmemLimitOnce done;
     const int items = P.p.L.max_chunks * P.p.d.H, sms = sm_count();
-    if (P.narrow_v) return launch_chunk_kernel(tc_intra_kernel<64>, done64, intra::SMEM_BYTES, ST_INTRA, items < sms ? items : sms, intra::kThreadsAll, P, st);
-    return launch_chunk_kernel(tc_intra_kernel<128>, done, intra::SMEM_BYTES, ST_INTRA, items < sms ? items : sms, intra::kThreadsAll, P, st);
+    return launch_chunk_kernel(tc_intra_kernel<DV, FACTORS>, done, intra::SMEM_BYTES, ST_INTRA, items < sms ? items : sms, intra::kThreadsAll, P, st);
+}
+static cudaError_t launch_intra(const TcParams& P, cudaStream_t st) {
+    if (P.lowrank) return P.narrow_v ? launch_intra_t<64, true>(P, st) : launch_intra_t<128, true>(P, st);
+    return P.narrow_v ? launch_intra_t<64, false>(P, st) : launch_intra_t<128, false>(P, st);
+}
+template <int DV, bool FACTORS>
+static cudaError_t launch_out_t(const TcParams& P, cudaStream_t st) {
+    static SmemLimitOnce done;
+    const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count();
+    return launch_chunk_kernel(tc_out_kernel<false, DV, FACTORS>, done, outk::SMEM_BYTES, ST_OUT, items < ctas ? items : ctas, kThreads, P, st);
 }
 static cudaError_t launch_out(const TcParams& P, cudaStream_t st) {
-    static SmemLimitOnce done, done64;
-    const int items = P.p.L.max_chunks * P.p.d.H, ctas = 2 * sm_count();
-    if (P.narrow_v) return launch_chunk_kernel(tc_out_kernel<false, 64>, done64, outk::SMEM_BYTES, ST_OUT, items < ctas ? items : ctas, kThreads, P, st);
-    return launch_chunk_kernel(tc_out_kernel<false, 128>, done, outk::SMEM_BYTES, ST_OUT, items < ctas ? items : ctas, kThreads, P, st);
+    if (P.lowrank) return P.narrow_v ? launch_out_t<64, true>(P, st) : launch_out_t<128, true>(P, st);
+    return P.narrow_v ? launch_out_t<64, false>(P, st) : launch_out_t<128, false>(P, st);
 }
 
 int tc_sm_count() { return sm_count(); }
@@ -1850,7 +2126,7 @@ cudaError_t tc_launch_out_channelwise(const Problem& p, cudaStream_t st) {
     P.p = p;
     if (!tc::make_tmap_bf16_heads(&P.tm_o, p.o, p.Ttot, p.d.H, p.d.d_v)) return cudaErrorUnknown;
     const int items = p.L.max_chunks * p.d.H, ctas = 2 * sm_count();
-    return launch_chunk_kernel(tc_out_kernel<true, 128>, done, outk::SMEM_BYTES, ST_OUT, items < ctas ? items : ctas, kThreads, P, st);
+    return launch_chunk_kernel(tc_out_kernel<true, 128, false>, done, outk::SMEM_BYTES, ST_OUT, items < ctas ? items : ctas, kThreads, P, st);
 }
 
 // Carries of the channel-wise path: dirs = 0 forward, 1 reverse, 2 both in one launch.  Needs the tile images the
@@ -1864,8 +2140,8 @@ cudaError_t tc_launch_scan_channelwise(const Problem& p, int dirs, cudaStream_t 
     const int ctas = p.d.N * p.d.H * (dirs == 2 ? 2 : 1);
     static SmemLimitOnce done2;
     if (dirs != 2 && 2 * ctas <= sm_count())
-        return launch_chunk_kernel(tc_scan_cw_kernel<2>, done2, scanlr::Cfg<2>::SMEM_BYTES, ST_SCANS, 2 * ctas, kThreads, P, st);
-    return launch_chunk_kernel(tc_scan_cw_kernel<1>, done, scanlr::Cfg<1>::SMEM_BYTES, ST_SCANS, ctas, kThreads, P, st);
+        return launch_chunk_kernel(tc_scan_cw_kernel<2>, done2, scancw::Cfg<2>::SMEM_BYTES, ST_SCANS, 2 * ctas, kThreads, P, st);
+    return launch_chunk_kernel(tc_scan_cw_kernel<1>, done, scancw::Cfg<1>::SMEM_BYTES, ST_SCANS, ctas, kThreads, P, st);
 }
 
 // A call with no tokens still owes the pass-through of the states.
@@ -1911,7 +2187,9 @@ cudaError_t tc_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st
         g_inject_timeout = 0;
         if ((e = cudaMemcpyToSymbolAsync(g_wait_limit_ns, &ns, sizeof(ns), 0, cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
     }
-    if ((e = skip_recompute ? launch_eprep(P, st) : P.lowrank ? launch_prep_lr(P, st) : launch_prep(P, st)) != cudaSuccess) return e;
+    if (!(skip_recompute && P.lowrank)) {
+        if ((e = skip_recompute ? launch_eprep(P, st) : P.lowrank ? launch_prep_lr(P, st) : launch_prep(P, st)) != cudaSuccess) return e;
+    }
     if ((e = launch_scan(P, st)) != cudaSuccess) return e;
     e = launch_intra(P, st);
     if (inject) {

@@ -60,13 +60,13 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// Copy the first `d` features of a staged [64 tokens][128 features] bf16 tile to a [T, H, d] tensor with 16-byte stores (rows
-// < len only).
-__device__ __forceinline__ void flush_rows(const unsigned char* tile, void* base, const ChunkInfo& x, int H, int d, int nthr) {
+// Copy the first `d` features of a staged [64 tokens][128 features] bf16 tile (rows row0 .. of one of R rows) to a [T, H, d] tensor with
+// 16-byte stores (rows < len only).
+__device__ __forceinline__ void flush_rows(const unsigned char* tile, void* base, const ChunkInfo& x, int H, int d, int nthr, int R = 64, int row0 = 0) {
     __nv_bfloat16* g = reinterpret_cast<__nv_bfloat16*>(base) + ((size_t)x.tok0 * H + x.hd) * d;
     for (int t = threadIdx.x; t < kC * 16; t += nthr) {
         const int i = t >> 4, chk = t & 15;
-        if (i < x.len && chk * 8 < d) *reinterpret_cast<uint4*>(g + (size_t)i * H * d + chk * 8) = *reinterpret_cast<const uint4*>(tile + tile_chunk_off(64, i, chk));
+        if (i < x.len && chk * 8 < d) *reinterpret_cast<uint4*>(g + (size_t)i * H * d + chk * 8) = *reinterpret_cast<const uint4*>(tile + tile_chunk_off(R, row0 + i, chk));
     }
 }
 

@@ -5,10 +5,10 @@
 // dead once its last product is done, so the next trip's are loaded right then, under the last readout and the stores
 // (look-ahead without a second buffer).
 //
-//   tc_prep_lr  gamma, P, T = (I + A)^-1, W^T, U~^T (the forward's share; Section 4.2), and E for the backward
-//   tc_eprep    E alone, for a backward that consumes a workspace fresh from the forward (no product, inversion or store of
-//               the forward is repeated)
-// The tc_prep kernel remains for carries in operator form, which also need Nm and Bf.
+//   tc_prep_lr  gamma, P, T = (I + A)^-1, W^T, U~^T (Section 4.2): all that carries in low-rank form need
+//   tc_eprep    carries in operator form: E alone, for a backward that consumes a workspace fresh from the forward (no product,
+//               inversion or store of the forward is repeated)
+// The tc_prep kernel remains for carries in operator form, which also need Nm, Bf and E.
 #pragma once
 
 namespace split {
@@ -173,32 +173,28 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
 }
 
 // ------------------------------------------------------------------------------------------------
-// tc_prep_lr: gamma, P = tril(Q K^T . D), T = (I + A)^-1, W^T, U~^T and, for a backward that recomputes the forward,
-// E = scale (Diag(Gam) Q - P W)^T dO.
+// tc_prep_lr: gamma, P = tril(Q K^T . D), T = (I + A)^-1, W^T, U~^T.  The forward's and the backward's preparation are the same: the
+// reverse carry takes Q, dO and P itself (tc_scan_lr).
 // Against one CTA per SM with sixteen readout warps, a loader and an issuer warp (the form tc_prep still has), two CTAs fill each
-// other's waits: 4 x 16 heads of 2048 tokens 98 -> 79 us (both bound by the chain of dependent phases of a chunk-head), 32 heads
-// of 32768 packed tokens 695 -> 562 us (144 KB of traffic per chunk-head at 4.2 TB/s).
-// The forward has an instance of its own: without the backward's part of the readouts gdn_fwd_recompute takes 1.2 us less (4 x 16
-// heads of 2048 tokens, no output: 123.9 -> 122.6 us).
-// P is the forward's to make, although only its output and the backward use it: Q K^T rides along with K K^T in one M = 128
-// product, and neither of those has to load K and wait for a product of its own (tc_out, tc_eprep).
+// other's waits (both are bound by the chain of dependent phases of a chunk-head).  4 x 16 heads of 2048 tokens 64.5 us, 8 packed
+// sequences, 32768 tokens, 32 heads 447 us (98 KB of traffic per chunk-head); with E for a backward 80 and 562 us.
+// P is made here, although the forward output and the reverse carry use it: Q K^T rides along with K K^T in one M = 128
+// product, and neither of those has to load K and wait for a product of its own.
 // ------------------------------------------------------------------------------------------------
 namespace preplr {
 constexpr uint32_t QK = 0;                  // [Q rows 0..63 ; K rows 64..127] x 128                            32 KB
-constexpr uint32_t VO = 32768;              // [V ; dO, later R = Diag(Gam) dO] x 128                           32 KB
-constexpr uint32_t XA = VO + 32768;         // fp32 A [64][kLdi], then the bf16 tiles T, T Diag(b Gam), T Diag(w) over A and T,
-constexpr uint32_t XT = XA + 17408;         // fp32 T [64][kLdi]        then W^T over the last two, finally the E image over all
+constexpr uint32_t VT = 32768;              // V [64][128], later U~^T [128][64]                                16 KB
+constexpr uint32_t XA = VT + 16384;         // fp32 A [64][kLdi], then the bf16 tiles T, T Diag(b Gam), T Diag(w) over A and T,
+constexpr uint32_t XT = XA + 17408;         // fp32 T [64][kLdi]        then W^T over the last two
 constexpr uint32_t PT = XT + 17408;         // P = tril(Q K^T . D)                                               8 KB
-constexpr uint32_t TT = XA, TP = XA + 8192, TPP = XA + 16384, WT = TP, ES = XA;
-// U~^T [128][64] over V and (P^T dO)^T [128][64] over K: two pieces of 64 rows each, 16 KB apart
-constexpr uint32_t UTT = VO, PDOT = QK + 8192;
+constexpr uint32_t TT = XA, TP = XA + 8192, TPP = XA + 16384, WT = TP, UTT = VT;
 constexpr uint32_t SMEM_BYTES = PT + 8192 + 1024 /* alignment slack */;
-constexpr uint32_t C_S1 = 0, C_PDO = 64, C_W = 128, C_U = 192, C_E = 0;   // TMEM columns (256 allocated; E over S1 and P^T dO)
-static_assert(TPP + 8192 <= PT && ES + 32768 <= PT && PT % 1024 == 0, "T tiles and the E image fit over the fp32 blocks");
+constexpr uint32_t C_S1 = 0, C_W = 128, C_U = 192;   // TMEM columns (256 allocated)
+static_assert(TPP + 8192 <= PT && PT % 1024 == 0, "T tiles fit over the fp32 blocks");
 static_assert(2 * (SMEM_BYTES + 4096) <= 228 * 1024, "two CTAs per SM");
 }  // namespace preplr
 
-template <bool bwd, int DV>   // with the backward's share
+template <int DV>
 __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_constant__ TcParams P) {
     wait_prerequisites();
     using namespace preplr;
@@ -210,7 +206,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
 
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sm = align1024(smem_raw);
-    __shared__ __align__(16) float gates[5][kC];   // gam log2e, Gam, b, w, b Gam
+    __shared__ __align__(16) float gates[4][kC];   // gam log2e, b, w, b Gam
     __shared__ uint64_t bar_in, bar_mma;
     __shared__ uint32_t tmem_slot;
     const int warp = warp_id(), lane = threadIdx.x & 31;
@@ -222,23 +218,23 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
-    const float *gl = gates[0], *Gam = gates[1], *bb = gates[2], *ww = gates[3], *bgam = gates[4];
+    const float *gl = gates[0], *bb = gates[1], *ww = gates[2], *bgam = gates[3];
     float* Af = reinterpret_cast<float*>(sm + XA);
     float* Tf = reinterpret_cast<float*>(sm + XT);
-    const float sc = p.d.scale;
     bool ok = true, pending = false;
     uint32_t mma_phase = 0, in_phase = 0;
-    // Every input tile of a trip is dead once its last product is done: the next trip's are loaded right then, under the
-    // readout of E and its store; the gate values of the next trip are fetched into registers at the same moment.
-    auto issue_loads = [&](const ChunkInfo& c, bool withhold) {   // thread 0
-        mbar_expect_tx(&bar_in, 49152 + (bwd ? 16384 : 0));
+    // Q and K of a trip are dead once its last product is done, V when U~^T, staged over it, has left: the next trip's are loaded right then, the
+    // gate values of the next trip fetched into registers at the same moment.
+    auto load_qk = [&](const ChunkInfo& c, bool withhold) {   // thread 0; announces the trip's bytes
+        mbar_expect_tx(&bar_in, 49152);
         for (int cb = 0; cb < 2; ++cb) {
             if (!(withhold && cb == 0)) tma_load_3d(sm + QK + cb * 16384, &P.tm_q, cb * 64, c.hd, c.tok0, &bar_in);
             tma_load_3d(sm + QK + cb * 16384 + 8192, &P.tm_k, cb * 64, c.hd, c.tok0, &bar_in);
-            tma_load_3d(sm + VO + cb * 16384, &P.tm_v, cb * 64, c.hd, c.tok0, &bar_in);
-            if (bwd) tma_load_3d(sm + VO + cb * 16384 + 8192, &P.tm_do, cb * 64, c.hd, c.tok0, &bar_in);
         }
         pending = true;
+    };
+    auto load_v = [&](const ChunkInfo& c) {
+        for (int cb = 0; cb < 2; ++cb) tma_load_3d(sm + VT + cb * 8192, &P.tm_v, cb * 64, c.hd, c.tok0, &bar_in);
     };
     float gg[2] = {0.f, 0.f}, gb[2] = {0.f, 0.f}, gw[2] = {0.f, 0.f};   // warp 0: log decay, erase gate, write gate of tokens lane, lane + 32
     auto fetch_gates = [&](const ChunkInfo& c) {   // warp 0
@@ -256,7 +252,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
     };
     ChunkInfo x;
     chunk_entry(p, x, blockIdx.x);
-    if (threadIdx.x == 0) issue_loads(x, P.withhold == WITHHOLD_PREP);
+    if (threadIdx.x == 0) { load_qk(x, P.withhold == WITHHOLD_PREP); load_v(x); }
     if (warp == 0) fetch_gates(x);
 #pragma unroll 1
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, in_phase ^= 1) {
@@ -277,10 +273,9 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
                 const int i = lane + 32 * h;
                 const float G = expf(gc[h]);
                 gates[0][i] = gc[h] * kLog2e;
-                gates[1][i] = G;
-                gates[2][i] = gb[h];
-                gates[3][i] = gw[h];
-                gates[4][i] = gb[h] * G;
+                gates[1][i] = gb[h];
+                gates[2][i] = gw[h];
+                gates[3][i] = gb[h] * G;
                 reinterpret_cast<float*>(p.ws + p.L.gamma)[(size_t)x.ch * kC + i] = gc[h];
             }
         }
@@ -292,8 +287,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
         if (ok && x.len < kC) {   // identity padding of a ragged tail
             zero_tail_rows(sm + QK, 128, 0, x.len, split::kT);
             zero_tail_rows(sm + QK, 128, 64, x.len, split::kT);
-            zero_tail_rows(sm + VO, 128, 0, x.len, split::kT);
-            if (bwd) zero_tail_rows(sm + VO, 128, 64, x.len, split::kT);
+            zero_tail_rows(sm + VT, 64, 0, x.len, split::kT);
             fence_async_smem();
         }
         __syncthreads();
@@ -301,7 +295,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 128>(tmem + C_S1, op_k_major(sm + QK, 128, 0), op_k_major(sm + QK, 128, 64), false);
-            bulk_wait_read<0>();   // (the previous trip's stores have read P and the E image: rewritten from here on)
+            bulk_wait_read<0>();   // (the previous trip's stores have read P and T: rewritten from here on)
             mma_commit(&bar_mma);
         }
         GDN_WAIT_MMA(2)
@@ -329,11 +323,8 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
         tc_fence_before();
         fence_async_smem();
         __syncthreads();
-        // (P^T dO)^T = dO^T P runs under the inversion and is covered by phase 2's commit
         if (warp == 0 && elect_one() && ok) {
-            tc_fence_after();
-            if (bwd) mma_tile<128, 64, 64>(tmem + C_PDO, op_mn_major(sm + VO, 128, 64), op_mn_major(sm + PT, 64), false);
-            bulk_store(p.ws + p.L.Pm + (size_t)x.ch * 8192, sm + PT, 8192);   // the forward output and the gradient stage read P from here
+            bulk_store(p.ws + p.L.Pm + (size_t)x.ch * 8192, sm + PT, 8192);   // the forward output and the reverse carry read P from here
             bulk_commit();
         }
         invert64(Af, Tf, [] { __syncthreads(); });
@@ -371,83 +362,37 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
         if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             mma_tile<128, 64, 64>(tmem + C_W, op_mn_major(sm + QK, 128, 64), op_k_major(sm + TP, 64), false);
-            mma_tile<128, 64, 64>(tmem + C_U, op_mn_major(sm + VO, 128, 0), op_k_major(sm + TPP, 64), false);
+            mma_tile<128, 64, 64>(tmem + C_U, op_mn_major(sm + VT, 64), op_k_major(sm + TPP, 64), false);
             mma_commit(&bar_mma);
             bulk_store(p.ws + p.L.Tm + (size_t)x.ch * 8192, sm + TT, 8192);
             bulk_commit();
         }
         GDN_WAIT_MMA(3)
+        if (ok && has_next && threadIdx.x == 0) load_qk(xn, false);
         if (ok) {
             const int f = q4 * 32 + lane, i0 = grp * 32;
-            unsigned char* ut = sm + UTT + (f >> 6) * 16384;      // this feature's half of the two-piece tiles
-            unsigned char* pd = sm + PDOT + (f >> 6) * 16384;
 #pragma unroll 1
             for (int part = 0; part < 4; ++part) {
                 const int ib = i0 + part * 8;
-                float a[8], b[8], c[8];
+                float a[8], b[8];
                 tmem_ld8(tmem + lane_base + C_W + ib, a);
                 tmem_ld8(tmem + lane_base + C_U + ib, b);
-                if (bwd) tmem_ld8(tmem + lane_base + C_PDO + ib, c);
                 tmem_wait_ld();
                 chunk_store(sm + WT, 128, f, ib >> 3, a);
-                chunk_store(ut, 64, f & 63, ib >> 3, b);
-                if (bwd) chunk_store(pd, 64, f & 63, ib >> 3, c);
-            }
-            if (bwd)
-#pragma unroll
-            for (int it = 0; it < 4; ++it) {   // R = Diag(Gam) dO, in place
-                const int i = (threadIdx.x >> 4) + 16 * it;
-                float v[8];
-                chunk_load(sm + VO, 128, 64 + i, threadIdx.x & 15, v);
-                const float G = Gam[i];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) v[k] *= G;
-                chunk_store(sm + VO, 128, 64 + i, threadIdx.x & 15, v);
+                chunk_store(sm + UTT, 128, f, ib >> 3, b);
             }
         }
         tc_fence_before();
         fence_async_smem();
         __syncthreads();
-        // ---- phase 3: E = Q^T R - W^T (P^T dO)   (the second operand of the second product in two pieces: 64 columns each)
-        if (warp == 0 && elect_one() && ok) {
-            tc_fence_after();
-            if (bwd) {
-                mma_tile<128, DV, 64>(tmem + C_E, op_mn_major(sm + QK, 128, 0), op_mn_major(sm + VO, 128, 64), false);
-                mma_tile<128, 64, 64>(tmem + C_E, op_k_major(sm + WT, 128), op_k_major(sm + PDOT, 64), true, /*neg_a=*/true);
-                if (DV == 128) mma_tile<128, 64, 64>(tmem + C_E + 64, op_k_major(sm + WT, 128), op_k_major(sm + PDOT + 16384, 64), true, /*neg_a=*/true);
-            }
+        if (threadIdx.x == 0 && ok) {
             bulk_store(p.ws + p.L.W + (size_t)x.ch * 16384, sm + WT, 16384);
-            bulk_store(p.ws + p.L.Ut + (size_t)x.ch * 16384, sm + UTT, 8192);
-            if (DV == 128) bulk_store(p.ws + p.L.Ut + (size_t)x.ch * 16384 + 8192, sm + UTT + 16384, 8192);
+            bulk_store(p.ws + p.L.Ut + (size_t)x.ch * 16384, sm + UTT, 128 * DV);
             bulk_commit();
-            bulk_wait_read<0>();   // T, W^T and U~^T have left: the E image and the next inputs go over them
-            mma_commit(&bar_mma);
+            bulk_wait_read<0>();   // W^T and U~^T have left: the fp32 blocks and V of the next trip (it waits for V) go over them
+            if (has_next) load_v(xn);
         }
-        GDN_WAIT_MMA(4)
-        if (ok && has_next) {   // every input tile has been read for the last time
-            if (threadIdx.x == 0) issue_loads(xn, false);
-            if (warp == 0) fetch_gates(xn);
-        }
-        if (ok && bwd) {   // E -> bf16 tile image
-            const int r = q4 * 32 + lane, c0 = grp * (DV / 2);
-#pragma unroll 2
-            for (int part = 0; part < DV / 16; ++part) {
-                const int cb = c0 + part * 8;
-                float v[8];
-                tmem_ld8(tmem + lane_base + C_E + cb, v);
-                tmem_wait_ld();
-#pragma unroll
-                for (int k = 0; k < 8; ++k) v[k] *= sc;
-                chunk_store(sm + ES, 128, r, cb >> 3, v);
-            }
-        }
-        tc_fence_before();
-        fence_async_smem();
-        __syncthreads();
-        if (warp == 0 && elect_one() && ok && bwd) {
-            bulk_store(p.ws + p.L.E + (size_t)x.ch * 32768, sm + ES, 256 * DV);
-            bulk_commit();
-        }
+        if (ok && has_next && warp == 0) fetch_gates(xn);
         if (!ok) break;
         x = xn;
     }
