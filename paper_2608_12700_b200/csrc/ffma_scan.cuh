@@ -209,15 +209,16 @@ __device__ __forceinline__ void scan_chain(const Problem& p, int chain, int part
 #pragma unroll
         for (int u = 0; u < NP; ++u) {
             const float* src = red + u * Sh::SLICES * Sl::FLOATS + tid * PW;
-            float d[PW];
-            ld_cols(d, src);
+            float v[Sh::SLICES][PW];   // summed in pairs
 #pragma unroll
-            for (int w = 1; w < Sh::SLICES; ++w) {
-                float v[PW];
-                ld_cols(v, src + w * Sl::FLOATS);
+            for (int w = 0; w < Sh::SLICES; ++w) ld_cols(v[w], src + w * Sl::FLOATS);
 #pragma unroll
-                for (int c = 0; c < PW; ++c) d[c] += v[c];
-            }
+            for (int h = Sh::SLICES / 2; h > 0; h /= 2)
+#pragma unroll
+                for (int w = 0; w < h; ++w)
+#pragma unroll
+                    for (int c = 0; c < PW; ++c) v[w][c] += v[w + h][c];
+            const float (&d)[PW] = v[0];
 #pragma unroll
             for (int c = 0; c < PW; ++c) state[u][c] = fmaf(G, state[u][c], REVERSE ? add[u][c] - d[c] : d[c]);
             st_cols(hs + u * Sl::FLOATS + tid * PW, state[u]);

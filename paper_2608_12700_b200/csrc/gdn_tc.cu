@@ -698,16 +698,26 @@ template <int S> struct Cfg {
     static_assert(UT + 16384 / S <= STAGE_BYTES && STAGE_BYTES % 1024 == 0, "U^T fits behind a forward slot's tiles");
 };
 struct Gates { float ee[2][kC], gq[2][kC], ge[2]; };   // e_j, scale Gam_j and Gam_e of a step, made during the step before it
+// What the threads of a CTA share besides the tiles.
+struct Shared {
+    Gates gates;
+    uint64_t full[2], mma;           // a ring slot has arrived; a product of the present step is done
+    uint64_t free1[2], free2[2];     // by step parity: the tiles that the first product was the last to read, and all others, may be loaded over
+    uint32_t tmem;
+};
+constexpr int kScanThreads = kThreads + 32;   // ... and a warp that only loads: a tile of the step after next goes over its predecessor as
+                                              // soon as the product that read it last is done
 }  // namespace scanlr
 
 // One direction of one chain (the direction is a compile-time constant: the two differ in operands and readouts).
 template <bool reverse, int S>
-__device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int part, scanlr::Gates& gates, uint64_t* bar_full, uint64_t& bar_mma,
-                                              uint32_t& tmem_slot) {
+__device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int part, scanlr::Shared& sh) {
     using namespace scanlr;
     using C = Cfg<S>;
     constexpr int NS = C::NS, NSH = C::NSH, STAGES = C::STAGES;
     constexpr uint32_t STAGE_BYTES = C::STAGE_BYTES, HT = C::HT, HT_BYTES = C::HT_BYTES, GT = C::GT, VALUE_BYTES = 16384 / S;
+    Gates& gates = sh.gates;
+    uint64_t *bar_full = sh.full, &bar_mma = sh.mma;
     const Problem& p = P.p;
     const int H = p.d.H, n = chain / H, hd = chain % H;
     const SeqGeom sg = seq_geom(p, n);
@@ -729,40 +739,66 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     const float sc = p.d.scale;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) mbar_init(&bar_full[s], 1);
+        for (int s = 0; s < STAGES; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&sh.free1[s], 1); mbar_init(&sh.free2[s], 1); }
         mbar_init(&bar_mma, 1);
         fence_mbar_init();
     }
-    if (warp == 0) { tmem_alloc(&tmem_slot, C::TMEM_COLS); tmem_relinquish(); }
+    if (warp == 0) { tmem_alloc(&sh.tmem, C::TMEM_COLS); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = sh.tmem;
 
     // this CTA's rows of U~^T, then U^T, or of dU^T (both images [d_v][tokens])
     char* y_base = p.ws + (reverse ? p.L.E : p.L.Ut) + part * VALUE_BYTES;
     char* keep_base = p.ws + (reverse ? p.L.dhn : p.L.hc) + part * HT_BYTES;
     const float* gamma = reinterpret_cast<const float*>(p.ws + p.L.gamma);
     // (L2 prefetches running ahead of the ring, as in tc_scan, made this kernel slower: 79.7 -> 78.5 us without)
-    auto fill = [&](int s) {   // thread 32: bring chunk step s into ring slot s % STAGES
+    // The tiles of step s into ring slot s % STAGES, in two parts: those whose predecessors are dead after the first product (W^T forward; K and P
+    // in reverse), which announce the slot's bytes, and the rest.
+    auto fill1 = [&](int s) {
         const int stage = s % STAGES, c = chunk_of(s), tok0 = sg.chunk_tok0(c);
         const size_t ch = (size_t)c * H + hd;
         unsigned char* slot = sm + stage * STAGE_BYTES;
         uint64_t* bar = &bar_full[stage];
         mbar_expect_tx(bar, 32768 + VALUE_BYTES + (reverse ? 24576 : 0));
-        if (!(P.withhold == WITHHOLD_CARRY && s == 0)) bulk_load(slot + WT, p.ws + p.L.W + ch * 16384, 16384, bar);
-        for (int cb = 0; cb < 2; ++cb) tma_load_3d(slot + KT + cb * 8192, &P.tm_k, cb * 64, hd, tok0, bar);
         if (reverse) {
+            for (int cb = 0; cb < 2; ++cb) tma_load_3d(slot + KT + cb * 8192, &P.tm_k, cb * 64, hd, tok0, bar);
             bulk_load(slot + PT, p.ws + p.L.Pm + ch * 8192, 8192, bar);
+        } else if (!(P.withhold == WITHHOLD_CARRY && s == 0)) {
+            bulk_load(slot + WT, p.ws + p.L.W + ch * 16384, 16384, bar);
+        }
+    };
+    auto fill2 = [&](int s) {
+        const int stage = s % STAGES, c = chunk_of(s), tok0 = sg.chunk_tok0(c);
+        const size_t ch = (size_t)c * H + hd;
+        unsigned char* slot = sm + stage * STAGE_BYTES;
+        uint64_t* bar = &bar_full[stage];
+        if (reverse) {
             for (int cb = 0; cb < 2 / S; ++cb) tma_load_3d(slot + OT + cb * 8192, &P.tm_do, part * NS + cb * 64, hd, tok0, bar);
             for (int cb = 0; cb < 2; ++cb) tma_load_3d(slot + QT + cb * 8192, &P.tm_q, cb * 64, hd, tok0, bar);
+            if (!(P.withhold == WITHHOLD_CARRY && s == 0)) bulk_load(slot + WT, p.ws + p.L.W + ch * 16384, 16384, bar);
         } else {
+            for (int cb = 0; cb < 2; ++cb) tma_load_3d(slot + KT + cb * 8192, &P.tm_k, cb * 64, hd, tok0, bar);
             bulk_load(slot + XT, y_base + ch * 16384, VALUE_BYTES, bar);
         }
     };
-    if (threadIdx.x == 32) {
-        for (int s = 0; s < STAGES && s < nsteps; ++s) fill(s);
+    if (warp == kThreads / 32) {
+        if (lane == 0) {
+            for (int s = 0; s < STAGES && s < nsteps; ++s) { fill1(s); fill2(s); }
+            int s = 0;
+            for (; s + STAGES < nsteps; ++s) {   // (a product two steps on needs the slot filled here: no phase of these barriers can be missed)
+                if (!mbar_wait(&sh.free1[s & 1], (s >> 1) & 1)) break;
+                fill1(s + STAGES);
+                if (!mbar_wait(&sh.free2[s & 1], (s >> 1) & 1)) { ++s; break; }
+                fill2(s + STAGES);
+            }
+            if (s + STAGES < nsteps) drain_ring<STAGES>(bar_full, s, nsteps);   // after a time-out loads may still be in flight
+        }
+        __syncthreads();
+        return;
     }
+    auto cta_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory"); };   // all warps but the loader
     // the gate arrays of the first step; the cumulative decays of the second are fetched now
     auto gate_row = [&](int s) { return gamma + ((size_t)chunk_of(s) * H + hd) * kC; };
     auto make_gates = [&](int set, float g, float gend) {
@@ -786,7 +822,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
             st[4 * k] = v.x; st[4 * k + 1] = v.y; st[4 * k + 2] = v.z; st[4 * k + 3] = v.w;
         }
     }
-    __syncthreads();
+    cta_sync();
     bool ok = true;
     uint32_t mma_phase = 0;
     int s = 0;
@@ -811,7 +847,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
             }
         }
         fence_async_smem();
-        __syncthreads();
+        cta_sync();
         const float Ge = gates.ge[s & 1];   // decay of the state over the chunk
         if (warp == 0 && elect_one()) {
             ok = mbar_wait_inline(&bar_full[stage], (s / STAGES) & 1);
@@ -828,8 +864,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
             bulk_commit();
             bulk_wait_read<1>();   // (the stores of the step before have read their tiles: they are rewritten from here on)
             mma_commit(&bar_mma);
-        } else if (threadIdx.x == 32) {
-            if (s >= 1 && s - 1 + STAGES < nsteps) fill(s - 1 + STAGES);
+            mma_commit(&sh.free1[s & 1]);
         }
         ok = mbar_wait_inline(&bar_full[stage], (s / STAGES) & 1);
         if (reverse) {   // scale Diag(Gam) Q in place, under the first product; its product by dO runs under the readout
@@ -846,7 +881,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
                 }
             }
             fence_async_smem();
-            __syncthreads();
+            cta_sync();
             if (warp == 0 && elect_one() && ok) mma_tile<128, NS, 64>(tmem + C_D2, op_mn_major(ring + QT, 64), op_mn_major(ring + OT, 64), false);
         }
         if (ok) ok = mbar_wait_inline(&bar_mma, mma_phase);
@@ -882,12 +917,13 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         }
         tc_fence_before();
         fence_async_smem();
-        __syncthreads();
+        cta_sync();
         if (warp == 0 && elect_one()) {
             tc_fence_after();
             if (reverse) mma_tile<128, NS, 64>(tmem + C_D2, op_k_major(ring + WT, 128), op_k_major(sm + GT, NS), true, /*neg_a=*/true);
             else mma_tile<128, NS, 64>(tmem + C_D2, op_mn_major(ring + KT, 64), op_k_major(sm + GT, NS), false);
             mma_commit(&bar_mma);
+            mma_commit(&sh.free2[s & 1]);
             bulk_store(y_base + ch * 16384, reverse ? sm + GT : ring + UT, VALUE_BYTES);
             bulk_commit();
         }
@@ -917,7 +953,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         for (int k = 0; k < NSH / 4; ++k) if (inside) *reinterpret_cast<float4*>(fin + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
     }
     if (warp == 0) bulk_wait_read<0>();
-    if (threadIdx.x == 32) drain_ring<STAGES>(bar_full, s, nsteps);
+    if (!ok && threadIdx.x == 32) drain_ring<STAGES>(bar_full, s, nsteps);
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, C::TMEM_COLS);
@@ -926,20 +962,18 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
 // Block index -> (chain, direction, column block): with both directions in one launch the direction is the low bit
 // (S = 1, or narrow_v, where the second column block is not there); with S = 2 (one direction per launch) the low bit is the column block.
 template <int S>
-__global__ void __launch_bounds__(kThreads, 1) tc_scan_lr_kernel(const __grid_constant__ TcParams P) {
+__global__ void __launch_bounds__(scanlr::kScanThreads, 1) tc_scan_lr_kernel(const __grid_constant__ TcParams P) {
     wait_prerequisites();
     using namespace scanlr;
-    __shared__ __align__(16) scanlr::Gates gates;
-    __shared__ uint64_t bar_full[Cfg<S>::STAGES], bar_mma;
-    __shared__ uint32_t tmem_slot;
+    __shared__ __align__(16) scanlr::Shared sh;
     const int bid = (int)blockIdx.x;
     if (reinterpret_cast<const WsHeader*>(P.p.ws)->status != GDN_OK) return;
     const bool halves = S == 2 && !P.narrow_v;
     const int rev = (!halves && P.scan_dirs == 2) ? (bid & 1) : P.scan_dirs;
     const int chain = (halves || P.scan_dirs == 2) ? (bid >> 1) : bid;
     const int part = halves ? (bid & 1) : 0;
-    if (rev) scan_lr_chain<true, S>(P, chain, part, gates, bar_full, bar_mma, tmem_slot);
-    else scan_lr_chain<false, S>(P, chain, part, gates, bar_full, bar_mma, tmem_slot);
+    if (rev) scan_lr_chain<true, S>(P, chain, part, sh);
+    else scan_lr_chain<false, S>(P, chain, part, sh);
 }
 
 namespace scancw {
@@ -2088,8 +2122,8 @@ static cudaError_t launch_scan(const TcParams& P, cudaStream_t st) {
         // the state columns (measured on 64 chains of 32 chunks: reverse 64 -> 58 us; the forward carry alone became
         // slower that way, 62 -> 66 us, and keeps one CTA per chain).  d_v = 64: half of the columns are all there are.
         if (P.narrow_v || (P.scan_dirs == 1 && half_ctas <= sm_count()))
-            return launch_chunk_kernel(tc_scan_lr_kernel<2>, done_lr2, scanlr::Cfg<2>::SMEM_BYTES, ST_SCANS, half_ctas, kThreads, P, st);
-        return launch_chunk_kernel(tc_scan_lr_kernel<1>, done_lr, scanlr::Cfg<1>::SMEM_BYTES, ST_SCANS, ctas, kThreads, P, st);
+            return launch_chunk_kernel(tc_scan_lr_kernel<2>, done_lr2, scanlr::Cfg<2>::SMEM_BYTES, ST_SCANS, half_ctas, scanlr::kScanThreads, P, st);
+        return launch_chunk_kernel(tc_scan_lr_kernel<1>, done_lr, scanlr::Cfg<1>::SMEM_BYTES, ST_SCANS, ctas, scanlr::kScanThreads, P, st);
     }
     // few chains: two CTAs per (chain, direction), each carrying half of the state columns
     if (half_ctas <= sm_count())
