@@ -48,20 +48,26 @@ struct Thread {
     }
 };
 
+// Unrolling of the products of the per-channel kernels (and of dU0) at DK key features.  At 128 such a kernel is 100 KB of code that a CTA runs
+// once, and with a CTA on most SMs two steps side by side cost more in instruction fetches than they give: 8 heads of 1024 tokens
+// 216 -> 206 us (6 of 800 tokens, on half of the SMs: 175 -> 176; d = 64: 87.3 -> 90.2); dU0 with E alone 23.1 -> 20.0 us.
+template <int DK>
+constexpr int kU = DK == 128 ? 1 : 2;
+
 enum AForm { A_ROW, A_COL };   // A(i, k) = A[i * pa + k] / A[k * pa + i]
 enum BForm { B_ROW, B_COL };   // B(k, j) = B[j * pb + k] / B[k * pb + j]
 
 // acc[R0 + 4 h + x][y] += sum over k in [k0, k1) of A_h(i + x, k) B(k, j + 8 y);  i, j: first row and column of this thread;
 // (k0, k1 multiples of 4; pointers at row / column 0)
-// (CS: distance of a thread's columns)
-template <int HALVES, AForm AF, BForm BF, int R0 = 0, int CS = 8, int R>
+// (CS: distance of a thread's columns; U: how far the loop is unrolled)
+template <int HALVES, AForm AF, BForm BF, int R0 = 0, int CS = 8, int U = 2, int R>
 __device__ __forceinline__ void mac(float (&acc)[R][4], const float* A0, const float* A1, int pa, int i, const float* B,
                                     int pb, int j, int k0, int k1) {
     static_assert(R0 + 4 * HALVES <= R, "rows of the accumulator");
     const float* a0 = AF == A_ROW ? A0 + i * pa : A0 + i;
     const float* a1 = HALVES == 2 ? (AF == A_ROW ? A1 + i * pa : A1 + i) : nullptr;
     const float* b0 = BF == B_ROW ? B + j * pb : B + j;
-#pragma unroll 2
+#pragma unroll U
     for (int k = k0; k < k1; k += 4) {
         float a[4 * HALVES][4], b[4][4];   // a[row][k], b[k][column]
 #pragma unroll
@@ -117,19 +123,19 @@ struct Out {
 // contraction in which one half of the rows meets only zeros is left out for those rows, in the narrow form the 16-row
 // blocks that a warp's rows do not reach.
 enum Tri { A_LOWER, A_UPPER };
-template <int N, AForm AF, Tri TRI>
+template <int N, AForm AF, Tri TRI, int U = 2>
 __device__ __forceinline__ void tri_product(const Thread& t, const float* A, const float* B, int pb, float (&acc)[N == 128 ? 8 : 4][4]) {
     const Out<N> o(t);
     zero(acc);
     if constexpr (N == 128) {
         const float* A1 = AF == A_ROW ? A + 32 * kPc : A + 32;
         constexpr bool low = TRI == A_LOWER;
-        mac<2, AF, B_COL>(acc, A, A1, kPc, o.r0, B, pb, o.c, low ? 0 : 32, low ? 32 : kC);
-        if constexpr (low) mac<1, AF, B_COL, 4>(acc, A1, nullptr, kPc, o.r0, B, pb, o.c, 32, kC);
-        else mac<1, AF, B_COL, 0>(acc, A, nullptr, kPc, o.r0, B, pb, o.c, 0, 32);
+        mac<2, AF, B_COL, 0, 8, U>(acc, A, A1, kPc, o.r0, B, pb, o.c, low ? 0 : 32, low ? 32 : kC);
+        if constexpr (low) mac<1, AF, B_COL, 4, 8, U>(acc, A1, nullptr, kPc, o.r0, B, pb, o.c, 32, kC);
+        else mac<1, AF, B_COL, 0, 8, U>(acc, A, nullptr, kPc, o.r0, B, pb, o.c, 0, 32);
     } else {
         const int w16 = (o.r0 >> 4) * 16;
-        mac<1, AF, B_COL>(acc, A, nullptr, kPc, o.r0, B, pb, o.c, TRI == A_LOWER ? 0 : w16, TRI == A_LOWER ? w16 + 16 : kC);
+        mac<1, AF, B_COL, 0, 8, U>(acc, A, nullptr, kPc, o.r0, B, pb, o.c, TRI == A_LOWER ? 0 : w16, TRI == A_LOWER ? w16 + 16 : kC);
     }
 }
 

@@ -203,7 +203,8 @@ struct SmemLimitOnce {
 // of 333 tokens, six launches: 63.5 -> 51.8 us; a backward of 4 x 16 heads of 2048 tokens, three: 307 -> 301 us.)  All threads
 // of all blocks wait, those without work too: a grid that ended without waiting would let the kernel after it run beside the
 // one before it.  No kernel triggers its dependents early (griddepcontrol.launch_dependents): their blocks then take up
-// room while others still work; the same two calls took 54.4 and 326 us that way.
+// room while others still work; the same two calls took 54.4 and 326 us that way.  In the last trip or step of every kernel it is no
+// better: the instruction itself costs some 2.7 us a launch (a six-launch call 89 -> 105 us).
 __device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... Params, class... Args>
 cudaError_t launch_kernel_cluster(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, unsigned cluster, Args&&... args) {

@@ -15,7 +15,7 @@
 // At d = 128 the gradient stage of a chunk-head is 5.6 M FMAs, 23 us at the rate of one SM; measured 55 us (forward preparation
 // 22 us, the backward's share of it 21 us): eight warps on an SM issue in half of the cycles, between barriers.  With the operands of every FMA read from
 // global memory, and the solve and the sums over a chunk done by single threads, the same stages took 907, 165 and 102 us
-// (2 x 4 heads of 1000 tokens); the smallest call, 2 heads of 128 tokens at d = 64, went from 370 to 53 us.
+// (2 x 4 heads of 1000 tokens); the smallest call, 2 heads of 128 tokens at d = 64, went from 370 to 35 us.
 #include <cooperative_groups.h>
 
 #include "ffma_scan.cuh"
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(kThreads, 1) prep_kernel(Problem p, int mode, 
     float* wsD = block_of(p, p.L.dU, x.ch, kC * DV);
     {
         float acc[Out<DV>::R][4];
-        tri_product<DV, A_COL, A_UPPER>(t, Pm, sO, PV, acc);
+        tri_product<DV, A_COL, A_UPPER, kU<DK>>(t, Pm, sO, PV, acc);
 #pragma unroll
         for (int r = 0; r < Out<DV>::R; ++r)
 #pragma unroll

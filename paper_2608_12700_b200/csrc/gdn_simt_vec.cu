@@ -20,7 +20,7 @@
 // One CTA handles one (chunk, head) in the parallel stages.  Every reduction has a fixed order: results are bit-identical
 // from run to run.  Measured against the plain statement (decay evaluated for every pair and channel, operands read from global
 // memory, one CTA per chain in the carries): 8 heads of 1024 tokens at d = 128, bf16 I/O, decay beyond the tensor-core route:
-// 4.4 ms -> 0.30 ms; a step of 2 x 4 heads of 500 tokens at d = 64, fp32: 1.01 -> 0.14 ms.  With bf16 I/O at d_k = d_v = 128 the path runs on the tensor cores instead (gdn_tc_cw.cu), with these
+// 4.4 ms -> 0.21 ms; a step of 2 x 4 heads of 500 tokens at d = 64, fp32: 1.01 -> 0.088 ms.  With bf16 I/O at d_k = d_v = 128 the path runs on the tensor cores instead (gdn_tc_cw.cu), with these
 // kernels enqueued behind it for gates that leave its range.
 #include "ffma_scan.cuh"
 
@@ -227,7 +227,7 @@ __device__ __forceinline__ void vprep_chunk(const Problem& p, int mode, const Ch
             const int I = blk == 0 ? 1 : blk < 3 ? 2 : 3, J = blk == 0 ? 0 : blk < 3 ? blk - 1 : blk - 3;
             float acc[4][4];
             zero(acc);
-            mac<1, A_ROW, B_ROW, 0, 4>(acc, which ? Q : R, nullptr, PK, I * kB + ti, C + (copy_row(I) + J * kB) * PK, PK, tj, 0, DK);
+            mac<1, A_ROW, B_ROW, 0, 4, kU<DK>>(acc, which ? Q : R, nullptr, PK, I * kB + ti, C + (copy_row(I) + J * kB) * PK, PK, tj, 0, DK);
             float* dst = (which ? Pm : A) + (I * kB + ti) * kPc + J * kB + tj;
 #pragma unroll
             for (int r = 0; r < 4; ++r)
@@ -262,7 +262,7 @@ __device__ __forceinline__ void vprep_chunk(const Problem& p, int mode, const Ch
         float* wsU = block_of(p, p.L.Ut, x.ch, kC * DV);
         {
             float acc[Out<DV>::R][4];
-            tri_product<DV, A_ROW, A_LOWER>(t, T, R, PV, acc);
+            tri_product<DV, A_ROW, A_LOWER, kU<DK>>(t, T, R, PV, acc);
 #pragma unroll
             for (int r = 0; r < Out<DV>::R; ++r)
 #pragma unroll
@@ -271,7 +271,7 @@ __device__ __forceinline__ void vprep_chunk(const Problem& p, int mode, const Ch
         float* wsW = block_of(p, p.L.W, x.ch, kC * DK);
         {
             float acc[Out<DK>::R][4];
-            tri_product<DK, A_ROW, A_LOWER>(t, T, K, PK, acc);
+            tri_product<DK, A_ROW, A_LOWER, kU<DK>>(t, T, K, PK, acc);
 #pragma unroll
             for (int r = 0; r < Out<DK>::R; ++r)
 #pragma unroll
@@ -303,7 +303,7 @@ __device__ __forceinline__ void vprep_chunk(const Problem& p, int mode, const Ch
     float* wsD = block_of(p, p.L.dU, x.ch, kC * DV);
     {
         float acc[Out<DV>::R][4];
-        tri_product<DV, A_COL, A_UPPER>(t, Pm, O, PV, acc);
+        tri_product<DV, A_COL, A_UPPER, kU<DK>>(t, Pm, O, PV, acc);
 #pragma unroll
         for (int r = 0; r < Out<DV>::R; ++r)
 #pragma unroll
@@ -387,8 +387,8 @@ __device__ __forceinline__ void vout_chunk(const Problem& p, const ChunkInfo& x)
     __syncthreads();
     float acc[R][4];
     zero(acc);
-    mac<R / 4, A_ROW, B_COL>(acc, sQ, sQ + 32 * PK, PK, o.r0, sH, PV, o.c, 0, DK);
-    mac<R / 4, A_ROW, B_COL>(acc, Pm, Pm + 32 * kPc, kPc, o.r0, sU, PV, o.c, 0, kC);
+    mac<R / 4, A_ROW, B_COL, 0, 8, kU<DK>>(acc, sQ, sQ + 32 * PK, PK, o.r0, sH, PV, o.c, 0, DK);
+    mac<R / 4, A_ROW, B_COL, 0, 8, kU<DK>>(acc, Pm, Pm + 32 * kPc, kPc, o.r0, sU, PV, o.c, 0, kC);
     IO* op = rows_of<IO>(p.o, x, H, DV);
     const size_t rv = (size_t)H * DV;
     const float sc = p.d.scale;
@@ -470,7 +470,7 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
     {   // dP = scale tril(dO U^T)
         float acc[4][4];
         zero(acc);
-        if (below) mac<1, A_ROW, B_ROW>(acc, s0, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
+        if (below) mac<1, A_ROW, B_ROW, 0, 8, kU<DK>>(acc, s0, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
@@ -491,7 +491,7 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
                 vv[r][y] = live ? ldf(vp + o.row(r) * rv + o.c + 8 * y) : 0.f;
                 ww[r][y] = live ? p.wv[base_v + o.row(r) * rv + o.c + 8 * y] : 0.f;
             }
-        tri_product<DV, A_COL, A_UPPER>(t, sT, s1, PV, acc);
+        tri_product<DV, A_COL, A_UPPER, kU<DK>>(t, sT, s1, PV, acc);
         __syncthreads();
 #pragma unroll
         for (int r = 0; r < Out<DV>::R; ++r)
@@ -510,7 +510,7 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
     {   // dA = -stril(dXv U^T), over T
         float acc[4][4];
         zero(acc);
-        if (below) mac<1, A_ROW, B_ROW>(acc, s1, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
+        if (below) mac<1, A_ROW, B_ROW, 0, 8, kU<DK>>(acc, s1, nullptr, PV, t.rn, sU, PV, t.cn, 0, DV);
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
@@ -521,7 +521,7 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
 #pragma unroll
     for (int n = 0; n < NH; ++n) {
         zero(acc[n]);
-        mac<2, A_ROW, B_ROW>(acc[n], s0, s1, PV, t.rn, sH + n * 64 * PV, PV, t.cn, 0, DV);
+        mac<2, A_ROW, B_ROW, 0, 8, kU<DK>>(acc[n], s0, s1, PV, t.rn, sH + n * 64 * PV, PV, t.cn, 0, DV);
     }
     __syncthreads();
     load_block<DK, DV>(sH, block_of(p, p.L.dhn, x.ch, DK * DV));
@@ -541,7 +541,7 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
 #pragma unroll
             for (int y = 0; y < 4; ++y) kr[r][y] = t.rn + r < x.len ? ldf(kp + (t.rn + r) * rk + n * 64 + t.cn + 8 * y) : 0.f;
         zero(col[n]);
-        mac<1, A_ROW, B_ROW>(col[n], sU, nullptr, PV, t.rn, sH + n * 64 * PV, PV, t.cn, 0, DV);
+        mac<1, A_ROW, B_ROW, 0, 8, kU<DK>>(col[n], sU, nullptr, PV, t.rn, sH + n * 64 * PV, PV, t.cn, 0, DV);
 #pragma unroll
         for (int y = 0; y < 4; ++y) {
             const int c = n * 64 + t.cn + 8 * y;
@@ -598,7 +598,7 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
     for (int n = 0; n < NH; ++n) {
         float tmp[8][4];
         zero(tmp);
-        mac<2, A_ROW, B_COL>(tmp, sP, sT, kPc, t.rn, C + copy_row(I) * PK + n * 64, PK, t.cn, 0, I * kB);
+        mac<2, A_ROW, B_COL, 0, 8, kU<DK>>(tmp, sP, sT, kPc, t.rn, C + copy_row(I) * PK + n * 64, PK, t.cn, 0, I * kB);
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
@@ -612,8 +612,8 @@ __device__ __forceinline__ void vintra_chunk(const Problem& p, const ChunkInfo& 
         for (int I2 = I + 1; I2 < kNB; ++I2) {
             float tc[4][4];
             zero(tc);
-            mac<1, A_COL, B_COL>(tc, sP, nullptr, kPc, t.rn, Q + n * 64, PK, t.cn, I2 * kB, I2 * kB + kB);
-            mac<1, A_COL, B_COL>(tc, sT, nullptr, kPc, t.rn, R + n * 64, PK, t.cn, I2 * kB, I2 * kB + kB);
+            mac<1, A_COL, B_COL, 0, 8, kU<DK>>(tc, sP, nullptr, kPc, t.rn, Q + n * 64, PK, t.cn, I2 * kB, I2 * kB + kB);
+            mac<1, A_COL, B_COL, 0, 8, kU<DK>>(tc, sT, nullptr, kPc, t.rn, R + n * 64, PK, t.cn, I2 * kB, I2 * kB + kB);
 #pragma unroll
             for (int r = 0; r < 4; ++r)
 #pragma unroll

@@ -2042,7 +2042,7 @@ thread_local int g_inject_timeout = 0;   // set by gdn_debug_inject_timeout, con
 static int sm_count();
 // Up to 37 chains (on 148 SMs) the operator form gives each direction of a chain two CTAs, and its one product per step wins; from
 // 38 on it would have one, and the low-rank form moves less.  Backward, us, operator / low-rank: 4 chains of 6 chunks 32.1 / 38.4,
-// 16 of 256 606 / 739, 37 of 32 172.7 / 175.0; 38 of 32 198.2 / 184.7, 64 of 32 290 / 260, 64 of 256 2270 / 1948; the line lies
+// 16 of 128 317 / 414, 32 of 32 154.8 / 158.9, 37 of 32 172.0 / 170.2; 38 of 32 198 / 173, 64 of 32 290 / 243; the line lies
 // there from 1 chunk to 256.  (A forward with its output and the backward on its workspace, each with one direction per launch,
 // would change sides near 64 chains: 38 of 32 250 / 266.)  The rule looks at the chains only, so the forward, the backward and
 // a backward on a workspace fresh from the forward agree on the form (and on the workspace layout that follows from it).
