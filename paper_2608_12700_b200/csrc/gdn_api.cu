@@ -317,25 +317,57 @@ gdn_status gdn_debug_read(const gdn_desc* desc, const void* workspace, const cha
     if (!q) return GDN_ERR_BAD_SHAPE;
     if (!L.has_operator && (q->off == L.Nm || q->off == L.Bf) && (strcmp(what, "Nm") == 0 || strcmp(what, "Bf") == 0))
         return GDN_ERR_BAD_SHAPE;   // not stored: the carries of this descriptor run in low-rank form
-    if (pick_path(*desc) == Path::TcBf16 && tc_carries_lowrank(*desc) && strcmp(what, "E") == 0) return GDN_ERR_BAD_SHAPE;   // (dU lies there)
+    const bool lowrank = pick_path(*desc) == Path::TcBf16 && tc_carries_lowrank(*desc);
+    if (lowrank && strcmp(what, "E") == 0) return GDN_ERR_BAD_SHAPE;   // (dU lies there)
     if (cudaDeviceSynchronize() != cudaSuccess) return GDN_ERR_CUDA;
-    const size_t n = (size_t)q->rows * q->cols;
-    const char* base = static_cast<const char*>(workspace) + q->off;
-    if (q->kind == 0 || !tcp) {
-        return cudaMemcpy(host_out, base + ch * n * 4, n * 4, cudaMemcpyDeviceToHost) == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
-    }
-    std::vector<uint16_t> img(n);
-    if (cudaMemcpy(img.data(), base + ch * n * 2, n * 2, cudaMemcpyDeviceToHost) != cudaSuccess) return GDN_ERR_CUDA;
-    const int R = q->kind == 2 ? q->cols : q->rows;       // rows of the stored tile
-    auto at = [&](int r, int c) -> float {                 // element (r, c) of the stored tile
-        const size_t off = (size_t)(c >> 6) * R * 128 + (size_t)r * 128 + ((((c & 63) >> 3) ^ (r & 7)) << 4) + ((c & 7) << 1);
-        const uint32_t bits = (uint32_t)img[off / 2] << 16;
-        float f;
-        memcpy(&f, &bits, 4);
-        return f;
+    auto read = [&](const Q& t, float* out) -> bool {
+        const size_t n = (size_t)t.rows * t.cols;
+        const char* base = static_cast<const char*>(workspace) + t.off;
+        if (t.kind == 0 || !tcp) return cudaMemcpy(out, base + ch * n * 4, n * 4, cudaMemcpyDeviceToHost) == cudaSuccess;
+        std::vector<uint16_t> img(n);
+        if (cudaMemcpy(img.data(), base + ch * n * 2, n * 2, cudaMemcpyDeviceToHost) != cudaSuccess) return false;
+        const int R = t.kind == 2 ? t.cols : t.rows;           // rows of the stored tile
+        auto at = [&](int r, int c) -> float {                 // element (r, c) of the stored tile
+            const size_t off = (size_t)(c >> 6) * R * 128 + (size_t)r * 128 + ((((c & 63) >> 3) ^ (r & 7)) << 4) + ((c & 7) << 1);
+            const uint32_t bits = (uint32_t)img[off / 2] << 16;
+            float f;
+            memcpy(&f, &bits, 4);
+            return f;
+        };
+        for (int r = 0; r < t.rows; ++r)
+            for (int c = 0; c < t.cols; ++c) out[(size_t)r * t.cols + c] = t.kind == 2 ? at(c, r) : at(r, c);
+        return true;
     };
-    for (int r = 0; r < q->rows; ++r)
-        for (int c = 0; c < q->cols; ++c) host_out[(size_t)r * q->cols + c] = q->kind == 2 ? at(c, r) : at(r, c);
+    if (!read(*q, host_out)) return GDN_ERR_CUDA;
+    // Two quantities lie in the workspace without a share that the carries took over; it is put back here.
+    const bool put_ut = lowrank && strcmp(what, "Ut") == 0, put_e = !tcp && strcmp(what, "E") == 0;
+    if (!desc->delta_rule || !(put_ut || put_e)) return GDN_OK;   // (without the delta rule W = 0)
+    std::vector<float> W((size_t)kC * dk), h((size_t)dk * dv);
+    if (!read({"W", L.W, kC, dk, 2}, W.data()) || !read(put_ut ? Q{"hc", L.hc, dk, dv, 1} : Q{"dhn", L.dhn, dk, dv, 1}, h.data())) return GDN_ERR_CUDA;
+    if (put_ut) {   // U~ = U + W h
+        for (int i = 0; i < kC; ++i)
+            for (int c = 0; c < dv; ++c) {
+                double a = host_out[(size_t)i * dv + c];
+                for (int j = 0; j < dk; ++j) a += (double)W[(size_t)i * dk + j] * h[(size_t)j * dv + c];
+                host_out[(size_t)i * dv + c] = (float)a;
+            }
+        return GDN_OK;
+    }
+    // scale (Gam Q)^T dO - W^T (scale P^T dO), of which the workspace has the first term and scale P^T dO = dU - Kb dh'
+    std::vector<float> Kb((size_t)kC * dk), X((size_t)kC * dv);
+    if (!read({"Kb", L.Kb, kC, dk, 0}, Kb.data()) || !read({"dU", L.dU, kC, dv, 0}, X.data())) return GDN_ERR_CUDA;
+    for (int i = 0; i < kC; ++i)
+        for (int c = 0; c < dv; ++c) {
+            double a = X[(size_t)i * dv + c];
+            for (int j = 0; j < dk; ++j) a -= (double)Kb[(size_t)i * dk + j] * h[(size_t)j * dv + c];
+            X[(size_t)i * dv + c] = (float)a;
+        }
+    for (int r = 0; r < dk; ++r)
+        for (int c = 0; c < dv; ++c) {
+            double a = host_out[(size_t)r * dv + c];
+            for (int i = 0; i < kC; ++i) a -= (double)W[(size_t)i * dk + r] * X[(size_t)i * dv + c];
+            host_out[(size_t)r * dv + c] = (float)a;
+        }
     return GDN_OK;
 }
 

@@ -132,3 +132,38 @@ def test_values_of_64_features_leave_half_of_the_tiles_alone(carries, d_k, lengt
     assert rel(fresh["o"], ref["o"]) < TOL["bf16"] and rel(fresh["hT"], ref["hT"]) < TOL["bf16"]
     for name in ("dq", "dk", "dv", "dg", "dbeta", "dh0"):
         assert np.array_equal(got[name], fresh[name]), name
+
+
+@pytest.mark.parametrize("dtype,carries", [("f32", 0), ("bf16", 1), ("bf16", OPERATOR), ("bf16", LOW_RANK)], indirect=["carries"])
+@pytest.mark.parametrize("d_v,delta_rule", [(128, 1), (64, 1), (128, 0)])
+def test_factors_read_back_are_those_of_the_chunk(dtype, carries, d_v, delta_rule):
+    """U~ = T Diag(w) V and E = scale (Diag(Gam) Q - P W)^T dO as gdn_debug_read gives them, whatever the carries left in their place."""
+    if dtype == "bf16" and d_v == 64 and carries != 1:
+        pytest.skip("a widened problem has nothing to read back")
+    lengths = [130, 70]
+    wl = synth.make_workload("read_back", dtype=dtype, lengths=lengths, H=2, d_k=128, d_v=d_v, delta_rule=delta_rule, scale=0.5, states=True, seed=52)
+    buf = runner.to_device(wl)
+    runner.run_bwd(buf)
+    chunk, start = 0, 0
+    for n in lengths:
+        for t0 in range(start, start + n, 64):
+            rows = slice(t0, min(t0 + 64, start + n))
+            for hd in range(2):
+                q, k, v, dO = (np.asarray(a[rows, hd], dtype=np.float64) for a in (wl.q, wl.k, wl.v, wl.dO))
+                gam = np.cumsum(wl.g[rows, hd].astype(np.float64))
+                L = len(gam)
+                b = wl.beta[rows, hd].astype(np.float64)[:, None] if delta_rule else np.zeros((L, 1))
+                w = b if delta_rule else np.ones((L, 1))
+                decay = np.tril(np.exp(gam[:, None] - gam[None, :]))
+                T = np.linalg.inv(np.eye(L) + np.tril(b * (k @ k.T) * decay, -1))
+                W, P, Gam = T @ (b * np.exp(gam)[:, None] * k), (q @ k.T) * decay, np.exp(gam)[:, None]
+                got = binding.gdn_debug_read(buf.desc, buf.workspace, "Ut", chunk, hd)
+                assert rel(got[:L], T @ (w * v)) < TOL[dtype]
+                if carries == LOW_RANK:
+                    with pytest.raises(binding.GdnError):
+                        binding.gdn_debug_read(buf.desc, buf.workspace, "E", chunk, hd)
+                else:
+                    got = binding.gdn_debug_read(buf.desc, buf.workspace, "E", chunk, hd)
+                    assert rel(got, 0.5 * (Gam * q - P @ W).T @ dO) < TOL[dtype]
+            chunk += 1
+        start += n
