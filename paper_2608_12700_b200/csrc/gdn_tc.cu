@@ -37,7 +37,8 @@ constexpr int kTG = kC / kGroups;             // token columns per group (16)
 constexpr int kIntraThreads = kWideThreads + 32;   // ... plus one warp whose first lane only issues MMAs; the kernels are
                                                    // launched with one more warp on top (kIntraThreads + 32) that only
                                                    // issues bulk copies and takes no part in the named barrier
-enum { WITHHOLD_PREP = 1, WITHHOLD_CARRY = 2, WITHHOLD_GRADIENT = 3 };   // values of TcParams::withhold and of gdn_debug_inject_timeout
+// values of TcParams::withhold and of gdn_debug_inject_timeout
+enum { WITHHOLD_PREP = 1, WITHHOLD_CARRY = 2, WITHHOLD_GRADIENT = 3, DISAGREE_CARRY = 5 };
 struct TcParams {
     Problem p;
     CUtensorMap tm_q, tm_k, tm_v, tm_do;   // [T_total, H, d] bf16, boxes of 64 tokens x 64 features of a head
@@ -48,7 +49,8 @@ struct TcParams {
     int lowrank;                           // carries in low-rank form (tc_scan_lr): prepared by tc_prep_lr without Nm, Bf
     int narrow_v;                          // d_v = 64: of the kernels whose CTAs carry 64 state columns only the first half is launched
     int withhold;                          // debugging hook: a kernel leaves out one of its first loads, so that the wait for
-                                           // it runs out (exercises the time-out path without any fault)
+                                           // it runs out, or half of its warps take a first wait for one that did (exercises
+                                           // the time-out path without any fault)
 };
 
 // ------------------------------------------------------------------------------------------------
@@ -704,6 +706,7 @@ struct Shared {
     uint64_t full[2], mma;           // a ring slot has arrived; a product of the present step is done
     uint64_t free1[2], free2[2];     // by step parity: the tiles that the first product was the last to read, and all others, may be loaded over
     uint32_t tmem;
+    uint32_t gave_up[2];             // a warp has given up (tc_common.cuh), by parity of the step that judges it: behind its first barrier
 };
 constexpr int kScanThreads = kThreads + 32;   // ... and a warp that only loads: a tile of the step after next goes over its predecessor as
                                               // soon as the product that read it last is done
@@ -741,6 +744,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&sh.free1[s], 1); mbar_init(&sh.free2[s], 1); }
         mbar_init(&bar_mma, 1);
+        sh.gave_up[0] = sh.gave_up[1] = 0;
         fence_mbar_init();
     }
     if (warp == 0) { tmem_alloc(&sh.tmem, C::TMEM_COLS); tmem_relinquish(); }
@@ -793,12 +797,12 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
                 if (!mbar_wait(&sh.free2[s & 1], (s >> 1) & 1)) { ++s; break; }
                 fill2(s + STAGES);
             }
-            if (s + STAGES < nsteps) drain_ring<STAGES>(bar_full, s, nsteps);   // after a time-out loads may still be in flight
+            drain_ring<STAGES>(bar_full, s, nsteps);   // (what is still in flight after a time-out; otherwise the workers wait for the same loads)
         }
-        __syncthreads();
         return;
     }
     auto cta_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory"); };   // all warps but the loader
+    const bool disagree = P.withhold == DISAGREE_CARRY && (warp & 1);
     // the gate arrays of the first step; the cumulative decays of the second are fetched now
     auto gate_row = [&](int s) { return gamma + ((size_t)chunk_of(s) * H + hd) * kC; };
     auto make_gates = [&](int set, float g, float gend) {
@@ -825,6 +829,11 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
     cta_sync();
     bool ok = true;
     uint32_t mma_phase = 0;
+    auto wait_for = [&](uint64_t* bar, uint32_t parity, int where, int judged) {
+        if (!ok) return;
+        ok = mbar_wait_inline(bar, parity);
+        if (!ok) { report_timeout(p.ws, where); sh.gave_up[judged & 1] = 1; }
+    };
     int s = 0;
 #pragma unroll 1
     for (; s < nsteps; ++s) {
@@ -837,8 +846,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
 #pragma unroll
         for (int k = 0; k < NSH / 8; ++k) *reinterpret_cast<uint4*>(Ht + tile_chunk_off(128, r, (lc0 >> 3) + k)) = pack8(st + 8 * k);
         if (len < kC) {   // ragged tail: the rows beyond the sequence belong to somebody else
-            ok = mbar_wait_inline(&bar_full[stage], (s / STAGES) & 1);
-            if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 12); break; }
+            wait_for(&bar_full[stage], (s / STAGES) & 1, 12, s);
             zero_tail_rows(ring + KT, 64, 0, len, kThreads);
             if (reverse) {
                 zero_tail_rows(ring + QT, 64, 0, len, kThreads);
@@ -848,25 +856,22 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         }
         fence_async_smem();
         cta_sync();
+        const uint32_t gone = sh.gave_up[s & 1];   // (of this step so far and of the step before)
         const float Ge = gates.ge[s & 1];   // decay of the state over the chunk
-        if (warp == 0 && elect_one()) {
-            ok = mbar_wait_inline(&bar_full[stage], (s / STAGES) & 1);
-            if (ok) {
-                tc_fence_after();
-                // forward (W h)^T = h^T W^T ; reverse (K dh')^T = dh'^T K^T : [d_v][tokens]
-                const Operand b = reverse ? op_k_major(ring + KT, 64) : op_mn_major(ring + WT, 128);
-                mma_tile<NS, 64, 128>(tmem + C_D1, op_mn_major(Ht, 128), b, false);
-                if (reverse) mma_tile<NS, 64, 64>(tmem + C_D3, op_mn_major(ring + OT, 64), op_mn_major(ring + PT, 64), false);   // (P^T dO)^T
-            } else {
-                report_timeout(p.ws, 10);
-            }
+        wait_for(&bar_full[stage], (s / STAGES) & 1, 10, s + 1);
+        if (warp == 0 && elect_one() && ok) {
+            tc_fence_after();
+            // forward (W h)^T = h^T W^T ; reverse (K dh')^T = dh'^T K^T : [d_v][tokens]
+            const Operand b = reverse ? op_k_major(ring + KT, 64) : op_mn_major(ring + WT, 128);
+            mma_tile<NS, 64, 128>(tmem + C_D1, op_mn_major(Ht, 128), b, false);
+            if (reverse) mma_tile<NS, 64, 64>(tmem + C_D3, op_mn_major(ring + OT, 64), op_mn_major(ring + PT, 64), false);   // (P^T dO)^T
             bulk_store(keep_base + ch * 32768, Ht, HT_BYTES);
             bulk_commit();
             bulk_wait_read<1>();   // (the stores of the step before have read their tiles: they are rewritten from here on)
             mma_commit(&bar_mma);
             mma_commit(&sh.free1[s & 1]);
         }
-        ok = mbar_wait_inline(&bar_full[stage], (s / STAGES) & 1);
+        if (disagree) { ok = false; report_timeout(p.ws, 14); sh.gave_up[(s + 1) & 1] = 1; }
         if (reverse) {   // scale Diag(Gam) Q in place, under the first product; its product by dO runs under the readout
             if (ok) {
 #pragma unroll
@@ -882,11 +887,11 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
             }
             fence_async_smem();
             cta_sync();
-            if (warp == 0 && elect_one() && ok) mma_tile<128, NS, 64>(tmem + C_D2, op_mn_major(ring + QT, 64), op_mn_major(ring + OT, 64), false);
+            if (warp == 0 && elect_one() && ok && !gone) mma_tile<128, NS, 64>(tmem + C_D2, op_mn_major(ring + QT, 64), op_mn_major(ring + OT, 64), false);
         }
-        if (ok) ok = mbar_wait_inline(&bar_mma, mma_phase);
+        wait_for(&bar_mma, mma_phase, 11, s + 1);
         mma_phase ^= 1;
-        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 11); break; }
+        if (gone) break;   // (here, where no product is in flight any more and nobody waits for the word)
         tc_fence_after();
         // operand of the second product, transposed: forward Diag(e) U (and U, for the workspace), reverse dU
 #pragma unroll
@@ -918,7 +923,7 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         tc_fence_before();
         fence_async_smem();
         cta_sync();
-        if (warp == 0 && elect_one()) {
+        if (warp == 0 && elect_one() && ok) {
             tc_fence_after();
             if (reverse) mma_tile<128, NS, 64>(tmem + C_D2, op_k_major(ring + WT, 128), op_k_major(sm + GT, NS), true, /*neg_a=*/true);
             else mma_tile<128, NS, 64>(tmem + C_D2, op_mn_major(ring + KT, 64), op_k_major(sm + GT, NS), false);
@@ -931,9 +936,8 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
             make_gates((s + 1) & 1, gnext, gend_next);
             if (s + 2 < nsteps) { gnext = gate_row(s + 2)[threadIdx.x]; gend_next = gate_row(s + 2)[kC - 1]; }
         }
-        ok = mbar_wait_inline(&bar_mma, mma_phase);
+        wait_for(&bar_mma, mma_phase, 13, s + 1);
         mma_phase ^= 1;
-        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 13); break; }
         tc_fence_after();
 #pragma unroll
         for (int k = 0; k < NSH / 8; ++k) {
@@ -945,6 +949,8 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
         }
         tc_fence_before();
     }
+    cta_sync();   // every reader of the accumulators is done
+    ok = !(sh.gave_up[0] | sh.gave_up[1]);
     float* fin = reverse ? p.dh0 : p.hT;
     if (fin && ok) {
         const bool inside = r < p.d.d_k && part * NS + lc0 < p.d.d_v;   // (a head dimension of 64: the rest of the state is zero)
@@ -952,11 +958,11 @@ __device__ __forceinline__ void scan_lr_chain(const TcParams& P, int chain, int 
 #pragma unroll
         for (int k = 0; k < NSH / 4; ++k) if (inside) *reinterpret_cast<float4*>(fin + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
     }
-    if (warp == 0) bulk_wait_read<0>();
-    if (!ok && threadIdx.x == 32) drain_ring<STAGES>(bar_full, s, nsteps);
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, C::TMEM_COLS);
+    if (warp == 0) {
+        bulk_wait_read<0>();
+        tc_fence_after();
+        tmem_dealloc(tmem, C::TMEM_COLS);
+    }
 }
 
 // Block index -> (chain, direction, column block): with both directions in one launch the direction is the low bit

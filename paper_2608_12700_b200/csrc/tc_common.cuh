@@ -86,6 +86,11 @@ __device__ __forceinline__ void write_dg_suffix(const float* v0, const float* v1
     if (lane + 32 < len) dg[(size_t)(lane + 32) * stride] = b;
 }
 
+// Warps judge by their own clocks whether a wait has run out, so the warps of a CTA may disagree about one that ends close to the limit.  None
+// leaves on a verdict of its own: the others would wait for it at their next barrier without a bound, or work on behind its teardown.  A
+// warp that gives up sets a word `gave_up` in shared memory and takes part in every barrier up to the place where all look at it, with
+// a barrier between the last write and the first look; up to there it issues nothing, and what it leaves out is read by nobody.
+
 // After a wait gave up in step `s` of a chain: waits (bounded) for the loads of the ring that are in flight, so that the CTA does
 // not retire under them.  By one thread.  (Without a time-out s = nsteps and there is nothing to wait for; at most one of the
 // waits is for a load that was never issued.)

@@ -60,6 +60,31 @@ def test_every_kernel_leaves_through_its_teardown(shape, where, form):
         binding.gdn_debug_force_family(0)
 
 
+@pytest.mark.parametrize("form,where", [(3, 5)], ids=["low_rank-carries"])
+@pytest.mark.parametrize("shape", [dict(lengths=[200, 64, 75], H=2, d_v=128), dict(B=3, T=700, H=10, d_v=128), dict(lengths=[300, 64], H=2, d_v=64)],
+                         ids=["small", "several_trips", "narrow_values"])
+def test_warps_that_disagree_about_a_wait_leave_together(shape, form, where):
+    """Each warp judges by its own clock whether a wait has run out.  Half of them say so here although nothing is missing: the call ends (the
+    warps that went on are not left behind at a barrier), reports it, and the next one is correct."""
+    try:
+        binding.gdn_debug_force_family(form)
+        wl = synth.make_workload("timeout_split", dtype="bf16", d_k=128, states=True, seed=93, **shape)
+        buf = runner.to_device(wl)
+        for v in buf.outputs.values():
+            if v is not None:
+                v.fill_(7.0)
+        binding.gdn_debug_inject_timeout(where)
+        runner.run_bwd(buf)
+        assert binding.gdn_last_device_status(buf.workspace) == GDN_ERR_DEVICE_TIMEOUT
+        for n in ("dq", "dk", "dv", "dg", "dbeta", "dh0"):
+            assert torch.all(buf.outputs[n] == 7.0), n
+        runner.run_bwd(buf)
+        check_against_oracle(wl, runner.fetch(buf))
+        assert binding.gdn_last_device_status(buf.workspace) == binding.GDN_OK
+    finally:
+        binding.gdn_debug_force_family(0)
+
+
 def test_a_cancelled_request_changes_nothing():
     wl = synth.make_workload("timeout_cancel", dtype="bf16", lengths=[100], H=1, d_k=128, d_v=128, states=True, seed=91)
     binding.gdn_debug_inject_timeout(True)
