@@ -238,8 +238,9 @@ gdn_status gdn_debug_force_family(int32_t family);
  * leaves out one of its input loads, so the wait for it runs out.  The CTAs leave through their normal teardown
  * (tensor memory released, no copy in flight), the remaining kernels of the call see the status word and write
  * nothing, gdn_bwd itself returns GDN_OK and gdn_last_device_status reports GDN_ERR_DEVICE_TIMEOUT.  The next call
- * is a normal one.  2 and 3: the same in the carries and in the gradient stage.  5: no load is left out, but half of the warps of the
- * carries (low-rank form) take their first wait for one that ran out, while the others go on.  0 cancels a pending request. */
+ * is a normal one.  2 and 3: the same in the carries and in the gradient stage.  4, 5 and 6: no load is left out, but half of the warps
+ * of the preparation, the carries or the gradient stage take a first wait for one that ran out, while the others go on.  0 cancels a
+ * pending request. */
 gdn_status gdn_debug_inject_timeout(int32_t on);
 
 #ifdef __cplusplus

@@ -258,5 +258,5 @@ def gdn_bwd_channelwise(desc, q, k, v, g, b, w, h0, dO, dhT, cu_seqlens, dq, dk,
 
 def gdn_debug_inject_timeout(on=True) -> None:
     """The next gdn_bwd of this thread on the tcgen05 d = 128 family makes one bounded device-side wait run out, in its first
-    chunk-level kernel (True or 1), in the carries (2) or in the gradient stage (3)."""
+    chunk-level kernel (True or 1), in the carries (2) or in the gradient stage (3); 4, 5 and 6: half of the warps there take one for run out."""
     lib().gdn_debug_inject_timeout(int(on))

@@ -291,7 +291,7 @@ gdn_status gdn_debug_force_family(int32_t family) {
 }
 
 gdn_status gdn_debug_inject_timeout(int32_t on) {
-    g_inject_timeout = on == 2 || on == 3 || on == 5 ? on : on ? 1 : 0;
+    g_inject_timeout = on >= 2 && on <= 6 ? on : on ? 1 : 0;
     return GDN_OK;
 }
 

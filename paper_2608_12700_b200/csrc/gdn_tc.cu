@@ -38,7 +38,7 @@ constexpr int kIntraThreads = kWideThreads + 32;   // ... plus one warp whose fi
                                                    // launched with one more warp on top (kIntraThreads + 32) that only
                                                    // issues bulk copies and takes no part in the named barrier
 // values of TcParams::withhold and of gdn_debug_inject_timeout
-enum { WITHHOLD_PREP = 1, WITHHOLD_CARRY = 2, WITHHOLD_GRADIENT = 3, DISAGREE_CARRY = 5 };
+enum { WITHHOLD_PREP = 1, WITHHOLD_CARRY = 2, WITHHOLD_GRADIENT = 3, DISAGREE_PREP = 4, DISAGREE_CARRY = 5, DISAGREE_GRADIENT = 6 };
 struct TcParams {
     Problem p;
     CUtensorMap tm_q, tm_k, tm_v, tm_do;   // [T_total, H, d] bf16, boxes of 64 tokens x 64 features of a head
@@ -205,9 +205,9 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
                 mbar_arrive(&bar_free);    // every staging tile may be rewritten
             }
             bulk_wait_read<0>();
-            if (!lok) {   // after a timeout a copy may still be in flight: wait for it before the CTA may retire
-                if (pend_qk) (void)mbar_wait(&bar_qk, ph ^ 1);
-                if (pend_vo) (void)mbar_wait(&bar_vo, ph ^ 1);
+            if (!lok) {   // after a timeout a copy may still be in flight, of this trip or of the next one: wait for it before the CTA may retire
+                (void)mbar_wait(&bar_qk, pend_qk ? ph ^ 1 : ph);
+                (void)mbar_wait(&bar_vo, pend_vo ? ph ^ 1 : ph);
             }
         }
         return;
@@ -279,8 +279,8 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     const float* bgam = gate_sets[in_phase][5];
     if (ok) {
         ok = mbar_wait(&bar_vo, in_phase);
-        ok = ok && mbar_wait(&bar_qk, in_phase);
-        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 1);
+        ok = ok && mbar_wait(&bar_qk, in_phase) && !(P.withhold == DISAGREE_PREP && (warp & 1));
+        if (!ok && lane == 0) report_timeout(p.ws, 1);
     }
     if (ok && x.len < kC) {   // identity padding of a ragged tail: rows beyond the sequence read as zero
         zero_tail_rows(sm + QK, 128, 0, x.len, kIntraThreads);
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     GDN_WAIT_MMA(2)
     if (ok && !first) {   // the previous trip's stores have read what lies under the fp32 A block and under P
         ok = mbar_wait(&bar_free1, in_phase ^ 1);
-        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 6);
+        if (!ok && lane == 0) report_timeout(p.ws, 6);
     }
     if (ok && worker) {
         const int i = (q4 & 1) * 32 + lane, j0 = grp * kTG;
@@ -357,12 +357,12 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     // ---- T = (I + A)^-1, blocked, fp32 (invert64)
     if (ok && !first) {   // ... and what lies under the fp32 T block
         ok = mbar_wait(&bar_free2, in_phase ^ 1);
-        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 8);
+        if (!ok && lane == 0) report_timeout(p.ws, 8);
     }
     invert64(Af, Tf, cta_sync);
     if (ok && !first) {   // every store of the previous trip has read its tile (the T tiles and the second readout are next)
         ok = mbar_wait(&bar_free, in_phase ^ 1);
-        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 5);
+        if (!ok && lane == 0) report_timeout(p.ws, 5);
     }
     if (threadIdx.x < kC * 4) {   // T -> bf16 tiles T, T Diag(b Gam), T Diag(w): a thread scales two rows of one 8-column piece
         const int cch = threadIdx.x & 7;
@@ -444,14 +444,14 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
         if (bwd) mma_tile<128, 128, 64>(tmem + C_E, op_k_major(sm + WT, 128), op_k_major(sm + XPDO, 128), true, /*neg_a=*/true);
         mma_commit(&bar_mma);
         mma_commit(&bar_ld1);   // Q, K have been read for the last time
-    } else if (threadIdx.x == 32) {
+    } else if (threadIdx.x == 32 && ok) {   // (a load is announced behind one that has arrived only)
         mbar_arrive(&bar_vofree);   // W^T, U~^T are staged; V, dO were last read by phase 2 and the pass that formed R
     }
     if (has_next && warp == 0) make_gates(in_phase ^ 1, xn.ch);   // the next trip's gate arrays, while the products run
     GDN_WAIT_MMA(4)
     if (ok) {   // the T tile, part of the Nm staging area, has left through its store
         ok = mbar_wait(&bar_tfree, in_phase);
-        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 7);
+        if (!ok && lane == 0) report_timeout(p.ws, 7);
     }
     if (ok && worker) {   // Nm, Bf, E -> bf16 tile images staged over tiles that no MMA reads any more
         const int r = q4 * 32 + lane, c0 = grp * (D / kGroups);
@@ -479,8 +479,8 @@ __global__ void __launch_bounds__(kIntraThreads + 32, 1) tc_prep_kernel(const __
     fence_async_smem();
     cta_sync();
     if (threadIdx.x == 32) mbar_arrive(&bar_st);   // the three images are staged: the loader stores them
-    if (!ok) {   // a load of this trip may still be in flight: wait for it (bounded) before the CTA retires
-        if (threadIdx.x == 0) { (void)mbar_wait(&bar_vo, in_phase); (void)mbar_wait(&bar_qk, in_phase); }
+    if (!ok) {   // (the loader, which gives up in turn, waits for the loads that are in flight)
+        stand_by_items<10>(item, n_items, cta_sync);
         break;
     }
     }
@@ -595,6 +595,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
         }
     }
     __syncthreads();
+    const bool disagree = P.withhold == DISAGREE_CARRY && (warp & 1);
     bool ok = true;
     uint32_t mma_phase = 0;
     int s = 0;
@@ -631,10 +632,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
             // to issue; a thread of another warp does it so that the MMA issue is not delayed.
             if (s >= 1 && s - 1 + STAGES < nsteps) fill(s - 1 + STAGES);
         }
-        ok = mbar_wait(&bar_full[stage], (s / STAGES) & 1);   // the additive term of this step is in shared memory
+        ok = mbar_wait(&bar_full[stage], (s / STAGES) & 1) && !disagree;   // the additive term of this step is in shared memory
         if (ok) ok = mbar_wait(&bar_mma, mma_phase);
         mma_phase ^= 1;
-        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 11); break; }
+        if (!ok) {
+            if (lane == 0) report_timeout(p.ws, 11);
+            stand_by(nsteps - 1 - s, [] { __syncthreads(); });
+            break;
+        }
         tc_fence_after();
 #pragma unroll
         for (int k = 0; k < NSH / 8; ++k) {
@@ -647,6 +652,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
         }
         tc_fence_before();
     }
+    if (threadIdx.x == 32) drain_ring<STAGES>(bar_full, s, nsteps);
+    ok = __syncthreads_and(ok);
     float* fin = reverse ? p.dh0 : p.hT;
     if (fin && ok) {
         const bool inside = r < p.d.d_k && gc0 < p.d.d_v;   // (a head dimension of 64: the rest of the state is zero)
@@ -654,11 +661,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
 #pragma unroll
         for (int k = 0; k < NSH / 4; ++k) if (inside) *reinterpret_cast<float4*>(fin + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
     }
-    if (warp == 0) bulk_wait_read<0>();
-    if (threadIdx.x == 32) drain_ring<STAGES>(bar_full, s, nsteps);
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, NS);
+    if (warp == 0) {
+        bulk_wait_read<0>();
+        tc_fence_after();
+        tmem_dealloc(tmem, NS);
+    }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1147,7 +1154,7 @@ __device__ __forceinline__ void scan_cw_chain(const TcParams& P, int chain, int 
         ok = mbar_wait_inline(&bar_full[stage], (s / STAGES) & 1);
         if (ok) ok = mbar_wait_inline(&bar_mma, mma_phase);
         mma_phase ^= 1;
-        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 11); break; }
+        if (!ok) { if (lane == 0) report_timeout(p.ws, 11); break; }
         tc_fence_after();
         // operand of the second product: forward Diag(e)(U~ - W h), reverse Diag(e)(K dh'), transposed
 #pragma unroll
@@ -1175,7 +1182,7 @@ __device__ __forceinline__ void scan_cw_chain(const TcParams& P, int chain, int 
         }
         ok = mbar_wait_inline(&bar_mma, mma_phase);
         mma_phase ^= 1;
-        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 13); break; }
+        if (!ok) { if (lane == 0) report_timeout(p.ws, 13); break; }
         tc_fence_after();
         if (!reverse) Ge *= pow2(cw_next.ref - ref);   // A
 #pragma unroll
@@ -1457,10 +1464,10 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
                 mbar_arrive(&bar_free);   // the staging regions may be rewritten
             }
             bulk_wait_read<0>();
-            if (!lok) {   // after a timeout a copy may still be in flight: wait for it before the CTA may retire
-                if (pend_a) (void)mbar_wait(&bar_a, ph ^ 1);
-                if (pend_b) (void)mbar_wait(&bar_b, ph ^ 1);
-                if (pend_u) (void)mbar_wait(&bar_u, ph ^ 1);
+            if (!lok) {   // after a timeout a copy may still be in flight, of this trip or of the next one: wait for it before the CTA may retire
+                (void)mbar_wait(&bar_a, pend_a ? ph ^ 1 : ph);
+                (void)mbar_wait(&bar_b, pend_b ? ph ^ 1 : ph);
+                (void)mbar_wait(&bar_u, pend_u ? ph ^ 1 : ph);
             }
         }
         return;
@@ -1543,16 +1550,17 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     float rs = 0.f;
     if (FACTORS && gates && have_prev && ok) finish_gates();   // the previous chunk's gate gradients (what they are made of is rewritten below)
     if (ok) {
-        ok = mbar_wait(&bar_a, in_phase);
-        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 20);
+        ok = mbar_wait(&bar_a, in_phase) && !(FACTORS && P.withhold == DISAGREE_GRADIENT && (warp & 1));
+        if (!FACTORS && P.withhold == DISAGREE_GRADIENT && (warp & 1)) ok = false;
+        if (!ok && lane == 0) report_timeout(p.ws, 20);
     }
     if (FACTORS && ok) {
         ok = mbar_wait(&bar_u, in_phase);
-        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 27);
+        if (!ok && lane == 0) report_timeout(p.ws, 27);
     }
     if (FACTORS && ok && !first) {   // dXv goes where the previous trip's dk is staged, dq over its dq: the stores must have read them
         ok = mbar_wait(&bar_free, in_phase ^ 1);
-        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 28);
+        if (!ok && lane == 0) report_timeout(p.ws, 28);
     }
     if (ok && !full) {
         if (!FACTORS) zero_tail_rows(sm + KT, 64, 0, x.len, kWideThreads);
@@ -1576,12 +1584,12 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     if (gates && have_prev && ok) finish_gates();   // the previous chunk's gate gradients
     if (ok) {
         ok = mbar_wait(&bar_u, in_phase);
-        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 27);
+        if (!ok && lane == 0) report_timeout(p.ws, 27);
     }
     GDN_WAIT_MMA(22)
     if (ok && !first) {   // U^T and dU^T held the previous trip's staged dk and dq: their stores must have read them
         ok = mbar_wait(&bar_free, in_phase ^ 1);
-        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 28);
+        if (!ok && lane == 0) report_timeout(p.ws, 28);
     }
     if (ok && worker && (DV == 128 || q4 < 2)) {
         const int f = q4 * 32 + lane;      // feature (lane of the transposed accumulators)
@@ -1613,13 +1621,13 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     }
     if (ok) {   // T and V are needed from phase 2 on, Q from phase 3 on
         ok = mbar_wait(&bar_b, in_phase);
-        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 31);
+        if (!ok && lane == 0) report_timeout(p.ws, 31);
     }
     if (ok && !full) zero_tail_rows(sm + QT, 64, 0, x.len, kWideThreads);
     tc_fence_before();
     fence_async_smem();
     cta_sync();
-    if (threadIdx.x == 32) mbar_arrive(&bar_e0);   // U~^T has been read
+    if (threadIdx.x == 32 && ok) mbar_arrive(&bar_e0);   // U~^T has been read (a load is announced behind one that has arrived only)
     }
     else { cta_sync(); }
 
@@ -1658,7 +1666,7 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     if (gates && has_next) fetch_gates(xn);
     if (FACTORS && ok) {   // V is needed now, Q from phase 3 on, K from phase 4 on
         ok = mbar_wait(&bar_b, in_phase);
-        if (!ok && threadIdx.x == 0) report_timeout(p.ws, 31);
+        if (!ok && lane == 0) report_timeout(p.ws, 31);
         if (ok && !full) {
             zero_tail_rows(sm + QT, 64, 0, x.len, kWideThreads);
             zero_tail_rows(sm + KT, 64, 0, x.len, kWideThreads);
@@ -1837,14 +1845,21 @@ __global__ void __launch_bounds__(intra::kThreadsAll, 1) tc_intra_kernel(const _
     have_prev = true;
     tc_fence_before();
     fence_async_smem();
-    cta_sync();   // every reader of this trip's tiles and scratch is done
+    // every reader of this trip's tiles and scratch is done.  (Without FACTORS the warps leave together on the outcome of the barrier: to stand by
+    // takes registers there, and spills: 16 heads of 16384 tokens 635 -> 646 us.  With FACTORS the outcome costs 0.2 %.)
+    if (FACTORS) {
+        cta_sync();
+    } else if (!named_barrier_and<kBarThreads>(ok)) {
+        if (warp == 0) tmem_dealloc(tmem, 512);
+        return;   // (the loader, which gives up in turn, waits for the loads that are in flight)
+    }
     if (threadIdx.x == 32) mbar_arrive(&bar_st2);   // dq, dk are staged: the loader stores them
     if (ok && !full) {
         flush_rows(sm + SQ, p.dq, x, H, p.d.d_k, kWideThreads);
         flush_rows(sm + SK, p.dk, x, H, p.d.d_k, kWideThreads, SK_ROWS, SK_ROW0);
     }
-    if (!ok) {   // a load of this trip may still be in flight: wait for it (bounded) before the CTA retires
-        if (threadIdx.x == 0) { (void)mbar_wait(&bar_a, in_phase); (void)mbar_wait(&bar_u, in_phase); (void)mbar_wait(&bar_b, in_phase); }
+    if (FACTORS && !ok) {
+        stand_by_items<4>(item, n_items, cta_sync);
         break;
     }
     }
@@ -1940,7 +1955,7 @@ __global__ void __launch_bounds__(kThreads, 2) tc_out_kernel(const __grid_consta
         }
         if (ok) {
             ok = mbar_wait(&bar_in, in_phase);
-            if (!ok && threadIdx.x == 0) report_timeout(p.ws, 30);
+            if (!ok && lane == 0) report_timeout(p.ws, 30);
             if (ok && threadIdx.x == 0) pending = false;
         }
         if (!CW && ok && x.len < kC) {   // ragged tail: rows beyond the sequence belong to somebody else (the images are padded)

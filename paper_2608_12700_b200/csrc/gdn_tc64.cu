@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kThreads64, 2) tc64_fwd_kernel(const __grid_co
         unsigned char* HT = sm + C::HT + (s & 1) * 8192;
         const float *gl = gl2[s & 1], *Gam = Gam2[s & 1], *ee = ee2[s & 1];
         ok = mbar_wait(&bar_full[stage], (s / STAGES) & 1);
-        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 40); give_up(s); break; }
+        if (!ok) { if (lane == 0) report_timeout(p.ws, 40); give_up(s); break; }
         if (len < kC) {
             zero_tail_rows64(tiles + KT, len);
             zero_tail_rows64(tiles + VT, len);
@@ -397,6 +397,8 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
     }
     bool ok = true;
     uint32_t mma_phase = 0;
+    // a warp that gives up in step s behind `passed` of its barriers (three, and a fourth in the first step if that chunk is a ragged tail)
+    auto leave = [&](int s, int passed) { stand_by((nsteps - s) * 3 - passed + (s == 0 && cg.chunk_len(c1 - 1) < kC ? 1 : 0), cta_sync); };
     int len_n = nsteps > 0 ? cg.chunk_len(c1 - 1) : 0, tok0_n = nsteps > 0 ? cg.chunk_tok0(c1 - 1) : 0;   // fetched a step ahead
 #pragma unroll 1
     for (int s = 0; s < nsteps; ++s) {
@@ -405,7 +407,7 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
         unsigned char* tiles = sm + stage * STAGE_BYTES;
         const float *gl = gl2[s & 1], *Gam = Gam2[s & 1], *ee = ee2[s & 1];
         ok = mbar_wait(&bar_full[stage], (s / STAGES) & 1);
-        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 50); break; }
+        if (!ok) { if (lane == 0) report_timeout(p.ws, 50); leave(s, 0); break; }
         if (len < kC) {
             zero_tail_rows64(tiles + QT, len);
             zero_tail_rows64(tiles + KT, len);
@@ -441,7 +443,7 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
             if (s + 2 < nsteps) { gnext = gate_row(s + 2)[threadIdx.x]; gend_next = gate_row(s + 2)[kC - 1]; }
         }
         GDN_WAIT_MMA(51)
-        if (!ok) break;
+        if (!ok) { leave(s, 1); break; }
         {   // A: P = tril(Q K^T . D)   B: dP . D = scale tril(dO V^T) . D
             const float glr = gl[r], f = ga ? 1.f : sc;
             unsigned char* dst = sm + (ga ? PX : DPD);
@@ -458,7 +460,7 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
             }
         }
         ok = mbar_wait(&bar_mma2, 0);
-        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 53); break; }
+        if (!ok) { if (lane == 0) report_timeout(p.ws, 53); leave(s, 1); break; }
         tc_fence_after();
 #pragma unroll
         for (int t = 0; t < 2; ++t) {   // Diag(Gam) dO over the dh' tile, which no MMA reads any more
@@ -486,7 +488,7 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
             mma_commit(&bar_mma2);
         }
         GDN_WAIT_MMA(52)
-        if (!ok) break;
+        if (!ok) { leave(s, 2); break; }
         // Gradient rows are staged token-major in place over this step's input tiles (dv over V, dk over K and dq over Q, where
         // a thread overwrites exactly the piece it has just read; every product that reads the tile is done) and leave by TMA
         // stores; generic global stores here would be one 16-byte piece per row.
@@ -515,7 +517,7 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
             if (ga) dot = 0.f;
         }
         ok = mbar_wait(&bar_mma2, 1);
-        if (!ok) { if (threadIdx.x == 0) report_timeout(p.ws, 54); break; }
+        if (!ok) { if (lane == 0) report_timeout(p.ws, 54); leave(s, 2); break; }
         tc_fence_after();
         {   // dq = scale Gam dO h^T + (dP.D) K ;  dh = Gam_e dh' + scale (Diag(Gam) Q)^T dO
             const float G = sc * Gam[r];
@@ -564,13 +566,16 @@ __global__ void __launch_bounds__(kThreads64 + 32, 2) tc64_bwd_kernel(const __gr
             write_dg_suffix(dgp[0], dgp[1], rsum + Ge * hsum, p.dg + (size_t)tok0 * H + hd, (size_t)H, len, lane);
         }
     }
+    tc_fence_before();
+    ok = named_barrier_and<kThreads64>(ok);
+    if (warp == 0) {
+        tc_fence_after();
+        tmem_dealloc(tmem, 256);
+    }
     if (p.dh0 && ok) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) *reinterpret_cast<float4*>(p.dh0 + soff + 4 * k) = make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
     }
-    tc_fence_before();
-    cta_sync();
-    if (warp == 0) tmem_dealloc(tmem, 256);
 }
 
 }  // namespace

@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kT, 2) cw_prep_kernel(const __grid_constant__ 
         {   // (waited for in any case: it is in flight)
             const bool okk = mbar_wait(&bar_k, in_phase);
             ok = ok && okk;
-            if (!ok && threadIdx.x == 0) report_timeout(p.ws, 40);
+            if (!ok && lane == 0) report_timeout(p.ws, 40);
         }
         if (ok && bwd && x.len < kC) {   // rows beyond the sequence belong to somebody else (the images have zeros there)
             zero_tail_rows(sm + VO, 128, 64, x.len, kT);
@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(kT, 2) cw_eprep_kernel(const __grid_constant__
         if (has_next) chunk_entry_tab(p, xn, item + gridDim.x);
         if (ok) {
             ok = mbar_wait(&bar_in, in_phase);
-            if (!ok && threadIdx.x == 0) report_timeout(p.ws, 46);
+            if (!ok && lane == 0) report_timeout(p.ws, 46);
             if (ok && threadIdx.x == 0) pending = false;
         }
         if (ok && x.len < kC) {
@@ -628,7 +628,7 @@ __global__ void __launch_bounds__(intracw::kWorkers, 1) cw_intra_kernel(const __
         const bool whole = live >= kTok;      // (two copies of the accesses: a condition at each of them costs more than it skips)
         if (ok) {   // everything step 1 reads (the carries left h~ and dh'', the forms used here)
             ok = mbar_wait(&bar_s, in_phase) && mbar_wait(&bar_k, in_phase) && mbar_wait(&bar_b, in_phase) && mbar_wait(&bar_a, in_phase);
-            if (!ok && threadIdx.x == 0) report_timeout(p.ws, 44);
+            if (!ok && lane == 0) report_timeout(p.ws, 44);
             if (ok) pend_s = pend_k = pend_a = pend_b = false;
         }
         if (ok && x.len < kC) {   // rows beyond the sequence belong to somebody else (the images have zeros there)

@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(split::kT, 2) tc_eprep_kernel(const __grid_con
         }
         if (ok) {
             ok = mbar_wait(&bar_in, in_phase);
-            if (!ok && threadIdx.x == 0) report_timeout(p.ws, 24);
+            if (!ok && lane == 0) report_timeout(p.ws, 24);
             if (ok && threadIdx.x == 0) pending = false;
         }
         if (ok && x.len < kC) {   // identity padding of a ragged tail
@@ -281,7 +281,8 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
         }
         if (ok) {
             ok = mbar_wait(&bar_in, in_phase);
-            if (!ok && threadIdx.x == 0) report_timeout(p.ws, 1);
+            if (P.withhold == DISAGREE_PREP && (warp & 1)) ok = false;
+            if (!ok && lane == 0) report_timeout(p.ws, 1);
             if (ok && threadIdx.x == 0) pending = false;
         }
         if (ok && x.len < kC) {   // identity padding of a ragged tail
@@ -393,7 +394,10 @@ __global__ void __launch_bounds__(split::kT, 2) tc_prep_lr_kernel(const __grid_c
             if (has_next) load_v(xn);
         }
         if (ok && has_next && warp == 0) fetch_gates(xn);
-        if (!ok) break;
+        if (!ok) {
+            stand_by_items<10>(item, n_items, [] { __syncthreads(); });
+            break;
+        }
         x = xn;
     }
     if (warp == 0) bulk_wait_read<0>();

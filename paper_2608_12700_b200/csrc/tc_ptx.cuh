@@ -94,6 +94,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
 #endif
 }
 
+// Named barrier 1 of COUNT threads; true if `v` was true in all of them.
+template <int COUNT>
+__device__ __forceinline__ bool named_barrier_and(bool v) {
+    uint32_t all;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "bar.red.and.pred q, 1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(all)
+        : "r"((uint32_t)v), "n"(COUNT)
+        : "memory");
+    return all != 0;
+}
+
 // ---------------------------------------------------------------- proxies and copies
 // Make generic-proxy writes to shared memory visible to the async proxy (TMA, tcgen05.mma).
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }

@@ -60,7 +60,8 @@ def test_every_kernel_leaves_through_its_teardown(shape, where, form):
         binding.gdn_debug_force_family(0)
 
 
-@pytest.mark.parametrize("form,where", [(3, 5)], ids=["low_rank-carries"])
+@pytest.mark.parametrize("form", [2, 3], ids=["operator", "low_rank"])
+@pytest.mark.parametrize("where", [4, 5, 6], ids=["preparation", "carries", "gradients"])
 @pytest.mark.parametrize("shape", [dict(lengths=[200, 64, 75], H=2, d_v=128), dict(B=3, T=700, H=10, d_v=128), dict(lengths=[300, 64], H=2, d_v=64)],
                          ids=["small", "several_trips", "narrow_values"])
 def test_warps_that_disagree_about_a_wait_leave_together(shape, form, where):
@@ -76,7 +77,7 @@ def test_warps_that_disagree_about_a_wait_leave_together(shape, form, where):
         binding.gdn_debug_inject_timeout(where)
         runner.run_bwd(buf)
         assert binding.gdn_last_device_status(buf.workspace) == GDN_ERR_DEVICE_TIMEOUT
-        for n in ("dq", "dk", "dv", "dg", "dbeta", "dh0"):
+        for n in ("dq", "dk", "dv", "dg", "dbeta", "dh0") if where < 6 else ():   # (the kernels behind the one in question, and its final states)
             assert torch.all(buf.outputs[n] == 7.0), n
         runner.run_bwd(buf)
         check_against_oracle(wl, runner.fetch(buf))
