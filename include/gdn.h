@@ -221,8 +221,9 @@ gdn_status gdn_stage_timing_read(int32_t max_stages, float* total_ms, int32_t* l
  *   "gamma" [64]   "T" [64,64]   "W" [64,d_k]   "Ut" [64,d_v]   "Nm" [d_k,d_k]
  *   "Bf", "E", "hc", "dhn" [d_k,d_v]
  * "Nm" and "Bf" are written only when the carries run in operator form (see below).  "E" is scale (Diag(Gam) Q - P W)^T dO, the term of
- * the reverse carry that depends on no state; the tcgen05 d = 128 kernels do not form it when their carries run in low-rank form (refused).
- * "Ut" is T Diag(w) V (read after a forward carry or a backward).
+ * the reverse carry that depends on no state; the tcgen05 d = 128 kernels do not form it when their carries run in low-rank form (refused;
+ * with gdn_debug_force_family(2) they do).  "Ut" is T Diag(w) V (read after a forward carry or a backward; in low-rank form it is put together
+ * from U, W and h as they are stored).
  * gdn_debug_force_family: 0 = automatic dispatch, 1 = always use the FFMA kernels (tests use this to
  * exercise both families on the same inputs); 2 / 3 = automatic family, but the tcgen05 d = 128 kernels carry the
  * state across chunks in operator form (one d x d matrix per chunk) / in low-rank form (two dependent products

@@ -50,7 +50,8 @@ struct Thread {
 
 // Unrolling of the products of the per-channel kernels (and of dU0) at DK key features.  At 128 such a kernel is 100 KB of code that a CTA runs
 // once, and with a CTA on most SMs two steps side by side cost more in instruction fetches than they give: 8 heads of 1024 tokens
-// 216 -> 206 us (6 of 800 tokens, on half of the SMs: 175 -> 176; d = 64: 87.3 -> 90.2); dU0 with E alone 23.1 -> 20.0 us.
+// 216 -> 206 us, and dU0 with E alone 3 us less.  (The line is drawn by DK alone: with fewer CTAs there is nothing to gain, 6 heads of 800 tokens, on
+// half of the SMs, 175 -> 176; at d = 64 the code is short enough for two steps, 87.3 us against 90.2.)
 template <int DK>
 constexpr int kU = DK == 128 ? 1 : 2;
 

@@ -12,8 +12,8 @@
 //   out    : forward output
 // One CTA handles one (chunk, head) in the parallel stages.  Operands are staged in shared memory, products are register
 // tiles (ffma_tile.cuh).  Every reduction has a fixed order: results are bit-identical from run to run.
-// At d = 128 the gradient stage of a chunk-head is 5.6 M FMAs, 23 us at the rate of one SM; measured 55 us (forward preparation
-// 22 us, the backward's share of it 21 us): eight warps on an SM issue in half of the cycles, between barriers.  With the operands of every FMA read from
+// At d = 128 the gradient stage of a chunk-head is 5.6 M FMAs, 23 us at the rate of one SM; measured 58 us (forward preparation
+// 27 us, the backward's share of it 22 us): eight warps on an SM issue in half of the cycles, between barriers.  With the operands of every FMA read from
 // global memory, and the solve and the sums over a chunk done by single threads, the same stages took 907, 165 and 102 us
 // (2 x 4 heads of 1000 tokens); the smallest call, 2 heads of 128 tokens at d = 64, went from 370 to 35 us.
 #include <cooperative_groups.h>

@@ -680,9 +680,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_scan_kernel(const __grid_const
 // (W h)^T or (K dh')^T with features on TMEM lanes and tokens on columns, the readout forms the bf16 operand of the second product in the
 // same orientation, the second product yields the d_k x d_v increment of the state, which lives in fp32 registers as in tc_scan.  P^T dO
 // and Q^T dO do not depend on the state: they are issued behind the first product and run under its readout.
-// 4 x 16 heads of 2048 tokens, both directions: 93 us, 216 KB per chunk-head at 4.8 TB/s, which bounds it (with the additive term E from the
+// 4 x 16 heads of 2048 tokens, both directions: 88 us, 216 KB per chunk-head at 4.8 TB/s, which bounds it (with the additive term E from the
 // preparation, U and dU left to the consumers, 77; the preparation took 80 us for 64, the gradient stage 115 for 105, the output of 6 x 16
-// heads of 1500 tokens 51 for 44, and a backward on the forward's workspace had a kernel more, of 38 us).
+// heads of 1500 tokens 51 for 44, and a backward on the forward's workspace had a kernel more, of 38 us).  What it costs: a forward without output,
+// which leaves U for a backward that may follow, 1 to 7 % (64 chains of 32 chunks 125 -> 134 us; with that backward 357 -> 333).
 // ------------------------------------------------------------------------------------------------
 namespace scanlr {
 constexpr uint32_t WT = 0, KT = 16384, XT = 32768;   // ring slot: W^T | K | forward: this CTA's part of U~^T (16 KB / S), and room for U^T behind it
@@ -690,9 +691,9 @@ constexpr uint32_t UT = 49152;
 constexpr uint32_t QT = 32768, PT = 49152, OT = 57344;   // reverse: Q | P | this CTA's columns of dO
 constexpr uint32_t C_D1 = 0, C_D3 = 64, C_D2 = 128;      // TMEM columns: first product (64), (P^T dO)^T (64), second product (128 / S)
 // S = number of CTAs that share a chain, each carrying 128 / S state columns (the columns of the state evolve
-// independently; W and K are needed whole by every one of them).  S = 2 serves calls that run one direction only with so
-// few chains that half of the SMs would idle (the forward, the backward on a fresh workspace): a step of a half is
-// shorter, and a step's latency is what bounds those launches.
+// independently; W and K are needed whole by every one of them).  S = 2 serves the reverse carry alone (the backward on a fresh workspace) with
+// so few chains that half of the SMs would idle: a step of a half is shorter, and a step's latency is what bounds that launch; and every
+// call with d_v = 64, where the first half is all there is.
 template <int S> struct Cfg {
     static constexpr int NS = D / S;                          // state columns of this CTA = rows of the first product
     static constexpr int NSH = NS / 2;                        // ... of one thread
@@ -2062,11 +2063,13 @@ thread_local int g_inject_timeout = 0;   // set by gdn_debug_inject_timeout, con
 
 static int sm_count();
 // Up to 37 chains (on 148 SMs) the operator form gives each direction of a chain two CTAs, and its one product per step wins; from
-// 38 on it would have one, and the low-rank form moves less.  Backward, us, operator / low-rank: 4 chains of 6 chunks 32.1 / 38.4,
-// 16 of 128 317 / 414, 32 of 32 154.8 / 158.9, 37 of 32 172.0 / 170.2; 38 of 32 198 / 173, 64 of 32 290 / 243; the line lies
-// there from 1 chunk to 256.  (A forward with its output and the backward on its workspace, each with one direction per launch,
-// would change sides near 64 chains: 38 of 32 250 / 266.)  The rule looks at the chains only, so the forward, the backward and
-// a backward on a workspace fresh from the forward agree on the form (and on the workspace layout that follows from it).
+// 38 on it would have one, and the low-rank form moves less.  Backward, us, operator / low-rank: 16 chains of 8 chunks 35.6 / 42.4, 16 of
+// 128 317 / 413, 32 of 32 155.4 / 158.9, 37 of 32 172.4 / 170.2; 38 of 32 197 / 177, 64 of 32 290 / 243.  One line for all numbers of chunks and
+// both calls has its price: 24 to 37 chains of 8 chunks (a step 79.0 / 74.4 at 32), steps of one chunk at any number of chains (42.5 / 39.0), and
+// steps of 38 to 48 chains of 128 chunks (823 / 914).  With d_v = 64 the operator form has one CTA of 64 columns per direction up to 74
+// chains; there too the low-rank form is faster from 38 on (38 of 32 172.6 / 159.6, 64 of 32 255 / 217; 38 of 128 570 / 574), in short calls from 24 on.
+// The rule looks at the chains only, so the forward, the backward and a backward on a workspace fresh from the forward agree on the form (and
+// on the workspace layout that follows from it).  All of it: profiles/carry_forms.md
 bool tc_carries_lowrank(const gdn_desc& d) {
     if (g_force_carries) return g_force_carries == 2;
     return 4 * (long long)d.N * d.H > sm_count();
@@ -2227,8 +2230,7 @@ cudaError_t tc_launch_fwd(const Problem& p, cudaStream_t st) {
 }
 
 // With a workspace fresh from gdn_fwd_recompute nothing of the forward is repeated: P, T, W, U~ and the per-chunk states
-// are taken from it, and only what needs dO is built (E; tc_eprep), followed by the reverse carry and the
-// gradient stage.  A status that the forward left stands.
+// are taken from it; the reverse carry and the gradient stage follow, in operator form behind E (tc_eprep).  A status that the forward left stands.
 cudaError_t tc_launch_bwd(const Problem& p, bool skip_recompute, cudaStream_t st) {
     TcParams P;
     cudaError_t e = launch_table_if_needed(p, skip_recompute, st);

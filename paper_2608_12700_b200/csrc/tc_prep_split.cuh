@@ -1,5 +1,5 @@
 // The chunk-local preparation of the tcgen05 d = 128 family with the carries in low-rank form (included by gdn_tc.cu), as
-// small kernels: about 105 KB of shared memory and 256 columns of tensor memory each, so that two CTAs share an SM.  A CTA
+// small kernels: about 90 KB of shared memory and 256 columns of tensor memory each, so that two CTAs share an SM.  A CTA
 // works through the dependent phases of one chunk-head (product -> readout -> product ...) while its neighbour is in another
 // phase of another chunk-head, which is what keeps the tensor pipe and the load/store path busy.  A trip's inputs are
 // dead once its last product is done, so the next trip's are loaded right then, under the last readout and the stores
